@@ -32,6 +32,9 @@ void free_device(mdp_plan *p) {
   cudaFree(p->d_subs);
   cudaFree(p->d_tables);
   cudaFree(p->d_piv);
+  cudaFree(p->d_sep);
+  cudaFree(p->alt_sep);
+  p->d_sep = p->alt_sep = nullptr;
   cudaFree(p->d_ws);
   cudaFree(p->d_status);
   cudaFree(p->d_fstatus);
@@ -77,7 +80,7 @@ mdp_status alloc_device(mdp_plan *p) {
   auto al = [&](void **ptr, size_t bytes) -> bool { return cudaMalloc(ptr, std::max<size_t>(bytes, 256)) == cudaSuccess; };
   if (!al((void **)&p->d_subs, p->subs.size() * sizeof(SubDesc)) ||
       !al((void **)&p->d_tables, p->host_tables.size() * sizeof(double)) ||
-      !al((void **)&p->d_piv, p->host_piv.size()) || !al((void **)&p->d_ws, (size_t)p->ws_doubles * 8) ||
+      !al((void **)&p->d_piv, p->host_piv.size()) || !al((void **)&p->d_sep, (size_t)p->sep_bytes) || !al((void **)&p->d_ws, (size_t)p->ws_doubles * 8) ||
       !al((void **)&p->d_status, sizeof(int)) || !al((void **)&p->d_fstatus, sizeof(int)) ||
       !p->sub_stage.alloc(p->subs.size(), true) || !p->h_fstatus.alloc(1, true))
     return MDP_ERR_NOMEM;
@@ -96,6 +99,23 @@ mdp_status alloc_device(mdp_plan *p) {
 #endif
   mdp_status st = upload_subs_tables(p);
   if (st != MDP_OK) return st;
+  for (int si = 0; si < p->n_subs; ++si) {
+    const SubDesc &d = p->subs[si].d;
+    if (d.leader != si) continue;
+    std::vector<double> ab(2 * (size_t)d.Nq);
+    for (int q = 1; q <= d.Nq; ++q) mode_entries(d, q, ab[2 * q - 2], ab[2 * q - 1]);
+    CK(cudaMemcpy(p->d_sep + d.sep_ab, ab.data(), ab.size() * sizeof(double), cudaMemcpyHostToDevice));
+  }
+  CK(launch_sep_tables(p, p->d_subs, p->d_tables, p->d_sep, false, nullptr));
+  CK(cudaStreamSynchronize(nullptr));
+#if MDP_CHECKED
+  if (fault && !std::strcmp(fault, "factor") && !p->subs.empty() && p->subs[0].d.tc_cols) {
+    double row[SEP_MTW];   // the same fault in the separable tables: the entries of mode 1
+    CK(cudaMemcpy(row, p->d_sep + p->subs[0].d.sep_mt, sizeof row, cudaMemcpyDeviceToHost));
+    for (double &v : row) v *= 1.5;
+    CK(cudaMemcpy(p->d_sep + p->subs[0].d.sep_mt, row, sizeof row, cudaMemcpyHostToDevice));
+  }
+#endif
   for (int sc = 0; sc < 3; ++sc) {
     auto &waves = p->sched[sc];
     auto &ditems = p->d_items[sc];
@@ -114,7 +134,7 @@ mdp_status alloc_device(mdp_plan *p) {
       for (int f = 0; f < NFAM; ++f)
         for (int i = 0; i < n; ++i)
           pre[(size_t)f * (n + 1) + i + 1] =
-              pre[(size_t)f * (n + 1) + i] + blocks_for((Fam)f, p->subs[w.items[i].sub].d, w.items[i].ncols);
+              pre[(size_t)f * (n + 1) + i] + blocks_for((Fam)f, p->subs[w.items[i].sub].d, w.items[i].ncols, w.items[i].col0);
 #if MDP_CHECKED
       if (fault && !std::strcmp(fault, "desc") && sc == S_PROJ && &w == &waves.front() && n > 0) {
         std::vector<Item> bad(w.items);
@@ -129,13 +149,13 @@ mdp_status alloc_device(mdp_plan *p) {
       // then by mode group (low modes first: the propagating modes carry the complex rows), then
       // item, then column block
       std::vector<int> order;
-      for (const Fam f : {F_TRI, F_ATRI}) {
+      for (const Fam f : {F_TRI, F_ATRI, F_PTRI}) {
         const int *pt = pre.data() + (size_t)f * (n + 1);
         std::vector<std::array<int, 4>> keys;
         keys.reserve(pt[n]);
         for (int i = 0; i < n; ++i) {
           const SubDesc &d = p->subs[w.items[i].sub].d;
-          const int cb = (w.items[i].ncols + 31) / 32, rows = f == F_TRI ? d.NYf : d.Nt;
+          const int cb = (w.items[i].ncols + 31) / 32, rows = f == F_ATRI ? d.Nt : d.NYf;
           for (int l = 0; l < pt[i + 1] - pt[i]; ++l) keys.push_back({-rows, l / cb, i, l});
         }
         std::stable_sort(keys.begin(), keys.end());
@@ -159,8 +179,10 @@ void wave_batches(const mdp_plan *p, size_t w, Batch *fb, int sc) {
     b.items = p->d_items[sc][w];
     b.prefix = p->d_prefix[sc][w] + (size_t)f * (n + 1);
     b.order = f == F_TRI ? p->d_order[sc][w]
-              : f == F_ATRI ? p->d_order[sc][w] + p->h_prefix[sc][w][(size_t)F_TRI * (n + 1) + n]
-                            : nullptr;
+              : f == F_ATRI || f == F_PTRI
+                  ? p->d_order[sc][w] + p->h_prefix[sc][w][(size_t)F_TRI * (n + 1) + n] +
+                        (f == F_PTRI ? p->h_prefix[sc][w][(size_t)F_ATRI * (n + 1) + n] : 0)
+                  : nullptr;
     b.n_items = n;
     b.total_blocks = p->h_prefix[sc][w][(size_t)f * (n + 1) + n];
     set_bounds(p, b, p->out_size, sc == S_GRAD);
@@ -175,7 +197,7 @@ void single_batches(const mdp_plan *p, const Item &it, Batch *fb, long long out_
     b.prefix = nullptr;
     b.n_items = 1;
     b.one = it;
-    b.total_blocks = blocks_for((Fam)f, p->subs[it.sub].d, it.ncols);
+    b.total_blocks = blocks_for((Fam)f, p->subs[it.sub].d, it.ncols, it.col0);
     set_bounds(p, b, out_n, false);
   }
 }
@@ -201,7 +223,7 @@ cudaError_t end_use(mdp_plan *p, cudaStream_t st) {
 mdp::HostBuf<SubDesc> &stage_of(mdp_plan *p, int set) { return set == 0 ? p->sub_stage : p->alt_stage; }
 
 void destroy_prof(mdp_plan *p) {
-  for (int f = 0; f < 16; ++f) {
+  for (int f = 0; f < 32; ++f) {
     for (auto &e : p->prof_ev[f]) { cudaEventDestroy(e.first); cudaEventDestroy(e.second); }
     p->prof_ev[f].clear();
     p->prof_used[f] = 0;
@@ -308,11 +330,12 @@ mdp_status mdp_plan_update_k_stream(mdp_plan *p, const double *k, void *cuda_str
   for (size_t i = 0; i < p->subs.size(); ++i) stage[i] = p->subs[i].d;
   CK(cudaMemcpyAsync(p->d_subs, stage.data(), p->subs.size() * sizeof(SubDesc), cudaMemcpyHostToDevice, s));
   CK(cudaMemsetAsync(p->d_fstatus, 0, sizeof(int), s));
-  CK(launch_factor(p, p->d_fstatus, s));
+  CK(launch_factor_to(p, p->d_subs, p->d_tables, p->d_piv, p->d_fstatus, false, s));
+  CK(launch_sep_tables(p, p->d_subs, p->d_tables, p->d_sep, true, s));
   CK(cudaMemcpyAsync(p->h_fstatus.data(), p->d_fstatus, sizeof(int), cudaMemcpyDeviceToHost, s));
   if (p->ready_ev[p->set]) CK(cudaEventRecord(p->ready_ev[p->set], s));
   CK(cudaStreamSynchronize(s));
-  p->host_stale = true;
+  p->host_stale = p->fs_stale = true;
   return (mdp_status)p->h_fstatus[0];
 }
 
@@ -329,6 +352,7 @@ mdp_status mdp_plan_update_k_async(mdp_plan *p, const double *k, void *cuda_stre
     const size_t np = std::max<size_t>(p->host_piv.size(), 256);
     const size_t ns = std::max<size_t>(p->subs.size() * sizeof(SubDesc), 256);
     if (cudaMalloc((void **)&p->alt_tables, nt) != cudaSuccess || cudaMalloc((void **)&p->alt_piv, np) != cudaSuccess ||
+        cudaMalloc((void **)&p->alt_sep, std::max<size_t>((size_t)p->sep_bytes, 256)) != cudaSuccess ||
         cudaMalloc((void **)&p->alt_subs, ns) != cudaSuccess || !p->alt_stage.alloc(p->subs.size(), true))
       return MDP_ERR_NOMEM;
     for (int s_ = 0; s_ < 2; ++s_) {
@@ -345,13 +369,15 @@ mdp_status mdp_plan_update_k_async(mdp_plan *p, const double *k, void *cuda_stre
   if (p->used_rec[b]) CK(cudaStreamWaitEvent(s, p->used_ev[b], 0));   // queued calls still reading set b
   for (size_t i = 0; i < p->subs.size(); ++i) stage[i] = p->subs[i].d;
   CK(cudaMemcpyAsync(p->alt_subs, stage.data(), p->subs.size() * sizeof(SubDesc), cudaMemcpyHostToDevice, s));
-  CK(launch_factor_to(p, p->alt_subs, p->alt_tables, p->alt_piv, p->d_status, s));
+  CK(launch_factor_to(p, p->alt_subs, p->alt_tables, p->alt_piv, p->d_status, false, s));
+  CK(launch_sep_tables(p, p->alt_subs, p->alt_tables, p->alt_sep, true, s));
   CK(cudaEventRecord(p->ready_ev[b], s));
   std::swap(p->d_subs, p->alt_subs);
   std::swap(p->d_tables, p->alt_tables);
   std::swap(p->d_piv, p->alt_piv);
+  std::swap(p->d_sep, p->alt_sep);
   p->set = b;
-  p->host_stale = true;
+  p->host_stale = p->fs_stale = true;
   return MDP_OK;
 }
 
@@ -390,6 +416,12 @@ mdp_status mdp_plan_read_tables(const mdp_plan *p, int device_side, double *tabl
     if (!device_ok(p)) return MDP_ERR_STATE;
     CK(cudaSetDevice(p->device));
     CK(cudaDeviceSynchronize());
+    if (p->fs_stale) {   // the sweep tables follow the wavenumbers only where they are read
+      mdp_plan *mp = const_cast<mdp_plan *>(p);
+      CK(launch_factor_to(p, p->d_subs, p->d_tables, p->d_piv, p->d_fstatus, true, nullptr));
+      CK(cudaStreamSynchronize(nullptr));
+      mp->fs_stale = false;
+    }
     CK(cudaMemcpy(tables, p->d_tables, p->host_tables.size() * sizeof(double), cudaMemcpyDeviceToHost));
     CK(cudaMemcpy(piv, p->d_piv, p->host_piv.size(), cudaMemcpyDeviceToHost));
     return MDP_OK;
@@ -685,7 +717,10 @@ mdp_status mdp_plan_set_receivers(mdp_plan *p, const int *rows) {
   std::vector<SubDesc> ds;
   for (auto &hs : p->subs) ds.push_back(hs.d);
   CK(cudaMemcpy(p->d_subs, ds.data(), ds.size() * sizeof(SubDesc), cudaMemcpyHostToDevice));
-  // the receiver kernel's block counts changed: refresh the prefix sums (same sizes)
+  // the receiver row's moments, into the tables in use (the other set is rebuilt by its next update)
+  CK(launch_sep_tables(p, p->d_subs, p->d_tables, p->d_sep, false, nullptr));
+  CK(cudaStreamSynchronize(nullptr));
+  // the block counts of the receiver kernel and of the contractions changed: refresh the prefix sums
   for (int sc = 0; sc < 3; ++sc) {
     auto &waves = p->sched[sc];
     auto &dpre = p->d_prefix[sc];
@@ -693,9 +728,11 @@ mdp_status mdp_plan_set_receivers(mdp_plan *p, const int *rows) {
     for (size_t w = 0; w < waves.size(); ++w) {
       const int n = (int)waves[w].items.size();
       auto &pre = hpre[w];
-      for (int i = 0; i < n; ++i)
-        pre[(size_t)F_IREC * (n + 1) + i + 1] =
-            pre[(size_t)F_IREC * (n + 1) + i] + blocks_for(F_IREC, p->subs[waves[w].items[i].sub].d, waves[w].items[i].ncols);
+      for (const Fam f : {F_IREC, F_G1B, F_G1U})
+        for (int i = 0; i < n; ++i)
+          pre[(size_t)f * (n + 1) + i + 1] =
+              pre[(size_t)f * (n + 1) + i] +
+              blocks_for(f, p->subs[waves[w].items[i].sub].d, waves[w].items[i].ncols, waves[w].items[i].col0);
       CK(cudaMemcpy(dpre[w], pre.data(), pre.size() * sizeof(int), cudaMemcpyHostToDevice));
     }
   }

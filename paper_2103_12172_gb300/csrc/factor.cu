@@ -7,7 +7,9 @@
 //   - factor rows (l, 1/d, du/d, du2/d), the swap flags and dT_q/dk rows (gradient pass,
 //     full-grid solves), with the run of exactly-real rows around the middle row;
 //   - the condensed, pivot-scaled forward-sweep rows of the projection (rows above the ring
-//     folded into the last pivot by their Schur complement), with its run of real rows.
+//     folded into the last pivot by their Schur complement), with its run of real rows; only for
+//     subdomains that project by sweeps (without the separable solve), or when `all` is set (table
+//     introspection).
 // The host plan builds the same tables at plan creation (plan.cpp: mode_matrix, band_lu,
 // factor_mode, build_fs_mode). Two kernels:
 //   k_factor_chain  the pivot recurrences, the only sequential part: one thread per (mode,
@@ -264,15 +266,16 @@ __device__ void chain_sweep(const SubDesc &d, int q, double *tab, int *status) {
 }
 
 __global__ void __launch_bounds__(32) k_factor_chain(const SubDesc *subs, int n_subs, int n_modes, double *tab,
-                                                      uint8_t *piv, int *status) {
+                                                      uint8_t *piv, int *status, int all) {
   int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= 2 * n_modes) return;
   const bool sweep = t >= n_modes;
   if (sweep) t -= n_modes;
   int si = mode_owner(subs, n_subs, t);
   if (si >= n_subs) return;
-  if (sweep) chain_sweep(subs[si], t + 1, tab, status);
-  else chain_full(subs[si], t + 1, tab, piv, status);
+  if (sweep) {
+    if (all || !subs[si].tc_cols) chain_sweep(subs[si], t + 1, tab, status);
+  } else chain_full(subs[si], t + 1, tab, piv, status);
 }
 
 constexpr int kRowsThreads = 256;
@@ -284,7 +287,7 @@ struct RunReduce {
   __device__ void init(int lo, int hi) { lastbad = lo - 1; firstbad = hi; midreal = 0; }
 };
 
-__global__ void __launch_bounds__(kRowsThreads) k_factor_rows(const SubDesc *subs, int n_subs, double *tab) {
+__global__ void __launch_bounds__(kRowsThreads) k_factor_rows(const SubDesc *subs, int n_subs, double *tab, int all) {
   __shared__ RunReduce run;
   __shared__ double raw[(kRowsThreads + 1) * 11];
   int t = blockIdx.x;
@@ -350,6 +353,7 @@ __global__ void __launch_bounds__(kRowsThreads) k_factor_rows(const SubDesc *sub
     }
     if (tid == 0) { sg[0] = 0; sg[1] = N; }
   }
+  if (d.tc_cols && !all) return;
   // ---- sweep rows i0 .. itop from the raw rows, in chunks of kRowsThreads rows
   const int itop = (int)sg[4], i0 = d.i0;
   const int mid = (i0 + itop) / 2;
@@ -413,18 +417,17 @@ __global__ void k_probe_rcp(const double *x, double *y, int n) {
 
 // The chains: one thread each, warps spread one per block so that they do not share an SM's
 // FP64 unit while there are fewer warps than SMs. The row kernel: one block per mode.
-cudaError_t launch_factor(const mdp_plan *p, int *status, cudaStream_t st) {
-  return launch_factor_to(p, p->d_subs, p->d_tables, p->d_piv, status, st);
-}
-
-cudaError_t launch_factor_to(const mdp_plan *p, const SubDesc *ds, double *tab, uint8_t *piv, int *status,
+cudaError_t launch_factor_to(const mdp_plan *p, const SubDesc *ds, double *tab, uint8_t *piv, int *status, bool all,
                              cudaStream_t st) {
   int n_modes = 0;
-  for (size_t i = 0; i < p->subs.size(); ++i)
+  bool sweeps = all;
+  for (size_t i = 0; i < p->subs.size(); ++i) {
+    sweeps = sweeps || !p->subs[i].d.tc_cols;
     if (p->subs[i].d.leader == (int)i) n_modes += p->subs[i].d.Nq;
-  const int threads = 2 * n_modes;
-  k_factor_chain<<<(threads + 31) / 32, 32, 0, st>>>(ds, (int)p->subs.size(), n_modes, tab, piv, status);
-  k_factor_rows<<<n_modes, kRowsThreads, 0, st>>>(ds, (int)p->subs.size(), tab);
+  }
+  const int threads = sweeps ? 2 * n_modes : n_modes;
+  k_factor_chain<<<(threads + 31) / 32, 32, 0, st>>>(ds, (int)p->subs.size(), n_modes, tab, piv, status, all);
+  k_factor_rows<<<n_modes, kRowsThreads, 0, st>>>(ds, (int)p->subs.size(), tab, all);
   return cudaGetLastError();
 }
 

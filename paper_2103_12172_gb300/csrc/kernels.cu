@@ -120,7 +120,6 @@ __global__ void __launch_bounds__(256) k_residual(Batch bt, const SubDesc *subs,
   const int b = (local % cb) * 32 + threadIdx.x;
   const int u = (local / cb) * 8 + threadIdx.y;
   const int units = d.xsym ? 4 * d.Ph + 2 * (d.Py - 4) : d.R;
-  if (!GRAD && u == 0 && b < it.ncols && d.tc_cols) reinterpret_cast<int *>(ws + it.red_off)[b] = 0;  // for k_tri
   if (b >= it.ncols || u >= units) return;
   double *r = ws + it.r_off;
   double *sb = ws + it.s_off;
@@ -770,8 +769,6 @@ __device__ __forceinline__ void tri_fs_body(const Item &it, const SubDesc &d, co
   }
   const int ikeep = nhi + 1 - nfirst;
   cplx x1 = cmk(0.0, 0.0), x2 = cmk(0.0, 0.0);
-  int emax = 0;   // largest biased exponent of the kept rows (integer compares only)
-  auto bexp = [](double v) { return (__double2hiint(v) >> 20) & 0x7ff; };
   for (i = itop; i >= i0; --i) {
     cp_async_wait<TRI_STAGES - 1>();
     __syncwarp(mask);
@@ -791,20 +788,76 @@ __device__ __forceinline__ void tri_fs_body(const Item &it, const SubDesc &d, co
     if (i - TRI_STAGES >= i0) fetch_back(i - TRI_STAGES); else cp_async_commit();
     if (i <= ikeep) {
       ystore(i, x);
-      emax = max(emax, max(bexp(x.re), bexp(x.im)));
     }
     x2 = x1; x1 = x;
   }
-  // per column, over every mode: the common power-of-two scale of the tensor-core gamma columns
-  if (d.tc_cols) atomicMax(reinterpret_cast<int *>(ws + it.red_off) + b, emax);
+}
+
+// The modes next to and below the cutoff (kinds 0, 1 of the mode table, the first tens of a
+// subdomain's): their pivots never settle, every row's rounding shifts the phase, and on fine grids
+// (1025^2 on) the recurrence is off by 1e-12 to 1e-11 of a mode's largest value. The closed form with
+// running moments stays within 1e-13:
+//   x_i = phi_1(i) (A + F (M_2 - 2 P_2(i))) + phi_2(i) (B + F (2 P_1(i) - M_1)),
+//   P_b(i) = sum_{j <= i} phi_b(j) g_j, M_b the sums over all rows, (A, B) = R M.
+template <bool CD, bool CIN>
+__device__ __forceinline__ void tri_phi_body(const Item &it, const SubDesc &d, const double *tab, const unsigned char *sep,
+                                             double *ws, int b, int q) {
+  const double *T = reinterpret_cast<const double *>(sep + d.sep_mt) + (long long)(q - 1) * SEP_MTW;
+  const double *P1 = reinterpret_cast<const double *>(sep + d.sep_phi) + (q - 1), *P2 = P1 + (long long)(d.Py + 2) * d.Nq;
+  const double *S = tab + d.sin_off, *r = ws + it.r_off, *gr = ws + it.gr_off;
+  const long long nc = it.ncols;
+  const int N2 = 2 * d.Nx, par = (q & 1) ? 0 : 1, ns = d.xsym ? 2 : 4;
+  const int ms[4] = {d.mlo, d.mlo + 1, d.mhi - 1, d.mhi};
+  double sn[4];
+#pragma unroll
+  for (int s = 0; s < 4; ++s) sn[s] = S[(int)(((long long)q * ms[s]) % N2)];
+  auto val = [&](const double *base, long long o) { return CIN ? ld2(base + 2 * o) : cmk(base[o], 0.0); };
+  auto axpy = [&](double s, cplx x, cplx y) { return CIN ? caxpy(s, x, y) : cmk(fma(s, x.re, y.re), 0.0); };
+  auto src = [&](int k) -> cplx {   // grid row nlo - 1 + k
+    const int n = d.nlo - 1 + k;
+    if (n < d.nlo || n > d.nhi) return cmk(0.0, 0.0);
+    const int rr = n == d.nlo ? 0 : n == d.nlo + 1 ? 1 : n == d.nhi - 1 ? 2 : n == d.nhi ? 3 : -1;
+    if (rr >= 0) return val(gr, ((long long)rr * d.Nq + (q - 1)) * nc + b);
+    const long long slot = d.xsym ? 8LL * d.Ph + 4 * (n - d.nlo - 2) + par : 2LL * d.Px + 4 * (n - d.nlo - 2);
+    cplx v = cmk(0.0, 0.0);
+#pragma unroll
+    for (int s = 0; s < 4; ++s)
+      if (s < ns) v = axpy(sn[s], val(r, (slot + (d.xsym ? 2 * s : s)) * nc + b), v);
+    return v;
+  };
+  const int rows = d.Py + 2;
+  cplx m1 = cmk(0.0, 0.0), m2 = m1;
+#pragma unroll 4
+  for (int k = 0; k < rows; ++k) {
+    const cplx g = src(k);
+    m1 = axpy(P1[(long long)k * d.Nq], g, m1);
+    m2 = axpy(P2[(long long)k * d.Nq], g, m2);
+  }
+  const cplx R11 = ld2(T + MT_R), R12 = ld2(T + MT_R + 2), R22 = ld2(T + MT_R + 4);
+  const double F = T[MT_F];
+  const cplx A = caxpy(F, m2, cadd(cmul(R11, m1), cmul(R12, m2))), B = caxpy(-F, m1, cadd(cmul(R12, m1), cmul(R22, m2)));
+  double *y = ws + it.y_off;
+  cplx p1 = cmk(0.0, 0.0), p2 = p1;
+#pragma unroll 4
+  for (int k = 0; k < rows; ++k) {
+    const cplx g = src(k);
+    const double f1 = P1[(long long)k * d.Nq], f2 = P2[(long long)k * d.Nq];
+    p1 = axpy(f1, g, p1);
+    p2 = axpy(f2, g, p2);
+    const cplx u = axpy(-2.0 * F, p2, cmk(0.0, 0.0)), v = axpy(2.0 * F, p1, cmk(0.0, 0.0));
+    const double re = fma(f1, A.re + u.re, f2 * (B.re + v.re));
+    const long long o = ((long long)(q - 1) * d.NYf + k) * nc + b;
+    if (CD) st2(y + 2 * o, cmk(re, fma(f1, A.im + u.im, f2 * (B.im + v.im))));
+    else y[o] = re;
+  }
 }
 
 template <bool CIN, bool FULL, int TRI_STAGES>
 __global__ void __launch_bounds__(32 * TRI_WARPS, 32 / TRI_WARPS) k_tri(Batch bt, const SubDesc *subs, const double *tab, const uint8_t *pivtab,
-                                             double *ws) {
+                                             double *ws, const unsigned char *sep) {
   Item it; int local;
   locate(bt, bt.order ? bt.order[blockIdx.x] : (int)blockIdx.x, it, local);
-  MDP_CHECK_ITEM(bt, subs, it, local, F_TRI);
+  MDP_CHECK_ITEM(bt, subs, it, local, FULL ? F_TRI : F_PTRI);
   const SubDesc &d = subs[it.sub];
   const int cb = (it.ncols + 31) >> 5;
   const int b = (local % cb) * 32 + threadIdx.x;
@@ -818,6 +871,9 @@ __global__ void __launch_bounds__(32 * TRI_WARPS, 32 / TRI_WARPS) k_tri(Batch bt
     char *sw = tri_sm + threadIdx.y * 2 * full_stage_bytes<CIN>();
     if (d.cplx) tri_full_body<true, CIN>(it, d, tab, pivtab, ws, b, q, sw, threadIdx.x, __popc(mask), mask);
     else tri_full_body<false, CIN>(it, d, tab, pivtab, ws, b, q, sw, threadIdx.x, __popc(mask), mask);
+  } else if ((int)reinterpret_cast<const double *>(sep + d.sep_mt)[(long long)(q - 1) * SEP_MTW + MT_KIND] < 2) {
+    if (d.cplx || CIN) tri_phi_body<true, CIN>(it, d, tab, sep, ws, b, q);
+    else tri_phi_body<false, CIN>(it, d, tab, sep, ws, b, q);
   } else {
     char *sw = tri_sm + threadIdx.y * TRI_STAGES * tri_stage_bytes<CIN>();
     if (d.cplx || CIN) tri_fs_body<true, CIN, TRI_STAGES>(it, d, tab, ws, b, q, sw, threadIdx.x, __popc(mask), mask);
@@ -835,6 +891,10 @@ __device__ __forceinline__ void write_out(const SubDesc &d, const Item &it, cons
   out[it.io_off + (long long)b * d.G + g] = make_double2(v.re, v.im);
 }
 
+// rows per mode of the projection's mode-space field: the swept ones, or the 4 gamma rows and the
+// receiver row that the separable solve keeps
+__device__ __forceinline__ int field_rows(const SubDesc &d) { return d.tc_cols ? 5 : d.NYf; }
+
 // u(m, n) = (2/Nx) sum_q sin(pi q m/Nx) yhat(q, n) for the 4 full gamma rows. Centred
 // subdomains: one thread gives u(m) = E + O and u(Nx - m) = E - O from the odd-q (E) and
 // even-q (O) partial sums, since sin(pi q (Nx-m)/Nx) = (-1)^(q+1) sin(pi q m/Nx).
@@ -845,11 +905,11 @@ __device__ __forceinline__ void inv_rows_body(const Item &it, const SubDesc &d, 
   const int span = d.xsym ? d.Ph + 1 : W;
   const int grow = task / span, dm = task % span, m = d.mlo - 1 + dm;
   const int n = grow == 0 ? d.nlo - 1 : grow == 1 ? d.nlo : grow == 2 ? d.nhi : d.nhi + 1;
-  const int yrow = n - (d.nlo - 1);
+  const int yrow = d.tc_cols ? grow : n - (d.nlo - 1);
   const double *Si = tab + d.sin_off + 2 * d.Nx;
   const int N2 = 2 * d.Nx;
   const double *y = ws + it.y_off;
-  const long long qstride = (long long)d.NYf * it.ncols;
+  const long long qstride = (long long)field_rows(d) * it.ncols;
   const long long base = (long long)yrow * it.ncols + b;
   auto yv = [&](int q) -> cplx {
     const long long o = base + (long long)(q - 1) * qstride;
@@ -894,9 +954,9 @@ __device__ __forceinline__ void inv_rows_fft_body(const Item &it, const SubDesc 
   while ((1 << lg) < N) ++lg;
   const double *sn = tab + d.sin_off;
   const int n = grow == 0 ? d.nlo - 1 : grow == 1 ? d.nlo : grow == 2 ? d.nhi : d.nhi + 1;
-  const int yrow = n - (d.nlo - 1);
+  const int yrow = d.tc_cols ? grow : n - (d.nlo - 1);
   const double *y = ws + it.y_off;
-  const long long qstride = (long long)d.NYf * it.ncols;
+  const long long qstride = (long long)field_rows(d) * it.ncols;
   auto yv = [&](int q, int f) -> cplx {   // yhat(q) of column b0 + f, q = 1 .. N-1
     const long long o = (long long)(q - 1) * qstride + (long long)yrow * it.ncols + b0 + f;
     return CD ? ld2(y + 2 * o) : cmk(y[o], 0.0);
@@ -1041,11 +1101,11 @@ template <bool CD>
 __device__ __forceinline__ void inv_rec_body(const Item &it, const SubDesc &d, const double *tab, const double *ws,
                                              double2 *out_rec, int b, int task) {
   const int m = d.mlo + 1 + task;
-  const int yrow = d.nrec - (d.nlo - 1);
+  const int yrow = d.tc_cols ? 4 : d.nrec - (d.nlo - 1);
   const double *Si = tab + d.sin_off + 2 * d.Nx;
   const int N2 = 2 * d.Nx;
   const double *y = ws + it.y_off;
-  const long long qstride = (long long)d.NYf * it.ncols;
+  const long long qstride = (long long)field_rows(d) * it.ncols;
   const long long base = (long long)yrow * it.ncols + b;
   auto yv = [&](int q) -> cplx {
     const long long o = base + (long long)(q - 1) * qstride;
@@ -1389,7 +1449,7 @@ cudaError_t launch_source_terms(mdp_plan *p, int sub, const double2 *f, const do
   Batch fb[NFAM];
   for (int f_ = 0; f_ < NFAM; ++f_) {
     std::memset(&fb[f_], 0, sizeof fb[f_]);
-    fb[f_].n_items = 1; fb[f_].one = it; fb[f_].total_blocks = blocks_for((Fam)f_, d, 1);
+    fb[f_].n_items = 1; fb[f_].one = it; fb[f_].total_blocks = blocks_for((Fam)f_, d, 1, 0);
     set_bounds(p, fb[f_], d.G, false);
   }
   e = launch_project(p, fb, MDP_OUT_Q, xi_i, F, nullptr, st);
@@ -1410,7 +1470,7 @@ cudaError_t launch_basis_densities(const mdp_plan *p, int sub, int col0, int nco
     it.xi_off = xo; it.r_off = ro; it.gr_off = go; it.y_off = yo; it.a_off = ao; it.s_off = so; it.red_off = reo;
     Batch b;
     std::memset(&b, 0, sizeof b);
-    b.n_items = 1; b.one = it; b.total_blocks = blocks_for(F_EXT, d, it.ncols);
+    b.n_items = 1; b.one = it; b.total_blocks = blocks_for(F_EXT, d, it.ncols, it.col0);
     set_bounds(p, b, (long long)ncols * d.G, false);
     k_extend<<<dim3((unsigned)b.total_blocks), 128, 0, st>>>(b, p->d_subs, p->d_tables, p->d_ws, 0);
     const long long n = (long long)it.ncols * d.G;
@@ -1434,6 +1494,7 @@ cudaError_t set_kernel_attributes() {
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fwd_rows<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, FFT_SMEM);
   if (e == cudaSuccess) e = set_adj_kernel_attributes();
   if (e == cudaSuccess) e = set_tc_kernel_attributes();
+  if (e == cudaSuccess) e = set_sep_kernel_attributes();
   // the sweep's staging buffers take 32 x 2.4 KiB per SM at full occupancy: prefer shared memory
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_tri<false, false, 2>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
@@ -1453,25 +1514,28 @@ cudaError_t launch_project(mdp_plan *p, const Batch *fb, int out_kind, const dou
   const double *tab = p->d_tables;
   double *ws = p->d_ws;
   const dim3 b8(32, 8), btri(32, TRI_WARPS);
-#define MDP_LAUNCH(fam, ...)                      \
+#define MDP_LAUNCH_AS(fam, as, ...)               \
   do {                                            \
     if (fb[fam].total_blocks > 0) {               \
-      prof_begin(p, fam, st);                     \
+      prof_begin(p, as, st);                      \
       __VA_ARGS__;                                \
-      prof_end(p, fam, st);                       \
+      prof_end(p, as, st);                        \
     }                                             \
   } while (0)
+#define MDP_LAUNCH(fam, ...) MDP_LAUNCH_AS(fam, fam, __VA_ARGS__)
   if (basis) MDP_LAUNCH(F_EXT, k_extend<<<grid1(fb[F_EXT].total_blocks), 128, 0, st>>>(fb[F_EXT], ds, tab, ws, 0));
   if (basis) MDP_LAUNCH(F_RES, k_residual<false, false><<<grid1(fb[F_RES].total_blocks), b8, 0, st>>>(fb[F_RES], ds, tab, ws, xi_user));
   else MDP_LAUNCH(F_RES, k_residual<true, false><<<grid1(fb[F_RES].total_blocks), b8, 0, st>>>(fb[F_RES], ds, tab, ws, xi_user));
   if (basis) MDP_LAUNCH(F_FROWS, k_fwd_rows<false><<<grid1(fb[F_FROWS].total_blocks), b8, p->fft_smem, st>>>(fb[F_FROWS], ds, tab, ws));
   else MDP_LAUNCH(F_FROWS, k_fwd_rows<true><<<grid1(fb[F_FROWS].total_blocks), b8, p->fft_smem, st>>>(fb[F_FROWS], ds, tab, ws));
+  cudaError_t e = launch_sep_project(p, fb, out_kind, xi_user, out, 0, st);
+  if (e != cudaSuccess) return e;
   if (p->tri_stages == 4) {
-    if (basis) MDP_LAUNCH(F_TRI, k_tri<false, false, 4><<<grid1(fb[F_TRI].total_blocks), btri, tri_smem_bytes<false, 4>(), st>>>(fb[F_TRI], ds, tab, p->d_piv, ws));
-    else MDP_LAUNCH(F_TRI, k_tri<true, false, 4><<<grid1(fb[F_TRI].total_blocks), btri, tri_smem_bytes<true, 4>(), st>>>(fb[F_TRI], ds, tab, p->d_piv, ws));
+    if (basis) MDP_LAUNCH_AS(F_PTRI, F_TRI, k_tri<false, false, 4><<<grid1(fb[F_PTRI].total_blocks), btri, tri_smem_bytes<false, 4>(), st>>>(fb[F_PTRI], ds, tab, p->d_piv, ws, p->d_sep));
+    else MDP_LAUNCH_AS(F_PTRI, F_TRI, k_tri<true, false, 4><<<grid1(fb[F_PTRI].total_blocks), btri, tri_smem_bytes<true, 4>(), st>>>(fb[F_PTRI], ds, tab, p->d_piv, ws, p->d_sep));
   } else {
-    if (basis) MDP_LAUNCH(F_TRI, k_tri<false, false, 2><<<grid1(fb[F_TRI].total_blocks), btri, tri_smem_bytes<false, 2>(), st>>>(fb[F_TRI], ds, tab, p->d_piv, ws));
-    else MDP_LAUNCH(F_TRI, k_tri<true, false, 2><<<grid1(fb[F_TRI].total_blocks), btri, tri_smem_bytes<true, 2>(), st>>>(fb[F_TRI], ds, tab, p->d_piv, ws));
+    if (basis) MDP_LAUNCH_AS(F_PTRI, F_TRI, k_tri<false, false, 2><<<grid1(fb[F_PTRI].total_blocks), btri, tri_smem_bytes<false, 2>(), st>>>(fb[F_PTRI], ds, tab, p->d_piv, ws, p->d_sep));
+    else MDP_LAUNCH_AS(F_PTRI, F_TRI, k_tri<true, false, 2><<<grid1(fb[F_PTRI].total_blocks), btri, tri_smem_bytes<true, 2>(), st>>>(fb[F_PTRI], ds, tab, p->d_piv, ws, p->d_sep));
   }
   if (basis) {
     MDP_LAUNCH(F_IROWS, k_inv_rows<false><<<grid1(fb[F_IROWS].total_blocks), b8, p->fft_smem, st>>>(fb[F_IROWS], ds, tab, ws, xi_user, out, out_kind));
@@ -1480,8 +1544,8 @@ cudaError_t launch_project(mdp_plan *p, const Batch *fb, int out_kind, const dou
     MDP_LAUNCH(F_IROWS, k_inv_rows<true><<<grid1(fb[F_IROWS].total_blocks), b8, p->fft_smem, st>>>(fb[F_IROWS], ds, tab, ws, xi_user, out, out_kind));
     MDP_LAUNCH(F_ICOLS, k_inv_cols<true><<<grid1(fb[F_ICOLS].total_blocks), b8, 0, st>>>(fb[F_ICOLS], ds, tab, ws, xi_user, out, out_kind));
   }
-  if (fb[F_TCOLS].total_blocks > 0)
-    MDP_LAUNCH(F_TCOLS, launch_inv_cols_tc(fb[F_TCOLS], ds, tab, ws, xi_user, out, out_kind, p->d_status, p->n_sm, st));
+  e = launch_sep_project(p, fb, out_kind, xi_user, out, 1, st);
+  if (e != cudaSuccess) return e;
   if (out_rec)
     MDP_LAUNCH(F_IREC, k_inv_rec<<<grid1(fb[F_IREC].total_blocks), b8, 0, st>>>(fb[F_IREC], ds, tab, ws, out_rec, basis ? 0 : 1));
   return cudaGetLastError();
@@ -1500,8 +1564,8 @@ cudaError_t launch_adjoint(mdp_plan *p, const Batch *fb, int out_kind, const dou
     else MDP_LAUNCH(F_RES, k_residual<true, true><<<grid1(fb[F_RES].total_blocks), b8, 0, st>>>(fb[F_RES], ds, tab, ws, xi_user));
     if (basis) MDP_LAUNCH(F_FROWS, k_fwd_rows<false><<<grid1(fb[F_FROWS].total_blocks), b8, p->fft_smem, st>>>(fb[F_FROWS], ds, tab, ws));
     else MDP_LAUNCH(F_FROWS, k_fwd_rows<true><<<grid1(fb[F_FROWS].total_blocks), b8, p->fft_smem, st>>>(fb[F_FROWS], ds, tab, ws));
-    if (basis) MDP_LAUNCH(F_TRI, k_tri<false, true, 2><<<grid1(fb[F_TRI].total_blocks), btri, TRI_WARPS * 2 * full_stage_bytes<false>(), st>>>(fb[F_TRI], ds, tab, p->d_piv, ws));
-    else MDP_LAUNCH(F_TRI, k_tri<true, true, 2><<<grid1(fb[F_TRI].total_blocks), btri, TRI_WARPS * 2 * full_stage_bytes<true>(), st>>>(fb[F_TRI], ds, tab, p->d_piv, ws));
+    if (basis) MDP_LAUNCH(F_TRI, k_tri<false, true, 2><<<grid1(fb[F_TRI].total_blocks), btri, TRI_WARPS * 2 * full_stage_bytes<false>(), st>>>(fb[F_TRI], ds, tab, p->d_piv, ws, p->d_sep));
+    else MDP_LAUNCH(F_TRI, k_tri<true, true, 2><<<grid1(fb[F_TRI].total_blocks), btri, TRI_WARPS * 2 * full_stage_bytes<true>(), st>>>(fb[F_TRI], ds, tab, p->d_piv, ws, p->d_sep));
   }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;

@@ -68,18 +68,18 @@ static __device__ __noinline__ bool item_in_bounds(const Batch &bt, const SubDes
   bool ok = it.sub >= 0 && it.sub < bt.n_subs && it.ncols >= 1 && local >= 0;
   if (ok) {
     const SubDesc &d = subs[it.sub];
-    ok = it.col0 >= 0 && it.col0 + it.ncols <= d.n_cols && local < blocks_for(fam, d, it.ncols);
+    ok = it.col0 >= 0 && it.col0 + it.ncols <= d.n_cols && local < blocks_for(fam, d, it.ncols, it.col0);
     long long xi, r, gr, y, a, s, red, tot;
     item_workspace(d, it.ncols, grad, xi, r, gr, y, a, s, red, tot);
     auto in_ws = [&](long long off, long long n) { return off >= 0 && off + n <= bt.ws_n; };
     ok = ok && in_ws(it.xi_off, r - xi) && in_ws(it.r_off, gr - r) && in_ws(it.gr_off, y - gr) &&
-         in_ws(it.y_off, a - y) && in_ws(it.red_off, tot - red) &&
-         (!grad || (in_ws(it.a_off, s - a) && in_ws(it.s_off, red - s)));
+         in_ws(it.y_off, a - y) && in_ws(it.a_off, s - a) &&
+         (!grad || (in_ws(it.s_off, red - s) && in_ws(it.red_off, tot - red)));
     auto in_tab = [&](long long off, long long n) { return off >= 0 && off + n <= bt.tab_n; };
     const long long qt = (long long)d.Nq * d.Nt;
     ok = ok && in_tab(d.fact_off, qt * (d.cplx ? 8 : 4)) && in_tab(d.dT_off, qt * 6) && in_tab(d.sin_off, 4LL * d.Nx) &&
          in_tab(d.geo_off, 4LL * d.G) && in_tab(d.seg_off, 5LL * d.Nq) && in_tab(d.fs_off, (long long)d.Nq * d.NYf * FSW) &&
-         (!d.tc_cols || in_tab(d.tcb_off, 256LL * ((d.Nq + 15) / 16)));
+         (!d.tc_cols || in_tab(d.tcb_off, 128LL * ((d.Nq + 15) / 16)));
     ok = ok && d.piv_off >= 0 && d.piv_off + qt <= bt.piv_n;
     ok = ok && it.io_off >= 0 && it.io_off + (long long)it.ncols * d.G <= bt.out_n;
   }
@@ -91,6 +91,31 @@ static __device__ __noinline__ bool item_in_bounds(const Batch &bt, const SubDes
   do {                                                                                          \
     if (MDP_CHECKED && !item_in_bounds(bt, subs, it, local, fam, bt.grad != 0)) return;         \
   } while (0)
+
+// per mode, MTW doubles (phi with their normalisation, rows relative to the ring):
+enum {
+  MT_P1D = 0,    // phi_1 at the 4 dense rows nlo, nlo+1, nhi-1, nhi
+  MT_P2D = 4,
+  MT_P1G = 8,    // phi_1 at the 4 gamma rows nlo-1, nlo, nhi, nhi+1
+  MT_P2G = 12,
+  MT_R = 16,     // R11, R12, R22 (complex)
+  MT_E1 = 22,    // what a dense row adds to A_1, A_2 on the middle rows through kappa
+  MT_E2 = 26,
+  MT_W1 = 30,    // what the moments add to the field of the 4 gamma rows through kappa
+  MT_W2 = 34,
+  MT_K = 38,     // kappa at 0, 1, 2, L-1, L, L+1 (L = nhi - nlo)
+  MT_REC = 44,   // receiver row: phi_1, phi_2, 1 / (scale of its moment table)
+  MT_T1 = 47,    // kappa(d) = T1 phi_1(J0 + d) + T2 phi_2(J0 + d)
+  MT_T2 = 48,
+  MT_RF = 49,    // scale of the receiver's moment table (a power of two)
+  MT_TH = 50,    // theta, kind, sign, normalisations of phi_1, phi_2 (for k_sep_phi)
+  MT_KIND = 51,
+  MT_SG = 52,
+  MT_N1 = 53,
+  MT_N2 = 54,
+  MT_F = 55,     // 1 / (2 a n1 n2): kappa(i - j) = F (phi_2(i) phi_1(j) - phi_1(i) phi_2(j)), i >= j (kinds 0, 1)
+};
+static_assert(MT_F < SEP_MTW, "mode table width");
 
 // gamma index of node (n, m), or -1 (row-major order of the 2-node ring around M+)
 __device__ __forceinline__ int gamma_index(const SubDesc &d, int n, int m) {

@@ -1,0 +1,899 @@
+// The projection's solves by the separable Green's function of the per-mode systems, with every
+// long sum on the tensor cores.
+//
+// Away from the two ends the rows of T_q (sine mode q along x, Section 3.2.1) have constant
+// coefficients (a, b, a), and the ring that carries r = L^(h) w lies strictly between the ends. On
+// those rows the inverse is therefore
+//   T_q^{-1}(i, j) = kappa_q(|i - j|) + sum_{a,b} phi_a(i) R_ab phi_b(j):
+// kappa_q is a fundamental solution of the constant-coefficient recurrence (cosh theta = -b/2a:
+// the decaying exponential for an evanescent mode, sin(|d| theta) / (2 a sin theta) for a
+// propagating one, its hyperbolic form next to the cutoff, where the exponential would cancel),
+// phi_1, phi_2 two homogeneous solutions (decaying away from either end, or cosine and sine about
+// the middle row), and the symmetric 2 x 2 matrix R follows from the rows at the two ends (the
+// Dirichlet or Sommerfeld conditions). Summed over q with the sine factors of the ring's columns
+// m_c and the trace's columns m_s, the middle rows need
+//   u(s, i) = sum_{c,j} K_sc(|i - j|) r_c(j) + sum_{q,b} (2/Nx) sin(pi q m_s/Nx) phi_b(i) A_b(q),
+//   K_sc(d) = (2/Nx) sum_q sin(pi q m_s/Nx) sin(pi q m_c/Nx) kappa_q(d),
+// where A_1, A_2 combine, per mode, the moments sum_{c,j} sin(pi q m_c/Nx) phi_b(j) r_c(j) and the
+// transforms of the 4 dense ring rows. So two contractions (k_sep_gemm) replace the recurrences:
+//   stage 1: r times [K | moment tables], K dimension (c, j);
+//   stage 2 (k_sep_modes): per (mode, column) R, the dense rows, the 4 gamma rows of the field;
+//   stage 3: A times [sines x phi], K dimension (b, q).
+// On x-centred subdomains odd and even modes separate (sums and differences of the mirrored
+// columns), which halves both dimensions: two classes with 2 columns each, else one with 4.
+//
+// Both contractions are to FP64 accuracy on the fp16 tensor cores by error-free splitting (Ozaki,
+// Ogita, Oishi and Rump, Numer. Algorithms 59, 2012): every operand value becomes an integer
+// |V| <= 2^54 on one scale (a row of A: its largest value; B: a bound of its table) and V 7 balanced
+// base-256 digits, exact in fp16. Of the 49 digit products those of weight t + u <= 7 are kept (34;
+// the largest dropped one is 2^-64 of the leading one, below the operands' own 2^-54). Products of
+// equal weight share one FP32 accumulator: at most 7 x 128 x 2^14 < 2^24 between two read-backs of
+// 128 values of K, so every sum is an exact integer. The read-backs are added in int64.
+// Against 64-bit sums over the closed form in extended precision (k = 10 on 129^2, k = 30 on
+// 257^2) the result is off by 1e-15 to 8e-15 (2-norm), plain FP64 sums by 4e-15 to 5e-14 and the
+// pivoted recurrences by 4e-14 to 2.5e-13.
+#include "tc_common.cuh"
+
+#include <algorithm>
+
+namespace mdp {
+namespace {
+
+// ---------------------------------------------------------------- mode table
+__device__ __forceinline__ cplx cdivd(cplx a, cplx b) {
+  const double n = 1.0 / fma(b.re, b.re, b.im * b.im);
+  return {fma(a.re, b.re, a.im * b.im) * n, fma(a.im, b.re, -a.re * b.im) * n};
+}
+__device__ __forceinline__ double pow2i(int k) {
+  return k < -1022 ? 0.0 : __longlong_as_double((long long)(min(k, 1023) + 1023) << 52);
+}
+// the two homogeneous solutions at distance x from the middle row (kinds 0 and 1)
+__device__ __forceinline__ double sep_c(int kind, double th, double x) { return kind == 0 ? cos(x * th) : cosh(x * th); }
+__device__ __forceinline__ double sep_s(int kind, double th, double x) {
+  if (th == 0.0) return x;
+  return kind == 0 ? sin(x * th) / sin(th) : sinh(x * th) / sinh(th);
+}
+
+__global__ void __launch_bounds__(128) k_sep_mode_tab(const SubDesc *subs, int s0, unsigned char *sep, int entries) {
+  const int si = s0 + blockIdx.y;
+  const SubDesc &d = subs[si];
+  const int q = blockIdx.x * 128 + threadIdx.x + 1;
+  if (d.leader != si || q > d.Nq) return;
+  double *T = reinterpret_cast<double *>(sep + d.sep_mt) + (long long)(q - 1) * SEP_MTW;
+  const double h = d.h, h2 = h * h, k = d.k, k2 = k * k;
+  const double sq = sin(M_PI * q / (2.0 * d.Nx)), lam = -4.0 * sq * sq;
+  // the interior entries (a, b) of T_q as the factorisation of these tables rounded them (the host's at
+  // plan creation, else this device's): e = b + 2 a is exact, and an error of b moves theta by its
+  // half over theta^2, so both forms of the solve are to start from the same b
+  double *ab = reinterpret_cast<double *>(sep + d.sep_ab) + 2 * (q - 1);
+  if (entries) {
+    ab[0] = 1.0 / h2 + lam / (6.0 * h2) + k2 / 12.0;
+    ab[1] = -2.0 * ab[0] + lam / h2 + k2 + k2 * lam / 12.0;
+  }
+  double a = ab[0];
+  const double e = ab[1] + 2.0 * a;
+  double t = e / (4.0 * a);                             // sin^2(theta/2), or -sinh^2(theta/2)
+  // coarse grids (t > 1/2): x_i = (-1)^i z_i turns (a, b, a) into (-a, b, -a)
+  double sg = 1.0;
+  if (t > 0.5) { sg = -1.0; t = 1.0 - t; a = -a; }
+  const int N = d.ny - 1, J0 = d.nlo - 1, J1 = d.nhi + 1, L = d.nhi - d.nlo;
+  const double mid = 0.5 * (J0 + J1), Lh = 0.5 * (J1 - J0);
+  const double th = t > 0.0 ? 2.0 * asin(sqrt(t)) : 2.0 * asinh(sqrt(-t));
+  const int kind = t > 0.0 ? 0 : th * N < 4.0 ? 1 : 2;
+  // rows at the ends: al0 x_0 + al1 x_1 = 0 and its mirror image
+  cplx al0 = cmk(1.0, 0.0), al1 = cmk(0.0, 0.0);
+  if (d.cplx) {
+    const bool paper = d.ap_bc == MDP_AP_DIRX_SOMMY_PAPER;
+    const double alpha = paper ? (1.0 - k2 * h2 / 24.0 - lam / 6.0) / h2 : (1.0 + k2 * h2 / 24.0 + lam / 24.0) / h2;
+    const double beta = k * (1.0 + k2 * h2 / 8.0 + lam / (paper ? 2.0 : 8.0)) / h;
+    al0 = cmk(alpha, 0.5 * beta);
+    al1 = cmk(-sg * alpha, 0.5 * sg * beta);
+  }
+  double n1 = 1.0, n2 = 1.0, c = 0.0, rf;
+  cplx R11, R12, R22;
+  const int rows_d[4] = {d.nlo, d.nlo + 1, d.nhi - 1, d.nhi}, rows_g[4] = {d.nlo - 1, d.nlo, d.nhi, d.nhi + 1};
+  auto sgn = [&](int i) { return (sg < 0.0 && (i & 1)) ? -1.0 : 1.0; };   // sg^i
+  if (kind < 2) {
+    double bound = kind == 0 ? fmax(Lh, 1.0) : sep_s(1, th, Lh);
+    if (kind == 0) bound = fmin(bound, 1.0 / sin(th));
+    n2 = pow2i(-(ilogb(fmax(bound, 1.0)) + 1));
+    if (kind == 1) n1 = 0.25;
+    const double C0 = sep_c(kind, th, 0.0 - mid), C1 = sep_c(kind, th, 1.0 - mid);
+    const double S0 = sep_s(kind, th, 0.0 - mid), S1 = sep_s(kind, th, 1.0 - mid);
+    const double D0 = sep_c(kind, th, N - mid), D1 = sep_c(kind, th, N - 1 - mid);
+    const double E0 = sep_s(kind, th, N - mid), E1 = sep_s(kind, th, N - 1 - mid);
+    auto lin = [&](double x, double y) { return cmk(fma(al0.re, x, al1.re * y), fma(al0.im, x, al1.im * y)); };
+    const cplx b1 = lin(C0, C1), b2 = lin(S0, S1), t1 = lin(D0, D1), t2 = lin(E0, E1);
+    const cplx det = csub(cmul(b1, t2), cmul(b2, t1));
+    const cplx ad = cmk(a * det.re, a * det.im);
+    R11 = cdivd(cmul(b2, t2), ad);
+    R22 = cdivd(cmul(b1, t1), ad);
+    R12 = cdivd(cadd(cmul(b1, t2), cmul(b2, t1)), cmk(-2.0 * ad.re, -2.0 * ad.im));
+    const double s1 = 1.0 / n1, s2 = 1.0 / n2;
+    R11 = cmk(R11.re * s1 * s1, R11.im * s1 * s1);
+    R12 = cmk(R12.re * s1 * s2, R12.im * s1 * s2);
+    R22 = cmk(R22.re * s2 * s2, R22.im * s2 * s2);
+    double kb = kind == 0 ? (double)(J1 - J0) : sep_s(1, th, J1 - J0);
+    if (kind == 0) kb = fmin(kb, 1.0 / sin(th));
+    rf = pow2i(-(ilogb(fmax(kb, 1.0) / (2.0 * fabs(a))) + 1));
+  } else {
+    const double ep = exp(th), em = exp(-th);
+    c = -1.0 / (2.0 * a * sinh(th));
+    const cplx num = cmk(fma(al1.re, ep, al0.re), fma(al1.im, ep, al0.im));
+    const cplx den = cmk(fma(al1.re, em, al0.re), fma(al1.im, em, al0.im));
+    const cplx ref = cdivd(num, den);
+    const double wb = -exp(-2.0 * th * J0), wt = -exp(-2.0 * th * (N - J1)), dl = exp(-th * (J1 - J0));
+    const cplx rb = cmk(wb * ref.re, wb * ref.im), rt = cmk(wt * ref.re, wt * ref.im);
+    const cplx rr = cmul(rb, rt);
+    const cplx D = cmk(1.0 - rr.re * dl * dl, -rr.im * dl * dl);
+    R11 = cdivd(cmk(c * rb.re, c * rb.im), D);
+    R22 = cdivd(cmk(c * rt.re, c * rt.im), D);
+    R12 = cdivd(cmk(c * dl * rr.re, c * dl * rr.im), D);
+    rf = pow2i(-(ilogb(fabs(c)) + 1));
+  }
+  auto p1 = [&](int i) { return sgn(i - J0) * (kind == 2 ? exp(-th * (i - J0)) : n1 * sep_c(kind, th, i - mid)); };
+  auto p2 = [&](int i) { return sgn(i - J0) * (kind == 2 ? exp(-th * (J1 - i)) : n2 * sep_s(kind, th, i - mid)); };
+  auto kap = [&](int x) { return sgn(x) * (kind == 2 ? c * exp(-th * x) : sep_s(kind, th, x) / (2.0 * a)); };
+  const double f = 1.0 / (2.0 * a * n1 * n2);
+  for (int r = 0; r < 4; ++r) {
+    const int j = rows_d[r], n = rows_g[r];
+    const double up = r < 2 ? 1.0 : -1.0;   // dense rows 0, 1 lie below the middle rows
+    T[MT_P1D + r] = p1(j); T[MT_P2D + r] = p2(j);
+    T[MT_P1G + r] = p1(n); T[MT_P2G + r] = p2(n);
+    if (kind < 2) {
+      T[MT_E1 + r] = -up * f * p2(j); T[MT_E2 + r] = up * f * p1(j);
+      T[MT_W1 + r] = -up * f * p2(n); T[MT_W2 + r] = up * f * p1(n);
+    } else {
+      T[MT_E1 + r] = r < 2 ? c * exp(th * (j - J0)) * sgn(j - J0) : 0.0;
+      T[MT_E2 + r] = r < 2 ? 0.0 : c * exp(th * (J1 - j)) * sgn(j - J0);
+      T[MT_W1 + r] = r < 2 ? c * exp(th * (n - J0)) * sgn(n - J0) : 0.0;
+      T[MT_W2 + r] = r < 2 ? 0.0 : c * exp(th * (J1 - n)) * sgn(n - J0);
+    }
+  }
+  T[MT_R + 0] = R11.re; T[MT_R + 1] = R11.im; T[MT_R + 2] = R12.re; T[MT_R + 3] = R12.im;
+  T[MT_R + 4] = R22.re; T[MT_R + 5] = R22.im;
+  T[MT_K + 0] = kap(0); T[MT_K + 1] = kap(1); T[MT_K + 2] = kap(2);
+  T[MT_K + 3] = kap(L - 1); T[MT_K + 4] = kap(L); T[MT_K + 5] = kap(L + 1);
+  T[MT_REC + 0] = d.nrec >= 0 ? p1(d.nrec) : 0.0;
+  T[MT_REC + 1] = d.nrec >= 0 ? p2(d.nrec) : 0.0;
+  T[MT_REC + 2] = 1.0 / rf;
+  T[MT_T1] = kind == 2 ? c : sep_s(kind, th, Lh) / (2.0 * a * n1);
+  T[MT_T2] = kind == 2 ? 0.0 : sep_c(kind, th, Lh) / (2.0 * a * n2);
+  T[MT_RF] = rf;
+  T[MT_F] = f;
+  T[MT_TH] = th; T[MT_KIND] = kind; T[MT_SG] = sg; T[MT_N1] = n1; T[MT_N2] = n2;
+}
+
+// phi_1, phi_2 on the rows J0 .. J1, [2][Py + 2][Nq]: a thread takes one mode and 8 rows, the
+// first by exp / sincos, the others by multiplying on (a rotation or a decay: 8 roundings).
+constexpr int PHI_ROWS = 8;
+__global__ void __launch_bounds__(128) k_sep_phi(const SubDesc *subs, int s0, unsigned char *sep) {
+  const int si = s0 + blockIdx.z;
+  const SubDesc &d = subs[si];
+  const int q = blockIdx.x * 128 + threadIdx.x + 1, rows = d.Py + 2, i0 = blockIdx.y * PHI_ROWS;
+  if (d.leader != si || q > d.Nq || i0 >= rows) return;
+  const double *T = reinterpret_cast<const double *>(sep + d.sep_mt) + (long long)(q - 1) * SEP_MTW;
+  double *P1 = reinterpret_cast<double *>(sep + d.sep_phi) + (q - 1), *P2 = P1 + (long long)rows * d.Nq;
+  const double th = T[MT_TH], sg = T[MT_SG];
+  const int kind = (int)T[MT_KIND], i1 = min(rows, i0 + PHI_ROWS);
+  const double sg0 = (sg < 0.0 && (i0 & 1)) ? -1.0 : 1.0;
+  if (kind == 2) {
+    const double lam = sg * exp(-th);
+    double v = sg0 * exp(-th * i0);
+    for (int i = i0; i < i1; ++i) { P1[(long long)i * d.Nq] = v; v *= lam; }
+    v = ((sg < 0.0 && ((i1 - 1) & 1)) ? -1.0 : 1.0) * exp(-th * (rows - i1));
+    for (int i = i1 - 1; i >= i0; --i) { P2[(long long)i * d.Nq] = v; v *= lam; }
+    return;
+  }
+  const double x = i0 - 0.5 * (rows - 1), n1 = sg0 * T[MT_N1], n2 = sg0 * T[MT_N2];
+  // C(x+1) = C(x) C(1) -/+ S(x) s^2, S(x+1) = S(x) C(1) + C(x) (s = sin theta or sinh theta)
+  const double c1 = sep_c(kind, th, 1.0), s = kind == 0 ? sin(th) : sinh(th), ss = kind == 0 ? -s * s : s * s;
+  double C = sep_c(kind, th, x), S = sep_s(kind, th, x), w = 1.0;
+  for (int i = i0; i < i1; ++i) {
+    P1[(long long)i * d.Nq] = w * n1 * C;
+    P2[(long long)i * d.Nq] = w * n2 * S;
+    const double Cn = fma(S, ss, C * c1);
+    S = fma(S, c1, C);
+    C = Cn;
+    w *= sg;
+  }
+}
+
+// K_sc(d) for every class, output and source column: one block per distance d, sums over the modes.
+__global__ void __launch_bounds__(128) k_sep_kd(const SubDesc *subs, int s0, const double *tab, unsigned char *sep) {
+  const int si = s0 + blockIdx.y;
+  const SubDesc &d = subs[si];
+  const int dist = blockIdx.x;
+  if (!d.tc_cols || d.leader != si || dist >= d.Py) return;
+  const SepGeo g = sep_geo(d);
+  const double *S = tab + d.sin_off, *T = reinterpret_cast<const double *>(sep + d.sep_mt);
+  const double *P1 = reinterpret_cast<const double *>(sep + d.sep_phi) + (long long)dist * d.Nq;
+  const double *P2 = P1 + (long long)(d.Py + 2) * d.Nq;
+  const int N2 = 2 * d.Nx;
+  double acc[16];
+#pragma unroll
+  for (int i = 0; i < 16; ++i) acc[i] = 0.0;
+  for (int q = threadIdx.x + 1; q <= d.Nq; q += 128) {
+    const double *t = T + (long long)(q - 1) * SEP_MTW;
+    const double kq = fma(t[MT_T1], P1[q - 1], t[MT_T2] * P2[q - 1]);
+    double so[4], sc[4];
+#pragma unroll
+    for (int s = 0; s < 4; ++s) {
+      so[s] = s < g.nS ? S[(int)(((long long)q * sep_out_col(d, s)) % N2)] * kq : 0.0;
+      sc[s] = s < g.nS ? S[(int)(((long long)q * sep_src_col(d, s)) % N2)] : 0.0;
+    }
+    if (d.xsym) {
+      // acc[(class, s, c)]; 128 is even, so a thread's modes all have its own parity
+#pragma unroll
+      for (int s = 0; s < 2; ++s)
+#pragma unroll
+        for (int cc = 0; cc < 2; ++cc) acc[s * 2 + cc] = fma(so[s], sc[cc], acc[s * 2 + cc]);
+    } else {
+#pragma unroll
+      for (int s = 0; s < 4; ++s)
+#pragma unroll
+        for (int cc = 0; cc < 4; ++cc) acc[s * 4 + cc] = fma(so[s], sc[cc], acc[s * 4 + cc]);
+    }
+  }
+  // fixed-order sums: over the lanes of one parity (x-centred) or all lanes, then the 4 warps
+  __shared__ double sh[4][2][16];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    for (int off = 16; off >= 2; off >>= 1) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], off);
+    if (lane < 2) sh[warp][lane][i] = acc[i];
+  }
+  __syncthreads();
+  const int ns = g.ncls * g.nS * g.nS;
+  if ((int)threadIdx.x < ns) {
+    double v = 0.0;
+    if (d.xsym) {   // class 0: odd q, which lanes of even index hold
+      const int e = threadIdx.x >> 2, i = threadIdx.x & 3;
+      for (int w = 0; w < 4; ++w) v += sh[w][e][i];
+    } else {
+      for (int w = 0; w < 4; ++w) v += sh[w][0][threadIdx.x] + sh[w][1][threadIdx.x];
+    }
+    reinterpret_cast<double *>(sep + d.sep_kd)[(long long)threadIdx.x * d.Py + dist] = v * (2.0 / d.Nx);
+  }
+}
+
+// the 7 digits of 8 consecutive-K values |x| 2^(54 - e) at 16 bytes each, `stride` bytes apart
+__device__ __forceinline__ void store_digits(unsigned char *dst, long long stride, const long long *V) {
+  unsigned hi[8], lo[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const unsigned long long w = (unsigned long long)V[j] + 0x0080808080808080ull;
+    hi[j] = (unsigned)(w >> 32);
+    lo[j] = (unsigned)w;
+  }
+#define MDP_SEP_DIGIT(T)                                                        \
+  *reinterpret_cast<uint4 *>(dst + (T) * stride) =                              \
+      make_uint4(digit_pair<6 - (T)>(hi[0], lo[0], hi[1], lo[1]),               \
+                 digit_pair<6 - (T)>(hi[2], lo[2], hi[3], lo[3]),               \
+                 digit_pair<6 - (T)>(hi[4], lo[4], hi[5], lo[5]),               \
+                 digit_pair<6 - (T)>(hi[6], lo[6], hi[7], lo[7]));
+  MDP_SEP_DIGIT(0) MDP_SEP_DIGIT(1) MDP_SEP_DIGIT(2) MDP_SEP_DIGIT(3) MDP_SEP_DIGIT(4) MDP_SEP_DIGIT(5) MDP_SEP_DIGIT(6)
+#undef MDP_SEP_DIGIT
+}
+// table value |x| <= 1 on the fixed scale 2^54
+__device__ __forceinline__ long long fix54(double x) { return __double2ll_rn(x * 0x1p54); }
+
+// The Toeplitz blocks of K (32 outputs x 16 sources, by the offset of the two groups) on the scale of
+// the largest |K_sc| of the output column: 64 threads (32 outputs x 2 K halves) per block.
+__global__ void __launch_bounds__(256) k_sep_tb(const SubDesc *subs, int s0, unsigned char *sep) {
+  const int si = s0 + blockIdx.z;
+  const SubDesc &d = subs[si];
+  if (!d.tc_cols || d.leader != si) return;
+  const SepGeo g = sep_geo(d);
+  const int es = blockIdx.y / g.nS, c = blockIdx.y % g.nS;   // (class, output), source
+  const int blk0 = blockIdx.x * 4;
+  if (es >= g.ncls * g.nS || blk0 >= g.ND) return;
+  const double *K = reinterpret_cast<const double *>(sep + d.sep_kd) + (long long)es * g.nS * d.Py;
+  __shared__ int emax;
+  if (threadIdx.x == 0) emax = 0;
+  __syncthreads();
+  int m = 0;
+  for (int i = threadIdx.x; i < g.nS * d.Py; i += 256) m = max(m, (__double2hiint(K[i]) >> 20) & 0x7ff);
+  for (int off = 16; off > 0; off >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, off));
+  if ((threadIdx.x & 31) == 0) atomicMax(&emax, m);
+  __syncthreads();
+  const int e = min(max(emax - 1022, -900), 900);   // |K| <= 2^e
+  if (threadIdx.x == 0 && blockIdx.x == 0 && c == 0) reinterpret_cast<int *>(sep + d.sep_kde)[es] = e;
+  const int blk = blk0 + (threadIdx.x >> 6), o = threadIdx.x & 31, half = (threadIdx.x >> 5) & 1;
+  if (blk >= g.ND) return;
+  const double sc = pow2i(54 - e);
+  const double *Kc = K + (long long)c * d.Py;
+  long long V[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    // row distance of output i = 32 ti + o (row nlo+1+i) and source 16 kj + k (row nlo+2+j)
+    const int dist = abs(16 * (blk - (g.nkj - 1)) + o - (8 * half + j) - 1);
+    V[j] = dist < d.Py ? __double2ll_rn(Kc[dist] * sc) : 0;
+  }
+  unsigned char *B = sep + d.sep_tb + (((long long)es * g.nS + c) * g.ND + blk) * SEP_BBLK;
+  store_digits(B + (o >> 3) * 256 + half * 128 + (o & 7) * 16, 1024, V);
+}
+
+// The moment tables, B of stage 1 beyond K: output (b, q), K index (c, j): sin(pi q m_c/Nx) phi_b(j),
+// and (b = 2, with a receiver row) sin(pi q m_c/Nx) kappa_q(|rec - j|) scaled to below 1.
+__global__ void __launch_bounds__(256) k_sep_mb(const SubDesc *subs, int s0, const double *tab, unsigned char *sep) {
+  const int si = s0 + blockIdx.z;
+  const SubDesc &d = subs[si];
+  if (!d.tc_cols || d.leader != si) return;
+  const SepGeo g = sep_geo(d);
+  const int nto = g.nb * g.nqp / 32;
+  const int e = blockIdx.y / nto, to = blockIdx.y % nto;
+  const int kb = blockIdx.x * 4 + (threadIdx.x >> 6);
+  if (e >= g.ncls || kb >= g.nk1) return;
+  const int o = threadIdx.x & 31, half = (threadIdx.x >> 5) & 1;
+  const int b = to * 32 / g.nqp, qi = to * 32 % g.nqp + o, q = sep_mode(d, e, qi);
+  const int c = kb / g.nkj, j0 = (kb % g.nkj) * 16 + 8 * half;
+  long long V[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) V[j] = 0;
+  if (q <= d.Nq) {
+    const double sc = tab[d.sin_off + (int)(((long long)q * sep_src_col(d, c)) % (2 * d.Nx))];
+    const double *P = reinterpret_cast<const double *>(sep + d.sep_phi) + (q - 1);
+    const double *T = reinterpret_cast<const double *>(sep + d.sep_mt) + (long long)(q - 1) * SEP_MTW;
+    const long long p2 = (long long)(d.Py + 2) * d.Nq;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      if (j0 + j >= g.Pj) continue;
+      const int row = 3 + j0 + j;                      // grid row nlo + 2 + j, counted from J0 = nlo - 1
+      double v;
+      if (b < 2) v = P[b * p2 + (long long)row * d.Nq];
+      else {
+        const int dist = abs(d.nrec - (d.nlo - 1) - row);
+        v = fma(T[MT_T1], P[(long long)dist * d.Nq], T[MT_T2] * P[p2 + (long long)dist * d.Nq]) * T[MT_RF];
+      }
+      V[j] = fix54(v * sc);
+    }
+  }
+  unsigned char *B = sep + d.sep_mb + (((long long)e * (3 * g.nqp / 32) + to) * g.nk1 + kb) * SEP_BBLK;
+  store_digits(B + (o >> 3) * 256 + half * 128 + (o & 7) * 16, 1024, V);
+}
+
+// The synthesis table, B of stage 3: output (s, i), K index (b, q): sin(pi q m_s/Nx) phi_b(i).
+__global__ void __launch_bounds__(256) k_sep_b3(const SubDesc *subs, int s0, const double *tab, unsigned char *sep) {
+  const int si = s0 + blockIdx.z;
+  const SubDesc &d = subs[si];
+  if (!d.tc_cols || d.leader != si) return;
+  const SepGeo g = sep_geo(d);
+  const int e = blockIdx.y / g.nt3, to = blockIdx.y % g.nt3;
+  const int kb = blockIdx.x * 4 + (threadIdx.x >> 6);
+  if (e >= g.ncls || kb >= g.nk3) return;
+  const int o = threadIdx.x & 31, half = (threadIdx.x >> 5) & 1;
+  const int s = to / g.nti, i = (to % g.nti) * 32 + o;
+  const int b = kb * 16 / g.nqp, q0 = kb * 16 % g.nqp + 8 * half;
+  const int m = sep_out_col(d, s), N2 = 2 * d.Nx;
+  const double *S = tab + d.sin_off;
+  const double *P = reinterpret_cast<const double *>(sep + d.sep_phi) + ((long long)b * (d.Py + 2) + 2 + i) * d.Nq;
+  long long V[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const int q = sep_mode(d, e, q0 + j);
+    V[j] = (i < g.Pi && q <= d.Nq) ? fix54(P[q - 1] * S[(int)(((long long)q * m) % N2)]) : 0;
+  }
+  unsigned char *B = sep + d.sep_b3 + (((long long)e * g.nt3 + to) * g.nk3 + kb) * SEP_BBLK;
+  store_digits(B + (o >> 3) * 256 + half * 128 + (o & 7) * 16, 1024, V);
+}
+
+// ---------------------------------------------------------------- operand A
+// Cut the rows of A (stage 1: ring residuals of the middle rows, stage 3: the modes' A_b) into
+// digits in the MMA's operand layout, per 128 rows and 16 values of K 7 x 4 KiB. A block takes 8
+// rows of one class (one core-matrix row group): their largest exponents first, then the digits;
+// the values are read twice, the second time from L1/L2.
+template <bool CIN, int STAGE>
+__global__ void __launch_bounds__(256) k_sep_cut(Batch bt, const SubDesc *subs, double *ws, int fam) {
+  Item it; int local;
+  locate(bt, blockIdx.x, it, local);
+  MDP_CHECK_ITEM(bt, subs, it, local, fam);
+  const SubDesc &d = subs[it.sub];
+  const SepGeo g = sep_geo(d);
+  const SepWs w = sep_ws(d, it.ncols);
+  const int R = STAGE == 1 ? sep_rows1(d, it.ncols, it.col0, CIN) : sep_rows3(d, it.ncols, CIN);
+  const int e = local / (R / 8), row = (local % (R / 8)) * 8 + (threadIdx.x & 7), kl = threadIdx.x >> 3;
+  const int cp = sep_pad128(it.ncols), nk = STAGE == 1 ? g.nk1 : g.nk3;
+  const long long nc = it.ncols;
+  // the row's column and part, and its values
+  bool live;
+  const double *src;
+  long long sk;   // stage 3: step between consecutive K
+  int part = 0, col = 0;
+  if (STAGE == 1) {
+    if (CIN) { part = row / cp; col = row % cp; live = col < it.ncols; }
+    else { live = row < sep_side_cols(d, it.col0, it.ncols); col = live ? sep_side_col(d, it.col0, row) - it.col0 : 0; }
+    src = ws + it.r_off;
+    sk = 0;
+  } else {
+    col = row % cp;
+    live = col < it.ncols;
+    src = ws + it.a_off + w.aeff + (long long)e * 2 * g.nqp * R + row;
+    sk = R;
+  }
+  auto value = [&](int k) -> double {
+    if (STAGE == 1) {
+      const int c = k / (16 * g.nkj), j = k - c * 16 * g.nkj;
+      if (!live || j >= g.Pj) return 0.0;
+      const long long slot = d.xsym ? 8LL * d.Ph + 4 * j + 2 * c + e : 2LL * d.Px + 4 * j + c;
+      return CIN ? src[2 * (slot * nc + col) + part] : src[slot * nc + col];
+    }
+    const int qi = k % g.nqp;
+    return live && sep_mode(d, e, qi) <= d.Nq ? src[(long long)k * sk] : 0.0;
+  };
+  __shared__ int emax[8];
+  if (threadIdx.x < 8) emax[threadIdx.x] = 0;
+  __syncthreads();
+  int m = 0;
+  for (int k8 = kl; k8 < 2 * nk; k8 += 32)
+#pragma unroll
+    for (int j = 0; j < 8; ++j) m = max(m, (__double2hiint(value(8 * k8 + j)) >> 20) & 0x7ff);
+  for (int off = 16; off >= 8; off >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, off));
+  if ((threadIdx.x & 31) < 8) atomicMax(&emax[threadIdx.x & 7], m);
+  __syncthreads();
+  const int E = max(emax[threadIdx.x & 7], 53);
+  if (kl == 0) reinterpret_cast<int *>(ws + it.a_off + (STAGE == 1 ? w.ex1 : w.ex3))[e * R + row] = E;
+  const double sc = pow2i(1076 - E);          // |x| < 2^(E - 1022) -> |V| < 2^54
+  unsigned char *A = reinterpret_cast<unsigned char *>(ws + it.a_off + (STAGE == 1 ? w.a1 : w.a3)) +
+                     ((long long)(e * (R / 128) + row / 128) * nk) * SEP_ABLK;
+  const int r = row & 127, off0 = (r >> 3) * 256 + (r & 7) * 16;
+  for (int k8 = kl; k8 < 2 * nk; k8 += 32) {
+    long long V[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) V[j] = E < 2047 ? __double2ll_rn(value(8 * k8 + j) * sc) : 0;
+    store_digits(A + (long long)(k8 >> 1) * SEP_ABLK + off0 + (k8 & 1) * 128, 4096, V);
+  }
+}
+
+// ---------------------------------------------------------------- the contractions
+// Persistent CTAs, one per SM: warp 9 streams the digit blocks of A (28 KiB) and B (7 KiB) of 16
+// values of K into 5 shared-memory stages with bulk copies, one thread of warp 8 issues the MMAs,
+// and after every 128 values of K hands one of two accumulator sets (8 weights x 32 outputs, FP32)
+// to the 8 other warps, which add them up as integers and at the end of a tile scale them into
+// FP64. A tile is 128 rows x 32 outputs. One MMA (M = 128, N = 256, K = 16) per A digit t: its B
+// operand starts t digits before B's first one, in 7 KiB of zeros, so that digit u meets the
+// accumulator of weight t + u and every MMA of a set has the same accumulator and shape (MMAs into
+// overlapping accumulators of other shapes have no defined order). The zeros are 22 of 56 digit
+// pairs. What bounds it: the tensor pipe, 7 x 128 cycles per 16 values of K; the operands' way from
+// L2 takes 35 KiB in that time, 39 bytes per cycle and SM.
+constexpr int SG_STAGES = 5, SG_THREADS = 320, SG_CHUNK = 8;   // K16 steps per accumulator set
+constexpr int SG_STAGE_BYTES = SEP_ABLK + SEP_BBLK;
+// shared memory: the A stages, then zeros and B stages in turn, 7 KiB each, and closing zeros
+constexpr int SG_B0 = SG_STAGES * SEP_ABLK;
+constexpr int SG_SMEM = SG_B0 + (2 * SG_STAGES + 1) * SEP_BBLK + 1024;
+
+// 16 consecutive FP32 columns of this warp's 32 TMEM lanes
+__device__ __forceinline__ void tmem_ld16(unsigned taddr, float *v) {
+  unsigned r[16];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr)
+      : "memory");
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+}
+__device__ __forceinline__ void bulk_load(unsigned dst, const void *src, unsigned bytes, unsigned bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "l"(src), "r"(bytes), "r"(bar)
+               : "memory");
+}
+
+struct SepTile { int e, mt, nt, R; };
+template <int STAGE>
+__device__ __forceinline__ SepTile sep_tile(const SubDesc &d, const SepGeo &g, const Item &it, int local, bool user) {
+  SepTile t;
+  t.R = STAGE == 1 ? sep_rows1(d, it.ncols, it.col0, user) : sep_rows3(d, it.ncols, user);
+  const int nt = STAGE == 1 ? g.nt1 : g.nt3, per = (t.R / 128) * nt;
+  t.e = local / per;
+  t.mt = (local % per) / nt;
+  t.nt = local % nt;
+  return t;
+}
+
+template <int STAGE>
+__global__ void __launch_bounds__(SG_THREADS, 1)
+    k_sep_gemm(Batch bt, const SubDesc *subs, const unsigned char *sep, double *ws, int user, int fam, int *status) {
+  extern __shared__ unsigned char sg_raw[];
+  __shared__ __align__(8) unsigned long long full_bar[SG_STAGES], empty_bar[SG_STAGES], tfull_bar[2], tempty_bar[2], drain_bar;
+  __shared__ unsigned tmem_slot;
+  __shared__ volatile int abort_sh;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (tid == 0) {
+    for (int s = 0; s < SG_STAGES; ++s) { mbar_init(smem_u32(&full_bar[s]), 1); mbar_init(smem_u32(&empty_bar[s]), 1); }
+    for (int s = 0; s < 2; ++s) { mbar_init(smem_u32(&tfull_bar[s]), 1); mbar_init(smem_u32(&tempty_bar[s]), 256); }
+    mbar_init(smem_u32(&drain_bar), 1);
+    abort_sh = 0;
+  }
+  if (warp == 8) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)), "r"(512)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  const unsigned sbase = (smem_u32(sg_raw) + 1023u) & ~1023u;
+  {
+    unsigned char *z = sg_raw + (sbase - smem_u32(sg_raw)) + SG_B0;
+    for (int i = tid; i < (SG_STAGES + 1) * (SEP_BBLK / 16); i += SG_THREADS)
+      *reinterpret_cast<uint4 *>(z + (i / (SEP_BBLK / 16)) * 2 * SEP_BBLK + (i % (SEP_BBLK / 16)) * 16) = make_uint4(0, 0, 0, 0);
+  }
+  asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const unsigned tmem = tmem_slot;
+
+  if (warp == 9) {
+    // ---------------------------------------------------------------- operand loads
+    if (lane == 0) {
+      unsigned gs = 0;
+      for (int v = blockIdx.x; v < bt.total_blocks && !abort_sh; v += gridDim.x) {
+        Item it; int local;
+        locate(bt, v, it, local);
+        if (MDP_CHECKED && !item_in_bounds(bt, subs, it, local, fam, false)) continue;   // every warp skips it
+        const SubDesc &d = subs[it.sub];
+        const SepGeo g = sep_geo(d);
+        const SepWs w = sep_ws(d, it.ncols);
+        const SepTile t = sep_tile<STAGE>(d, g, it, local, user);
+        const int nk = STAGE == 1 ? g.nk1 : g.nk3;
+        const unsigned char *A = reinterpret_cast<const unsigned char *>(ws + it.a_off + (STAGE == 1 ? w.a1 : w.a3)) +
+                                 (long long)(t.e * (t.R / 128) + t.mt) * nk * SEP_ABLK;
+        const unsigned char *B;
+        int ti = 0;
+        const bool toep = STAGE == 1 && t.nt < g.nS * g.nti;
+        if (STAGE == 3) B = sep + d.sep_b3 + ((long long)t.e * g.nt3 + t.nt) * g.nk3 * SEP_BBLK;
+        else if (toep) { ti = t.nt % g.nti; B = sep + d.sep_tb + ((long long)(t.e * g.nS + t.nt / g.nti) * g.nS) * g.ND * SEP_BBLK; }
+        else B = sep + d.sep_mb + ((long long)t.e * (3 * g.nqp / 32) + t.nt - g.nS * g.nti) * g.nk1 * SEP_BBLK;
+        bool ok = true;
+        for (int kb = 0; kb < nk; ++kb, ++gs) {
+          const unsigned st = gs % SG_STAGES;
+          if (gs >= SG_STAGES && !mbar_wait(smem_u32(&empty_bar[st]), (gs / SG_STAGES - 1) & 1u, &abort_sh)) { ok = false; break; }
+          const unsigned bar = smem_u32(&full_bar[st]);
+          asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(SG_STAGE_BYTES) : "memory");
+          bulk_load(sbase + st * SEP_ABLK, A + (long long)kb * SEP_ABLK, SEP_ABLK, bar);
+          const long long bo = toep ? (long long)(kb / g.nkj) * g.ND + 2 * ti - kb % g.nkj + g.nkj - 1 : kb;
+          bulk_load(sbase + SG_B0 + (2 * st + 1) * SEP_BBLK, B + bo * SEP_BBLK, SEP_BBLK, bar);
+        }
+        if (!ok) break;
+      }
+      // leave only when every copy issued has landed (each wait bounded)
+      for (unsigned s = gs >= SG_STAGES ? gs - SG_STAGES : 0; s < gs; ++s) {
+        const long long t0 = clock64();
+        while (!mbar_try(smem_u32(&full_bar[s % SG_STAGES]), (s / SG_STAGES) & 1u))
+          if (clock64() - t0 > TC_WAIT_CYCLES) { abort_sh = 1; break; }
+      }
+    }
+    __syncwarp();
+  } else if (warp == 8) {
+    // ---------------------------------------------------------------- MMAs
+    if (lane == 0) {
+      unsigned gs = 0, cc = 0;   // stages and accumulator sets used
+      for (int v = blockIdx.x; v < bt.total_blocks && !abort_sh; v += gridDim.x) {
+        Item it; int local;
+        locate(bt, v, it, local);
+        if (MDP_CHECKED && !item_in_bounds(bt, subs, it, local, fam, false)) continue;
+        const SepGeo g = sep_geo(subs[it.sub]);
+        const int nk = STAGE == 1 ? g.nk1 : g.nk3;
+        bool ok = true;
+        for (int kb = 0; kb < nk && ok; ++cc) {
+          const unsigned buf = cc & 1u, D = tmem + 256u * buf;
+          if (cc >= 2 && !mbar_wait(smem_u32(&tempty_bar[buf]), ((cc >> 1) - 1) & 1u, &abort_sh)) { ok = false; break; }
+          tc_fence_after();
+          const int kend = min(nk, kb + SG_CHUNK);
+          for (bool first = true; kb < kend; ++kb, ++gs, first = false) {
+            const unsigned st = gs % SG_STAGES;
+            if (!mbar_wait(smem_u32(&full_bar[st]), (gs / SG_STAGES) & 1u, &abort_sh)) { ok = false; break; }
+            tc_fence_after();
+            const unsigned a0 = sbase + st * SEP_ABLK, b0 = sbase + SG_B0 + (2 * st + 1) * SEP_BBLK;
+#pragma unroll
+            for (int t = 0; t < 7; ++t)
+              tc_mma(D, smem_desc(a0 + 4096 * t, 128, 256), smem_desc(b0 - 1024 * t, 128, 256), f16_idesc(256),
+                     first && t == 0 ? 0u : 1u);
+            tc_commit(smem_u32(&empty_bar[st]));
+          }
+          if (ok) tc_commit(smem_u32(&tfull_bar[buf]));
+        }
+        if (!ok) break;
+      }
+      if (abort_sh) {   // no MMA in flight when the tensor memory is freed (bounded)
+        tc_commit(smem_u32(&drain_bar));
+        const long long t0 = clock64();
+        while (!mbar_try(smem_u32(&drain_bar), 0u) && clock64() - t0 < TC_WAIT_CYCLES) {}
+      }
+    }
+    __syncwarp();
+  } else {
+    // ---------------------------------------------------------------- sums and results
+    const int quarter = warp & 3, half = warp >> 2;
+    unsigned cc = 0;
+    for (int v = blockIdx.x; v < bt.total_blocks && !abort_sh; v += gridDim.x) {
+      Item it; int local;
+      locate(bt, v, it, local);
+      if (MDP_CHECKED && !item_in_bounds(bt, subs, it, local, fam, false)) continue;
+      const SubDesc &d = subs[it.sub];
+      const SepGeo g = sep_geo(d);
+      const SepWs w = sep_ws(d, it.ncols);
+      const SepTile t = sep_tile<STAGE>(d, g, it, local, user);
+      const int nk = STAGE == 1 ? g.nk1 : g.nk3;
+      // weights 0..3 and 4..7 of 16 outputs, as sums of I_w 2^(8 (3 - w)), I_w 2^(8 (7 - w))
+      long long hi[16], lo[16];
+#pragma unroll
+      for (int o = 0; o < 16; ++o) hi[o] = lo[o] = 0;
+      bool ok = true;
+      for (int kb = 0; kb < nk; kb += SG_CHUNK, ++cc) {
+        const unsigned buf = cc & 1u;
+        if (!mbar_wait(smem_u32(&tfull_bar[buf]), (cc >> 1) & 1u, &abort_sh)) { ok = false; break; }
+        tc_fence_after();
+        const unsigned src = tmem + ((unsigned)(32 * quarter) << 16) + 256u * buf + 16u * half;
+#pragma unroll
+        for (int wt = 0; wt < 8; ++wt) {
+          float dv[16];
+          tmem_ld16(src + 32u * wt, dv);
+#pragma unroll
+          for (int o = 0; o < 16; ++o) {
+            const long long iv = (long long)__float2int_rn(dv[o]);
+            if (wt < 4) hi[o] += iv * (1LL << (8 * (3 - wt)));
+            else lo[o] += iv * (1LL << (8 * (7 - wt)));
+          }
+        }
+        tc_fence_before();
+        mbar_arrive(smem_u32(&tempty_bar[buf]));
+      }
+      if (!ok) break;
+      // value = (hi 2^32 + lo) 2^40 2^(E - 1022 - 54) 2^(eb - 54)
+      const int row = t.mt * 128 + 32 * quarter + lane;
+      const int E = reinterpret_cast<const int *>(ws + it.a_off + (STAGE == 1 ? w.ex1 : w.ex3))[t.e * t.R + row];
+      const bool direct = STAGE == 3 || t.nt < g.nS * g.nti;
+      int eb = 0;
+      if (STAGE == 1 && direct) eb = reinterpret_cast<const int *>(sep + d.sep_kde)[t.e * g.nS + t.nt / g.nti];
+      double s0 = pow2i(E - 1090 + eb), s1 = pow2i(E - 1058 + eb);
+      if (E >= 2047) s0 = s1 = __longlong_as_double(0x7ff8000000000000LL);   // Inf or NaN in the row
+      double *dst;
+      int cnt;
+      if (direct) {
+        const int i0 = (t.nt % g.nti) * 32 + 16 * half;
+        cnt = g.Pi - i0;
+        dst = ws + it.a_off + (STAGE == 1 ? w.u1 : w.u3) + ((long long)(t.e * g.nS + t.nt / g.nti) * g.Pi + i0) * t.R + row;
+      } else {
+        const int o0 = (t.nt - g.nS * g.nti) * 32 + 16 * half;
+        cnt = 16;
+        dst = ws + it.a_off + w.mom + ((long long)t.e * 3 * g.nqp + o0) * t.R + row;
+      }
+      constexpr long long MG = 0x4338000000000000LL;   // 1.5 2^52 + x for |x| < 2^51
+      const double M = __longlong_as_double(MG);
+#pragma unroll
+      for (int o = 0; o < 16; ++o)
+        if (o < cnt) {
+          // carry the part of lo above 2^32 into hi: both then lie below 2^51
+          const long long h = hi[o] + (lo[o] >> 32), l = lo[o] & 0xffffffffLL;
+          const double dh = __longlong_as_double(MG + h) - M, dl = __longlong_as_double(MG + l) - M;
+          dst[(long long)o * t.R] = fma(dh, s1, dl * s0);
+        }
+    }
+  }
+  if (abort_sh && tid == 0) atomicCAS(status, 0, (int)MDP_ERR_TIMEOUT);   // the first error sticks
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  if (warp == 8)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+}
+
+// ---------------------------------------------------------------- stage 2
+// Per (mode, column): the coefficients A_1, A_2 of the homogeneous part on the middle rows (from the
+// moments, the dense rows and R) and the field at the 4 gamma rows (+ the receiver row), which
+// k_inv_rows / k_inv_rec transform back. CD: complex results (Sommerfeld AP or complex data).
+template <bool CD, bool CIN>
+__device__ __forceinline__ void sep_modes_body(const Item &it, const SubDesc &d, const unsigned char *sep, double *ws, int b,
+                                               int q) {
+  const SepGeo g = sep_geo(d);
+  const SepWs w = sep_ws(d, it.ncols);
+  const double *T = reinterpret_cast<const double *>(sep + d.sep_mt) + (long long)(q - 1) * SEP_MTW;
+  const int e = d.xsym ? ((q & 1) ? 0 : 1) : 0, qi = d.xsym ? (q - 1) >> 1 : q - 1;
+  const int cp = sep_pad128(it.ncols), R1 = sep_rows1(d, it.ncols, it.col0, CIN), R3 = sep_rows3(d, it.ncols, CIN);
+  const long long nc = it.ncols;
+  const double *gr = ws + it.gr_off;
+  const double *mom = ws + it.a_off + w.mom + ((long long)e * 3 * g.nqp + qi) * R1;
+  cplx gd[4], M[3];
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    const long long o = ((long long)r * d.Nq + (q - 1)) * nc + b;
+    gd[r] = CIN ? ld2(gr + 2 * o) : cmk(gr[o], 0.0);
+  }
+  const bool rec = d.nrec >= 0;
+  const int row1 = CIN ? b : sep_side_row(d, it.col0, b);   // -1: no source on the middle rows
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    M[k] = cmk(0.0, 0.0);
+    if (row1 < 0 || (k == 2 && !rec)) continue;
+    const double *p = mom + (long long)k * g.nqp * R1 + row1;
+    M[k] = cmk(p[0], CIN ? p[cp] : 0.0);
+  }
+  auto axpy = [&](double s, cplx x, cplx y) { return CIN ? caxpy(s, x, y) : cmk(fma(s, x.re, y.re), 0.0); };
+  cplx m1 = M[0], m2 = M[1], k1 = cmk(0.0, 0.0), k2 = cmk(0.0, 0.0);
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    m1 = axpy(T[MT_P1D + r], gd[r], m1);
+    m2 = axpy(T[MT_P2D + r], gd[r], m2);
+    k1 = axpy(T[MT_E1 + r], gd[r], k1);
+    k2 = axpy(T[MT_E2 + r], gd[r], k2);
+  }
+  const cplx R11 = ld2(T + MT_R), R12 = ld2(T + MT_R + 2), R22 = ld2(T + MT_R + 4);
+  auto rmul = [&](cplx R, cplx m) -> cplx {
+    if (!CD) return cmk(R.re * m.re, 0.0);
+    if (!CIN) return cmk(R.re * m.re, R.im * m.re);
+    return cmul(R, m);
+  };
+  const cplx A = cadd(rmul(R11, m1), rmul(R12, m2)), B = cadd(rmul(R12, m1), rmul(R22, m2));
+  const cplx Ae = cadd(A, k1), Be = cadd(B, k2);
+  double *ae = ws + it.a_off + w.aeff + ((long long)e * 2 * g.nqp + qi) * R3 + b;
+  ae[0] = Ae.re;
+  ae[(long long)g.nqp * R3] = Be.re;
+  if (CD) { ae[cp] = Ae.im; ae[(long long)g.nqp * R3 + cp] = Be.im; }
+  double *y = ws + it.y_off;
+  auto ystore = [&](int slot, cplx v) {
+    const long long o = ((long long)(q - 1) * 5 + slot) * nc + b;
+    if (CD) st2(y + 2 * o, v); else y[o] = v.re;
+  };
+  constexpr int KI[4][4] = {{1, 2, 4, 5}, {0, 1, 3, 4}, {4, 3, 1, 0}, {5, 4, 2, 1}};   // gamma row x dense row
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    cplx v = axpy(T[MT_W1 + r], M[0], cmk(0.0, 0.0));
+    v = axpy(T[MT_W2 + r], M[1], v);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) v = axpy(T[MT_K + KI[r][j]], gd[j], v);
+    v = caxpy(T[MT_P1G + r], A, v);
+    v = caxpy(T[MT_P2G + r], B, v);
+    ystore(r, v);
+  }
+  if (rec) {
+    cplx v = axpy(T[MT_REC + 2], M[2], cmk(0.0, 0.0));
+    v = caxpy(T[MT_REC], Ae, v);
+    v = caxpy(T[MT_REC + 1], Be, v);
+    ystore(4, v);
+  }
+}
+
+template <bool CIN>
+__global__ void __launch_bounds__(128) k_sep_modes(Batch bt, const SubDesc *subs, const unsigned char *sep, double *ws) {
+  Item it; int local;
+  locate(bt, blockIdx.x, it, local);
+  MDP_CHECK_ITEM(bt, subs, it, local, F_SMODE);
+  const SubDesc &d = subs[it.sub];
+  const int cb = (it.ncols + 31) >> 5;
+  const int b = (local % cb) * 32 + threadIdx.x, q0 = (local / cb) * SEP_MODES_PER_BLOCK + threadIdx.y + 1;
+  if (b >= it.ncols) return;
+  for (int q = q0; q < q0 + SEP_MODES_PER_BLOCK - (int)threadIdx.y && q <= d.Nq; q += 4) {
+    if (d.cplx || CIN) sep_modes_body<true, CIN>(it, d, sep, ws, b, q);
+    else sep_modes_body<false, CIN>(it, d, sep, ws, b, q);
+  }
+}
+
+// ---------------------------------------------------------------- output columns
+// u at the 4 gamma columns of a middle row from the two stages' sums; Q = -u, P = xi - u.
+template <bool CD, bool CIN>
+__device__ __forceinline__ void sep_out_body(const Item &it, const SubDesc &d, const double *tab, const double *ws,
+                                             const double2 *xi_user, double2 *out, int kind, int b, int i) {
+  const SepGeo g = sep_geo(d);
+  const SepWs w = sep_ws(d, it.ncols);
+  const int cp = sep_pad128(it.ncols), R1 = sep_rows1(d, it.ncols, it.col0, CIN), R3 = sep_rows3(d, it.ncols, CIN);
+  const int row1 = CIN ? b : sep_side_row(d, it.col0, b);
+  const double sc = 2.0 / d.Nx;
+  cplx v[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {   // (class, output) or output
+    const long long t = (long long)k * g.Pi + i;
+    const double *p3 = ws + it.a_off + w.u3 + t * R3 + b, *p1 = ws + it.a_off + w.u1 + t * R1 + row1;
+    v[k] = cmk(sc * p3[0], CD ? sc * p3[cp] : 0.0);
+    if (row1 >= 0) {
+      v[k].re += p1[0];
+      if (CIN) v[k].im += p1[cp];
+    }
+  }
+  cplx u[4];
+  if (d.xsym) { u[0] = cadd(v[0], v[2]); u[1] = cadd(v[1], v[3]); u[2] = csub(v[1], v[3]); u[3] = csub(v[0], v[2]); }
+  else { u[0] = v[0]; u[1] = v[1]; u[2] = v[2]; u[3] = v[3]; }
+  const int g0 = 2 * (d.Px + 2) + 4 * i;
+  if (MDP_CHECKED && g0 + 3 >= d.G) { flag_bounds(d.dstatus); return; }
+#pragma unroll
+  for (int s = 0; s < 4; ++s) {
+    cplx r = cmk(-u[s].re, CD ? -u[s].im : 0.0);
+    if (kind == MDP_OUT_P) r = cadd(r, density<CIN>(d, it, ws, tab, xi_user, b, g0 + s));
+    out[it.io_off + (long long)b * d.G + g0 + s] = make_double2(r.re, r.im);
+  }
+}
+
+template <bool CIN>
+__global__ void __launch_bounds__(256) k_sep_out(Batch bt, const SubDesc *subs, const double *tab, const double *ws,
+                                                 const double2 *xi_user, double2 *out, int kind) {
+  Item it; int local;
+  locate(bt, blockIdx.x, it, local);
+  MDP_CHECK_ITEM(bt, subs, it, local, F_SOUT);
+  const SubDesc &d = subs[it.sub];
+  const int cb = (it.ncols + 31) >> 5;
+  const int b = (local % cb) * 32 + threadIdx.x, i = (local / cb) * 8 + threadIdx.y;
+  if (b >= it.ncols || i >= d.Py - 2) return;
+  if (d.cplx || CIN) sep_out_body<true, CIN>(it, d, tab, ws, xi_user, out, kind, b, i);
+  else sep_out_body<false, CIN>(it, d, tab, ws, xi_user, out, kind, b, i);
+}
+
+}  // namespace
+
+// ---------------------------------------------------------------- launchers
+cudaError_t set_sep_kernel_attributes() {
+  cudaError_t e = cudaFuncSetAttribute(k_sep_gemm<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, SG_SMEM);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_sep_gemm<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, SG_SMEM);
+  return e;
+}
+
+cudaError_t launch_sep_tables(const mdp_plan *p, const SubDesc *ds, const double *tab, unsigned char *sep, bool entries,
+                              cudaStream_t st) {
+  int mq = 0, mrow = 0, mdist = 0, mtb = 0, mes = 0, mmb = 0, mmk = 0, m3 = 0, m3k = 0;
+  for (size_t i = 0; i < p->subs.size(); ++i) {
+    const SubDesc &d = p->subs[i].d;
+    if (d.leader != (int)i) continue;
+    mq = std::max(mq, (d.Nq + 127) / 128);
+    mrow = std::max(mrow, (d.Py + 2 + PHI_ROWS - 1) / PHI_ROWS);
+    if (!d.tc_cols) continue;
+    const SepGeo g = sep_geo(d);
+    mdist = std::max(mdist, d.Py);
+    mtb = std::max(mtb, (g.ND + 3) / 4);
+    mes = std::max(mes, g.ncls * g.nS * g.nS);
+    mmb = std::max(mmb, g.ncls * g.nb * g.nqp / 32);
+    mmk = std::max(mmk, (g.nk1 + 3) / 4);
+    m3 = std::max(m3, g.ncls * g.nt3);
+    m3k = std::max(m3k, (g.nk3 + 3) / 4);
+  }
+  const int ns = (int)p->subs.size();
+  for (int s0 = 0; s0 < ns; s0 += 65535) {   // subdomains per launch: a grid's y / z limit
+    const unsigned n = (unsigned)std::min(65535, ns - s0);
+    k_sep_mode_tab<<<dim3(mq, n), 128, 0, st>>>(ds, s0, sep, entries);
+    k_sep_phi<<<dim3(mq, mrow, n), 128, 0, st>>>(ds, s0, sep);
+    if (mdist == 0) continue;   // no subdomain on the tensor cores
+    k_sep_kd<<<dim3(mdist, n), 128, 0, st>>>(ds, s0, tab, sep);
+    k_sep_tb<<<dim3(mtb, mes, n), 256, 0, st>>>(ds, s0, sep);
+    k_sep_mb<<<dim3(mmk, mmb, n), 256, 0, st>>>(ds, s0, tab, sep);
+    k_sep_b3<<<dim3(m3k, m3, n), 256, 0, st>>>(ds, s0, tab, sep);
+  }
+  return cudaGetLastError();
+}
+
+cudaError_t launch_sep_project(mdp_plan *p, const Batch *fb, int out_kind, const double2 *xi_user, double2 *out,
+                               int part, cudaStream_t st) {
+  const bool user = xi_user != nullptr;
+  const SubDesc *ds = p->d_subs;
+  const double *tab = p->d_tables;
+  double *ws = p->d_ws;
+  const int f1c = user ? F_C1U : F_C1B, f1 = user ? F_G1U : F_G1B, f3c = user ? F_C3U : F_C3B, f3 = user ? F_G3U : F_TCOLS;
+  auto grid = [](int n) { return dim3((unsigned)n); };
+  auto gemm_grid = [&](int n) { return dim3((unsigned)std::max(1, std::min(n, p->n_sm))); };
+#define SEP_LAUNCH(fam, as, ...)                  \
+  do {                                            \
+    if (fb[fam].total_blocks > 0) {               \
+      prof_begin(p, as, st);                      \
+      __VA_ARGS__;                                \
+      prof_end(p, as, st);                        \
+    }                                             \
+  } while (0)
+  if (part == 0) {
+    if (user) SEP_LAUNCH(f1c, F_C1B, k_sep_cut<true, 1><<<grid(fb[f1c].total_blocks), 256, 0, st>>>(fb[f1c], ds, ws, f1c));
+    else SEP_LAUNCH(f1c, F_C1B, k_sep_cut<false, 1><<<grid(fb[f1c].total_blocks), 256, 0, st>>>(fb[f1c], ds, ws, f1c));
+    SEP_LAUNCH(f1, F_G1B, k_sep_gemm<1><<<gemm_grid(fb[f1].total_blocks), SG_THREADS, SG_SMEM, st>>>(
+                              fb[f1], ds, p->d_sep, ws, user, f1, p->d_status));
+    if (user) SEP_LAUNCH(F_SMODE, F_SMODE, k_sep_modes<true><<<grid(fb[F_SMODE].total_blocks), dim3(32, 4), 0, st>>>(fb[F_SMODE], ds, p->d_sep, ws));
+    else SEP_LAUNCH(F_SMODE, F_SMODE, k_sep_modes<false><<<grid(fb[F_SMODE].total_blocks), dim3(32, 4), 0, st>>>(fb[F_SMODE], ds, p->d_sep, ws));
+    return cudaGetLastError();
+  }
+  if (user) SEP_LAUNCH(f3c, F_C3B, k_sep_cut<true, 3><<<grid(fb[f3c].total_blocks), 256, 0, st>>>(fb[f3c], ds, ws, f3c));
+  else SEP_LAUNCH(f3c, F_C3B, k_sep_cut<false, 3><<<grid(fb[f3c].total_blocks), 256, 0, st>>>(fb[f3c], ds, ws, f3c));
+  SEP_LAUNCH(f3, F_TCOLS, k_sep_gemm<3><<<gemm_grid(fb[f3].total_blocks), SG_THREADS, SG_SMEM, st>>>(
+                              fb[f3], ds, p->d_sep, ws, user, f3, p->d_status));
+  if (user) SEP_LAUNCH(F_SOUT, F_SOUT, k_sep_out<true><<<grid(fb[F_SOUT].total_blocks), dim3(32, 8), 0, st>>>(fb[F_SOUT], ds, tab, ws, xi_user, out, out_kind));
+  else SEP_LAUNCH(F_SOUT, F_SOUT, k_sep_out<false><<<grid(fb[F_SOUT].total_blocks), dim3(32, 8), 0, st>>>(fb[F_SOUT], ds, tab, ws, xi_user, out, out_kind));
+#undef SEP_LAUNCH
+  return cudaGetLastError();
+}
+
+}  // namespace mdp

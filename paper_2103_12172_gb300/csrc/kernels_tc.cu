@@ -1,13 +1,15 @@
-// k_inv_cols_tc: the inverse sine transform at the 4 gamma columns of the middle rows
-// (Section 3.2.1 / 3.6: the AP solution u(m, n) = (2/Nx) sum_q sin(pi q m/Nx) yhat(q, n), taken
-// only where the trace on gamma needs it, Eqs. def_Pgamma and Q_construction) as a contraction
-// over the mode index q on the tensor cores, to FP64 accuracy.
+// k_adj_cols_tc: the adjoint's inverse sine transform at the 4 ring columns mlo, mlo+1, mhi-1, mhi of
+// the inner middle rows (the sums of k_adj_ring_cols: (2/Nx) sum_q sin(pi q m/Nx) muhat(q, n) of the
+// adjoint mode field) as a contraction over the mode index q on the tensor cores, to FP64 accuracy.
 //
-// For one middle row n and a tile of 64 columns the sums are a product D = A B with
-//   A[r][q] = yhat(q, n) of matrix row r = (column, real or imaginary part): 128 rows, K = Nq;
+// For one middle row n = nlo + 2 + t and a tile of 64 columns the sums are a product D = A B with
+//   A[r][q] = muhat(q, n) of matrix row r = (column, real or imaginary part): 128 rows, K = Nq;
 //   B[q][s] = sin(pi q m_s / Nx) for the outputs s (x-centred subdomains: the odd-q and even-q
-//            partial sums at m = mlo-1 and mlo, which give all four gamma columns; otherwise the
-//            four columns mlo-1, mlo, mhi, mhi+1 directly).
+//            partial sums at m = mlo and mlo+1, which give all four columns; otherwise the four
+//            columns directly).
+// The 4 sums per row and column go to the workspace rows 2 Px + 4 t + s that k_adj_gamma reads, and
+// with dk the k-gradient partials -Re <sum, s> of each warp of the first producer half, 4 per tile,
+// into the item's reduction slots (summed in order by k_red_items).
 // FP64 accuracy from fp16 operands follows the error-free splitting of Ozaki, Ogita, Oishi and
 // Rump (Numer. Algorithms 59, 2012). Every value x of a column becomes a signed fixed-point
 // integer V on one scale common to the column: with p set by the column's largest exponent
@@ -39,9 +41,9 @@
 // has a time limit; a wait that runs out sets the plan's status word to MDP_ERR_TIMEOUT and every
 // warp leaves its loop, frees the tensor memory and returns; the two producer halves exchange
 // their partial sums through an mbarrier (`xbar`) with the same limit. The scale of a column is the
-// largest exponent over its modes and kept rows, which the per-mode sweep (k_tri) records as it
-// stores them.
-#include "kernels_common.cuh"
+// largest exponent over its modes and inner middle rows, which the adjoint sweep (k_adj_tri)
+// records as it stores them.
+#include "tc_common.cuh"
 
 namespace mdp {
 namespace {
@@ -55,43 +57,6 @@ constexpr int TC_A_BYTES = 128 * TC_KC * 2;   // one digit of A: 128 rows x 16 b
 constexpr int TC_B_BYTES = 32 * TC_KC * 2;    // B: 4 outputs x 8 rows x 16 bf16
 constexpr int TC_STAGE_BYTES = TC_DIG * TC_A_BYTES + TC_B_BYTES;
 constexpr int TC_TMEM_COLS = 256;             // D: 7 A digits x 32 FP32 columns
-constexpr long long TC_WAIT_CYCLES = 4000000000LL;   // about 2 s at the maximum clock
-
-__device__ __forceinline__ uint64_t smem_desc(unsigned addr, unsigned lbo, unsigned sbo) {
-  // shared-memory matrix descriptor: start address, leading (K) and stride (M/N) byte offsets of
-  // the 8 x 16-byte core matrices, descriptor version 1, no swizzle
-  return (uint64_t)((addr >> 4) & 0x3FFF) | ((uint64_t)((lbo >> 4) & 0x3FFF) << 16) |
-         ((uint64_t)((sbo >> 4) & 0x3FFF) << 32) | ((uint64_t)1 << 46);
-}
-// instruction descriptor of kind::f16: FP32 accumulator, fp16 A and B, both K-major, N = 32, M = 128
-constexpr uint32_t TC_IDESC = (1u << 4) | ((32u >> 3) << 17) | ((128u >> 4) << 24);
-
-__device__ __forceinline__ bool mbar_try(unsigned addr, unsigned parity) {
-  unsigned ok;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-      : "=r"(ok) : "r"(addr), "r"(parity) : "memory");
-  return ok != 0;
-}
-// wait for the completion of the phase with parity `parity`, at most TC_WAIT_CYCLES; false when
-// the limit ran out or another warp has already given up (*abort)
-__device__ __forceinline__ bool mbar_wait(unsigned addr, unsigned parity, volatile int *abort) {
-  const long long t0 = clock64();
-  while (!mbar_try(addr, parity)) {
-    if (*abort) return false;
-    if (clock64() - t0 > TC_WAIT_CYCLES) { *abort = 1; return false; }
-  }
-  return true;
-}
-__device__ __forceinline__ void mbar_arrive(unsigned addr) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(addr) : "memory");
-}
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_commit(unsigned mbar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar) : "memory");
-}
-
 // 32 consecutive FP32 columns of this warp's 32 TMEM lanes
 __device__ __forceinline__ void tmem_ld32(unsigned taddr, float *v) {
   unsigned r[32];
@@ -135,35 +100,14 @@ __device__ __forceinline__ void digits52i(double x, int E, unsigned &hi, unsigne
   hi = (unsigned)(w >> 32);
   lo = (unsigned)w;
 }
-// two fp16 digits in one word: byte K (0 = least significant) of the values a (low half) and b
-// (high half), each under the fp16 exponent of 1024, minus 1024 + 128 (exact)
-template <int K>
-__device__ __forceinline__ unsigned digit_pair(unsigned ahi, unsigned alo, unsigned bhi, unsigned blo) {
-  constexpr unsigned k = K & 3;
-  constexpr unsigned sel = k | (k << 4) | ((4 + k) << 8) | ((4 + k) << 12);
-  const unsigned w = __byte_perm(K >= 4 ? ahi : alo, K >= 4 ? bhi : blo, sel);
-  unsigned r;
-  asm("{\n .reg .b32 t;\n lop3.b32 t, %1, %2, %3, 0xEA;\n sub.rn.f16x2 %0, t, %4;\n}\n"
-      : "=r"(r) : "r"(w), "r"(0x00FF00FFu), "r"(0x64006400u), "r"(0x64806480u));
-  return r;
-}
-
 }  // namespace
 
-// One CTA: tiles blockIdx.x, blockIdx.x + gridDim.x, ... of the launch's virtual blocks (F_TCOLS
-// numbering: per item, (Py - 2) middle rows x ceil(ncols / 64) column tiles, column tile fastest).
+// One CTA: tiles blockIdx.x, blockIdx.x + gridDim.x, ... of the launch's virtual blocks (F_ATCOLS
+// numbering: per item, (Py - 4) middle rows x ceil(ncols / 64) column tiles, column tile fastest).
 constexpr int TC_PREFETCH = 3;   // stages ahead of the L2 prefetch of the field
 
-// ADJ: the adjoint's sums (k_adj_ring_cols) instead: A[r][q] = muhat(q, n) on the inner middle
-// rows n = nlo + 2 + t, B at the ring columns mlo, mlo+1, mhi-1, mhi (the plan's second digit
-// block), the 4 sums per row and column written to the workspace rows 2 Px + 4 t + s that
-// k_adj_gamma reads, and with kind != 0 the k-gradient partials -Re <sum, s> of each warp of the
-// first producer half, 4 per tile, into the item's reduction slots (summed in order by
-// k_red_items).
-template <bool CIN, bool ADJ>
 __global__ void __launch_bounds__(TC_THREADS, 2)
-    k_inv_cols_tc(Batch bt, const SubDesc *subs, const double *tab, const double *ws, const double2 *xi_user,
-                  double2 *out, int kind, int *status) {
+    k_adj_cols_tc(Batch bt, const SubDesc *subs, const double *tab, double *ws, int dk, int *status) {
   extern __shared__ __align__(1024) unsigned char tc_sm[];
   __shared__ __align__(8) unsigned long long full_bar[TC_STAGES], empty_bar[TC_STAGES], tfull_bar, tempty_bar, xbar;
   __shared__ unsigned tmem_slot;
@@ -200,7 +144,7 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
       for (int v = blockIdx.x; v < bt.total_blocks && !abort_sh; v += gridDim.x) {
         Item it; int local;
         locate(bt, v, it, local);
-        if (MDP_CHECKED && !item_in_bounds(bt, subs, it, local, ADJ ? F_ATCOLS : F_TCOLS, ADJ)) continue;   // every warp skips it
+        if (MDP_CHECKED && !item_in_bounds(bt, subs, it, local, F_ATCOLS, true)) continue;   // every warp skips it
         const int nchunk = (subs[it.sub].Nq + TC_KC - 1) / TC_KC;
         if (T > 0 && !mbar_wait(smem_u32(&tempty_bar), (T - 1) & 1u, &abort_sh)) break;
         tc_fence_after();
@@ -218,7 +162,7 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
             asm volatile(
                 "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
                 " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem + 32u * dgt),
-                "l"(da), "l"(db), "r"(TC_IDESC), "r"(acc)
+                "l"(da), "l"(db), "r"(f16_idesc(32)), "r"(acc)
                 : "memory");
           }
           tc_commit(smem_u32(&empty_bar[st]));
@@ -237,34 +181,22 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
     for (int v = blockIdx.x; v < bt.total_blocks && !abort_sh; v += gridDim.x) {
       Item it; int local;
       locate(bt, v, it, local);
-      if (MDP_CHECKED && !item_in_bounds(bt, subs, it, local, ADJ ? F_ATCOLS : F_TCOLS, ADJ)) continue;     // every warp skips it
+      if (MDP_CHECKED && !item_in_bounds(bt, subs, it, local, F_ATCOLS, true)) continue;     // every warp skips it
       const SubDesc &d = subs[it.sub];
-      const bool CD = ADJ || d.cplx || CIN;
       const int nct = (it.ncols + 63) >> 6;
       const int t = local / nct, b0 = (local % nct) * 64;
       const int b = b0 + (r >> 1), ri = r & 1;
-      const bool live = b < it.ncols && (CD || ri == 0);
+      const bool live = b < it.ncols;
       const int Nq = d.Nq;
       const int nchunk = (Nq + TC_KC - 1) / TC_KC;
       int rbase[5];
-      if (ADJ) red_slots(d, it.ncols, rbase);
+      red_slots(d, it.ncols, rbase);
       // this thread's value of mode q = 1 at y, of mode q at y + (q - 1) qstride; the column's
       // scale: its largest biased exponent, recorded by the sweep that stored the field
-      const double *y;
-      long long qstride;
-      int E;
-      if (ADJ) {
-        const int j = d.nlo + 2 + t - d.nfirst;   // inner middle row n = nlo + 2 + t (matrix numbering)
-        qstride = 2LL * d.Nt * it.ncols;
-        y = ws + it.a_off + 2LL * ((long long)j * it.ncols + b) + ri;
-        E = live ? reinterpret_cast<const int *>(ws + it.red_off + rbase[4] + 1)[b] : 0;
-      } else {
-        const int yrow = t + 2;                 // middle row n = nlo + 1 + t
-        const long long ncd = (long long)it.ncols * (CD ? 2 : 1);   // doubles per stored row
-        qstride = (long long)d.NYf * ncd;
-        y = ws + it.y_off + (long long)yrow * ncd + (CD ? 2LL * b + ri : (long long)b);
-        E = live ? reinterpret_cast<const int *>(ws + it.red_off)[b] : 0;
-      }
+      const int j0 = d.nlo + 2 + t - d.nfirst;   // middle row n = nlo + 2 + t (matrix numbering)
+      const long long qstride = 2LL * d.Nt * it.ncols;
+      const double *y = ws + it.a_off + 2LL * ((long long)j0 * it.ncols + b) + ri;
+      const int E = live ? reinterpret_cast<const int *>(ws + it.red_off + rbase[4] + 1)[b] : 0;
       const long long mb = magic_bits(E);
       const double magic = __longlong_as_double(mb);
       const long long cb = mb - 0x0080808080808080LL;
@@ -329,7 +261,7 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
         // B: the plan's 1 KiB block of sine digits for these 16 modes, 16 bytes per thread
         if (tid < 64)
           *reinterpret_cast<uint4 *>(sa + TC_DIG * TC_A_BYTES + 16 * tid) =
-              reinterpret_cast<const uint4 *>(tab + d.tcb_off + (ADJ ? 128LL * nchunk : 0LL))[c * 64 + tid];
+              reinterpret_cast<const uint4 *>(tab + d.tcb_off)[c * 64 + tid];
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic stores -> MMA reads
         mbar_arrive(smem_u32(&full_bar[st]));
 #pragma unroll
@@ -383,37 +315,20 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
         } else {
           u4[0] = val[0]; u4[1] = val[1]; u4[2] = val[2]; u4[3] = val[3];
         }
-        if (ADJ) {
-          // each lane writes its part (real: even lane, imaginary: odd lane) of the 4 sums
-          double *wsw = const_cast<double *>(ws);   // rows and slots no other lane of the launch reads
-          double part = 0.0;
-          if (b < it.ncols) {
+        // each lane writes its part (real: even lane, imaginary: odd lane) of the 4 sums
+        double part = 0.0;
+        if (b < it.ncols) {
 #pragma unroll
-            for (int s = 0; s < 4; ++s) {
-              const long long o = 2LL * ((long long)(2 * d.Px + 4 * t + s) * it.ncols + b) + ri;
-              wsw[it.r_off + o] = u4[s];
-              if (kind) part = fma(-u4[s], ws[it.s_off + o], part);
-            }
+          for (int s = 0; s < 4; ++s) {
+            const long long o = 2LL * ((long long)(2 * d.Px + 4 * t + s) * it.ncols + b) + ri;
+            ws[it.r_off + o] = u4[s];
+            if (dk) part = fma(-u4[s], ws[it.s_off + o], part);
           }
-          if (kind) {
+        }
+        if (dk) {
 #pragma unroll
-            for (int off = 16; off > 0; off >>= 1) part += __shfl_xor_sync(0xffffffffu, part, off);
-            if (lane == 0) wsw[it.red_off + rbase[2] + 4 * local + quarter] = part;
-          }
-        } else {
-          // lanes 2i (real part) and 2i+1 (imaginary part) of column b: the even lane writes
-          double o4[4];
-#pragma unroll
-          for (int s = 0; s < 4; ++s) o4[s] = __shfl_xor_sync(0xffffffffu, u4[s], 1);
-          if (ri == 0 && b < it.ncols) {
-            const int g0 = 2 * (d.Px + 2) + 4 * t;
-#pragma unroll
-            for (int s = 0; s < 4; ++s) {
-              cplx uv = cmk(-u4[s], CD ? -o4[s] : 0.0);
-              if (kind == MDP_OUT_P) uv = cadd(uv, density<CIN>(d, it, ws, tab, xi_user, b, g0 + s));
-              out[it.io_off + (long long)b * d.G + g0 + s] = make_double2(uv.re, uv.im);
-            }
-          }
+          for (int off = 16; off > 0; off >>= 1) part += __shfl_xor_sync(0xffffffffu, part, off);
+          if (lane == 0) ws[it.red_off + rbase[2] + 4 * local + quarter] = part;
         }
       }
       // half_sh is rewritten only in the next tile's epilogue, which no producer reaches before
@@ -432,29 +347,13 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
 int tc_cols_smem_bytes() { return TC_STAGES * TC_STAGE_BYTES; }
 
 cudaError_t set_tc_kernel_attributes() {
-  const int sm = tc_cols_smem_bytes();
-  cudaError_t e = cudaFuncSetAttribute(k_inv_cols_tc<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_inv_cols_tc<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_inv_cols_tc<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-  return e;
-}
-
-cudaError_t launch_inv_cols_tc(const Batch &b, const SubDesc *subs, const double *tab, const double *ws,
-                               const double2 *xi_user, double2 *out, int kind, int *status, int n_sm,
-                               cudaStream_t st) {
-  const int grid = std::max(1, std::min(b.total_blocks, 2 * n_sm));
-  if (xi_user)
-    k_inv_cols_tc<true, false><<<grid, TC_THREADS, tc_cols_smem_bytes(), st>>>(b, subs, tab, ws, xi_user, out, kind, status);
-  else
-    k_inv_cols_tc<false, false><<<grid, TC_THREADS, tc_cols_smem_bytes(), st>>>(b, subs, tab, ws, xi_user, out, kind, status);
-  return cudaGetLastError();
+  return cudaFuncSetAttribute(k_adj_cols_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, tc_cols_smem_bytes());
 }
 
 cudaError_t launch_adj_cols_tc(const Batch &b, const SubDesc *subs, const double *tab, double *ws, bool dk,
                                int *status, int n_sm, cudaStream_t st) {
   const int grid = std::max(1, std::min(b.total_blocks, 2 * n_sm));
-  k_inv_cols_tc<false, true><<<grid, TC_THREADS, tc_cols_smem_bytes(), st>>>(b, subs, tab, ws, nullptr, nullptr,
-                                                                            dk ? 1 : 0, status);
+  k_adj_cols_tc<<<grid, TC_THREADS, tc_cols_smem_bytes(), st>>>(b, subs, tab, ws, dk ? 1 : 0, status);
   return cudaGetLastError();
 }
 

@@ -44,7 +44,8 @@ struct SubDesc {
   int rows_fft;     // inverse transform of the gamma rows by FFT (Nx a power of 2, 2Nx <= 4096)
   int fpb;          // FFTs (columns) per block of the dense-row kernels: max(1, 1024 / (2 Nx))
   int leader;       // index of the subdomain owning this one's tables (itself unless deduplicated)
-  int tc_cols;      // 1: the gamma columns of the middle rows are summed on the tensor cores (k_inv_cols_tc)
+  int tc_cols;      // 1: the projection runs through the separable Green's function (kernels_sep.cu) and the
+                    // adjoint's ring columns through k_adj_cols_tc; 0: per-mode sweeps and FP64 sums
   double h, k;
   double x0, x1, y0, y1, ax0, ay0;
   double c0, c1, c2;  // 9-point coefficients: centre, edge, corner (Eq. FD_scheme)
@@ -57,9 +58,15 @@ struct SubDesc {
   long long seg_off;    // doubles: per mode [Nq][5] = (rlo, rhi, frlo, frhi, itop): real rows of the
                         // factor table, real rows of the forward-sweep table, last swept row
   long long fs_off;     // doubles: projection forward-sweep table [Nq][NYf][FSW] (rows i0..)
-  long long tcb_off;    // doubles: tensor-core sums: per 16 modes a 1 KiB block of the fp16 sine digits at the
-                        // gamma columns, then as many at the adjoint's ring columns (one column further in)
-                        // of the sines, in the shared-memory operand layout of k_inv_cols_tc
+  long long tcb_off;    // doubles: per 16 modes a 1 KiB block of the fp16 digits of the sines at the adjoint's
+                        // ring columns, in the shared-memory operand layout of k_adj_cols_tc
+  // bytes into the plan's separable tables (kernels_sep.cu), device only; without tc_cols the first three
+  long long sep_ab;     // doubles [Nq][2]: interior entries (off-diagonal, diagonal) of T_q
+  long long sep_mt;     // per mode SEP_MTW doubles
+  long long sep_phi;    // doubles [2][Py + 2][Nq]: phi_1, phi_2 on the rows nlo-1 .. nhi+1
+  long long sep_kd;     // doubles [class][output][source][Py]: K by row distance
+  long long sep_kde;    // ints [class][output]: exponent of the largest |K|
+  long long sep_tb, sep_mb, sep_b3;   // digit blocks of K (Toeplitz), of the moments, of the synthesis
   long long out_off;    // complex elements: start of the subdomain's output block
   long long rec_off;    // complex elements: start of the receiver block [n_cols][Px - 2]
   int *dstatus;         // the plan's device status word (bounds-checked build: first error; else unused)
@@ -73,10 +80,10 @@ struct Item {
   long long r_off;    // ring residual [R][ncols] (real or complex)
   long long gr_off;   // forward sine transform of the 4 dense ring rows [4][Nq][ncols]
   long long y_off;    // mode-space field [Nq][NY][ncols]
-  long long a_off;    // adjoint mode-space field [Nq][Nt][ncols] (gradient pass)
+  long long a_off;    // adjoint mode-space field [Nq][Nt][ncols] (gradient pass), or in the projection the
+                      // operands and sums of the separable solve (SepWs)
   long long s_off;    // gradient source on the ring [R][ncols] (complex)
-  long long red_off;  // per-block partial sums of the k-gradient (gradient pass); in the projection,
-                      // per column the largest biased exponent of the stored mode-space rows (int)
+  long long red_off;  // per-block partial sums of the k-gradient (gradient pass)
   long long io_off;   // complex elements: column col0 of this item in xi / out / cot / grad_xi
 };
 
@@ -102,6 +109,103 @@ struct Batch {
 };
 
 constexpr int FSW = 24;  // doubles per forward-sweep table row
+
+// ---- separable projection (kernels_sep.cu)
+constexpr int SEP_MTW = 56;               // doubles per mode of the mode table
+constexpr int SEP_ABLK = 7 * 128 * 16 * 2;  // bytes of A: 7 digits x 128 rows x 16 values of K, fp16
+constexpr int SEP_BBLK = 7 * 32 * 16 * 2;   // bytes of B: 7 digits x 32 outputs x 16 values of K
+constexpr int SEP_MODES_PER_BLOCK = 32;   // k_sep_modes
+
+// Sizes of a subdomain's contractions.
+struct SepGeo {
+  int ncls, nS;        // classes of modes (odd, even) on x-centred subdomains, else 1; output (and source) columns
+  int nqp;             // modes per class, padded to 32
+  int Pi, Pj;          // output rows nlo+1 .. nhi-1, source rows nlo+2 .. nhi-2
+  int nti, nkj;        // groups of 32 outputs, of 16 sources per column
+  int nb;              // moments per mode: 2, or 3 with a receiver row
+  int nk1, nk3;        // K in units of 16: stage 1 (source column, row), stage 3 (b, mode)
+  int nt1, nt3;        // tiles of 32 outputs
+  int ND;              // distinct Toeplitz blocks per (output, source) column
+};
+inline __host__ __device__ SepGeo sep_geo(const SubDesc &d) {
+  SepGeo g;
+  g.ncls = d.xsym ? 2 : 1;
+  g.nS = d.xsym ? 2 : 4;
+  g.nqp = ((d.xsym ? (d.Nq + 1) / 2 : d.Nq) + 31) / 32 * 32;
+  g.Pi = d.Py - 2;
+  g.Pj = d.Py - 4;
+  g.nti = (g.Pi + 31) / 32;
+  g.nkj = (g.Pj + 15) / 16;
+  g.nb = d.nrec >= 0 ? 3 : 2;
+  g.nk1 = g.nS * g.nkj;
+  g.nk3 = 2 * g.nqp / 16;
+  g.nt3 = g.nS * g.nti;
+  g.nt1 = g.nt3 + g.nb * g.nqp / 32;
+  g.ND = 2 * g.nti + g.nkj;
+  return g;
+}
+// mode number of entry qi of class e (past Nq: padding)
+inline __host__ __device__ int sep_mode(const SubDesc &d, int e, int qi) { return d.xsym ? 2 * qi + 1 + e : qi + 1; }
+// grid column of output s (gamma) and of source c (ring); x-centred: the left ones, the right ones mirrored
+inline __host__ __device__ int sep_out_col(const SubDesc &d, int s) {
+  return s == 0 ? d.mlo - 1 : s == 1 ? d.mlo : s == 2 ? d.mhi : d.mhi + 1;
+}
+inline __host__ __device__ int sep_src_col(const SubDesc &d, int c) {
+  return c == 0 ? d.mlo : c == 1 ? d.mlo + 1 : c == 2 ? d.mhi - 1 : d.mhi;
+}
+inline __host__ __device__ int sep_pad128(int n) { return (n + 127) / 128 * 128; }
+// Only the basis columns of sides 3 and 4 have residuals on the middle ring rows (the gamma nodes
+// next to them belong to these sides), so stage 1 has only their rows: sep_side_before counts such
+// columns below column c, sep_side_col gives the row-th one from column c0 on, sep_side_row the
+// row of an item's column b (-1: a column of side 1 or 2).
+inline __host__ __device__ int sep_side_before(const SubDesc &d, int c) {
+  const int M = d.n_modes, r = c % (4 * M) - 2 * M;
+  return (c / (4 * M)) * 2 * M + (r > 0 ? r : 0);
+}
+inline __host__ __device__ int sep_side_cols(const SubDesc &d, int c0, int ncols) {
+  return sep_side_before(d, c0 + ncols) - sep_side_before(d, c0);
+}
+inline __host__ __device__ int sep_side_col(const SubDesc &d, int c0, int row) {
+  const int f = sep_side_before(d, c0) + row, M2 = 2 * d.n_modes;
+  return (f / M2) * 2 * M2 + M2 + f % M2;
+}
+inline __host__ __device__ int sep_side_row(const SubDesc &d, int c0, int b) {
+  return (c0 + b) % (4 * d.n_modes) < 2 * d.n_modes ? -1 : sep_side_before(d, c0 + b) - sep_side_before(d, c0);
+}
+// Rows of A, padded to the MMA's 128: stage 1 (columns, or real and imaginary parts of user
+// densities), stage 3 (columns, or real and imaginary parts); the parts are sep_pad128(ncols) apart.
+inline __host__ __device__ int sep_rows1(const SubDesc &d, int ncols, int col0, bool user) {
+  return user ? 2 * sep_pad128(ncols) : sep_pad128(sep_side_cols(d, col0, ncols));
+}
+inline __host__ __device__ int sep_rows3(const SubDesc &d, int ncols, bool user) {
+  return (user || d.cplx ? 2 : 1) * sep_pad128(ncols);
+}
+// Workspace of an item's separable solve, in doubles from its a_off (sized for complex data).
+struct SepWs {
+  long long u1, u3;    // sums at the gamma columns [class][output][Pi][rows] of stage 1 and stage 3
+  long long mom;       // moments [class][3][nqp][rows]
+  long long aeff;      // A_b [class][2][nqp][rows]
+  long long a1, a3;    // digit blocks of A
+  long long ex1, ex3;  // exponents of A's rows (ints) [class][rows]
+  long long total;
+};
+inline __host__ __device__ SepWs sep_ws(const SubDesc &d, int ncols) {
+  const SepGeo g = sep_geo(d);
+  const long long R = 2LL * sep_pad128(ncols), u = g.ncls * (long long)g.nS * g.Pi * R;
+  SepWs w;
+  long long off = 0;
+  auto take = [&](long long n) { const long long o = off; off += (n + 31) & ~31LL; return o; };
+  w.a1 = take(g.ncls * (R / 128) * g.nk1 * (SEP_ABLK / 8));
+  w.a3 = take(g.ncls * (R / 128) * g.nk3 * (SEP_ABLK / 8));
+  w.u1 = take(u);
+  w.u3 = take(u);
+  w.mom = take(g.ncls * 3LL * g.nqp * R);
+  w.aeff = take(g.ncls * 2LL * g.nqp * R);
+  w.ex1 = take(g.ncls * R / 2);
+  w.ex3 = take(g.ncls * R / 2);
+  w.total = off;
+  return w;
+}
 constexpr int TRI_WARPS = 1;  // warps (modes) per block of the per-mode sweep kernel k_tri
 constexpr int FFT_POINTS = 4096;        // longest transform (2 Nx) of the dense-row FFT kernels (64 KiB)
 constexpr int FFT_BLOCK_POINTS = 1024;  // complex values per block when 2 Nx is shorter: fpb = 1024 / (2 Nx)
@@ -181,6 +285,8 @@ struct mdp_plan {
   mdp::SubDesc *d_subs = nullptr;
   double *d_tables = nullptr;
   uint8_t *d_piv = nullptr;
+  unsigned char *d_sep = nullptr;        // separable tables (kernels_sep.cu), rebuilt with the factor tables
+  long long sep_bytes = 0;
   double *d_ws = nullptr;
   long long ws_doubles = 0;
   int *d_status = nullptr;
@@ -190,12 +296,15 @@ struct mdp_plan {
   mdp::HostBuf<mdp::SubDesc> sub_stage;  // pinned copy of the subdomain descriptors (async upload)
   mdp::HostBuf<int> h_fstatus;           // pinned read-back of d_fstatus
   bool host_stale = false;               // device tables refactored since the host tables were built
+  bool fs_stale = false;                 // device sweep tables older than the wavenumbers (not read by the
+                                         // separable solve; rebuilt when mdp_plan_read_tables asks)
   // second table set of mdp_plan_update_k_async (allocated by its first call). d_subs, d_tables
   // and d_piv name physical set `set`; the alt_* pointers the other. ready_ev[s]: after the last
   // refactorisation into set s; used_ev[s]: after the last compute call that read it.
   mdp::SubDesc *alt_subs = nullptr;
   double *alt_tables = nullptr;
   uint8_t *alt_piv = nullptr;
+  unsigned char *alt_sep = nullptr;
   mdp::HostBuf<mdp::SubDesc> alt_stage;  // pinned descriptor stage of set 1 (sub_stage: set 0)
   int set = 0;
   cudaEvent_t ready_ev[2] = {nullptr, nullptr};
@@ -213,8 +322,8 @@ struct mdp_plan {
   std::vector<GraphEntry> graphs;
   // per-kernel event timing (mdp_plan_profile)
   bool prof_on = false;
-  std::vector<std::pair<cudaEvent_t, cudaEvent_t>> prof_ev[16];
-  int prof_used[16] = {0};
+  std::vector<std::pair<cudaEvent_t, cudaEvent_t>> prof_ev[32];
+  int prof_used[32] = {0};
 };
 
 namespace mdp {
@@ -233,13 +342,17 @@ inline void set_bounds(const mdp_plan *p, Batch &b, long long out_n, bool grad) 
   b.status = p->d_status;
 }
 
-// kernel families (each has its own block decomposition of an item); F_A* are the adjoint's
+// kernel families (each has its own block decomposition of an item); F_A* are the adjoint's. F_TRI is
+// the gradient pass's full sweep, F_PTRI the projection's (subdomains without the separable solve);
+// F_C* cut operands, F_G* contract (stage 1 and 3, B: basis columns, U: user densities; F_TCOLS is
+// stage 3 for basis columns), F_SMODE and F_SOUT are the separable solve's other kernels.
 enum Fam { F_EXT = 0, F_RES, F_FROWS, F_TRI, F_IROWS, F_ICOLS, F_AFWD, F_ATRI, F_ARING, F_ARINGC, F_AGAM, F_IREC,
-           F_ACOLS, F_TCOLS, F_ATCOLS, NFAM };
+           F_ACOLS, F_TCOLS, F_ATCOLS, F_PTRI, F_C1B, F_C1U, F_G1B, F_G1U, F_SMODE, F_C3B, F_C3U, F_G3U, F_SOUT, NFAM };
+static_assert(NFAM <= 32, "per-family event lists of mdp_plan");
 
 // Blocks of kernel family f for an item of ncols columns: 32 columns (x) times BY tasks (y).
 // The same function numbers the blocks on the host (prefix sums) and in the kernels.
-inline __host__ __device__ int blocks_for(int f, const SubDesc &d, int ncols) {
+inline __host__ __device__ int blocks_for(int f, const SubDesc &d, int ncols, int col0) {
   const int cb = (ncols + 31) / 32;
   switch (f) {
     case F_EXT: return (d.G + 127) / 128;
@@ -252,7 +365,21 @@ inline __host__ __device__ int blocks_for(int f, const SubDesc &d, int ncols) {
       if (d.rows_fft) return 4 * ((ncols + d.fpb - 1) / d.fpb);
       return cb * (((d.xsym ? 4 * (d.Ph + 1) : 4 * (d.Px + 2)) + 7) / 8);
     case F_ICOLS: return d.tc_cols ? 0 : cb * ((d.Py - 2 + 7) / 8);
-    case F_TCOLS: return d.tc_cols ? ((ncols + 63) / 64) * (d.Py - 2) : 0;   // tiles: middle row x 64 columns
+    case F_PTRI: return d.tc_cols ? 0 : cb * ((d.Nq + TRI_WARPS - 1) / TRI_WARPS);
+    case F_C1B: case F_C1U: case F_G1B: case F_G1U: {
+      if (!d.tc_cols) return 0;
+      const SepGeo g = sep_geo(d);
+      const int R = sep_rows1(d, ncols, col0, f == F_C1U || f == F_G1U);
+      return f == F_C1B || f == F_C1U ? g.ncls * (R / 8) : g.ncls * (R / 128) * g.nt1;
+    }
+    case F_C3B: case F_C3U: case F_TCOLS: case F_G3U: {
+      if (!d.tc_cols) return 0;
+      const SepGeo g = sep_geo(d);
+      const int R = sep_rows3(d, ncols, f == F_C3U || f == F_G3U);
+      return f == F_C3B || f == F_C3U ? g.ncls * (R / 8) : g.ncls * (R / 128) * g.nt3;
+    }
+    case F_SMODE: return d.tc_cols ? cb * ((d.Nq + SEP_MODES_PER_BLOCK - 1) / SEP_MODES_PER_BLOCK) : 0;
+    case F_SOUT: return d.tc_cols ? cb * ((d.Py - 2 + 7) / 8) : 0;
     case F_AFWD:
       if (d.rows_fft) return 5 * ((ncols + d.fpb - 1) / d.fpb);
       return cb * ((d.Nx / 2 + 7) / 8);
@@ -273,16 +400,17 @@ inline __host__ __device__ int blocks_for(int f, const SubDesc &d, int ncols) {
 // tile | AGAM], total
 inline __host__ __device__ void red_slots(const SubDesc &d, int ncols, int base[5]) {
   base[0] = 0;
-  base[1] = base[0] + blocks_for(F_ATRI, d, ncols);
-  base[2] = base[1] + blocks_for(F_ARING, d, ncols);
-  base[3] = base[2] + blocks_for(F_ARINGC, d, ncols) + 4 * blocks_for(F_ATCOLS, d, ncols);
-  base[4] = base[3] + blocks_for(F_AGAM, d, ncols);
+  base[1] = base[0] + blocks_for(F_ATRI, d, ncols, 0);
+  base[2] = base[1] + blocks_for(F_ARING, d, ncols, 0);
+  base[3] = base[2] + blocks_for(F_ARINGC, d, ncols, 0) + 4 * blocks_for(F_ATCOLS, d, ncols, 0);
+  base[4] = base[3] + blocks_for(F_AGAM, d, ncols, 0);
 }
 // Workspace slices of an item of ncols columns, in doubles from the item's base (each 256-byte
 // aligned): basis densities, ring residual, dense-row transforms, mode-space field, and for the
-// gradient pass the adjoint field, k-source and per-block partials; the last slice holds per
-// column the largest biased exponent (ints) of the kept mode-space rows (projection) or of the
-// adjoint field's inner middle rows (gradient pass, after the partials and their total).
+// gradient pass the adjoint field, k-source and per-block partials; its last slice holds, after the
+// partials and their total, per column the largest biased exponent (ints) of the adjoint field's
+// inner middle rows. With the separable solve the projection keeps only the 4 gamma rows and the
+// receiver row of the mode-space field ([Nq][5][ncols]), and its operands and sums (SepWs).
 inline __host__ __device__ void item_workspace(const SubDesc &d, int ncols, bool grad, long long &xi, long long &r,
                                                long long &gr, long long &y, long long &a, long long &s,
                                                long long &red, long long &total) {
@@ -291,12 +419,12 @@ inline __host__ __device__ void item_workspace(const SubDesc &d, int ncols, bool
   xi = off; off += al((long long)d.G * ncols * (grad ? 2 : 1));
   r = off;  off += al((long long)(d.R > d.R2 ? d.R : d.R2) * ncols * 2);
   gr = off; off += al(5LL * d.Nq * ncols * 2);  // 4 dense rows (+ the receiver row in the adjoint)
-  y = off;  off += al((long long)d.Nq * (grad ? d.Nt : d.NYf) * ncols * 2);
-  a = off;  off += grad ? al((long long)d.Nq * d.Nt * ncols * 2) : 0;
+  y = off;  off += al((long long)d.Nq * (grad ? d.Nt : d.tc_cols ? 5 : d.NYf) * ncols * 2);
+  a = off;  off += grad ? al((long long)d.Nq * d.Nt * ncols * 2) : d.tc_cols ? sep_ws(d, ncols).total : 0;
   s = off;  off += grad ? al((long long)d.R * ncols * 2) : 0;
   int rs[5];
   red_slots(d, ncols, rs);
-  red = off; off += grad ? al(rs[4] + 1 + (ncols + 1) / 2) : al((ncols + 1) / 2);
+  red = off; off += grad ? al(rs[4] + 1 + (ncols + 1) / 2) : 0;
   total = off;
 }
 const char *fam_name(int f);
@@ -306,10 +434,11 @@ void prof_end(mdp_plan *p, int fam, cudaStream_t st);
 // plan construction (host)
 mdp_status build_host_plan(mdp_plan *p, const mdp_subdomain *subs, int n);
 mdp_status refactor_host(mdp_plan *p, const double *k);
+void mode_entries(const SubDesc &d, int q, double &off, double &diag);   // interior entries of T_q
 mdp_status set_k_fields(mdp_plan *p, const double *k);   // validate k, update the k-dependent SubDesc fields
-cudaError_t launch_factor(const mdp_plan *p, int *status, cudaStream_t st);   // factor.cu
-// the same into an explicit table set (descriptors ds, tables tab, pivot flags piv)
-cudaError_t launch_factor_to(const mdp_plan *p, const SubDesc *ds, double *tab, uint8_t *piv, int *status,
+// factor.cu: the factor tables into a table set (descriptors ds, tables tab, pivot flags piv); the
+// sweep tables of subdomains that project through the separable solve only with `all`
+cudaError_t launch_factor_to(const mdp_plan *p, const SubDesc *ds, double *tab, uint8_t *piv, int *status, bool all,
                              cudaStream_t st);
 void host_mode_solve(const HostSub &hs, int q, int adjoint, const double *b, double *x);
 // kernel launchers (kernels.cu)
@@ -317,10 +446,15 @@ enum { PASS_FWD = 0, PASS_GRAD = 1 };
 cudaError_t set_kernel_attributes();      // kernels.cu: opt-in shared memory of the FFT kernels
 cudaError_t set_adj_kernel_attributes();  // kernels_adj.cu
 cudaError_t set_tc_kernel_attributes();   // kernels_tc.cu
-// the gamma columns of the middle rows on the tensor cores (items whose subdomain has tc_cols)
-cudaError_t launch_inv_cols_tc(const Batch &b, const SubDesc *subs, const double *tab, const double *ws,
-                               const double2 *xi_user, double2 *out, int kind, int *status, int n_sm,
-                               cudaStream_t st);
+cudaError_t set_sep_kernel_attributes();  // kernels_sep.cu
+// the separable tables of every subdomain that takes them, for the wavenumbers of the descriptors ds;
+// entries: from matrix entries computed here, else from the stored ones (sep_ab)
+cudaError_t launch_sep_tables(const mdp_plan *p, const SubDesc *ds, const double *tab, unsigned char *sep, bool entries,
+                              cudaStream_t st);
+// the separable solve of the projection: part 0 up to the field on the 4 gamma rows, part 1 the
+// gamma columns of the middle rows
+cudaError_t launch_sep_project(mdp_plan *p, const Batch *fb, int out_kind, const double2 *xi_user, double2 *out,
+                               int part, cudaStream_t st);
 // the adjoint's sums at the 4 ring columns of the inner middle rows (dk: with the k-gradient partials)
 cudaError_t launch_adj_cols_tc(const Batch &b, const SubDesc *subs, const double *tab, double *ws, bool dk,
                                int *status, int n_sm, cudaStream_t st);

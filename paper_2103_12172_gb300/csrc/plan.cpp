@@ -23,7 +23,9 @@ static const double kSingularTol = 1e-13; // pivot below this x max|T| -> singul
 const char *fam_name(int f) {
   static const char *names[NFAM] = {"k_extend", "k_residual", "k_fwd_rows", "k_tri", "k_inv_rows", "k_inv_cols",
                                     "k_adj_rows", "k_adj_tri", "k_adj_ring_rows", "k_adj_ring_cols", "k_adj_gamma",
-                                    "k_inv_rec", "k_adj_cols", "k_inv_cols_tc", "k_adj_ring_cols_tc"};
+                                    "k_inv_rec", "k_adj_cols", "k_inv_cols_tc", "k_adj_ring_cols_tc", "k_tri(projection)",
+                                    "k_sep_cut1", "k_sep_cut1(user)", "k_sep_gemm1", "k_sep_gemm1(user)", "k_sep_modes",
+                                    "k_sep_cut3", "k_sep_cut3(user)", "k_inv_cols_tc(user)", "k_sep_out"};
   return (f >= 0 && f < NFAM) ? names[f] : "?";
 }
 
@@ -65,9 +67,10 @@ static mdp_status geometry(const mdp_subdomain &in, HostSub &hs, unsigned flags,
   d.nrec = -1;
   d.rows_fft = !(flags & MDP_PLAN_DIRECT_ROWS) && (d.Nx & (d.Nx - 1)) == 0 && 2 * d.Nx <= FFT_POINTS && d.Nx >= 8;
   d.fpb = d.rows_fft ? std::max(1, fft_block_points / (2 * d.Nx)) : 0;
-  // gamma columns on the tensor cores: exact integer accumulation needs at most 1024 modes per
-  // output (a parity half of Nq on centred subdomains); MDP_PLAN_FP64_COLS (or the environment
-  // MDP_TC_COLS=0) keeps the FP64 sums
+  // the separable solve and the adjoint's ring columns on the tensor cores: the adjoint's exact
+  // integer accumulation needs at most 1024 modes per output (a parity half of Nq on centred
+  // subdomains); MDP_PLAN_FP64_COLS (or the environment MDP_TC_COLS=0) keeps the sweeps and the
+  // FP64 sums
   {
     const char *tc = std::getenv("MDP_TC_COLS");
     const bool on = !(flags & MDP_PLAN_FP64_COLS) && !(tc && tc[0] == '0' && tc[1] == 0);
@@ -107,6 +110,11 @@ static mdp_status geometry(const mdp_subdomain &in, HostSub &hs, unsigned flags,
     }
   }
   if ((int)hs.owner.size() != d.G) return MDP_ERR_ARG;
+  // the separable solve takes basis columns of sides 1 and 2 as free of residual on the middle ring
+  // rows: the gamma nodes there are nearest to a side x = const
+  const int W = d.Px + 2;
+  for (int i = 2 * W; i < 2 * W + 4 * (d.Py - 2); ++i)
+    if (hs.owner[i] < 3) d.tc_cols = 0;
   return MDP_OK;
 }
 
@@ -121,6 +129,12 @@ static mdp_status geometry(const mdp_subdomain &in, HostSub &hs, unsigned flags,
 //     alpha = (1 - k^2h^2/24 - lambda/6)/h^2,   beta = i k (1 + k^2h^2/8 + lambda/2)/h.
 // Factorisation: Gaussian elimination with partial pivoting on the band (row swaps create
 // one extra super-diagonal), the textbook algorithm for banded LU.
+void mode_entries(const SubDesc &d, int q, double &off, double &diag) {
+  const double h2 = d.h * d.h, k2 = d.k * d.k;
+  const double sq = std::sin(M_PI * q / (2.0 * d.Nx)), lam = -4.0 * sq * sq;
+  off = 1.0 / h2 + lam / (6.0 * h2) + k2 / 12.0;
+  diag = -2.0 * off + lam / h2 + k2 + k2 * lam / 12.0;
+}
 // The tridiagonal T_q of sine mode q (rows 0..Nt-1) and, when dT != nullptr, its k-derivative
 // rows (sub, diag, super; complex). dl[i] = T[i+1][i], dg[i] = T[i][i], du[i] = T[i][i+1].
 static void mode_matrix(const SubDesc &d, int q, cd *dl, cd *dg, cd *du, double *dT) {
@@ -128,8 +142,8 @@ static void mode_matrix(const SubDesc &d, int q, cd *dl, cd *dg, cd *du, double 
   const double h = d.h, h2 = h * h, k = d.k, k2 = k * k;
   const double sq = std::sin(M_PI * q / (2.0 * d.Nx));
   const double lam = -4.0 * sq * sq;
-  const double a = 1.0 / h2 + lam / (6.0 * h2) + k2 / 12.0;
-  const double dd = -2.0 * a + lam / h2 + k2 + k2 * lam / 12.0;
+  double a, dd;
+  mode_entries(d, q, a, dd);
   const double da = k / 6.0;
   const double ddd = -2.0 * da + 2.0 * k + 2.0 * k * lam / 12.0;
   const bool paper = d.ap_bc == MDP_AP_DIRX_SOMMY_PAPER;
@@ -386,7 +400,7 @@ void host_mode_solve(const HostSub &hs, int q, int adjoint, const double *b, dou
 
 // ---------------------------------------------------------------- tables
 static bool layout_tables(mdp_plan *p) {
-  long long off = 0, poff = 0, out = 0;
+  long long off = 0, poff = 0, out = 0, sep = 0;
   auto al = [](long long v) { return (v + 31) & ~31LL; };
   for (auto &hs : p->subs) {
     SubDesc &d = hs.d;
@@ -394,8 +408,23 @@ static bool layout_tables(mdp_plan *p) {
       const SubDesc &ld = p->subs[d.leader].d;
       d.fact_off = ld.fact_off; d.dT_off = ld.dT_off; d.sin_off = ld.sin_off; d.geo_off = ld.geo_off;
       d.seg_off = ld.seg_off; d.fs_off = ld.fs_off; d.piv_off = ld.piv_off; d.tcb_off = ld.tcb_off;
+      d.sep_ab = ld.sep_ab; d.sep_mt = ld.sep_mt; d.sep_phi = ld.sep_phi; d.sep_kd = ld.sep_kd; d.sep_kde = ld.sep_kde;
+      d.sep_tb = ld.sep_tb; d.sep_mb = ld.sep_mb; d.sep_b3 = ld.sep_b3;
       d.out_off = out;  out += (long long)d.G * d.n_cols;
       continue;
+    }
+    auto take = [&](long long bytes) { const long long o = sep; sep += (bytes + 255) & ~255LL; return o; };
+    d.sep_ab = take(16LL * d.Nq);
+    d.sep_mt = take(8LL * SEP_MTW * d.Nq);
+    d.sep_phi = take(16LL * (d.Py + 2) * d.Nq);
+    if (d.tc_cols) {
+      const SepGeo g = sep_geo(d);
+      const long long pairs = (long long)g.ncls * g.nS * g.nS;
+      d.sep_kd = take(8 * pairs * d.Py);
+      d.sep_kde = take(4LL * g.ncls * g.nS);
+      d.sep_tb = take(pairs * g.ND * SEP_BBLK);
+      d.sep_mb = take((long long)g.ncls * (3 * g.nqp / 32) * g.nk1 * SEP_BBLK);   // room for receivers
+      d.sep_b3 = take((long long)g.ncls * g.nt3 * g.nk3 * SEP_BBLK);
     }
     const int FW = d.cplx ? 8 : 4;
     d.fact_off = off; off += al((long long)d.Nq * d.Nt * FW);
@@ -404,7 +433,7 @@ static bool layout_tables(mdp_plan *p) {
     d.geo_off = off;  off += al(4LL * d.G);
     d.seg_off = off;  off += al(5LL * d.Nq);
     d.fs_off = off;   off += al((long long)d.Nq * d.NYf * FSW);
-    d.tcb_off = off;  off += d.tc_cols ? al(256LL * ((d.Nq + 15) / 16)) : 0;
+    d.tcb_off = off;  off += d.tc_cols ? al(128LL * ((d.Nq + 15) / 16)) : 0;
     d.piv_off = poff; poff += al((long long)d.Nq * d.Nt);
     d.out_off = out;  out += (long long)d.G * d.n_cols;
   }
@@ -418,6 +447,7 @@ static bool layout_tables(mdp_plan *p) {
     hs.piv = p->host_piv.data() + d.piv_off;
   }
   p->out_size = out;
+  p->sep_bytes = sep;
   return true;
 }
 
@@ -431,17 +461,15 @@ static uint16_t f16_of_small_int(int v) {
   return (uint16_t)(sgn | ((unsigned)(e + 15) << 10) | ((a << (10 - e)) & 0x3FFu));
 }
 
-// The B operand of k_inv_cols_tc (the sine factors of the gamma-column sums) for every 16 modes:
-// row n = 8 so + u holds digit u (u < 7; row 7 zero) of output so, where the outputs are, on a
-// centred subdomain, sin(pi q m/Nx) at m = mlo-1, mlo for odd q, then the same for even q (zero
-// at the other parity), else the columns mlo-1, mlo, mhi, mhi+1. A factor s becomes the integer
+// The B operand of k_adj_cols_tc (the sine factors of the adjoint's ring-column sums) for every 16
+// modes: row n = 8 so + u holds digit u (u < 7; row 7 zero) of output so, where the outputs are, on
+// a centred subdomain, sin(pi q m/Nx) at m = mlo, mlo+1 for odd q, then the same for even q (zero
+// at the other parity), else the columns mlo, mlo+1, mhi-1, mhi. A factor s becomes the integer
 // W = round(s 2^50) through the bits of s + 6 (exact: |s| <= 1 keeps the sum in [4, 8)), written
 // in 7 balanced base-256 digits (the bytes of W + 0x0080808080808080, each minus 128). Stored in
 // the operand layout: 8 x 16-byte core matrices, K (the mode) fastest, 128 B between the two
 // K halves and 256 B between groups of 8 rows.
-// inner: the adjoint's ring columns mlo, mlo+1, mhi-1, mhi instead of the gamma columns
-// mlo-1, mlo, mhi, mhi+1 (one column further in on either side)
-static void fill_tc_block(const SubDesc &d, const double *S, uint16_t *blk, bool inner) {
+static void fill_tc_block(const SubDesc &d, const double *S, uint16_t *blk) {
   const int nch = (d.Nq + 15) / 16, N2 = 2 * d.Nx;
   int64_t magic, w;
   const double six = 6.0;
@@ -451,8 +479,8 @@ static void fill_tc_block(const SubDesc &d, const double *S, uint16_t *blk, bool
       for (int kk = 0; kk < 16; ++kk) {
         const int q = c * 16 + 1 + kk;
         int m, par = -1;
-        if (d.xsym) { m = ((so & 1) ? d.mlo : d.mlo - 1) + (inner ? 1 : 0); par = so < 2 ? 1 : 0; }
-        else m = (so == 0 ? d.mlo - 1 : so == 1 ? d.mlo : so == 2 ? d.mhi : d.mhi + 1) + (inner ? (so < 2 ? 1 : -1) : 0);
+        if (d.xsym) { m = (so & 1) ? d.mlo + 1 : d.mlo; par = so < 2 ? 1 : 0; }
+        else m = so == 0 ? d.mlo : so == 1 ? d.mlo + 1 : so == 2 ? d.mhi - 1 : d.mhi;
         const double s = (q <= d.Nq && (par < 0 || (q & 1) == par)) ? S[(int)(((long long)q * m) % N2)] : 0.0;
         const double y = s + six;
         std::memcpy(&w, &y, 8);
@@ -476,10 +504,7 @@ static void fill_tables(mdp_plan *p) {
       S[2 * d.Nx + j] = (2.0 / d.Nx) * S[j];
     }
     for (int i = 0; i < 5 * d.Nq; ++i) p->host_tables[d.seg_off + i] = hs.seg[i];
-    if (d.tc_cols) {
-      fill_tc_block(d, S, reinterpret_cast<uint16_t *>(&p->host_tables[d.tcb_off]), false);
-      fill_tc_block(d, S, reinterpret_cast<uint16_t *>(&p->host_tables[d.tcb_off + 128LL * ((d.Nq + 15) / 16)]), true);
-    }
+    if (d.tc_cols) fill_tc_block(d, S, reinterpret_cast<uint16_t *>(&p->host_tables[d.tcb_off]));
     double *g = &p->host_tables[d.geo_off];
     for (int i = 0; i < d.G; ++i) {
       g[4 * i + 0] = hs.owner[i];
@@ -530,6 +555,13 @@ static void schedule(mdp_plan *p) {
   long long mx = 0;
   for (auto &sc : p->sched)
     for (auto &w : sc) mx = std::max(mx, w.ws_doubles);
+  // one column of source terms: its item and the scratch of launch_source_terms
+  for (auto &hs : p->subs) {
+    const SubDesc &d = hs.d;
+    long long xi, r, gr, y, a, s, red, tot;
+    item_workspace(d, 1, false, xi, r, gr, y, a, s, red, tot);
+    mx = std::max(mx, std::max((long long)d.Nq * d.Nt * 2, tot) + 2LL * d.G + 2LL * d.nx * d.ny + 128);
+  }
   p->ws_doubles = mx;
 }
 

@@ -1,0 +1,83 @@
+"""The separable solve of the projection (kernels_sep.cu) where its tiles and its closed form change:
+row counts around the 16- and 32-row groups, unequal grids along x and y, wavenumbers next to a
+mode's cutoff (hyperbolic and trigonometric form) and grids so coarse that modes alternate in sign,
+single columns, column ranges across the sides, and every receiver row. Bar: the oracle's, 1e-10 of
+a column's largest value."""
+import numpy as np
+import pytest
+
+import workloads as W
+from oracle.projection import APSystem
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+TOL = 1e-10
+
+
+def rel_col_err(got, ref):
+    return float((np.abs(got - ref).max(axis=1) / np.abs(ref).max(axis=1)).max())
+
+
+def box(nx, ny, k, ap, n_modes, dx=0.0):
+    """A rectangle of equal cells with margins of about a tenth (dx more on the left)."""
+    h = 1.2 / (nx - 1)
+    height = h * (ny - 1) / 1.2
+    return W.Subdomain(0.0, 1.0, 0.0, height, -0.1 - dx, -0.1 * height, h, nx + int(round(dx / h)), ny, k, ap, n_modes)
+
+
+def near_cutoff(n, q, shift, ap):
+    """The wavenumber at which mode q's interior rows have e = b + 2a = shift k^2 (cutoff: 0)."""
+    h = 1.2 / (n - 1)
+    lam = -4 * np.sin(np.pi * q / (2 * (n - 1))) ** 2
+    return float(np.sqrt(-(lam / h**2) / ((1 + lam / 12) - shift)))
+
+
+CASES = [(f"n{n}", W.small_subdomain(n, 9.0, W.AP_DIRX_SOMMY, 2)) for n in (15, 17, 38, 40, 41, 42, 59, 60, 61)]
+CASES += [("wide", box(65, 33, 8.0, W.AP_DIRX_SOMMY, 2)), ("tall", box(33, 97, 8.0, W.AP_DIRX_SOMMY, 3)),
+          ("tall_dir4", box(33, 90, 8.0, W.AP_DIRICHLET4, 2)), ("off_centre", box(49, 49, 9.0, W.AP_DIRX_SOMMY_PAPER, 2, dx=0.1)),
+          ("coarse_k", W.small_subdomain(17, 24.0, W.AP_DIRX_SOMMY, 2)), ("coarse_k40", W.small_subdomain(17, 40.0, W.AP_DIRX_SOMMY, 1))]
+CASES += [(f"cutoff_{shift:g}", W.small_subdomain(65, near_cutoff(65, 3, shift, 1), W.AP_DIRX_SOMMY, 2))
+          for shift in (0.0, 1e-14, 1e-9, -1e-9, 1e-4, -1e-4, -1e-2)]
+
+
+@pytest.mark.parametrize("user", [False, True])
+@pytest.mark.parametrize("name,sub", CASES, ids=[c[0] for c in CASES])
+def test_columns_match_the_oracle(mdp, name, sub, user):
+    plan = mdp.Plan([sub])
+    G, nc, _, _ = plan.layout(0)
+    xi = W.random_complex((nc, G), seed=5) if user else None
+    got = plan.project(xi=None if xi is None else torch.from_numpy(xi.ravel()).cuda(), kind="P").cpu().numpy().reshape(nc, G)
+    plan.status()
+    assert rel_col_err(got, APSystem(sub).columns(xi=xi, kind="P")) < TOL
+
+
+@pytest.mark.parametrize("fp64", [False, True])
+def test_column_ranges_and_tiles_give_the_same_columns(mdp, fp64):
+    """Any range of columns (single ones, ranges across the sides) and any tile width: bit for bit
+    the columns of the whole call."""
+    sub = W.small_subdomain(45, 9.0, W.AP_DIRX_SOMMY, 5)
+    plan = mdp.Plan([sub], fp64_cols=fp64)
+    G, nc, _, _ = plan.layout(0)
+    ref = plan.project().view(nc, G)
+    for c0, n in ((0, 1), (9, 1), (10, 1), (3, 14), (8, 5), (19, 2), (29, 11), (0, 40)):
+        assert torch.equal(plan.project_columns(0, c0, n).view(n, G), ref[c0:c0 + n])
+    assert torch.equal(mdp.Plan([sub], fp64_cols=fp64, tile_cols=7).project().view(nc, G), ref)
+
+
+@pytest.mark.parametrize("off", [0.0, 0.1])
+def test_every_receiver_row(mdp, off):
+    sub = box(37, 33, 9.0, W.AP_DIRX_SOMMY, 1, dx=off)
+    plan = mdp.Plan([sub])
+    G, nc, _, nm = plan.layout(0)
+    S = APSystem(sub)
+    xi = plan.basis_densities(0)
+    pot = plan.potential(0, xi).cpu().numpy()
+    nlo, nhi = nm[:, 0].min() + 1, nm[:, 0].max() - 1
+    for row in range(nlo + 1, nhi):
+        plan.set_receivers([row])
+        _, m0, cnt, _ = plan.receiver_layout(0)
+        out, rec = plan.project(out_rec=True)
+        ref = pot[:, row, m0:m0 + cnt]
+        assert rel_col_err(rec[:nc * cnt].cpu().numpy().reshape(nc, cnt), ref) < TOL, row
+    assert rel_col_err(out.cpu().numpy().reshape(nc, G), S.columns()) < TOL
