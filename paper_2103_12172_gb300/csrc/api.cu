@@ -106,6 +106,7 @@ mdp_status alloc_device(mdp_plan *p) {
     for (int q = 1; q <= d.Nq; ++q) mode_entries(d, q, ab[2 * q - 2], ab[2 * q - 1]);
     CK(cudaMemcpy(p->d_sep + d.sep_ab, ab.data(), ab.size() * sizeof(double), cudaMemcpyHostToDevice));
   }
+  CK(launch_sep_sines(p, p->d_subs, p->d_tables, p->d_sep, nullptr));
   CK(launch_sep_tables(p, p->d_subs, p->d_tables, p->d_sep, false, nullptr));
   CK(cudaStreamSynchronize(nullptr));
 #if MDP_CHECKED
@@ -362,6 +363,8 @@ mdp_status mdp_plan_update_k_async(mdp_plan *p, const double *k, void *cuda_stre
     CK(cudaDeviceSynchronize());
     CK(cudaMemcpy(p->alt_tables, p->d_tables, nt, cudaMemcpyDeviceToDevice));
     CK(cudaMemcpy(p->alt_piv, p->d_piv, np, cudaMemcpyDeviceToDevice));
+    CK(launch_sep_sines(p, p->d_subs, p->d_tables, p->alt_sep, nullptr));
+    CK(cudaStreamSynchronize(nullptr));
   }
   const int b = 1 - p->set;
   HostBuf<SubDesc> &stage = stage_of(p, b);
@@ -728,7 +731,7 @@ mdp_status mdp_plan_set_receivers(mdp_plan *p, const int *rows) {
     for (size_t w = 0; w < waves.size(); ++w) {
       const int n = (int)waves[w].items.size();
       auto &pre = hpre[w];
-      for (const Fam f : {F_IREC, F_G1B, F_G1U})
+      for (const Fam f : {F_IREC, F_G1B, F_G1U, F_C3B, F_C3U, F_TCOLS, F_G3U, F_SOUT})
         for (int i = 0; i < n; ++i)
           pre[(size_t)f * (n + 1) + i + 1] =
               pre[(size_t)f * (n + 1) + i] +

@@ -120,6 +120,11 @@ __global__ void __launch_bounds__(256) k_residual(Batch bt, const SubDesc *subs,
   const int b = (local % cb) * 32 + threadIdx.x;
   const int u = (local / cb) * 8 + threadIdx.y;
   const int units = d.xsym ? 4 * d.Ph + 2 * (d.Py - 4) : d.R;
+  if (!GRAD && d.tc_cols) {   // clear the K masks of the separable solve's operands
+    unsigned *mask = reinterpret_cast<unsigned *>(ws + it.a_off + sep_ws(d, it.ncols).mask);
+    const int n = sep_mask_words(it.ncols), stride = 256 * blocks_for(F_RES, d, it.ncols, it.col0);
+    for (int i = local * 256 + threadIdx.y * 32 + threadIdx.x; i < n; i += stride) mask[i] = 0;
+  }
   if (b >= it.ncols || u >= units) return;
   double *r = ws + it.r_off;
   double *sb = ws + it.s_off;
@@ -891,10 +896,6 @@ __device__ __forceinline__ void write_out(const SubDesc &d, const Item &it, cons
   out[it.io_off + (long long)b * d.G + g] = make_double2(v.re, v.im);
 }
 
-// rows per mode of the projection's mode-space field: the swept ones, or the 4 gamma rows and the
-// receiver row that the separable solve keeps
-__device__ __forceinline__ int field_rows(const SubDesc &d) { return d.tc_cols ? 5 : d.NYf; }
-
 // u(m, n) = (2/Nx) sum_q sin(pi q m/Nx) yhat(q, n) for the 4 full gamma rows. Centred
 // subdomains: one thread gives u(m) = E + O and u(Nx - m) = E - O from the odd-q (E) and
 // even-q (O) partial sums, since sin(pi q (Nx-m)/Nx) = (-1)^(q+1) sin(pi q m/Nx).
@@ -905,11 +906,11 @@ __device__ __forceinline__ void inv_rows_body(const Item &it, const SubDesc &d, 
   const int span = d.xsym ? d.Ph + 1 : W;
   const int grow = task / span, dm = task % span, m = d.mlo - 1 + dm;
   const int n = grow == 0 ? d.nlo - 1 : grow == 1 ? d.nlo : grow == 2 ? d.nhi : d.nhi + 1;
-  const int yrow = d.tc_cols ? grow : n - (d.nlo - 1);
+  const int yrow = n - (d.nlo - 1);
   const double *Si = tab + d.sin_off + 2 * d.Nx;
   const int N2 = 2 * d.Nx;
   const double *y = ws + it.y_off;
-  const long long qstride = (long long)field_rows(d) * it.ncols;
+  const long long qstride = (long long)d.NYf * it.ncols;
   const long long base = (long long)yrow * it.ncols + b;
   auto yv = [&](int q) -> cplx {
     const long long o = base + (long long)(q - 1) * qstride;
@@ -954,9 +955,9 @@ __device__ __forceinline__ void inv_rows_fft_body(const Item &it, const SubDesc 
   while ((1 << lg) < N) ++lg;
   const double *sn = tab + d.sin_off;
   const int n = grow == 0 ? d.nlo - 1 : grow == 1 ? d.nlo : grow == 2 ? d.nhi : d.nhi + 1;
-  const int yrow = d.tc_cols ? grow : n - (d.nlo - 1);
+  const int yrow = n - (d.nlo - 1);
   const double *y = ws + it.y_off;
-  const long long qstride = (long long)field_rows(d) * it.ncols;
+  const long long qstride = (long long)d.NYf * it.ncols;
   auto yv = [&](int q, int f) -> cplx {   // yhat(q) of column b0 + f, q = 1 .. N-1
     const long long o = (long long)(q - 1) * qstride + (long long)yrow * it.ncols + b0 + f;
     return CD ? ld2(y + 2 * o) : cmk(y[o], 0.0);
@@ -1101,11 +1102,11 @@ template <bool CD>
 __device__ __forceinline__ void inv_rec_body(const Item &it, const SubDesc &d, const double *tab, const double *ws,
                                              double2 *out_rec, int b, int task) {
   const int m = d.mlo + 1 + task;
-  const int yrow = d.tc_cols ? 4 : d.nrec - (d.nlo - 1);
+  const int yrow = d.nrec - (d.nlo - 1);
   const double *Si = tab + d.sin_off + 2 * d.Nx;
   const int N2 = 2 * d.Nx;
   const double *y = ws + it.y_off;
-  const long long qstride = (long long)field_rows(d) * it.ncols;
+  const long long qstride = (long long)d.NYf * it.ncols;
   const long long base = (long long)yrow * it.ncols + b;
   auto yv = [&](int q) -> cplx {
     const long long o = base + (long long)(q - 1) * qstride;
@@ -1526,9 +1527,9 @@ cudaError_t launch_project(mdp_plan *p, const Batch *fb, int out_kind, const dou
   if (basis) MDP_LAUNCH(F_EXT, k_extend<<<grid1(fb[F_EXT].total_blocks), 128, 0, st>>>(fb[F_EXT], ds, tab, ws, 0));
   if (basis) MDP_LAUNCH(F_RES, k_residual<false, false><<<grid1(fb[F_RES].total_blocks), b8, 0, st>>>(fb[F_RES], ds, tab, ws, xi_user));
   else MDP_LAUNCH(F_RES, k_residual<true, false><<<grid1(fb[F_RES].total_blocks), b8, 0, st>>>(fb[F_RES], ds, tab, ws, xi_user));
-  if (basis) MDP_LAUNCH(F_FROWS, k_fwd_rows<false><<<grid1(fb[F_FROWS].total_blocks), b8, p->fft_smem, st>>>(fb[F_FROWS], ds, tab, ws));
-  else MDP_LAUNCH(F_FROWS, k_fwd_rows<true><<<grid1(fb[F_FROWS].total_blocks), b8, p->fft_smem, st>>>(fb[F_FROWS], ds, tab, ws));
-  cudaError_t e = launch_sep_project(p, fb, out_kind, xi_user, out, 0, st);
+  if (basis) MDP_LAUNCH_AS(F_PROWS, F_FROWS, k_fwd_rows<false><<<grid1(fb[F_PROWS].total_blocks), b8, p->fft_smem, st>>>(fb[F_PROWS], ds, tab, ws));
+  else MDP_LAUNCH_AS(F_PROWS, F_FROWS, k_fwd_rows<true><<<grid1(fb[F_PROWS].total_blocks), b8, p->fft_smem, st>>>(fb[F_PROWS], ds, tab, ws));
+  cudaError_t e = launch_sep_project(p, fb, out_kind, xi_user, out, out_rec, st);
   if (e != cudaSuccess) return e;
   if (p->tri_stages == 4) {
     if (basis) MDP_LAUNCH_AS(F_PTRI, F_TRI, k_tri<false, false, 4><<<grid1(fb[F_PTRI].total_blocks), btri, tri_smem_bytes<false, 4>(), st>>>(fb[F_PTRI], ds, tab, p->d_piv, ws, p->d_sep));
@@ -1544,8 +1545,6 @@ cudaError_t launch_project(mdp_plan *p, const Batch *fb, int out_kind, const dou
     MDP_LAUNCH(F_IROWS, k_inv_rows<true><<<grid1(fb[F_IROWS].total_blocks), b8, p->fft_smem, st>>>(fb[F_IROWS], ds, tab, ws, xi_user, out, out_kind));
     MDP_LAUNCH(F_ICOLS, k_inv_cols<true><<<grid1(fb[F_ICOLS].total_blocks), b8, 0, st>>>(fb[F_ICOLS], ds, tab, ws, xi_user, out, out_kind));
   }
-  e = launch_sep_project(p, fb, out_kind, xi_user, out, 1, st);
-  if (e != cudaSuccess) return e;
   if (out_rec)
     MDP_LAUNCH(F_IREC, k_inv_rec<<<grid1(fb[F_IREC].total_blocks), b8, 0, st>>>(fb[F_IREC], ds, tab, ws, out_rec, basis ? 0 : 1));
   return cudaGetLastError();

@@ -92,28 +92,26 @@ static __device__ __noinline__ bool item_in_bounds(const Batch &bt, const SubDes
     if (MDP_CHECKED && !item_in_bounds(bt, subs, it, local, fam, bt.grad != 0)) return;         \
   } while (0)
 
-// per mode, MTW doubles (phi with their normalisation, rows relative to the ring):
+// Mode table of the separable solve, SEP_MTW doubles per mode (phi with their normalisation):
 enum {
-  MT_P1D = 0,    // phi_1 at the 4 dense rows nlo, nlo+1, nhi-1, nhi
-  MT_P2D = 4,
-  MT_P1G = 8,    // phi_1 at the 4 gamma rows nlo-1, nlo, nhi, nhi+1
-  MT_P2G = 12,
-  MT_R = 16,     // R11, R12, R22 (complex)
-  MT_E1 = 22,    // what a dense row adds to A_1, A_2 on the middle rows through kappa
-  MT_E2 = 26,
-  MT_W1 = 30,    // what the moments add to the field of the 4 gamma rows through kappa
-  MT_W2 = 34,
-  MT_K = 38,     // kappa at 0, 1, 2, L-1, L, L+1 (L = nhi - nlo)
-  MT_REC = 44,   // receiver row: phi_1, phi_2, 1 / (scale of its moment table)
-  MT_T1 = 47,    // kappa(d) = T1 phi_1(J0 + d) + T2 phi_2(J0 + d)
-  MT_T2 = 48,
-  MT_RF = 49,    // scale of the receiver's moment table (a power of two)
-  MT_TH = 50,    // theta, kind, sign, normalisations of phi_1, phi_2 (for k_sep_phi)
-  MT_KIND = 51,
-  MT_SG = 52,
-  MT_N1 = 53,
-  MT_N2 = 54,
-  MT_F = 55,     // 1 / (2 a n1 n2): kappa(i - j) = F (phi_2(i) phi_1(j) - phi_1(i) phi_2(j)), i >= j (kinds 0, 1)
+  MT_MAT = 0,    // [6][6]: what the 4 dense rows' transforms and the 2 moments give, in real numbers, to A_1,
+                 // A_2 and the field at the 4 gamma rows nlo-1, nlo, nhi, nhi+1 (R's real part included)
+  MT_P1D = 36,   // phi_1 at the 4 dense rows nlo, nlo+1, nhi-1, nhi
+  MT_P2D = 40,
+  MT_P1G = 44,   // phi_1 at the 4 gamma rows
+  MT_P2G = 48,
+  MT_R = 52,     // R11, R12, R22 (complex)
+  MT_IMAG = 58,  // 1: R's imaginary part counts (above 2^-62 of kappa's scale)
+  MT_REC = 59,   // receiver row: phi_1, phi_2, 1 / (scale of its moment table)
+  MT_T1 = 62,    // kappa(d) = T1 phi_1(J0 + d) + T2 phi_2(J0 + d)
+  MT_T2 = 63,
+  MT_RF = 64,    // scale of the receiver's moment table (a power of two)
+  MT_TH = 65,    // theta, kind, sign, normalisations of phi_1, phi_2 (for k_sep_phi)
+  MT_KIND = 66,
+  MT_SG = 67,
+  MT_N1 = 68,
+  MT_N2 = 69,
+  MT_F = 70,     // 1 / (2 a n1 n2): kappa(i - j) = F (phi_2(i) phi_1(j) - phi_1(i) phi_2(j)), i >= j (kinds 0, 1)
 };
 static_assert(MT_F < SEP_MTW, "mode table width");
 

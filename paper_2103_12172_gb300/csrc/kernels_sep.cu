@@ -16,9 +16,12 @@
 //   K_sc(d) = (2/Nx) sum_q sin(pi q m_s/Nx) sin(pi q m_c/Nx) kappa_q(d),
 // where A_1, A_2 combine, per mode, the moments sum_{c,j} sin(pi q m_c/Nx) phi_b(j) r_c(j) and the
 // transforms of the 4 dense ring rows. So two contractions (k_sep_gemm) replace the recurrences:
-//   stage 1: r times [K | moment tables], K dimension (c, j);
-//   stage 2 (k_sep_modes): per (mode, column) R, the dense rows, the 4 gamma rows of the field;
-//   stage 3: A times [sines x phi], K dimension (b, q).
+//   stage 1: r times [K | moment tables], K dimension (c, j); the dense rows times sines;
+//   stage 2 (k_sep_modes): per (mode, column) A_1, A_2 and the 4 gamma rows of the field;
+//   stage 3: A times [sines x phi], K dimension (b, q); the gamma rows' field times sines.
+// The sine transforms of the 8 full rows are direct sums too: at up to 1025^2 the tensor cores take
+// less time for N^2/2 exact products (odd and even modes on folded columns) than the FP64 pipe for a
+// length-N FFT, on any N (257^2, 1024 columns: 58 + 117 us by FFT, 4 x 257^2).
 // On x-centred subdomains odd and even modes separate (sums and differences of the mirrored
 // columns), which halves both dimensions: two classes with 2 columns each, else one with 4.
 //
@@ -76,7 +79,7 @@ __global__ void __launch_bounds__(128) k_sep_mode_tab(const SubDesc *subs, int s
   // coarse grids (t > 1/2): x_i = (-1)^i z_i turns (a, b, a) into (-a, b, -a)
   double sg = 1.0;
   if (t > 0.5) { sg = -1.0; t = 1.0 - t; a = -a; }
-  const int N = d.ny - 1, J0 = d.nlo - 1, J1 = d.nhi + 1, L = d.nhi - d.nlo;
+  const int N = d.ny - 1, J0 = d.nlo - 1, J1 = d.nhi + 1;
   const double mid = 0.5 * (J0 + J1), Lh = 0.5 * (J1 - J0);
   const double th = t > 0.0 ? 2.0 * asin(sqrt(t)) : 2.0 * asinh(sqrt(-t));
   const int kind = t > 0.0 ? 0 : th * N < 4.0 ? 1 : 2;
@@ -135,25 +138,42 @@ __global__ void __launch_bounds__(128) k_sep_mode_tab(const SubDesc *subs, int s
   auto p2 = [&](int i) { return sgn(i - J0) * (kind == 2 ? exp(-th * (J1 - i)) : n2 * sep_s(kind, th, i - mid)); };
   auto kap = [&](int x) { return sgn(x) * (kind == 2 ? c * exp(-th * x) : sep_s(kind, th, x) / (2.0 * a)); };
   const double f = 1.0 / (2.0 * a * n1 * n2);
+  // an imaginary part below 2^-62 of kappa's scale is zero to working precision
+  const bool imag = kind < 2 ? d.cplx : fmax(fmax(fabs(R11.im), fabs(R12.im)), fabs(R22.im)) > 0x1p-62 * fabs(c);
+  double *mat = T + MT_MAT;
   for (int r = 0; r < 4; ++r) {
-    const int j = rows_d[r], n = rows_g[r];
-    const double up = r < 2 ? 1.0 : -1.0;   // dense rows 0, 1 lie below the middle rows
-    T[MT_P1D + r] = p1(j); T[MT_P2D + r] = p2(j);
-    T[MT_P1G + r] = p1(n); T[MT_P2G + r] = p2(n);
-    if (kind < 2) {
-      T[MT_E1 + r] = -up * f * p2(j); T[MT_E2 + r] = up * f * p1(j);
-      T[MT_W1 + r] = -up * f * p2(n); T[MT_W2 + r] = up * f * p1(n);
-    } else {
-      T[MT_E1 + r] = r < 2 ? c * exp(th * (j - J0)) * sgn(j - J0) : 0.0;
-      T[MT_E2 + r] = r < 2 ? 0.0 : c * exp(th * (J1 - j)) * sgn(j - J0);
-      T[MT_W1 + r] = r < 2 ? c * exp(th * (n - J0)) * sgn(n - J0) : 0.0;
-      T[MT_W2 + r] = r < 2 ? 0.0 : c * exp(th * (J1 - n)) * sgn(n - J0);
+    T[MT_P1D + r] = p1(rows_d[r]); T[MT_P2D + r] = p2(rows_d[r]);
+    T[MT_P1G + r] = p1(rows_g[r]); T[MT_P2G + r] = p2(rows_g[r]);
+  }
+  for (int k = 0; k < 6; ++k) {   // inputs: dense rows, moments
+    const double f1 = k < 4 ? T[MT_P1D + k] : k == 4 ? 1.0 : 0.0, f2 = k < 4 ? T[MT_P2D + k] : k == 5 ? 1.0 : 0.0;
+    const double A = fma(R11.re, f1, R12.re * f2), B = fma(R12.re, f1, R22.re * f2);
+    double E1 = 0.0, E2 = 0.0;    // a dense row through kappa, on the middle rows
+    if (k < 4) {
+      const int j = rows_d[k];
+      const double up = k < 2 ? 1.0 : -1.0;   // dense rows 0, 1 lie below the middle rows
+      if (kind < 2) { E1 = -up * f * f2; E2 = up * f * f1; }
+      else if (k < 2) E1 = c * exp(th * (j - J0)) * sgn(j - J0);
+      else E2 = c * exp(th * (J1 - j)) * sgn(j - J0);
+    }
+    mat[k] = A + E1;
+    mat[6 + k] = B + E2;
+    for (int r = 0; r < 4; ++r) {
+      const int n = rows_g[r];
+      double w;                   // the input's field at gamma row n through kappa
+      if (k < 4) w = kap(abs(n - rows_d[k]));
+      else {
+        const double up = r < 2 ? 1.0 : -1.0;   // gamma rows 0, 1 lie below the middle rows
+        if (kind < 2) w = k == 4 ? -up * f * T[MT_P2G + r] : up * f * T[MT_P1G + r];
+        else if (k == 4) w = r < 2 ? c * exp(th * (n - J0)) * sgn(n - J0) : 0.0;
+        else w = r < 2 ? 0.0 : c * exp(th * (J1 - n)) * sgn(n - J0);
+      }
+      mat[6 * (2 + r) + k] = fma(T[MT_P1G + r], A, fma(T[MT_P2G + r], B, w));
     }
   }
   T[MT_R + 0] = R11.re; T[MT_R + 1] = R11.im; T[MT_R + 2] = R12.re; T[MT_R + 3] = R12.im;
   T[MT_R + 4] = R22.re; T[MT_R + 5] = R22.im;
-  T[MT_K + 0] = kap(0); T[MT_K + 1] = kap(1); T[MT_K + 2] = kap(2);
-  T[MT_K + 3] = kap(L - 1); T[MT_K + 4] = kap(L); T[MT_K + 5] = kap(L + 1);
+  T[MT_IMAG] = imag ? 1.0 : 0.0;
   T[MT_REC + 0] = d.nrec >= 0 ? p1(d.nrec) : 0.0;
   T[MT_REC + 1] = d.nrec >= 0 ? p2(d.nrec) : 0.0;
   T[MT_REC + 2] = 1.0 / rf;
@@ -378,51 +398,84 @@ __global__ void __launch_bounds__(256) k_sep_b3(const SubDesc *subs, int s0, con
   store_digits(B + (o >> 3) * 256 + half * 128 + (o & 7) * 16, 1024, V);
 }
 
+// The sine tables of the full rows' transforms. FWD: output q of parity e, K index m' - mf; INV: output
+// m' - mg, K index q of parity e; both sin(pi q m'/Nx) over the folded columns m' <= Nx/2.
+__global__ void __launch_bounds__(256) k_sep_sines(const SubDesc *subs, int s0, const double *tab, unsigned char *sep, int inv) {
+  const int si = s0 + blockIdx.z;
+  const SubDesc &d = subs[si];
+  if (!d.tc_cols || d.leader != si) return;
+  const SepGeo g = sep_geo(d);
+  const int nto = inv ? g.ntg : g.nqh / 32, nk = inv ? g.nqh / 16 : g.nkf;
+  const int e = blockIdx.y / nto, to = blockIdx.y % nto;
+  const int kb = blockIdx.x * 4 + (threadIdx.x >> 6);
+  if (e >= 2 || kb >= nk) return;
+  const int o = threadIdx.x & 31, half = (threadIdx.x >> 5) & 1;
+  const double *S = tab + d.sin_off;
+  long long V[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const int ko = to * 32 + o, kk = kb * 16 + 8 * half + j;
+    const int q = sep_parity_mode(e, inv ? kk : ko), m = inv ? g.mg + ko : g.mf + kk;
+    V[j] = q <= d.Nq && 2 * m <= d.Nx ? fix54(S[(int)(((long long)q * m) % (2 * d.Nx))]) : 0;
+  }
+  unsigned char *B = sep + (inv ? d.sep_bi : d.sep_bf) + (((long long)e * nto + to) * nk + kb) * SEP_BBLK;
+  store_digits(B + (o >> 3) * 256 + half * 128 + (o & 7) * 16, 1024, V);
+}
+
 // ---------------------------------------------------------------- operand A
-// Cut the rows of A (stage 1: ring residuals of the middle rows, stage 3: the modes' A_b) into
-// digits in the MMA's operand layout, per 128 rows and 16 values of K 7 x 4 KiB. A block takes 8
-// rows of one class (one core-matrix row group): their largest exponents first, then the digits;
-// the values are read twice, the second time from L1/L2.
-template <bool CIN, int STAGE>
-__global__ void __launch_bounds__(256) k_sep_cut(Batch bt, const SubDesc *subs, double *ws, int fam) {
-  Item it; int local;
-  locate(bt, blockIdx.x, it, local);
-  MDP_CHECK_ITEM(bt, subs, it, local, fam);
-  const SubDesc &d = subs[it.sub];
+// Cut the rows of A into digits in the MMA's operand layout, per 128 rows and 16 values of K 7 x 4 KiB:
+//   MID: ring residuals of the middle rows, FWD: of the dense rows (folded columns),
+//   SYN: A_b of the modes, INV: the modes' field at the rows to transform back.
+// A block takes 8 rows of one class (one core-matrix row group): their largest exponents first, then
+// the digits; the values are read twice, the second time from L1/L2. Groups of 16 values of K whose
+// digits are all zero in 128 rows (the imaginary parts of evanescent modes, the ring away from a
+// column's side) are left out of the contraction by their bit in the tile's mask.
+template <bool CIN, int JOB>
+__device__ __forceinline__ void sep_cut_body(const Item &it, const SubDesc &d, double *ws, int local) {
   const SepGeo g = sep_geo(d);
   const SepWs w = sep_ws(d, it.ncols);
-  const int R = STAGE == 1 ? sep_rows1(d, it.ncols, it.col0, CIN) : sep_rows3(d, it.ncols, CIN);
+  const int R = sep_rows(d, JOB, it.ncols, it.col0, CIN);
   const int e = local / (R / 8), row = (local % (R / 8)) * 8 + (threadIdx.x & 7), kl = threadIdx.x >> 3;
-  const int cp = sep_pad128(it.ncols), nk = STAGE == 1 ? g.nk1 : g.nk3;
+  const int cp = sep_pad128(it.ncols), nk = sep_nk(g, JOB);
   const long long nc = it.ncols;
   // the row's column and part, and its values
-  bool live;
-  const double *src;
-  long long sk;   // stage 3: step between consecutive K
-  int part = 0, col = 0;
-  if (STAGE == 1) {
-    if (CIN) { part = row / cp; col = row % cp; live = col < it.ncols; }
-    else { live = row < sep_side_cols(d, it.col0, it.ncols); col = live ? sep_side_col(d, it.col0, row) - it.col0 : 0; }
-    src = ws + it.r_off;
-    sk = 0;
-  } else {
-    col = row % cp;
-    live = col < it.ncols;
-    src = ws + it.a_off + w.aeff + (long long)e * 2 * g.nqp * R + row;
-    sk = R;
+  constexpr bool IN = JOB == J_MID || JOB == J_FWD;
+  const int parts = IN ? (CIN ? 2 : 1) : (d.cplx || CIN ? 2 : 1);
+  int col = row % cp, part = (row / cp) % parts;
+  const int rr = row / (cp * parts);
+  bool live = col < it.ncols;
+  if (JOB == J_MID && !CIN) {
+    live = row < sep_side_cols(d, it.col0, it.ncols);
+    col = live ? sep_side_col(d, it.col0, row) - it.col0 : 0;
+    part = 0;
   }
+  const double *src = JOB == J_SYN ? ws + it.a_off + w.aeff + (long long)e * 2 * g.nqp * R + row
+                      : JOB == J_INV ? ws + it.y_off : ws + it.r_off;
+  auto ring = [&](long long slot) { return CIN ? src[2 * (slot * nc + col) + part] : src[slot * nc + col]; };
   auto value = [&](int k) -> double {
-    if (STAGE == 1) {
+    if (!live) return 0.0;
+    if (JOB == J_MID) {
       const int c = k / (16 * g.nkj), j = k - c * 16 * g.nkj;
-      if (!live || j >= g.Pj) return 0.0;
-      const long long slot = d.xsym ? 8LL * d.Ph + 4 * j + 2 * c + e : 2LL * d.Px + 4 * j + c;
-      return CIN ? src[2 * (slot * nc + col) + part] : src[slot * nc + col];
+      if (j >= g.Pj) return 0.0;
+      return ring(d.xsym ? 8LL * d.Ph + 4 * j + 2 * c + e : 2LL * d.Px + 4 * j + c);
     }
-    const int qi = k % g.nqp;
-    return live && sep_mode(d, e, qi) <= d.Nq ? src[(long long)k * sk] : 0.0;
+    if (JOB == J_FWD) {
+      if (k >= g.Kf) return 0.0;
+      if (d.xsym) return ring((long long)rr * 2 * d.Ph + 2 * k + e);
+      const long long rb = rr < 2 ? (long long)rr * d.Px : (long long)rr * d.Px + 4 * (d.Py - 4);
+      const int m = g.mf + k, m2 = d.Nx - m;
+      const double a = m >= d.mlo && m <= d.mhi ? ring(rb + m - d.mlo) : 0.0;
+      const double b = m2 != m && m2 >= d.mlo && m2 <= d.mhi ? ring(rb + m2 - d.mlo) : 0.0;
+      return e == 0 ? a + b : a - b;
+    }
+    if (JOB == J_SYN) return sep_mode(d, e, k % g.nqp) <= d.Nq ? src[(long long)k * R] : 0.0;
+    const int q = sep_parity_mode(e, k);
+    const long long o = ((long long)(q - 1) * 5 + rr) * nc + col;
+    return q <= d.Nq ? (parts == 2 ? src[2 * o + part] : src[o]) : 0.0;
   };
   __shared__ int emax[8];
-  if (threadIdx.x < 8) emax[threadIdx.x] = 0;
+  __shared__ unsigned smask[SEP_MASK];
+  if (threadIdx.x < 8) { emax[threadIdx.x] = 0; smask[threadIdx.x] = 0; }
   __syncthreads();
   int m = 0;
   for (int k8 = kl; k8 < 2 * nk; k8 += 32)
@@ -432,17 +485,38 @@ __global__ void __launch_bounds__(256) k_sep_cut(Batch bt, const SubDesc *subs, 
   if ((threadIdx.x & 31) < 8) atomicMax(&emax[threadIdx.x & 7], m);
   __syncthreads();
   const int E = max(emax[threadIdx.x & 7], 53);
-  if (kl == 0) reinterpret_cast<int *>(ws + it.a_off + (STAGE == 1 ? w.ex1 : w.ex3))[e * R + row] = E;
+  if (kl == 0) reinterpret_cast<int *>(ws + it.a_off + w.ex[JOB])[e * R + row] = E;
   const double sc = pow2i(1076 - E);          // |x| < 2^(E - 1022) -> |V| < 2^54
-  unsigned char *A = reinterpret_cast<unsigned char *>(ws + it.a_off + (STAGE == 1 ? w.a1 : w.a3)) +
+  unsigned char *A = reinterpret_cast<unsigned char *>(ws + it.a_off + w.a[JOB]) +
                      ((long long)(e * (R / 128) + row / 128) * nk) * SEP_ABLK;
   const int r = row & 127, off0 = (r >> 3) * 256 + (r & 7) * 16;
   for (int k8 = kl; k8 < 2 * nk; k8 += 32) {
-    long long V[8];
+    long long V[8], any = 0;
 #pragma unroll
-    for (int j = 0; j < 8; ++j) V[j] = E < 2047 ? __double2ll_rn(value(8 * k8 + j) * sc) : 0;
+    for (int j = 0; j < 8; ++j) {
+      V[j] = E < 2047 ? __double2ll_rn(value(8 * k8 + j) * sc) : 0;
+      any |= V[j];
+    }
+    if (any) atomicOr(&smask[k8 >> 6], 1u << ((k8 >> 1) & 31));
     store_digits(A + (long long)(k8 >> 1) * SEP_ABLK + off0 + (k8 & 1) * 128, 4096, V);
   }
+  __syncthreads();
+  if (threadIdx.x < SEP_MASK && smask[threadIdx.x])
+    atomicOr(reinterpret_cast<unsigned *>(ws + it.a_off + w.mask) + sep_mask_of(JOB, it.ncols) +
+                 (e * (R / 128) + row / 128) * SEP_MASK + threadIdx.x,
+             smask[threadIdx.x]);
+}
+
+template <bool CIN, int STAGE>
+__global__ void __launch_bounds__(256) k_sep_cut(Batch bt, const SubDesc *subs, double *ws, int fam) {
+  Item it; int local;
+  locate(bt, blockIdx.x, it, local);
+  MDP_CHECK_ITEM(bt, subs, it, local, fam);
+  const SubDesc &d = subs[it.sub];
+  constexpr int J0 = STAGE == 1 ? J_MID : J_SYN, J1 = STAGE == 1 ? J_FWD : J_INV;
+  const int n0 = sep_cut_blocks(d, sep_geo(d), J0, it.ncols, it.col0, CIN);
+  if (local < n0) sep_cut_body<CIN, J0>(it, d, ws, local);
+  else sep_cut_body<CIN, J1>(it, d, ws, local - n0);
 }
 
 // ---------------------------------------------------------------- the contractions
@@ -481,15 +555,25 @@ __device__ __forceinline__ void bulk_load(unsigned dst, const void *src, unsigne
                : "memory");
 }
 
-struct SepTile { int e, mt, nt, R; };
+struct SepTile {
+  int job, e, mt, nt, R, nk;
+  const unsigned *mask;   // groups of K with nonzero digits in the tile's rows
+};
 template <int STAGE>
-__device__ __forceinline__ SepTile sep_tile(const SubDesc &d, const SepGeo &g, const Item &it, int local, bool user) {
+__device__ __forceinline__ SepTile sep_tile(const SubDesc &d, const SepGeo &g, const SepWs &w, const Item &it, int local,
+                                            bool user, const double *ws) {
   SepTile t;
-  t.R = STAGE == 1 ? sep_rows1(d, it.ncols, it.col0, user) : sep_rows3(d, it.ncols, user);
-  const int nt = STAGE == 1 ? g.nt1 : g.nt3, per = (t.R / 128) * nt;
+  t.job = STAGE == 1 ? J_MID : J_SYN;
+  const int n0 = sep_tiles(d, g, t.job, it.ncols, it.col0, user);
+  if (local >= n0) { ++t.job; local -= n0; }
+  t.R = sep_rows(d, t.job, it.ncols, it.col0, user);
+  t.nk = sep_nk(g, t.job);
+  const int nt = sep_nt(g, t.job), per = (t.R / 128) * nt;
   t.e = local / per;
   t.mt = (local % per) / nt;
   t.nt = local % nt;
+  t.mask = reinterpret_cast<const unsigned *>(ws + it.a_off + w.mask) + sep_mask_of(t.job, it.ncols) +
+           (t.e * (t.R / 128) + t.mt) * SEP_MASK;
   return t;
 }
 
@@ -536,26 +620,29 @@ __global__ void __launch_bounds__(SG_THREADS, 1)
         const SubDesc &d = subs[it.sub];
         const SepGeo g = sep_geo(d);
         const SepWs w = sep_ws(d, it.ncols);
-        const SepTile t = sep_tile<STAGE>(d, g, it, local, user);
-        const int nk = STAGE == 1 ? g.nk1 : g.nk3;
-        const unsigned char *A = reinterpret_cast<const unsigned char *>(ws + it.a_off + (STAGE == 1 ? w.a1 : w.a3)) +
-                                 (long long)(t.e * (t.R / 128) + t.mt) * nk * SEP_ABLK;
+        const SepTile t = sep_tile<STAGE>(d, g, w, it, local, user, ws);
+        const unsigned char *A = reinterpret_cast<const unsigned char *>(ws + it.a_off + w.a[t.job]) +
+                                 (long long)(t.e * (t.R / 128) + t.mt) * t.nk * SEP_ABLK;
         const unsigned char *B;
         int ti = 0;
-        const bool toep = STAGE == 1 && t.nt < g.nS * g.nti;
-        if (STAGE == 3) B = sep + d.sep_b3 + ((long long)t.e * g.nt3 + t.nt) * g.nk3 * SEP_BBLK;
+        const bool toep = t.job == J_MID && t.nt < g.nt3;
+        if (t.job == J_SYN) B = sep + d.sep_b3 + ((long long)t.e * g.nt3 + t.nt) * t.nk * SEP_BBLK;
+        else if (t.job == J_INV) B = sep + d.sep_bi + ((long long)t.e * g.ntg + t.nt) * t.nk * SEP_BBLK;
+        else if (t.job == J_FWD) B = sep + d.sep_bf + ((long long)t.e * (g.nqh / 32) + t.nt) * t.nk * SEP_BBLK;
         else if (toep) { ti = t.nt % g.nti; B = sep + d.sep_tb + ((long long)(t.e * g.nS + t.nt / g.nti) * g.nS) * g.ND * SEP_BBLK; }
-        else B = sep + d.sep_mb + ((long long)t.e * (3 * g.nqp / 32) + t.nt - g.nS * g.nti) * g.nk1 * SEP_BBLK;
+        else B = sep + d.sep_mb + ((long long)t.e * (3 * g.nqp / 32) + t.nt - g.nt3) * t.nk * SEP_BBLK;
         bool ok = true;
-        for (int kb = 0; kb < nk; ++kb, ++gs) {
-          const unsigned st = gs % SG_STAGES;
-          if (gs >= SG_STAGES && !mbar_wait(smem_u32(&empty_bar[st]), (gs / SG_STAGES - 1) & 1u, &abort_sh)) { ok = false; break; }
-          const unsigned bar = smem_u32(&full_bar[st]);
-          asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(SG_STAGE_BYTES) : "memory");
-          bulk_load(sbase + st * SEP_ABLK, A + (long long)kb * SEP_ABLK, SEP_ABLK, bar);
-          const long long bo = toep ? (long long)(kb / g.nkj) * g.ND + 2 * ti - kb % g.nkj + g.nkj - 1 : kb;
-          bulk_load(sbase + SG_B0 + (2 * st + 1) * SEP_BBLK, B + bo * SEP_BBLK, SEP_BBLK, bar);
-        }
+        for (int wd = 0; wd < SEP_MASK && ok; ++wd)
+          for (unsigned bits = t.mask[wd]; bits; bits &= bits - 1, ++gs) {
+            const int kb = 32 * wd + __ffs(bits) - 1;
+            const unsigned st = gs % SG_STAGES;
+            if (gs >= SG_STAGES && !mbar_wait(smem_u32(&empty_bar[st]), (gs / SG_STAGES - 1) & 1u, &abort_sh)) { ok = false; break; }
+            const unsigned bar = smem_u32(&full_bar[st]);
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(SG_STAGE_BYTES) : "memory");
+            bulk_load(sbase + st * SEP_ABLK, A + (long long)kb * SEP_ABLK, SEP_ABLK, bar);
+            const long long bo = toep ? (long long)(kb / g.nkj) * g.ND + 2 * ti - kb % g.nkj + g.nkj - 1 : kb;
+            bulk_load(sbase + SG_B0 + (2 * st + 1) * SEP_BBLK, B + bo * SEP_BBLK, SEP_BBLK, bar);
+          }
         if (!ok) break;
       }
       // leave only when every copy issued has landed (each wait bounded)
@@ -574,23 +661,26 @@ __global__ void __launch_bounds__(SG_THREADS, 1)
         Item it; int local;
         locate(bt, v, it, local);
         if (MDP_CHECKED && !item_in_bounds(bt, subs, it, local, fam, false)) continue;
-        const SepGeo g = sep_geo(subs[it.sub]);
-        const int nk = STAGE == 1 ? g.nk1 : g.nk3;
+        const SubDesc &d = subs[it.sub];
+        const SepGeo g = sep_geo(d);
+        const SepTile t = sep_tile<STAGE>(d, g, sep_ws(d, it.ncols), it, local, user, ws);
+        int n = 0;   // steps: groups of K left by the mask
+        for (int wd = 0; wd < SEP_MASK; ++wd) n += __popc(t.mask[wd]);
         bool ok = true;
-        for (int kb = 0; kb < nk && ok; ++cc) {
+        for (int s = 0; s < n && ok; ++cc) {
           const unsigned buf = cc & 1u, D = tmem + 256u * buf;
           if (cc >= 2 && !mbar_wait(smem_u32(&tempty_bar[buf]), ((cc >> 1) - 1) & 1u, &abort_sh)) { ok = false; break; }
           tc_fence_after();
-          const int kend = min(nk, kb + SG_CHUNK);
-          for (bool first = true; kb < kend; ++kb, ++gs, first = false) {
+          const int send = min(n, s + SG_CHUNK);
+          for (bool first = true; s < send; ++s, ++gs, first = false) {
             const unsigned st = gs % SG_STAGES;
             if (!mbar_wait(smem_u32(&full_bar[st]), (gs / SG_STAGES) & 1u, &abort_sh)) { ok = false; break; }
             tc_fence_after();
             const unsigned a0 = sbase + st * SEP_ABLK, b0 = sbase + SG_B0 + (2 * st + 1) * SEP_BBLK;
 #pragma unroll
-            for (int t = 0; t < 7; ++t)
-              tc_mma(D, smem_desc(a0 + 4096 * t, 128, 256), smem_desc(b0 - 1024 * t, 128, 256), f16_idesc(256),
-                     first && t == 0 ? 0u : 1u);
+            for (int dg = 0; dg < 7; ++dg)
+              tc_mma(D, smem_desc(a0 + 4096 * dg, 128, 256), smem_desc(b0 - 1024 * dg, 128, 256), f16_idesc(256),
+                     first && dg == 0 ? 0u : 1u);
             tc_commit(smem_u32(&empty_bar[st]));
           }
           if (ok) tc_commit(smem_u32(&tfull_bar[buf]));
@@ -615,14 +705,15 @@ __global__ void __launch_bounds__(SG_THREADS, 1)
       const SubDesc &d = subs[it.sub];
       const SepGeo g = sep_geo(d);
       const SepWs w = sep_ws(d, it.ncols);
-      const SepTile t = sep_tile<STAGE>(d, g, it, local, user);
-      const int nk = STAGE == 1 ? g.nk1 : g.nk3;
+      const SepTile t = sep_tile<STAGE>(d, g, w, it, local, user, ws);
+      int n = 0;
+      for (int wd = 0; wd < SEP_MASK; ++wd) n += __popc(t.mask[wd]);
       // weights 0..3 and 4..7 of 16 outputs, as sums of I_w 2^(8 (3 - w)), I_w 2^(8 (7 - w))
       long long hi[16], lo[16];
 #pragma unroll
       for (int o = 0; o < 16; ++o) hi[o] = lo[o] = 0;
       bool ok = true;
-      for (int kb = 0; kb < nk; kb += SG_CHUNK, ++cc) {
+      for (int s = 0; s < n; s += SG_CHUNK, ++cc) {
         const unsigned buf = cc & 1u;
         if (!mbar_wait(smem_u32(&tfull_bar[buf]), (cc >> 1) & 1u, &abort_sh)) { ok = false; break; }
         tc_fence_after();
@@ -644,22 +735,32 @@ __global__ void __launch_bounds__(SG_THREADS, 1)
       if (!ok) break;
       // value = (hi 2^32 + lo) 2^40 2^(E - 1022 - 54) 2^(eb - 54)
       const int row = t.mt * 128 + 32 * quarter + lane;
-      const int E = reinterpret_cast<const int *>(ws + it.a_off + (STAGE == 1 ? w.ex1 : w.ex3))[t.e * t.R + row];
-      const bool direct = STAGE == 3 || t.nt < g.nS * g.nti;
+      const int E = reinterpret_cast<const int *>(ws + it.a_off + w.ex[t.job])[t.e * t.R + row];
+      const bool direct = t.job == J_MID && t.nt < g.nt3;
       int eb = 0;
-      if (STAGE == 1 && direct) eb = reinterpret_cast<const int *>(sep + d.sep_kde)[t.e * g.nS + t.nt / g.nti];
+      if (direct) eb = reinterpret_cast<const int *>(sep + d.sep_kde)[t.e * g.nS + t.nt / g.nti];
       double s0 = pow2i(E - 1090 + eb), s1 = pow2i(E - 1058 + eb);
       if (E >= 2047) s0 = s1 = __longlong_as_double(0x7ff8000000000000LL);   // Inf or NaN in the row
       double *dst;
-      int cnt;
-      if (direct) {
+      int cnt;                   // outputs of this thread, `step` doubles apart
+      long long step = t.R;
+      const int o0 = t.nt * 32 + 16 * half;
+      if (t.job == J_SYN || direct) {
         const int i0 = (t.nt % g.nti) * 32 + 16 * half;
         cnt = g.Pi - i0;
-        dst = ws + it.a_off + (STAGE == 1 ? w.u1 : w.u3) + ((long long)(t.e * g.nS + t.nt / g.nti) * g.Pi + i0) * t.R + row;
-      } else {
-        const int o0 = (t.nt - g.nS * g.nti) * 32 + 16 * half;
+        dst = ws + it.a_off + (direct ? w.u1 : w.u3) + ((long long)(t.e * g.nS + t.nt / g.nti) * g.Pi + i0) * t.R + row;
+      } else if (t.job == J_MID) {
         cnt = 16;
-        dst = ws + it.a_off + w.mom + ((long long)t.e * 3 * g.nqp + o0) * t.R + row;
+        dst = ws + it.a_off + w.mom + ((long long)t.e * 3 * g.nqp + o0 - 32 * g.nt3) * t.R + row;
+      } else if (t.job == J_INV) {
+        cnt = g.Ng - o0;
+        dst = ws + it.a_off + w.ui + ((long long)t.e * g.Ng + o0) * t.R + row;
+      } else {                   // the dense rows' transforms: modes q = 2 (o0 + o) + 1 + e
+        const int cp = sep_pad128(it.ncols), parts = user ? 2 : 1, col = row % cp;
+        cnt = col < it.ncols ? (d.Nq - (1 + t.e) - 2 * o0) / 2 + 1 : 0;
+        if (2 * o0 + (1 + t.e) > d.Nq) cnt = 0;
+        step = 2LL * it.ncols * parts;
+        dst = ws + it.gr_off + (((long long)(row / (cp * parts)) * d.Nq + 2 * o0 + t.e) * it.ncols + col) * parts + (row / cp) % parts;
       }
       constexpr long long MG = 0x4338000000000000LL;   // 1.5 2^52 + x for |x| < 2^51
       const double M = __longlong_as_double(MG);
@@ -669,7 +770,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1)
           // carry the part of lo above 2^32 into hi: both then lie below 2^51
           const long long h = hi[o] + (lo[o] >> 32), l = lo[o] & 0xffffffffLL;
           const double dh = __longlong_as_double(MG + h) - M, dl = __longlong_as_double(MG + l) - M;
-          dst[(long long)o * t.R] = fma(dh, s1, dl * s0);
+          dst[o * step] = fma(dh, s1, dl * s0);
         }
     }
   }
@@ -682,77 +783,77 @@ __global__ void __launch_bounds__(SG_THREADS, 1)
 }
 
 // ---------------------------------------------------------------- stage 2
-// Per (mode, column): the coefficients A_1, A_2 of the homogeneous part on the middle rows (from the
-// moments, the dense rows and R) and the field at the 4 gamma rows (+ the receiver row), which
-// k_inv_rows / k_inv_rec transform back. CD: complex results (Sommerfeld AP or complex data).
+// Per (mode, column): the coefficients A_1, A_2 of the homogeneous part on the middle rows and the field
+// at the 4 gamma rows (+ the receiver row) from the 4 dense rows' transforms and the moments: a 6 x 6
+// real matrix per mode (36 FMAs a part), and where R has an imaginary part 20 more. CD: complex
+// results (Sommerfeld AP or complex data). FP64-bound.
 template <bool CD, bool CIN>
-__device__ __forceinline__ void sep_modes_body(const Item &it, const SubDesc &d, const unsigned char *sep, double *ws, int b,
-                                               int q) {
-  const SepGeo g = sep_geo(d);
-  const SepWs w = sep_ws(d, it.ncols);
+__device__ __forceinline__ void sep_modes_body(const Item &it, const SubDesc &d, const SepGeo &g, const SepWs &w,
+                                               const unsigned char *sep, double *ws, int b, int row1, int q) {
   const double *T = reinterpret_cast<const double *>(sep + d.sep_mt) + (long long)(q - 1) * SEP_MTW;
   const int e = d.xsym ? ((q & 1) ? 0 : 1) : 0, qi = d.xsym ? (q - 1) >> 1 : q - 1;
-  const int cp = sep_pad128(it.ncols), R1 = sep_rows1(d, it.ncols, it.col0, CIN), R3 = sep_rows3(d, it.ncols, CIN);
+  const int cp = sep_pad128(it.ncols), R1 = sep_rows(d, J_MID, it.ncols, it.col0, CIN), R3 = (CD ? 2 : 1) * cp;
   const long long nc = it.ncols;
   const double *gr = ws + it.gr_off;
-  const double *mom = ws + it.a_off + w.mom + ((long long)e * 3 * g.nqp + qi) * R1;
-  cplx gd[4], M[3];
+  const double *mom = ws + it.a_off + w.mom + ((long long)e * 3 * g.nqp + qi) * R1 + row1;
+  const bool rec = d.nrec >= 0;
+  constexpr int P = CIN ? 2 : 1;
+  double in[P][6], m3[P], out[2][6];   // [part][input], [part][output]
 #pragma unroll
   for (int r = 0; r < 4; ++r) {
     const long long o = ((long long)r * d.Nq + (q - 1)) * nc + b;
-    gd[r] = CIN ? ld2(gr + 2 * o) : cmk(gr[o], 0.0);
+    if (CIN) { const cplx v = ld2(gr + 2 * o); in[0][r] = v.re; in[P - 1][r] = v.im; }
+    else in[0][r] = gr[o];
   }
-  const bool rec = d.nrec >= 0;
-  const int row1 = CIN ? b : sep_side_row(d, it.col0, b);   // -1: no source on the middle rows
 #pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    M[k] = cmk(0.0, 0.0);
-    if (row1 < 0 || (k == 2 && !rec)) continue;
-    const double *p = mom + (long long)k * g.nqp * R1 + row1;
-    M[k] = cmk(p[0], CIN ? p[cp] : 0.0);
+  for (int p = 0; p < P; ++p) {        // row1 < 0: no source on the middle rows
+    in[p][4] = row1 >= 0 ? mom[p * cp] : 0.0;
+    in[p][5] = row1 >= 0 ? mom[(long long)g.nqp * R1 + p * cp] : 0.0;
+    m3[p] = rec && row1 >= 0 ? mom[2LL * g.nqp * R1 + p * cp] : 0.0;
   }
-  auto axpy = [&](double s, cplx x, cplx y) { return CIN ? caxpy(s, x, y) : cmk(fma(s, x.re, y.re), 0.0); };
-  cplx m1 = M[0], m2 = M[1], k1 = cmk(0.0, 0.0), k2 = cmk(0.0, 0.0);
 #pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    m1 = axpy(T[MT_P1D + r], gd[r], m1);
-    m2 = axpy(T[MT_P2D + r], gd[r], m2);
-    k1 = axpy(T[MT_E1 + r], gd[r], k1);
-    k2 = axpy(T[MT_E2 + r], gd[r], k2);
+  for (int o = 0; o < 6; ++o)
+#pragma unroll
+    for (int p = 0; p < P; ++p) {
+      double v = T[MT_MAT + 6 * o] * in[p][0];
+#pragma unroll
+      for (int k = 1; k < 6; ++k) v = fma(T[MT_MAT + 6 * o + k], in[p][k], v);
+      out[p][o] = v;
+    }
+  if (CD && !CIN)
+#pragma unroll
+    for (int o = 0; o < 6; ++o) out[1][o] = 0.0;
+  if (CD && T[MT_IMAG] != 0.0) {       // i Im R times the moments of all rows
+#pragma unroll
+    for (int p = 0; p < P; ++p) {
+      double m1 = in[p][4], m2 = in[p][5];
+#pragma unroll
+      for (int r = 0; r < 4; ++r) { m1 = fma(T[MT_P1D + r], in[p][r], m1); m2 = fma(T[MT_P2D + r], in[p][r], m2); }
+      double A = fma(T[MT_R + 1], m1, T[MT_R + 3] * m2), B = fma(T[MT_R + 3], m1, T[MT_R + 5] * m2);
+      if (p == 1) { A = -A; B = -B; }
+      out[1 - p][0] += A;
+      out[1 - p][1] += B;
+#pragma unroll
+      for (int r = 0; r < 4; ++r) out[1 - p][2 + r] = fma(T[MT_P1G + r], A, fma(T[MT_P2G + r], B, out[1 - p][2 + r]));
+    }
   }
-  const cplx R11 = ld2(T + MT_R), R12 = ld2(T + MT_R + 2), R22 = ld2(T + MT_R + 4);
-  auto rmul = [&](cplx R, cplx m) -> cplx {
-    if (!CD) return cmk(R.re * m.re, 0.0);
-    if (!CIN) return cmk(R.re * m.re, R.im * m.re);
-    return cmul(R, m);
-  };
-  const cplx A = cadd(rmul(R11, m1), rmul(R12, m2)), B = cadd(rmul(R12, m1), rmul(R22, m2));
-  const cplx Ae = cadd(A, k1), Be = cadd(B, k2);
   double *ae = ws + it.a_off + w.aeff + ((long long)e * 2 * g.nqp + qi) * R3 + b;
-  ae[0] = Ae.re;
-  ae[(long long)g.nqp * R3] = Be.re;
-  if (CD) { ae[cp] = Ae.im; ae[(long long)g.nqp * R3 + cp] = Be.im; }
+  ae[0] = out[0][0];
+  ae[(long long)g.nqp * R3] = out[0][1];
+  if (CD) { ae[cp] = out[1][0]; ae[(long long)g.nqp * R3 + cp] = out[1][1]; }
   double *y = ws + it.y_off;
-  auto ystore = [&](int slot, cplx v) {
+  auto ystore = [&](int slot, double re, double im) {
     const long long o = ((long long)(q - 1) * 5 + slot) * nc + b;
-    if (CD) st2(y + 2 * o, v); else y[o] = v.re;
+    if (CD) st2(y + 2 * o, cmk(re, im)); else y[o] = re;
   };
-  constexpr int KI[4][4] = {{1, 2, 4, 5}, {0, 1, 3, 4}, {4, 3, 1, 0}, {5, 4, 2, 1}};   // gamma row x dense row
 #pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    cplx v = axpy(T[MT_W1 + r], M[0], cmk(0.0, 0.0));
-    v = axpy(T[MT_W2 + r], M[1], v);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) v = axpy(T[MT_K + KI[r][j]], gd[j], v);
-    v = caxpy(T[MT_P1G + r], A, v);
-    v = caxpy(T[MT_P2G + r], B, v);
-    ystore(r, v);
-  }
+  for (int r = 0; r < 4; ++r) ystore(r, out[0][2 + r], CD ? out[1][2 + r] : 0.0);
   if (rec) {
-    cplx v = axpy(T[MT_REC + 2], M[2], cmk(0.0, 0.0));
-    v = caxpy(T[MT_REC], Ae, v);
-    v = caxpy(T[MT_REC + 1], Be, v);
-    ystore(4, v);
+    const double p1 = T[MT_REC], p2 = T[MT_REC + 1], f = T[MT_REC + 2];
+    const double re = fma(p1, out[0][0], fma(p2, out[0][1], f * m3[0]));
+    double im = 0.0;
+    if (CD) im = fma(p1, out[1][0], fma(p2, out[1][1], CIN ? f * m3[P - 1] : 0.0));
+    ystore(4, re, im);
   }
 }
 
@@ -765,9 +866,12 @@ __global__ void __launch_bounds__(128) k_sep_modes(Batch bt, const SubDesc *subs
   const int cb = (it.ncols + 31) >> 5;
   const int b = (local % cb) * 32 + threadIdx.x, q0 = (local / cb) * SEP_MODES_PER_BLOCK + threadIdx.y + 1;
   if (b >= it.ncols) return;
+  const SepGeo g = sep_geo(d);
+  const SepWs w = sep_ws(d, it.ncols);
+  const int row1 = CIN ? b : sep_side_row(d, it.col0, b);
   for (int q = q0; q < q0 + SEP_MODES_PER_BLOCK - (int)threadIdx.y && q <= d.Nq; q += 4) {
-    if (d.cplx || CIN) sep_modes_body<true, CIN>(it, d, sep, ws, b, q);
-    else sep_modes_body<false, CIN>(it, d, sep, ws, b, q);
+    if (d.cplx || CIN) sep_modes_body<true, CIN>(it, d, g, w, sep, ws, b, row1, q);
+    else sep_modes_body<false, CIN>(it, d, g, w, sep, ws, b, row1, q);
   }
 }
 
@@ -778,7 +882,7 @@ __device__ __forceinline__ void sep_out_body(const Item &it, const SubDesc &d, c
                                              const double2 *xi_user, double2 *out, int kind, int b, int i) {
   const SepGeo g = sep_geo(d);
   const SepWs w = sep_ws(d, it.ncols);
-  const int cp = sep_pad128(it.ncols), R1 = sep_rows1(d, it.ncols, it.col0, CIN), R3 = sep_rows3(d, it.ncols, CIN);
+  const int cp = sep_pad128(it.ncols), R1 = sep_rows(d, J_MID, it.ncols, it.col0, CIN), R3 = (CD ? 2 : 1) * cp;
   const int row1 = CIN ? b : sep_side_row(d, it.col0, b);
   const double sc = 2.0 / d.Nx;
   cplx v[4];
@@ -805,14 +909,70 @@ __device__ __forceinline__ void sep_out_body(const Item &it, const SubDesc &d, c
   }
 }
 
+// The full gamma rows and the receiver row: u(m) = (2/Nx) (U_0(m) + U_1(m)), u(Nx - m) = (2/Nx) (U_0(m) -
+// U_1(m)) from the two parities' sums over the folded columns. A block takes one row, 32 folded columns
+// m and 32 basis columns, turned through shared memory so that the loads run along the columns and
+// the stores along m.
+template <bool CD, bool CIN>
+__device__ __forceinline__ void sep_rows_out_body(const Item &it, const SubDesc &d, const double *tab, const double *ws,
+                                                  const double2 *xi_user, double2 *out, double2 *out_rec, int kind, int b0,
+                                                  int slot, int mt, double2 (*sh)[32][33]) {
+  const SepGeo g = sep_geo(d);
+  const int cp = sep_pad128(it.ncols), parts = CD ? 2 : 1, R = sep_rows(d, J_INV, it.ncols, it.col0, CIN);
+  const double *ui = ws + it.a_off + sep_ws(d, it.ncols).ui, sc = 2.0 / d.Nx;
+  const int b = b0 + threadIdx.x, row = slot * parts * cp + b;
+  for (int k = threadIdx.y; k < 32; k += 8) {
+    const int m = mt * 32 + k;
+    cplx u0 = cmk(0.0, 0.0), u1 = u0;
+    if (m < g.Ng && b < it.ncols) {
+      const double *p0 = ui + (long long)m * R + row, *p1 = p0 + (long long)g.Ng * R;
+      u0 = cmk(p0[0], CD ? p0[cp] : 0.0);
+      u1 = cmk(p1[0], CD ? p1[cp] : 0.0);
+    }
+    const cplx s = cadd(u0, u1), t = csub(u0, u1);
+    sh[0][k][threadIdx.x] = make_double2(sc * s.re, sc * s.im);
+    sh[1][k][threadIdx.x] = make_double2(sc * t.re, sc * t.im);
+  }
+  __syncthreads();
+  const int W = d.Px + 2, m1 = g.mg + mt * 32 + (int)threadIdx.x;
+  if (2 * m1 > d.Nx) return;
+  const int gbase = slot <= 1 ? slot * W : 2 * W + 4 * (d.Py - 2) + (slot - 2) * W;
+  for (int k = threadIdx.y; k < 32 && b0 + k < it.ncols; k += 8)
+#pragma unroll
+    for (int side = 0; side < 2; ++side) {
+      const int m = side == 0 ? m1 : d.Nx - m1;
+      if (side == 1 && m == m1) continue;
+      const double2 v = sh[side][threadIdx.x][k];
+      if (slot == 4) {
+        if (out_rec && m >= d.mlo + 1 && m <= d.mhi - 1)
+          out_rec[d.rec_off + (long long)(it.col0 + b0 + k) * (d.Px - 2) + (m - d.mlo - 1)] = make_double2(-v.x, -v.y);
+        continue;
+      }
+      if (m < d.mlo - 1 || m > d.mhi + 1) continue;
+      const int gi = gbase + m - (d.mlo - 1);
+      cplx r = cmk(-v.x, CD ? -v.y : 0.0);
+      if (kind == MDP_OUT_P) r = cadd(r, density<CIN>(d, it, ws, tab, xi_user, b0 + k, gi));
+      out[it.io_off + (long long)(b0 + k) * d.G + gi] = make_double2(r.re, r.im);
+    }
+}
+
 template <bool CIN>
 __global__ void __launch_bounds__(256) k_sep_out(Batch bt, const SubDesc *subs, const double *tab, const double *ws,
-                                                 const double2 *xi_user, double2 *out, int kind) {
+                                                 const double2 *xi_user, double2 *out, double2 *out_rec, int kind) {
+  __shared__ double2 sh[2][32][33];
   Item it; int local;
   locate(bt, blockIdx.x, it, local);
   MDP_CHECK_ITEM(bt, subs, it, local, F_SOUT);
   const SubDesc &d = subs[it.sub];
-  const int cb = (it.ncols + 31) >> 5;
+  const int cb = (it.ncols + 31) >> 5, nmid = cb * ((d.Py - 2 + 7) / 8);
+  if (local >= nmid) {
+    local -= nmid;
+    const int t = local / cb, ntg = sep_geo(d).ntg;
+    const int b0 = (local % cb) * 32;
+    if (d.cplx || CIN) sep_rows_out_body<true, CIN>(it, d, tab, ws, xi_user, out, out_rec, kind, b0, t / ntg, t % ntg, sh);
+    else sep_rows_out_body<false, CIN>(it, d, tab, ws, xi_user, out, out_rec, kind, b0, t / ntg, t % ntg, sh);
+    return;
+  }
   const int b = (local % cb) * 32 + threadIdx.x, i = (local / cb) * 8 + threadIdx.y;
   if (b >= it.ncols || i >= d.Py - 2) return;
   if (d.cplx || CIN) sep_out_body<true, CIN>(it, d, tab, ws, xi_user, out, kind, b, i);
@@ -860,38 +1020,50 @@ cudaError_t launch_sep_tables(const mdp_plan *p, const SubDesc *ds, const double
   return cudaGetLastError();
 }
 
+cudaError_t launch_sep_sines(const mdp_plan *p, const SubDesc *ds, const double *tab, unsigned char *sep, cudaStream_t st) {
+  int k[2] = {0, 0}, t[2] = {0, 0};
+  for (size_t i = 0; i < p->subs.size(); ++i) {
+    const SubDesc &d = p->subs[i].d;
+    if (!d.tc_cols || d.leader != (int)i) continue;
+    const SepGeo g = sep_geo(d);
+    for (int inv = 0; inv < 2; ++inv) {
+      k[inv] = std::max(k[inv], ((inv ? g.nqh / 16 : g.nkf) + 3) / 4);
+      t[inv] = std::max(t[inv], 2 * (inv ? g.ntg : g.nqh / 32));
+    }
+  }
+  const int ns = (int)p->subs.size();
+  if (t[0] == 0) return cudaSuccess;
+  for (int s0 = 0; s0 < ns; s0 += 65535)
+    for (int inv = 0; inv < 2; ++inv)
+      k_sep_sines<<<dim3(k[inv], t[inv], (unsigned)std::min(65535, ns - s0)), 256, 0, st>>>(ds, s0, tab, sep, inv);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_sep_project(mdp_plan *p, const Batch *fb, int out_kind, const double2 *xi_user, double2 *out,
-                               int part, cudaStream_t st) {
+                               double2 *out_rec, cudaStream_t st) {
   const bool user = xi_user != nullptr;
+  if (fb[F_SMODE].total_blocks == 0) return cudaSuccess;
   const SubDesc *ds = p->d_subs;
-  const double *tab = p->d_tables;
   double *ws = p->d_ws;
   const int f1c = user ? F_C1U : F_C1B, f1 = user ? F_G1U : F_G1B, f3c = user ? F_C3U : F_C3B, f3 = user ? F_G3U : F_TCOLS;
-  auto grid = [](int n) { return dim3((unsigned)n); };
-  auto gemm_grid = [&](int n) { return dim3((unsigned)std::max(1, std::min(n, p->n_sm))); };
-#define SEP_LAUNCH(fam, as, ...)                  \
-  do {                                            \
-    if (fb[fam].total_blocks > 0) {               \
-      prof_begin(p, as, st);                      \
-      __VA_ARGS__;                                \
-      prof_end(p, as, st);                        \
-    }                                             \
+  auto grid = [&](int f) { return dim3((unsigned)fb[f].total_blocks); };
+  auto gemm_grid = [&](int f) { return dim3((unsigned)std::min(fb[f].total_blocks, p->n_sm)); };
+#define SEP_LAUNCH(as, ...)   \
+  do {                        \
+    prof_begin(p, as, st);    \
+    __VA_ARGS__;              \
+    prof_end(p, as, st);      \
   } while (0)
-  if (part == 0) {
-    if (user) SEP_LAUNCH(f1c, F_C1B, k_sep_cut<true, 1><<<grid(fb[f1c].total_blocks), 256, 0, st>>>(fb[f1c], ds, ws, f1c));
-    else SEP_LAUNCH(f1c, F_C1B, k_sep_cut<false, 1><<<grid(fb[f1c].total_blocks), 256, 0, st>>>(fb[f1c], ds, ws, f1c));
-    SEP_LAUNCH(f1, F_G1B, k_sep_gemm<1><<<gemm_grid(fb[f1].total_blocks), SG_THREADS, SG_SMEM, st>>>(
-                              fb[f1], ds, p->d_sep, ws, user, f1, p->d_status));
-    if (user) SEP_LAUNCH(F_SMODE, F_SMODE, k_sep_modes<true><<<grid(fb[F_SMODE].total_blocks), dim3(32, 4), 0, st>>>(fb[F_SMODE], ds, p->d_sep, ws));
-    else SEP_LAUNCH(F_SMODE, F_SMODE, k_sep_modes<false><<<grid(fb[F_SMODE].total_blocks), dim3(32, 4), 0, st>>>(fb[F_SMODE], ds, p->d_sep, ws));
-    return cudaGetLastError();
-  }
-  if (user) SEP_LAUNCH(f3c, F_C3B, k_sep_cut<true, 3><<<grid(fb[f3c].total_blocks), 256, 0, st>>>(fb[f3c], ds, ws, f3c));
-  else SEP_LAUNCH(f3c, F_C3B, k_sep_cut<false, 3><<<grid(fb[f3c].total_blocks), 256, 0, st>>>(fb[f3c], ds, ws, f3c));
-  SEP_LAUNCH(f3, F_TCOLS, k_sep_gemm<3><<<gemm_grid(fb[f3].total_blocks), SG_THREADS, SG_SMEM, st>>>(
-                              fb[f3], ds, p->d_sep, ws, user, f3, p->d_status));
-  if (user) SEP_LAUNCH(F_SOUT, F_SOUT, k_sep_out<true><<<grid(fb[F_SOUT].total_blocks), dim3(32, 8), 0, st>>>(fb[F_SOUT], ds, tab, ws, xi_user, out, out_kind));
-  else SEP_LAUNCH(F_SOUT, F_SOUT, k_sep_out<false><<<grid(fb[F_SOUT].total_blocks), dim3(32, 8), 0, st>>>(fb[F_SOUT], ds, tab, ws, xi_user, out, out_kind));
+  if (user) SEP_LAUNCH(F_C1B, k_sep_cut<true, 1><<<grid(f1c), 256, 0, st>>>(fb[f1c], ds, ws, f1c));
+  else SEP_LAUNCH(F_C1B, k_sep_cut<false, 1><<<grid(f1c), 256, 0, st>>>(fb[f1c], ds, ws, f1c));
+  SEP_LAUNCH(F_G1B, k_sep_gemm<1><<<gemm_grid(f1), SG_THREADS, SG_SMEM, st>>>(fb[f1], ds, p->d_sep, ws, user, f1, p->d_status));
+  if (user) SEP_LAUNCH(F_SMODE, k_sep_modes<true><<<grid(F_SMODE), dim3(32, 4), 0, st>>>(fb[F_SMODE], ds, p->d_sep, ws));
+  else SEP_LAUNCH(F_SMODE, k_sep_modes<false><<<grid(F_SMODE), dim3(32, 4), 0, st>>>(fb[F_SMODE], ds, p->d_sep, ws));
+  if (user) SEP_LAUNCH(F_C3B, k_sep_cut<true, 3><<<grid(f3c), 256, 0, st>>>(fb[f3c], ds, ws, f3c));
+  else SEP_LAUNCH(F_C3B, k_sep_cut<false, 3><<<grid(f3c), 256, 0, st>>>(fb[f3c], ds, ws, f3c));
+  SEP_LAUNCH(F_TCOLS, k_sep_gemm<3><<<gemm_grid(f3), SG_THREADS, SG_SMEM, st>>>(fb[f3], ds, p->d_sep, ws, user, f3, p->d_status));
+  if (user) SEP_LAUNCH(F_SOUT, k_sep_out<true><<<grid(F_SOUT), dim3(32, 8), 0, st>>>(fb[F_SOUT], ds, p->d_tables, ws, xi_user, out, out_rec, out_kind));
+  else SEP_LAUNCH(F_SOUT, k_sep_out<false><<<grid(F_SOUT), dim3(32, 8), 0, st>>>(fb[F_SOUT], ds, p->d_tables, ws, xi_user, out, out_rec, out_kind));
 #undef SEP_LAUNCH
   return cudaGetLastError();
 }

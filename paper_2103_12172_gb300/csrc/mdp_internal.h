@@ -67,6 +67,7 @@ struct SubDesc {
   long long sep_kd;     // doubles [class][output][source][Py]: K by row distance
   long long sep_kde;    // ints [class][output]: exponent of the largest |K|
   long long sep_tb, sep_mb, sep_b3;   // digit blocks of K (Toeplitz), of the moments, of the synthesis
+  long long sep_bf, sep_bi;           // of the dense rows' transform and of the gamma rows' (sines only)
   long long out_off;    // complex elements: start of the subdomain's output block
   long long rec_off;    // complex elements: start of the receiver block [n_cols][Px - 2]
   int *dstatus;         // the plan's device status word (bounds-checked build: first error; else unused)
@@ -111,32 +112,52 @@ struct Batch {
 constexpr int FSW = 24;  // doubles per forward-sweep table row
 
 // ---- separable projection (kernels_sep.cu)
-constexpr int SEP_MTW = 56;               // doubles per mode of the mode table
+constexpr int SEP_MTW = 72;               // doubles per mode of the mode table
 constexpr int SEP_ABLK = 7 * 128 * 16 * 2;  // bytes of A: 7 digits x 128 rows x 16 values of K, fp16
 constexpr int SEP_BBLK = 7 * 32 * 16 * 2;   // bytes of B: 7 digits x 32 outputs x 16 values of K
-constexpr int SEP_MODES_PER_BLOCK = 32;   // k_sep_modes
+constexpr int SEP_MODES_PER_BLOCK = 16;   // k_sep_modes
+constexpr int SEP_MASK = 8;               // words of a K mask: at most 256 groups of 16
+
+// The contractions (jobs) of the projection: stage 1 runs MID (ring residuals of the middle rows
+// against K and the moments) and FWD (sine transform of the 4 dense ring rows), stage 3 SYN (the
+// middle rows' gamma columns from the modes) and INV (inverse sine transform of the 4 gamma rows and
+// the receiver row).
+enum SepJob { J_MID = 0, J_FWD, J_SYN, J_INV };
 
 // Sizes of a subdomain's contractions.
 struct SepGeo {
-  int ncls, nS;        // classes of modes (odd, even) on x-centred subdomains, else 1; output (and source) columns
+  int ncls, nS;        // MID, SYN: classes of modes (odd, even) on x-centred subdomains, else 1; output (and
+                       // source) columns. FWD, INV: always the two parities
   int nqp;             // modes per class, padded to 32
+  int nqh;             // modes per parity, padded to 32 (x-centred: nqp)
   int Pi, Pj;          // output rows nlo+1 .. nhi-1, source rows nlo+2 .. nhi-2
   int nti, nkj;        // groups of 32 outputs, of 16 sources per column
   int nb;              // moments per mode: 2, or 3 with a receiver row
-  int nk1, nk3;        // K in units of 16: stage 1 (source column, row), stage 3 (b, mode)
-  int nt1, nt3;        // tiles of 32 outputs
+  int mf, Kf, nkf;     // FWD: folded columns m = mf .. Nx/2 of the dense ring rows (m with Nx - m), groups of 16
+  int mg, Ng, ntg;     // INV: folded columns m = mg .. Nx/2 of the gamma rows, groups of 32
+  int slots;           // INV: rows transformed back: 4 gamma rows (+ the receiver row)
+  int nk1, nk3;        // K of MID (source column, row) and SYN (b, mode) in units of 16
+  int nt1, nt3;        // MID, SYN: tiles of 32 outputs
   int ND;              // distinct Toeplitz blocks per (output, source) column
 };
 inline __host__ __device__ SepGeo sep_geo(const SubDesc &d) {
   SepGeo g;
   g.ncls = d.xsym ? 2 : 1;
   g.nS = d.xsym ? 2 : 4;
-  g.nqp = ((d.xsym ? (d.Nq + 1) / 2 : d.Nq) + 31) / 32 * 32;
+  g.nqh = ((d.Nq + 1) / 2 + 31) / 32 * 32;
+  g.nqp = d.xsym ? g.nqh : (d.Nq + 31) / 32 * 32;
   g.Pi = d.Py - 2;
   g.Pj = d.Py - 4;
   g.nti = (g.Pi + 31) / 32;
   g.nkj = (g.Pj + 15) / 16;
   g.nb = d.nrec >= 0 ? 3 : 2;
+  g.mf = d.mlo < d.Nx - d.mhi ? d.mlo : d.Nx - d.mhi;
+  g.Kf = d.Nx / 2 - g.mf + 1;
+  g.nkf = (g.Kf + 15) / 16;
+  g.mg = g.mf - 1;
+  g.Ng = g.Kf + 1;
+  g.ntg = (g.Ng + 31) / 32;
+  g.slots = d.nrec >= 0 ? 5 : 4;
   g.nk1 = g.nS * g.nkj;
   g.nk3 = 2 * g.nqp / 16;
   g.nt3 = g.nS * g.nti;
@@ -144,8 +165,9 @@ inline __host__ __device__ SepGeo sep_geo(const SubDesc &d) {
   g.ND = 2 * g.nti + g.nkj;
   return g;
 }
-// mode number of entry qi of class e (past Nq: padding)
+// mode number of entry qi of class e (past Nq: padding), of entry qi of parity e (0: odd modes)
 inline __host__ __device__ int sep_mode(const SubDesc &d, int e, int qi) { return d.xsym ? 2 * qi + 1 + e : qi + 1; }
+inline __host__ __device__ int sep_parity_mode(int e, int qi) { return 2 * qi + 1 + e; }
 // grid column of output s (gamma) and of source c (ring); x-centred: the left ones, the right ones mirrored
 inline __host__ __device__ int sep_out_col(const SubDesc &d, int s) {
   return s == 0 ? d.mlo - 1 : s == 1 ? d.mlo : s == 2 ? d.mhi : d.mhi + 1;
@@ -155,7 +177,7 @@ inline __host__ __device__ int sep_src_col(const SubDesc &d, int c) {
 }
 inline __host__ __device__ int sep_pad128(int n) { return (n + 127) / 128 * 128; }
 // Only the basis columns of sides 3 and 4 have residuals on the middle ring rows (the gamma nodes
-// next to them belong to these sides), so stage 1 has only their rows: sep_side_before counts such
+// next to them belong to these sides), so MID has only their rows: sep_side_before counts such
 // columns below column c, sep_side_col gives the row-th one from column c0 on, sep_side_row the
 // row of an item's column b (-1: a column of side 1 or 2).
 inline __host__ __device__ int sep_side_before(const SubDesc &d, int c) {
@@ -172,40 +194,69 @@ inline __host__ __device__ int sep_side_col(const SubDesc &d, int c0, int row) {
 inline __host__ __device__ int sep_side_row(const SubDesc &d, int c0, int b) {
   return (c0 + b) % (4 * d.n_modes) < 2 * d.n_modes ? -1 : sep_side_before(d, c0 + b) - sep_side_before(d, c0);
 }
-// Rows of A, padded to the MMA's 128: stage 1 (columns, or real and imaginary parts of user
-// densities), stage 3 (columns, or real and imaginary parts); the parts are sep_pad128(ncols) apart.
-inline __host__ __device__ int sep_rows1(const SubDesc &d, int ncols, int col0, bool user) {
-  return user ? 2 * sep_pad128(ncols) : sep_pad128(sep_side_cols(d, col0, ncols));
+// Rows of A, a multiple of the MMA's 128: the item's columns padded to 128, times real and imaginary
+// parts where the data (MID, FWD: user densities) or the results (SYN, INV) are complex, times the
+// 4 dense rows (FWD) or the rows transformed back (INV), in the order (row, part, column).
+inline __host__ __device__ int sep_rows(const SubDesc &d, int job, int ncols, int col0, bool user) {
+  const int cp = sep_pad128(ncols);
+  switch (job) {
+    case J_MID: return user ? 2 * cp : sep_pad128(sep_side_cols(d, col0, ncols));
+    case J_FWD: return (user ? 8 : 4) * cp;
+    case J_SYN: return (user || d.cplx ? 2 : 1) * cp;
+    default: return (d.nrec >= 0 ? 5 : 4) * (user || d.cplx ? 2 : 1) * cp;
+  }
 }
-inline __host__ __device__ int sep_rows3(const SubDesc &d, int ncols, bool user) {
-  return (user || d.cplx ? 2 : 1) * sep_pad128(ncols);
+inline __host__ __device__ int sep_classes(const SepGeo &g, int job) { return job == J_MID || job == J_SYN ? g.ncls : 2; }
+inline __host__ __device__ int sep_nk(const SepGeo &g, int job) {
+  return job == J_MID ? g.nk1 : job == J_FWD ? g.nkf : job == J_SYN ? g.nk3 : g.nqh / 16;
 }
-// Workspace of an item's separable solve, in doubles from its a_off (sized for complex data).
+inline __host__ __device__ int sep_nt(const SepGeo &g, int job) {
+  return job == J_MID ? g.nt1 : job == J_FWD ? g.nqh / 32 : job == J_SYN ? g.nt3 : g.ntg;
+}
+// blocks of 8 rows (operand cutting) and tiles of 128 rows x 32 outputs of a job
+inline __host__ __device__ int sep_cut_blocks(const SubDesc &d, const SepGeo &g, int job, int ncols, int col0, bool user) {
+  return sep_classes(g, job) * (sep_rows(d, job, ncols, col0, user) / 8);
+}
+inline __host__ __device__ int sep_tiles(const SubDesc &d, const SepGeo &g, int job, int ncols, int col0, bool user) {
+  return sep_classes(g, job) * (sep_rows(d, job, ncols, col0, user) / 128) * sep_nt(g, job);
+}
+// Workspace of an item's separable solve, in doubles from its a_off (sized for complex data and a
+// receiver row). Per job: digit blocks of A, exponents of A's rows (ints) [class][rows], masks of
+// the nonzero groups of K (words) [class][rows / 128][SEP_MASK]; then the sums.
 struct SepWs {
-  long long u1, u3;    // sums at the gamma columns [class][output][Pi][rows] of stage 1 and stage 3
+  long long a[4], ex[4], mask;   // mask: of all jobs, job after job
+  long long u1, u3;    // sums at the gamma columns [class][output][Pi][rows] of MID and SYN
   long long mom;       // moments [class][3][nqp][rows]
   long long aeff;      // A_b [class][2][nqp][rows]
-  long long a1, a3;    // digit blocks of A
-  long long ex1, ex3;  // exponents of A's rows (ints) [class][rows]
+  long long ui;        // sums on the gamma rows and the receiver row [parity][Ng][rows]
   long long total;
 };
 inline __host__ __device__ SepWs sep_ws(const SubDesc &d, int ncols) {
   const SepGeo g = sep_geo(d);
-  const long long R = 2LL * sep_pad128(ncols), u = g.ncls * (long long)g.nS * g.Pi * R;
+  const long long cp = sep_pad128(ncols), R = 2 * cp, u = g.ncls * (long long)g.nS * g.Pi * R;
+  const long long rows[4] = {R, 4 * R, R, 5 * R};
   SepWs w;
   long long off = 0;
   auto take = [&](long long n) { const long long o = off; off += (n + 31) & ~31LL; return o; };
-  w.a1 = take(g.ncls * (R / 128) * g.nk1 * (SEP_ABLK / 8));
-  w.a3 = take(g.ncls * (R / 128) * g.nk3 * (SEP_ABLK / 8));
+  for (int j = 0; j < 4; ++j) {
+    w.a[j] = take(sep_classes(g, j) * (rows[j] / 128) * sep_nk(g, j) * (SEP_ABLK / 8));
+    w.ex[j] = take(sep_classes(g, j) * rows[j] / 2);
+  }
+  w.mask = take(2 * 11 * (R / 128) * SEP_MASK / 2);
   w.u1 = take(u);
   w.u3 = take(u);
   w.mom = take(g.ncls * 3LL * g.nqp * R);
   w.aeff = take(g.ncls * 2LL * g.nqp * R);
-  w.ex1 = take(g.ncls * R / 2);
-  w.ex3 = take(g.ncls * R / 2);
+  w.ui = take(2LL * g.Ng * 5 * R);
   w.total = off;
   return w;
 }
+// first mask word of a job, in words from SepWs::mask (jobs of at most R, 4 R, R, 5 R rows)
+inline __host__ __device__ int sep_mask_of(int job, int ncols) {
+  const int t = 2 * (2 * sep_pad128(ncols) / 128) * SEP_MASK;
+  return job == J_MID ? 0 : job == J_FWD ? t : job == J_SYN ? 5 * t : 6 * t;
+}
+inline __host__ __device__ int sep_mask_words(int ncols) { return 11 * 2 * (2 * sep_pad128(ncols) / 128) * SEP_MASK; }
 constexpr int TRI_WARPS = 1;  // warps (modes) per block of the per-mode sweep kernel k_tri
 constexpr int FFT_POINTS = 4096;        // longest transform (2 Nx) of the dense-row FFT kernels (64 KiB)
 constexpr int FFT_BLOCK_POINTS = 1024;  // complex values per block when 2 Nx is shorter: fpb = 1024 / (2 Nx)
@@ -343,11 +394,12 @@ inline void set_bounds(const mdp_plan *p, Batch &b, long long out_n, bool grad) 
 }
 
 // kernel families (each has its own block decomposition of an item); F_A* are the adjoint's. F_TRI is
-// the gradient pass's full sweep, F_PTRI the projection's (subdomains without the separable solve);
-// F_C* cut operands, F_G* contract (stage 1 and 3, B: basis columns, U: user densities; F_TCOLS is
-// stage 3 for basis columns), F_SMODE and F_SOUT are the separable solve's other kernels.
+// the gradient pass's full sweep, F_PTRI the projection's (subdomains without the separable solve),
+// F_FROWS and F_PROWS likewise for the dense rows' transform; F_C* cut operands, F_G* contract (stage 1
+// and 3, B: basis columns, U: user densities; F_TCOLS is stage 3 for basis columns), F_SMODE and F_SOUT
+// are the separable solve's other kernels.
 enum Fam { F_EXT = 0, F_RES, F_FROWS, F_TRI, F_IROWS, F_ICOLS, F_AFWD, F_ATRI, F_ARING, F_ARINGC, F_AGAM, F_IREC,
-           F_ACOLS, F_TCOLS, F_ATCOLS, F_PTRI, F_C1B, F_C1U, F_G1B, F_G1U, F_SMODE, F_C3B, F_C3U, F_G3U, F_SOUT, NFAM };
+           F_ACOLS, F_TCOLS, F_ATCOLS, F_PTRI, F_C1B, F_C1U, F_G1B, F_G1U, F_SMODE, F_C3B, F_C3U, F_G3U, F_SOUT, F_PROWS, NFAM };
 static_assert(NFAM <= 32, "per-family event lists of mdp_plan");
 
 // Blocks of kernel family f for an item of ncols columns: 32 columns (x) times BY tasks (y).
@@ -361,25 +413,28 @@ inline __host__ __device__ int blocks_for(int f, const SubDesc &d, int ncols, in
       if (d.rows_fft) return 4 * ((ncols + d.fpb - 1) / d.fpb);
       return cb * ((d.Nx / 2 + 7) / 8);
     case F_TRI: return cb * ((d.Nq + TRI_WARPS - 1) / TRI_WARPS);
+    case F_PROWS: return d.tc_cols ? 0 : blocks_for(F_FROWS, d, ncols, col0);
     case F_IROWS:
+      if (d.tc_cols) return 0;
       if (d.rows_fft) return 4 * ((ncols + d.fpb - 1) / d.fpb);
       return cb * (((d.xsym ? 4 * (d.Ph + 1) : 4 * (d.Px + 2)) + 7) / 8);
     case F_ICOLS: return d.tc_cols ? 0 : cb * ((d.Py - 2 + 7) / 8);
     case F_PTRI: return d.tc_cols ? 0 : cb * ((d.Nq + TRI_WARPS - 1) / TRI_WARPS);
-    case F_C1B: case F_C1U: case F_G1B: case F_G1U: {
+    case F_C1B: case F_C1U: case F_G1B: case F_G1U: case F_C3B: case F_C3U: case F_TCOLS: case F_G3U: {
       if (!d.tc_cols) return 0;
       const SepGeo g = sep_geo(d);
-      const int R = sep_rows1(d, ncols, col0, f == F_C1U || f == F_G1U);
-      return f == F_C1B || f == F_C1U ? g.ncls * (R / 8) : g.ncls * (R / 128) * g.nt1;
-    }
-    case F_C3B: case F_C3U: case F_TCOLS: case F_G3U: {
-      if (!d.tc_cols) return 0;
-      const SepGeo g = sep_geo(d);
-      const int R = sep_rows3(d, ncols, f == F_C3U || f == F_G3U);
-      return f == F_C3B || f == F_C3U ? g.ncls * (R / 8) : g.ncls * (R / 128) * g.nt3;
+      const bool user = f == F_C1U || f == F_G1U || f == F_C3U || f == F_G3U;
+      const int j = f == F_C1B || f == F_C1U || f == F_G1B || f == F_G1U ? J_MID : J_SYN;   // and the next job
+      if (f == F_C1B || f == F_C1U || f == F_C3B || f == F_C3U)
+        return sep_cut_blocks(d, g, j, ncols, col0, user) + sep_cut_blocks(d, g, j + 1, ncols, col0, user);
+      return sep_tiles(d, g, j, ncols, col0, user) + sep_tiles(d, g, j + 1, ncols, col0, user);
     }
     case F_SMODE: return d.tc_cols ? cb * ((d.Nq + SEP_MODES_PER_BLOCK - 1) / SEP_MODES_PER_BLOCK) : 0;
-    case F_SOUT: return d.tc_cols ? cb * ((d.Py - 2 + 7) / 8) : 0;
+    case F_SOUT: {   // middle rows, 8 per block, then 32 folded columns of each row transformed back
+      if (!d.tc_cols) return 0;
+      const SepGeo g = sep_geo(d);
+      return cb * ((d.Py - 2 + 7) / 8) + cb * g.slots * g.ntg;
+    }
     case F_AFWD:
       if (d.rows_fft) return 5 * ((ncols + d.fpb - 1) / d.fpb);
       return cb * ((d.Nx / 2 + 7) / 8);
@@ -390,7 +445,7 @@ inline __host__ __device__ int blocks_for(int f, const SubDesc &d, int ncols, in
     case F_ARINGC: return d.tc_cols ? 0 : cb * ((d.Py - 4 + 7) / 8);
     case F_ATCOLS: return d.tc_cols && d.Py > 4 ? ((ncols + 63) / 64) * (d.Py - 4) : 0;   // tiles: inner middle row x 64 columns
     case F_AGAM: return cb * ((d.G + 7) / 8);
-    case F_IREC: return d.nrec < 0 ? 0 : cb * (((d.xsym ? d.Ph - 1 : d.Px - 2) + 7) / 8);
+    case F_IREC: return d.nrec < 0 || d.tc_cols ? 0 : cb * (((d.xsym ? d.Ph - 1 : d.Px - 2) + 7) / 8);
     case F_ACOLS: return cb * ((d.Py - 2 + 7) / 8);
     default: return 0;
   }
@@ -451,10 +506,11 @@ cudaError_t set_sep_kernel_attributes();  // kernels_sep.cu
 // entries: from matrix entries computed here, else from the stored ones (sep_ab)
 cudaError_t launch_sep_tables(const mdp_plan *p, const SubDesc *ds, const double *tab, unsigned char *sep, bool entries,
                               cudaStream_t st);
-// the separable solve of the projection: part 0 up to the field on the 4 gamma rows, part 1 the
-// gamma columns of the middle rows
+// the sine tables among them, which no wavenumber enters
+cudaError_t launch_sep_sines(const mdp_plan *p, const SubDesc *ds, const double *tab, unsigned char *sep, cudaStream_t st);
+// the separable solve of the projection, from the ring residuals to the output columns
 cudaError_t launch_sep_project(mdp_plan *p, const Batch *fb, int out_kind, const double2 *xi_user, double2 *out,
-                               int part, cudaStream_t st);
+                               double2 *out_rec, cudaStream_t st);
 // the adjoint's sums at the 4 ring columns of the inner middle rows (dk: with the k-gradient partials)
 cudaError_t launch_adj_cols_tc(const Batch &b, const SubDesc *subs, const double *tab, double *ws, bool dk,
                                int *status, int n_sm, cudaStream_t st);

@@ -25,7 +25,7 @@ const char *fam_name(int f) {
                                     "k_adj_rows", "k_adj_tri", "k_adj_ring_rows", "k_adj_ring_cols", "k_adj_gamma",
                                     "k_inv_rec", "k_adj_cols", "k_inv_cols_tc", "k_adj_ring_cols_tc", "k_tri(projection)",
                                     "k_sep_cut1", "k_sep_cut1(user)", "k_sep_gemm1", "k_sep_gemm1(user)", "k_sep_modes",
-                                    "k_sep_cut3", "k_sep_cut3(user)", "k_inv_cols_tc(user)", "k_sep_out"};
+                                    "k_sep_cut3", "k_sep_cut3(user)", "k_inv_cols_tc(user)", "k_sep_out", "k_fwd_rows(projection)"};
   return (f >= 0 && f < NFAM) ? names[f] : "?";
 }
 
@@ -409,7 +409,7 @@ static bool layout_tables(mdp_plan *p) {
       d.fact_off = ld.fact_off; d.dT_off = ld.dT_off; d.sin_off = ld.sin_off; d.geo_off = ld.geo_off;
       d.seg_off = ld.seg_off; d.fs_off = ld.fs_off; d.piv_off = ld.piv_off; d.tcb_off = ld.tcb_off;
       d.sep_ab = ld.sep_ab; d.sep_mt = ld.sep_mt; d.sep_phi = ld.sep_phi; d.sep_kd = ld.sep_kd; d.sep_kde = ld.sep_kde;
-      d.sep_tb = ld.sep_tb; d.sep_mb = ld.sep_mb; d.sep_b3 = ld.sep_b3;
+      d.sep_tb = ld.sep_tb; d.sep_mb = ld.sep_mb; d.sep_b3 = ld.sep_b3; d.sep_bf = ld.sep_bf; d.sep_bi = ld.sep_bi;
       d.out_off = out;  out += (long long)d.G * d.n_cols;
       continue;
     }
@@ -425,6 +425,8 @@ static bool layout_tables(mdp_plan *p) {
       d.sep_tb = take(pairs * g.ND * SEP_BBLK);
       d.sep_mb = take((long long)g.ncls * (3 * g.nqp / 32) * g.nk1 * SEP_BBLK);   // room for receivers
       d.sep_b3 = take((long long)g.ncls * g.nt3 * g.nk3 * SEP_BBLK);
+      d.sep_bf = take(2LL * (g.nqh / 32) * g.nkf * SEP_BBLK);
+      d.sep_bi = take(2LL * g.ntg * (g.nqh / 16) * SEP_BBLK);
     }
     const int FW = d.cplx ? 8 : 4;
     d.fact_off = off; off += al((long long)d.Nq * d.Nt * FW);
