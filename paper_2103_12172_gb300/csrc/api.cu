@@ -293,6 +293,7 @@ mdp_status mdp_ap_plan_ex(const mdp_subdomain *subs, int n_subs, unsigned flags,
   p->tile_cols = (int)std::max(1LL, env_ll("MDP_TILE_COLS", 256));
   p->ws_budget = env_ll("MDP_WS_MB", 4096) << 20;
   if (opt && opt->tile_cols > 0) p->tile_cols = opt->tile_cols;
+  if ((opt && opt->tile_cols > 0) || env_ll("MDP_TILE_COLS", 0) > 0) p->sep_cols = p->tile_cols;
   if (opt && opt->workspace_bytes > 0) p->ws_budget = opt->workspace_bytes;
   if (opt && opt->fft_block_points > 0) p->fft_block_points = opt->fft_block_points;
   if (opt && opt->tri_stages > 0) p->tri_stages = opt->tri_stages;
@@ -536,10 +537,11 @@ mdp_status mdp_project_columns(mdp_plan *p, int sub, int col0, int ncols, const 
   CK(cudaSetDevice(p->device));
   cudaStream_t st = (cudaStream_t)cuda_stream;
   CK(begin_use(p, st));
-  for (int c = 0; c < ncols; c += p->tile_cols) {
+  const int cols = d.tc_cols ? p->sep_cols : p->tile_cols;
+  for (int c = 0; c < ncols; c += cols) {
     Item it;
     std::memset(&it, 0, sizeof it);
-    it.sub = sub; it.col0 = col0 + c; it.ncols = std::min(p->tile_cols, ncols - c);
+    it.sub = sub; it.col0 = col0 + c; it.ncols = std::min(cols, ncols - c);
     long long xo, ro, go, yo, ao, so, reo, tot;
     item_workspace(d, it.ncols, false, xo, ro, go, yo, ao, so, reo, tot);
     it.xi_off = xo; it.r_off = ro; it.gr_off = go; it.y_off = yo; it.a_off = ao; it.s_off = so; it.red_off = reo;

@@ -295,6 +295,13 @@ __device__ __forceinline__ void store_digits(unsigned char *dst, long long strid
   MDP_SEP_DIGIT(0) MDP_SEP_DIGIT(1) MDP_SEP_DIGIT(2) MDP_SEP_DIGIT(3) MDP_SEP_DIGIT(4) MDP_SEP_DIGIT(5) MDP_SEP_DIGIT(6)
 #undef MDP_SEP_DIGIT
 }
+// set bit kb of a tile's mask if the warp (32 outputs, one half of the 16 values of K) has a nonzero digit
+__device__ __forceinline__ void mark_group(unsigned *mask, int kb, const long long *V) {
+  long long any = 0;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) any |= V[j];
+  if (__any_sync(0xffffffffu, any != 0) && (threadIdx.x & 31) == 0) atomicOr(mask + (kb >> 5), 1u << (kb & 31));
+}
 // table value |x| <= 1 on the fixed scale 2^54
 __device__ __forceinline__ long long fix54(double x) { return __double2ll_rn(x * 0x1p54); }
 
@@ -369,6 +376,7 @@ __global__ void __launch_bounds__(256) k_sep_mb(const SubDesc *subs, int s0, con
       V[j] = fix54(v * sc);
     }
   }
+  mark_group(reinterpret_cast<unsigned *>(sep + d.sep_zm) + (e * (3 * g.nqp / 32) + to) * SEP_MASK, kb, V);
   unsigned char *B = sep + d.sep_mb + (((long long)e * (3 * g.nqp / 32) + to) * g.nk1 + kb) * SEP_BBLK;
   store_digits(B + (o >> 3) * 256 + half * 128 + (o & 7) * 16, 1024, V);
 }
@@ -394,6 +402,7 @@ __global__ void __launch_bounds__(256) k_sep_b3(const SubDesc *subs, int s0, con
     const int q = sep_mode(d, e, q0 + j);
     V[j] = (i < g.Pi && q <= d.Nq) ? fix54(P[q - 1] * S[(int)(((long long)q * m) % N2)]) : 0;
   }
+  mark_group(reinterpret_cast<unsigned *>(sep + d.sep_z3) + (e * g.nt3 + to) * SEP_MASK, kb, V);
   unsigned char *B = sep + d.sep_b3 + (((long long)e * g.nt3 + to) * g.nk3 + kb) * SEP_BBLK;
   store_digits(B + (o >> 3) * 256 + half * 128 + (o & 7) * 16, 1024, V);
 }
@@ -429,7 +438,8 @@ __global__ void __launch_bounds__(256) k_sep_sines(const SubDesc *subs, int s0, 
 // A block takes 8 rows of one class (one core-matrix row group): their largest exponents first, then
 // the digits; the values are read twice, the second time from L1/L2. Groups of 16 values of K whose
 // digits are all zero in 128 rows (the imaginary parts of evanescent modes, the ring away from a
-// column's side) are left out of the contraction by their bit in the tile's mask.
+// column's side) are left out of the contraction by their bit in the tile's mask; so are those of the
+// moment and synthesis tables, where phi has decayed below 2^-55 (nine tenths of them at 1025^2).
 template <bool CIN, int JOB>
 __device__ __forceinline__ void sep_cut_body(const Item &it, const SubDesc &d, double *ws, int local) {
   const SepGeo g = sep_geo(d);
@@ -444,10 +454,9 @@ __device__ __forceinline__ void sep_cut_body(const Item &it, const SubDesc &d, d
   int col = row % cp, part = (row / cp) % parts;
   const int rr = row / (cp * parts);
   bool live = col < it.ncols;
-  if (JOB == J_MID && !CIN) {
-    live = row < sep_side_cols(d, it.col0, it.ncols);
-    col = live ? sep_side_col(d, it.col0, row) - it.col0 : 0;
-    part = 0;
+  if (!CIN) {   // basis columns: the rows are ordered by side
+    if (JOB == J_MID) { col = row + sep_first34(d, it.col0, it.ncols); part = 0; live = col < it.ncols; }
+    col = live ? sep_col_of(d, it.col0, it.ncols, col) : 0;
   }
   const double *src = JOB == J_SYN ? ws + it.a_off + w.aeff + (long long)e * 2 * g.nqp * R + row
                       : JOB == J_INV ? ws + it.y_off : ws + it.r_off;
@@ -557,11 +566,17 @@ __device__ __forceinline__ void bulk_load(unsigned dst, const void *src, unsigne
 
 struct SepTile {
   int job, e, mt, nt, R, nk;
-  const unsigned *mask;   // groups of K with nonzero digits in the tile's rows
+  const unsigned *ma, *mb;   // groups of K with nonzero digits in the tile's rows, in its outputs (or null)
+  __device__ __forceinline__ unsigned mask(int wd) const { return mb ? ma[wd] & mb[wd] : ma[wd]; }
+  __device__ __forceinline__ int groups() const {
+    int n = 0;
+    for (int wd = 0; wd < SEP_MASK; ++wd) n += __popc(mask(wd));
+    return n;
+  }
 };
 template <int STAGE>
 __device__ __forceinline__ SepTile sep_tile(const SubDesc &d, const SepGeo &g, const SepWs &w, const Item &it, int local,
-                                            bool user, const double *ws) {
+                                            bool user, const double *ws, const unsigned char *sep) {
   SepTile t;
   t.job = STAGE == 1 ? J_MID : J_SYN;
   const int n0 = sep_tiles(d, g, t.job, it.ncols, it.col0, user);
@@ -572,8 +587,12 @@ __device__ __forceinline__ SepTile sep_tile(const SubDesc &d, const SepGeo &g, c
   t.e = local / per;
   t.mt = (local % per) / nt;
   t.nt = local % nt;
-  t.mask = reinterpret_cast<const unsigned *>(ws + it.a_off + w.mask) + sep_mask_of(t.job, it.ncols) +
-           (t.e * (t.R / 128) + t.mt) * SEP_MASK;
+  t.ma = reinterpret_cast<const unsigned *>(ws + it.a_off + w.mask) + sep_mask_of(t.job, it.ncols) +
+         (t.e * (t.R / 128) + t.mt) * SEP_MASK;
+  t.mb = nullptr;
+  if (t.job == J_SYN) t.mb = reinterpret_cast<const unsigned *>(sep + d.sep_z3) + (t.e * g.nt3 + t.nt) * SEP_MASK;
+  if (t.job == J_MID && t.nt >= g.nt3)
+    t.mb = reinterpret_cast<const unsigned *>(sep + d.sep_zm) + (t.e * (3 * g.nqp / 32) + t.nt - g.nt3) * SEP_MASK;
   return t;
 }
 
@@ -620,7 +639,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1)
         const SubDesc &d = subs[it.sub];
         const SepGeo g = sep_geo(d);
         const SepWs w = sep_ws(d, it.ncols);
-        const SepTile t = sep_tile<STAGE>(d, g, w, it, local, user, ws);
+        const SepTile t = sep_tile<STAGE>(d, g, w, it, local, user, ws, sep);
         const unsigned char *A = reinterpret_cast<const unsigned char *>(ws + it.a_off + w.a[t.job]) +
                                  (long long)(t.e * (t.R / 128) + t.mt) * t.nk * SEP_ABLK;
         const unsigned char *B;
@@ -633,7 +652,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1)
         else B = sep + d.sep_mb + ((long long)t.e * (3 * g.nqp / 32) + t.nt - g.nt3) * t.nk * SEP_BBLK;
         bool ok = true;
         for (int wd = 0; wd < SEP_MASK && ok; ++wd)
-          for (unsigned bits = t.mask[wd]; bits; bits &= bits - 1, ++gs) {
+          for (unsigned bits = t.mask(wd); bits; bits &= bits - 1, ++gs) {
             const int kb = 32 * wd + __ffs(bits) - 1;
             const unsigned st = gs % SG_STAGES;
             if (gs >= SG_STAGES && !mbar_wait(smem_u32(&empty_bar[st]), (gs / SG_STAGES - 1) & 1u, &abort_sh)) { ok = false; break; }
@@ -663,9 +682,8 @@ __global__ void __launch_bounds__(SG_THREADS, 1)
         if (MDP_CHECKED && !item_in_bounds(bt, subs, it, local, fam, false)) continue;
         const SubDesc &d = subs[it.sub];
         const SepGeo g = sep_geo(d);
-        const SepTile t = sep_tile<STAGE>(d, g, sep_ws(d, it.ncols), it, local, user, ws);
-        int n = 0;   // steps: groups of K left by the mask
-        for (int wd = 0; wd < SEP_MASK; ++wd) n += __popc(t.mask[wd]);
+        const SepTile t = sep_tile<STAGE>(d, g, sep_ws(d, it.ncols), it, local, user, ws, sep);
+        const int n = t.groups();   // steps
         bool ok = true;
         for (int s = 0; s < n && ok; ++cc) {
           const unsigned buf = cc & 1u, D = tmem + 256u * buf;
@@ -705,9 +723,8 @@ __global__ void __launch_bounds__(SG_THREADS, 1)
       const SubDesc &d = subs[it.sub];
       const SepGeo g = sep_geo(d);
       const SepWs w = sep_ws(d, it.ncols);
-      const SepTile t = sep_tile<STAGE>(d, g, w, it, local, user, ws);
-      int n = 0;
-      for (int wd = 0; wd < SEP_MASK; ++wd) n += __popc(t.mask[wd]);
+      const SepTile t = sep_tile<STAGE>(d, g, w, it, local, user, ws, sep);
+      const int n = t.groups();
       // weights 0..3 and 4..7 of 16 outputs, as sums of I_w 2^(8 (3 - w)), I_w 2^(8 (7 - w))
       long long hi[16], lo[16];
 #pragma unroll
@@ -756,8 +773,10 @@ __global__ void __launch_bounds__(SG_THREADS, 1)
         cnt = g.Ng - o0;
         dst = ws + it.a_off + w.ui + ((long long)t.e * g.Ng + o0) * t.R + row;
       } else {                   // the dense rows' transforms: modes q = 2 (o0 + o) + 1 + e
-        const int cp = sep_pad128(it.ncols), parts = user ? 2 : 1, col = row % cp;
+        const int cp = sep_pad128(it.ncols), parts = user ? 2 : 1;
+        int col = row % cp;
         cnt = col < it.ncols ? (d.Nq - (1 + t.e) - 2 * o0) / 2 + 1 : 0;
+        if (!user && cnt > 0) col = sep_col_of(d, it.col0, it.ncols, col);
         if (2 * o0 + (1 + t.e) > d.Nq) cnt = 0;
         step = 2LL * it.ncols * parts;
         dst = ws + it.gr_off + (((long long)(row / (cp * parts)) * d.Nq + 2 * o0 + t.e) * it.ncols + col) * parts + (row / cp) % parts;
@@ -789,7 +808,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1)
 // results (Sommerfeld AP or complex data). FP64-bound.
 template <bool CD, bool CIN>
 __device__ __forceinline__ void sep_modes_body(const Item &it, const SubDesc &d, const SepGeo &g, const SepWs &w,
-                                               const unsigned char *sep, double *ws, int b, int row1, int q) {
+                                               const unsigned char *sep, double *ws, int b, int row, int row1, int q) {
   const double *T = reinterpret_cast<const double *>(sep + d.sep_mt) + (long long)(q - 1) * SEP_MTW;
   const int e = d.xsym ? ((q & 1) ? 0 : 1) : 0, qi = d.xsym ? (q - 1) >> 1 : q - 1;
   const int cp = sep_pad128(it.ncols), R1 = sep_rows(d, J_MID, it.ncols, it.col0, CIN), R3 = (CD ? 2 : 1) * cp;
@@ -837,7 +856,7 @@ __device__ __forceinline__ void sep_modes_body(const Item &it, const SubDesc &d,
       for (int r = 0; r < 4; ++r) out[1 - p][2 + r] = fma(T[MT_P1G + r], A, fma(T[MT_P2G + r], B, out[1 - p][2 + r]));
     }
   }
-  double *ae = ws + it.a_off + w.aeff + ((long long)e * 2 * g.nqp + qi) * R3 + b;
+  double *ae = ws + it.a_off + w.aeff + ((long long)e * 2 * g.nqp + qi) * R3 + row;
   ae[0] = out[0][0];
   ae[(long long)g.nqp * R3] = out[0][1];
   if (CD) { ae[cp] = out[1][0]; ae[(long long)g.nqp * R3 + cp] = out[1][1]; }
@@ -868,10 +887,11 @@ __global__ void __launch_bounds__(128) k_sep_modes(Batch bt, const SubDesc *subs
   if (b >= it.ncols) return;
   const SepGeo g = sep_geo(d);
   const SepWs w = sep_ws(d, it.ncols);
-  const int row1 = CIN ? b : sep_side_row(d, it.col0, b);
+  const int row = CIN ? b : sep_row_of(d, it.col0, it.ncols, b);
+  const int row1 = CIN ? b : row - sep_first34(d, it.col0, it.ncols);
   for (int q = q0; q < q0 + SEP_MODES_PER_BLOCK - (int)threadIdx.y && q <= d.Nq; q += 4) {
-    if (d.cplx || CIN) sep_modes_body<true, CIN>(it, d, g, w, sep, ws, b, row1, q);
-    else sep_modes_body<false, CIN>(it, d, g, w, sep, ws, b, row1, q);
+    if (d.cplx || CIN) sep_modes_body<true, CIN>(it, d, g, w, sep, ws, b, row, row1, q);
+    else sep_modes_body<false, CIN>(it, d, g, w, sep, ws, b, row, row1, q);
   }
 }
 
@@ -883,13 +903,14 @@ __device__ __forceinline__ void sep_out_body(const Item &it, const SubDesc &d, c
   const SepGeo g = sep_geo(d);
   const SepWs w = sep_ws(d, it.ncols);
   const int cp = sep_pad128(it.ncols), R1 = sep_rows(d, J_MID, it.ncols, it.col0, CIN), R3 = (CD ? 2 : 1) * cp;
-  const int row1 = CIN ? b : sep_side_row(d, it.col0, b);
+  const int row = CIN ? b : sep_row_of(d, it.col0, it.ncols, b);
+  const int row1 = CIN ? b : row - sep_first34(d, it.col0, it.ncols);
   const double sc = 2.0 / d.Nx;
   cplx v[4];
 #pragma unroll
   for (int k = 0; k < 4; ++k) {   // (class, output) or output
     const long long t = (long long)k * g.Pi + i;
-    const double *p3 = ws + it.a_off + w.u3 + t * R3 + b, *p1 = ws + it.a_off + w.u1 + t * R1 + row1;
+    const double *p3 = ws + it.a_off + w.u3 + t * R3 + row, *p1 = ws + it.a_off + w.u1 + t * R1 + row1;
     v[k] = cmk(sc * p3[0], CD ? sc * p3[cp] : 0.0);
     if (row1 >= 0) {
       v[k].re += p1[0];
@@ -920,7 +941,8 @@ __device__ __forceinline__ void sep_rows_out_body(const Item &it, const SubDesc 
   const SepGeo g = sep_geo(d);
   const int cp = sep_pad128(it.ncols), parts = CD ? 2 : 1, R = sep_rows(d, J_INV, it.ncols, it.col0, CIN);
   const double *ui = ws + it.a_off + sep_ws(d, it.ncols).ui, sc = 2.0 / d.Nx;
-  const int b = b0 + threadIdx.x, row = slot * parts * cp + b;
+  const int b = b0 + threadIdx.x;
+  const int row = slot * parts * cp + (CIN || b >= it.ncols ? b : sep_row_of(d, it.col0, it.ncols, b));
   for (int k = threadIdx.y; k < 32; k += 8) {
     const int m = mt * 32 + k;
     cplx u0 = cmk(0.0, 0.0), u1 = u0;
@@ -1005,6 +1027,10 @@ cudaError_t launch_sep_tables(const mdp_plan *p, const SubDesc *ds, const double
     mmk = std::max(mmk, (g.nk1 + 3) / 4);
     m3 = std::max(m3, g.ncls * g.nt3);
     m3k = std::max(m3k, (g.nk3 + 3) / 4);
+  }
+  if (p->sep_masks > 0) {
+    const cudaError_t e = cudaMemsetAsync(sep, 0, (size_t)p->sep_masks, st);
+    if (e != cudaSuccess) return e;
   }
   const int ns = (int)p->subs.size();
   for (int s0 = 0; s0 < ns; s0 += 65535) {   // subdomains per launch: a grid's y / z limit

@@ -61,6 +61,7 @@ struct SubDesc {
   long long tcb_off;    // doubles: per 16 modes a 1 KiB block of the fp16 digits of the sines at the adjoint's
                         // ring columns, in the shared-memory operand layout of k_adj_cols_tc
   // bytes into the plan's separable tables (kernels_sep.cu), device only; without tc_cols the first three
+  long long sep_zm, sep_z3;   // words: masks of the nonzero groups of K of sep_mb's and sep_b3's tiles
   long long sep_ab;     // doubles [Nq][2]: interior entries (off-diagonal, diagonal) of T_q
   long long sep_mt;     // per mode SEP_MTW doubles
   long long sep_phi;    // doubles [2][Py + 2][Nq]: phi_1, phi_2 on the rows nlo-1 .. nhi+1
@@ -176,23 +177,34 @@ inline __host__ __device__ int sep_src_col(const SubDesc &d, int c) {
   return c == 0 ? d.mlo : c == 1 ? d.mlo + 1 : c == 2 ? d.mhi - 1 : d.mhi;
 }
 inline __host__ __device__ int sep_pad128(int n) { return (n + 127) / 128 * 128; }
-// Only the basis columns of sides 3 and 4 have residuals on the middle ring rows (the gamma nodes
-// next to them belong to these sides), so MID has only their rows: sep_side_before counts such
-// columns below column c, sep_side_col gives the row-th one from column c0 on, sep_side_row the
-// row of an item's column b (-1: a column of side 1 or 2).
-inline __host__ __device__ int sep_side_before(const SubDesc &d, int c) {
-  const int M = d.n_modes, r = c % (4 * M) - 2 * M;
-  return (c / (4 * M)) * 2 * M + (r > 0 ? r : 0);
+// The rows of A take an item's basis columns side by side (Dirichlet, then Neumann columns of side 1,
+// of side 2, ...), so that a tile's columns share their zeros; user densities stay in order.
+// Columns c0 .. c0 + ncols - 1 that are of side s (0..3) and kind k:
+inline __host__ __device__ int sep_seg(const SubDesc &d, int c0, int ncols, int s, int k) {
+  const int M = d.n_modes, lo = (4 * k + s) * M, hi = lo + M;
+  const int a = c0 > lo ? c0 : lo, b = c0 + ncols < hi ? c0 + ncols : hi;
+  return b > a ? b - a : 0;
 }
-inline __host__ __device__ int sep_side_cols(const SubDesc &d, int c0, int ncols) {
-  return sep_side_before(d, c0 + ncols) - sep_side_before(d, c0);
+// row of the item's column b, and its column
+inline __host__ __device__ int sep_row_of(const SubDesc &d, int c0, int ncols, int b) {
+  const int M = d.n_modes, c = c0 + b, k = c / (4 * M), s = (c % (4 * M)) / M, lo = (4 * k + s) * M;
+  int row = c - (c0 > lo ? c0 : lo);
+  for (int t = 0; t < s; ++t) row += sep_seg(d, c0, ncols, t, 0) + sep_seg(d, c0, ncols, t, 1);
+  return k ? row + sep_seg(d, c0, ncols, s, 0) : row;
 }
-inline __host__ __device__ int sep_side_col(const SubDesc &d, int c0, int row) {
-  const int f = sep_side_before(d, c0) + row, M2 = 2 * d.n_modes;
-  return (f / M2) * 2 * M2 + M2 + f % M2;
+inline __host__ __device__ int sep_col_of(const SubDesc &d, int c0, int ncols, int row) {
+  for (int s = 0; s < 4; ++s)
+    for (int k = 0; k < 2; ++k) {
+      const int n = sep_seg(d, c0, ncols, s, k), lo = (4 * k + s) * d.n_modes;
+      if (row < n) return (c0 > lo ? c0 : lo) + row - c0;
+      row -= n;
+    }
+  return 0;
 }
-inline __host__ __device__ int sep_side_row(const SubDesc &d, int c0, int b) {
-  return (c0 + b) % (4 * d.n_modes) < 2 * d.n_modes ? -1 : sep_side_before(d, c0 + b) - sep_side_before(d, c0);
+// Only the basis columns of sides 3 and 4 have residuals on the middle ring rows (the gamma nodes next
+// to them belong to these sides): MID has their rows only, the item's last ones; columns of sides 1, 2:
+inline __host__ __device__ int sep_first34(const SubDesc &d, int c0, int ncols) {
+  return sep_seg(d, c0, ncols, 0, 0) + sep_seg(d, c0, ncols, 0, 1) + sep_seg(d, c0, ncols, 1, 0) + sep_seg(d, c0, ncols, 1, 1);
 }
 // Rows of A, a multiple of the MMA's 128: the item's columns padded to 128, times real and imaginary
 // parts where the data (MID, FWD: user densities) or the results (SYN, INV) are complex, times the
@@ -200,7 +212,7 @@ inline __host__ __device__ int sep_side_row(const SubDesc &d, int c0, int b) {
 inline __host__ __device__ int sep_rows(const SubDesc &d, int job, int ncols, int col0, bool user) {
   const int cp = sep_pad128(ncols);
   switch (job) {
-    case J_MID: return user ? 2 * cp : sep_pad128(sep_side_cols(d, col0, ncols));
+    case J_MID: return user ? 2 * cp : sep_pad128(ncols - sep_first34(d, col0, ncols));
     case J_FWD: return (user ? 8 : 4) * cp;
     case J_SYN: return (user || d.cplx ? 2 : 1) * cp;
     default: return (d.nrec >= 0 ? 5 : 4) * (user || d.cplx ? 2 : 1) * cp;
@@ -323,7 +335,8 @@ struct mdp_plan {
   mdp::HostBuf<uint8_t> host_piv;
   long long out_size = 0;
   long long rec_size = 0;
-  int tile_cols = 256;                   // columns per work item
+  int tile_cols = 256;                   // columns per work item of sweeps and of the gradient pass
+  int sep_cols = 512;                    // columns per work item of the separable solve
   int fft_block_points = mdp::FFT_BLOCK_POINTS;  // complex values per block of the dense-row FFT kernels
   int tri_stages = 2;                    // table rows the projection sweep stages ahead (2 or 4)
   long long ws_budget = 0;               // bytes of workspace
@@ -337,7 +350,7 @@ struct mdp_plan {
   double *d_tables = nullptr;
   uint8_t *d_piv = nullptr;
   unsigned char *d_sep = nullptr;        // separable tables (kernels_sep.cu), rebuilt with the factor tables
-  long long sep_bytes = 0;
+  long long sep_bytes = 0, sep_masks = 0;   // size; its first bytes: the masks, cleared before a rebuild
   double *d_ws = nullptr;
   long long ws_doubles = 0;
   int *d_status = nullptr;

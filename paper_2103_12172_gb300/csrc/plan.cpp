@@ -402,18 +402,26 @@ void host_mode_solve(const HostSub &hs, int q, int adjoint, const double *b, dou
 static bool layout_tables(mdp_plan *p) {
   long long off = 0, poff = 0, out = 0, sep = 0;
   auto al = [](long long v) { return (v + 31) & ~31LL; };
+  auto take = [&](long long bytes) { const long long o = sep; sep += (bytes + 255) & ~255LL; return o; };
+  for (auto &hs : p->subs) {
+    SubDesc &d = hs.d;
+    if (d.leader != (int)(&hs - p->subs.data()) || !d.tc_cols) continue;
+    const SepGeo g = sep_geo(d);
+    d.sep_zm = take(4LL * SEP_MASK * g.ncls * (3 * g.nqp / 32));
+    d.sep_z3 = take(4LL * SEP_MASK * g.ncls * g.nt3);
+  }
+  p->sep_masks = sep;
   for (auto &hs : p->subs) {
     SubDesc &d = hs.d;
     if (d.leader != (int)(&hs - p->subs.data())) {   // a duplicate: the leader's tables
       const SubDesc &ld = p->subs[d.leader].d;
       d.fact_off = ld.fact_off; d.dT_off = ld.dT_off; d.sin_off = ld.sin_off; d.geo_off = ld.geo_off;
       d.seg_off = ld.seg_off; d.fs_off = ld.fs_off; d.piv_off = ld.piv_off; d.tcb_off = ld.tcb_off;
-      d.sep_ab = ld.sep_ab; d.sep_mt = ld.sep_mt; d.sep_phi = ld.sep_phi; d.sep_kd = ld.sep_kd; d.sep_kde = ld.sep_kde;
+      d.sep_zm = ld.sep_zm; d.sep_z3 = ld.sep_z3; d.sep_ab = ld.sep_ab; d.sep_mt = ld.sep_mt; d.sep_phi = ld.sep_phi; d.sep_kd = ld.sep_kd; d.sep_kde = ld.sep_kde;
       d.sep_tb = ld.sep_tb; d.sep_mb = ld.sep_mb; d.sep_b3 = ld.sep_b3; d.sep_bf = ld.sep_bf; d.sep_bi = ld.sep_bi;
       d.out_off = out;  out += (long long)d.G * d.n_cols;
       continue;
     }
-    auto take = [&](long long bytes) { const long long o = sep; sep += (bytes + 255) & ~255LL; return o; };
     d.sep_ab = take(16LL * d.Nq);
     d.sep_mt = take(8LL * SEP_MTW * d.Nq);
     d.sep_phi = take(16LL * (d.Py + 2) * d.Nq);
@@ -525,10 +533,11 @@ static void schedule_pass(mdp_plan *p, bool grad, bool leaders_only, std::vector
   for (int si = 0; si < (int)p->subs.size(); ++si) {
     if (leaders_only && p->leader[si] != si) continue;
     const SubDesc &d = p->subs[si].d;
-    for (int c0 = 0; c0 < d.n_cols; c0 += p->tile_cols) {
+    const int cols = grad || !d.tc_cols ? p->tile_cols : p->sep_cols;
+    for (int c0 = 0; c0 < d.n_cols; c0 += cols) {
       Item it;
       std::memset(&it, 0, sizeof it);
-      it.sub = si; it.col0 = c0; it.ncols = std::min(p->tile_cols, d.n_cols - c0);
+      it.sub = si; it.col0 = c0; it.ncols = std::min(cols, d.n_cols - c0);
       long long xi, r, gr, y, a, s, red, tot;
       item_workspace(d, it.ncols, grad, xi, r, gr, y, a, s, red, tot);
       if (!cur.items.empty() && cur.ws_doubles + tot > budget) {
