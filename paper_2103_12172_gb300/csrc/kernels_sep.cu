@@ -38,6 +38,7 @@
 #include "tc_common.cuh"
 
 #include <algorithm>
+#include <climits>
 
 namespace mdp {
 namespace {
@@ -440,6 +441,18 @@ __global__ void __launch_bounds__(256) k_sep_sines(const SubDesc *subs, int s0, 
 // digits are all zero in 128 rows (the imaginary parts of evanescent modes, the ring away from a
 // column's side) are left out of the contraction by their bit in the tile's mask; so are those of the
 // moment and synthesis tables, where phi has decayed below 2^-55 (nine tenths of them at 1025^2).
+// round(x 2^(1076 - E)) for |x| < 2^(E - 1022), 53 <= E (nothing for E = 2047: Inf or NaN in the row), by
+// integer operations: the significand (53 bits) lies e - 1075 up, so it moves up one bit for e = E and
+// down E - e - 1 bits otherwise, rounded half up
+__device__ __forceinline__ long long fixed_of(double x, int E) {
+  const long long b = __double_as_longlong(x);
+  const int e = (int)((b >> 52) & 0x7ff);
+  const unsigned long long m = (e ? 1ULL << 52 : 0ULL) | (b & 0xfffffffffffffLL);
+  const int s = min(E - (e ? e : 1), 63);          // 0: up one bit
+  const long long v = (long long)(((m << 2) >> s) + 1) >> 1;
+  return E < 2047 ? (b < 0 ? -v : v) : 0;
+}
+
 template <bool CIN, int JOB>
 __device__ __forceinline__ void sep_cut_body(const Item &it, const SubDesc &d, double *ws, int local) {
   const SepGeo g = sep_geo(d);
@@ -486,8 +499,14 @@ __device__ __forceinline__ void sep_cut_body(const Item &it, const SubDesc &d, d
   __shared__ unsigned smask[SEP_MASK];
   if (threadIdx.x < 8) { emax[threadIdx.x] = 0; smask[threadIdx.x] = 0; }
   __syncthreads();
+  // the first 256 values of K stay in registers between the two passes
+  double x[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) x[j] = kl < 2 * nk ? value(8 * kl + j) : 0.0;
   int m = 0;
-  for (int k8 = kl; k8 < 2 * nk; k8 += 32)
+#pragma unroll
+  for (int j = 0; j < 8; ++j) m = max(m, (__double2hiint(x[j]) >> 20) & 0x7ff);
+  for (int k8 = kl + 32; k8 < 2 * nk; k8 += 32)
 #pragma unroll
     for (int j = 0; j < 8; ++j) m = max(m, (__double2hiint(value(8 * k8 + j)) >> 20) & 0x7ff);
   for (int off = 16; off >= 8; off >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, off));
@@ -495,7 +514,6 @@ __device__ __forceinline__ void sep_cut_body(const Item &it, const SubDesc &d, d
   __syncthreads();
   const int E = max(emax[threadIdx.x & 7], 53);
   if (kl == 0) reinterpret_cast<int *>(ws + it.a_off + w.ex[JOB])[e * R + row] = E;
-  const double sc = pow2i(1076 - E);          // |x| < 2^(E - 1022) -> |V| < 2^54
   unsigned char *A = reinterpret_cast<unsigned char *>(ws + it.a_off + w.a[JOB]) +
                      ((long long)(e * (R / 128) + row / 128) * nk) * SEP_ABLK;
   const int r = row & 127, off0 = (r >> 3) * 256 + (r & 7) * 16;
@@ -503,7 +521,7 @@ __device__ __forceinline__ void sep_cut_body(const Item &it, const SubDesc &d, d
     long long V[8], any = 0;
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
-      V[j] = E < 2047 ? __double2ll_rn(value(8 * k8 + j) * sc) : 0;
+      V[j] = fixed_of(k8 == kl ? x[j] : value(8 * k8 + j), E);   // |x| < 2^(E - 1022) -> |V| <= 2^54
       any |= V[j];
     }
     if (any) atomicOr(&smask[k8 >> 6], 1u << ((k8 >> 1) & 31));
@@ -562,6 +580,25 @@ __device__ __forceinline__ void bulk_load(unsigned dst, const void *src, unsigne
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
                "l"(src), "r"(bytes), "r"(bar)
                : "memory");
+}
+
+// (hi 2^32 + lo) 2^ex, rounded to nearest, by integer operations: the FP64 pipe takes 64 cycles per warp
+// instruction, and three conversions per output had taken as long as the tile's MMAs.
+__device__ __forceinline__ double sum_to_double(long long hi, long long lo, int ex) {
+  long long h = hi + (lo >> 32);          // |h| < 2^51
+  unsigned l = (unsigned)lo;
+  const bool neg = h < 0;
+  if (neg) { h = ~h + (l == 0 ? 1 : 0); l = 0u - l; }
+  const int lz = h ? __clzll(h) : 64 + __clz((int)l);
+  // the leading 64 bits of the 96, then 53 of them rounded
+  unsigned long long top = lz <= 32 ? ((unsigned long long)l << lz) >> 32 : (unsigned long long)l << ((lz - 32) & 63);
+  if (lz < 64) top |= (unsigned long long)h << lz;
+  const int e = 1023 + 95 - lz + ex;      // biased exponent
+  unsigned long long v = ((unsigned long long)(e - 1) << 52) + (top >> 11) + ((top >> 10) & 1);
+  if (lz == 96 || e < 1) v = 0;
+  if (e > 2046) v = 0x7ff0000000000000ULL;
+  if (ex == INT_MAX) v = 0x7ff8000000000000ULL;
+  return __longlong_as_double((long long)(v | ((unsigned long long)neg << 63)));
 }
 
 struct SepTile {
@@ -756,8 +793,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1)
       const bool direct = t.job == J_MID && t.nt < g.nt3;
       int eb = 0;
       if (direct) eb = reinterpret_cast<const int *>(sep + d.sep_kde)[t.e * g.nS + t.nt / g.nti];
-      double s0 = pow2i(E - 1090 + eb), s1 = pow2i(E - 1058 + eb);
-      if (E >= 2047) s0 = s1 = __longlong_as_double(0x7ff8000000000000LL);   // Inf or NaN in the row
+      const int ex = E < 2047 ? E - 1090 + eb : INT_MAX;   // Inf or NaN in the row: NaN
       double *dst;
       int cnt;                   // outputs of this thread, `step` doubles apart
       long long step = t.R;
@@ -781,16 +817,9 @@ __global__ void __launch_bounds__(SG_THREADS, 1)
         step = 2LL * it.ncols * parts;
         dst = ws + it.gr_off + (((long long)(row / (cp * parts)) * d.Nq + 2 * o0 + t.e) * it.ncols + col) * parts + (row / cp) % parts;
       }
-      constexpr long long MG = 0x4338000000000000LL;   // 1.5 2^52 + x for |x| < 2^51
-      const double M = __longlong_as_double(MG);
 #pragma unroll
       for (int o = 0; o < 16; ++o)
-        if (o < cnt) {
-          // carry the part of lo above 2^32 into hi: both then lie below 2^51
-          const long long h = hi[o] + (lo[o] >> 32), l = lo[o] & 0xffffffffLL;
-          const double dh = __longlong_as_double(MG + h) - M, dl = __longlong_as_double(MG + l) - M;
-          dst[o * step] = fma(dh, s1, dl * s0);
-        }
+        if (o < cnt) dst[o * step] = sum_to_double(hi[o], lo[o], ex);
     }
   }
   if (abort_sh && tid == 0) atomicCAS(status, 0, (int)MDP_ERR_TIMEOUT);   // the first error sticks
