@@ -1264,6 +1264,7 @@ __global__ void k_full_inv(const SubDesc *subs, int sub, const double *tab, cons
 cudaError_t launch_solve(const mdp_plan *p, int sub, int nrhs, const double2 *g, double2 *u, int adjoint,
                          cudaStream_t st) {
   const SubDesc &d = p->subs[sub].d;
+  if (!adjoint && d.tc_cols) return launch_full_solve(p, sub, nrhs, g, u, st);
   const long long per = (long long)d.Nq * d.Nt * 2;
   long long chunk = p->ws_doubles / per;
   if (chunk < 1) return cudaErrorMemoryAllocation;
@@ -1430,7 +1431,7 @@ cudaError_t launch_source_terms(mdp_plan *p, int sub, const double2 *f, const do
   const long long scratch = 2LL * d.G + 2 * npt + 64;
   long long xo, ro, go, yo, ao, so, reo, tot;
   item_workspace(d, 1, false, xo, ro, go, yo, ao, so, reo, tot);
-  const long long need = std::max((long long)d.Nq * d.Nt * 2, tot) + scratch;
+  const long long need = std::max({(long long)d.Nq * d.Nt * 2, tot, d.tc_cols ? full_ws(d, 1).total : 0}) + scratch;
   if (p->ws_doubles < need) return cudaErrorMemoryAllocation;
   const long long top = (p->ws_doubles - scratch) & ~31LL;
   double2 *xi_i = reinterpret_cast<double2 *>(p->d_ws + top);
@@ -1496,6 +1497,7 @@ cudaError_t set_kernel_attributes() {
   if (e == cudaSuccess) e = set_adj_kernel_attributes();
   if (e == cudaSuccess) e = set_tc_kernel_attributes();
   if (e == cudaSuccess) e = set_sep_kernel_attributes();
+  if (e == cudaSuccess) e = set_full_kernel_attributes();
   // the sweep's staging buffers take 32 x 2.4 KiB per SM at full occupancy: prefer shared memory
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_tri<false, false, 2>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);

@@ -25,74 +25,35 @@
 // On x-centred subdomains odd and even modes separate (sums and differences of the mirrored
 // columns), which halves both dimensions: two classes with 2 columns each, else one with 4.
 //
-// Both contractions are to FP64 accuracy on the fp16 tensor cores by error-free splitting (Ozaki,
-// Ogita, Oishi and Rump, Numer. Algorithms 59, 2012): every operand value becomes an integer
-// |V| <= 2^54 on one scale (a row of A: its largest value; B: a bound of its table) and V 7 balanced
-// base-256 digits, exact in fp16. Of the 49 digit products those of weight t + u <= 7 are kept (34;
-// the largest dropped one is 2^-64 of the leading one, below the operands' own 2^-54). Products of
-// equal weight share one FP32 accumulator: at most 7 x 128 x 2^14 < 2^24 between two read-backs of
-// 128 values of K, so every sum is an exact integer. The read-backs are added in int64.
+// Both contractions are to FP64 accuracy on the fp16 tensor cores (digit_gemm.cuh).
 // Against 64-bit sums over the closed form in extended precision (k = 10 on 129^2, k = 30 on
 // 257^2) the result is off by 1e-15 to 8e-15 (2-norm), plain FP64 sums by 4e-15 to 5e-14 and the
 // pivoted recurrences by 4e-14 to 2.5e-13.
-#include "tc_common.cuh"
+#include "sep_modes.cuh"
 
 #include <algorithm>
-#include <climits>
 
 namespace mdp {
 namespace {
 
 // ---------------------------------------------------------------- mode table
-__device__ __forceinline__ cplx cdivd(cplx a, cplx b) {
-  const double n = 1.0 / fma(b.re, b.re, b.im * b.im);
-  return {fma(a.re, b.re, a.im * b.im) * n, fma(a.im, b.re, -a.re * b.im) * n};
-}
-__device__ __forceinline__ double pow2i(int k) {
-  return k < -1022 ? 0.0 : __longlong_as_double((long long)(min(k, 1023) + 1023) << 52);
-}
-// the two homogeneous solutions at distance x from the middle row (kinds 0 and 1)
-__device__ __forceinline__ double sep_c(int kind, double th, double x) { return kind == 0 ? cos(x * th) : cosh(x * th); }
-__device__ __forceinline__ double sep_s(int kind, double th, double x) {
-  if (th == 0.0) return x;
-  return kind == 0 ? sin(x * th) / sin(th) : sinh(x * th) / sinh(th);
-}
-
 __global__ void __launch_bounds__(128) k_sep_mode_tab(const SubDesc *subs, int s0, unsigned char *sep, int entries) {
   const int si = s0 + blockIdx.y;
   const SubDesc &d = subs[si];
   const int q = blockIdx.x * 128 + threadIdx.x + 1;
   if (d.leader != si || q > d.Nq) return;
   double *T = reinterpret_cast<double *>(sep + d.sep_mt) + (long long)(q - 1) * SEP_MTW;
-  const double h = d.h, h2 = h * h, k = d.k, k2 = k * k;
-  const double sq = sin(M_PI * q / (2.0 * d.Nx)), lam = -4.0 * sq * sq;
-  // the interior entries (a, b) of T_q as the factorisation of these tables rounded them (the host's at
-  // plan creation, else this device's): e = b + 2 a is exact, and an error of b moves theta by its
-  // half over theta^2, so both forms of the solve are to start from the same b
   double *ab = reinterpret_cast<double *>(sep + d.sep_ab) + 2 * (q - 1);
-  if (entries) {
+  if (entries) {   // as mode_rows of factor.cu
+    const double h2 = d.h * d.h, k2 = d.k * d.k;
+    const double sq = sin(M_PI * q / (2.0 * d.Nx)), lam = -4.0 * sq * sq;
     ab[0] = 1.0 / h2 + lam / (6.0 * h2) + k2 / 12.0;
     ab[1] = -2.0 * ab[0] + lam / h2 + k2 + k2 * lam / 12.0;
   }
-  double a = ab[0];
-  const double e = ab[1] + 2.0 * a;
-  double t = e / (4.0 * a);                             // sin^2(theta/2), or -sinh^2(theta/2)
-  // coarse grids (t > 1/2): x_i = (-1)^i z_i turns (a, b, a) into (-a, b, -a)
-  double sg = 1.0;
-  if (t > 0.5) { sg = -1.0; t = 1.0 - t; a = -a; }
-  const int N = d.ny - 1, J0 = d.nlo - 1, J1 = d.nhi + 1;
+  const ModeShape ms = mode_shape(d, q, ab);
+  const double a = ms.a, sg = ms.sg, th = ms.th;
+  const int kind = ms.kind, N = d.ny - 1, J0 = d.nlo - 1, J1 = d.nhi + 1;
   const double mid = 0.5 * (J0 + J1), Lh = 0.5 * (J1 - J0);
-  const double th = t > 0.0 ? 2.0 * asin(sqrt(t)) : 2.0 * asinh(sqrt(-t));
-  const int kind = t > 0.0 ? 0 : th * N < 4.0 ? 1 : 2;
-  // rows at the ends: al0 x_0 + al1 x_1 = 0 and its mirror image
-  cplx al0 = cmk(1.0, 0.0), al1 = cmk(0.0, 0.0);
-  if (d.cplx) {
-    const bool paper = d.ap_bc == MDP_AP_DIRX_SOMMY_PAPER;
-    const double alpha = paper ? (1.0 - k2 * h2 / 24.0 - lam / 6.0) / h2 : (1.0 + k2 * h2 / 24.0 + lam / 24.0) / h2;
-    const double beta = k * (1.0 + k2 * h2 / 8.0 + lam / (paper ? 2.0 : 8.0)) / h;
-    al0 = cmk(alpha, 0.5 * beta);
-    al1 = cmk(-sg * alpha, 0.5 * sg * beta);
-  }
   double n1 = 1.0, n2 = 1.0, c = 0.0, rf;
   cplx R11, R12, R22;
   const int rows_d[4] = {d.nlo, d.nlo + 1, d.nhi - 1, d.nhi}, rows_g[4] = {d.nlo - 1, d.nlo, d.nhi, d.nhi + 1};
@@ -102,17 +63,7 @@ __global__ void __launch_bounds__(128) k_sep_mode_tab(const SubDesc *subs, int s
     if (kind == 0) bound = fmin(bound, 1.0 / sin(th));
     n2 = pow2i(-(ilogb(fmax(bound, 1.0)) + 1));
     if (kind == 1) n1 = 0.25;
-    const double C0 = sep_c(kind, th, 0.0 - mid), C1 = sep_c(kind, th, 1.0 - mid);
-    const double S0 = sep_s(kind, th, 0.0 - mid), S1 = sep_s(kind, th, 1.0 - mid);
-    const double D0 = sep_c(kind, th, N - mid), D1 = sep_c(kind, th, N - 1 - mid);
-    const double E0 = sep_s(kind, th, N - mid), E1 = sep_s(kind, th, N - 1 - mid);
-    auto lin = [&](double x, double y) { return cmk(fma(al0.re, x, al1.re * y), fma(al0.im, x, al1.im * y)); };
-    const cplx b1 = lin(C0, C1), b2 = lin(S0, S1), t1 = lin(D0, D1), t2 = lin(E0, E1);
-    const cplx det = csub(cmul(b1, t2), cmul(b2, t1));
-    const cplx ad = cmk(a * det.re, a * det.im);
-    R11 = cdivd(cmul(b2, t2), ad);
-    R22 = cdivd(cmul(b1, t1), ad);
-    R12 = cdivd(cadd(cmul(b1, t2), cmul(b2, t1)), cmk(-2.0 * ad.re, -2.0 * ad.im));
+    reflect_cs(ms, N, mid, R11, R12, R22);
     const double s1 = 1.0 / n1, s2 = 1.0 / n2;
     R11 = cmk(R11.re * s1 * s1, R11.im * s1 * s1);
     R12 = cmk(R12.re * s1 * s2, R12.im * s1 * s2);
@@ -121,18 +72,8 @@ __global__ void __launch_bounds__(128) k_sep_mode_tab(const SubDesc *subs, int s
     if (kind == 0) kb = fmin(kb, 1.0 / sin(th));
     rf = pow2i(-(ilogb(fmax(kb, 1.0) / (2.0 * fabs(a))) + 1));
   } else {
-    const double ep = exp(th), em = exp(-th);
     c = -1.0 / (2.0 * a * sinh(th));
-    const cplx num = cmk(fma(al1.re, ep, al0.re), fma(al1.im, ep, al0.im));
-    const cplx den = cmk(fma(al1.re, em, al0.re), fma(al1.im, em, al0.im));
-    const cplx ref = cdivd(num, den);
-    const double wb = -exp(-2.0 * th * J0), wt = -exp(-2.0 * th * (N - J1)), dl = exp(-th * (J1 - J0));
-    const cplx rb = cmk(wb * ref.re, wb * ref.im), rt = cmk(wt * ref.re, wt * ref.im);
-    const cplx rr = cmul(rb, rt);
-    const cplx D = cmk(1.0 - rr.re * dl * dl, -rr.im * dl * dl);
-    R11 = cdivd(cmk(c * rb.re, c * rb.im), D);
-    R22 = cdivd(cmk(c * rt.re, c * rt.im), D);
-    R12 = cdivd(cmk(c * dl * rr.re, c * dl * rr.im), D);
+    reflect_exp(ms, N, J0, J1, c, R11, R12, R22);
     rf = pow2i(-(ilogb(fabs(c)) + 1));
   }
   auto p1 = [&](int i) { return sgn(i - J0) * (kind == 2 ? exp(-th * (i - J0)) : n1 * sep_c(kind, th, i - mid)); };
@@ -278,24 +219,6 @@ __global__ void __launch_bounds__(128) k_sep_kd(const SubDesc *subs, int s0, con
   }
 }
 
-// the 7 digits of 8 consecutive-K values |x| 2^(54 - e) at 16 bytes each, `stride` bytes apart
-__device__ __forceinline__ void store_digits(unsigned char *dst, long long stride, const long long *V) {
-  unsigned hi[8], lo[8];
-#pragma unroll
-  for (int j = 0; j < 8; ++j) {
-    const unsigned long long w = (unsigned long long)V[j] + 0x0080808080808080ull;
-    hi[j] = (unsigned)(w >> 32);
-    lo[j] = (unsigned)w;
-  }
-#define MDP_SEP_DIGIT(T)                                                        \
-  *reinterpret_cast<uint4 *>(dst + (T) * stride) =                              \
-      make_uint4(digit_pair<6 - (T)>(hi[0], lo[0], hi[1], lo[1]),               \
-                 digit_pair<6 - (T)>(hi[2], lo[2], hi[3], lo[3]),               \
-                 digit_pair<6 - (T)>(hi[4], lo[4], hi[5], lo[5]),               \
-                 digit_pair<6 - (T)>(hi[6], lo[6], hi[7], lo[7]));
-  MDP_SEP_DIGIT(0) MDP_SEP_DIGIT(1) MDP_SEP_DIGIT(2) MDP_SEP_DIGIT(3) MDP_SEP_DIGIT(4) MDP_SEP_DIGIT(5) MDP_SEP_DIGIT(6)
-#undef MDP_SEP_DIGIT
-}
 // set bit kb of a tile's mask if the warp (32 outputs, one half of the 16 values of K) has a nonzero digit
 __device__ __forceinline__ void mark_group(unsigned *mask, int kb, const long long *V) {
   long long any = 0;
@@ -303,9 +226,6 @@ __device__ __forceinline__ void mark_group(unsigned *mask, int kb, const long lo
   for (int j = 0; j < 8; ++j) any |= V[j];
   if (__any_sync(0xffffffffu, any != 0) && (threadIdx.x & 31) == 0) atomicOr(mask + (kb >> 5), 1u << (kb & 31));
 }
-// table value |x| <= 1 on the fixed scale 2^54
-__device__ __forceinline__ long long fix54(double x) { return __double2ll_rn(x * 0x1p54); }
-
 // The Toeplitz blocks of K (32 outputs x 16 sources, by the offset of the two groups) on the scale of
 // the largest |K_sc| of the output column: 64 threads (32 outputs x 2 K halves) per block.
 __global__ void __launch_bounds__(256) k_sep_tb(const SubDesc *subs, int s0, unsigned char *sep) {
@@ -408,14 +328,17 @@ __global__ void __launch_bounds__(256) k_sep_b3(const SubDesc *subs, int s0, con
   store_digits(B + (o >> 3) * 256 + half * 128 + (o & 7) * 16, 1024, V);
 }
 
-// The sine tables of the full rows' transforms. FWD: output q of parity e, K index m' - mf; INV: output
-// m' - mg, K index q of parity e; both sin(pi q m'/Nx) over the folded columns m' <= Nx/2.
-__global__ void __launch_bounds__(256) k_sep_sines(const SubDesc *subs, int s0, const double *tab, unsigned char *sep, int inv) {
+// The sine tables of the full rows' transforms (which: 0 FWD, 1 INV, 2, 3 the same over every folded column
+// for full-grid solves). FWD: output q of parity e, K index m' - mf; INV: output m' - mg, K index q of
+// parity e; both sin(pi q m'/Nx) over the folded columns m' <= Nx/2.
+__global__ void __launch_bounds__(256) k_sep_sines(const SubDesc *subs, int s0, const double *tab, unsigned char *sep, int which) {
   const int si = s0 + blockIdx.z;
   const SubDesc &d = subs[si];
   if (!d.tc_cols || d.leader != si) return;
   const SepGeo g = sep_geo(d);
-  const int nto = inv ? g.ntg : g.nqh / 32, nk = inv ? g.nqh / 16 : g.nkf;
+  const bool inv = which & 1, full = which & 2;
+  const int nto = inv ? (full ? g.ntx : g.ntg) : g.nqh / 32, nk = inv ? g.nqh / 16 : full ? g.nkx : g.nkf;
+  const int m0 = full ? 1 : inv ? g.mg : g.mf;
   const int e = blockIdx.y / nto, to = blockIdx.y % nto;
   const int kb = blockIdx.x * 4 + (threadIdx.x >> 6);
   if (e >= 2 || kb >= nk) return;
@@ -425,10 +348,10 @@ __global__ void __launch_bounds__(256) k_sep_sines(const SubDesc *subs, int s0, 
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
     const int ko = to * 32 + o, kk = kb * 16 + 8 * half + j;
-    const int q = sep_parity_mode(e, inv ? kk : ko), m = inv ? g.mg + ko : g.mf + kk;
+    const int q = sep_parity_mode(e, inv ? kk : ko), m = m0 + (inv ? ko : kk);
     V[j] = q <= d.Nq && 2 * m <= d.Nx ? fix54(S[(int)(((long long)q * m) % (2 * d.Nx))]) : 0;
   }
-  unsigned char *B = sep + (inv ? d.sep_bi : d.sep_bf) + (((long long)e * nto + to) * nk + kb) * SEP_BBLK;
+  unsigned char *B = sep + (full ? (inv ? d.sep_xi : d.sep_xf) : inv ? d.sep_bi : d.sep_bf) + (((long long)e * nto + to) * nk + kb) * SEP_BBLK;
   store_digits(B + (o >> 3) * 256 + half * 128 + (o & 7) * 16, 1024, V);
 }
 
@@ -441,18 +364,6 @@ __global__ void __launch_bounds__(256) k_sep_sines(const SubDesc *subs, int s0, 
 // digits are all zero in 128 rows (the imaginary parts of evanescent modes, the ring away from a
 // column's side) are left out of the contraction by their bit in the tile's mask; so are those of the
 // moment and synthesis tables, where phi has decayed below 2^-55 (nine tenths of them at 1025^2).
-// round(x 2^(1076 - E)) for |x| < 2^(E - 1022), 53 <= E (nothing for E = 2047: Inf or NaN in the row), by
-// integer operations: the significand (53 bits) lies e - 1075 up, so it moves up one bit for e = E and
-// down E - e - 1 bits otherwise, rounded half up
-__device__ __forceinline__ long long fixed_of(double x, int E) {
-  const long long b = __double_as_longlong(x);
-  const int e = (int)((b >> 52) & 0x7ff);
-  const unsigned long long m = (e ? 1ULL << 52 : 0ULL) | (b & 0xfffffffffffffLL);
-  const int s = min(E - (e ? e : 1), 63);          // 0: up one bit
-  const long long v = (long long)(((m << 2) >> s) + 1) >> 1;
-  return E < 2047 ? (b < 0 ? -v : v) : 0;
-}
-
 template <bool CIN, int JOB>
 __device__ __forceinline__ void sep_cut_body(const Item &it, const SubDesc &d, double *ws, int local) {
   const SepGeo g = sep_geo(d);
@@ -547,287 +458,93 @@ __global__ void __launch_bounds__(256) k_sep_cut(Batch bt, const SubDesc *subs, 
 }
 
 // ---------------------------------------------------------------- the contractions
-// Persistent CTAs, one per SM: warp 9 streams the digit blocks of A (28 KiB) and B (7 KiB) of 16
-// values of K into 5 shared-memory stages with bulk copies, one thread of warp 8 issues the MMAs,
-// and after every 128 values of K hands one of two accumulator sets (8 weights x 32 outputs, FP32)
-// to the 8 other warps, which add them up as integers and at the end of a tile scale them into
-// FP64. A tile is 128 rows x 32 outputs. One MMA (M = 128, N = 256, K = 16) per A digit t: its B
-// operand starts t digits before B's first one, in 7 KiB of zeros, so that digit u meets the
-// accumulator of weight t + u and every MMA of a set has the same accumulator and shape (MMAs into
-// overlapping accumulators of other shapes have no defined order). The zeros are 22 of 56 digit
-// pairs. What bounds it: the tensor pipe, 7 x 128 cycles per 16 values of K; the operands' way from
-// L2 takes 35 KiB in that time, 39 bytes per cycle and SM.
-constexpr int SG_STAGES = 5, SG_THREADS = 320, SG_CHUNK = 8;   // K16 steps per accumulator set
-constexpr int SG_STAGE_BYTES = SEP_ABLK + SEP_BBLK;
-// shared memory: the A stages, then zeros and B stages in turn, 7 KiB each, and closing zeros
-constexpr int SG_B0 = SG_STAGES * SEP_ABLK;
-constexpr int SG_SMEM = SG_B0 + (2 * SG_STAGES + 1) * SEP_BBLK + 1024;
-
-// 16 consecutive FP32 columns of this warp's 32 TMEM lanes
-__device__ __forceinline__ void tmem_ld16(unsigned taddr, float *v) {
-  unsigned r[16];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr)
-      : "memory");
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
-}
-__device__ __forceinline__ void bulk_load(unsigned dst, const void *src, unsigned bytes, unsigned bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
-               "l"(src), "r"(bytes), "r"(bar)
-               : "memory");
-}
-
-// (hi 2^32 + lo) 2^ex, rounded to nearest, by integer operations: the FP64 pipe takes 64 cycles per warp
-// instruction, and three conversions per output had taken as long as the tile's MMAs.
-__device__ __forceinline__ double sum_to_double(long long hi, long long lo, int ex) {
-  long long h = hi + (lo >> 32);          // |h| < 2^51
-  unsigned l = (unsigned)lo;
-  const bool neg = h < 0;
-  if (neg) { h = ~h + (l == 0 ? 1 : 0); l = 0u - l; }
-  const int lz = h ? __clzll(h) : 64 + __clz((int)l);
-  // the leading 64 bits of the 96, then 53 of them rounded
-  unsigned long long top = lz <= 32 ? ((unsigned long long)l << lz) >> 32 : (unsigned long long)l << ((lz - 32) & 63);
-  if (lz < 64) top |= (unsigned long long)h << lz;
-  const int e = 1023 + 95 - lz + ex;      // biased exponent
-  unsigned long long v = ((unsigned long long)(e - 1) << 52) + (top >> 11) + ((top >> 10) & 1);
-  if (lz == 96 || e < 1) v = 0;
-  if (e > 2046) v = 0x7ff0000000000000ULL;
-  if (ex == INT_MAX) v = 0x7ff8000000000000ULL;
-  return __longlong_as_double((long long)(v | ((unsigned long long)neg << 63)));
-}
-
-struct SepTile {
-  int job, e, mt, nt, R, nk;
-  const unsigned *ma, *mb;   // groups of K with nonzero digits in the tile's rows, in its outputs (or null)
-  __device__ __forceinline__ unsigned mask(int wd) const { return mb ? ma[wd] & mb[wd] : ma[wd]; }
-  __device__ __forceinline__ int groups() const {
-    int n = 0;
-    for (int wd = 0; wd < SEP_MASK; ++wd) n += __popc(mask(wd));
-    return n;
+template <int STAGE>
+struct SepSrc {
+  Batch bt;
+  const SubDesc *subs;
+  const unsigned char *sep;
+  double *ws;
+  int user, fam;
+  struct Tile : DigitTile {
+    Item it;
+    int job, e, mt, nt, R;
+  };
+  __device__ __forceinline__ int total() const { return bt.total_blocks; }
+  __device__ __forceinline__ bool tile(int v, Tile &t) const {
+    int local;
+    locate(bt, v, t.it, local);
+    const Item &it = t.it;
+    if (MDP_CHECKED && !item_in_bounds(bt, subs, it, local, fam, false)) return false;
+    const SubDesc &d = subs[it.sub];
+    const SepGeo g = sep_geo(d);
+    const SepWs w = sep_ws(d, it.ncols);
+    t.job = STAGE == 1 ? J_MID : J_SYN;
+    const int n0 = sep_tiles(d, g, t.job, it.ncols, it.col0, user);
+    if (local >= n0) { ++t.job; local -= n0; }
+    t.R = sep_rows(d, t.job, it.ncols, it.col0, user);
+    const int nk = sep_nk(g, t.job), nt = sep_nt(g, t.job), per = (t.R / 128) * nt;
+    t.e = local / per;
+    t.mt = (local % per) / nt;
+    t.nt = local % nt;
+    const int tr = t.e * (t.R / 128) + t.mt;   // tile row
+    t.A = reinterpret_cast<const unsigned char *>(ws + it.a_off + w.a[t.job]) + (long long)tr * nk * SEP_ABLK;
+    t.ex = reinterpret_cast<const int *>(ws + it.a_off + w.ex[t.job]) + tr * 128;
+    t.ma = reinterpret_cast<const unsigned *>(ws + it.a_off + w.mask) + sep_mask_of(t.job, it.ncols) + tr * SEP_MASK;
+    t.mb = nullptr;
+    t.eb = t.nkj = t.ND = t.ti = 0;
+    if (t.job == J_SYN) {
+      t.B = sep + d.sep_b3 + ((long long)t.e * g.nt3 + t.nt) * nk * SEP_BBLK;
+      t.mb = reinterpret_cast<const unsigned *>(sep + d.sep_z3) + (t.e * g.nt3 + t.nt) * SEP_MASK;
+    } else if (t.job == J_INV) {
+      t.B = sep + d.sep_bi + ((long long)t.e * g.ntg + t.nt) * nk * SEP_BBLK;
+    } else if (t.job == J_FWD) {
+      t.B = sep + d.sep_bf + ((long long)t.e * (g.nqh / 32) + t.nt) * nk * SEP_BBLK;
+    } else if (t.nt < g.nt3) {   // K
+      const int es = t.e * g.nS + t.nt / g.nti;
+      t.B = sep + d.sep_tb + (long long)es * g.nS * g.ND * SEP_BBLK;
+      t.nkj = g.nkj; t.ND = g.ND; t.ti = t.nt % g.nti;
+      t.eb = reinterpret_cast<const int *>(sep + d.sep_kde)[es];
+    } else {                     // moments
+      const int mt = t.e * (3 * g.nqp / 32) + t.nt - g.nt3;
+      t.B = sep + d.sep_mb + (long long)mt * nk * SEP_BBLK;
+      t.mb = reinterpret_cast<const unsigned *>(sep + d.sep_zm) + mt * SEP_MASK;
+    }
+    return true;
+  }
+  __device__ __forceinline__ void dest(const Tile &t, int r, int o, double *&dst, long long &step, int &cnt) const {
+    const Item &it = t.it;
+    const SubDesc &d = subs[it.sub];
+    const SepGeo g = sep_geo(d);
+    const SepWs w = sep_ws(d, it.ncols);
+    const int row = t.mt * 128 + r, o0 = t.nt * 32 + o;
+    const bool direct = t.nkj > 0;
+    step = t.R;
+    if (t.job == J_SYN || direct) {
+      const int i0 = (t.nt % g.nti) * 32 + o;
+      cnt = g.Pi - i0;
+      dst = ws + it.a_off + (direct ? w.u1 : w.u3) + ((long long)(t.e * g.nS + t.nt / g.nti) * g.Pi + i0) * t.R + row;
+    } else if (t.job == J_MID) {
+      cnt = 16;
+      dst = ws + it.a_off + w.mom + ((long long)t.e * 3 * g.nqp + o0 - 32 * g.nt3) * t.R + row;
+    } else if (t.job == J_INV) {
+      cnt = g.Ng - o0;
+      dst = ws + it.a_off + w.ui + ((long long)t.e * g.Ng + o0) * t.R + row;
+    } else {                   // the dense rows' transforms: modes q = 2 (o0 + k) + 1 + e
+      const int cp = sep_pad128(it.ncols), parts = user ? 2 : 1;
+      int col = row % cp;
+      cnt = col < it.ncols && 2 * o0 + 1 + t.e <= d.Nq ? (d.Nq - (1 + t.e) - 2 * o0) / 2 + 1 : 0;
+      if (!user && cnt > 0) col = sep_col_of(d, it.col0, it.ncols, col);
+      step = 2LL * it.ncols * parts;
+      dst = ws + it.gr_off + (((long long)(row / (cp * parts)) * d.Nq + 2 * o0 + t.e) * it.ncols + col) * parts + (row / cp) % parts;
+    }
   }
 };
-template <int STAGE>
-__device__ __forceinline__ SepTile sep_tile(const SubDesc &d, const SepGeo &g, const SepWs &w, const Item &it, int local,
-                                            bool user, const double *ws, const unsigned char *sep) {
-  SepTile t;
-  t.job = STAGE == 1 ? J_MID : J_SYN;
-  const int n0 = sep_tiles(d, g, t.job, it.ncols, it.col0, user);
-  if (local >= n0) { ++t.job; local -= n0; }
-  t.R = sep_rows(d, t.job, it.ncols, it.col0, user);
-  t.nk = sep_nk(g, t.job);
-  const int nt = sep_nt(g, t.job), per = (t.R / 128) * nt;
-  t.e = local / per;
-  t.mt = (local % per) / nt;
-  t.nt = local % nt;
-  t.ma = reinterpret_cast<const unsigned *>(ws + it.a_off + w.mask) + sep_mask_of(t.job, it.ncols) +
-         (t.e * (t.R / 128) + t.mt) * SEP_MASK;
-  t.mb = nullptr;
-  if (t.job == J_SYN) t.mb = reinterpret_cast<const unsigned *>(sep + d.sep_z3) + (t.e * g.nt3 + t.nt) * SEP_MASK;
-  if (t.job == J_MID && t.nt >= g.nt3)
-    t.mb = reinterpret_cast<const unsigned *>(sep + d.sep_zm) + (t.e * (3 * g.nqp / 32) + t.nt - g.nt3) * SEP_MASK;
-  return t;
-}
 
 template <int STAGE>
 __global__ void __launch_bounds__(SG_THREADS, 1)
     k_sep_gemm(Batch bt, const SubDesc *subs, const unsigned char *sep, double *ws, int user, int fam, int *status) {
-  extern __shared__ unsigned char sg_raw[];
-  __shared__ __align__(8) unsigned long long full_bar[SG_STAGES], empty_bar[SG_STAGES], tfull_bar[2], tempty_bar[2], drain_bar;
-  __shared__ unsigned tmem_slot;
-  __shared__ volatile int abort_sh;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  if (tid == 0) {
-    for (int s = 0; s < SG_STAGES; ++s) { mbar_init(smem_u32(&full_bar[s]), 1); mbar_init(smem_u32(&empty_bar[s]), 1); }
-    for (int s = 0; s < 2; ++s) { mbar_init(smem_u32(&tfull_bar[s]), 1); mbar_init(smem_u32(&tempty_bar[s]), 256); }
-    mbar_init(smem_u32(&drain_bar), 1);
-    abort_sh = 0;
-  }
-  if (warp == 8) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)), "r"(512)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-  }
-  const unsigned sbase = (smem_u32(sg_raw) + 1023u) & ~1023u;
-  {
-    unsigned char *z = sg_raw + (sbase - smem_u32(sg_raw)) + SG_B0;
-    for (int i = tid; i < (SG_STAGES + 1) * (SEP_BBLK / 16); i += SG_THREADS)
-      *reinterpret_cast<uint4 *>(z + (i / (SEP_BBLK / 16)) * 2 * SEP_BBLK + (i % (SEP_BBLK / 16)) * 16) = make_uint4(0, 0, 0, 0);
-  }
-  asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const unsigned tmem = tmem_slot;
-
-  if (warp == 9) {
-    // ---------------------------------------------------------------- operand loads
-    if (lane == 0) {
-      unsigned gs = 0;
-      for (int v = blockIdx.x; v < bt.total_blocks && !abort_sh; v += gridDim.x) {
-        Item it; int local;
-        locate(bt, v, it, local);
-        if (MDP_CHECKED && !item_in_bounds(bt, subs, it, local, fam, false)) continue;   // every warp skips it
-        const SubDesc &d = subs[it.sub];
-        const SepGeo g = sep_geo(d);
-        const SepWs w = sep_ws(d, it.ncols);
-        const SepTile t = sep_tile<STAGE>(d, g, w, it, local, user, ws, sep);
-        const unsigned char *A = reinterpret_cast<const unsigned char *>(ws + it.a_off + w.a[t.job]) +
-                                 (long long)(t.e * (t.R / 128) + t.mt) * t.nk * SEP_ABLK;
-        const unsigned char *B;
-        int ti = 0;
-        const bool toep = t.job == J_MID && t.nt < g.nt3;
-        if (t.job == J_SYN) B = sep + d.sep_b3 + ((long long)t.e * g.nt3 + t.nt) * t.nk * SEP_BBLK;
-        else if (t.job == J_INV) B = sep + d.sep_bi + ((long long)t.e * g.ntg + t.nt) * t.nk * SEP_BBLK;
-        else if (t.job == J_FWD) B = sep + d.sep_bf + ((long long)t.e * (g.nqh / 32) + t.nt) * t.nk * SEP_BBLK;
-        else if (toep) { ti = t.nt % g.nti; B = sep + d.sep_tb + ((long long)(t.e * g.nS + t.nt / g.nti) * g.nS) * g.ND * SEP_BBLK; }
-        else B = sep + d.sep_mb + ((long long)t.e * (3 * g.nqp / 32) + t.nt - g.nt3) * t.nk * SEP_BBLK;
-        bool ok = true;
-        for (int wd = 0; wd < SEP_MASK && ok; ++wd)
-          for (unsigned bits = t.mask(wd); bits; bits &= bits - 1, ++gs) {
-            const int kb = 32 * wd + __ffs(bits) - 1;
-            const unsigned st = gs % SG_STAGES;
-            if (gs >= SG_STAGES && !mbar_wait(smem_u32(&empty_bar[st]), (gs / SG_STAGES - 1) & 1u, &abort_sh)) { ok = false; break; }
-            const unsigned bar = smem_u32(&full_bar[st]);
-            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(SG_STAGE_BYTES) : "memory");
-            bulk_load(sbase + st * SEP_ABLK, A + (long long)kb * SEP_ABLK, SEP_ABLK, bar);
-            const long long bo = toep ? (long long)(kb / g.nkj) * g.ND + 2 * ti - kb % g.nkj + g.nkj - 1 : kb;
-            bulk_load(sbase + SG_B0 + (2 * st + 1) * SEP_BBLK, B + bo * SEP_BBLK, SEP_BBLK, bar);
-          }
-        if (!ok) break;
-      }
-      // leave only when every copy issued has landed (each wait bounded)
-      for (unsigned s = gs >= SG_STAGES ? gs - SG_STAGES : 0; s < gs; ++s) {
-        const long long t0 = clock64();
-        while (!mbar_try(smem_u32(&full_bar[s % SG_STAGES]), (s / SG_STAGES) & 1u))
-          if (clock64() - t0 > TC_WAIT_CYCLES) { abort_sh = 1; break; }
-      }
-    }
-    __syncwarp();
-  } else if (warp == 8) {
-    // ---------------------------------------------------------------- MMAs
-    if (lane == 0) {
-      unsigned gs = 0, cc = 0;   // stages and accumulator sets used
-      for (int v = blockIdx.x; v < bt.total_blocks && !abort_sh; v += gridDim.x) {
-        Item it; int local;
-        locate(bt, v, it, local);
-        if (MDP_CHECKED && !item_in_bounds(bt, subs, it, local, fam, false)) continue;
-        const SubDesc &d = subs[it.sub];
-        const SepGeo g = sep_geo(d);
-        const SepTile t = sep_tile<STAGE>(d, g, sep_ws(d, it.ncols), it, local, user, ws, sep);
-        const int n = t.groups();   // steps
-        bool ok = true;
-        for (int s = 0; s < n && ok; ++cc) {
-          const unsigned buf = cc & 1u, D = tmem + 256u * buf;
-          if (cc >= 2 && !mbar_wait(smem_u32(&tempty_bar[buf]), ((cc >> 1) - 1) & 1u, &abort_sh)) { ok = false; break; }
-          tc_fence_after();
-          const int send = min(n, s + SG_CHUNK);
-          for (bool first = true; s < send; ++s, ++gs, first = false) {
-            const unsigned st = gs % SG_STAGES;
-            if (!mbar_wait(smem_u32(&full_bar[st]), (gs / SG_STAGES) & 1u, &abort_sh)) { ok = false; break; }
-            tc_fence_after();
-            const unsigned a0 = sbase + st * SEP_ABLK, b0 = sbase + SG_B0 + (2 * st + 1) * SEP_BBLK;
-#pragma unroll
-            for (int dg = 0; dg < 7; ++dg)
-              tc_mma(D, smem_desc(a0 + 4096 * dg, 128, 256), smem_desc(b0 - 1024 * dg, 128, 256), f16_idesc(256),
-                     first && dg == 0 ? 0u : 1u);
-            tc_commit(smem_u32(&empty_bar[st]));
-          }
-          if (ok) tc_commit(smem_u32(&tfull_bar[buf]));
-        }
-        if (!ok) break;
-      }
-      if (abort_sh) {   // no MMA in flight when the tensor memory is freed (bounded)
-        tc_commit(smem_u32(&drain_bar));
-        const long long t0 = clock64();
-        while (!mbar_try(smem_u32(&drain_bar), 0u) && clock64() - t0 < TC_WAIT_CYCLES) {}
-      }
-    }
-    __syncwarp();
-  } else {
-    // ---------------------------------------------------------------- sums and results
-    const int quarter = warp & 3, half = warp >> 2;
-    unsigned cc = 0;
-    for (int v = blockIdx.x; v < bt.total_blocks && !abort_sh; v += gridDim.x) {
-      Item it; int local;
-      locate(bt, v, it, local);
-      if (MDP_CHECKED && !item_in_bounds(bt, subs, it, local, fam, false)) continue;
-      const SubDesc &d = subs[it.sub];
-      const SepGeo g = sep_geo(d);
-      const SepWs w = sep_ws(d, it.ncols);
-      const SepTile t = sep_tile<STAGE>(d, g, w, it, local, user, ws, sep);
-      const int n = t.groups();
-      // weights 0..3 and 4..7 of 16 outputs, as sums of I_w 2^(8 (3 - w)), I_w 2^(8 (7 - w))
-      long long hi[16], lo[16];
-#pragma unroll
-      for (int o = 0; o < 16; ++o) hi[o] = lo[o] = 0;
-      bool ok = true;
-      for (int s = 0; s < n; s += SG_CHUNK, ++cc) {
-        const unsigned buf = cc & 1u;
-        if (!mbar_wait(smem_u32(&tfull_bar[buf]), (cc >> 1) & 1u, &abort_sh)) { ok = false; break; }
-        tc_fence_after();
-        const unsigned src = tmem + ((unsigned)(32 * quarter) << 16) + 256u * buf + 16u * half;
-#pragma unroll
-        for (int wt = 0; wt < 8; ++wt) {
-          float dv[16];
-          tmem_ld16(src + 32u * wt, dv);
-#pragma unroll
-          for (int o = 0; o < 16; ++o) {
-            const long long iv = (long long)__float2int_rn(dv[o]);
-            if (wt < 4) hi[o] += iv * (1LL << (8 * (3 - wt)));
-            else lo[o] += iv * (1LL << (8 * (7 - wt)));
-          }
-        }
-        tc_fence_before();
-        mbar_arrive(smem_u32(&tempty_bar[buf]));
-      }
-      if (!ok) break;
-      // value = (hi 2^32 + lo) 2^40 2^(E - 1022 - 54) 2^(eb - 54)
-      const int row = t.mt * 128 + 32 * quarter + lane;
-      const int E = reinterpret_cast<const int *>(ws + it.a_off + w.ex[t.job])[t.e * t.R + row];
-      const bool direct = t.job == J_MID && t.nt < g.nt3;
-      int eb = 0;
-      if (direct) eb = reinterpret_cast<const int *>(sep + d.sep_kde)[t.e * g.nS + t.nt / g.nti];
-      const int ex = E < 2047 ? E - 1090 + eb : INT_MAX;   // Inf or NaN in the row: NaN
-      double *dst;
-      int cnt;                   // outputs of this thread, `step` doubles apart
-      long long step = t.R;
-      const int o0 = t.nt * 32 + 16 * half;
-      if (t.job == J_SYN || direct) {
-        const int i0 = (t.nt % g.nti) * 32 + 16 * half;
-        cnt = g.Pi - i0;
-        dst = ws + it.a_off + (direct ? w.u1 : w.u3) + ((long long)(t.e * g.nS + t.nt / g.nti) * g.Pi + i0) * t.R + row;
-      } else if (t.job == J_MID) {
-        cnt = 16;
-        dst = ws + it.a_off + w.mom + ((long long)t.e * 3 * g.nqp + o0 - 32 * g.nt3) * t.R + row;
-      } else if (t.job == J_INV) {
-        cnt = g.Ng - o0;
-        dst = ws + it.a_off + w.ui + ((long long)t.e * g.Ng + o0) * t.R + row;
-      } else {                   // the dense rows' transforms: modes q = 2 (o0 + o) + 1 + e
-        const int cp = sep_pad128(it.ncols), parts = user ? 2 : 1;
-        int col = row % cp;
-        cnt = col < it.ncols ? (d.Nq - (1 + t.e) - 2 * o0) / 2 + 1 : 0;
-        if (!user && cnt > 0) col = sep_col_of(d, it.col0, it.ncols, col);
-        if (2 * o0 + (1 + t.e) > d.Nq) cnt = 0;
-        step = 2LL * it.ncols * parts;
-        dst = ws + it.gr_off + (((long long)(row / (cp * parts)) * d.Nq + 2 * o0 + t.e) * it.ncols + col) * parts + (row / cp) % parts;
-      }
-#pragma unroll
-      for (int o = 0; o < 16; ++o)
-        if (o < cnt) dst[o * step] = sum_to_double(hi[o], lo[o], ex);
-    }
-  }
-  if (abort_sh && tid == 0) atomicCAS(status, 0, (int)MDP_ERR_TIMEOUT);   // the first error sticks
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  if (warp == 8)
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+  const SepSrc<STAGE> src{bt, subs, sep, ws, user, fam};
+  digit_gemm(src, status);
 }
 
 // ---------------------------------------------------------------- stage 2
@@ -1065,6 +782,7 @@ cudaError_t launch_sep_tables(const mdp_plan *p, const SubDesc *ds, const double
   for (int s0 = 0; s0 < ns; s0 += 65535) {   // subdomains per launch: a grid's y / z limit
     const unsigned n = (unsigned)std::min(65535, ns - s0);
     k_sep_mode_tab<<<dim3(mq, n), 128, 0, st>>>(ds, s0, sep, entries);
+    k_full_modes<<<dim3(mq, n), 128, 0, st>>>(ds, s0, sep);
     k_sep_phi<<<dim3(mq, mrow, n), 128, 0, st>>>(ds, s0, sep);
     if (mdist == 0) continue;   // no subdomain on the tensor cores
     k_sep_kd<<<dim3(mdist, n), 128, 0, st>>>(ds, s0, tab, sep);
@@ -1076,21 +794,22 @@ cudaError_t launch_sep_tables(const mdp_plan *p, const SubDesc *ds, const double
 }
 
 cudaError_t launch_sep_sines(const mdp_plan *p, const SubDesc *ds, const double *tab, unsigned char *sep, cudaStream_t st) {
-  int k[2] = {0, 0}, t[2] = {0, 0};
+  int k[4] = {0, 0, 0, 0}, t[4] = {0, 0, 0, 0};
   for (size_t i = 0; i < p->subs.size(); ++i) {
     const SubDesc &d = p->subs[i].d;
     if (!d.tc_cols || d.leader != (int)i) continue;
     const SepGeo g = sep_geo(d);
-    for (int inv = 0; inv < 2; ++inv) {
-      k[inv] = std::max(k[inv], ((inv ? g.nqh / 16 : g.nkf) + 3) / 4);
-      t[inv] = std::max(t[inv], 2 * (inv ? g.ntg : g.nqh / 32));
+    const int nk[4] = {g.nkf, g.nqh / 16, g.nkx, g.nqh / 16}, nt[4] = {g.nqh / 32, g.ntg, g.nqh / 32, g.ntx};
+    for (int w = 0; w < 4; ++w) {
+      k[w] = std::max(k[w], (nk[w] + 3) / 4);
+      t[w] = std::max(t[w], 2 * nt[w]);
     }
   }
   const int ns = (int)p->subs.size();
   if (t[0] == 0) return cudaSuccess;
   for (int s0 = 0; s0 < ns; s0 += 65535)
-    for (int inv = 0; inv < 2; ++inv)
-      k_sep_sines<<<dim3(k[inv], t[inv], (unsigned)std::min(65535, ns - s0)), 256, 0, st>>>(ds, s0, tab, sep, inv);
+    for (int w = 0; w < 4; ++w)
+      k_sep_sines<<<dim3(k[w], t[w], (unsigned)std::min(65535, ns - s0)), 256, 0, st>>>(ds, s0, tab, sep, w);
   return cudaGetLastError();
 }
 

@@ -69,6 +69,8 @@ struct SubDesc {
   long long sep_kde;    // ints [class][output]: exponent of the largest |K|
   long long sep_tb, sep_mb, sep_b3;   // digit blocks of K (Toeplitz), of the moments, of the synthesis
   long long sep_bf, sep_bi;           // of the dense rows' transform and of the gamma rows' (sines only)
+  long long sep_xf, sep_xi;           // of the full-grid transforms
+  long long sep_mx;     // per mode SEP_MXW doubles: the full-grid solve along y (kernels_full.cu)
   long long out_off;    // complex elements: start of the subdomain's output block
   long long rec_off;    // complex elements: start of the receiver block [n_cols][Px - 2]
   int *dstatus;         // the plan's device status word (bounds-checked build: first error; else unused)
@@ -114,6 +116,7 @@ constexpr int FSW = 24;  // doubles per forward-sweep table row
 
 // ---- separable projection (kernels_sep.cu)
 constexpr int SEP_MTW = 72;               // doubles per mode of the mode table
+constexpr int SEP_MXW = 16;               // doubles per mode of the full-grid solve's table
 constexpr int SEP_ABLK = 7 * 128 * 16 * 2;  // bytes of A: 7 digits x 128 rows x 16 values of K, fp16
 constexpr int SEP_BBLK = 7 * 32 * 16 * 2;   // bytes of B: 7 digits x 32 outputs x 16 values of K
 constexpr int SEP_MODES_PER_BLOCK = 16;   // k_sep_modes
@@ -137,6 +140,7 @@ struct SepGeo {
   int mf, Kf, nkf;     // FWD: folded columns m = mf .. Nx/2 of the dense ring rows (m with Nx - m), groups of 16
   int mg, Ng, ntg;     // INV: folded columns m = mg .. Nx/2 of the gamma rows, groups of 32
   int slots;           // INV: rows transformed back: 4 gamma rows (+ the receiver row)
+  int nkx, ntx;        // full-grid transforms: folded columns m = 1 .. Nx/2 in groups of 16, of 32
   int nk1, nk3;        // K of MID (source column, row) and SYN (b, mode) in units of 16
   int nt1, nt3;        // MID, SYN: tiles of 32 outputs
   int ND;              // distinct Toeplitz blocks per (output, source) column
@@ -158,6 +162,8 @@ inline __host__ __device__ SepGeo sep_geo(const SubDesc &d) {
   g.mg = g.mf - 1;
   g.Ng = g.Kf + 1;
   g.ntg = (g.Ng + 31) / 32;
+  g.nkx = (d.Nx / 2 + 15) / 16;
+  g.ntx = (d.Nx / 2 + 31) / 32;
   g.slots = d.nrec >= 0 ? 5 : 4;
   g.nk1 = g.nS * g.nkj;
   g.nk3 = 2 * g.nqp / 16;
@@ -260,6 +266,33 @@ inline __host__ __device__ SepWs sep_ws(const SubDesc &d, int ncols) {
   w.mom = take(g.ncls * 3LL * g.nqp * R);
   w.aeff = take(g.ncls * 2LL * g.nqp * R);
   w.ui = take(2LL * g.Ng * 5 * R);
+  w.total = off;
+  return w;
+}
+// Workspace of a full-grid solve of nr right-hand sides, in doubles (kernels_full.cu).
+struct FullWs {
+  int rows, R;            // rows of A: (right-hand side, unknown row, part), padded to 128
+  int ldf, ldu;           // row lengths of f and u
+  long long a, ex, mask;  // digit blocks, exponents (ints) [parity][R], masks (words) [parity][R / 128][SEP_MASK]
+  long long f;            // mode space [rows][parity][nqh]
+  long long u;            // sums over one parity [parity][R][folded columns]
+  long long total;
+};
+inline __host__ __device__ FullWs full_ws(const SubDesc &d, int nr) {
+  const SepGeo g = sep_geo(d);
+  FullWs w;
+  w.rows = 2 * nr * d.Nt;
+  w.R = sep_pad128(w.rows);
+  w.ldf = 2 * g.nqh;
+  w.ldu = 32 * g.ntx;
+  const long long nk = g.nkx > g.nqh / 16 ? g.nkx : g.nqh / 16;
+  long long off = 0;
+  auto take = [&](long long n) { const long long o = off; off += (n + 31) & ~31LL; return o; };
+  w.a = take(2LL * (w.R / 128) * nk * (SEP_ABLK / 8));
+  w.ex = take(w.R);
+  w.mask = take(2LL * (w.R / 128) * SEP_MASK);   // two masks: of the forward and of the inverse transform
+  w.f = take((long long)w.R * w.ldf);
+  w.u = take(2LL * w.R * w.ldu);
   w.total = off;
   return w;
 }
@@ -540,6 +573,10 @@ cudaError_t launch_potential(const mdp_plan *p, int sub, int ncols, const double
 cudaError_t launch_source_terms(mdp_plan *p, int sub, const double2 *f, const double2 *src4, double2 *F, double2 *u,
                                 cudaStream_t st);
 cudaError_t launch_basis_densities(const mdp_plan *p, int sub, int col0, int ncols, double2 *out, cudaStream_t st);
+// the full-grid solve through the separable Green's function (subdomains with tc_cols; kernels_full.cu)
+cudaError_t launch_full_solve(const mdp_plan *p, int sub, int nrhs, const double2 *g, double2 *u, cudaStream_t st);
+cudaError_t set_full_kernel_attributes();
+__global__ void k_full_modes(const SubDesc *subs, int s0, unsigned char *sep);
 cudaError_t launch_solve(const mdp_plan *p, int sub, int nrhs, const double2 *g, double2 *u, int adjoint,
                          cudaStream_t st);
 cudaError_t launch_solve_raw(const SubDesc *d_sub, const SubDesc &hd, const double *tab, const uint8_t *piv,

@@ -418,12 +418,13 @@ static bool layout_tables(mdp_plan *p) {
       d.fact_off = ld.fact_off; d.dT_off = ld.dT_off; d.sin_off = ld.sin_off; d.geo_off = ld.geo_off;
       d.seg_off = ld.seg_off; d.fs_off = ld.fs_off; d.piv_off = ld.piv_off; d.tcb_off = ld.tcb_off;
       d.sep_zm = ld.sep_zm; d.sep_z3 = ld.sep_z3; d.sep_ab = ld.sep_ab; d.sep_mt = ld.sep_mt; d.sep_phi = ld.sep_phi; d.sep_kd = ld.sep_kd; d.sep_kde = ld.sep_kde;
-      d.sep_tb = ld.sep_tb; d.sep_mb = ld.sep_mb; d.sep_b3 = ld.sep_b3; d.sep_bf = ld.sep_bf; d.sep_bi = ld.sep_bi;
+      d.sep_tb = ld.sep_tb; d.sep_mb = ld.sep_mb; d.sep_b3 = ld.sep_b3; d.sep_bf = ld.sep_bf; d.sep_bi = ld.sep_bi; d.sep_xf = ld.sep_xf; d.sep_xi = ld.sep_xi; d.sep_mx = ld.sep_mx;
       d.out_off = out;  out += (long long)d.G * d.n_cols;
       continue;
     }
     d.sep_ab = take(16LL * d.Nq);
     d.sep_mt = take(8LL * SEP_MTW * d.Nq);
+    d.sep_mx = take(8LL * SEP_MXW * d.Nq);
     d.sep_phi = take(16LL * (d.Py + 2) * d.Nq);
     if (d.tc_cols) {
       const SepGeo g = sep_geo(d);
@@ -435,6 +436,8 @@ static bool layout_tables(mdp_plan *p) {
       d.sep_b3 = take((long long)g.ncls * g.nt3 * g.nk3 * SEP_BBLK);
       d.sep_bf = take(2LL * (g.nqh / 32) * g.nkf * SEP_BBLK);
       d.sep_bi = take(2LL * g.ntg * (g.nqh / 16) * SEP_BBLK);
+      d.sep_xf = take(2LL * (g.nqh / 32) * g.nkx * SEP_BBLK);
+      d.sep_xi = take(2LL * g.ntx * (g.nqh / 16) * SEP_BBLK);
     }
     const int FW = d.cplx ? 8 : 4;
     d.fact_off = off; off += al((long long)d.Nq * d.Nt * FW);
@@ -571,7 +574,7 @@ static void schedule(mdp_plan *p) {
     const SubDesc &d = hs.d;
     long long xi, r, gr, y, a, s, red, tot;
     item_workspace(d, 1, false, xi, r, gr, y, a, s, red, tot);
-    mx = std::max(mx, std::max((long long)d.Nq * d.Nt * 2, tot) + 2LL * d.G + 2LL * d.nx * d.ny + 128);
+    mx = std::max(mx, std::max({(long long)d.Nq * d.Nt * 2, tot, d.tc_cols ? full_ws(d, 1).total : 0}) + 2LL * d.G + 2LL * d.nx * d.ny + 128);
   }
   p->ws_doubles = mx;
 }

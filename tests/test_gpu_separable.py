@@ -81,3 +81,30 @@ def test_every_receiver_row(mdp, off):
         ref = pot[:, row, m0:m0 + cnt]
         assert rel_col_err(rec[:nc * cnt].cpu().numpy().reshape(nc, cnt), ref) < TOL, row
     assert rel_col_err(out.cpu().numpy().reshape(nc, G), S.columns()) < TOL
+
+
+@pytest.mark.parametrize("name,sub", CASES, ids=[c[0] for c in CASES])
+def test_full_grid_solves_match_the_oracle(mdp, name, sub):
+    """Whole-grid solves: data on every node, on the rows next to the ends, and none at all."""
+    plan = mdp.Plan([sub])
+    g = W.random_complex((3, sub.ny, sub.nx), seed=9)
+    g[1, 3:-3] = 0
+    g[2] = 0
+    got = plan.solve(0, torch.from_numpy(g).cuda()).cpu().numpy()
+    plan.status()
+    S = APSystem(sub)
+    ref = np.stack([S.solve(x) for x in g[:2]])
+    assert rel_col_err(got[:2].reshape(2, -1), ref.reshape(2, -1)) < TOL
+    assert not got[2].any()
+
+
+def test_full_grid_solves_in_passes(mdp):
+    """More right-hand sides than the workspace takes at once: bit for bit those of single calls, also in
+    place."""
+    sub = W.small_subdomain(65, 9.0, W.AP_DIRX_SOMMY, 2)
+    plan = mdp.Plan([sub], workspace_bytes=1 << 20)
+    g = torch.from_numpy(W.random_complex((40, 65, 65), seed=10)).cuda()
+    one = torch.cat([plan.solve(0, g[i:i + 1]) for i in range(40)])
+    assert torch.equal(plan.solve(0, g), one)
+    plan.solve(0, g, out=g)
+    assert torch.equal(g, one)
