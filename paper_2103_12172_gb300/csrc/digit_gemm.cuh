@@ -35,6 +35,9 @@ __device__ __forceinline__ void store_digits(unsigned char *dst, long long strid
   MDP_SEP_DIGIT(0) MDP_SEP_DIGIT(1) MDP_SEP_DIGIT(2) MDP_SEP_DIGIT(3) MDP_SEP_DIGIT(4) MDP_SEP_DIGIT(5) MDP_SEP_DIGIT(6)
 #undef MDP_SEP_DIGIT
 }
+// 2/Nx = inv_scale 2^inv_exp, inv_scale in (1/2, 1]: the normalisation of the inverse transforms, in their tables
+__device__ __forceinline__ int inv_exp(const SubDesc &d) { return __clz(d.Nx) - 30; }
+__device__ __forceinline__ double inv_scale(const SubDesc &d) { return (double)(1 << (31 - __clz(d.Nx))) / d.Nx; }
 // table value |x| <= 1 on the fixed scale 2^54
 __device__ __forceinline__ long long fix54(double x) { return __double2ll_rn(x * 0x1p54); }
 
@@ -68,31 +71,33 @@ struct DigitTile {
   }
 };
 
-// Persistent CTAs, one per SM: warp 9 streams the digit blocks of A (28 KiB) and B (7 KiB) of 16
-// values of K into 5 shared-memory stages with bulk copies, one thread of warp 8 issues the MMAs,
+// Persistent CTAs, one per SM: warp 17 streams the digit blocks of A (28 KiB) and B (7 KiB) of 16
+// values of K into 5 shared-memory stages with bulk copies, one thread of warp 16 issues the MMAs,
 // and after every 128 values of K hands one of two accumulator sets (8 weights x 32 outputs, FP32)
-// to the 8 other warps, which add them up as integers and at the end of a tile scale them into
-// FP64. A tile is 128 rows x 32 outputs. One MMA (M = 128, N = 256, K = 16) per A digit t: its B
+// to the 16 other warps (a quarter of the rows and 8 outputs each; 8 warps left their latencies in the
+// open), which add them up as integers and at the end of a tile scale them into FP64. A tile is 128 rows x 32 outputs. One MMA (M = 128, N = 256, K = 16) per A digit t: its B
 // operand starts t digits before B's first one, in 7 KiB of zeros, so that digit u meets the
 // accumulator of weight t + u and every MMA of a set has the same accumulator and shape (MMAs into
 // overlapping accumulators of other shapes have no defined order). The zeros are 22 of 56 digit
 // pairs. What bounds it: the tensor pipe, 7 x 128 cycles per 16 values of K; the operands' way from
 // L2 takes 35 KiB in that time, 39 bytes per cycle and SM.
-constexpr int SG_STAGES = 5, SG_THREADS = 320, SG_CHUNK = 8;   // K16 steps per accumulator set
+constexpr int SG_STAGES = 5, SG_EPI = 16, SG_THREADS = 32 * (SG_EPI + 2), SG_CHUNK = 8;   // K16 steps per accumulator set
 constexpr int SG_STAGE_BYTES = SEP_ABLK + SEP_BBLK;
 // shared memory: the A stages, then zeros and B stages in turn, 7 KiB each, and closing zeros
 constexpr int SG_B0 = SG_STAGES * SEP_ABLK;
 constexpr int SG_SMEM = SG_B0 + (2 * SG_STAGES + 1) * SEP_BBLK + 1024;
 
-// 16 consecutive FP32 columns of this warp's 32 TMEM lanes
-__device__ __forceinline__ void tmem_ld16(unsigned taddr, float *v) {
+// 8 consecutive FP32 columns of this warp's 32 TMEM lanes, twice (two weights in flight)
+__device__ __forceinline__ void tmem_ld8x2(unsigned ta, unsigned tb, float *v) {
   unsigned r[16];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr)
-      : "memory");
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(ta)
+               : "memory");
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+               : "r"(tb)
+               : "memory");
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
@@ -123,7 +128,7 @@ __device__ __forceinline__ double sum_to_double(long long hi, long long lo, int 
 }
 
 // Src: total() tiles, tile(v, t) fills tile v (false: skipped by every warp), dest(t, row, o, ...) says where
-// the 16 outputs from o on of a row go. One CTA of SG_THREADS threads per SM with SG_SMEM bytes.
+// the 8 outputs from o on of a row go. One CTA of SG_THREADS threads per SM with SG_SMEM bytes.
 template <class Src>
 __device__ __forceinline__ void digit_gemm(const Src &src, int *status) {
   extern __shared__ unsigned char sg_raw[];
@@ -134,11 +139,11 @@ __device__ __forceinline__ void digit_gemm(const Src &src, int *status) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid == 0) {
     for (int s = 0; s < SG_STAGES; ++s) { mbar_init(smem_u32(&full_bar[s]), 1); mbar_init(smem_u32(&empty_bar[s]), 1); }
-    for (int s = 0; s < 2; ++s) { mbar_init(smem_u32(&tfull_bar[s]), 1); mbar_init(smem_u32(&tempty_bar[s]), 256); }
+    for (int s = 0; s < 2; ++s) { mbar_init(smem_u32(&tfull_bar[s]), 1); mbar_init(smem_u32(&tempty_bar[s]), 32 * SG_EPI); }
     mbar_init(smem_u32(&drain_bar), 1);
     abort_sh = 0;
   }
-  if (warp == 8) {
+  if (warp == SG_EPI) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)), "r"(512)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -156,7 +161,7 @@ __device__ __forceinline__ void digit_gemm(const Src &src, int *status) {
   tc_fence_after();
   const unsigned tmem = tmem_slot;
 
-  if (warp == 9) {
+  if (warp == SG_EPI + 1) {
     // ---------------------------------------------------------------- operand loads
     if (lane == 0) {
       unsigned gs = 0;
@@ -185,7 +190,7 @@ __device__ __forceinline__ void digit_gemm(const Src &src, int *status) {
       }
     }
     __syncwarp();
-  } else if (warp == 8) {
+  } else if (warp == SG_EPI) {
     // ---------------------------------------------------------------- MMAs
     if (lane == 0) {
       unsigned gs = 0, cc = 0;   // stages and accumulator sets used
@@ -223,31 +228,30 @@ __device__ __forceinline__ void digit_gemm(const Src &src, int *status) {
     __syncwarp();
   } else {
     // ---------------------------------------------------------------- sums and results
-    const int quarter = warp & 3, half = warp >> 2;
+    const int quarter = warp & 3, part = warp >> 2;   // TMEM lanes of the warp, its outputs
     unsigned cc = 0;
     for (int v = blockIdx.x; v < total && !abort_sh; v += gridDim.x) {
       typename Src::Tile t;
       if (!src.tile(v, t)) continue;
       const int n = t.groups();
-      // weights 0..3 and 4..7 of 16 outputs, as sums of I_w 2^(8 (3 - w)), I_w 2^(8 (7 - w))
-      long long hi[16], lo[16];
+      // weights 0..3 and 4..7 of 8 outputs, as sums of I_w 2^(8 (3 - w)), I_w 2^(8 (7 - w))
+      long long hi[8], lo[8];
 #pragma unroll
-      for (int o = 0; o < 16; ++o) hi[o] = lo[o] = 0;
+      for (int o = 0; o < 8; ++o) hi[o] = lo[o] = 0;
       bool ok = true;
       for (int s = 0; s < n; s += SG_CHUNK, ++cc) {
         const unsigned buf = cc & 1u;
         if (!mbar_wait(smem_u32(&tfull_bar[buf]), (cc >> 1) & 1u, &abort_sh)) { ok = false; break; }
         tc_fence_after();
-        const unsigned acc = tmem + ((unsigned)(32 * quarter) << 16) + 256u * buf + 16u * half;
+        const unsigned acc = tmem + ((unsigned)(32 * quarter) << 16) + 256u * buf + 8u * part;
 #pragma unroll
-        for (int wt = 0; wt < 8; ++wt) {
+        for (int wt = 0; wt < 4; ++wt) {
           float dv[16];
-          tmem_ld16(acc + 32u * wt, dv);
+          tmem_ld8x2(acc + 32u * wt, acc + 32u * (wt + 4), dv);
 #pragma unroll
-          for (int o = 0; o < 16; ++o) {
-            const long long iv = (long long)__float2int_rn(dv[o]);
-            if (wt < 4) hi[o] += iv * (1LL << (8 * (3 - wt)));
-            else lo[o] += iv * (1LL << (8 * (7 - wt)));
+          for (int o = 0; o < 8; ++o) {
+            hi[o] += (long long)__float2int_rn(dv[o]) * (1LL << (8 * (3 - wt)));
+            lo[o] += (long long)__float2int_rn(dv[8 + o]) * (1LL << (8 * (3 - wt)));
           }
         }
         tc_fence_before();
@@ -259,17 +263,17 @@ __device__ __forceinline__ void digit_gemm(const Src &src, int *status) {
       const int E = t.ex[row];
       const int ex = E < 2047 ? E - 1090 + t.eb : INT_MAX;   // Inf or NaN in the row: NaN
       double *dst;
-      int cnt;                   // outputs of this thread, `step` doubles apart
+      int cnt;                   // outputs of this thread (of 8), `step` doubles apart
       long long step;
-      src.dest(t, row, 16 * half, dst, step, cnt);
-      if (step == 1 && cnt >= 16) {
+      src.dest(t, row, 8 * part, dst, step, cnt);
+      if (step == 1 && cnt >= 8) {
 #pragma unroll
-        for (int o = 0; o < 16; o += 2)
+        for (int o = 0; o < 8; o += 2)
           *reinterpret_cast<double2 *>(dst + o) =
               make_double2(sum_to_double(hi[o], lo[o], ex), sum_to_double(hi[o + 1], lo[o + 1], ex));
       } else {
 #pragma unroll
-        for (int o = 0; o < 16; ++o)
+        for (int o = 0; o < 8; ++o)
           if (o < cnt) dst[o * step] = sum_to_double(hi[o], lo[o], ex);
       }
     }
@@ -278,7 +282,7 @@ __device__ __forceinline__ void digit_gemm(const Src &src, int *status) {
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if (warp == 8)
+  if (warp == SG_EPI)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
 }
 

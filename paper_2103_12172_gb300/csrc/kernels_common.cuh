@@ -112,8 +112,9 @@ enum {
   MT_N1 = 68,
   MT_N2 = 69,
   MT_F = 70,     // 1 / (2 a n1 n2): kappa(i - j) = F (phi_2(i) phi_1(j) - phi_1(i) phi_2(j)), i >= j (kinds 0, 1)
+  MT_FAR = 71,   // 1: the two ends' coupling is below 2^-90
 };
-static_assert(MT_F < SEP_MTW, "mode table width");
+static_assert(MT_FAR < SEP_MTW, "mode table width");
 
 // gamma index of node (n, m), or -1 (row-major order of the 2-node ring around M+)
 __device__ __forceinline__ int gamma_index(const SubDesc &d, int n, int m) {

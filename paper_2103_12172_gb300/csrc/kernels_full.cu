@@ -11,17 +11,22 @@
 
 #include <algorithm>
 
+#include <cooperative_groups.h>
+
+namespace cg = cooperative_groups;
+
 namespace mdp {
 
-// per mode: kind, theta, lambda (with its sign), kappa(0) = c, c (1 - lambda^2), sign, R11, R12, R22, F
-enum { MX_KIND = 0, MX_TH, MX_LAM, MX_C, MX_C1, MX_SG, MX_R = 6, MX_F = 12 };
+// per mode: kind, lambda (with its sign), kappa(0) = c, c (1 - lambda^2), sign, R11, R12, R22, F, and of the
+// rotation of kinds 0, 1: -+s^2 (s = sin or sinh theta), C(1), C and S at row 0
+enum { MX_KIND = 0, MX_LAM, MX_C, MX_C1, MX_SG, MX_R = 6, MX_F = 12, MX_SS, MX_CS1, MX_CS0 };   // CS0: 2
 
 // The table of the solve along y, over all rows 0 .. N: evanescent modes phi = (lambda^n, lambda^(N-n)),
 // the others C and S about the middle row.
 __global__ void k_full_modes(const SubDesc *subs, int s0, unsigned char *sep) {
   const int si = s0 + blockIdx.y;
   const SubDesc &d = subs[si];
-  const int q = blockIdx.x * 128 + threadIdx.x + 1;
+  const int q = blockIdx.x * 32 + threadIdx.x + 1;
   if (d.leader != si || q > d.Nq) return;
   double *T = reinterpret_cast<double *>(sep + d.sep_mx) + (long long)(q - 1) * SEP_MXW;
   const ModeShape m = mode_shape(d, q, reinterpret_cast<const double *>(sep + d.sep_ab) + 2 * (q - 1));
@@ -34,7 +39,12 @@ __global__ void k_full_modes(const SubDesc *subs, int s0, unsigned char *sep) {
     // phi_2 = lambda^(N-n) carries the sign sg^N more than (-1)^n e^{-theta (N - n)}
     if (m.sg < 0.0 && (N & 1)) R12 = cmk(-R12.re, -R12.im);
   }
-  T[MX_KIND] = m.kind; T[MX_TH] = m.th; T[MX_LAM] = lam; T[MX_C] = c;
+  const double sth = m.kind == 0 ? sin(m.th) : m.kind == 1 ? sinh(m.th) : 0.0;
+  T[MX_SS] = m.kind == 0 ? -sth * sth : sth * sth;
+  T[MX_CS1] = m.kind < 2 ? sep_c(m.kind, m.th, 1.0) : 0.0;
+  T[MX_CS0] = m.kind < 2 ? sep_c(m.kind, m.th, -0.5 * N) : 0.0;
+  T[MX_CS0 + 1] = m.kind < 2 ? sep_s(m.kind, m.th, -0.5 * N) : 0.0;
+  T[MX_KIND] = m.kind; T[MX_LAM] = lam; T[MX_C] = c;
   T[MX_C1] = -c * expm1(-2.0 * m.th);
   T[MX_SG] = m.sg;
   T[MX_R] = R11.re; T[MX_R + 1] = R11.im; T[MX_R + 2] = R12.re; T[MX_R + 3] = R12.im;
@@ -44,13 +54,25 @@ __global__ void k_full_modes(const SubDesc *subs, int s0, unsigned char *sep) {
 
 namespace {
 
+// What every kernel of a pass reads, as a kernel argument: the first loads of a block would otherwise be a
+// chain of dependent reads of the descriptor.
+struct FullArg {
+  SubDesc d;
+  SepGeo g;
+  FullWs w;
+  int nr;
+  const unsigned char *sep;
+  double *ws;
+};
+
 // A: the grid's rows on folded columns (INV false: g(m) +- g(Nx - m)) or the modes (INV), cut into digits.
 // Row order (right-hand side, unknown row, part): a block's 8 rows are 4 grid rows, complex parts in turn.
 template <bool INV>
-__global__ void __launch_bounds__(256) k_full_cut(const SubDesc *subs, int sub, const double2 *g, double *ws, int nr) {
-  const SubDesc &d = subs[sub];
-  const SepGeo geo = sep_geo(d);
-  const FullWs w = full_ws(d, nr);
+__global__ void __launch_bounds__(256) k_full_cut(const __grid_constant__ FullArg p, const double2 *g) {
+  const SubDesc &d = p.d;
+  const SepGeo &geo = p.g;
+  const FullWs &w = p.w;
+  double *ws = p.ws;
   const int e = blockIdx.y, row = blockIdx.x * 8 + (threadIdx.x & 7), kl = threadIdx.x >> 3;
   const int nk = INV ? geo.nqh / 16 : geo.nkx, part = row & 1;
   const int n = (row >> 1) % d.Nt + d.nfirst, N = d.Nx;
@@ -102,95 +124,156 @@ __global__ void __launch_bounds__(256) k_full_cut(const SubDesc *subs, int sub, 
 
 template <bool INV>
 struct FullSrc {
-  const SubDesc *subs;
-  int sub, nr;
-  const unsigned char *sep;
-  double *ws;
+  const FullArg &p;
   struct Tile : DigitTile {
     int e, mt, nt;
   };
-  __device__ __forceinline__ int total() const {
-    const SubDesc &d = subs[sub];
-    const SepGeo g = sep_geo(d);
-    return 2 * (full_ws(d, nr).R / 128) * (INV ? g.ntx : g.nqh / 32);
-  }
+  __device__ __forceinline__ int total() const { return 2 * (p.w.R / 128) * (INV ? p.g.ntx : p.g.nqh / 32); }
   __device__ __forceinline__ bool tile(int v, Tile &t) const {
-    const SubDesc &d = subs[sub];
-    const SepGeo g = sep_geo(d);
-    const FullWs w = full_ws(d, nr);
-    const int nt = INV ? g.ntx : g.nqh / 32, nk = INV ? g.nqh / 16 : g.nkx, tr = v / nt;
+    const int nt = INV ? p.g.ntx : p.g.nqh / 32, nk = INV ? p.g.nqh / 16 : p.g.nkx, tr = v / nt, nm = p.w.R / 128;
     t.nt = v % nt;
-    t.e = tr / (w.R / 128);
-    t.mt = tr % (w.R / 128);
-    t.A = reinterpret_cast<const unsigned char *>(ws + w.a) + (long long)tr * nk * SEP_ABLK;
-    t.B = sep + (INV ? d.sep_xi : d.sep_xf) + ((long long)t.e * nt + t.nt) * nk * SEP_BBLK;
-    t.nkj = t.ND = t.ti = t.eb = 0;
-    t.ma = reinterpret_cast<const unsigned *>(ws + w.mask) + ((INV ? 2 * (w.R / 128) : 0) + tr) * SEP_MASK;
+    t.e = tr / nm;
+    t.mt = tr % nm;
+    t.A = reinterpret_cast<const unsigned char *>(p.ws + p.w.a) + (long long)tr * nk * SEP_ABLK;
+    t.B = p.sep + (INV ? p.d.sep_xi : p.d.sep_xf) + ((long long)t.e * nt + t.nt) * nk * SEP_BBLK;
+    t.nkj = t.ND = t.ti = 0;
+    t.eb = INV ? inv_exp(p.d) : 0;
+    t.ma = reinterpret_cast<const unsigned *>(p.ws + p.w.mask) + ((INV ? 2 * nm : 0) + tr) * SEP_MASK;
     t.mb = nullptr;
-    t.ex = reinterpret_cast<const int *>(ws + w.ex) + tr * 128;
+    t.ex = reinterpret_cast<const int *>(p.ws + p.w.ex) + tr * 128;
     return true;
   }
   __device__ __forceinline__ void dest(const Tile &t, int r, int o, double *&dst, long long &step, int &cnt) const {
-    const SubDesc &d = subs[sub];
-    const FullWs w = full_ws(d, nr);
     const int row = t.mt * 128 + r, o0 = t.nt * 32 + o;
     step = 1;
-    cnt = row < w.rows ? 16 : 0;
-    dst = INV ? ws + w.u + ((long long)t.e * w.R + row) * w.ldu + o0
-              : ws + w.f + (long long)row * w.ldf + t.e * (w.ldf / 2) + o0;
+    cnt = row < p.w.rows ? 8 : 0;
+    dst = INV ? p.ws + p.w.u + ((long long)t.e * p.w.R + row) * p.w.ldu + o0
+              : p.ws + p.w.f + (long long)row * p.w.ldf + t.e * (p.w.ldf / 2) + o0;
   }
 };
 
 template <bool INV>
-__global__ void __launch_bounds__(SG_THREADS, 1)
-    k_full_gemm(const SubDesc *subs, int sub, int nr, const unsigned char *sep, double *ws, int *status) {
-  const FullSrc<INV> src{subs, sub, nr, sep, ws};
+__global__ void __launch_bounds__(SG_THREADS, 1) k_full_gemm(const __grid_constant__ FullArg p, int *status) {
+  const FullSrc<INV> src{p};
   digit_gemm(src, status);
 }
 
-// x = T_q^{-1} g along y, in place on f: a block takes 32 modes of one right-hand side, warp s the rows of
-// segment s. Evanescent modes: y_n = lambda y_{n-1} + g_n upwards, x_n = lambda x_{n+1} + c (1 - lambda^2) y_n
-// downwards (their composition is c sum_j lambda^|n-j| g_j), each with the carry of the other segments,
-// then R's part. The others: x_n = phi_1 (A + F (M_2 - 2 P_2(n))) + phi_2 (B + F (2 P_1(n) - M_1)) with the running
-// moments P_b. Bound by the chain of dependent FP64 operations of a segment (3 passes of its rows) and
-// by reading f three times, mostly from L2.
-__global__ void __launch_bounds__(768) k_full_y(const SubDesc *subs, int sub, const unsigned char *sep, double *ws, int nr) {
-  extern __shared__ double ysh[];   // [4][warps][32]
-  const SubDesc &d = subs[sub];
-  const SepGeo g = sep_geo(d);
-  const FullWs w = full_ws(d, nr);
-  const int lane = threadIdx.x, s = threadIdx.y, NW = blockDim.y, Nt = d.Nt, N = d.ny - 1;
-  const int ci = blockIdx.x * 32 + lane, e = ci / g.nqh, q = sep_parity_mode(e, ci - e * g.nqh);
+// x = T_q^{-1} g along y, in place on f: a block takes 16 modes of one right-hand side (lanes 0..15 their real,
+// 16..31 their imaginary parts), warp s the rows of segment s. Evanescent modes: y_n = lambda y_{n-1} + g_n
+// upwards, x_n = lambda x_{n+1} + c (1 - lambda^2) y_n downwards (their composition is c sum_j
+// lambda^|n-j| g_j), each with the carry of the other segments, then R's part. The others: x_n =
+// phi_1 (A + F (M_2 - 2 P_2(n))) + phi_2 (B + F (2 P_1(n) - M_1)) with the running moments P_b. The
+// segments of a block are spread over a cluster of 4 SMs, their rows in shared memory: the warps that hold
+// the propagating modes take 3 times the others' FP64 instructions, and a warp's FP64 instruction holds
+// its SM's pipe for 19 cycles (a block on one SM: 207 us for 513^2, 4 right-hand sides, 24 % of the pipe).
+__device__ __forceinline__ double ipow(double x, int n) {
+  double r = 1.0;
+  for (; n; n >>= 1, x *= x)
+    if (n & 1) r *= x;
+  return r;
+}
+constexpr int FULL_Y_CTAS = 4, FULL_Y_WARPS = 8;   // CTAs of a cluster, most warps of one
+__global__ void __cluster_dims__(1, 1, FULL_Y_CTAS) __launch_bounds__(32 * FULL_Y_WARPS) k_full_y(const __grid_constant__ FullArg p) {
+  extern __shared__ double ysh[];   // [2][warps][32] of this CTA, [2][all warps][32], then this CTA's rows [rows][32]
+  const cg::cluster_group cl = cg::this_cluster();
+  const SubDesc &d = p.d;
+  const SepGeo &g = p.g;
+  const FullWs &w = p.w;
+  double *ws = p.ws;
+  const int lane = threadIdx.x, nw = blockDim.y, NW = nw * FULL_Y_CTAS, s = blockIdx.z * nw + threadIdx.y;
+  const int Nt = d.Nt, N = d.ny - 1;
+  const int ci = blockIdx.x * 16 + (lane & 15), im = lane >> 4, e = ci / g.nqh, q = sep_parity_mode(e, ci - e * g.nqh);
   const bool live = q <= d.Nq;
   const int seg = (Nt + NW - 1) / NW, i0 = min(Nt, s * seg), i1 = min(Nt, i0 + seg);
-  const long long step = 2LL * w.ldf;
-  double *f = ws + w.f + (long long)blockIdx.y * Nt * step + ci;   // row i: f[i step], its imaginary part ldf on
-  const double *T = reinterpret_cast<const double *>(sep + d.sep_mx) + (long long)(live ? q - 1 : 0) * SEP_MXW;
+  const long long gstep = 2LL * w.ldf;
+  double *fg = ws + w.f + (long long)blockIdx.y * Nt * gstep + im * w.ldf + ci;
+  double *f = ysh + (2 * nw + 2 * NW) * 32 + lane - 32LL * blockIdx.z * nw * seg;   // row i: f[32 i]
+#pragma unroll 8
+  for (int i = i0; i < i1; ++i) f[32 * i] = fg[i * gstep];   // a thread reads only what it writes
+  const double *T = reinterpret_cast<const double *>(p.sep + d.sep_mx) + (long long)(live ? q - 1 : 0) * SEP_MXW;
   const int kind = (int)T[MX_KIND];
-  const double th = T[MX_TH], lam = T[MX_LAM], sg = T[MX_SG];
-  double *sh[4];
-  for (int k = 0; k < 4; ++k) sh[k] = ysh + (k * NW) * 32;
-  const int me = s * 32 + lane;
+  const double lam = T[MX_LAM], sg = T[MX_SG];
+  // what every segment has to say, gathered from the cluster's CTAs after each exchange
+  double *mine0 = ysh, *mine1 = ysh + nw * 32, *sh0 = ysh + 2 * nw * 32, *sh1 = sh0 + NW * 32;
+  const int me = threadIdx.y * 32 + lane;
+  auto exchange = [&](double a, double b) {
+    mine0[me] = a;
+    mine1[me] = b;
+    cl.sync();
+    for (int k = threadIdx.y; k < NW; k += nw) {
+      const double *r0 = cl.map_shared_rank(mine0, k / nw), *r1 = cl.map_shared_rank(mine1, k / nw);
+      sh0[k * 32 + lane] = r0[(k % nw) * 32 + lane];
+      sh1[k * 32 + lane] = r1[(k % nw) * 32 + lane];
+    }
+    cl.sync();   // the values may be overwritten, and the CTA may end
+  };
+  // the other part of a lane's mode: (re, im) of a value that this lane holds one part of
+  auto both = [&](double v) { const double o = __shfl_xor_sync(0xffffffffu, v, 16); return im ? cmk(o, v) : cmk(v, o); };
+  auto part = [&](cplx v) { return im ? v.im : v.re; };
   // rotation state of kinds 0, 1 at the segment's first row
-  const double sth = kind == 0 ? sin(th) : sinh(th), ss = kind == 0 ? -sth * sth : sth * sth;
-  const double c1 = kind < 2 ? sep_c(kind, th, 1.0) : 0.0;
-  double C0 = 0.0, S0 = 0.0, w0 = 1.0;
-  cplx a = cmk(0.0, 0.0), b = a;
-  if (live) {
-    if (kind == 2) {
-      for (int i = i0; i < i1; ++i) {
-        a.re = fma(lam, a.re, f[i * step]);
-        a.im = fma(lam, a.im, f[i * step + w.ldf]);
-      }
-    } else {
-      const double x = i0 + d.nfirst - 0.5 * N;
-      C0 = sep_c(kind, th, x); S0 = sep_s(kind, th, x);
-      w0 = sg < 0.0 && ((i0 + d.nfirst) & 1) ? -1.0 : 1.0;
+  double ss = 0.0, c1 = 0.0, C0 = 0.0, S0 = 0.0, w0 = 1.0, a = 0.0, b = 0.0;
+  if (live && kind < 2) {
+    ss = T[MX_SS];
+    c1 = T[MX_CS1];
+    C0 = T[MX_CS0];
+    S0 = T[MX_CS0 + 1];
+    double Cp = c1, Sp = 1.0;   // the rotation by 1, 2, 4, ... rows
+    for (int m = i0 + d.nfirst; m; m >>= 1) {
+      if (m & 1) { const double Cn = fma(S0 * ss, Sp, C0 * Cp); S0 = fma(S0, Cp, C0 * Sp); C0 = Cn; }
+      const double Cq = fma(Sp * ss, Sp, Cp * Cp);
+      Sp = 2.0 * Sp * Cp;
+      Cp = Cq;
+    }
+    w0 = sg < 0.0 && ((i0 + d.nfirst) & 1) ? -1.0 : 1.0;
+    double C = C0, S = S0, v = w0;
+    for (int i = i0; i < i1; ++i) {
+      const double gv = v * f[32 * i];
+      a = fma(C, gv, a);
+      b = fma(S, gv, b);
+      const double Cn = fma(S, ss, C * c1);
+      S = fma(S, c1, C);
+      C = Cn;
+      v *= sg;
+    }
+  } else if (live) {
+#pragma unroll 4
+    for (int i = i0; i < i1; ++i) a = fma(lam, a, f[32 * i]);
+  }
+  exchange(a, b);
+  const double ll = kind == 2 ? ipow(lam, seg) : 0.0;   // lambda^seg
+  double ytop = 0.0, m1 = 0.0, m2 = 0.0, p1 = 0.0, p2 = 0.0;
+  if (live && kind == 2) {
+    double y = 0.0;
+    for (int k = 0; k < s; ++k) y = fma(ll, y, sh0[k * 32 + lane]);
+#pragma unroll 4
+    for (int i = i0; i < i1; ++i) {   // upwards
+      y = fma(lam, y, f[32 * i]);
+      f[32 * i] = y;
+    }
+    ytop = y;
+    a = 0.0;                          // the segment's part of the downward sum, sum lambda^(i - i0) y_i
+#pragma unroll 4
+    for (int i = i1 - 1; i >= i0; --i) a = fma(lam, a, f[32 * i]);
+  } else if (live) {
+    for (int k = 0; k < NW; ++k) {
+      const double u = sh0[k * 32 + lane], v = sh1[k * 32 + lane];
+      if (k < s) { p1 += u; p2 += v; }
+      m1 += u;
+      m2 += v;
+    }
+  }
+  const cplx R11 = ld2(T + MX_R), R12 = ld2(T + MX_R + 2), R22 = ld2(T + MX_R + 4);
+  {   // every lane takes part in the exchange; kind 2 has no moments yet
+    const cplx M1 = both(m1), M2 = both(m2);
+    if (live && kind < 2) {
+      const double F = T[MX_F];
+      const double A = fma(F, m2, part(cadd(cmul(R11, M1), cmul(R12, M2)))), B = fma(-F, m1, part(cadd(cmul(R12, M1), cmul(R22, M2))));
       double C = C0, S = S0, v = w0;
       for (int i = i0; i < i1; ++i) {
-        const double gr = v * f[i * step], gi = v * f[i * step + w.ldf];
-        a = cmk(fma(C, gr, a.re), fma(C, gi, a.im));
-        b = cmk(fma(S, gr, b.re), fma(S, gi, b.im));
+        const double gv = v * f[32 * i];
+        p1 = fma(C, gv, p1);
+        p2 = fma(S, gv, p2);
+        f[32 * i] = v * fma(C, fma(-2.0 * F, p2, A), S * fma(2.0 * F, p1, B));
         const double Cn = fma(S, ss, C * c1);
         S = fma(S, c1, C);
         C = Cn;
@@ -198,110 +281,76 @@ __global__ void __launch_bounds__(768) k_full_y(const SubDesc *subs, int sub, co
       }
     }
   }
-  sh[0][me] = a.re; sh[1][me] = a.im; sh[2][me] = b.re; sh[3][me] = b.im;
-  __syncthreads();
-  const double ll = kind == 2 ? exp(-th * seg) * (sg < 0.0 && (seg & 1) ? -1.0 : 1.0) : 0.0;   // lambda^seg
-  cplx ytop = cmk(0.0, 0.0);
-  if (live && kind == 2) {
-    cplx y = cmk(0.0, 0.0);
-    for (int k = 0; k < s; ++k) { y.re = fma(ll, y.re, sh[0][k * 32 + lane]); y.im = fma(ll, y.im, sh[1][k * 32 + lane]); }
-    // upwards; on the way the segment's part of the downward sum, a = sum lambda^(i - i0) y_i
-    double pw = 1.0;
-    a = cmk(0.0, 0.0);
-    for (int i = i0; i < i1; ++i) {
-      y.re = fma(lam, y.re, f[i * step]);
-      y.im = fma(lam, y.im, f[i * step + w.ldf]);
-      f[i * step] = y.re;
-      f[i * step + w.ldf] = y.im;
-      a.re = fma(pw, y.re, a.re);
-      a.im = fma(pw, y.im, a.im);
-      pw *= lam;
-    }
-    ytop = y;
-  } else if (live) {
-    cplx m1 = cmk(0.0, 0.0), m2 = m1, p1 = m1, p2 = m1;
-    for (int k = 0; k < NW; ++k) {
-      const cplx u = cmk(sh[0][k * 32 + lane], sh[1][k * 32 + lane]), v = cmk(sh[2][k * 32 + lane], sh[3][k * 32 + lane]);
-      if (k < s) { p1 = cadd(p1, u); p2 = cadd(p2, v); }
-      m1 = cadd(m1, u);
-      m2 = cadd(m2, v);
-    }
-    const cplx R11 = ld2(T + MX_R), R12 = ld2(T + MX_R + 2), R22 = ld2(T + MX_R + 4);
-    const double F = T[MX_F];
-    const cplx A = caxpy(F, m2, cadd(cmul(R11, m1), cmul(R12, m2))), B = caxpy(-F, m1, cadd(cmul(R12, m1), cmul(R22, m2)));
-    double C = C0, S = S0, v = w0;
-    for (int i = i0; i < i1; ++i) {
-      const double gr = v * f[i * step], gi = v * f[i * step + w.ldf];
-      p1 = cmk(fma(C, gr, p1.re), fma(C, gi, p1.im));
-      p2 = cmk(fma(S, gr, p2.re), fma(S, gi, p2.im));
-      f[i * step] = v * fma(C, fma(-2.0 * F, p2.re, A.re), S * fma(2.0 * F, p1.re, B.re));
-      f[i * step + w.ldf] = v * fma(C, fma(-2.0 * F, p2.im, A.im), S * fma(2.0 * F, p1.im, B.im));
-      const double Cn = fma(S, ss, C * c1);
-      S = fma(S, c1, C);
-      C = Cn;
-      v *= sg;
-    }
-  }
-  __syncthreads();
-  sh[0][me] = a.re; sh[1][me] = a.im; sh[2][me] = ytop.re; sh[3][me] = ytop.im;
-  __syncthreads();
-  if (!live || kind != 2) return;
+  exchange(a, ytop);
   const double c = T[MX_C], cc = T[MX_C1];
   // the top row takes x = c y there: as if the row above held c lambda y. Empty last segments pass on.
   const int last = (Nt - 1) / seg;
-  const cplx yt = cmk(sh[2][last * 32 + lane], sh[3][last * 32 + lane]);
-  cplx x = cmk(c * lam * yt.re, c * lam * yt.im), mine = x;   // x just above segment k
+  const double yt = sh1[last * 32 + lane];
+  double x = c * lam * yt, mine = x;   // x just above segment k
   for (int k = last; k >= 0; --k) {
     if (k == s) mine = x;
     const int len = min(seg, Nt - k * seg);
-    const double l = len == seg ? ll : exp(-th * len) * (sg < 0.0 && (len & 1) ? -1.0 : 1.0);
-    x.re = fma(l, x.re, cc * sh[0][k * 32 + lane]);
-    x.im = fma(l, x.im, cc * sh[1][k * 32 + lane]);
+    x = fma(len == seg ? ll : ipow(lam, len), x, cc * sh0[k * 32 + lane]);
   }
-  if (i0 >= i1) return;
   // moments of phi = (lambda^n, lambda^(N-n)) from the two ends: c M_1 is x continued to row 0, M_2 is y at row N
   const double e1 = d.nfirst ? lam : 1.0;
-  const cplx m1 = cmk(e1 * x.re / c, e1 * x.im / c), m2 = cmk(e1 * yt.re, e1 * yt.im);
-  const cplx R11 = ld2(T + MX_R), R12 = ld2(T + MX_R + 2), R22 = ld2(T + MX_R + 4);
-  const cplx A = cadd(cmul(R11, m1), cmul(R12, m2)), B = cadd(cmul(R12, m1), cmul(R22, m2));
-  const int nt = i1 - 1 + d.nfirst;   // grid row of the segment's last row
-  double pa = exp(-th * nt) * (sg < 0.0 && (nt & 1) ? -1.0 : 1.0), pb = exp(-th * (N - nt)) * (sg < 0.0 && ((N - nt) & 1) ? -1.0 : 1.0);
-  const double li = 1.0 / lam;
-  x = mine;
-  for (int i = i1 - 1; i >= i0; --i) {
-    x.re = fma(lam, x.re, cc * f[i * step]);
-    x.im = fma(lam, x.im, cc * f[i * step + w.ldf]);
-    f[i * step] = fma(pa, A.re, fma(pb, B.re, x.re));
-    f[i * step + w.ldf] = fma(pa, A.im, fma(pb, B.im, x.im));
-    pa *= li;
-    pb *= lam;
+  const cplx M1 = both(kind == 2 ? e1 * x / c : 0.0), M2 = both(e1 * yt);
+  if (live && kind == 2) {
+    const double A = part(cadd(cmul(R11, M1), cmul(R12, M2))), B = part(cadd(cmul(R12, M1), cmul(R22, M2)));
+    const int nt = i1 - 1 + d.nfirst;   // grid row of the segment's last row
+    double pa = i1 > i0 ? ipow(lam, i0 + d.nfirst) : 0.0, pb = i1 > i0 ? ipow(lam, N - nt) : 0.0;
+    x = mine;
+    // 2^-90 of the reflected waves is zero to working precision: the rows far from both ends
+    if (__all_sync(__activemask(), fabs(pa) < 0x1p-90 && fabs(pb) < 0x1p-90)) {
+#pragma unroll 4
+      for (int i = i1 - 1; i >= i0; --i) {
+        x = fma(lam, x, cc * f[32 * i]);
+        fg[i * gstep] = x;
+      }
+    } else {
+      const double li = 1.0 / lam;
+      pa = i1 > i0 ? ipow(lam, nt) : 0.0;
+#pragma unroll 4
+      for (int i = i1 - 1; i >= i0; --i) {
+        x = fma(lam, x, cc * f[32 * i]);
+        fg[i * gstep] = fma(pa, A, fma(pb, B, x));
+        pa *= li;
+        pb *= lam;
+      }
+    }
+  } else if (live) {
+    for (int i = i0; i < i1; ++i) fg[i * gstep] = f[32 * i];
   }
 }
 
-// u(m) = (2/Nx) (U_0 + U_1), u(Nx - m) = (2/Nx) (U_0 - U_1) on the unknown rows, 0 on the Dirichlet ends.
-__global__ void __launch_bounds__(128) k_full_out(const SubDesc *subs, int sub, const double *ws, double2 *u, int nr) {
-  const SubDesc &d = subs[sub];
-  const FullWs w = full_ws(d, nr);
-  const int m = blockIdx.x * 128 + threadIdx.x, n = blockIdx.y, rl = blockIdx.z, i = n - d.nfirst, N = d.Nx;
+// u(m) = U_0 + U_1, u(Nx - m) = U_0 - U_1 on the unknown rows, 0 on the Dirichlet ends.
+__global__ void __launch_bounds__(256) k_full_out(const __grid_constant__ FullArg p, double2 *u) {
+  const SubDesc &d = p.d;
+  const FullWs &w = p.w;
+  const double *ws = p.ws;
+  const int m = blockIdx.x * blockDim.x + threadIdx.x, n = blockIdx.y, rl = blockIdx.z, i = n - d.nfirst, N = d.Nx;
   if (2 * m > N) return;
-  double2 p = make_double2(0.0, 0.0), q = p;
+  double2 up = make_double2(0.0, 0.0), um = up;
   if (m >= 1 && i >= 0 && i < d.Nt) {
     const double *U = ws + w.u + (2LL * (rl * (long long)d.Nt + i)) * w.ldu + m - 1;
     const long long other = (long long)w.R * w.ldu;
-    const double sc = 2.0 / N, a = U[0], b = U[other], ai = U[w.ldu], bi = U[other + w.ldu];
-    p = make_double2(sc * (a + b), sc * (ai + bi));
-    q = make_double2(sc * (a - b), sc * (ai - bi));
+    const double a = U[0], b = U[other], ai = U[w.ldu], bi = U[other + w.ldu];
+    up = make_double2(a + b, ai + bi);
+    um = make_double2(a - b, ai - bi);
   }
   double2 *row = u + ((long long)rl * d.ny + n) * d.nx;
-  row[m] = p;
-  if (2 * m != N) row[N - m] = q;
+  row[m] = up;
+  if (2 * m != N) row[N - m] = um;
 }
 
 }  // namespace
 
+static constexpr int FULL_Y_SMEM = 227 * 1024;
+
 cudaError_t set_full_kernel_attributes() {
   cudaError_t e = cudaFuncSetAttribute(k_full_gemm<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SG_SMEM);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_full_gemm<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SG_SMEM);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_full_y, cudaFuncAttributeMaxDynamicSharedMemorySize, FULL_Y_SMEM);
   return e;
 }
 
@@ -312,22 +361,29 @@ cudaError_t launch_full_solve(const mdp_plan *p, int sub, int nrhs, const double
   int chunk = (int)std::min<long long>(std::min(nrhs, 32768), std::max<long long>(1, p->ws_doubles / full_ws(d, 1).total));
   while (chunk > 1 && full_ws(d, chunk).total > p->ws_doubles) --chunk;
   if (full_ws(d, chunk).total > p->ws_doubles) return cudaErrorMemoryAllocation;
-  // segments of about 16 rows along y, at most 24 (768 threads of 80 registers)
-  const int nw = std::min(24, (d.Nt + 15) / 16);
+
   for (int r0 = 0; r0 < nrhs; r0 += chunk) {
     const int nr = std::min(chunk, nrhs - r0);
     const FullWs w = full_ws(d, nr);
+    // segments along y, a multiple of the cluster's 4: of about 32 rows where the blocks fill the chip (each
+    // segment has a fixed cost of some 100 FP64 instructions), else of 16
+    const int rows = nr * (w.ldf / 16) >= 2 * p->n_sm ? 32 : 16;
+    const int nw = std::min(FULL_Y_WARPS, std::max(1, (d.Nt + rows * FULL_Y_CTAS - 1) / (rows * FULL_Y_CTAS)));
+    const int seg = (d.Nt + nw * FULL_Y_CTAS - 1) / (nw * FULL_Y_CTAS);
+    const int ysm = ((2 + 2 * FULL_Y_CTAS) * nw + nw * seg) * 256;
     const double2 *gc = g + (long long)r0 * d.nx * d.ny;
     double2 *uc = u + (long long)r0 * d.nx * d.ny;
     auto gemm_grid = [&](int nt) { return dim3((unsigned)std::min(p->n_sm, 2 * (w.R / 128) * nt)); };
     cudaError_t e = cudaMemsetAsync(p->d_ws + w.mask, 0, 2LL * (w.R / 128) * SEP_MASK * 8, st);
     if (e != cudaSuccess) return e;
-    k_full_cut<false><<<dim3(w.R / 8, 2), 256, 0, st>>>(p->d_subs, sub, gc, p->d_ws, nr);
-    k_full_gemm<false><<<gemm_grid(geo.nqh / 32), SG_THREADS, SG_SMEM, st>>>(p->d_subs, sub, nr, p->d_sep, p->d_ws, p->d_status);
-    k_full_y<<<dim3(w.ldf / 32, nr), dim3(32, nw), 4 * nw * 32 * sizeof(double), st>>>(p->d_subs, sub, p->d_sep, p->d_ws, nr);
-    k_full_cut<true><<<dim3(w.R / 8, 2), 256, 0, st>>>(p->d_subs, sub, gc, p->d_ws, nr);
-    k_full_gemm<true><<<gemm_grid(geo.ntx), SG_THREADS, SG_SMEM, st>>>(p->d_subs, sub, nr, p->d_sep, p->d_ws, p->d_status);
-    k_full_out<<<dim3((d.Nx / 2 + 128) / 128, d.ny, nr), 128, 0, st>>>(p->d_subs, sub, p->d_ws, uc, nr);
+    const FullArg a{d, geo, w, nr, p->d_sep, p->d_ws};
+    k_full_cut<false><<<dim3(w.R / 8, 2), 256, 0, st>>>(a, gc);
+    k_full_gemm<false><<<gemm_grid(geo.nqh / 32), SG_THREADS, SG_SMEM, st>>>(a, p->d_status);
+    k_full_y<<<dim3(w.ldf / 16, nr, FULL_Y_CTAS), dim3(32, nw), ysm, st>>>(a);
+    k_full_cut<true><<<dim3(w.R / 8, 2), 256, 0, st>>>(a, gc);
+    k_full_gemm<true><<<gemm_grid(geo.ntx), SG_THREADS, SG_SMEM, st>>>(a, p->d_status);
+    const int nm = d.Nx / 2 + 1, tm = std::min(256, (nm + 31) / 32 * 32);
+    k_full_out<<<dim3((nm + tm - 1) / tm, d.ny, nr), tm, 0, st>>>(a, uc);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }

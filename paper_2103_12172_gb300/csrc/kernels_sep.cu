@@ -37,10 +37,10 @@ namespace mdp {
 namespace {
 
 // ---------------------------------------------------------------- mode table
-__global__ void __launch_bounds__(128) k_sep_mode_tab(const SubDesc *subs, int s0, unsigned char *sep, int entries) {
+__global__ void __launch_bounds__(32) k_sep_mode_tab(const SubDesc *subs, int s0, unsigned char *sep, int entries) {
   const int si = s0 + blockIdx.y;
   const SubDesc &d = subs[si];
-  const int q = blockIdx.x * 128 + threadIdx.x + 1;
+  const int q = blockIdx.x * 32 + threadIdx.x + 1;   // one warp per block: the FP64 pipe is an SM's
   if (d.leader != si || q > d.Nq) return;
   double *T = reinterpret_cast<double *>(sep + d.sep_mt) + (long long)(q - 1) * SEP_MTW;
   double *ab = reinterpret_cast<double *>(sep + d.sep_ab) + 2 * (q - 1);
@@ -57,28 +57,63 @@ __global__ void __launch_bounds__(128) k_sep_mode_tab(const SubDesc *subs, int s
   double n1 = 1.0, n2 = 1.0, c = 0.0, rf;
   cplx R11, R12, R22;
   const int rows_d[4] = {d.nlo, d.nlo + 1, d.nhi - 1, d.nhi}, rows_g[4] = {d.nlo - 1, d.nlo, d.nhi, d.nhi + 1};
-  auto sgn = [&](int i) { return (sg < 0.0 && (i & 1)) ? -1.0 : 1.0; };   // sg^i
+  const int L = d.nhi - d.nlo;   // J1 - J0 - 2
+  // phi_1, phi_2 at the 3 rows from either end (J0 + k, J1 - k), kappa at 0, 1, 2, L-1, L, L+1 without the sign
+  // sg^i; kappa(d) = T1 phi_1(J0 + d) + T2 phi_2(J0 + d). An FP64 instruction takes this thread's warp 64
+  // cycles whatever its lanes do, a transcendental function some 50 of them: the neighbouring rows
+  // follow by one rotation or one factor.
+  double lo1[3], lo2[3], hi1[3], hi2[3], kv[6], T1, T2 = 0.0, el[3] = {0.0, 0.0, 0.0};
   if (kind < 2) {
-    double bound = kind == 0 ? fmax(Lh, 1.0) : sep_s(1, th, Lh);
-    if (kind == 0) bound = fmin(bound, 1.0 / sin(th));
+    const double sth = kind == 0 ? sin(th) : sinh(th), c1 = sep_c(kind, th, 1.0), ss = kind == 0 ? -sth * sth : sth * sth;
+    auto cs = [&](double x, double &C, double &S) {
+      if (th == 0.0) { C = 1.0; S = x; return; }
+      if (kind == 0) { sincos(x * th, &S, &C); S /= sth; }
+      else { C = cosh(x * th); S = sinh(x * th) / sth; }
+    };
+    auto up = [&](double &C, double &S) { const double Cn = fma(S, ss, C * c1); S = fma(S, c1, C); C = Cn; };
+    double CL, SL, Ch, Sh, C2, S2;
+    cs(Lh, Ch, Sh);              // the end rows: C even, S odd about the middle
+    cs(L - 1, CL, SL);
+    cs(J1 - J0, C2, S2);
+    double bound = kind == 0 ? fmin(fmax(Lh, 1.0), 1.0 / sth) : Sh;
     n2 = pow2i(-(ilogb(fmax(bound, 1.0)) + 1));
     if (kind == 1) n1 = 0.25;
     reflect_cs(ms, N, mid, R11, R12, R22);
-    const double s1 = 1.0 / n1, s2 = 1.0 / n2;
+    const double s1 = 1.0 / n1, s2 = 1.0 / n2;   // powers of two
     R11 = cmk(R11.re * s1 * s1, R11.im * s1 * s1);
     R12 = cmk(R12.re * s1 * s2, R12.im * s1 * s2);
     R22 = cmk(R22.re * s2 * s2, R22.im * s2 * s2);
-    double kb = kind == 0 ? (double)(J1 - J0) : sep_s(1, th, J1 - J0);
-    if (kind == 0) kb = fmin(kb, 1.0 / sin(th));
+    double C = Ch, S = -Sh;
+    for (int k = 0; k < 3; ++k) {
+      lo1[k] = hi1[k] = n1 * C;
+      lo2[k] = n2 * S;
+      hi2[k] = -n2 * S;
+      up(C, S);
+    }
+    const double ia = 1.0 / (2.0 * a);
+    kv[0] = 0.0; kv[1] = ia; kv[2] = 2.0 * c1 * ia;
+    for (int k = 3; k < 6; ++k) { kv[k] = SL * ia; up(CL, SL); }
+    T1 = Sh * ia / n1;
+    T2 = Ch * ia / n2;
+    const double kb = kind == 0 ? fmin((double)(J1 - J0), 1.0 / sth) : S2;
     rf = pow2i(-(ilogb(fmax(kb, 1.0) / (2.0 * fabs(a))) + 1));
   } else {
-    c = -1.0 / (2.0 * a * sinh(th));
+    const double em = exp(-th), ep = exp(th), fl = exp(-th * (L - 1));
+    c = -1.0 / (a * (ep - em));
     reflect_exp(ms, N, J0, J1, c, R11, R12, R22);
+    const double far = fl * em * em * em;   // J1 - J0 = L + 2
+    lo1[0] = hi2[0] = 1.0; lo1[1] = hi2[1] = em; lo1[2] = hi2[2] = em * em;
+    hi1[0] = lo2[0] = far; hi1[1] = lo2[1] = fl * em * em; hi1[2] = lo2[2] = fl * em;
+    kv[0] = c; kv[1] = c * em; kv[2] = c * em * em;
+    kv[3] = c * fl; kv[4] = c * fl * em; kv[5] = c * fl * em * em;
+    el[0] = c; el[1] = c * ep; el[2] = c * ep * ep;   // kappa as a wave from J0: c e^{theta k} at the sources J0 + k
+    T1 = c;
     rf = pow2i(-(ilogb(fabs(c)) + 1));
   }
-  auto p1 = [&](int i) { return sgn(i - J0) * (kind == 2 ? exp(-th * (i - J0)) : n1 * sep_c(kind, th, i - mid)); };
-  auto p2 = [&](int i) { return sgn(i - J0) * (kind == 2 ? exp(-th * (J1 - i)) : n2 * sep_s(kind, th, i - mid)); };
-  auto kap = [&](int x) { return sgn(x) * (kind == 2 ? c * exp(-th * x) : sep_s(kind, th, x) / (2.0 * a)); };
+  auto sgn = [&](int i) { return (sg < 0.0 && (i & 1)) ? -1.0 : 1.0; };   // sg^i
+  auto p1 = [&](int i) { return sgn(i - J0) * (i - J0 < 3 ? lo1[i - J0] : hi1[J1 - i]); };
+  auto p2 = [&](int i) { return sgn(i - J0) * (i - J0 < 3 ? lo2[i - J0] : hi2[J1 - i]); };
+  auto kap = [&](int x) { return sgn(x) * (x < 3 ? kv[x] : kv[x - L + 4]); };
   const double f = 1.0 / (2.0 * a * n1 * n2);
   // an imaginary part below 2^-62 of kappa's scale is zero to working precision
   const bool imag = kind < 2 ? d.cplx : fmax(fmax(fabs(R11.im), fabs(R12.im)), fabs(R22.im)) > 0x1p-62 * fabs(c);
@@ -95,8 +130,8 @@ __global__ void __launch_bounds__(128) k_sep_mode_tab(const SubDesc *subs, int s
       const int j = rows_d[k];
       const double up = k < 2 ? 1.0 : -1.0;   // dense rows 0, 1 lie below the middle rows
       if (kind < 2) { E1 = -up * f * f2; E2 = up * f * f1; }
-      else if (k < 2) E1 = c * exp(th * (j - J0)) * sgn(j - J0);
-      else E2 = c * exp(th * (J1 - j)) * sgn(j - J0);
+      else if (k < 2) E1 = el[j - J0] * sgn(j - J0);
+      else E2 = el[J1 - j] * sgn(j - J0);
     }
     mat[k] = A + E1;
     mat[6 + k] = B + E2;
@@ -107,8 +142,8 @@ __global__ void __launch_bounds__(128) k_sep_mode_tab(const SubDesc *subs, int s
       else {
         const double up = r < 2 ? 1.0 : -1.0;   // gamma rows 0, 1 lie below the middle rows
         if (kind < 2) w = k == 4 ? -up * f * T[MT_P2G + r] : up * f * T[MT_P1G + r];
-        else if (k == 4) w = r < 2 ? c * exp(th * (n - J0)) * sgn(n - J0) : 0.0;
-        else w = r < 2 ? 0.0 : c * exp(th * (J1 - n)) * sgn(n - J0);
+        else if (k == 4) w = r < 2 ? el[n - J0] * sgn(n - J0) : 0.0;
+        else w = r < 2 ? 0.0 : el[J1 - n] * sgn(n - J0);
       }
       mat[6 * (2 + r) + k] = fma(T[MT_P1G + r], A, fma(T[MT_P2G + r], B, w));
     }
@@ -116,11 +151,14 @@ __global__ void __launch_bounds__(128) k_sep_mode_tab(const SubDesc *subs, int s
   T[MT_R + 0] = R11.re; T[MT_R + 1] = R11.im; T[MT_R + 2] = R12.re; T[MT_R + 3] = R12.im;
   T[MT_R + 4] = R22.re; T[MT_R + 5] = R22.im;
   T[MT_IMAG] = imag ? 1.0 : 0.0;
-  T[MT_REC + 0] = d.nrec >= 0 ? p1(d.nrec) : 0.0;
-  T[MT_REC + 1] = d.nrec >= 0 ? p2(d.nrec) : 0.0;
+  T[MT_FAR] = kind == 2 && lo2[0] < 0x1p-90 ? 1.0 : 0.0;   // 2^-90 of the other end is zero to working precision
+  if (d.nrec >= 0) {
+    T[MT_REC + 0] = sgn(d.nrec - J0) * (kind == 2 ? exp(-th * (d.nrec - J0)) : n1 * sep_c(kind, th, d.nrec - mid));
+    T[MT_REC + 1] = sgn(d.nrec - J0) * (kind == 2 ? exp(-th * (J1 - d.nrec)) : n2 * sep_s(kind, th, d.nrec - mid));
+  }
   T[MT_REC + 2] = 1.0 / rf;
-  T[MT_T1] = kind == 2 ? c : sep_s(kind, th, Lh) / (2.0 * a * n1);
-  T[MT_T2] = kind == 2 ? 0.0 : sep_c(kind, th, Lh) / (2.0 * a * n2);
+  T[MT_T1] = T1;
+  T[MT_T2] = T2;
   T[MT_RF] = rf;
   T[MT_F] = f;
   T[MT_TH] = th; T[MT_KIND] = kind; T[MT_SG] = sg; T[MT_N1] = n1; T[MT_N2] = n2;
@@ -302,7 +340,7 @@ __global__ void __launch_bounds__(256) k_sep_mb(const SubDesc *subs, int s0, con
   store_digits(B + (o >> 3) * 256 + half * 128 + (o & 7) * 16, 1024, V);
 }
 
-// The synthesis table, B of stage 3: output (s, i), K index (b, q): sin(pi q m_s/Nx) phi_b(i).
+// The synthesis table, B of stage 3: output (s, i), K index (b, q): (2/Nx) sin(pi q m_s/Nx) phi_b(i).
 __global__ void __launch_bounds__(256) k_sep_b3(const SubDesc *subs, int s0, const double *tab, unsigned char *sep) {
   const int si = s0 + blockIdx.z;
   const SubDesc &d = subs[si];
@@ -315,13 +353,13 @@ __global__ void __launch_bounds__(256) k_sep_b3(const SubDesc *subs, int s0, con
   const int s = to / g.nti, i = (to % g.nti) * 32 + o;
   const int b = kb * 16 / g.nqp, q0 = kb * 16 % g.nqp + 8 * half;
   const int m = sep_out_col(d, s), N2 = 2 * d.Nx;
-  const double *S = tab + d.sin_off;
+  const double *S = tab + d.sin_off, sc = inv_scale(d);
   const double *P = reinterpret_cast<const double *>(sep + d.sep_phi) + ((long long)b * (d.Py + 2) + 2 + i) * d.Nq;
   long long V[8];
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
     const int q = sep_mode(d, e, q0 + j);
-    V[j] = (i < g.Pi && q <= d.Nq) ? fix54(P[q - 1] * S[(int)(((long long)q * m) % N2)]) : 0;
+    V[j] = (i < g.Pi && q <= d.Nq) ? fix54(P[q - 1] * (sc * S[(int)(((long long)q * m) % N2)])) : 0;
   }
   mark_group(reinterpret_cast<unsigned *>(sep + d.sep_z3) + (e * g.nt3 + to) * SEP_MASK, kb, V);
   unsigned char *B = sep + d.sep_b3 + (((long long)e * g.nt3 + to) * g.nk3 + kb) * SEP_BBLK;
@@ -330,13 +368,14 @@ __global__ void __launch_bounds__(256) k_sep_b3(const SubDesc *subs, int s0, con
 
 // The sine tables of the full rows' transforms (which: 0 FWD, 1 INV, 2, 3 the same over every folded column
 // for full-grid solves). FWD: output q of parity e, K index m' - mf; INV: output m' - mg, K index q of
-// parity e; both sin(pi q m'/Nx) over the folded columns m' <= Nx/2.
+// parity e; both sin(pi q m'/Nx) over the folded columns m' <= Nx/2, the inverse times 2/Nx.
 __global__ void __launch_bounds__(256) k_sep_sines(const SubDesc *subs, int s0, const double *tab, unsigned char *sep, int which) {
   const int si = s0 + blockIdx.z;
   const SubDesc &d = subs[si];
   if (!d.tc_cols || d.leader != si) return;
   const SepGeo g = sep_geo(d);
   const bool inv = which & 1, full = which & 2;
+  const double sc = inv ? inv_scale(d) : 1.0;
   const int nto = inv ? (full ? g.ntx : g.ntg) : g.nqh / 32, nk = inv ? g.nqh / 16 : full ? g.nkx : g.nkf;
   const int m0 = full ? 1 : inv ? g.mg : g.mf;
   const int e = blockIdx.y / nto, to = blockIdx.y % nto;
@@ -349,7 +388,7 @@ __global__ void __launch_bounds__(256) k_sep_sines(const SubDesc *subs, int s0, 
   for (int j = 0; j < 8; ++j) {
     const int ko = to * 32 + o, kk = kb * 16 + 8 * half + j;
     const int q = sep_parity_mode(e, inv ? kk : ko), m = m0 + (inv ? ko : kk);
-    V[j] = q <= d.Nq && 2 * m <= d.Nx ? fix54(S[(int)(((long long)q * m) % (2 * d.Nx))]) : 0;
+    V[j] = q <= d.Nq && 2 * m <= d.Nx ? fix54(sc * S[(int)(((long long)q * m) % (2 * d.Nx))]) : 0;
   }
   unsigned char *B = sep + (full ? (inv ? d.sep_xi : d.sep_xf) : inv ? d.sep_bi : d.sep_bf) + (((long long)e * nto + to) * nk + kb) * SEP_BBLK;
   store_digits(B + (o >> 3) * 256 + half * 128 + (o & 7) * 16, 1024, V);
@@ -495,8 +534,10 @@ struct SepSrc {
     if (t.job == J_SYN) {
       t.B = sep + d.sep_b3 + ((long long)t.e * g.nt3 + t.nt) * nk * SEP_BBLK;
       t.mb = reinterpret_cast<const unsigned *>(sep + d.sep_z3) + (t.e * g.nt3 + t.nt) * SEP_MASK;
+      t.eb = inv_exp(d);
     } else if (t.job == J_INV) {
       t.B = sep + d.sep_bi + ((long long)t.e * g.ntg + t.nt) * nk * SEP_BBLK;
+      t.eb = inv_exp(d);
     } else if (t.job == J_FWD) {
       t.B = sep + d.sep_bf + ((long long)t.e * (g.nqh / 32) + t.nt) * nk * SEP_BBLK;
     } else if (t.nt < g.nt3) {   // K
@@ -524,7 +565,7 @@ struct SepSrc {
       cnt = g.Pi - i0;
       dst = ws + it.a_off + (direct ? w.u1 : w.u3) + ((long long)(t.e * g.nS + t.nt / g.nti) * g.Pi + i0) * t.R + row;
     } else if (t.job == J_MID) {
-      cnt = 16;
+      cnt = 8;
       dst = ws + it.a_off + w.mom + ((long long)t.e * 3 * g.nqp + o0 - 32 * g.nt3) * t.R + row;
     } else if (t.job == J_INV) {
       cnt = g.Ng - o0;
@@ -550,7 +591,8 @@ __global__ void __launch_bounds__(SG_THREADS, 1)
 // ---------------------------------------------------------------- stage 2
 // Per (mode, column): the coefficients A_1, A_2 of the homogeneous part on the middle rows and the field
 // at the 4 gamma rows (+ the receiver row) from the 4 dense rows' transforms and the moments: a 6 x 6
-// real matrix per mode (36 FMAs a part), and where R has an imaginary part 20 more. CD: complex
+// real matrix per mode (36 FMAs a part, 18 where the ends are far apart for the mode), and where R has an
+// imaginary part 20 more. CD: complex
 // results (Sommerfeld AP or complex data). FP64-bound.
 template <bool CD, bool CIN>
 __device__ __forceinline__ void sep_modes_body(const Item &it, const SubDesc &d, const SepGeo &g, const SepWs &w,
@@ -576,15 +618,26 @@ __device__ __forceinline__ void sep_modes_body(const Item &it, const SubDesc &d,
     in[p][5] = row1 >= 0 ? mom[(long long)g.nqp * R1 + p * cp] : 0.0;
     m3[p] = rec && row1 >= 0 ? mom[2LL * g.nqp * R1 + p * cp] : 0.0;
   }
+  if (T[MT_FAR] != 0.0) {   // the two ends do not see each other: two 3 x 3 blocks
 #pragma unroll
-  for (int o = 0; o < 6; ++o)
+    for (int o = 0; o < 6; ++o) {
+      const int end = o < 2 ? o : (o - 2) >> 1, k0 = 2 * end;   // outputs A_1, A_2, gamma rows 0..3
 #pragma unroll
-    for (int p = 0; p < P; ++p) {
-      double v = T[MT_MAT + 6 * o] * in[p][0];
-#pragma unroll
-      for (int k = 1; k < 6; ++k) v = fma(T[MT_MAT + 6 * o + k], in[p][k], v);
-      out[p][o] = v;
+      for (int p = 0; p < P; ++p)
+        out[p][o] = fma(T[MT_MAT + 6 * o + k0], in[p][k0],
+                        fma(T[MT_MAT + 6 * o + k0 + 1], in[p][k0 + 1], T[MT_MAT + 6 * o + 4 + end] * in[p][4 + end]));
     }
+  } else {
+#pragma unroll
+    for (int o = 0; o < 6; ++o)
+#pragma unroll
+      for (int p = 0; p < P; ++p) {
+        double v = T[MT_MAT + 6 * o] * in[p][0];
+#pragma unroll
+        for (int k = 1; k < 6; ++k) v = fma(T[MT_MAT + 6 * o + k], in[p][k], v);
+        out[p][o] = v;
+      }
+  }
   if (CD && !CIN)
 #pragma unroll
     for (int o = 0; o < 6; ++o) out[1][o] = 0.0;
@@ -651,13 +704,12 @@ __device__ __forceinline__ void sep_out_body(const Item &it, const SubDesc &d, c
   const int cp = sep_pad128(it.ncols), R1 = sep_rows(d, J_MID, it.ncols, it.col0, CIN), R3 = (CD ? 2 : 1) * cp;
   const int row = CIN ? b : sep_row_of(d, it.col0, it.ncols, b);
   const int row1 = CIN ? b : row - sep_first34(d, it.col0, it.ncols);
-  const double sc = 2.0 / d.Nx;
   cplx v[4];
 #pragma unroll
   for (int k = 0; k < 4; ++k) {   // (class, output) or output
     const long long t = (long long)k * g.Pi + i;
     const double *p3 = ws + it.a_off + w.u3 + t * R3 + row, *p1 = ws + it.a_off + w.u1 + t * R1 + row1;
-    v[k] = cmk(sc * p3[0], CD ? sc * p3[cp] : 0.0);
+    v[k] = cmk(p3[0], CD ? p3[cp] : 0.0);
     if (row1 >= 0) {
       v[k].re += p1[0];
       if (CIN) v[k].im += p1[cp];
@@ -676,8 +728,7 @@ __device__ __forceinline__ void sep_out_body(const Item &it, const SubDesc &d, c
   }
 }
 
-// The full gamma rows and the receiver row: u(m) = (2/Nx) (U_0(m) + U_1(m)), u(Nx - m) = (2/Nx) (U_0(m) -
-// U_1(m)) from the two parities' sums over the folded columns. A block takes one row, 32 folded columns
+// The full gamma rows and the receiver row: u(m) = U_0(m) + U_1(m), u(Nx - m) = U_0(m) - U_1(m) from the two parities' sums over the folded columns. A block takes one row, 32 folded columns
 // m and 32 basis columns, turned through shared memory so that the loads run along the columns and
 // the stores along m.
 template <bool CD, bool CIN>
@@ -686,7 +737,7 @@ __device__ __forceinline__ void sep_rows_out_body(const Item &it, const SubDesc 
                                                   int slot, int mt, double2 (*sh)[32][33]) {
   const SepGeo g = sep_geo(d);
   const int cp = sep_pad128(it.ncols), parts = CD ? 2 : 1, R = sep_rows(d, J_INV, it.ncols, it.col0, CIN);
-  const double *ui = ws + it.a_off + sep_ws(d, it.ncols).ui, sc = 2.0 / d.Nx;
+  const double *ui = ws + it.a_off + sep_ws(d, it.ncols).ui;
   const int b = b0 + threadIdx.x;
   const int row = slot * parts * cp + (CIN || b >= it.ncols ? b : sep_row_of(d, it.col0, it.ncols, b));
   for (int k = threadIdx.y; k < 32; k += 8) {
@@ -698,8 +749,8 @@ __device__ __forceinline__ void sep_rows_out_body(const Item &it, const SubDesc 
       u1 = cmk(p1[0], CD ? p1[cp] : 0.0);
     }
     const cplx s = cadd(u0, u1), t = csub(u0, u1);
-    sh[0][k][threadIdx.x] = make_double2(sc * s.re, sc * s.im);
-    sh[1][k][threadIdx.x] = make_double2(sc * t.re, sc * t.im);
+    sh[0][k][threadIdx.x] = make_double2(s.re, s.im);
+    sh[1][k][threadIdx.x] = make_double2(t.re, t.im);
   }
   __syncthreads();
   const int W = d.Px + 2, m1 = g.mg + mt * 32 + (int)threadIdx.x;
@@ -781,8 +832,8 @@ cudaError_t launch_sep_tables(const mdp_plan *p, const SubDesc *ds, const double
   const int ns = (int)p->subs.size();
   for (int s0 = 0; s0 < ns; s0 += 65535) {   // subdomains per launch: a grid's y / z limit
     const unsigned n = (unsigned)std::min(65535, ns - s0);
-    k_sep_mode_tab<<<dim3(mq, n), 128, 0, st>>>(ds, s0, sep, entries);
-    k_full_modes<<<dim3(mq, n), 128, 0, st>>>(ds, s0, sep);
+    k_sep_mode_tab<<<dim3(4 * mq, n), 32, 0, st>>>(ds, s0, sep, entries);
+    k_full_modes<<<dim3(4 * mq, n), 32, 0, st>>>(ds, s0, sep);
     k_sep_phi<<<dim3(mq, mrow, n), 128, 0, st>>>(ds, s0, sep);
     if (mdist == 0) continue;   // no subdomain on the tensor cores
     k_sep_kd<<<dim3(mdist, n), 128, 0, st>>>(ds, s0, tab, sep);

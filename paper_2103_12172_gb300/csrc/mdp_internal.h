@@ -116,7 +116,7 @@ constexpr int FSW = 24;  // doubles per forward-sweep table row
 
 // ---- separable projection (kernels_sep.cu)
 constexpr int SEP_MTW = 72;               // doubles per mode of the mode table
-constexpr int SEP_MXW = 16;               // doubles per mode of the full-grid solve's table
+constexpr int SEP_MXW = 18;               // doubles per mode of the full-grid solve's table
 constexpr int SEP_ABLK = 7 * 128 * 16 * 2;  // bytes of A: 7 digits x 128 rows x 16 values of K, fp16
 constexpr int SEP_BBLK = 7 * 32 * 16 * 2;   // bytes of B: 7 digits x 32 outputs x 16 values of K
 constexpr int SEP_MODES_PER_BLOCK = 16;   // k_sep_modes
