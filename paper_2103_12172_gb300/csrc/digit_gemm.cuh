@@ -55,18 +55,28 @@ __device__ __forceinline__ long long fixed_of(double x, int E) {
 
 // A tile of 128 rows x 32 outputs: the digit blocks of its rows and outputs, consecutive in groups of 16
 // values of K, except that with nkj the B block of group kb is a Toeplitz one (nkj groups per source
-// column, ND blocks per column, output group ti); the masks of groups with nonzero digits (mb may be
-// null); the exponents of the rows and of the table.
+// column, ND blocks per column, output group ti); the mask of groups with nonzero digits; the exponents of the rows and of the table.
 struct DigitTile {
   const unsigned char *A, *B;
   int nkj, ND, ti;
-  const unsigned *ma, *mb;
+  unsigned m[SEP_MASK];      // groups of K with nonzero digits in the tile's rows and in its outputs
   const int *ex;
   int eb;
-  __device__ __forceinline__ unsigned mask(int wd) const { return mb ? ma[wd] & mb[wd] : ma[wd]; }
+  __device__ __forceinline__ void masks(const unsigned *ma, const unsigned *mb) {   // mb may be null
+    const uint4 *p = reinterpret_cast<const uint4 *>(ma);
+    uint4 a = p[0], b = p[1];
+    if (mb) {
+      const uint4 *r = reinterpret_cast<const uint4 *>(mb);
+      const uint4 c = r[0], e = r[1];
+      a.x &= c.x; a.y &= c.y; a.z &= c.z; a.w &= c.w;
+      b.x &= e.x; b.y &= e.y; b.z &= e.z; b.w &= e.w;
+    }
+    m[0] = a.x; m[1] = a.y; m[2] = a.z; m[3] = a.w; m[4] = b.x; m[5] = b.y; m[6] = b.z; m[7] = b.w;
+  }
   __device__ __forceinline__ int groups() const {
     int n = 0;
-    for (int wd = 0; wd < SEP_MASK; ++wd) n += __popc(mask(wd));
+#pragma unroll
+    for (int wd = 0; wd < SEP_MASK; ++wd) n += __popc(m[wd]);
     return n;
   }
 };
@@ -169,8 +179,9 @@ __device__ __forceinline__ void digit_gemm(const Src &src, int *status) {
         typename Src::Tile t;
         if (!src.tile(v, t)) continue;   // every warp skips it
         bool ok = true;
-        for (int wd = 0; wd < SEP_MASK && ok; ++wd)
-          for (unsigned bits = t.mask(wd); bits; bits &= bits - 1, ++gs) {
+#pragma unroll
+        for (int wd = 0; wd < SEP_MASK; ++wd)
+          for (unsigned bits = ok ? t.m[wd] : 0u; bits; bits &= bits - 1, ++gs) {
             const int kb = 32 * wd + __ffs(bits) - 1;
             const unsigned st = gs % SG_STAGES;
             if (gs >= SG_STAGES && !mbar_wait(smem_u32(&empty_bar[st]), (gs / SG_STAGES - 1) & 1u, &abort_sh)) { ok = false; break; }

@@ -20,55 +20,58 @@
 namespace mdp {
 
 // ---------------------------------------------------------------- k_extend
-// One thread per gamma node: the Chebyshev recurrences for T_j, T_j'', T_j'''' (with T', T'''
-// as intermediates) run once over j and serve every column of the owner side in the item.
-// Writes xi[g][c - col0] (real) for those columns; with grad also d xi / dk after G*ncols.
-__global__ void __launch_bounds__(128) k_extend(Batch bt, const SubDesc *subs, const double *tab, double *ws, int grad) {
+// One thread per gamma node: the recurrences for T_j and its first four derivatives along the side run
+// once over j and serve every column of the owner side in the item. Writes xi[g][c - col0] (real) for
+// those columns; with grad also d xi / dk after G*ncols. The extension is linear in psi, psi^(2), psi^(4) with
+// coefficients that depend on the node only, and the derivatives are carried per unit of arc length, so a
+// step is 14 FP64 instructions (22 with the terms formed one by one). Blocks of one warp: the few warps of a
+// call (a node each thread) share no SM's FP64 pipe.
+__global__ void __launch_bounds__(32) k_extend(Batch bt, const SubDesc *subs, const double *tab, double *ws, int grad) {
   Item it; int local;
   locate(bt, blockIdx.x, it, local);
   MDP_CHECK_ITEM(bt, subs, it, local, F_EXT);
   const SubDesc &d = subs[it.sub];
-  const int g = local * 128 + threadIdx.x;
+  const int g = local * 32 + threadIdx.x;
   if (g >= d.G) return;
   const double *geo = tab + d.geo_off + 4 * g;
   const int side = (int)geo[0];
   const double s = geo[1], rho = geo[2], L = geo[3];
   const int M = d.n_modes;
   const int baseD = (side - 1) * M, baseN = 4 * M + (side - 1) * M;
-  const int c0 = it.col0, c1 = it.col0 + it.ncols;
+  const int c0 = it.col0, c1 = it.col0 + it.ncols, nc = it.ncols;
   // j range needed: any j with baseD + j or baseN + j inside [c0, c1)
   int jmax = 0;
   if (c1 > baseD) jmax = max(jmax, min(M, c1 - baseD));
   if (c1 > baseN) jmax = max(jmax, min(M, c1 - baseN));
-  double *xi = ws + it.xi_off;
+  double *xi = ws + it.xi_off + (long long)g * nc, *dxi = xi + (long long)d.G * nc;
   const double k = d.k, k2 = k * k, k4 = k2 * k2;
-  const double sc2 = (2.0 / L) * (2.0 / L), sc4 = sc2 * sc2;
   const double a2 = 0.5 * rho * rho, a4 = a2 * a2 / 6.0, a3 = a2 * rho / 3.0;
+  // Dirichlet: psi + rho^2/2 (-psi^(2) - k^2 psi) + rho^4/24 (psi^(4) + 2 k^2 psi^(2) + k^4 psi)
+  const double d0 = fma(a4, k4, fma(-a2, k2, 1.0)), d2 = fma(2.0 * a4, k2, -a2);
+  // Neumann: rho psi + rho^3/6 (-psi^(2) - k^2 psi)
+  const double e0 = fma(-a3, k2, rho);
+  const double dk0 = fma(4.0 * a4 * k, k2, -2.0 * a2 * k), dk2 = 4.0 * a4 * k, ek0 = -2.0 * a3 * k;
+  const double sc = 2.0 / L, s2 = 2.0 * s, f1 = 2.0 * sc, f2 = 4.0 * sc, f3 = 6.0 * sc, f4 = 8.0 * sc;
   double t0 = 1.0, t1 = 0.0, t2 = 0.0, t3 = 0.0, t4 = 0.0;
   double p0 = 0.0, p1 = 0.0, p2 = 0.0, p3 = 0.0, p4 = 0.0;
-  const double s2 = 2.0 * s;
   for (int j = 0; j < jmax; ++j) {
-    const double psi = t0, psi2 = t2 * sc2, psi4 = t4 * sc4;
-    const double tt = fma(-k2, psi, -psi2);                // -psi'' - k^2 psi
     const int cD = baseD + j, cN = baseN + j;
     if (cD >= c0 && cD < c1) {
-      const double v4 = fma(k4, psi, fma(2.0 * k2, psi2, psi4));
-      xi[(long long)g * it.ncols + (cD - c0)] = fma(a4, v4, fma(a2, tt, psi));
-      if (grad) xi[(long long)d.G * it.ncols + (long long)g * it.ncols + (cD - c0)] =
-          fma(a2, -2.0 * k * psi, a4 * (4.0 * k * psi2 + 4.0 * k * k2 * psi));
+      xi[cD - c0] = fma(a4, t4, fma(d2, t2, d0 * t0));
+      if (grad) dxi[cD - c0] = fma(dk2, t2, dk0 * t0);
     }
     if (cN >= c0 && cN < c1) {
-      xi[(long long)g * it.ncols + (cN - c0)] = fma(a3, tt, rho * psi);
-      if (grad) xi[(long long)d.G * it.ncols + (long long)g * it.ncols + (cN - c0)] = a3 * (-2.0 * k * psi);
+      xi[cN - c0] = fma(-a3, t2, e0 * t0);
+      if (grad) dxi[cN - c0] = ek0 * t0;
     }
     double n0, n1, n2, n3, n4;
-    if (j == 0) { n0 = s; n1 = 1.0; n2 = 0.0; n3 = 0.0; n4 = 0.0; }
+    if (j == 0) { n0 = s; n1 = sc; n2 = 0.0; n3 = 0.0; n4 = 0.0; }
     else {
       n0 = fma(s2, t0, -p0);
-      n1 = fma(s2, t1, fma(2.0, t0, -p1));
-      n2 = fma(s2, t2, fma(4.0, t1, -p2));
-      n3 = fma(s2, t3, fma(6.0, t2, -p3));
-      n4 = fma(s2, t4, fma(8.0, t3, -p4));
+      n1 = fma(s2, t1, fma(f1, t0, -p1));
+      n2 = fma(s2, t2, fma(f2, t1, -p2));
+      n3 = fma(s2, t3, fma(f3, t2, -p3));
+      n4 = fma(s2, t4, fma(f4, t3, -p4));
     }
     p0 = t0; p1 = t1; p2 = t2; p3 = t3; p4 = t4;
     t0 = n0; t1 = n1; t2 = n2; t3 = n3; t4 = n4;
@@ -160,6 +163,109 @@ __global__ void __launch_bounds__(256) k_residual(Batch bt, const SubDesc *subs,
   if (GRAD) {
     st2(sb + 2 * ((long long)ring_index(d, n, m1) * nc + b), s1);
     if (m2 != m1) st2(sb + 2 * ((long long)ring_index(d, n, m2) * nc + b), s2);
+  }
+}
+
+// ---------------------------------------------------------------- k_ring
+// The ring residuals of basis columns for the separable solve, in k_residual's layout, only where they are
+// not zero by construction (sep_support in the operand cutting): a column's density lives on its own side,
+// so a column of side 1 or 2 has them on the two dense rows next to it, one of side 3 or 4 on the two ring
+// columns next to it and the ends of the dense rows. One thread per (unit, column); a unit is, for sides 1
+// and 2, a node pair (m, Nx - m) of both dense rows (x-centred; else a node of them), and for sides 3 and 4 a
+// middle row, or one of the 8 nodes at its end of the dense rows. k_residual evaluates all 9 neighbours
+// of every ring node for every column: 49 us for 4 x 257^2, 1024 columns, bound by instruction issue.
+__device__ __forceinline__ double side_density(const SubDesc &d, const Item &it, const double *ws, const double *tab, int b,
+                                               int side, int g) {
+  if (MDP_CHECKED && (g < 0 || g >= d.G || b < 0 || b >= it.ncols)) { flag_bounds(d.dstatus); return 0.0; }
+  // owners are 1.0 .. 4.0: their high words tell them apart without the FP64 pipe
+  const bool own = __double2hiint(tab[d.geo_off + 4 * g]) == __double2hiint((double)side);
+  return own ? ws[it.xi_off + (long long)g * it.ncols + b] : 0.0;
+}
+__global__ void __launch_bounds__(256) k_ring(Batch bt, const SubDesc *subs, const double *tab, double *ws) {
+  Item it; int local;
+  locate(bt, blockIdx.x, it, local);
+  MDP_CHECK_ITEM(bt, subs, it, local, F_RING);
+  const SubDesc &d = subs[it.sub];
+  const int nb = blocks_for(F_RING, d, it.ncols, it.col0);
+  {   // clear the K masks of the separable solve's operands
+    unsigned *mask = reinterpret_cast<unsigned *>(ws + it.a_off + sep_ws(d, it.ncols).mask);
+    const int n = sep_mask_words(it.ncols);
+    for (int i = local * 256 + threadIdx.y * 32 + threadIdx.x; i < n; i += 256 * nb) mask[i] = 0;
+  }
+  const int cb = (it.ncols + 31) >> 5;
+  const int b = (local % cb) * 32 + threadIdx.x, u = (local / cb) * 8 + threadIdx.y;
+  if (b >= it.ncols) return;
+  const int side = col_side(d, it.col0 + b);
+  const long long nc = it.ncols;
+  double *r = ws + it.r_off + b;
+  const double C0 = d.c0, C1 = d.c1, C2 = d.c2;
+  auto den = [&](int g) { return side_density(d, it, ws, tab, b, side, g); };
+  if (side <= 2) {
+    const int np = d.xsym ? d.Ph : d.Px;
+    if (u >= np) return;
+    const int W = d.Px + 2, base = side == 1 ? 0 : 2 * W + 4 * (d.Py - 2);
+    const int go = side == 1 ? base : base + W, gi = side == 1 ? base + W : base;   // outer, inner gamma row
+    // residuals at ring node m of the dense row at the side and of the next one
+    auto pair = [&](int m, double &r0, double &r1) {
+      const int k = m - (d.mlo - 1);   // gamma column of m
+      const double i0 = den(gi + k - 1), i1 = den(gi + k), i2 = den(gi + k + 1);
+      const double o0 = den(go + k - 1), o1 = den(go + k), o2 = den(go + k + 1);
+      const double is = i0 + i2;
+      r0 = fma(C0, i1, fma(C1, is + o1, C2 * (o0 + o2)));
+      r1 = fma(C1, i1, C2 * is);
+    };
+    const int ra = side == 1 ? 0 : 3, rb = side == 1 ? 1 : 2;   // dense row numbers
+    double a0, a1;
+    pair(d.mlo + u, a0, a1);
+    if (!d.xsym) {
+      const long long off[4] = {0, d.Px, 2LL * d.Px + 4 * (d.Py - 4), 3LL * d.Px + 4 * (d.Py - 4)};
+      r[(off[ra] + u) * nc] = a0;
+      r[(off[rb] + u) * nc] = a1;
+      return;
+    }
+    double b0 = 0.0, b1 = 0.0;
+    if (2 * (d.mlo + u) != d.Nx) pair(d.Nx - (d.mlo + u), b0, b1);
+    double *pa = r + ((long long)ra * 2 * d.Ph + 2 * u) * nc, *pb = r + ((long long)rb * 2 * d.Ph + 2 * u) * nc;
+    pa[0] = a0 + b0; pa[nc] = a0 - b0;
+    pb[0] = a1 + b1; pb[nc] = a1 - b1;
+    return;
+  }
+  if (u < d.Py - 4) {   // middle row n = nlo + 2 + u: gamma columns (outer, inner) of rows n - 1, n, n + 1
+    const int g = 2 * (d.Px + 2) + 4 * u + (side == 3 ? 0 : 2), o = side == 3 ? 0 : 1, i = 1 - o;
+    const double o0 = den(g + o), o1 = den(g + 4 + o), o2 = den(g + 8 + o);
+    const double i0 = den(g + i), i1 = den(g + 4 + i), i2 = den(g + 8 + i), is = i0 + i2;
+    const double r0 = fma(C0, i1, fma(C1, is + o1, C2 * (o0 + o2))), r1 = fma(C1, i1, C2 * is);
+    if (d.xsym) {
+      double *p = r + (8LL * d.Ph + 4 * u) * nc;
+      p[0] = r0; p[nc] = side == 3 ? r0 : -r0;
+      p[2 * nc] = r1; p[3 * nc] = side == 3 ? r1 : -r1;
+    } else {
+      double *p = r + (2LL * d.Px + 4 * u) * nc;
+      p[(side == 3 ? 0 : 3) * nc] = r0;
+      p[(side == 3 ? 1 : 2) * nc] = r1;
+    }
+    return;
+  }
+  const int t = u - (d.Py - 4);
+  if (t >= 8) return;
+  const int rr = t >> 1, k = t & 1;   // dense row, node counted from the side
+  const int n = rr == 0 ? d.nlo : rr == 1 ? d.nlo + 1 : rr == 2 ? d.nhi - 1 : d.nhi;
+  const int m = side == 3 ? d.mlo + k : d.mhi - k;
+  double v = 0.0;
+#pragma unroll
+  for (int dn = -1; dn <= 1; ++dn)
+#pragma unroll
+    for (int dm = -1; dm <= 1; ++dm) {
+      const int g = gamma_index(d, n + dn, m + dm);
+      const int nbr = (dn != 0) + (dm != 0);
+      if (g >= 0) v = fma(nbr == 0 ? C0 : nbr == 1 ? C1 : C2, den(g), v);
+    }
+  if (d.xsym) {
+    double *p = r + ((long long)rr * 2 * d.Ph + 2 * k) * nc;
+    p[0] = v; p[nc] = side == 3 ? v : -v;
+  } else {
+    const long long rb = (long long)rr * d.Px + (rr < 2 ? 0 : 4 * (d.Py - 4));
+    r[(rb + m - d.mlo) * nc] = v;
   }
 }
 
@@ -1474,7 +1580,7 @@ cudaError_t launch_basis_densities(const mdp_plan *p, int sub, int col0, int nco
     std::memset(&b, 0, sizeof b);
     b.n_items = 1; b.one = it; b.total_blocks = blocks_for(F_EXT, d, it.ncols, it.col0);
     set_bounds(p, b, (long long)ncols * d.G, false);
-    k_extend<<<dim3((unsigned)b.total_blocks), 128, 0, st>>>(b, p->d_subs, p->d_tables, p->d_ws, 0);
+    k_extend<<<dim3((unsigned)b.total_blocks), 32, 0, st>>>(b, p->d_subs, p->d_tables, p->d_ws, 0);
     const long long n = (long long)it.ncols * d.G;
     k_basis_out<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(it, p->d_subs, p->d_tables, p->d_ws,
                                                               out + (long long)c * d.G);
@@ -1526,9 +1632,11 @@ cudaError_t launch_project(mdp_plan *p, const Batch *fb, int out_kind, const dou
     }                                             \
   } while (0)
 #define MDP_LAUNCH(fam, ...) MDP_LAUNCH_AS(fam, fam, __VA_ARGS__)
-  if (basis) MDP_LAUNCH(F_EXT, k_extend<<<grid1(fb[F_EXT].total_blocks), 128, 0, st>>>(fb[F_EXT], ds, tab, ws, 0));
-  if (basis) MDP_LAUNCH(F_RES, k_residual<false, false><<<grid1(fb[F_RES].total_blocks), b8, 0, st>>>(fb[F_RES], ds, tab, ws, xi_user));
-  else MDP_LAUNCH(F_RES, k_residual<true, false><<<grid1(fb[F_RES].total_blocks), b8, 0, st>>>(fb[F_RES], ds, tab, ws, xi_user));
+  if (basis) MDP_LAUNCH(F_EXT, k_extend<<<grid1(fb[F_EXT].total_blocks), 32, 0, st>>>(fb[F_EXT], ds, tab, ws, 0));
+  if (basis) {
+    MDP_LAUNCH_AS(F_RING, F_RES, k_ring<<<grid1(fb[F_RING].total_blocks), b8, 0, st>>>(fb[F_RING], ds, tab, ws));
+    MDP_LAUNCH_AS(F_PRES, F_RES, k_residual<false, false><<<grid1(fb[F_PRES].total_blocks), b8, 0, st>>>(fb[F_PRES], ds, tab, ws, xi_user));
+  } else MDP_LAUNCH(F_RES, k_residual<true, false><<<grid1(fb[F_RES].total_blocks), b8, 0, st>>>(fb[F_RES], ds, tab, ws, xi_user));
   if (basis) MDP_LAUNCH_AS(F_PROWS, F_FROWS, k_fwd_rows<false><<<grid1(fb[F_PROWS].total_blocks), b8, p->fft_smem, st>>>(fb[F_PROWS], ds, tab, ws));
   else MDP_LAUNCH_AS(F_PROWS, F_FROWS, k_fwd_rows<true><<<grid1(fb[F_PROWS].total_blocks), b8, p->fft_smem, st>>>(fb[F_PROWS], ds, tab, ws));
   cudaError_t e = launch_sep_project(p, fb, out_kind, xi_user, out, out_rec, st);
@@ -1560,7 +1668,7 @@ cudaError_t launch_adjoint(mdp_plan *p, const Batch *fb, int out_kind, const dou
   double *ws = p->d_ws;
   const dim3 b8(32, 8), btri(32, TRI_WARPS);
   if (grad_k) {  // forward recompute with every mode-space row kept, and the k-derivative sources
-    if (basis) MDP_LAUNCH(F_EXT, k_extend<<<grid1(fb[F_EXT].total_blocks), 128, 0, st>>>(fb[F_EXT], ds, tab, ws, 1));
+    if (basis) MDP_LAUNCH(F_EXT, k_extend<<<grid1(fb[F_EXT].total_blocks), 32, 0, st>>>(fb[F_EXT], ds, tab, ws, 1));
     if (basis) MDP_LAUNCH(F_RES, k_residual<false, true><<<grid1(fb[F_RES].total_blocks), b8, 0, st>>>(fb[F_RES], ds, tab, ws, xi_user));
     else MDP_LAUNCH(F_RES, k_residual<true, true><<<grid1(fb[F_RES].total_blocks), b8, 0, st>>>(fb[F_RES], ds, tab, ws, xi_user));
     if (basis) MDP_LAUNCH(F_FROWS, k_fwd_rows<false><<<grid1(fb[F_FROWS].total_blocks), b8, p->fft_smem, st>>>(fb[F_FROWS], ds, tab, ws));

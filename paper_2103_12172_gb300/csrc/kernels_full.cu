@@ -18,8 +18,10 @@ namespace cg = cooperative_groups;
 namespace mdp {
 
 // per mode: kind, lambda (with its sign), kappa(0) = c, c (1 - lambda^2), sign, R11, R12, R22, F, and of the
-// rotation of kinds 0, 1: -+s^2 (s = sin or sinh theta), C(1), C and S at row 0
-enum { MX_KIND = 0, MX_LAM, MX_C, MX_C1, MX_SG, MX_R = 6, MX_F = 12, MX_SS, MX_CS1, MX_CS0 };   // CS0: 2
+// rotation of kinds 0, 1: -+s^2 (s = sin or sinh theta), C(1), C and S at row 0;
+// 1 / lambda, 1 / c, log2 |lambda|
+enum { MX_KIND = 0, MX_LAM, MX_C, MX_C1, MX_SG, MX_R = 6, MX_F = 12, MX_SS, MX_CS1, MX_CS0,   // CS0: 2
+       MX_LI = 17, MX_CI, MX_L2 };
 
 // The table of the solve along y, over all rows 0 .. N: evanescent modes phi = (lambda^n, lambda^(N-n)),
 // the others C and S about the middle row.
@@ -47,6 +49,9 @@ __global__ void k_full_modes(const SubDesc *subs, int s0, unsigned char *sep) {
   T[MX_KIND] = m.kind; T[MX_LAM] = lam; T[MX_C] = c;
   T[MX_C1] = -c * expm1(-2.0 * m.th);
   T[MX_SG] = m.sg;
+  T[MX_LI] = m.sg * exp(m.th);
+  T[MX_CI] = -2.0 * m.a * sinh(m.th);
+  T[MX_L2] = -m.th * 1.4426950408889634;
   T[MX_R] = R11.re; T[MX_R + 1] = R11.im; T[MX_R + 2] = R12.re; T[MX_R + 3] = R12.im;
   T[MX_R + 4] = R22.re; T[MX_R + 5] = R22.im;
   T[MX_F] = 1.0 / (2.0 * m.a);
@@ -138,8 +143,7 @@ struct FullSrc {
     t.B = p.sep + (INV ? p.d.sep_xi : p.d.sep_xf) + ((long long)t.e * nt + t.nt) * nk * SEP_BBLK;
     t.nkj = t.ND = t.ti = 0;
     t.eb = INV ? inv_exp(p.d) : 0;
-    t.ma = reinterpret_cast<const unsigned *>(p.ws + p.w.mask) + ((INV ? 2 * nm : 0) + tr) * SEP_MASK;
-    t.mb = nullptr;
+    t.masks(reinterpret_cast<const unsigned *>(p.ws + p.w.mask) + ((INV ? 2 * nm : 0) + tr) * SEP_MASK, nullptr);
     t.ex = reinterpret_cast<const int *>(p.ws + p.w.ex) + tr * 128;
     return true;
   }
@@ -281,8 +285,8 @@ __global__ void __cluster_dims__(1, 1, FULL_Y_CTAS) __launch_bounds__(32 * FULL_
       }
     }
   }
-  exchange(a, ytop);
   const double c = T[MX_C], cc = T[MX_C1];
+  exchange(cc * a, ytop);
   // the top row takes x = c y there: as if the row above held c lambda y. Empty last segments pass on.
   const int last = (Nt - 1) / seg;
   const double yt = sh1[last * 32 + lane];
@@ -290,26 +294,26 @@ __global__ void __cluster_dims__(1, 1, FULL_Y_CTAS) __launch_bounds__(32 * FULL_
   for (int k = last; k >= 0; --k) {
     if (k == s) mine = x;
     const int len = min(seg, Nt - k * seg);
-    x = fma(len == seg ? ll : ipow(lam, len), x, cc * sh0[k * 32 + lane]);
+    x = fma(len == seg ? ll : ipow(lam, len), x, sh0[k * 32 + lane]);
   }
   // moments of phi = (lambda^n, lambda^(N-n)) from the two ends: c M_1 is x continued to row 0, M_2 is y at row N
   const double e1 = d.nfirst ? lam : 1.0;
-  const cplx M1 = both(kind == 2 ? e1 * x / c : 0.0), M2 = both(e1 * yt);
+  const cplx M1 = both(kind == 2 ? e1 * x * T[MX_CI] : 0.0), M2 = both(e1 * yt);
   if (live && kind == 2) {
     const double A = part(cadd(cmul(R11, M1), cmul(R12, M2))), B = part(cadd(cmul(R12, M1), cmul(R22, M2)));
     const int nt = i1 - 1 + d.nfirst;   // grid row of the segment's last row
-    double pa = i1 > i0 ? ipow(lam, i0 + d.nfirst) : 0.0, pb = i1 > i0 ? ipow(lam, N - nt) : 0.0;
+    const float l2 = (float)T[MX_L2];
     x = mine;
     // 2^-90 of the reflected waves is zero to working precision: the rows far from both ends
-    if (__all_sync(__activemask(), fabs(pa) < 0x1p-90 && fabs(pb) < 0x1p-90)) {
+    if (__all_sync(__activemask(), l2 * (i0 + d.nfirst) < -90.0f && l2 * (N - nt) < -90.0f)) {
 #pragma unroll 4
       for (int i = i1 - 1; i >= i0; --i) {
         x = fma(lam, x, cc * f[32 * i]);
         fg[i * gstep] = x;
       }
     } else {
-      const double li = 1.0 / lam;
-      pa = i1 > i0 ? ipow(lam, nt) : 0.0;
+      const double li = T[MX_LI];
+      double pa = i1 > i0 ? ipow(lam, nt) : 0.0, pb = i1 > i0 ? ipow(lam, N - nt) : 0.0;
 #pragma unroll 4
       for (int i = i1 - 1; i >= i0; --i) {
         x = fma(lam, x, cc * f[32 * i]);
@@ -365,9 +369,9 @@ cudaError_t launch_full_solve(const mdp_plan *p, int sub, int nrhs, const double
   for (int r0 = 0; r0 < nrhs; r0 += chunk) {
     const int nr = std::min(chunk, nrhs - r0);
     const FullWs w = full_ws(d, nr);
-    // segments along y, a multiple of the cluster's 4: of about 32 rows where the blocks fill the chip (each
-    // segment has a fixed cost of some 100 FP64 instructions), else of 16
-    const int rows = nr * (w.ldf / 16) >= 2 * p->n_sm ? 32 : 16;
+    // segments along y, a multiple of the cluster's 4: of about 64 rows where the blocks fill the chip (each
+    // segment has a fixed cost of some 60 FP64 instructions), else of 16
+    const int rows = nr * (w.ldf / 16) >= 2 * p->n_sm ? 64 : 16;
     const int nw = std::min(FULL_Y_WARPS, std::max(1, (d.Nt + rows * FULL_Y_CTAS - 1) / (rows * FULL_Y_CTAS)));
     const int seg = (d.Nt + nw * FULL_Y_CTAS - 1) / (nw * FULL_Y_CTAS);
     const int ysm = ((2 + 2 * FULL_Y_CTAS) * nw + nw * seg) * 256;

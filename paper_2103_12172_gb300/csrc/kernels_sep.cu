@@ -423,21 +423,27 @@ __device__ __forceinline__ void sep_cut_body(const Item &it, const SubDesc &d, d
   }
   const double *src = JOB == J_SYN ? ws + it.a_off + w.aeff + (long long)e * 2 * g.nqp * R + row
                       : JOB == J_INV ? ws + it.y_off : ws + it.r_off;
+  // basis columns: what k_ring leaves unwritten is zero (side: 0..3)
+  const int side = CIN || !live ? 0 : col_side(d, it.col0 + col) - 1;
   auto ring = [&](long long slot) { return CIN ? src[2 * (slot * nc + col) + part] : src[slot * nc + col]; };
   auto value = [&](int k) -> double {
     if (!live) return 0.0;
     if (JOB == J_MID) {
       const int c = k / (16 * g.nkj), j = k - c * 16 * g.nkj;
       if (j >= g.Pj) return 0.0;
+      if (!CIN && !d.xsym && (c < 2) != (side == 2)) return 0.0;
       return ring(d.xsym ? 8LL * d.Ph + 4 * j + 2 * c + e : 2LL * d.Px + 4 * j + c);
     }
     if (JOB == J_FWD) {
       if (k >= g.Kf) return 0.0;
+      if (!CIN && side < 2 && (rr < 2) != (side == 0)) return 0.0;
+      if (!CIN && side >= 2 && d.xsym && k > 1) return 0.0;
       if (d.xsym) return ring((long long)rr * 2 * d.Ph + 2 * k + e);
       const long long rb = rr < 2 ? (long long)rr * d.Px : (long long)rr * d.Px + 4 * (d.Py - 4);
       const int m = g.mf + k, m2 = d.Nx - m;
-      const double a = m >= d.mlo && m <= d.mhi ? ring(rb + m - d.mlo) : 0.0;
-      const double b = m2 != m && m2 >= d.mlo && m2 <= d.mhi ? ring(rb + m2 - d.mlo) : 0.0;
+      const int lo = !CIN && side == 3 ? d.mhi - 1 : d.mlo, hi = !CIN && side == 2 ? d.mlo + 1 : d.mhi;   // the row's support
+      const double a = m >= lo && m <= hi ? ring(rb + m - d.mlo) : 0.0;
+      const double b = m2 != m && m2 >= lo && m2 <= hi ? ring(rb + m2 - d.mlo) : 0.0;
       return e == 0 ? a + b : a - b;
     }
     if (JOB == J_SYN) return sep_mode(d, e, k % g.nqp) <= d.Nq ? src[(long long)k * R] : 0.0;
@@ -528,12 +534,12 @@ struct SepSrc {
     const int tr = t.e * (t.R / 128) + t.mt;   // tile row
     t.A = reinterpret_cast<const unsigned char *>(ws + it.a_off + w.a[t.job]) + (long long)tr * nk * SEP_ABLK;
     t.ex = reinterpret_cast<const int *>(ws + it.a_off + w.ex[t.job]) + tr * 128;
-    t.ma = reinterpret_cast<const unsigned *>(ws + it.a_off + w.mask) + sep_mask_of(t.job, it.ncols) + tr * SEP_MASK;
-    t.mb = nullptr;
+    const unsigned *ma = reinterpret_cast<const unsigned *>(ws + it.a_off + w.mask) + sep_mask_of(t.job, it.ncols) + tr * SEP_MASK;
+    const unsigned *mb = nullptr;
     t.eb = t.nkj = t.ND = t.ti = 0;
     if (t.job == J_SYN) {
       t.B = sep + d.sep_b3 + ((long long)t.e * g.nt3 + t.nt) * nk * SEP_BBLK;
-      t.mb = reinterpret_cast<const unsigned *>(sep + d.sep_z3) + (t.e * g.nt3 + t.nt) * SEP_MASK;
+      mb = reinterpret_cast<const unsigned *>(sep + d.sep_z3) + (t.e * g.nt3 + t.nt) * SEP_MASK;
       t.eb = inv_exp(d);
     } else if (t.job == J_INV) {
       t.B = sep + d.sep_bi + ((long long)t.e * g.ntg + t.nt) * nk * SEP_BBLK;
@@ -548,8 +554,9 @@ struct SepSrc {
     } else {                     // moments
       const int mt = t.e * (3 * g.nqp / 32) + t.nt - g.nt3;
       t.B = sep + d.sep_mb + (long long)mt * nk * SEP_BBLK;
-      t.mb = reinterpret_cast<const unsigned *>(sep + d.sep_zm) + mt * SEP_MASK;
+      mb = reinterpret_cast<const unsigned *>(sep + d.sep_zm) + mt * SEP_MASK;
     }
+    t.masks(ma, mb);
     return true;
   }
   __device__ __forceinline__ void dest(const Tile &t, int r, int o, double *&dst, long long &step, int &cnt) const {

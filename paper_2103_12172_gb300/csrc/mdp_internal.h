@@ -116,7 +116,7 @@ constexpr int FSW = 24;  // doubles per forward-sweep table row
 
 // ---- separable projection (kernels_sep.cu)
 constexpr int SEP_MTW = 72;               // doubles per mode of the mode table
-constexpr int SEP_MXW = 18;               // doubles per mode of the full-grid solve's table
+constexpr int SEP_MXW = 20;               // doubles per mode of the full-grid solve's table
 constexpr int SEP_ABLK = 7 * 128 * 16 * 2;  // bytes of A: 7 digits x 128 rows x 16 values of K, fp16
 constexpr int SEP_BBLK = 7 * 32 * 16 * 2;   // bytes of B: 7 digits x 32 outputs x 16 values of K
 constexpr int SEP_MODES_PER_BLOCK = 16;   // k_sep_modes
@@ -441,11 +441,12 @@ inline void set_bounds(const mdp_plan *p, Batch &b, long long out_n, bool grad) 
 
 // kernel families (each has its own block decomposition of an item); F_A* are the adjoint's. F_TRI is
 // the gradient pass's full sweep, F_PTRI the projection's (subdomains without the separable solve),
-// F_FROWS and F_PROWS likewise for the dense rows' transform; F_C* cut operands, F_G* contract (stage 1
+// F_FROWS and F_PROWS likewise for the dense rows' transform, F_RES, F_PRES and F_RING (basis columns of the
+// separable solve) for the ring residuals; F_C* cut operands, F_G* contract (stage 1
 // and 3, B: basis columns, U: user densities; F_TCOLS is stage 3 for basis columns), F_SMODE and F_SOUT
 // are the separable solve's other kernels.
 enum Fam { F_EXT = 0, F_RES, F_FROWS, F_TRI, F_IROWS, F_ICOLS, F_AFWD, F_ATRI, F_ARING, F_ARINGC, F_AGAM, F_IREC,
-           F_ACOLS, F_TCOLS, F_ATCOLS, F_PTRI, F_C1B, F_C1U, F_G1B, F_G1U, F_SMODE, F_C3B, F_C3U, F_G3U, F_SOUT, F_PROWS, NFAM };
+           F_ACOLS, F_TCOLS, F_ATCOLS, F_PTRI, F_C1B, F_C1U, F_G1B, F_G1U, F_SMODE, F_C3B, F_C3U, F_G3U, F_SOUT, F_PROWS, F_RING, F_PRES, NFAM };
 static_assert(NFAM <= 32, "per-family event lists of mdp_plan");
 
 // Blocks of kernel family f for an item of ncols columns: 32 columns (x) times BY tasks (y).
@@ -453,8 +454,14 @@ static_assert(NFAM <= 32, "per-family event lists of mdp_plan");
 inline __host__ __device__ int blocks_for(int f, const SubDesc &d, int ncols, int col0) {
   const int cb = (ncols + 31) / 32;
   switch (f) {
-    case F_EXT: return (d.G + 127) / 128;
+    case F_EXT: return (d.G + 31) / 32;
     case F_RES: return cb * (((d.xsym ? 4 * d.Ph + 2 * (d.Py - 4) : d.R) + 7) / 8);
+    case F_PRES: return d.tc_cols ? 0 : blocks_for(F_RES, d, ncols, col0);
+    case F_RING: {
+      if (!d.tc_cols) return 0;
+      const int dense = d.xsym ? d.Ph : d.Px, side = d.Py + 4;
+      return cb * (((dense > side ? dense : side) + 7) / 8);
+    }
     case F_FROWS:
       if (d.rows_fft) return 4 * ((ncols + d.fpb - 1) / d.fpb);
       return cb * ((d.Nx / 2 + 7) / 8);

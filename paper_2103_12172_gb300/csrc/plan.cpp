@@ -25,7 +25,7 @@ const char *fam_name(int f) {
                                     "k_adj_rows", "k_adj_tri", "k_adj_ring_rows", "k_adj_ring_cols", "k_adj_gamma",
                                     "k_inv_rec", "k_adj_cols", "k_inv_cols_tc", "k_adj_ring_cols_tc", "k_tri(projection)",
                                     "k_sep_cut1", "k_sep_cut1(user)", "k_sep_gemm1", "k_sep_gemm1(user)", "k_sep_modes",
-                                    "k_sep_cut3", "k_sep_cut3(user)", "k_inv_cols_tc(user)", "k_sep_out", "k_fwd_rows(projection)"};
+                                    "k_sep_cut3", "k_sep_cut3(user)", "k_inv_cols_tc(user)", "k_sep_out", "k_fwd_rows(projection)", "k_ring", "k_residual(projection)"};
   return (f >= 0 && f < NFAM) ? names[f] : "?";
 }
 
