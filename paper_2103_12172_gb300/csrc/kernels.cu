@@ -1370,7 +1370,7 @@ __global__ void k_full_inv(const SubDesc *subs, int sub, const double *tab, cons
 cudaError_t launch_solve(const mdp_plan *p, int sub, int nrhs, const double2 *g, double2 *u, int adjoint,
                          cudaStream_t st) {
   const SubDesc &d = p->subs[sub].d;
-  if (!adjoint && d.tc_cols) return launch_full_solve(p, sub, nrhs, g, u, st);
+  if (!adjoint && d.tc_cols && full_solve_fits(d)) return launch_full_solve(p, sub, nrhs, g, u, st);
   const long long per = (long long)d.Nq * d.Nt * 2;
   long long chunk = p->ws_doubles / per;
   if (chunk < 1) return cudaErrorMemoryAllocation;

@@ -358,6 +358,14 @@ cudaError_t set_full_kernel_attributes() {
   return e;
 }
 
+// k_full_y keeps a quarter of the rows of 32 columns in a CTA's shared memory (157 KB at 2459 rows); above some
+// 3500 rows they do not fit and the solve goes by the factors.
+static int full_y_smem(int nw, int seg) { return ((2 + 2 * FULL_Y_CTAS) * nw + nw * seg) * 256; }
+bool full_solve_fits(const SubDesc &d) {
+  const int nw = FULL_Y_WARPS;   // the widest segments' and the most warps' need
+  return full_y_smem(nw, (d.Nt + nw * FULL_Y_CTAS - 1) / (nw * FULL_Y_CTAS) + 1) <= FULL_Y_SMEM;
+}
+
 cudaError_t launch_full_solve(const mdp_plan *p, int sub, int nrhs, const double2 *g, double2 *u, cudaStream_t st) {
   const SubDesc &d = p->subs[sub].d;
   const SepGeo geo = sep_geo(d);
@@ -374,7 +382,7 @@ cudaError_t launch_full_solve(const mdp_plan *p, int sub, int nrhs, const double
     const int rows = nr * (w.ldf / 16) >= 2 * p->n_sm ? 64 : 16;
     const int nw = std::min(FULL_Y_WARPS, std::max(1, (d.Nt + rows * FULL_Y_CTAS - 1) / (rows * FULL_Y_CTAS)));
     const int seg = (d.Nt + nw * FULL_Y_CTAS - 1) / (nw * FULL_Y_CTAS);
-    const int ysm = ((2 + 2 * FULL_Y_CTAS) * nw + nw * seg) * 256;
+    const int ysm = full_y_smem(nw, seg);
     const double2 *gc = g + (long long)r0 * d.nx * d.ny;
     double2 *uc = u + (long long)r0 * d.nx * d.ny;
     auto gemm_grid = [&](int nt) { return dim3((unsigned)std::min(p->n_sm, 2 * (w.R / 128) * nt)); };

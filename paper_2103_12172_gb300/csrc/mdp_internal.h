@@ -581,6 +581,7 @@ cudaError_t launch_source_terms(mdp_plan *p, int sub, const double2 *f, const do
                                 cudaStream_t st);
 cudaError_t launch_basis_densities(const mdp_plan *p, int sub, int col0, int ncols, double2 *out, cudaStream_t st);
 // the full-grid solve through the separable Green's function (subdomains with tc_cols; kernels_full.cu)
+bool full_solve_fits(const SubDesc &d);   // the grid has no more rows than the separable full-grid solve takes
 cudaError_t launch_full_solve(const mdp_plan *p, int sub, int nrhs, const double2 *g, double2 *u, cudaStream_t st);
 cudaError_t set_full_kernel_attributes();
 __global__ void k_full_modes(const SubDesc *subs, int s0, unsigned char *sep);

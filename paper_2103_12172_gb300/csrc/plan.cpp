@@ -74,7 +74,10 @@ static mdp_status geometry(const mdp_subdomain &in, HostSub &hs, unsigned flags,
   {
     const char *tc = std::getenv("MDP_TC_COLS");
     const bool on = !(flags & MDP_PLAN_FP64_COLS) && !(tc && tc[0] == '0' && tc[1] == 0);
-    d.tc_cols = on && (d.xsym ? d.Nq <= 2047 : d.Nq <= 1023);
+    // the mask of a tile's groups of K holds 256 of them, which K of the middle rows (2 or 4 columns of up
+    // to Py - 2 rows) has to fit
+    d.tc_cols = on && (d.xsym ? d.Nq <= 2047 : d.Nq <= 1023) &&
+                (d.xsym ? 2 : 4) * ((d.Py - 2 + 15) / 16) <= 32 * SEP_MASK;
   }
   d.nfirst = d.cplx ? 0 : 1;
   d.Nt = d.cplx ? in.ny : in.ny - 2;

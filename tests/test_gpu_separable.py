@@ -108,3 +108,28 @@ def test_full_grid_solves_in_passes(mdp):
     assert torch.equal(plan.solve(0, g), one)
     plan.solve(0, g, out=g)
     assert torch.equal(g, one)
+
+
+def tall(ny, low=False):
+    """A grid of 33 x ny nodes; the subdomain takes ten twelfths of its height, or (low) half."""
+    h = 1.2 / 32
+    height = h * (ny - 1)
+    y0, y1 = (0.25, 0.75) if low else (0.1, 0.9)
+    return W.Subdomain(0.0, 1.0, 0.0, (y1 - y0) * height, -0.1, -y0 * height, h, 33, ny, 8.0, W.AP_DIRX_SOMMY, 1)
+
+
+@pytest.mark.parametrize("sub", [tall(2561), tall(2564), tall(2600), tall(3480, True), tall(3600, True)],
+                         ids=["n2561", "n2564", "n2600", "low3480", "low3600"])
+def test_tall_grids_around_the_limits_of_the_separable_solve(mdp, sub):
+    """The operand masks hold 256 groups of 16 rows and columns, the solve along y some 3500 rows: on either
+    side of both limits the columns and the full-grid solves are those of the sweeps. Bar: the sweeps'
+    own error at 3600 rows (1e-12 to 1e-11 at 1025), 1e-9."""
+    plan, ref = mdp.Plan([sub]), mdp.Plan([sub], fp64_cols=True)
+    G, nc, _, _ = plan.layout(0)
+    a, b = (p.project().view(nc, G).cpu().numpy() for p in (plan, ref))
+    plan.status()
+    assert rel_col_err(a, b) < 1e-9
+    g = torch.from_numpy(W.random_complex((2, sub.ny, sub.nx), seed=11)).cuda()
+    a, b = (p.solve(0, g).view(2, -1).cpu().numpy() for p in (plan, ref))
+    plan.status()
+    assert rel_col_err(a, b) < 1e-9
