@@ -34,6 +34,8 @@ void free_device(mdp_plan *p) {
   cudaFree(p->d_piv);
   cudaFree(p->d_sep);
   cudaFree(p->alt_sep);
+  cudaFree(p->d_adj);
+  p->d_adj = nullptr;
   p->d_sep = p->alt_sep = nullptr;
   cudaFree(p->d_ws);
   cudaFree(p->d_status);
@@ -150,7 +152,7 @@ mdp_status alloc_device(mdp_plan *p) {
       // then by mode group (low modes first: the propagating modes carry the complex rows), then
       // item, then column block
       std::vector<int> order;
-      for (const Fam f : {F_TRI, F_ATRI, F_PTRI}) {
+      for (const Fam f : {F_TRI, F_ATRI}) {
         const int *pt = pre.data() + (size_t)f * (n + 1);
         std::vector<std::array<int, 4>> keys;
         keys.reserve(pt[n]);
@@ -180,10 +182,7 @@ void wave_batches(const mdp_plan *p, size_t w, Batch *fb, int sc) {
     b.items = p->d_items[sc][w];
     b.prefix = p->d_prefix[sc][w] + (size_t)f * (n + 1);
     b.order = f == F_TRI ? p->d_order[sc][w]
-              : f == F_ATRI || f == F_PTRI
-                  ? p->d_order[sc][w] + p->h_prefix[sc][w][(size_t)F_TRI * (n + 1) + n] +
-                        (f == F_PTRI ? p->h_prefix[sc][w][(size_t)F_ATRI * (n + 1) + n] : 0)
-                  : nullptr;
+              : f == F_ATRI ? p->d_order[sc][w] + p->h_prefix[sc][w][(size_t)F_TRI * (n + 1) + n] : nullptr;
     b.n_items = n;
     b.total_blocks = p->h_prefix[sc][w][(size_t)f * (n + 1) + n];
     set_bounds(p, b, p->out_size, sc == S_GRAD);
@@ -221,10 +220,42 @@ cudaError_t end_use(mdp_plan *p, cudaStream_t st) {
   p->used_rec[p->set] = true;
   return cudaEventRecord(p->used_ev[p->set], st);
 }
+
+// The gradient tables follow the wavenumbers only where a gradient is asked for: allocated by the first such
+// call, rebuilt by the first after a change. In a capture they are always rebuilt, so that a replay
+// follows the tables that it finds (and the allocation is no stream operation).
+cudaError_t ensure_adj_tables(mdp_plan *p, cudaStream_t st) {
+  if (p->adj_bytes == 0) return cudaSuccess;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  cudaError_t e = cudaStreamIsCapturing(st, &cap);
+  if (e != cudaSuccess) return e;
+  if (!p->d_adj) {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    e = cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e != cudaSuccess) return e;
+    const cudaError_t m = cudaMalloc((void **)&p->d_adj, (size_t)p->adj_bytes);
+    e = cudaThreadExchangeStreamCaptureMode(&mode);
+    if (m != cudaSuccess || e != cudaSuccess) return m != cudaSuccess ? m : e;
+    p->adj_sines = false;
+    p->adj_stale = true;
+  }
+  const bool live = cap == cudaStreamCaptureStatusNone;
+  if (!p->adj_sines || !live) {
+    e = launch_adj_sines(p, st);
+    if (e != cudaSuccess) return e;
+    if (live) p->adj_sines = true;
+  }
+  if (p->adj_stale || !live) {
+    e = launch_adj_tables(p, st);
+    if (e != cudaSuccess) return e;
+    if (live) p->adj_stale = false;
+  }
+  return cudaSuccess;
+}
 mdp::HostBuf<SubDesc> &stage_of(mdp_plan *p, int set) { return set == 0 ? p->sub_stage : p->alt_stage; }
 
 void destroy_prof(mdp_plan *p) {
-  for (int f = 0; f < 32; ++f) {
+  for (int f = 0; f < NFAM; ++f) {
     for (auto &e : p->prof_ev[f]) { cudaEventDestroy(e.first); cudaEventDestroy(e.second); }
     p->prof_ev[f].clear();
     p->prof_used[f] = 0;
@@ -337,7 +368,7 @@ mdp_status mdp_plan_update_k_stream(mdp_plan *p, const double *k, void *cuda_str
   CK(cudaMemcpyAsync(p->h_fstatus.data(), p->d_fstatus, sizeof(int), cudaMemcpyDeviceToHost, s));
   if (p->ready_ev[p->set]) CK(cudaEventRecord(p->ready_ev[p->set], s));
   CK(cudaStreamSynchronize(s));
-  p->host_stale = p->fs_stale = true;
+  p->host_stale = p->fs_stale = p->adj_stale = true;
   return (mdp_status)p->h_fstatus[0];
 }
 
@@ -381,7 +412,7 @@ mdp_status mdp_plan_update_k_async(mdp_plan *p, const double *k, void *cuda_stre
   std::swap(p->d_piv, p->alt_piv);
   std::swap(p->d_sep, p->alt_sep);
   p->set = b;
-  p->host_stale = p->fs_stale = true;
+  p->host_stale = p->fs_stale = p->adj_stale = true;
   return MDP_OK;
 }
 
@@ -610,6 +641,9 @@ mdp_status mdp_ap_adjoint_rec(mdp_plan *p, const mdp_c64 *xi, const mdp_c64 *cot
   CK(cudaSetDevice(p->device));
   cudaStream_t st = (cudaStream_t)cuda_stream;
   CK(begin_use(p, st));
+  const cudaError_t te = ensure_adj_tables(p, st);
+  if (te == cudaErrorMemoryAllocation) { cudaGetLastError(); return MDP_ERR_NOMEM; }
+  CK(te);
   for (size_t w = 0; w < p->sched[S_GRAD].size(); ++w) {
     Batch fb[NFAM];
     wave_batches(p, w, fb, S_GRAD);
@@ -725,6 +759,7 @@ mdp_status mdp_plan_set_receivers(mdp_plan *p, const int *rows) {
   // the receiver row's moments, into the tables in use (the other set is rebuilt by its next update)
   CK(launch_sep_tables(p, p->d_subs, p->d_tables, p->d_sep, false, nullptr));
   CK(cudaStreamSynchronize(nullptr));
+  p->adj_stale = true;
   // the block counts of the receiver kernel and of the contractions changed: refresh the prefix sums
   for (int sc = 0; sc < 3; ++sc) {
     auto &waves = p->sched[sc];
@@ -733,7 +768,7 @@ mdp_status mdp_plan_set_receivers(mdp_plan *p, const int *rows) {
     for (size_t w = 0; w < waves.size(); ++w) {
       const int n = (int)waves[w].items.size();
       auto &pre = hpre[w];
-      for (const Fam f : {F_IREC, F_G1B, F_G1U, F_C3B, F_C3U, F_TCOLS, F_G3U, F_SOUT})
+      for (const Fam f : {F_IREC, F_G1B, F_G1U, F_C3B, F_C3U, F_TCOLS, F_G3U, F_SOUT, F_GG1B, F_GG1U, F_AC1, F_AG1, F_ATCOLS})
         for (int i = 0; i < n; ++i)
           pre[(size_t)f * (n + 1) + i + 1] =
               pre[(size_t)f * (n + 1) + i] +

@@ -968,7 +968,7 @@ __global__ void __launch_bounds__(32 * TRI_WARPS, 32 / TRI_WARPS) k_tri(Batch bt
                                              double *ws, const unsigned char *sep) {
   Item it; int local;
   locate(bt, bt.order ? bt.order[blockIdx.x] : (int)blockIdx.x, it, local);
-  MDP_CHECK_ITEM(bt, subs, it, local, FULL ? F_TRI : F_PTRI);
+  MDP_CHECK_ITEM(bt, subs, it, local, F_TRI);
   const SubDesc &d = subs[it.sub];
   const int cb = (it.ncols + 31) >> 5;
   const int b = (local % cb) * 32 + threadIdx.x;
@@ -1601,7 +1601,7 @@ cudaError_t set_kernel_attributes() {
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fwd_rows<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, FFT_SMEM);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fwd_rows<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, FFT_SMEM);
   if (e == cudaSuccess) e = set_adj_kernel_attributes();
-  if (e == cudaSuccess) e = set_tc_kernel_attributes();
+  if (e == cudaSuccess) e = set_sepadj_kernel_attributes();
   if (e == cudaSuccess) e = set_sep_kernel_attributes();
   if (e == cudaSuccess) e = set_full_kernel_attributes();
   // the sweep's staging buffers take 32 x 2.4 KiB per SM at full occupancy: prefer shared memory
@@ -1637,16 +1637,16 @@ cudaError_t launch_project(mdp_plan *p, const Batch *fb, int out_kind, const dou
     MDP_LAUNCH_AS(F_RING, F_RES, k_ring<<<grid1(fb[F_RING].total_blocks), b8, 0, st>>>(fb[F_RING], ds, tab, ws));
     MDP_LAUNCH_AS(F_PRES, F_RES, k_residual<false, false><<<grid1(fb[F_PRES].total_blocks), b8, 0, st>>>(fb[F_PRES], ds, tab, ws, xi_user));
   } else MDP_LAUNCH(F_RES, k_residual<true, false><<<grid1(fb[F_RES].total_blocks), b8, 0, st>>>(fb[F_RES], ds, tab, ws, xi_user));
-  if (basis) MDP_LAUNCH_AS(F_PROWS, F_FROWS, k_fwd_rows<false><<<grid1(fb[F_PROWS].total_blocks), b8, p->fft_smem, st>>>(fb[F_PROWS], ds, tab, ws));
-  else MDP_LAUNCH_AS(F_PROWS, F_FROWS, k_fwd_rows<true><<<grid1(fb[F_PROWS].total_blocks), b8, p->fft_smem, st>>>(fb[F_PROWS], ds, tab, ws));
+  if (basis) MDP_LAUNCH(F_FROWS, k_fwd_rows<false><<<grid1(fb[F_FROWS].total_blocks), b8, p->fft_smem, st>>>(fb[F_FROWS], ds, tab, ws));
+  else MDP_LAUNCH(F_FROWS, k_fwd_rows<true><<<grid1(fb[F_FROWS].total_blocks), b8, p->fft_smem, st>>>(fb[F_FROWS], ds, tab, ws));
   cudaError_t e = launch_sep_project(p, fb, out_kind, xi_user, out, out_rec, st);
   if (e != cudaSuccess) return e;
   if (p->tri_stages == 4) {
-    if (basis) MDP_LAUNCH_AS(F_PTRI, F_TRI, k_tri<false, false, 4><<<grid1(fb[F_PTRI].total_blocks), btri, tri_smem_bytes<false, 4>(), st>>>(fb[F_PTRI], ds, tab, p->d_piv, ws, p->d_sep));
-    else MDP_LAUNCH_AS(F_PTRI, F_TRI, k_tri<true, false, 4><<<grid1(fb[F_PTRI].total_blocks), btri, tri_smem_bytes<true, 4>(), st>>>(fb[F_PTRI], ds, tab, p->d_piv, ws, p->d_sep));
+    if (basis) MDP_LAUNCH(F_TRI, k_tri<false, false, 4><<<grid1(fb[F_TRI].total_blocks), btri, tri_smem_bytes<false, 4>(), st>>>(fb[F_TRI], ds, tab, p->d_piv, ws, p->d_sep));
+    else MDP_LAUNCH(F_TRI, k_tri<true, false, 4><<<grid1(fb[F_TRI].total_blocks), btri, tri_smem_bytes<true, 4>(), st>>>(fb[F_TRI], ds, tab, p->d_piv, ws, p->d_sep));
   } else {
-    if (basis) MDP_LAUNCH_AS(F_PTRI, F_TRI, k_tri<false, false, 2><<<grid1(fb[F_PTRI].total_blocks), btri, tri_smem_bytes<false, 2>(), st>>>(fb[F_PTRI], ds, tab, p->d_piv, ws, p->d_sep));
-    else MDP_LAUNCH_AS(F_PTRI, F_TRI, k_tri<true, false, 2><<<grid1(fb[F_PTRI].total_blocks), btri, tri_smem_bytes<true, 2>(), st>>>(fb[F_PTRI], ds, tab, p->d_piv, ws, p->d_sep));
+    if (basis) MDP_LAUNCH(F_TRI, k_tri<false, false, 2><<<grid1(fb[F_TRI].total_blocks), btri, tri_smem_bytes<false, 2>(), st>>>(fb[F_TRI], ds, tab, p->d_piv, ws, p->d_sep));
+    else MDP_LAUNCH(F_TRI, k_tri<true, false, 2><<<grid1(fb[F_TRI].total_blocks), btri, tri_smem_bytes<true, 2>(), st>>>(fb[F_TRI], ds, tab, p->d_piv, ws, p->d_sep));
   }
   if (basis) {
     MDP_LAUNCH(F_IROWS, k_inv_rows<false><<<grid1(fb[F_IROWS].total_blocks), b8, p->fft_smem, st>>>(fb[F_IROWS], ds, tab, ws, xi_user, out, out_kind));
@@ -1667,7 +1667,9 @@ cudaError_t launch_adjoint(mdp_plan *p, const Batch *fb, int out_kind, const dou
   const double *tab = p->d_tables;
   double *ws = p->d_ws;
   const dim3 b8(32, 8), btri(32, TRI_WARPS);
-  if (grad_k) {  // forward recompute with every mode-space row kept, and the k-derivative sources
+  cudaError_t e = launch_adj_clear(p, fb, st);
+  if (e != cudaSuccess) return e;
+  if (grad_k) {  // the residual and the k-derivative sources; by sweeps: forward recompute with every mode-space row kept
     if (basis) MDP_LAUNCH(F_EXT, k_extend<<<grid1(fb[F_EXT].total_blocks), 32, 0, st>>>(fb[F_EXT], ds, tab, ws, 1));
     if (basis) MDP_LAUNCH(F_RES, k_residual<false, true><<<grid1(fb[F_RES].total_blocks), b8, 0, st>>>(fb[F_RES], ds, tab, ws, xi_user));
     else MDP_LAUNCH(F_RES, k_residual<true, true><<<grid1(fb[F_RES].total_blocks), b8, 0, st>>>(fb[F_RES], ds, tab, ws, xi_user));
@@ -1675,8 +1677,10 @@ cudaError_t launch_adjoint(mdp_plan *p, const Batch *fb, int out_kind, const dou
     else MDP_LAUNCH(F_FROWS, k_fwd_rows<true><<<grid1(fb[F_FROWS].total_blocks), b8, p->fft_smem, st>>>(fb[F_FROWS], ds, tab, ws));
     if (basis) MDP_LAUNCH(F_TRI, k_tri<false, true, 2><<<grid1(fb[F_TRI].total_blocks), btri, TRI_WARPS * 2 * full_stage_bytes<false>(), st>>>(fb[F_TRI], ds, tab, p->d_piv, ws, p->d_sep));
     else MDP_LAUNCH(F_TRI, k_tri<true, true, 2><<<grid1(fb[F_TRI].total_blocks), btri, TRI_WARPS * 2 * full_stage_bytes<true>(), st>>>(fb[F_TRI], ds, tab, p->d_piv, ws, p->d_sep));
+    e = launch_sep_adj_residual(p, fb, !basis, st);
+    if (e != cudaSuccess) return e;
   }
-  cudaError_t e = cudaGetLastError();
+  e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   return launch_adjoint_tail(p, fb, out_kind, xi_user, cot, cot_rec, grad_xi, grad_k, st);
 }

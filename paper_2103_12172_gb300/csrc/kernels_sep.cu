@@ -871,6 +871,12 @@ cudaError_t launch_sep_sines(const mdp_plan *p, const SubDesc *ds, const double 
   return cudaGetLastError();
 }
 
+cudaError_t launch_sep_cut1(const Batch &b, const SubDesc *subs, double *ws, bool user, int fam, cudaStream_t st) {
+  if (user) k_sep_cut<true, 1><<<b.total_blocks, 256, 0, st>>>(b, subs, ws, fam);
+  else k_sep_cut<false, 1><<<b.total_blocks, 256, 0, st>>>(b, subs, ws, fam);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_sep_project(mdp_plan *p, const Batch *fb, int out_kind, const double2 *xi_user, double2 *out,
                                double2 *out_rec, cudaStream_t st) {
   const bool user = xi_user != nullptr;

@@ -44,8 +44,8 @@ struct SubDesc {
   int rows_fft;     // inverse transform of the gamma rows by FFT (Nx a power of 2, 2Nx <= 4096)
   int fpb;          // FFTs (columns) per block of the dense-row kernels: max(1, 1024 / (2 Nx))
   int leader;       // index of the subdomain owning this one's tables (itself unless deduplicated)
-  int tc_cols;      // 1: the projection runs through the separable Green's function (kernels_sep.cu) and the
-                    // adjoint's ring columns through k_adj_cols_tc; 0: per-mode sweeps and FP64 sums
+  int tc_cols;      // 1: the projection, the gradient pass and the full-grid solves run through the separable
+                    // Green's function (kernels_sep.cu, kernels_sepadj.cu, kernels_full.cu); 0: per-mode sweeps
   double h, k;
   double x0, x1, y0, y1, ax0, ay0;
   double c0, c1, c2;  // 9-point coefficients: centre, edge, corner (Eq. FD_scheme)
@@ -58,8 +58,6 @@ struct SubDesc {
   long long seg_off;    // doubles: per mode [Nq][5] = (rlo, rhi, frlo, frhi, itop): real rows of the
                         // factor table, real rows of the forward-sweep table, last swept row
   long long fs_off;     // doubles: projection forward-sweep table [Nq][NYf][FSW] (rows i0..)
-  long long tcb_off;    // doubles: per 16 modes a 1 KiB block of the fp16 digits of the sines at the adjoint's
-                        // ring columns, in the shared-memory operand layout of k_adj_cols_tc
   // bytes into the plan's separable tables (kernels_sep.cu), device only; without tc_cols the first three
   long long sep_zm, sep_z3;   // words: masks of the nonzero groups of K of sep_mb's and sep_b3's tiles
   long long sep_ab;     // doubles [Nq][2]: interior entries (off-diagonal, diagonal) of T_q
@@ -70,6 +68,11 @@ struct SubDesc {
   long long sep_tb, sep_mb, sep_b3;   // digit blocks of K (Toeplitz), of the moments, of the synthesis
   long long sep_bf, sep_bi;           // of the dense rows' transform and of the gamma rows' (sines only)
   long long sep_xf, sep_xi;           // of the full-grid transforms
+  // bytes into the plan's gradient tables (kernels_sepadj.cu): masks of adj_mb, adj_b3, adj_dmb (words); per mode
+  // ADJ_MDW doubles; k-derivatives of phi and K; digit blocks of K with gamma and the ring exchanged, of the
+  // moments, of the synthesis, of the full rows' transforms, and of dK/dk and d phi/dk for the residual
+  long long adj_zm, adj_z3, adj_zd, adj_md, adj_phid, adj_kdd, adj_kde, adj_tb, adj_mb, adj_b3, adj_bf, adj_bi, adj_dtb,
+      adj_dmb;
   long long sep_mx;     // per mode SEP_MXW doubles: the full-grid solve along y (kernels_full.cu)
   long long out_off;    // complex elements: start of the subdomain's output block
   long long rec_off;    // complex elements: start of the receiver block [n_cols][Px - 2]
@@ -296,6 +299,95 @@ inline __host__ __device__ FullWs full_ws(const SubDesc &d, int nr) {
   w.total = off;
   return w;
 }
+// ---- separable gradient pass (kernels_sepadj.cu): the same contractions with gamma and the ring exchanged
+constexpr int ADJ_MDW = 68;               // doubles per mode of the k-derivative table
+constexpr int ADJ_MOM = 4;                // moments of the cotangent per mode: phi_1, phi_2, their k-derivatives
+constexpr int ADJ_DMOM = 3;               // k-derivative moments of the residual: phi_1, phi_2, receiver
+enum AdjJob { A_MID = 0, A_FWD, A_SYN, A_INV };
+struct AdjGeo {
+  int ncls, nS, nqp, nqh;
+  int nti, nkj, ND;        // output groups (ring rows nlo+2 .. nhi-2), source groups (gamma rows nlo+1 .. nhi-1)
+  int nt3, nt1;            // tiles of 32: ring columns; with the moments
+  int nk1, nk3;            // K of MID, SYN ((b, mode), b < 2 or with a receiver row 3)
+  int nb;                  // K blocks of SYN
+  int nkf, ntr;            // FWD: folded columns mg .. of the gamma rows by 16, INV: mf .. of the ring rows by 32
+};
+inline __host__ __device__ AdjGeo adj_geo(const SubDesc &d, const SepGeo &g) {
+  AdjGeo a;
+  a.ncls = g.ncls; a.nS = g.nS; a.nqp = g.nqp; a.nqh = g.nqh;
+  a.nti = (g.Pj + 31) / 32;
+  a.nkj = (g.Pi + 15) / 16;
+  a.ND = 2 * a.nti + a.nkj;
+  a.nt3 = g.nS * a.nti;
+  a.nt1 = a.nt3 + ADJ_MOM * g.nqp / 32;
+  a.nk1 = g.nS * a.nkj;
+  a.nb = d.nrec >= 0 ? 3 : 2;
+  a.nk3 = a.nb * g.nqp / 16;
+  a.nkf = (g.Ng + 15) / 16;
+  a.ntr = (g.Kf + 31) / 32;
+  return a;
+}
+// rows of A: the columns padded to 128, real and imaginary parts, times the rows transformed
+inline __host__ __device__ int adj_rows(const SubDesc &d, int job, int ncols) {
+  const int r = 2 * sep_pad128(ncols);
+  return job == A_FWD ? (d.nrec >= 0 ? 5 : 4) * r : job == A_INV ? 4 * r : r;
+}
+inline __host__ __device__ int adj_classes(const AdjGeo &a, int job) { return job == A_MID || job == A_SYN ? a.ncls : 2; }
+inline __host__ __device__ int adj_nk(const AdjGeo &a, int job) {
+  return job == A_MID ? a.nk1 : job == A_FWD ? a.nkf : job == A_SYN ? a.nk3 : a.nqh / 16;
+}
+inline __host__ __device__ int adj_nt(const AdjGeo &a, int job) {
+  return job == A_MID ? a.nt1 : job == A_FWD ? a.nqh / 32 : job == A_SYN ? a.nt3 : a.ntr;
+}
+inline __host__ __device__ int adj_cut_blocks(const SubDesc &d, const AdjGeo &a, int job, int ncols) {
+  return adj_classes(a, job) * (adj_rows(d, job, ncols) / 8);
+}
+inline __host__ __device__ int adj_tiles(const SubDesc &d, const AdjGeo &a, int job, int ncols) {
+  return adj_classes(a, job) * (adj_rows(d, job, ncols) / 128) * adj_nt(a, job);
+}
+// tiles of the forward pass's stage 1 for the gradient: dK/dk, the moments and their derivatives, the dense rows
+inline __host__ __device__ int grad_mid_tiles(const SubDesc &d, const SepGeo &g) {
+  return g.nt3 + (2 + (d.nrec >= 0 ? 3 : 2)) * g.nqp / 32;
+}
+// Workspace of an item's gradient pass after the projection's (SepWs, whose stage 1 it shares), in doubles.
+struct AdjWs {
+  long long a[4], ex[4], mask;
+  long long dmom;        // k-derivative moments of the residual [class][ADJ_DMOM][nqp][rows] (its moments: SepWs::mom)
+  long long mom;         // moments of the cotangent [class][ADJ_MOM][nqp][rows]
+  long long ga;          // transforms of its gamma rows and receiver row [5][Nq][ncols] (complex)
+  long long u1, u3;      // sums at the ring columns [class][column][Pj][rows]
+  long long aeff;        // coefficients [class][3][nqp][rows]
+  long long ui;          // sums on the dense ring rows [parity][Kf][rows]
+  long long total;
+};
+inline __host__ __device__ int adj_mask_of(int job, int ncols) {   // jobs of at most R, 5 R, R, 4 R rows
+  const int t = 2 * (2 * sep_pad128(ncols) / 128) * SEP_MASK;
+  return job == A_MID ? 0 : job == A_FWD ? t : job == A_SYN ? 6 * t : 7 * t;
+}
+inline __host__ __device__ int adj_mask_words(int ncols) { return 11 * 2 * (2 * sep_pad128(ncols) / 128) * SEP_MASK; }
+inline __host__ __device__ AdjWs adj_ws(const SubDesc &d, int ncols) {
+  const SepGeo g = sep_geo(d);
+  const AdjGeo a = adj_geo(d, g);
+  const long long cp = sep_pad128(ncols), R = 2 * cp;
+  const long long rows[4] = {R, 5 * R, R, 4 * R}, nk3 = 3LL * g.nqp / 16;   // with room for a receiver row
+  AdjWs w;
+  long long off = sep_ws(d, ncols).total;
+  auto take = [&](long long n) { const long long o = off; off += (n + 31) & ~31LL; return o; };
+  for (int j = 0; j < 4; ++j) {
+    w.a[j] = take(adj_classes(a, j) * (rows[j] / 128) * (j == A_SYN ? nk3 : adj_nk(a, j)) * (SEP_ABLK / 8));
+    w.ex[j] = take(adj_classes(a, j) * rows[j] / 2);
+  }
+  w.mask = take(adj_mask_words(ncols) / 2);
+  w.dmom = take(g.ncls * (long long)ADJ_DMOM * g.nqp * R);
+  w.mom = take(g.ncls * (long long)ADJ_MOM * g.nqp * R);
+  w.ga = take(10LL * d.Nq * ncols);
+  w.u1 = take(g.ncls * (long long)g.nS * g.Pj * R);
+  w.u3 = take(g.ncls * (long long)g.nS * g.Pj * R);
+  w.aeff = take(g.ncls * 3LL * g.nqp * R);
+  w.ui = take(2LL * g.Kf * 4 * R);
+  w.total = off;
+  return w;
+}
 // first mask word of a job, in words from SepWs::mask (jobs of at most R, 4 R, R, 5 R rows)
 inline __host__ __device__ int sep_mask_of(int job, int ncols) {
   const int t = 2 * (2 * sep_pad128(ncols) / 128) * SEP_MASK;
@@ -383,6 +475,9 @@ struct mdp_plan {
   double *d_tables = nullptr;
   uint8_t *d_piv = nullptr;
   unsigned char *d_sep = nullptr;        // separable tables (kernels_sep.cu), rebuilt with the factor tables
+  unsigned char *d_adj = nullptr;        // gradient tables (kernels_sepadj.cu), one set: rebuilt by the gradient
+  long long adj_bytes = 0, adj_masks = 0;   // pass when the wavenumbers have changed since (adj_stale)
+  bool adj_stale = true, adj_sines = false;
   long long sep_bytes = 0, sep_masks = 0;   // size; its first bytes: the masks, cleared before a rebuild
   double *d_ws = nullptr;
   long long ws_doubles = 0;
@@ -419,8 +514,8 @@ struct mdp_plan {
   std::vector<GraphEntry> graphs;
   // per-kernel event timing (mdp_plan_profile)
   bool prof_on = false;
-  std::vector<std::pair<cudaEvent_t, cudaEvent_t>> prof_ev[32];
-  int prof_used[32] = {0};
+  std::vector<std::pair<cudaEvent_t, cudaEvent_t>> prof_ev[48];
+  int prof_used[48] = {0};
 };
 
 namespace mdp {
@@ -439,15 +534,14 @@ inline void set_bounds(const mdp_plan *p, Batch &b, long long out_n, bool grad) 
   b.status = p->d_status;
 }
 
-// kernel families (each has its own block decomposition of an item); F_A* are the adjoint's. F_TRI is
-// the gradient pass's full sweep, F_PTRI the projection's (subdomains without the separable solve),
-// F_FROWS and F_PROWS likewise for the dense rows' transform, F_RES, F_PRES and F_RING (basis columns of the
-// separable solve) for the ring residuals; F_C* cut operands, F_G* contract (stage 1
-// and 3, B: basis columns, U: user densities; F_TCOLS is stage 3 for basis columns), F_SMODE and F_SOUT
-// are the separable solve's other kernels.
+// kernel families (each has its own block decomposition of an item). F_A* are the adjoint's. F_RING (basis
+// columns of the separable solve), F_PRES and F_RES make the ring residuals. F_C* cut operands, F_G* contract
+// (stage 1 and 3, B: basis columns, U: user densities; F_TCOLS is stage 3 for basis columns), F_SMODE and
+// F_SOUT are the separable solve's other kernels; F_ACLR to F_AOUT and F_ATCOLS its gradient pass.
 enum Fam { F_EXT = 0, F_RES, F_FROWS, F_TRI, F_IROWS, F_ICOLS, F_AFWD, F_ATRI, F_ARING, F_ARINGC, F_AGAM, F_IREC,
-           F_ACOLS, F_TCOLS, F_ATCOLS, F_PTRI, F_C1B, F_C1U, F_G1B, F_G1U, F_SMODE, F_C3B, F_C3U, F_G3U, F_SOUT, F_PROWS, F_RING, F_PRES, NFAM };
-static_assert(NFAM <= 32, "per-family event lists of mdp_plan");
+           F_ACOLS, F_TCOLS, F_ATCOLS, F_C1B, F_C1U, F_G1B, F_G1U, F_SMODE, F_C3B, F_C3U, F_G3U, F_SOUT, F_RING, F_PRES,
+           F_ACLR, F_GG1B, F_GG1U, F_AC1, F_AG1, F_AMODE, F_AC3, F_AOUT, NFAM };
+static_assert(NFAM <= 48, "per-family event lists of mdp_plan");
 
 // Blocks of kernel family f for an item of ncols columns: 32 columns (x) times BY tasks (y).
 // The same function numbers the blocks on the host (prefix sums) and in the kernels.
@@ -463,16 +557,15 @@ inline __host__ __device__ int blocks_for(int f, const SubDesc &d, int ncols, in
       return cb * (((dense > side ? dense : side) + 7) / 8);
     }
     case F_FROWS:
+      if (d.tc_cols) return 0;
       if (d.rows_fft) return 4 * ((ncols + d.fpb - 1) / d.fpb);
       return cb * ((d.Nx / 2 + 7) / 8);
-    case F_TRI: return cb * ((d.Nq + TRI_WARPS - 1) / TRI_WARPS);
-    case F_PROWS: return d.tc_cols ? 0 : blocks_for(F_FROWS, d, ncols, col0);
+    case F_TRI: return d.tc_cols ? 0 : cb * ((d.Nq + TRI_WARPS - 1) / TRI_WARPS);
     case F_IROWS:
       if (d.tc_cols) return 0;
       if (d.rows_fft) return 4 * ((ncols + d.fpb - 1) / d.fpb);
       return cb * (((d.xsym ? 4 * (d.Ph + 1) : 4 * (d.Px + 2)) + 7) / 8);
     case F_ICOLS: return d.tc_cols ? 0 : cb * ((d.Py - 2 + 7) / 8);
-    case F_PTRI: return d.tc_cols ? 0 : cb * ((d.Nq + TRI_WARPS - 1) / TRI_WARPS);
     case F_C1B: case F_C1U: case F_G1B: case F_G1U: case F_C3B: case F_C3U: case F_TCOLS: case F_G3U: {
       if (!d.tc_cols) return 0;
       const SepGeo g = sep_geo(d);
@@ -482,6 +575,26 @@ inline __host__ __device__ int blocks_for(int f, const SubDesc &d, int ncols, in
         return sep_cut_blocks(d, g, j, ncols, col0, user) + sep_cut_blocks(d, g, j + 1, ncols, col0, user);
       return sep_tiles(d, g, j, ncols, col0, user) + sep_tiles(d, g, j + 1, ncols, col0, user);
     }
+    case F_ACLR: return d.tc_cols ? 1 : 0;
+    case F_GG1B: case F_GG1U: {
+      if (!d.tc_cols) return 0;
+      const SepGeo g = sep_geo(d);
+      return g.ncls * (sep_rows(d, J_MID, ncols, col0, f == F_GG1U) / 128) * grad_mid_tiles(d, g) +
+             sep_tiles(d, g, J_FWD, ncols, col0, f == F_GG1U);
+    }
+    case F_AC1: case F_AC3: case F_AG1: case F_ATCOLS: {
+      if (!d.tc_cols) return 0;
+      const AdjGeo a = adj_geo(d, sep_geo(d));
+      const int j = f == F_AC1 || f == F_AG1 ? A_MID : A_SYN;   // and the next job
+      if (f == F_AC1 || f == F_AC3) return adj_cut_blocks(d, a, j, ncols) + adj_cut_blocks(d, a, j + 1, ncols);
+      return adj_tiles(d, a, j, ncols) + adj_tiles(d, a, j + 1, ncols);
+    }
+    case F_AMODE: return d.tc_cols ? cb * ((d.Nq + SEP_MODES_PER_BLOCK - 1) / SEP_MODES_PER_BLOCK) : 0;
+    case F_AOUT: {   // ring columns of the middle rows; dense ring rows; dK/dk against the cotangent
+      if (!d.tc_cols) return 0;
+      const SepGeo g = sep_geo(d);
+      return cb * ((g.Pj + 7) / 8 + (4 * g.Kf + 7) / 8 + (g.Pi + 7) / 8);
+    }
     case F_SMODE: return d.tc_cols ? cb * ((d.Nq + SEP_MODES_PER_BLOCK - 1) / SEP_MODES_PER_BLOCK) : 0;
     case F_SOUT: {   // middle rows, 8 per block, then 32 folded columns of each row transformed back
       if (!d.tc_cols) return 0;
@@ -489,14 +602,15 @@ inline __host__ __device__ int blocks_for(int f, const SubDesc &d, int ncols, in
       return cb * ((d.Py - 2 + 7) / 8) + cb * g.slots * g.ntg;
     }
     case F_AFWD:
+      if (d.tc_cols) return 0;
       if (d.rows_fft) return 5 * ((ncols + d.fpb - 1) / d.fpb);
       return cb * ((d.Nx / 2 + 7) / 8);
-    case F_ATRI: return cb * ((d.Nq + 3) / 4);
+    case F_ATRI: return d.tc_cols ? 0 : cb * ((d.Nq + 3) / 4);
     case F_ARING:
+      if (d.tc_cols) return 0;
       if (d.rows_fft) return 4 * ((ncols + d.fpb - 1) / d.fpb);
       return cb * ((4 * d.Px + 7) / 8);
     case F_ARINGC: return d.tc_cols ? 0 : cb * ((d.Py - 4 + 7) / 8);
-    case F_ATCOLS: return d.tc_cols && d.Py > 4 ? ((ncols + 63) / 64) * (d.Py - 4) : 0;   // tiles: inner middle row x 64 columns
     case F_AGAM: return cb * ((d.G + 7) / 8);
     case F_IREC: return d.nrec < 0 || d.tc_cols ? 0 : cb * (((d.xsym ? d.Ph - 1 : d.Px - 2) + 7) / 8);
     case F_ACOLS: return cb * ((d.Py - 2 + 7) / 8);
@@ -504,21 +618,20 @@ inline __host__ __device__ int blocks_for(int f, const SubDesc &d, int ncols, in
   }
 }
 
-// slot bases of the per-block gradient partials of an item: [ATRI | ARING | ARINGC or 4 per ATCOLS
-// tile | AGAM], total
+// slot bases of the per-block gradient partials of an item: [ATRI or AMODE | ARING or AOUT | ARINGC | AGAM],
+// total
 inline __host__ __device__ void red_slots(const SubDesc &d, int ncols, int base[5]) {
   base[0] = 0;
-  base[1] = base[0] + blocks_for(F_ATRI, d, ncols, 0);
-  base[2] = base[1] + blocks_for(F_ARING, d, ncols, 0);
-  base[3] = base[2] + blocks_for(F_ARINGC, d, ncols, 0) + 4 * blocks_for(F_ATCOLS, d, ncols, 0);
+  base[1] = base[0] + blocks_for(F_ATRI, d, ncols, 0) + blocks_for(F_AMODE, d, ncols, 0);
+  base[2] = base[1] + blocks_for(F_ARING, d, ncols, 0) + blocks_for(F_AOUT, d, ncols, 0);
+  base[3] = base[2] + blocks_for(F_ARINGC, d, ncols, 0);
   base[4] = base[3] + blocks_for(F_AGAM, d, ncols, 0);
 }
 // Workspace slices of an item of ncols columns, in doubles from the item's base (each 256-byte
 // aligned): basis densities, ring residual, dense-row transforms, mode-space field, and for the
-// gradient pass the adjoint field, k-source and per-block partials; its last slice holds, after the
-// partials and their total, per column the largest biased exponent (ints) of the adjoint field's
-// inner middle rows. With the separable solve the projection keeps only the 4 gamma rows and the
-// receiver row of the mode-space field ([Nq][5][ncols]), and its operands and sums (SepWs).
+// gradient pass the adjoint field, k-source and per-block partials. With the separable solve the projection
+// keeps only the 4 gamma rows and the receiver row of the mode-space field ([Nq][5][ncols]), and its
+// operands and sums (SepWs); the gradient pass the adjoint field of the 4 dense ring rows, SepWs and AdjWs.
 inline __host__ __device__ void item_workspace(const SubDesc &d, int ncols, bool grad, long long &xi, long long &r,
                                                long long &gr, long long &y, long long &a, long long &s,
                                                long long &red, long long &total) {
@@ -527,12 +640,13 @@ inline __host__ __device__ void item_workspace(const SubDesc &d, int ncols, bool
   xi = off; off += al((long long)d.G * ncols * (grad ? 2 : 1));
   r = off;  off += al((long long)(d.R > d.R2 ? d.R : d.R2) * ncols * 2);
   gr = off; off += al(5LL * d.Nq * ncols * 2);  // 4 dense rows (+ the receiver row in the adjoint)
-  y = off;  off += al((long long)d.Nq * (grad ? d.Nt : d.tc_cols ? 5 : d.NYf) * ncols * 2);
-  a = off;  off += grad ? al((long long)d.Nq * d.Nt * ncols * 2) : d.tc_cols ? sep_ws(d, ncols).total : 0;
+  y = off;  off += al((long long)d.Nq * (d.tc_cols ? 5 : grad ? d.Nt : d.NYf) * ncols * 2);
+  a = off;  off += d.tc_cols ? (grad ? adj_ws(d, ncols).total : sep_ws(d, ncols).total)
+                             : grad ? al((long long)d.Nq * d.Nt * ncols * 2) : 0;
   s = off;  off += grad ? al((long long)d.R * ncols * 2) : 0;
   int rs[5];
   red_slots(d, ncols, rs);
-  red = off; off += grad ? al(rs[4] + 1 + (ncols + 1) / 2) : 0;
+  red = off; off += grad ? al(rs[4] + 1) : 0;
   total = off;
 }
 const char *fam_name(int f);
@@ -553,7 +667,6 @@ void host_mode_solve(const HostSub &hs, int q, int adjoint, const double *b, dou
 enum { PASS_FWD = 0, PASS_GRAD = 1 };
 cudaError_t set_kernel_attributes();      // kernels.cu: opt-in shared memory of the FFT kernels
 cudaError_t set_adj_kernel_attributes();  // kernels_adj.cu
-cudaError_t set_tc_kernel_attributes();   // kernels_tc.cu
 cudaError_t set_sep_kernel_attributes();  // kernels_sep.cu
 // the separable tables of every subdomain that takes them, for the wavenumbers of the descriptors ds;
 // entries: from matrix entries computed here, else from the stored ones (sep_ab)
@@ -564,9 +677,16 @@ cudaError_t launch_sep_sines(const mdp_plan *p, const SubDesc *ds, const double 
 // the separable solve of the projection, from the ring residuals to the output columns
 cudaError_t launch_sep_project(mdp_plan *p, const Batch *fb, int out_kind, const double2 *xi_user, double2 *out,
                                double2 *out_rec, cudaStream_t st);
-// the adjoint's sums at the 4 ring columns of the inner middle rows (dk: with the k-gradient partials)
-cudaError_t launch_adj_cols_tc(const Batch &b, const SubDesc *subs, const double *tab, double *ws, bool dk,
-                               int *status, int n_sm, cudaStream_t st);
+// kernels_sepadj.cu: the gradient tables for the wavenumbers of the plan's current set, and the k-independent
+// ones; the separable gradient pass of a wave (forward: with the k-gradient)
+cudaError_t launch_adj_tables(const mdp_plan *p, cudaStream_t st);
+cudaError_t launch_adj_sines(const mdp_plan *p, cudaStream_t st);
+cudaError_t launch_adj_clear(mdp_plan *p, const Batch *fb, cudaStream_t st);
+cudaError_t launch_sep_adj_residual(mdp_plan *p, const Batch *fb, bool user, cudaStream_t st);
+cudaError_t launch_sep_adjoint(mdp_plan *p, const Batch *fb, bool user, bool dk, const double2 *cot, const double2 *cot_rec,
+                               cudaStream_t st);
+cudaError_t launch_sep_cut1(const Batch &b, const SubDesc *subs, double *ws, bool user, int fam, cudaStream_t st);
+cudaError_t set_sepadj_kernel_attributes();
 cudaError_t launch_project(mdp_plan *p, const Batch *fam_batches, int out_kind, const double2 *xi_user,
                            double2 *out, double2 *out_rec, cudaStream_t st);
 cudaError_t launch_adjoint(mdp_plan *p, const Batch *fam_batches, int out_kind, const double2 *xi_user,

@@ -62,7 +62,7 @@ extern "C" mdp_status mdp_ap_solve_noalloc(const mdp_subdomain *sub, int nrhs, c
   hd.fact_off = 0;
   hd.sin_off = (long long)((n_fact + 31) & ~(size_t)31);
   hd.piv_off = 0;
-  hd.dT_off = hd.geo_off = hd.seg_off = hd.fs_off = hd.tcb_off = 0;
+  hd.dT_off = hd.geo_off = hd.seg_off = hd.fs_off = 0;
   const size_t off_tab = align256(sizeof(mdp::SubDesc));
   const size_t off_piv = off_tab + align256(((size_t)hd.sin_off + n_sin) * sizeof(double));
   const size_t off_buf = off_piv + align256(n_piv);

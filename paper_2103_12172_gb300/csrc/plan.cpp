@@ -23,9 +23,11 @@ static const double kSingularTol = 1e-13; // pivot below this x max|T| -> singul
 const char *fam_name(int f) {
   static const char *names[NFAM] = {"k_extend", "k_residual", "k_fwd_rows", "k_tri", "k_inv_rows", "k_inv_cols",
                                     "k_adj_rows", "k_adj_tri", "k_adj_ring_rows", "k_adj_ring_cols", "k_adj_gamma",
-                                    "k_inv_rec", "k_adj_cols", "k_inv_cols_tc", "k_adj_ring_cols_tc", "k_tri(projection)",
+                                    "k_inv_rec", "k_adj_cols", "k_inv_cols_tc", "k_adj_ring_cols_tc",
                                     "k_sep_cut1", "k_sep_cut1(user)", "k_sep_gemm1", "k_sep_gemm1(user)", "k_sep_modes",
-                                    "k_sep_cut3", "k_sep_cut3(user)", "k_inv_cols_tc(user)", "k_sep_out", "k_fwd_rows(projection)", "k_ring", "k_residual(projection)"};
+                                    "k_sep_cut3", "k_sep_cut3(user)", "k_inv_cols_tc(user)", "k_sep_out", "k_ring", "k_residual(projection)",
+                                    "k_adj_clear", "k_grad_gemm", "k_grad_gemm(user)", "k_adj_cut1", "k_adj_gemm1", "k_adj_modes",
+                                    "k_adj_cut3", "k_adj_out"};
   return (f >= 0 && f < NFAM) ? names[f] : "?";
 }
 
@@ -67,15 +69,13 @@ static mdp_status geometry(const mdp_subdomain &in, HostSub &hs, unsigned flags,
   d.nrec = -1;
   d.rows_fft = !(flags & MDP_PLAN_DIRECT_ROWS) && (d.Nx & (d.Nx - 1)) == 0 && 2 * d.Nx <= FFT_POINTS && d.Nx >= 8;
   d.fpb = d.rows_fft ? std::max(1, fft_block_points / (2 * d.Nx)) : 0;
-  // the separable solve and the adjoint's ring columns on the tensor cores: the adjoint's exact
-  // integer accumulation needs at most 1024 modes per output (a parity half of Nq on centred
-  // subdomains); MDP_PLAN_FP64_COLS (or the environment MDP_TC_COLS=0) keeps the sweeps and the
-  // FP64 sums
+  // the separable solve on the tensor cores: the sines of a row's transform and the synthesis take at most
+  // 1024 modes per class (a parity half of Nq on centred subdomains), and the mask of a tile's groups of K
+  // holds 256 of them, which K of the middle rows (2 or 4 columns of up to Py - 2 rows) has to fit;
+  // MDP_PLAN_FP64_COLS (or the environment MDP_TC_COLS=0) keeps the sweeps and the FP64 sums
   {
     const char *tc = std::getenv("MDP_TC_COLS");
     const bool on = !(flags & MDP_PLAN_FP64_COLS) && !(tc && tc[0] == '0' && tc[1] == 0);
-    // the mask of a tile's groups of K holds 256 of them, which K of the middle rows (2 or 4 columns of up
-    // to Py - 2 rows) has to fit
     d.tc_cols = on && (d.xsym ? d.Nq <= 2047 : d.Nq <= 1023) &&
                 (d.xsym ? 2 : 4) * ((d.Py - 2 + 15) / 16) <= 32 * SEP_MASK;
   }
@@ -414,14 +414,28 @@ static bool layout_tables(mdp_plan *p) {
     d.sep_z3 = take(4LL * SEP_MASK * g.ncls * g.nt3);
   }
   p->sep_masks = sep;
+  long long adj = 0;
+  auto take_adj = [&](long long bytes) { const long long o = adj; adj += (bytes + 255) & ~255LL; return o; };
+  for (auto &hs : p->subs) {
+    SubDesc &d = hs.d;
+    if (d.leader != (int)(&hs - p->subs.data()) || !d.tc_cols) continue;
+    const SepGeo g = sep_geo(d);
+    const AdjGeo a = adj_geo(d, g);
+    d.adj_zm = take_adj(4LL * SEP_MASK * g.ncls * (ADJ_MOM * g.nqp / 32));
+    d.adj_z3 = take_adj(4LL * SEP_MASK * g.ncls * a.nt3);
+    d.adj_zd = take_adj(4LL * SEP_MASK * g.ncls * (ADJ_DMOM * g.nqp / 32));
+  }
+  p->adj_masks = adj;
   for (auto &hs : p->subs) {
     SubDesc &d = hs.d;
     if (d.leader != (int)(&hs - p->subs.data())) {   // a duplicate: the leader's tables
       const SubDesc &ld = p->subs[d.leader].d;
       d.fact_off = ld.fact_off; d.dT_off = ld.dT_off; d.sin_off = ld.sin_off; d.geo_off = ld.geo_off;
-      d.seg_off = ld.seg_off; d.fs_off = ld.fs_off; d.piv_off = ld.piv_off; d.tcb_off = ld.tcb_off;
+      d.seg_off = ld.seg_off; d.fs_off = ld.fs_off; d.piv_off = ld.piv_off;
       d.sep_zm = ld.sep_zm; d.sep_z3 = ld.sep_z3; d.sep_ab = ld.sep_ab; d.sep_mt = ld.sep_mt; d.sep_phi = ld.sep_phi; d.sep_kd = ld.sep_kd; d.sep_kde = ld.sep_kde;
       d.sep_tb = ld.sep_tb; d.sep_mb = ld.sep_mb; d.sep_b3 = ld.sep_b3; d.sep_bf = ld.sep_bf; d.sep_bi = ld.sep_bi; d.sep_xf = ld.sep_xf; d.sep_xi = ld.sep_xi; d.sep_mx = ld.sep_mx;
+      d.adj_zm = ld.adj_zm; d.adj_z3 = ld.adj_z3; d.adj_zd = ld.adj_zd; d.adj_md = ld.adj_md; d.adj_phid = ld.adj_phid; d.adj_kdd = ld.adj_kdd; d.adj_kde = ld.adj_kde;
+      d.adj_tb = ld.adj_tb; d.adj_mb = ld.adj_mb; d.adj_b3 = ld.adj_b3; d.adj_bf = ld.adj_bf; d.adj_bi = ld.adj_bi; d.adj_dtb = ld.adj_dtb; d.adj_dmb = ld.adj_dmb;
       d.out_off = out;  out += (long long)d.G * d.n_cols;
       continue;
     }
@@ -441,6 +455,18 @@ static bool layout_tables(mdp_plan *p) {
       d.sep_bi = take(2LL * g.ntg * (g.nqh / 16) * SEP_BBLK);
       d.sep_xf = take(2LL * (g.nqh / 32) * g.nkx * SEP_BBLK);
       d.sep_xi = take(2LL * g.ntx * (g.nqh / 16) * SEP_BBLK);
+      const AdjGeo a = adj_geo(d, g);
+      d.adj_md = take_adj(8LL * ADJ_MDW * d.Nq);
+      d.adj_phid = take_adj(16LL * (d.Py + 2) * d.Nq);
+      d.adj_kdd = take_adj(8 * pairs * d.Py);
+      d.adj_kde = take_adj(8LL * g.ncls * g.nS);
+      d.adj_tb = take_adj(pairs * a.ND * SEP_BBLK);
+      d.adj_mb = take_adj((long long)g.ncls * (ADJ_MOM * g.nqp / 32) * a.nk1 * SEP_BBLK);
+      d.adj_b3 = take_adj((long long)g.ncls * a.nt3 * (3 * g.nqp / 16) * SEP_BBLK);   // room for receivers
+      d.adj_bf = take_adj(2LL * (g.nqh / 32) * a.nkf * SEP_BBLK);
+      d.adj_bi = take_adj(2LL * a.ntr * (g.nqh / 16) * SEP_BBLK);
+      d.adj_dtb = take_adj(pairs * g.ND * SEP_BBLK);
+      d.adj_dmb = take_adj((long long)g.ncls * (ADJ_DMOM * g.nqp / 32) * g.nk1 * SEP_BBLK);
     }
     const int FW = d.cplx ? 8 : 4;
     d.fact_off = off; off += al((long long)d.Nq * d.Nt * FW);
@@ -449,7 +475,6 @@ static bool layout_tables(mdp_plan *p) {
     d.geo_off = off;  off += al(4LL * d.G);
     d.seg_off = off;  off += al(5LL * d.Nq);
     d.fs_off = off;   off += al((long long)d.Nq * d.NYf * FSW);
-    d.tcb_off = off;  off += d.tc_cols ? al(128LL * ((d.Nq + 15) / 16)) : 0;
     d.piv_off = poff; poff += al((long long)d.Nq * d.Nt);
     d.out_off = out;  out += (long long)d.G * d.n_cols;
   }
@@ -464,50 +489,8 @@ static bool layout_tables(mdp_plan *p) {
   }
   p->out_size = out;
   p->sep_bytes = sep;
+  p->adj_bytes = adj;
   return true;
-}
-
-// fp16 bit pattern of the integer v, |v| <= 128 (exact)
-static uint16_t f16_of_small_int(int v) {
-  if (v == 0) return 0;
-  const unsigned sgn = v < 0 ? 0x8000u : 0u;
-  unsigned a = (unsigned)std::abs(v);
-  int e = 0;
-  while ((a >> (e + 1)) != 0) ++e;
-  return (uint16_t)(sgn | ((unsigned)(e + 15) << 10) | ((a << (10 - e)) & 0x3FFu));
-}
-
-// The B operand of k_adj_cols_tc (the sine factors of the adjoint's ring-column sums) for every 16
-// modes: row n = 8 so + u holds digit u (u < 7; row 7 zero) of output so, where the outputs are, on
-// a centred subdomain, sin(pi q m/Nx) at m = mlo, mlo+1 for odd q, then the same for even q (zero
-// at the other parity), else the columns mlo, mlo+1, mhi-1, mhi. A factor s becomes the integer
-// W = round(s 2^50) through the bits of s + 6 (exact: |s| <= 1 keeps the sum in [4, 8)), written
-// in 7 balanced base-256 digits (the bytes of W + 0x0080808080808080, each minus 128). Stored in
-// the operand layout: 8 x 16-byte core matrices, K (the mode) fastest, 128 B between the two
-// K halves and 256 B between groups of 8 rows.
-static void fill_tc_block(const SubDesc &d, const double *S, uint16_t *blk) {
-  const int nch = (d.Nq + 15) / 16, N2 = 2 * d.Nx;
-  int64_t magic, w;
-  const double six = 6.0;
-  std::memcpy(&magic, &six, 8);
-  for (int c = 0; c < nch; ++c)
-    for (int so = 0; so < 4; ++so)
-      for (int kk = 0; kk < 16; ++kk) {
-        const int q = c * 16 + 1 + kk;
-        int m, par = -1;
-        if (d.xsym) { m = (so & 1) ? d.mlo + 1 : d.mlo; par = so < 2 ? 1 : 0; }
-        else m = so == 0 ? d.mlo : so == 1 ? d.mlo + 1 : so == 2 ? d.mhi - 1 : d.mhi;
-        const double s = (q <= d.Nq && (par < 0 || (q & 1) == par)) ? S[(int)(((long long)q * m) % N2)] : 0.0;
-        const double y = s + six;
-        std::memcpy(&w, &y, 8);
-        const uint64_t b = (uint64_t)(w - magic) + 0x0080808080808080ull;
-        for (int u = 0; u < 8; ++u) {
-          const int n = so * 8 + u;
-          const int dig = u < 7 ? (int)((b >> (8 * (6 - u))) & 0xFF) - 128 : 0;
-          blk[(size_t)c * 512 + (((n >> 3) * 256 + (kk >> 3) * 128 + (n & 7) * 16 + (kk & 7) * 2) >> 1)] =
-              f16_of_small_int(dig);
-        }
-      }
 }
 
 static void fill_tables(mdp_plan *p) {
@@ -520,7 +503,6 @@ static void fill_tables(mdp_plan *p) {
       S[2 * d.Nx + j] = (2.0 / d.Nx) * S[j];
     }
     for (int i = 0; i < 5 * d.Nq; ++i) p->host_tables[d.seg_off + i] = hs.seg[i];
-    if (d.tc_cols) fill_tc_block(d, S, reinterpret_cast<uint16_t *>(&p->host_tables[d.tcb_off]));
     double *g = &p->host_tables[d.geo_off];
     for (int i = 0; i < d.G; ++i) {
       g[4 * i + 0] = hs.owner[i];
@@ -539,7 +521,7 @@ static void schedule_pass(mdp_plan *p, bool grad, bool leaders_only, std::vector
   for (int si = 0; si < (int)p->subs.size(); ++si) {
     if (leaders_only && p->leader[si] != si) continue;
     const SubDesc &d = p->subs[si].d;
-    const int cols = grad || !d.tc_cols ? p->tile_cols : p->sep_cols;
+    const int cols = d.tc_cols ? p->sep_cols : p->tile_cols;
     for (int c0 = 0; c0 < d.n_cols; c0 += cols) {
       Item it;
       std::memset(&it, 0, sizeof it);

@@ -133,3 +133,30 @@ def test_tall_grids_around_the_limits_of_the_separable_solve(mdp, sub):
     a, b = (p.solve(0, g).view(2, -1).cpu().numpy() for p in (plan, ref))
     plan.status()
     assert rel_col_err(a, b) < 1e-9
+
+
+@pytest.mark.parametrize("name,sub", CASES, ids=[c[0] for c in CASES])
+@pytest.mark.parametrize("user,rec,kind", [(False, False, "P"), (True, False, "Q"), (False, True, "Q"), (True, True, "P")])
+def test_gradient_is_that_of_the_sweeps(mdp, name, sub, user, rec, kind):
+    """The gradient pass by the separable solve against the recurrences: basis and user densities, with a
+    receiver row's cotangent, both kinds; the second pass (after a change of k) on rebuilt tables. Bar:
+    1e-10 for the gradients by densities, 1e-9 for the one by k (the oracle's bars)."""
+    plan, ref = mdp.Plan([sub]), mdp.Plan([sub], fp64_cols=True)
+    G, nc, _, nm = plan.layout(0)
+    row = int(nm[:, 0].min() + 2 + (np.ptp(nm[:, 0]) - 4) // 3)
+    cot = torch.from_numpy(W.random_complex(nc * G, seed=12)).cuda()
+    xi = torch.from_numpy(W.random_complex(nc * G, seed=13)).cuda() if user else None
+    cr = None
+    if rec:
+        for p in (plan, ref):
+            p.set_receivers([row])
+        cr = torch.from_numpy(W.random_complex(nc * plan.receiver_layout(0)[2], seed=14)).cuda()
+    for k in (None, sub.k * 1.01):
+        if k is not None:
+            for p in (plan, ref):
+                p.update_k([k])
+        (ga, ka), (gb, kb) = (p.adjoint(cot, xi=xi, kind=kind, grad_xi=user, cot_rec=cr) for p in (plan, ref))
+        plan.status()
+        if user:
+            assert rel_col_err(ga.view(nc, G).cpu().numpy(), gb.view(nc, G).cpu().numpy()) < 1e-10
+        assert abs(ka.item() - kb.item()) < 1e-9 * abs(kb.item())
