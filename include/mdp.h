@@ -250,6 +250,46 @@ mdp_status mdp_householder_qr_batched(int batch, int m, int n, int nrhs, mdp_c64
 mdp_status mdp_triangular_solve(int n, int nrhs, const mdp_c64 *R, long long ldr, int conj_trans, mdp_c64 *B,
                                 long long ldb, void *cuda_stream);
 
+/* The coupled system of a layout of subdomains (Sections 3.3-3.5): per subdomain j the Chebyshev
+ * coefficients of the boundary data are c_j = S_j x + e_j (8 M values: c^(0) of sides 1..4, then c^(1)),
+ * with x the unknowns, entries 1, -1 or rho[q] in S_j and eps[q][m] in e_j (q: an outer side), and x
+ * minimises sum_j ||Q_j c_j - f_j||^2. Every unknown belongs to one subdomain's rows (private) or two (shared).
+ * tables: device ints, in this order: rows G[n_blocks]; unknowns of a subdomain [n_blocks] (private ones
+ * first), private ones of them, first row in the shared matrix, first row of the stacked rows; then
+ * [n_blocks][max_cols] of a subdomain's unknowns: number, coefficient of entry 1 or -1, 1 if it is -1,
+ * coefficient of entry rho or -1, its q, index among the shared ones; [n_blocks][8 M] of a
+ * coefficient: its unknown or -1, entry (0: 1, 1: -1, 2 + q: rho[q]), index into eps or -1; [n][2] of an unknown:
+ * subdomain * max_cols + position, or -1; [n_shared] numbers of the shared unknowns; [n_outer] of an outer
+ * side: subdomain, first coefficient of eps, first coefficient of rho or -1, first unknown.
+ * offsets: device, first element of Q_j in Q (stored [8 M][G_j]). rows: sum of the G_j. */
+typedef struct mdp_couple {
+  int n_blocks, n_modes, n, n_shared, shared_rows, max_rows, max_cols, n_outer, rows;
+  const int *tables;
+  const long long *offsets;
+} mdp_couple;
+/* Complex elements of the buffers and ints of work below; 0: not a system the calls take (more unknowns
+ * of a subdomain than rows, or triangles beyond a CTA's shared memory). */
+long long mdp_couple_buffer(const mdp_couple *c);
+long long mdp_couple_grad_buffer(const mdp_couple *c);
+long long mdp_couple_work_ints(const mdp_couple *c);
+/* x [n] and the coefficients coef [n_blocks][8 M]. src: f [rows] or null (zero). buf: kept for the gradient.
+ * work: mdp_couple_work_ints ints; after the stream has finished work[n_blocks] and (with shared
+ * unknowns) work[mdp_householder_qr_work_ints(n_blocks) + 1] are the status words of the two QR launches. */
+mdp_status mdp_couple_solve(const mdp_couple *c, const mdp_c64 *Q, const mdp_c64 *rho, const mdp_c64 *eps,
+                            const mdp_c64 *src, mdp_c64 *buf, int *work, mdp_c64 *x, mdp_c64 *coef, void *cuda_stream);
+/* From g = dLoss/d conj(coef) [n_blocks][8 M]: the gradients by Q (gQ, may be null), rho [n_outer] and
+ * eps [n_outer][M]. tmp: mdp_couple_grad_buffer elements. */
+mdp_status mdp_couple_grad(const mdp_couple *c, const mdp_c64 *Q, const mdp_c64 *rho, const mdp_c64 *src,
+                           const mdp_c64 *buf, const mdp_c64 *x, const mdp_c64 *coef, const mdp_c64 *g, mdp_c64 *tmp,
+                           mdp_c64 *gQ, mdp_c64 *grho, mdp_c64 *geps, void *cuda_stream);
+/* y_j = B_j v_j for blocks B_j stored [cols][len_j] from off_j, v [n_blocks][cols], y_j from yoff_j (all on the
+ * device); and the gradients gB = gy v^H, gv = B^H gy (either may be null). max_len: the largest len_j. */
+mdp_status mdp_block_values(int n_blocks, int cols, int max_len, const int *len, const int *yoff, const long long *off,
+                            const mdp_c64 *B, const mdp_c64 *v, mdp_c64 *y, void *cuda_stream);
+mdp_status mdp_block_values_grad(int n_blocks, int cols, int max_len, const int *len, const int *yoff,
+                                 const long long *off, const mdp_c64 *B, const mdp_c64 *v, const mdp_c64 *gy, mdp_c64 *gB,
+                                 mdp_c64 *gv, void *cuda_stream);
+
 /* C = op(A) op(B), or C += op(A) op(B) if accumulate != 0, for the small dense products of the
  * coupled system's assembly (Sections 3.3-3.5: Q times a coefficient vector, the Chebyshev
  * transform of boundary data, the receiver values). op(A) is m x k with element (i, l) at

@@ -17,7 +17,7 @@ CSRC = os.path.join(PKG, "csrc")
 BUILD = os.path.join(ROOT, "_build")
 LIB = os.path.join(PKG, "libmdp.so")
 LIB_CHECKED = os.path.join(PKG, "libmdp_checked.so")   # MDP_CHECKED=1: bounds-checked kernels
-SOURCES = ["plan.cpp", "kernels.cu", "kernels_adj.cu", "kernels_sepadj.cu", "kernels_sep.cu", "kernels_full.cu", "factor.cu", "qr.cu", "api.cu", "probe.cu",
+SOURCES = ["plan.cpp", "kernels.cu", "kernels_adj.cu", "kernels_sepadj.cu", "kernels_sep.cu", "kernels_full.cu", "factor.cu", "qr.cu", "couple.cu", "api.cu", "probe.cu",
            "noalloc.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

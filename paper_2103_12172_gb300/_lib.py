@@ -35,6 +35,11 @@ class mdp_plan_options(C.Structure):
                 ("tri_stages", C.c_int)]
 
 
+class mdp_couple(C.Structure):
+    _fields_ = [(f, C.c_int) for f in ("n_blocks", "n_modes", "n", "n_shared", "shared_rows", "max_rows", "max_cols",
+                                       "n_outer", "rows")] + [("tables", C.c_void_p), ("offsets", C.c_void_p)]
+
+
 class MdpError(RuntimeError):
     def __init__(self, code, what):
         self.code = code
@@ -71,6 +76,13 @@ def lib():
         "mdp_householder_qr_batched": (i, [i, i, i, i, vp, ll, ll, vp, vp, vp]),
         "mdp_triangular_solve": (i, [i, i, vp, ll, i, vp, ll, vp]),
         "mdp_complex_matmul": (i, [i, i, i, vp, ll, ll, i, vp, ll, ll, i, vp, ll, ll, i, vp]),
+        "mdp_couple_buffer": (ll, [C.POINTER(mdp_couple)]),
+        "mdp_couple_grad_buffer": (ll, [C.POINTER(mdp_couple)]),
+        "mdp_couple_work_ints": (ll, [C.POINTER(mdp_couple)]),
+        "mdp_couple_solve": (i, [C.POINTER(mdp_couple)] + [vp] * 9),
+        "mdp_couple_grad": (i, [C.POINTER(mdp_couple)] + [vp] * 12),
+        "mdp_block_values": (i, [i, i, i] + [vp] * 7),
+        "mdp_block_values_grad": (i, [i, i, i] + [vp] * 9),
         "mdp_probe_rcp": (i, [vp, vp, i, vp]),
         "mdp_plan_read_tables": (i, [vp, i, vp, vp]),
         "mdp_plan_table_offsets": (i, [vp, i, C.POINTER(ll)]),

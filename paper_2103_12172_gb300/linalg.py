@@ -32,18 +32,23 @@ def check_work(work, index, what):
         raise _lib.MdpError(st, what)
 
 
-_pending = []   # (pinned host copy of status words, CUDA event after the copy) not yet checked
+_pending = []   # (pinned host copy of a work tensor, CUDA event after the copy, status words in it) not yet checked
+
+
+def defer_status(work, indices):
+    """Queue the status words work[indices] of QR launches for a later check_pending, without waiting for the
+    stream: their copy to pinned host memory is enqueued behind the launches."""
+    host = torch.empty(work.shape, dtype=torch.int32, pin_memory=True)
+    host.copy_(work, non_blocking=True)
+    ev = torch.cuda.Event()
+    ev.record()
+    _pending.append((host, ev, indices))
 
 
 def defer_check(factor):
-    """Queue the status words of a factor's QR launches for a later check_pending, without waiting
-    for the stream: their copy to pinned host memory is enqueued behind the launches."""
+    """defer_status for every QR launch behind a factor."""
     for work, index in factor.works:
-        host = torch.empty(1, dtype=torch.int32, pin_memory=True)
-        host.copy_(work[index:index + 1], non_blocking=True)
-        ev = torch.cuda.Event()
-        ev.record()
-        _pending.append((host, ev))
+        defer_status(work, [index])
 
 
 def check_pending(wait=False):
@@ -51,16 +56,16 @@ def check_pending(wait=False):
     have completed are examined (the others stay queued)."""
     global _pending
     keep = []
-    for host, ev in _pending:
+    for host, ev, indices in _pending:
         if wait:
             ev.synchronize()
         elif not ev.query():
-            keep.append((host, ev))
+            keep.append((host, ev, indices))
             continue
-        st = int(host[0])
-        if st != _lib.MDP_OK:
-            _pending = keep
-            raise _lib.MdpError(st, "mdp_householder_qr (deferred status)")
+        for st in (int(host[i]) for i in indices):
+            if st != _lib.MDP_OK:
+                _pending = keep
+                raise _lib.MdpError(st, "mdp_householder_qr (deferred status)")
     _pending = keep
 
 

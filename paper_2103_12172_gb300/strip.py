@@ -17,11 +17,12 @@ mdp_ap_adjoint_rec).
 """
 from __future__ import annotations
 
+import ctypes as C
 import math
 
 import torch
 
-from . import Plan, linalg
+from . import Plan, _lib, linalg
 
 
 class ProjectWithReceivers(torch.autograd.Function):
@@ -95,6 +96,148 @@ class LeastSquares(torch.autograd.Function):
         return grad_A, grad_b, None
 
 
+def _ptr(t):
+    return None if t is None else t.data_ptr()
+
+
+class _Blocks:
+    """Blocks [cols][len_j] of one tensor and the ranges of a stacked vector they act on, with the index
+    tensors on the device."""
+
+    def __init__(self, cols, lens, offs, device):
+        self.n, self.cols, self.lens = len(lens), cols, list(lens)
+        self.starts = [sum(lens[:j]) for j in range(len(lens))]
+        self.total, self.max = sum(lens), max(max(lens), 1)
+        self.ints = torch.tensor(self.lens + self.starts, dtype=torch.int32).to(device)
+        self.offs = torch.tensor(list(offs), dtype=torch.int64).to(device)
+        self.args = (self.n, self.cols, self.max, self.ints.data_ptr(), self.ints.data_ptr() + 4 * self.n,
+                     self.offs.data_ptr())
+
+
+class BlockValues(torch.autograd.Function):
+    """y_j = B_j v_j for every block of a _Blocks layout: B flat, v [blocks, cols], y stacked."""
+
+    @staticmethod
+    def forward(ctx, B, v, blocks):
+        v = v.contiguous()
+        y = torch.empty(max(blocks.total, 1), dtype=torch.complex128, device=B.device)[:blocks.total]
+        _lib.check(_lib.lib().mdp_block_values(*blocks.args, _ptr(B), _ptr(v), _ptr(y), linalg._stream()),
+                   "mdp_block_values")
+        ctx.save_for_backward(B, v)
+        ctx.blocks = blocks
+        return y
+
+    @staticmethod
+    def backward(ctx, gy):
+        B, v = ctx.saved_tensors
+        gy = gy.resolve_conj().contiguous()
+        gB = torch.empty_like(B) if ctx.needs_input_grad[0] else None
+        gv = torch.empty_like(v) if ctx.needs_input_grad[1] else None
+        _lib.check(_lib.lib().mdp_block_values_grad(*ctx.blocks.args, _ptr(B), _ptr(v), _ptr(gy), _ptr(gB), _ptr(gv),
+                                                    linalg._stream()), "mdp_block_values_grad")
+        return gB, gv, None
+
+
+class CoupledSystem:
+    """The index tables of mdp_couple for a structure of unknowns (LayeredStrip._structure) whose outer
+    sides have the given kinds ("robin", "dirichlet"), on the device; ok: the library takes the system."""
+
+    def __init__(self, st, kinds, M, rows, offs, device):
+        N, n, cols = len(rows), st["n"], st["col_sets"]
+        count = {}
+        for cj in cols:
+            for c in cj:
+                count[c] = count.get(c, 0) + 1
+        shared = sorted(c for c, v in count.items() if v > 1)
+        order = [[c for c in cj if count[c] == 1] + [c for c in cj if count[c] > 1] for cj in cols]
+        private = [sum(count[c] == 1 for c in cj) for cj in cols]
+        pos = {c: i for i, c in enumerate(shared)}
+        nmax, mmax = max(len(o) for o in order), max(rows)
+        s0 = [sum(len(order[i]) - private[i] for i in range(j)) for j in range(N)]
+        ms = sum(len(o) - p for o, p in zip(order, private))
+        per_col = [[[0] * nmax for _ in range(N)] for _ in range(6)]   # unk, slot0, neg0, slot1, rho, sidx
+        per_coef = [[[v] * (8 * M) for _ in range(N)] for v in (-1, 0, -1)]   # su, sf, se
+        touch = [[] for _ in range(n)]
+        sides = []                                                     # qj, qe, qr, qu
+        q = 0
+        for j in range(N):
+            entry = {}                                                 # unknown -> (slot0, neg0, slot1, q)
+            for side, spec in enumerate(st["sides"][j]):
+                z, o = side * M, (4 + side) * M
+                c = spec[1]
+                for m in range(M):
+                    if spec[0] == "if":
+                        entry[c + m] = (z + m, 0, -1, 0)
+                        entry[c + M + m] = (o + m, int(spec[2] < 0), -1, 0)
+                        links = [(z + m, c + m, 0), (o + m, c + M + m, int(spec[2] < 0))]
+                    elif kinds[q] == "robin":
+                        entry[c + m] = (z + m, 0, o + m, q)
+                        links = [(z + m, c + m, 0), (o + m, c + m, 2 + q)]
+                        per_coef[2][j][o + m] = q * M + m
+                    else:
+                        entry[c + m] = (o + m, 0, -1, 0)
+                        links = [(o + m, c + m, 0)]
+                        per_coef[2][j][z + m] = q * M + m
+                    for slot, u, f in links:
+                        per_coef[0][j][slot], per_coef[1][j][slot] = u, f
+                if spec[0] != "if":
+                    sides.append((j, o if kinds[q] == "robin" else z, o if kinds[q] == "robin" else -1, c))
+                    q += 1
+            for p, u in enumerate(order[j]):
+                for t, v in zip(per_col, (u,) + entry[u] + (pos.get(u, 0),)):
+                    t[j][p] = v
+                touch[u].append(j * nmax + p)
+        flat = [rows, [len(o) for o in order], private, s0, [sum(rows[:j]) for j in range(N)]]
+        flat += [r for t in per_col + per_coef for r in t]
+        flat += [(t + [-1, -1])[:2] for t in touch] + [shared] + [[s[i] for s in sides] for i in range(4)]
+        self.ints = torch.tensor([v for r in flat for v in r], dtype=torch.int32).to(device)
+        self.offs = torch.tensor(list(offs), dtype=torch.int64).to(device)
+        self.c = _lib.mdp_couple(N, M, n, len(shared), ms, mmax, nmax, q, sum(rows), self.ints.data_ptr(),
+                                 self.offs.data_ptr())
+        L = _lib.lib()
+        self.buffer, self.grad_buffer = L.mdp_couple_buffer(self.c), L.mdp_couple_grad_buffer(self.c)
+        self.work_ints = L.mdp_couple_work_ints(self.c)
+        self.ok = self.buffer > 0 and all(len(t) in (1, 2) for t in touch)
+        self.status = [N] + ([int(L.mdp_householder_qr_work_ints(N)) + 1] if shared else [])
+
+
+class CoupledSolve(torch.autograd.Function):
+    """The coefficients [N, 8 M] of every subdomain's boundary data from the projection columns `out`, the
+    outer sides' rho [sides] and eps [sides, M] and the sources' F [rows] or None, by mdp_couple_solve: the
+    least squares of LeastSquares on the structured system, assembled, solved and differentiated in a
+    few launches."""
+
+    @staticmethod
+    def forward(ctx, out, rho, eps, src, cs):
+        linalg.check_pending()                         # status words of earlier solves that have completed
+        dev = out.device
+        rho, eps = rho.resolve_conj().contiguous(), eps.resolve_conj().contiguous()
+        buf = torch.empty(cs.buffer, dtype=torch.complex128, device=dev)
+        work = torch.empty(cs.work_ints, dtype=torch.int32, device=dev)
+        x = torch.empty(cs.c.n, dtype=torch.complex128, device=dev)
+        coef = torch.empty((cs.c.n_blocks, 8 * cs.c.n_modes), dtype=torch.complex128, device=dev)
+        _lib.check(_lib.lib().mdp_couple_solve(cs.c, _ptr(out), _ptr(rho), _ptr(eps), _ptr(src), _ptr(buf), _ptr(work),
+                                               _ptr(x), _ptr(coef), linalg._stream()), "mdp_couple_solve")
+        linalg.defer_status(work, cs.status)           # checked later, without stalling the stream
+        ctx.save_for_backward(out, rho, src, buf, x, coef)
+        ctx.cs = cs
+        return coef
+
+    @staticmethod
+    def backward(ctx, g):
+        out, rho, src, buf, x, coef = ctx.saved_tensors
+        cs = ctx.cs
+        g = g.resolve_conj().contiguous()
+        tmp = torch.empty(cs.grad_buffer, dtype=torch.complex128, device=out.device)
+        gout = torch.empty_like(out) if ctx.needs_input_grad[0] else None
+        grho = torch.empty_like(rho)
+        geps = torch.empty((cs.c.n_outer, cs.c.n_modes), dtype=torch.complex128, device=out.device)
+        _lib.check(_lib.lib().mdp_couple_grad(cs.c, _ptr(out), _ptr(rho), _ptr(src), _ptr(buf), _ptr(x), _ptr(coef),
+                                              _ptr(g), _ptr(tmp), _ptr(gout), _ptr(grho), _ptr(geps), linalg._stream()),
+                   "mdp_couple_grad")
+        return gout, grho, geps, None, None
+
+
 def cheb_coeffs(fvals, n):
     """Chebyshev coefficients of the degree n-1 interpolant from values at the n first-kind
     Chebyshev points x_i = cos(pi (i + 1/2) / n) (i = 0..n-1): c_m = (2/n) sum_i f(x_i) T_m(x_i),
@@ -131,6 +274,8 @@ class LayeredStrip:
         self.plan.set_receivers(receiver_rows)
         self.layout = [self.plan.layout(j) for j in range(self.N)]
         self.rlayout = [self.plan.receiver_layout(j) for j in range(self.N)]
+        self._rec_blocks = None
+        self._consts = {}
 
     def neighbour(self, j, side):
         i, jj = self.pos[j]
@@ -170,13 +315,14 @@ class LayeredStrip:
         (without a source; the source terms are not differentiated)."""
         if self.source is not None and k.requires_grad:
             raise NotImplementedError("the k-gradient of the source terms is not implemented")
-        cvecs, rec = self.coefficients(k)
+        coef, rec = self._coefficients(k)
+        if self._rec_blocks is None:
+            self._rec_blocks = _Blocks(self.layout[0][1], [r[2] for r in self.rlayout], [r[3] for r in self.rlayout],
+                                       rec.device)
+        vals = BlockValues.apply(rec, coef, self._rec_blocks)
         res = []
-        for j in range(self.N):
-            row, m0, cnt, roff = self.rlayout[j]
-            nc = self.layout[j][1]
-            K = rec[roff:roff + nc * cnt].view(nc, cnt).transpose(0, 1)    # [cnt, 8M]
-            val = linalg.matmul(K, cvecs[j])
+        for j, val in enumerate(vals.split(self._rec_blocks.lens)):
+            row, m0, cnt, _ = self.rlayout[j]
             st = self.source_terms(j, self.plan_k(j))
             if st is not None:
                 val = val + st[1][row, m0:m0 + cnt]
@@ -243,12 +389,32 @@ class LayeredStrip:
         w = torch.full((M,), 2.0 / M, dtype=torch.float64, device=device)
         w[0] = 1.0 / M
         self._st = {"device": device, "n": n, "sides": sides, "col_sets": col_sets, "pts": pts,
-                    "cheb": (T.transpose(0, 1).to(torch.complex128).contiguous(), w)}
+                    "cheb": (T.transpose(0, 1).to(torch.complex128).contiguous(), w), "systems": {}}
         return self._st
+
+    def _scalars(self, vals, device):
+        """The values as one complex tensor: numbers that are no tensors are put on the device once."""
+        if not any(isinstance(v, torch.Tensor) for v in vals):
+            key = (str(device),) + tuple(complex(v) for v in vals)
+            t = self._consts.get(key)
+            if t is None:
+                if len(self._consts) >= 8:
+                    self._consts.clear()
+                t = self._consts[key] = torch.tensor(key[1:], dtype=torch.complex128).to(device)
+            return t
+        ts = [(v if isinstance(v, torch.Tensor) else torch.tensor(v)).to(torch.complex128) for v in vals]
+        if len({t.device for t in ts}) > 1:
+            ts = [t.to(device) for t in ts]
+        return torch.stack(ts).to(device)
 
     def coefficients(self, k):
         """The Chebyshev coefficients [c^(0) sides 1..4, c^(1) sides 1..4] of every layer's boundary
-        data from the coupled least-squares solve, and the receiver output of the projection.
+        data from the coupled least-squares solve, and the receiver output of the projection."""
+        coef, rec = self._coefficients(k)
+        return list(coef.unbind(0)), rec
+
+    def _coefficients(self, k):
+        """coefficients() as one tensor [N, 8 M].
         Outer side of unknown block u: alpha c0 + beta c1 = d (d the Chebyshev coefficients of
         the data); with beta != 0 the unknown is c0 and the side's rows read Q0 - (alpha/beta) Q1
         against u and -Q1 d / beta on the right; with beta = 0 the unknown is c1 (rows Q1) and
@@ -256,18 +422,44 @@ class LayeredStrip:
         M, N = self.M, self.N
         out, rec = ProjectWithReceivers.apply(k, self.plan)
         st = self._structure(out.device)
-        n = st["n"]
         # boundary data of every outer side, analysed into Chebyshev coefficients in one product
         bcs, phis = [], []
         for j in range(N):
+            kj = None
             for side, spec in zip((1, 2, 3, 4), st["sides"][j]):
                 if spec[0] == "outer":
+                    kj = k[j] if kj is None else kj
                     x, y = st["pts"][(j, side)]
-                    alpha, beta, phi = self.bc(j, side, k[j], x, y)
+                    alpha, beta, phi = self.bc(j, side, kj, x, y)
                     bcs.append((alpha, beta))
                     phis.append(phi.to(torch.complex128))
         Tt, w = st["cheb"]
         d_all = linalg.matmul(torch.stack(phis), Tt) * w if phis else None   # [outer sides, M]
+        kinds = tuple("robin" if beta != 0 else "dirichlet" for _, beta in bcs)
+        cs = st["systems"].get(kinds)
+        if cs is None:
+            cs = st["systems"][kinds] = CoupledSystem(st, kinds, M, [lay[0] for lay in self.layout],
+                                                      [lay[2] for lay in self.layout], out.device)
+        if not cs.ok:
+            return torch.stack(self._dense_coefficients(out, bcs, d_all, st)), rec
+        if bcs:
+            div = self._scalars([b if kd == "robin" else a for (a, b), kd in zip(bcs, kinds)], out.device)
+            rho = -self._scalars([a if kd == "robin" else 0.0 for (a, b), kd in zip(bcs, kinds)], out.device) / div
+            eps = d_all / div[:, None]
+        else:
+            rho = eps = torch.empty(0, dtype=torch.complex128, device=out.device)
+        src = [self.source_terms(j, self.plan_k(j)) for j in range(N)]
+        if any(t is not None for t in src):
+            src = torch.cat([torch.zeros(lay[0], dtype=torch.complex128, device=out.device) if t is None else t[0].reshape(-1)
+                             for t, lay in zip(src, self.layout)])
+        else:
+            src = None
+        return CoupledSolve.apply(out, rho, eps, src, cs), rec
+
+    def _dense_coefficients(self, out, bcs, d_all, st):
+        """The coefficients by single tensor operations and LeastSquares, for systems CoupledSolve does not
+        take (a layer with fewer gamma nodes than unknowns, or triangles beyond a CTA's shared memory)."""
+        M, N, n = self.M, self.N, st["n"]
         A_rows, b_rows, coef = [], [], []
         q = 0
         for j in range(N):
@@ -331,17 +523,18 @@ class LayeredStrip:
                     parts0.append(xsol[c:c + M])
                     parts1.append(sgn * xsol[c + M:c + 2 * M])
             cvecs.append(torch.cat(parts0 + parts1))
-        return cvecs, rec
+        return cvecs
 
 
 def incident_impedance_bc(theta):
     """Outer data of config `strip4x1`: impedance sides du/dn + i k_j u = phi with phi from the
     plane wave exp(i k_j (x cos theta + y sin theta)) of the layer's own wavenumber."""
+    ct, sn = math.cos(theta), math.sin(theta)
+    dirs = {1: -sn, 2: sn, 3: -ct, 4: ct}   # outward normal times direction
+
     def bc(j, side, kj, x, y):
-        kx, ky = kj * math.cos(theta), kj * math.sin(theta)
-        u = torch.exp(1j * (kx * x + ky * y))
-        dn = {1: -1j * ky, 2: 1j * ky, 3: -1j * kx, 4: 1j * kx}[side] * u
-        return 1j * kj, 1.0, dn + 1j * kj * u
+        ik = 1j * kj
+        return ik, 1.0, torch.exp(ik * torch.add(x * ct, y, alpha=sn)) * (ik * (1.0 + dirs[side]))
     return bc
 
 

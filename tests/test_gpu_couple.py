@@ -1,0 +1,49 @@
+"""The coupled solve of a layout in a few launches (mdp_couple_solve, mdp_couple_grad) against the same
+system by single tensor operations and the dense least squares (LayeredStrip._dense_coefficients): a strip and
+a block of 2 x 2, Robin sides with wavenumber-dependent and constant data, Dirichlet sides, grids of
+different sizes. Bar: receivers and gradients to 1e-8 (rounding, 1e-16 with a few hundred terms, in systems of
+condition 1e7)."""
+import pytest
+
+import workloads as W
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+LAYOUTS = {"one": ([(0, 0)], [33]), "strip3": ([(0, 0), (1, 0), (2, 0)], [33, 41, 33]),
+           "block": ([(0, 0), (1, 0), (0, 1), (1, 1)], [33, 45, 45, 33])}
+
+
+def bc(j, side, kj, x, y):
+    u = torch.exp(1j * (kj * x * 0.8 + 2.0 * y))
+    if side == 1:                                   # Dirichlet
+        return 1.0 + 0.0 * kj, 0.0, u
+    if side == 2:                                   # constants
+        return 2.0 + 1j, 0.5, u * (1.0 + x)
+    return 1j * kj, 1.0 + 0.1 * kj, (1j * kj + 0.3) * u
+
+
+@pytest.mark.parametrize("M", [5, 8])
+@pytest.mark.parametrize("name", list(LAYOUTS))
+def test_coupled_solve_and_gradient_are_those_of_the_dense_path(mdp, name, M):
+    from paper_2103_12172_gb300.strip import LayeredStrip
+    pos, grids = LAYOUTS[name]
+    ks = [4.0 + 0.7 * j for j in range(len(pos))]
+    subs = [W.unit_subdomain(i, jj, n, k, W.AP_DIRX_SOMMY, M) for (i, jj), n, k in zip(pos, grids, ks)]
+    got = []
+    for dense in (False, True):
+        lay = LayeredStrip(subs, bc, [s.ny // 2 for s in subs], positions=pos)
+        k = torch.tensor(ks, dtype=torch.float64, device="cuda", requires_grad=True)
+        if dense:
+            lay.receivers(k.detach())
+            systems = lay._st["systems"]
+            assert all(cs.ok for cs in systems.values())
+            for cs in systems.values():
+                cs.ok = False
+        u = lay.receivers(k)
+        w = [torch.linspace(0.2, 1.0, v.numel(), device="cuda") for v in u]
+        loss = sum(((v - 0.3j).abs().square() * t).sum() for v, t in zip(u, w))
+        (g,) = torch.autograd.grad(loss, k)
+        got.append((torch.cat(u).detach(), g, torch.cat([c for c in lay.coefficients(k.detach())[0]])))
+    for a, b in zip(*got):
+        assert (a - b).abs().max() < 1e-8 * b.abs().max()
