@@ -32,6 +32,10 @@
 //     release store of k + 2 to the matrix's progress counter;
 //   - other columns take a dot pass, one reduction and an update pass per reflector, v_k read
 //     from L2 into registers once per pass (rows beyond the register cache are read again).
+// What bounds it: a reflector's chain, some 5 us of dependent FP64 instructions (64 cycles each for a warp) and
+// 2 us through L2 (counter, then column), and, early on, the 4 columns of a CTA. At 4 x (856 x 144) 1.65 ms,
+// 288 x 144 1.02 ms; 1.76 and 1.11 with one more division and 6 instead of 4 FP64 instructions per updated
+// element, a fence and an acquire of every thread beside the barriers, and a sleep between looks at the counters.
 // Every wait is on a published counter and bounded. The chain of a matrix depends only on its
 // own earlier reflectors, so with every CTA resident the waits end. Reductions run in a fixed
 // order: the result does not depend on timing.
@@ -71,7 +75,7 @@ __device__ __forceinline__ void st_release_gpu(int *p, int v) {
 
 // a - v s (complex), with explicit FMAs so that every thread that evaluates it gets the same bits
 __device__ __forceinline__ double2 sub_vs(double2 a, double2 v, double2 s) {
-  return make_double2(a.x - fma(v.x, s.x, -v.y * s.y), a.y - fma(v.x, s.y, v.y * s.x));
+  return make_double2(fma(-v.x, s.x, fma(v.y, s.y, a.x)), fma(-v.x, s.y, fma(-v.y, s.x, a.y)));
 }
 
 // Reduce-scatter of 8 values over a warp: lane l returns the warp's total of value (l >> 2) & 7
@@ -114,8 +118,8 @@ __device__ __forceinline__ void block_sum8(const double (&v)[8], double *red, do
 // The reflector of a column from alpha = x(c) and xn2 = ||x(c+1:)||^2: beta, tau, and
 // inv = 1 / (alpha - beta); false if the column is already beta e_c with beta real (H = I).
 // With g = beta - Re(alpha) (no cancellation: beta has the sign opposite to Re(alpha)),
-// tau = (g - i Im(alpha)) / beta and inv = (-g - i Im(alpha))^* / (g^2 + Im(alpha)^2): two
-// independent divisions.
+// tau = (g - i Im(alpha)) / beta and inv = (-g - i Im(alpha))^* / (g^2 + Im(alpha)^2): one reciprocal
+// square root (a Newton step each for the norm and its reciprocal) and one independent division.
 __device__ __forceinline__ bool reflector_of(double2 a, double xn2, double &beta, double2 &tau, double2 &inv) {
   if (xn2 == 0.0 && a.y == 0.0) {
     beta = a.x;
@@ -123,10 +127,11 @@ __device__ __forceinline__ bool reflector_of(double2 a, double xn2, double &beta
     inv = make_double2(0.0, 0.0);
     return false;
   }
-  const double nrm = sqrt(fma(a.x, a.x, fma(a.y, a.y, xn2)));
+  const double s = fma(a.x, a.x, fma(a.y, a.y, xn2)), y = rsqrt(s), n0 = s * y;
+  const double nrm = fma(0.5 * y, fma(-n0, n0, s), n0), rn = fma(y, fma(-nrm, y, 1.0), y);
   beta = a.x >= 0.0 ? -nrm : nrm;
   const double g = beta - a.x;
-  const double rb = 1.0 / beta, rd = 1.0 / fma(g, g, a.y * a.y);
+  const double rb = a.x >= 0.0 ? -rn : rn, rd = 1.0 / fma(g, g, a.y * a.y);
   inv = make_double2(-g * rd, -a.y * rd);   // conj(alpha - beta) / |alpha - beta|^2
   tau = make_double2(g * rb, -a.y * rb);
   return true;
@@ -176,8 +181,7 @@ __global__ void __launch_bounds__(kQrThreads) k_qr_cta(QrArgs q) {
     return gcol(b, c);
   };
   auto publish = [&](int b, int c) {   // after every thread wrote its part of column (b, c)
-    __threadfence();
-    __syncthreads();
+    __syncthreads();                   // the release is cumulative: it covers the other threads' writes
     if (tid == 0) st_release_gpu(q.progress + b, c + 1);
   };
 
@@ -226,6 +230,7 @@ __global__ void __launch_bounds__(kQrThreads) k_qr_cta(QrArgs q) {
     if (warp == 0) {
       __syncwarp();   // tid 0's updates of nxt
       const long long t0 = clock64();
+      int spins = 0;
       while (true) {
         long long best = 0x7fffffffffffffffLL;
         int pending = 0;
@@ -275,6 +280,7 @@ __global__ void __launch_bounds__(kQrThreads) k_qr_cta(QrArgs q) {
           }
           break;
         }
+        if (++spins & 15) continue;   // a look at the abort flag costs as much as one at the counters
         const int ab = ld_acquire_gpu(q.status + 1);
         const bool late = __shfl_sync(0xffffffffu, clock64() - t0 > kQrWaitCycles, 0);
         if (__any_sync(0xffffffffu, ab != 0) || late) {
@@ -287,7 +293,6 @@ __global__ void __launch_bounds__(kQrThreads) k_qr_cta(QrArgs q) {
           }
           break;
         }
-        __nanosleep(64);
       }
     }
     __syncthreads();
@@ -295,7 +300,7 @@ __global__ void __launch_bounds__(kQrThreads) k_qr_cta(QrArgs q) {
     if (it.kind == 2) return;
     if (it.kind == 1) break;
     const int b = it.b, k = it.j;
-    (void)ld_acquire_gpu(q.progress + b);   // each thread's own acquire of the published reflector
+    // warp 0's acquire and the barrier order the reads of the reflector below, which go to L2
     const double2 *vg = gcol(b, k);
     const double2 t = __ldcg(q.tau + (long long)b * q.n + k);
     const bool apply = t.x != 0.0 || t.y != 0.0;
@@ -375,8 +380,6 @@ __global__ void __launch_bounds__(kQrThreads) k_qr_cta(QrArgs q) {
       const bool refl = reflector_of(alpha, xn2, beta, tn, inv);
       const double2 si = cmul(s, inv);   // (a - s v) inv = a inv - (s inv) v
       double2 *gc = gcol(b, k + 1);
-      if (SMEM)   // rows of R above row k are final: copy them out
-        for (int i = tid; i < k; i += kQrThreads) gc[i] = x[i];
 #pragma unroll
       for (int u = 0; u < kQrRv; ++u) {
         if (u >= nu) break;
@@ -402,6 +405,8 @@ __global__ void __launch_bounds__(kQrThreads) k_qr_cta(QrArgs q) {
         nxt[it.slot[0]] = k + 1;
       }
       publish(b, k + 1);
+      if (SMEM)   // rows of R above row k are final: copy them out
+        for (int i = tid; i < k; i += kQrThreads) gc[i] = x[i];
       continue;
     }
     const int nc = it.nc;
