@@ -12,7 +12,8 @@
 //
 // A pass is some 25 kernels where the assembly, the permutations and their gradients as single tensor
 // operations were 260 (750 with the gradient), bound by their launches: 4 layers of 129^2, 24 modes per side,
-// 7.4 -> 4.2 ms to the receivers, 21.7 -> 6.1 ms with the gradient by the wavenumbers. Each kernel is a stream
+// 7.4 -> 4.2 ms to the receivers, 21.7 -> 6.1 ms with the gradient by the wavenumbers (3.3 and 4.5 with the
+// boundary data of all sides at once and a shorter QR). Each kernel is a stream
 // over Q (10 MB there, in L2) with an FP64 product or two per element, 5 to 15 us; the triangular solves take
 // the two levels' triangles, so that the chain is the shared unknowns and one subdomain's own ones instead of
 // all (195 us for 144 + 72, 309 us for all 384 in one CTA).

@@ -389,7 +389,8 @@ class LayeredStrip:
         w = torch.full((M,), 2.0 / M, dtype=torch.float64, device=device)
         w[0] = 1.0 / M
         self._st = {"device": device, "n": n, "sides": sides, "col_sets": col_sets, "pts": pts,
-                    "cheb": (T.transpose(0, 1).to(torch.complex128).contiguous(), w), "systems": {}}
+                    "cheb": (T.transpose(0, 1).to(torch.complex128).contiguous(), w), "systems": {}, "layer": {},
+                    "outer": list(pts), "xy": [torch.stack(t) for t in zip(*pts.values())]}
         return self._st
 
     def _scalars(self, vals, device):
@@ -423,31 +424,47 @@ class LayeredStrip:
         out, rec = ProjectWithReceivers.apply(k, self.plan)
         st = self._structure(out.device)
         # boundary data of every outer side, analysed into Chebyshev coefficients in one product
-        bcs, phis = [], []
-        for j in range(N):
-            kj = None
-            for side, spec in zip((1, 2, 3, 4), st["sides"][j]):
-                if spec[0] == "outer":
-                    kj = k[j] if kj is None else kj
-                    x, y = st["pts"][(j, side)]
-                    alpha, beta, phi = self.bc(j, side, kj, x, y)
-                    bcs.append((alpha, beta))
-                    phis.append(phi.to(torch.complex128))
+        alphas = bcs = phi = None
+        if hasattr(self.bc, "sides") and st["outer"]:
+            layer = st["layer"].get(str(k.device))
+            if layer is None:
+                layer = st["layer"][str(k.device)] = torch.tensor([j for j, _ in st["outer"]]).to(k.device)
+            alphas, betas, phi = self.bc.sides(k.index_select(0, layer), [s for _, s in st["outer"]], *st["xy"])
+            if any(beta == 0 for beta in betas):
+                alphas, bcs = None, list(zip(alphas.unbind(0), betas))
+        else:
+            bcs, phis = [], []
+            for j in range(N):
+                kj = None
+                for side, spec in zip((1, 2, 3, 4), st["sides"][j]):
+                    if spec[0] == "outer":
+                        kj = k[j] if kj is None else kj
+                        x, y = st["pts"][(j, side)]
+                        alpha, beta, ph = self.bc(j, side, kj, x, y)
+                        bcs.append((alpha, beta))
+                        phis.append(ph.to(torch.complex128))
+            betas = [beta for _, beta in bcs]
+            phi = torch.stack(phis) if phis else None
         Tt, w = st["cheb"]
-        d_all = linalg.matmul(torch.stack(phis), Tt) * w if phis else None   # [outer sides, M]
-        kinds = tuple("robin" if beta != 0 else "dirichlet" for _, beta in bcs)
+        d_all = linalg.matmul(phi, Tt) * w if phi is not None else None   # [outer sides, M]
+        kinds = tuple("robin" if beta != 0 else "dirichlet" for beta in betas)
         cs = st["systems"].get(kinds)
         if cs is None:
             cs = st["systems"][kinds] = CoupledSystem(st, kinds, M, [lay[0] for lay in self.layout],
                                                       [lay[2] for lay in self.layout], out.device)
         if not cs.ok:
+            bcs = list(zip(alphas.unbind(0), betas)) if bcs is None else bcs
             return torch.stack(self._dense_coefficients(out, bcs, d_all, st)), rec
-        if bcs:
-            div = self._scalars([b if kd == "robin" else a for (a, b), kd in zip(bcs, kinds)], out.device)
-            rho = -self._scalars([a if kd == "robin" else 0.0 for (a, b), kd in zip(bcs, kinds)], out.device) / div
-            eps = d_all / div[:, None]
-        else:
+        if not betas:
             rho = eps = torch.empty(0, dtype=torch.complex128, device=out.device)
+        else:
+            if bcs is None:
+                div = self._scalars(betas, out.device)
+            else:
+                div = self._scalars([b if kd == "robin" else a for (a, b), kd in zip(bcs, kinds)], out.device)
+                alphas = self._scalars([a if kd == "robin" else 0.0 for (a, b), kd in zip(bcs, kinds)], out.device)
+            rho = -alphas / div
+            eps = d_all / div[:, None]
         src = [self.source_terms(j, self.plan_k(j)) for j in range(N)]
         if any(t is not None for t in src):
             src = torch.cat([torch.zeros(lay[0], dtype=torch.complex128, device=out.device) if t is None else t[0].reshape(-1)
@@ -526,16 +543,28 @@ class LayeredStrip:
         return cvecs
 
 
-def incident_impedance_bc(theta):
+class incident_impedance_bc:
     """Outer data of config `strip4x1`: impedance sides du/dn + i k_j u = phi with phi from the
-    plane wave exp(i k_j (x cos theta + y sin theta)) of the layer's own wavenumber."""
-    ct, sn = math.cos(theta), math.sin(theta)
-    dirs = {1: -sn, 2: sn, 3: -ct, 4: ct}   # outward normal times direction
+    plane wave exp(i k_j (x cos theta + y sin theta)) of the layer's own wavenumber. sides() gives the data of
+    many sides at once: their layers' wavenumbers [S], side numbers, points x, y [S, M] -> alpha [S],
+    the numbers beta, phi [S, M]; LayeredStrip takes it where a boundary condition has it."""
 
-    def bc(j, side, kj, x, y):
+    def __init__(self, theta):
+        self.ct, self.sn = math.cos(theta), math.sin(theta)
+        self.dirs = {1: -self.sn, 2: self.sn, 3: -self.ct, 4: self.ct}   # outward normal times direction
+        self._key = self._n = None
+
+    def __call__(self, j, side, kj, x, y):
         ik = 1j * kj
-        return ik, 1.0, torch.exp(ik * torch.add(x * ct, y, alpha=sn)) * (ik * (1.0 + dirs[side]))
-    return bc
+        return ik, 1.0, torch.exp(ik * torch.add(x * self.ct, y, alpha=self.sn)) * (ik * (1.0 + self.dirs[side]))
+
+    def sides(self, ks, side, x, y):
+        ik = 1j * ks.to(x.device)
+        key = (tuple(side), x.dtype, x.device)
+        if key != self._key:   # the factors of these sides, on the device once
+            self._n, self._key = torch.tensor([1.0 + self.dirs[s] for s in side], dtype=x.dtype).to(x.device), key
+        n = self._n
+        return ik, [1.0] * len(side), torch.exp(ik[:, None] * torch.add(x * self.ct, y, alpha=self.sn)) * (ik * n)[:, None]
 
 
 def receiver_row(sub, y_target=0.9):
