@@ -15,8 +15,11 @@
 //   k_factor_chain  the pivot recurrences, the only sequential part: one thread per (mode,
 //                   table) streams the rows with O(1) state and stores each raw LU row (l, d,
 //                   1/d, du, du2, swap) in place in its table row. A chain is a long sequence of
-//                   dependent FP64 operations, so it does nothing else, and its interior
-//                   no-swap steps take a real-coefficient fast path.
+//                   dependent FP64 operations (64 cycles each for a warp, whatever its lanes), so it
+//                   does nothing else, and its interior steps take real coefficients: 13
+//                   operations after a kept pivot, 18 after a swap, 6 for a swap. Propagating modes
+//                   swap every few rows, each at its own, so they have a warp each; 4 x 257^2: 471 us
+//                   with 32 neighbouring modes to a warp and general complex steps around swaps.
 //   k_factor_rows   everything row-local, one block per mode: u1 = du/d, u2 = du2/d, the
 //                   sweep rows (which also need row i+1's pivot, read through shared memory in
 //                   chunks so the rows can be rewritten in place), the dT/dk rows, and the runs
@@ -141,9 +144,8 @@ __device__ __forceinline__ int mode_owner(const SubDesc *subs, int n_subs, int &
 }
 
 // The pivoted LU of rows 0..n-1 of T_q (diagonal of row `mod` reduced by sigma), calling
-// out(i, l, d, dinv, du, du2, sw) for every row in order. Interior steps (real a, dd entries,
-// super-diagonal of the pivot row still the original a) that keep the pivot take the fast path
-// with real coefficients. Returns false (status set) on a singular pivot.
+// out(i, l, d, dinv, du, du2, sw) for every row in order. Interior steps (real a, dd entries) take
+// real coefficients. Returns false (status set) on a singular pivot.
 template <class Out>
 __device__ bool lu_chain(const ModeRows &M, int n, int mod, cplx sigma, double tol2, int *status, Out out) {
   const int N = M.N;
@@ -159,31 +161,45 @@ __device__ bool lu_chain(const ModeRows &M, int n, int mod, cplx sigma, double t
   ent(0, dl0, g, u);
   bool u_is_a = !M.cplx_ap;   // u still equals the original interior entry a
   int i = 0;
-  double r = 0.0;             // 1/|g|^2 of the previous fast step
+  double r = 0.0;             // 1/|g|^2 of the previous kept pivot
+  const double ia = crecip(cmk(a, 0.0)).re;
   while (i < n - 1) {
-    if (u_is_a) {
-      // Fast path: keep the pivot while |g| >= a. Then |g|^2 >= a^2 > tol2 (a >= 1/(3h^2) is
-      // within a factor 7 of max|T|), so no singularity test is needed. The pivots of a mode
-      // settle to a fixed point, so 1/|g|^2 is refined from the previous row's: with
-      // e = 1 - n2 r0, 1/n2 = r0 / (1 - e) = r0 (1 + e + e^2) + O(e^3 r0), full precision for
-      // |e| < 2^-20; otherwise a division.
-      // The loop-carried chain is g -> |g|^2 -> 1/|g|^2 -> g' = dd - a^2 conj(g)/|g|^2; the
-      // swap test and the row's outputs branch off it.
-      const double a2dd = a2;
+    // Interior steps: the pivot is kept while |g| >= a. Then |g|^2 >= a^2 > tol2 (a >= 1/(3h^2) is
+    // within a factor 7 of max|T|), so no singularity test is needed. The pivots of a mode
+    // settle to a fixed point, so 1/|g|^2 is refined from the previous row's: with
+    // e = 1 - n2 r0, 1/n2 = r0 / (1 - e) = r0 (1 + e + e^2) + O(e^3 r0), full precision for
+    // |e| < 2^-20; otherwise a division.
+    // The loop-carried chain is g -> |g|^2 -> 1/|g|^2 -> g' = dd - a u conj(g)/|g|^2 (u = a after a kept
+    // pivot); the row's outputs branch off it. A swap takes row i+1 = (a, dd, a) as the pivot row.
+    if (i > 0 || !M.cplx_ap)
       for (; i < fast_end; ++i) {
         const double n2 = fma(g.re, g.re, g.im * g.im);
-        const double e = fma(-n2, r, 1.0);
-        double rn = fma(r, fma(e, e, e), r);
-        if (!(fabs(e) < 0x1p-20)) rn = rcp_pos(n2);
-        if (n2 < a2) break;
-        r = rn;
-        const double gr = g.re * r, gi = g.im * r;   // 1/g = (gr, -gi)
-        const cplx gnext = cmk(fma(-a2dd, gr, dd), a2dd * gi);
-        out(i, cmk(a * gr, -a * gi), g, cmk(gr, -gi), cmk(a, 0.0), cmk(0.0, 0.0), (uint8_t)0);
-        g = gnext;
+        if (n2 >= a2) {
+          const double e = fma(-n2, r, 1.0);
+          double rn = fma(r, fma(e, e, e), r);
+          if (!(fabs(e) < 0x1p-20)) rn = rcp_pos(n2);
+          r = rn;
+          const double gr = g.re * r, gi = g.im * r;   // 1/g = (gr, -gi)
+          cplx gnext;
+          if (u_is_a) gnext = cmk(fma(-a2, gr, dd), a2 * gi);
+          else {
+            const double lr = a * u.re, li = a * u.im;
+            gnext = cmk(fma(-lr, gr, fma(-li, gi, dd)), fma(lr, gi, -li * gr));
+          }
+          out(i, cmk(a * gr, -a * gi), g, cmk(gr, -gi), u, cmk(0.0, 0.0), (uint8_t)0);
+          g = gnext;
+          u = cmk(a, 0.0);
+          u_is_a = true;
+        } else {
+          if (i == n - 2) break;
+          const cplx f = cmk(g.re * ia, g.im * ia);
+          out(i, f, cmk(a, 0.0), cmk(ia, 0.0), cmk(dd, 0.0), cmk(a, 0.0), (uint8_t)1);
+          g = cmk(fma(-f.re, dd, u.re), fma(-f.im, dd, u.im));
+          u = cmk(-f.re * a, -f.im * a);
+          u_is_a = false;
+        }
       }
-      if (i >= n - 1) break;
-    }
+    if (i >= n - 1) break;
     cplx lsub, gi, ui, gn, un, dln;
     ent(i, lsub, gi, ui);
     ent(i + 1, dln, gn, un);
@@ -265,17 +281,27 @@ __device__ void chain_sweep(const SubDesc &d, int q, double *tab, int *status) {
            });
 }
 
-__global__ void __launch_bounds__(32) k_factor_chain(const SubDesc *subs, int n_subs, int n_modes, double *tab,
-                                                      uint8_t *piv, int *status, int all) {
-  int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= 2 * n_modes) return;
-  const bool sweep = t >= n_modes;
-  if (sweep) t -= n_modes;
-  int si = mode_owner(subs, n_subs, t);
+// Blocks of one warp: n_prop of them with a propagating mode each, then the other modes 32 to a block; and
+// the same again for the sweep tables.
+__global__ void __launch_bounds__(32) k_factor_chain(const SubDesc *subs, int n_subs, int n_prop, int n_rest, double *tab,
+                                                     uint8_t *piv, int *status, int all) {
+  const int per = n_prop + (n_rest + 31) / 32, sweep = blockIdx.x >= per, blk = blockIdx.x - (sweep ? per : 0);
+  const bool prop = blk < n_prop;
+  int t = prop ? blk : (blk - n_prop) * 32 + threadIdx.x;
+  if (prop ? threadIdx.x > 0 : t >= n_rest) return;
+  int si = 0;
+  for (; si < n_subs; ++si) {
+    const SubDesc &d = subs[si];
+    if (d.leader != si) continue;
+    const int n = prop ? d.n_prop : d.Nq - d.n_prop;
+    if (t < n) break;
+    t -= n;
+  }
   if (si >= n_subs) return;
+  const int q = prop ? t + 1 : subs[si].n_prop + t + 1;
   if (sweep) {
-    if (all || !subs[si].tc_cols) chain_sweep(subs[si], t + 1, tab, status);
-  } else chain_full(subs[si], t + 1, tab, piv, status);
+    if (all || !subs[si].tc_cols) chain_sweep(subs[si], q, tab, status);
+  } else chain_full(subs[si], q, tab, piv, status);
 }
 
 constexpr int kRowsThreads = 256;
@@ -308,9 +334,9 @@ __global__ void __launch_bounds__(kRowsThreads) k_factor_rows(const SubDesc *sub
   const ModeRows &M = Ms;
   const int N = M.N;
   double *sg = tab + d.seg_off + 5 * (q - 1);
-  // ---- dT/dk rows (sub, diag, super)
+  // ---- dT/dk rows (sub, diag, super): only the gradient pass by sweeps reads them
   double *dT = tab + d.dT_off + (long long)(q - 1) * N * 6;
-  for (int i = tid; i < N; i += kRowsThreads) {
+  for (int i = d.tc_cols && !all ? N : tid; i < N; i += kRowsThreads) {
     cplx ts = cmk(M.da, 0.0), tg = cmk(M.ddd, 0.0), tu = cmk(M.da, 0.0);
     if (M.cplx_ap && i == 0) { tg = M.tp; tu = M.tm; ts = cmk(0.0, 0.0); }
     if (M.cplx_ap && i == N - 1) { tg = M.tp; ts = M.tm; tu = cmk(0.0, 0.0); }
@@ -419,14 +445,14 @@ __global__ void k_probe_rcp(const double *x, double *y, int n) {
 // FP64 unit while there are fewer warps than SMs. The row kernel: one block per mode.
 cudaError_t launch_factor_to(const mdp_plan *p, const SubDesc *ds, double *tab, uint8_t *piv, int *status, bool all,
                              cudaStream_t st) {
-  int n_modes = 0;
+  int n_modes = 0, n_prop = 0;
   bool sweeps = all;
   for (size_t i = 0; i < p->subs.size(); ++i) {
     sweeps = sweeps || !p->subs[i].d.tc_cols;
-    if (p->subs[i].d.leader == (int)i) n_modes += p->subs[i].d.Nq;
+    if (p->subs[i].d.leader == (int)i) { n_modes += p->subs[i].d.Nq; n_prop += p->subs[i].d.n_prop; }
   }
-  const int threads = sweeps ? 2 * n_modes : n_modes;
-  k_factor_chain<<<(threads + 31) / 32, 32, 0, st>>>(ds, (int)p->subs.size(), n_modes, tab, piv, status, all);
+  const int blocks = n_prop + (n_modes - n_prop + 31) / 32;
+  k_factor_chain<<<sweeps ? 2 * blocks : blocks, 32, 0, st>>>(ds, (int)p->subs.size(), n_prop, n_modes - n_prop, tab, piv, status, all);
   k_factor_rows<<<n_modes, kRowsThreads, 0, st>>>(ds, (int)p->subs.size(), tab, all);
   return cudaGetLastError();
 }

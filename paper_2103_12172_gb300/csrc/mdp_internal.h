@@ -5,6 +5,7 @@
 #include <string>
 #include <algorithm>
 #include <cstdlib>
+#include <cmath>
 #include <cstring>
 #include <cuda_runtime.h>
 #include "mdp.h"
@@ -46,6 +47,7 @@ struct SubDesc {
   int leader;       // index of the subdomain owning this one's tables (itself unless deduplicated)
   int tc_cols;      // 1: the projection, the gradient pass and the full-grid solves run through the separable
                     // Green's function (kernels_sep.cu, kernels_sepadj.cu, kernels_full.cu); 0: per-mode sweeps
+  int n_prop;       // modes q = 1 .. n_prop below the cutoff (a matter of scheduling: k_factor_chain)
   double h, k;
   double x0, x1, y0, y1, ax0, ay0;
   double c0, c1, c2;  // 9-point coefficients: centre, edge, corner (Eq. FD_scheme)
@@ -148,6 +150,11 @@ struct SepGeo {
   int nt1, nt3;        // MID, SYN: tiles of 32 outputs
   int ND;              // distinct Toeplitz blocks per (output, source) column
 };
+// modes below the cutoff at the subdomain's k: 4 sin^2(pi q / (2 Nx)) (1/h^2 + k^2/12) < k^2
+inline int propagating_modes(const SubDesc &d) {
+  const double s = 0.5 * std::sqrt(d.k * d.k / (1.0 / (d.h * d.h) + d.k * d.k / 12.0));
+  return s >= 1.0 ? d.Nq : std::min(d.Nq, (int)(2.0 * d.Nx / M_PI * std::asin(s)) + 1);
+}
 inline __host__ __device__ SepGeo sep_geo(const SubDesc &d) {
   SepGeo g;
   g.ncls = d.xsym ? 2 : 1;

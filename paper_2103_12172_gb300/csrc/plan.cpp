@@ -90,6 +90,7 @@ static mdp_status geometry(const mdp_subdomain &in, HostSub &hs, unsigned flags,
   d.c0 = -4.0 / h2 + 4.0 / (6.0 * h2) + 8.0 * k2 / 12.0;
   d.dc1 = in.k / 6.0;
   d.dc0 = 8.0 * in.k / 6.0;
+  d.n_prop = propagating_modes(d);
   // gamma nodes in row-major order with side ownership
   hs.gamma_nm.clear(); hs.owner.clear(); hs.rho.clear(); hs.s.clear(); hs.L.clear();
   const double lx = in.x1 - in.x0, ly = in.y1 - in.y0;
@@ -626,6 +627,7 @@ mdp_status set_k_fields(mdp_plan *p, const double *k) {
     hs.d.c0 = -4.0 / h2 + 4.0 / (6.0 * h2) + 8.0 * k2 / 12.0;
     hs.d.dc1 = k[i] / 6.0;
     hs.d.dc0 = 8.0 * k[i] / 6.0;
+    hs.d.n_prop = propagating_modes(hs.d);
   }
   return MDP_OK;
 }
