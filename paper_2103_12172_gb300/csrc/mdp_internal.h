@@ -485,6 +485,8 @@ struct mdp_plan {
   unsigned char *d_adj = nullptr;        // gradient tables (kernels_sepadj.cu), one set: rebuilt by the gradient
   long long adj_bytes = 0, adj_masks = 0;   // pass when the wavenumbers have changed since (adj_stale)
   bool adj_stale = true, adj_sines = false;
+  cudaStream_t side = nullptr;           // an update's factorisation beside its separable tables, with the events
+  cudaEvent_t fork_ev = nullptr, join_ev = nullptr;   // that fork it from and join it to the caller's stream
   long long sep_bytes = 0, sep_masks = 0;   // size; its first bytes: the masks, cleared before a rebuild
   double *d_ws = nullptr;
   long long ws_doubles = 0;
