@@ -173,14 +173,16 @@ __global__ void __launch_bounds__(256) k_residual(Batch bt, const SubDesc *subs,
 // columns next to it and the ends of the dense rows. One thread per (unit, column); a unit is, for sides 1
 // and 2, a node pair (m, Nx - m) of both dense rows (x-centred; else a node of them), and for sides 3 and 4 a
 // middle row, or one of the 8 nodes at its end of the dense rows. k_residual evaluates all 9 neighbours
-// of every ring node for every column: 49 us for 4 x 257^2, 1024 columns, bound by instruction issue.
+// of every ring node for every column: 49 us for 4 x 257^2, 1024 columns, bound by instruction issue; 86 us
+// with the gradient's s, 13 and 22 us here. GRAD: s too, real, in the plain layout [ri][b].
 __device__ __forceinline__ double side_density(const SubDesc &d, const Item &it, const double *ws, const double *tab, int b,
-                                               int side, int g) {
+                                               int side, int g, int deriv = 0) {   // deriv: 0, or G for the k-derivative
   if (MDP_CHECKED && (g < 0 || g >= d.G || b < 0 || b >= it.ncols)) { flag_bounds(d.dstatus); return 0.0; }
   // owners are 1.0 .. 4.0: their high words tell them apart without the FP64 pipe
   const bool own = __double2hiint(tab[d.geo_off + 4 * g]) == __double2hiint((double)side);
-  return own ? ws[it.xi_off + (long long)g * it.ncols + b] : 0.0;
+  return own ? ws[it.xi_off + ((long long)g + deriv) * it.ncols + b] : 0.0;
 }
+template <bool GRAD>
 __global__ void __launch_bounds__(256) k_ring(Batch bt, const SubDesc *subs, const double *tab, double *ws) {
   Item it; int local;
   locate(bt, blockIdx.x, it, local);
@@ -200,11 +202,16 @@ __global__ void __launch_bounds__(256) k_ring(Batch bt, const SubDesc *subs, con
   double *r = ws + it.r_off + b;
   const double C0 = d.c0, C1 = d.c1, C2 = d.c2;
   auto den = [&](int g) { return side_density(d, it, ws, tab, b, side, g); };
+  const double D0 = d.dc0, D1 = d.dc1;
+  double *sb = ws + it.s_off + b;
+  auto dden = [&](int g) { return GRAD ? side_density(d, it, ws, tab, b, side, g, d.G) : 0.0; };
   if (side <= 2) {
     const int np = d.xsym ? d.Ph : d.Px;
     if (u >= np) return;
     const int W = d.Px + 2, base = side == 1 ? 0 : 2 * W + 4 * (d.Py - 2);
     const int go = side == 1 ? base : base + W, gi = side == 1 ? base + W : base;   // outer, inner gamma row
+    const int ra = side == 1 ? 0 : 3, rb = side == 1 ? 1 : 2;   // dense row numbers
+    const long long off[4] = {0, d.Px, 2LL * d.Px + 4 * (d.Py - 4), 3LL * d.Px + 4 * (d.Py - 4)};
     // residuals at ring node m of the dense row at the side and of the next one
     auto pair = [&](int m, double &r0, double &r1) {
       const int k = m - (d.mlo - 1);   // gamma column of m
@@ -213,12 +220,16 @@ __global__ void __launch_bounds__(256) k_ring(Batch bt, const SubDesc *subs, con
       const double is = i0 + i2;
       r0 = fma(C0, i1, fma(C1, is + o1, C2 * (o0 + o2)));
       r1 = fma(C1, i1, C2 * is);
+      if (GRAD) {
+        const double j0 = dden(gi + k - 1), j1 = dden(gi + k), j2 = dden(gi + k + 1);
+        const double p0 = dden(go + k - 1), p1 = dden(go + k), p2 = dden(go + k + 1), js = j0 + j2;
+        sb[(off[ra] + m - d.mlo) * nc] = fma(D0, i1, fma(D1, is + o1, fma(C0, j1, fma(C1, js + p1, C2 * (p0 + p2)))));
+        sb[(off[rb] + m - d.mlo) * nc] = fma(D1, i1, fma(C1, j1, C2 * js));
+      }
     };
-    const int ra = side == 1 ? 0 : 3, rb = side == 1 ? 1 : 2;   // dense row numbers
     double a0, a1;
     pair(d.mlo + u, a0, a1);
     if (!d.xsym) {
-      const long long off[4] = {0, d.Px, 2LL * d.Px + 4 * (d.Py - 4), 3LL * d.Px + 4 * (d.Py - 4)};
       r[(off[ra] + u) * nc] = a0;
       r[(off[rb] + u) * nc] = a1;
       return;
@@ -235,6 +246,13 @@ __global__ void __launch_bounds__(256) k_ring(Batch bt, const SubDesc *subs, con
     const double o0 = den(g + o), o1 = den(g + 4 + o), o2 = den(g + 8 + o);
     const double i0 = den(g + i), i1 = den(g + 4 + i), i2 = den(g + 8 + i), is = i0 + i2;
     const double r0 = fma(C0, i1, fma(C1, is + o1, C2 * (o0 + o2))), r1 = fma(C1, i1, C2 * is);
+    if (GRAD) {
+      const double j0 = dden(g + i), j1 = dden(g + 4 + i), j2 = dden(g + 8 + i), js = j0 + j2;
+      const double p0 = dden(g + o), p1 = dden(g + 4 + o), p2 = dden(g + 8 + o);
+      double *q = sb + (2LL * d.Px + 4 * u) * nc;
+      q[(side == 3 ? 0 : 3) * nc] = fma(D0, i1, fma(D1, is + o1, fma(C0, j1, fma(C1, js + p1, C2 * (p0 + p2)))));
+      q[(side == 3 ? 1 : 2) * nc] = fma(D1, i1, fma(C1, j1, C2 * js));
+    }
     if (d.xsym) {
       double *p = r + (8LL * d.Ph + 4 * u) * nc;
       p[0] = r0; p[nc] = side == 3 ? r0 : -r0;
@@ -251,15 +269,20 @@ __global__ void __launch_bounds__(256) k_ring(Batch bt, const SubDesc *subs, con
   const int rr = t >> 1, k = t & 1;   // dense row, node counted from the side
   const int n = rr == 0 ? d.nlo : rr == 1 ? d.nlo + 1 : rr == 2 ? d.nhi - 1 : d.nhi;
   const int m = side == 3 ? d.mlo + k : d.mhi - k;
-  double v = 0.0;
+  double v = 0.0, sv = 0.0;
 #pragma unroll
   for (int dn = -1; dn <= 1; ++dn)
 #pragma unroll
     for (int dm = -1; dm <= 1; ++dm) {
       const int g = gamma_index(d, n + dn, m + dm);
       const int nbr = (dn != 0) + (dm != 0);
-      if (g >= 0) v = fma(nbr == 0 ? C0 : nbr == 1 ? C1 : C2, den(g), v);
+      const double c = nbr == 0 ? C0 : nbr == 1 ? C1 : C2;
+      if (g < 0) continue;
+      const double x = den(g);
+      v = fma(c, x, v);
+      if (GRAD) sv = fma(c, dden(g), fma(nbr == 0 ? D0 : nbr == 1 ? D1 : 0.0, x, sv));
     }
+  if (GRAD) sb[((long long)rr * d.Px + (rr < 2 ? 0 : 4 * (d.Py - 4)) + m - d.mlo) * nc] = sv;
   if (d.xsym) {
     double *p = r + ((long long)rr * 2 * d.Ph + 2 * k) * nc;
     p[0] = v; p[nc] = side == 3 ? v : -v;
@@ -1634,7 +1657,7 @@ cudaError_t launch_project(mdp_plan *p, const Batch *fb, int out_kind, const dou
 #define MDP_LAUNCH(fam, ...) MDP_LAUNCH_AS(fam, fam, __VA_ARGS__)
   if (basis) MDP_LAUNCH(F_EXT, k_extend<<<grid1(fb[F_EXT].total_blocks), 32, 0, st>>>(fb[F_EXT], ds, tab, ws, 0));
   if (basis) {
-    MDP_LAUNCH_AS(F_RING, F_RES, k_ring<<<grid1(fb[F_RING].total_blocks), b8, 0, st>>>(fb[F_RING], ds, tab, ws));
+    MDP_LAUNCH_AS(F_RING, F_RES, k_ring<false><<<grid1(fb[F_RING].total_blocks), b8, 0, st>>>(fb[F_RING], ds, tab, ws));
     MDP_LAUNCH_AS(F_PRES, F_RES, k_residual<false, false><<<grid1(fb[F_PRES].total_blocks), b8, 0, st>>>(fb[F_PRES], ds, tab, ws, xi_user));
   } else MDP_LAUNCH(F_RES, k_residual<true, false><<<grid1(fb[F_RES].total_blocks), b8, 0, st>>>(fb[F_RES], ds, tab, ws, xi_user));
   if (basis) MDP_LAUNCH(F_FROWS, k_fwd_rows<false><<<grid1(fb[F_FROWS].total_blocks), b8, p->fft_smem, st>>>(fb[F_FROWS], ds, tab, ws));
@@ -1671,8 +1694,10 @@ cudaError_t launch_adjoint(mdp_plan *p, const Batch *fb, int out_kind, const dou
   if (e != cudaSuccess) return e;
   if (grad_k) {  // the residual and the k-derivative sources; by sweeps: forward recompute with every mode-space row kept
     if (basis) MDP_LAUNCH(F_EXT, k_extend<<<grid1(fb[F_EXT].total_blocks), 32, 0, st>>>(fb[F_EXT], ds, tab, ws, 1));
-    if (basis) MDP_LAUNCH(F_RES, k_residual<false, true><<<grid1(fb[F_RES].total_blocks), b8, 0, st>>>(fb[F_RES], ds, tab, ws, xi_user));
-    else MDP_LAUNCH(F_RES, k_residual<true, true><<<grid1(fb[F_RES].total_blocks), b8, 0, st>>>(fb[F_RES], ds, tab, ws, xi_user));
+    if (basis) {
+      MDP_LAUNCH_AS(F_RING, F_RES, k_ring<true><<<grid1(fb[F_RING].total_blocks), b8, 0, st>>>(fb[F_RING], ds, tab, ws));
+      MDP_LAUNCH_AS(F_PRES, F_RES, k_residual<false, true><<<grid1(fb[F_PRES].total_blocks), b8, 0, st>>>(fb[F_PRES], ds, tab, ws, xi_user));
+    } else MDP_LAUNCH(F_RES, k_residual<true, true><<<grid1(fb[F_RES].total_blocks), b8, 0, st>>>(fb[F_RES], ds, tab, ws, xi_user));
     if (basis) MDP_LAUNCH(F_FROWS, k_fwd_rows<false><<<grid1(fb[F_FROWS].total_blocks), b8, p->fft_smem, st>>>(fb[F_FROWS], ds, tab, ws));
     else MDP_LAUNCH(F_FROWS, k_fwd_rows<true><<<grid1(fb[F_FROWS].total_blocks), b8, p->fft_smem, st>>>(fb[F_FROWS], ds, tab, ws));
     if (basis) MDP_LAUNCH(F_TRI, k_tri<false, true, 2><<<grid1(fb[F_TRI].total_blocks), btri, TRI_WARPS * 2 * full_stage_bytes<false>(), st>>>(fb[F_TRI], ds, tab, p->d_piv, ws, p->d_sep));

@@ -12,7 +12,7 @@
 // against d phi/dk (extra outputs of the stage 1 contractions) times the other side's coefficients; and
 // sum conj(c) (dK/dk r) on the middle rows, one more Toeplitz product of the residual. The recomputed field
 // of every mode and row and its adjoint, most of the pass by the recurrences, are gone: 4 x 257^2 with 1024
-// basis columns takes 720 us (4415 by the recurrences), 257^2 and 513^2 with user densities 686 us (4532).
+// basis columns takes 630 us (4415 by the recurrences), 257^2 and 513^2 with user densities 680 us (4532).
 // A first pass after a change of the wavenumbers makes the tables too, 400 us more.
 #include "sep_modes.cuh"
 
@@ -756,10 +756,14 @@ __global__ void __launch_bounds__(SG_THREADS, 1)
 }
 
 // ---------------------------------------------------------------- modes
+// FP64-bound: some 200 instructions per mode and 32 columns with both ends (100 in two 3 x 3 blocks where they do
+// not see each other, as for most modes; a body each, so that the table's loads are not behind branches: 93 us
+// for 4 x 257^2 with 1024 columns, 116 by the full matrix, 152 with the branches inside).
 // Per (mode, column): the transpose of the projection's modes' matrix on the cotangent's moments and gamma
 // rows (F): A_b for the middle ring rows, the field at the 4 dense ring rows. With DK the mode's part of
 // <c, Tr G' r>, returned.
-template <bool CIN, bool DK>
+// far: the two ends do not see each other, two 3 x 3 blocks of the matrix
+template <bool CIN, bool DK, bool far>
 __device__ __forceinline__ double adj_modes_body(const Item &it, const SubDesc &d, const SepGeo &g, const SepWs &sw, const AdjWs &w,
                                                  const unsigned char *sep, const unsigned char *adj, double *ws, bool rec, int b,
                                                  int row1, int q) {
@@ -794,15 +798,21 @@ __device__ __forceinline__ double adj_modes_body(const Item &it, const SubDesc &
     iA = cmk(-u.im, u.re);
     iB = cmk(-v.im, v.re);
   }
+  auto column = [&](int k, cplx v) {   // F^T times column k of the matrix, added to v
+    if (far) {
+      const int e_ = k < 4 ? k >> 1 : k - 4;
+      v = caxpy(T[MT_MAT + 6 * e_ + k], F[e_], v);
+      v = caxpy(T[MT_MAT + 6 * (2 + 2 * e_) + k], F[2 + 2 * e_], v);
+      return caxpy(T[MT_MAT + 6 * (3 + 2 * e_) + k], F[3 + 2 * e_], v);
+    }
+#pragma unroll
+    for (int o = 0; o < 6; ++o) v = caxpy(T[MT_MAT + 6 * o + k], F[o], v);
+    return v;
+  };
   // coefficients on the middle rows (columns 4, 5 of the matrix)
   cplx A[2];
 #pragma unroll
-  for (int k = 0; k < 2; ++k) {
-    cplx v = k == 0 ? iA : iB;
-#pragma unroll
-    for (int o = 0; o < 6; ++o) v = caxpy(T[MT_MAT + 6 * o + 4 + k], F[o], v);
-    A[k] = v;
-  }
+  for (int k = 0; k < 2; ++k) A[k] = column(4 + k, k == 0 ? iA : iB);
   double *ae = ws + it.a_off + w.aeff + ((long long)e * 3 * g.nqp + qi) * R + b;
 #pragma unroll
   for (int k = 0; k < 2; ++k) { ae[(long long)k * g.nqp * R] = A[k].re; ae[(long long)k * g.nqp * R + cp] = A[k].im; }
@@ -815,8 +825,7 @@ __device__ __forceinline__ double adj_modes_body(const Item &it, const SubDesc &
 #pragma unroll
   for (int r = 0; r < 4; ++r) {
     cplx v = imag ? caxpy(T[MT_P1D + r], iA, cmk(T[MT_P2D + r] * iB.re, T[MT_P2D + r] * iB.im)) : cmk(0.0, 0.0);
-#pragma unroll
-    for (int o = 0; o < 6; ++o) v = caxpy(T[MT_MAT + 6 * o + r], F[o], v);
+    v = column(r, v);
     st2(y + 2 * (((long long)(q - 1) * 5 + r) * nc + b), v);
   }
   if (!DK) return 0.0;
@@ -841,20 +850,25 @@ __device__ __forceinline__ double adj_modes_body(const Item &it, const SubDesc &
 #pragma unroll
   for (int k = 0; k < 2; ++k) { in[4 + k] = at(rm, k, 1.0); dm[k] = at(rd, k, inv2(D[MD_RHO1 + k])); }
   auto redot = [&](cplx x, cplx z) { return CIN ? fma(x.re, z.re, -x.im * z.im) : x.re * z.re; };   // Re x z
+  auto row = [&](const double *M, int o) {   // row o of a matrix times the residual's inputs
+    cplx v = zero;
+    if (far) {
+      const int e_ = o < 2 ? o : (o - 2) >> 1;
+      v = axpy(M[6 * o + 2 * e_], in[2 * e_], v);
+      v = axpy(M[6 * o + 2 * e_ + 1], in[2 * e_ + 1], v);
+      return axpy(M[6 * o + 4 + e_], in[4 + e_], v);
+    }
+#pragma unroll
+    for (int k = 0; k < 6; ++k) v = axpy(M[6 * o + k], in[k], v);
+    return v;
+  };
   double s = 0.0;
 #pragma unroll
-  for (int o = 0; o < 6; ++o) {
-    cplx v = zero;
-#pragma unroll
-    for (int k = 0; k < 6; ++k) v = axpy(D[MD_MAT + 6 * o + k], in[k], v);
-    s += redot(F[o], v);
-  }
+  for (int o = 0; o < 6; ++o) s += redot(F[o], row(D + MD_MAT, o));
 #pragma unroll
   for (int k = 0; k < 2; ++k) s += redot(A[k], dm[k]);
   // forward coefficients against the cotangent's derivative moments, with i Im R and its derivative
-  cplx a0 = zero, a1 = zero;
-#pragma unroll
-  for (int k = 0; k < 6; ++k) { a0 = axpy(T[MT_MAT + k], in[k], a0); a1 = axpy(T[MT_MAT + 6 + k], in[k], a1); }
+  cplx a0 = row(T + MT_MAT, 0), a1 = row(T + MT_MAT, 1);
   if (imag) {
     cplx r1 = in[4], r2 = in[5], e1 = zero, e2 = zero, h1 = zero, h2 = zero;   // moments of all rows; d phi/dk parts of the full rows
 #pragma unroll
@@ -902,7 +916,9 @@ __global__ void __launch_bounds__(128) k_adj_modes(Batch bt, const SubDesc *subs
     const AdjWs w = adj_ws(d, it.ncols);
     const int row1 = CIN ? b : sep_row_of(d, it.col0, it.ncols, b) - sep_first34(d, it.col0, it.ncols);
     for (int q = q0; q < q0 + SEP_MODES_PER_BLOCK - (int)threadIdx.y && q <= d.Nq; q += 4)
-      s += adj_modes_body<CIN, DK>(it, d, g, sw, w, sep, adj, ws, has_rec && d.nrec >= 0, b, row1, q);
+      s += reinterpret_cast<const double *>(sep + d.sep_mt)[(long long)(q - 1) * SEP_MTW + MT_FAR] != 0.0
+               ? adj_modes_body<CIN, DK, true>(it, d, g, sw, w, sep, adj, ws, has_rec && d.nrec >= 0, b, row1, q)
+               : adj_modes_body<CIN, DK, false>(it, d, g, sw, w, sep, adj, ws, has_rec && d.nrec >= 0, b, row1, q);
   }
   if (DK) {
     s = block_sum<128>(s, sh);
@@ -928,13 +944,16 @@ __global__ void __launch_bounds__(256) k_adj_out(Batch bt, const SubDesc *subs, 
   const int part = local < n0 ? 0 : local < n0 + n1 ? 1 : 2, l = part == 0 ? local : part == 1 ? local - n0 : local - n0 - n1;
   const int b = (l % cb) * 32 + threadIdx.x, u = (l / cb) * 8 + threadIdx.y;
   double dk = 0.0;
-  auto put = [&](int ri, cplx v) {   // v = conj(mu)
+  auto put = [&](int ri, cplx v, bool support) {   // v = conj(mu); s of basis columns (k_ring): real, on its support
     st2(ws + it.r_off + 2 * ((long long)ri * nc + b), cmk(v.re, -v.im));
-    if (DK) {
+    if (DK && CIN) {
       const cplx s = ld2(ws + it.s_off + 2 * ((long long)ri * nc + b));
       dk -= fma(v.re, s.re, -v.im * s.im);   // Re conj(mu) s
+    } else if (DK && support) {
+      dk = fma(-v.re, ws[it.s_off + (long long)ri * nc + b], dk);
     }
   };
+  const int side = CIN || b >= it.ncols ? 0 : col_side(d, it.col0 + b);
   if (b < it.ncols && part == 0 && u < g.Pj) {
     cplx v[4];
 #pragma unroll
@@ -944,15 +963,19 @@ __global__ void __launch_bounds__(256) k_adj_out(Batch bt, const SubDesc *subs, 
       v[k] = cmk(p1[0] + p3[0], p1[cp] + p3[cp]);
     }
     const int r0 = 2 * d.Px + 4 * u;
-    if (d.xsym) { put(r0, cadd(v[0], v[2])); put(r0 + 1, cadd(v[1], v[3])); put(r0 + 2, csub(v[1], v[3])); put(r0 + 3, csub(v[0], v[2])); }
-    else { put(r0, v[0]); put(r0 + 1, v[1]); put(r0 + 2, v[2]); put(r0 + 3, v[3]); }
+    const bool l = side == 3, r = side == 4;
+    if (d.xsym) { put(r0, cadd(v[0], v[2]), l); put(r0 + 1, cadd(v[1], v[3]), l); put(r0 + 2, csub(v[1], v[3]), r); put(r0 + 3, csub(v[0], v[2]), r); }
+    else { put(r0, v[0], l); put(r0 + 1, v[1], l); put(r0 + 2, v[2], r); put(r0 + 3, v[3], r); }
   } else if (b < it.ncols && part == 1 && u < 4 * g.Kf) {
     const int rr = u / g.Kf, k = u % g.Kf, m = g.mf + k, m2 = d.Nx - m, Ri = adj_rows(d, A_INV, it.ncols);
     const double *p0 = ws + it.a_off + w.ui + (long long)k * Ri + rr * R + b, *p1 = p0 + (long long)g.Kf * Ri;
     const cplx x = cmk(p0[0], p0[cp]), y = cmk(p1[0], p1[cp]);
     const int base = rr * d.Px + (rr < 2 ? 0 : 4 * (d.Py - 4)) - d.mlo;
-    if (m >= d.mlo && m <= d.mhi) put(base + m, cadd(x, y));
-    if (m2 != m && m2 >= d.mlo && m2 <= d.mhi) put(base + m2, csub(x, y));
+    auto support = [&](int mm) {
+      return side == 1 ? rr < 2 : side == 2 ? rr >= 2 : side == 3 ? mm <= d.mlo + 1 : mm >= d.mhi - 1;
+    };
+    if (m >= d.mlo && m <= d.mhi) put(base + m, cadd(x, y), support(m));
+    if (m2 != m && m2 >= d.mlo && m2 <= d.mhi) put(base + m2, csub(x, y), support(m2));
   } else if (DK && b < it.ncols && part == 2 && u < g.Pi) {
     const int row1 = CIN ? b : sep_row_of(d, it.col0, it.ncols, b) - sep_first34(d, it.col0, it.ncols);
     if (row1 >= 0) {

@@ -555,6 +555,10 @@ static void schedule(mdp_plan *p) {
   long long mx = 0;
   for (auto &sc : p->sched)
     for (auto &w : sc) mx = std::max(mx, w.ws_doubles);
+  // room for the right-hand sides of full-grid solves: a complex field and its operands of every column's grid
+  long long grids = 0;
+  for (auto &hs : p->subs) grids += 4LL * hs.d.Nq * hs.d.Nt * hs.d.n_cols;
+  mx = std::max(mx, std::min(grids, p->ws_budget / 8));
   // one column of source terms: its item and the scratch of launch_source_terms
   for (auto &hs : p->subs) {
     const SubDesc &d = hs.d;
