@@ -85,7 +85,7 @@ mdp_status alloc_device(mdp_plan *p) {
   CK(set_kernel_attributes());
   auto al = [&](void **ptr, size_t bytes) -> bool { return cudaMalloc(ptr, std::max<size_t>(bytes, 256)) == cudaSuccess; };
   if (!al((void **)&p->d_subs, p->subs.size() * sizeof(SubDesc)) ||
-      !al((void **)&p->d_tables, p->host_tables.size() * sizeof(double)) ||
+      !al((void **)&p->d_tables, p->n_tables * sizeof(double)) ||
       !al((void **)&p->d_piv, p->host_piv.size()) || !al((void **)&p->d_sep, (size_t)p->sep_bytes) || !al((void **)&p->d_ws, (size_t)p->ws_doubles * 8) ||
       !al((void **)&p->d_status, sizeof(int)) || !al((void **)&p->d_fstatus, sizeof(int)) ||
       !p->sub_stage.alloc(p->subs.size(), true) || !p->h_fstatus.alloc(1, true))
@@ -100,11 +100,12 @@ mdp_status alloc_device(mdp_plan *p) {
   // projection item's mode-space slice past the end of the workspace (the checks must catch it and
   // skip every access through it)
   const char *fault = std::getenv("MDP_FAULT_INJECT");
-  if (fault && !std::strcmp(fault, "factor") && !p->subs.empty() && p->subs[0].d.NYf > 6)
+  if (fault && !std::strcmp(fault, "factor") && !p->subs.empty() && p->subs[0].d.NYf > 6 && p->subs[0].fs)
     for (int j = 0; j < FSW; ++j) p->host_tables[p->subs[0].d.fs_off + 5 * FSW + j] *= 1.5;
 #endif
   mdp_status st = upload_subs_tables(p);
   if (st != MDP_OK) return st;
+  p->host_stale = p->fs_stale = p->n_light < p->n_tables;
   for (int si = 0; si < p->n_subs; ++si) {
     const SubDesc &d = p->subs[si].d;
     if (d.leader != si) continue;
@@ -402,7 +403,7 @@ mdp_status mdp_plan_update_k_async(mdp_plan *p, const double *k, void *cuda_stre
   CK(cudaSetDevice(p->device));
   cudaStream_t s = (cudaStream_t)cuda_stream;
   if (!p->alt_tables) {   // first call: the second set starts as a copy of the first (k-independent tables)
-    const size_t nt = std::max<size_t>(p->host_tables.size() * sizeof(double), 256);
+    const size_t nt = std::max<size_t>(p->n_tables * sizeof(double), 256);
     const size_t np = std::max<size_t>(p->host_piv.size(), 256);
     const size_t ns = std::max<size_t>(p->subs.size() * sizeof(SubDesc), 256);
     if (cudaMalloc((void **)&p->alt_tables, nt) != cudaSuccess || cudaMalloc((void **)&p->alt_piv, np) != cudaSuccess ||
@@ -441,6 +442,7 @@ mdp_status mdp_plan_update_k_async(mdp_plan *p, const double *k, void *cuda_stre
 static mdp_status ensure_host_tables(const mdp_plan *cp) {
   mdp_plan *p = const_cast<mdp_plan *>(cp);
   if (!p->host_stale) return MDP_OK;
+  if ((long long)p->host_tables.size() < p->n_tables && !bind_tables(p, p->n_tables, false)) return MDP_ERR_NOMEM;
   std::vector<double> k;
   for (auto &hs : p->subs) k.push_back(hs.d.k);
   const mdp_status st = refactor_host(p, k.data());
@@ -452,7 +454,7 @@ long long mdp_plan_update_bytes(const mdp_plan *p) { return p ? (long long)(p->s
 
 mdp_status mdp_plan_table_sizes(const mdp_plan *p, long long *n_doubles, long long *n_piv) {
   if (!p) return MDP_ERR_ARG;
-  if (n_doubles) *n_doubles = (long long)p->host_tables.size();
+  if (n_doubles) *n_doubles = p->n_tables;
   if (n_piv) *n_piv = (long long)p->host_piv.size();
   return MDP_OK;
 }
@@ -477,13 +479,13 @@ mdp_status mdp_plan_read_tables(const mdp_plan *p, int device_side, double *tabl
       CK(cudaStreamSynchronize(nullptr));
       mp->fs_stale = false;
     }
-    CK(cudaMemcpy(tables, p->d_tables, p->host_tables.size() * sizeof(double), cudaMemcpyDeviceToHost));
+    CK(cudaMemcpy(tables, p->d_tables, p->n_tables * sizeof(double), cudaMemcpyDeviceToHost));
     CK(cudaMemcpy(piv, p->d_piv, p->host_piv.size(), cudaMemcpyDeviceToHost));
     return MDP_OK;
   }
   const mdp_status st = ensure_host_tables(p);
   if (st != MDP_OK) return st;
-  std::memcpy(tables, p->host_tables.data(), p->host_tables.size() * sizeof(double));
+  std::memcpy(tables, p->host_tables.data(), p->n_tables * sizeof(double));
   std::memcpy(piv, p->host_piv.data(), p->host_piv.size());
   return MDP_OK;
 }
@@ -814,7 +816,7 @@ mdp_status mdp_plan_receiver_layout(const mdp_plan *p, int sub, int *row, int *m
 long long mdp_plan_receiver_size(const mdp_plan *p) { return p ? p->rec_size : 0; }
 
 long long mdp_plan_table_bytes(const mdp_plan *p) {
-  return p ? (long long)(p->host_tables.size() * sizeof(double) + p->host_piv.size()) : 0;
+  return p ? (long long)(p->n_tables * sizeof(double) + p->host_piv.size()) : 0;
 }
 
 int mdp_kernel_family_count(void) { return NFAM; }

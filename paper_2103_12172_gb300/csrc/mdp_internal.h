@@ -463,7 +463,8 @@ struct mdp_plan {
   int n_subs = 0;
   int device = -1;
   std::vector<mdp::HostSub> subs;
-  mdp::HostBuf<double> host_tables;      // all factor / dT / sweep / sine / geometry tables
+  mdp::HostBuf<double> host_tables;      // factor / dT / sweep / sine / geometry tables: the first n_light doubles
+  long long n_tables = 0, n_light = 0;   // of n_tables, or all of them (bind_tables)
   mdp::HostBuf<uint8_t> host_piv;
   long long out_size = 0;
   long long rec_size = 0;
@@ -537,7 +538,7 @@ inline void set_bounds(const mdp_plan *p, Batch &b, long long out_n, bool grad) 
   b.n_subs = p->n_subs;
   b.grad = grad ? 1 : 0;
   b.ws_n = p->ws_doubles;
-  b.tab_n = (long long)p->host_tables.size();
+  b.tab_n = p->n_tables;
   b.piv_n = (long long)p->host_piv.size();
   b.out_n = out_n;
   b.status = p->d_status;
@@ -663,6 +664,7 @@ const char *fam_name(int f);
 void prof_begin(mdp_plan *p, int fam, cudaStream_t st);
 void prof_end(mdp_plan *p, int fam, cudaStream_t st);
 // plan construction (host)
+bool bind_tables(mdp_plan *p, long long n, bool pinned);
 mdp_status build_host_plan(mdp_plan *p, const mdp_subdomain *subs, int n);
 mdp_status refactor_host(mdp_plan *p, const double *k);
 void mode_entries(const SubDesc &d, int q, double &off, double &diag);   // interior entries of T_q

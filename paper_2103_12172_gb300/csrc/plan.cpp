@@ -243,6 +243,7 @@ static mdp_status build_fs_mode(HostSub &hs, int q) {
     if (!band_lu(n, dl.data(), dg.data(), du.data(), du2.data(), pv.data())) return MDP_ERR_SINGULAR;
     for (int i = 0; i < n; ++i)
       if (std::abs(dg[i]) < kSingularTol * scale) return MDP_ERR_SINGULAR;
+    if (!hs.fs) return MDP_OK;   // checked for resonance only
     const int N2 = 2 * d.Nx;
     const int ms[4] = {d.mlo, d.mlo + 1, d.mhi - 1, d.mhi};
     double sines[4];
@@ -403,6 +404,18 @@ void host_mode_solve(const HostSub &hs, int q, int adjoint, const double *b, dou
 }
 
 // ---------------------------------------------------------------- tables
+// Host tables of n doubles (n_light: without the sweep tables at the end).
+bool bind_tables(mdp_plan *p, long long n, bool pinned) {
+  if (!p->host_tables.alloc((size_t)n, pinned)) return false;
+  for (auto &hs : p->subs) {
+    const SubDesc &d = hs.d;
+    hs.fact = p->host_tables.data() + d.fact_off;
+    hs.dT = p->host_tables.data() + d.dT_off;
+    hs.fs = d.fs_off < n ? p->host_tables.data() + d.fs_off : nullptr;
+    hs.piv = p->host_piv.data() + d.piv_off;
+  }
+  return true;
+}
 static bool layout_tables(mdp_plan *p) {
   long long off = 0, poff = 0, out = 0, sep = 0;
   auto al = [](long long v) { return (v + 31) & ~31LL; };
@@ -475,19 +488,26 @@ static bool layout_tables(mdp_plan *p) {
     d.sin_off = off;  off += al(4LL * d.Nx);
     d.geo_off = off;  off += al(4LL * d.G);
     d.seg_off = off;  off += al(5LL * d.Nq);
-    d.fs_off = off;   off += al((long long)d.Nq * d.NYf * FSW);
+    if (!d.tc_cols) { d.fs_off = off; off += al((long long)d.Nq * d.NYf * FSW); }
     d.piv_off = poff; poff += al((long long)d.Nq * d.Nt);
     d.out_off = out;  out += (long long)d.G * d.n_cols;
   }
-  const bool pinned = !(p->flags & MDP_PLAN_HOST_ONLY);
-  if (!p->host_tables.alloc((size_t)off, pinned) || !p->host_piv.alloc((size_t)poff, pinned)) return false;
+  // last, the projection's sweep tables of subdomains that take the separable solve: a device plan makes them
+  // for introspection alone (they were two thirds of the page-locked memory and of the upload)
+  p->n_light = off;
   for (auto &hs : p->subs) {
-    const SubDesc &d = hs.d;
-    hs.fact = p->host_tables.data() + d.fact_off;
-    hs.dT = p->host_tables.data() + d.dT_off;
-    hs.fs = p->host_tables.data() + d.fs_off;
-    hs.piv = p->host_piv.data() + d.piv_off;
+    SubDesc &d = hs.d;
+    if (!d.tc_cols) continue;
+    if (d.leader != (int)(&hs - p->subs.data())) {
+      d.fs_off = p->subs[d.leader].d.fs_off;
+      continue;
+    }
+    d.fs_off = off;   off += al((long long)d.Nq * d.NYf * FSW);
   }
+  p->n_tables = off;
+  const bool device = !(p->flags & MDP_PLAN_HOST_ONLY);
+  if (!device) p->n_light = off;
+  if (!p->host_piv.alloc((size_t)poff, device) || !bind_tables(p, p->n_light, device)) return false;
   p->out_size = out;
   p->sep_bytes = sep;
   p->adj_bytes = adj;
