@@ -246,7 +246,8 @@ cudaError_t launch_update(mdp_plan *p, const SubDesc *ds, double *tab, uint8_t *
 
 // The gradient tables follow the wavenumbers only where a gradient is asked for: allocated by the first such
 // call, rebuilt by the first after a change. In a capture they are always rebuilt, so that a replay
-// follows the tables that it finds (and the allocation is no stream operation).
+// follows the tables that it finds (and the allocation is no stream operation); from then on every call rebuilds
+// them, as a replay may have left those of another table set.
 cudaError_t ensure_adj_tables(mdp_plan *p, cudaStream_t st) {
   if (p->adj_bytes == 0) return cudaSuccess;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
@@ -263,12 +264,13 @@ cudaError_t ensure_adj_tables(mdp_plan *p, cudaStream_t st) {
     p->adj_stale = true;
   }
   const bool live = cap == cudaStreamCaptureStatusNone;
+  if (!live) p->adj_captured = true;
   if (!p->adj_sines || !live) {
     e = launch_adj_sines(p, st);
     if (e != cudaSuccess) return e;
     if (live) p->adj_sines = true;
   }
-  if (p->adj_stale || !live) {
+  if (p->adj_stale || p->adj_captured) {
     e = launch_adj_tables(p, st);
     if (e != cudaSuccess) return e;
     if (live) p->adj_stale = false;

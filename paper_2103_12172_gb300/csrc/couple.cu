@@ -63,6 +63,7 @@ __device__ __forceinline__ double2 zero2() { return make_double2(0.0, 0.0); }
 
 // cv = S x + eps (either may be null: left out)
 __global__ void __launch_bounds__(128) k_cp_vec(Cp p, const double2 *x, const double2 *rho, const double2 *eps, double2 *cv) {
+  pdl_wait();
   const int i = blockIdx.x * 128 + threadIdx.x;
   if (i >= p.N * p.C) return;
   double2 v = zero2();
@@ -81,6 +82,7 @@ template <int T>
 __global__ void __launch_bounds__(512) k_cp_gemv(const double2 *B, const long long *off, const int *len, const int *yoff, int C,
                                                  const double2 *v, long long vs, double2 *y, long long ys, double sg0,
                                                  double sg1, const double2 *add) {
+  pdl_wait();
   __shared__ double2 sh[T][16][32];
   const int j = blockIdx.y, L = len[j], g = blockIdx.x * 32 + threadIdx.x;
   if (blockIdx.x * 32 >= L) return;
@@ -130,6 +132,7 @@ __device__ __forceinline__ void block_total(double2 (&a)[T]) {
 template <int T>
 __global__ void __launch_bounds__(128) k_cp_dots(const double2 *B, const long long *off, const int *len, const int *yoff, int C,
                                                  const double2 *u, long long us, double2 *z, long long zs) {
+  pdl_wait();
   const int c = blockIdx.x, j = blockIdx.y, L = len[j];
   const double2 *b = B + off[j] + (long long)c * L, *uj = u + yoff[j];
   double2 acc[T];
@@ -151,6 +154,7 @@ __global__ void __launch_bounds__(128) k_cp_dots(const double2 *B, const long lo
 template <int T>
 __global__ void __launch_bounds__(128) k_cp_outer(const long long *off, const int *len, const int *yoff, int C, const double2 *u,
                                                   long long us, const double2 *a, const double2 *b, double2 *gB) {
+  pdl_wait();
   const int c = blockIdx.y, j = blockIdx.z, L = len[j], g = blockIdx.x * 128 + threadIdx.x;
   if (g >= L) return;
   const double2 ac = a[(long long)j * C + c], u0 = u[yoff[j] + g];
@@ -172,6 +176,7 @@ __device__ __forceinline__ double2 a_entry(const Cp &p, const double2 *Q, const 
 
 // D = 1 / the norms of A's columns: one block per unknown
 __global__ void __launch_bounds__(128) k_cp_norm(Cp p, const double2 *Q, const double2 *rho, double *D) {
+  pdl_wait();
   const int u = blockIdx.x;
   double2 acc[1] = {zero2()};
   for (int t = 0; t < 2; ++t) {
@@ -190,6 +195,7 @@ __global__ void __launch_bounds__(128) k_cp_norm(Cp p, const double2 *Q, const d
 // the subdomains' matrices [A_j D | b_j], column-major, padded with zeros to nmax + 1 columns of mmax rows
 __global__ void __launch_bounds__(128) k_cp_build(Cp p, const double2 *Q, const double2 *rho, const double *D, const double2 *b,
                                                   double2 *Mx) {
+  pdl_wait();
   const int g = blockIdx.x * 128 + threadIdx.x, c = blockIdx.y, j = blockIdx.z, L = p.G[j];
   if (g >= p.mmax) return;
   double2 v = zero2();
@@ -207,6 +213,7 @@ __global__ void __launch_bounds__(128) k_cp_build(Cp p, const double2 *Q, const 
 
 // [S | q_s]: the stacked R_ss of the subdomains in the shared columns
 __global__ void __launch_bounds__(128) k_cp_gather(Cp p, const double2 *Mx, double2 *S) {
+  pdl_wait();
   const int r = blockIdx.x * 128 + threadIdx.x, c = blockIdx.y;
   if (r >= p.ms) return;
   int j = 0;
@@ -229,6 +236,7 @@ __global__ void __launch_bounds__(128) k_cp_gather(Cp p, const double2 *Mx, doub
 template <bool GRAM>
 __global__ void __launch_bounds__(kTrThreads) k_cp_shared(Cp p, const double2 *S, const double *D, const double2 *gx,
                                                           const double2 *part, double2 *ys, double2 *x) {
+  pdl_wait();
   extern __shared__ __align__(16) double2 xs[];
   for (int c = threadIdx.x; c < p.ns; c += kTrThreads) {
     if (!GRAM) { xs[c] = S[(long long)p.ns * p.ms + c]; continue; }
@@ -254,6 +262,7 @@ __global__ void __launch_bounds__(kTrThreads) k_cp_shared(Cp p, const double2 *S
 // a subdomain's own unknowns: x_p = R_pp^{-1} (rhs - R_ps x_s), rhs from the QR's last column or (yp) given
 __global__ void __launch_bounds__(kTrThreads) k_cp_private(Cp p, const double2 *Mx, const double *D, const double2 *ys,
                                                            const double2 *yp, double2 *x) {
+  pdl_wait();
   extern __shared__ __align__(16) double2 xs[];   // [pj], then [8][pj] partial sums
   const int j = blockIdx.x, pj = p.pj[j], sj = p.nj[j] - pj, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const double2 *Mj = Mx + (long long)j * (p.nmax + 1) * p.mmax;
@@ -280,6 +289,7 @@ __global__ void __launch_bounds__(kTrThreads) k_cp_private(Cp p, const double2 *
 
 // yp = R_pp^{-H} gx_p and the subdomain's part R_ps^H yp of the shared right-hand side
 __global__ void __launch_bounds__(kTrThreads) k_cp_private_h(Cp p, const double2 *Mx, const double2 *gx, double2 *yp, double2 *part) {
+  pdl_wait();
   extern __shared__ __align__(16) double2 xs[];
   const int j = blockIdx.x, pj = p.pj[j], lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const double2 *Mj = Mx + (long long)j * (p.nmax + 1) * p.mmax;
@@ -300,6 +310,7 @@ __global__ void __launch_bounds__(kTrThreads) k_cp_private_h(Cp p, const double2
 
 // gx = D S^H g
 __global__ void __launch_bounds__(128) k_cp_gx(Cp p, const double2 *g, const double2 *rho, const double *D, double2 *gx) {
+  pdl_wait();
   const int u = blockIdx.x * 128 + threadIdx.x;
   if (u >= p.n) return;
   double2 v = zero2();
@@ -317,6 +328,7 @@ __global__ void __launch_bounds__(128) k_cp_gx(Cp p, const double2 *g, const dou
 // gradients by the boundary data of an outer side: grad eps = h, grad rho = h x^H + z w^H; one block per side
 __global__ void __launch_bounds__(128) k_cp_sides(Cp p, const double2 *g, const double2 *z, const double2 *x, const double2 *w,
                                                   double2 *grho, double2 *geps) {
+  pdl_wait();
   const int q = blockIdx.x;
   const long long o = (long long)p.qj[q] * p.C, zs = (long long)p.N * p.C;
   const int e = p.qe[q], r = p.qr[q], u = p.qu[q];
@@ -406,24 +418,24 @@ extern "C" mdp_status mdp_couple_solve(const mdp_couple *c, const mdp_c64 *Q_, c
   const size_t sms = (size_t)p.ns * 16, smp = (size_t)p.nmax * 9 * 16;
   if (!smem_ok(k_cp_shared<false>, sms) || !smem_ok(k_cp_private, smp)) return MDP_ERR_CUDA;
   const unsigned nv = (unsigned)((p.N * p.C + 127) / 128);
-  k_cp_vec<<<nv, 128, 0, st>>>(p, nullptr, rho, eps, buf + w.cv);
-  k_cp_gemv<1><<<dim3((p.mmax + 31) / 32, p.N), dim3(32, 16), 0, st>>>(Q, p.off, p.G, p.r0, p.C, buf + w.cv, 0, buf + w.b, 0, -1.0, 0.0, src);
-  k_cp_norm<<<p.n, 128, 0, st>>>(p, Q, rho, D);
-  k_cp_build<<<dim3((p.mmax + 127) / 128, p.nmax + 1, p.N), 128, 0, st>>>(p, Q, rho, D, buf + w.b, buf + w.M);
+  pdl(k_cp_vec, dim3(nv), dim3(128), 0, st, p, nullptr, rho, eps, buf + w.cv);
+  pdl(k_cp_gemv<1>, dim3((p.mmax + 31) / 32, p.N), dim3(32, 16), 0, st, Q, p.off, p.G, p.r0, p.C, buf + w.cv, 0, buf + w.b, 0, -1.0, 0.0, src);
+  pdl(k_cp_norm, dim3(p.n), dim3(128), 0, st, p, Q, rho, D);
+  pdl(k_cp_build, dim3((p.mmax + 127) / 128, p.nmax + 1, p.N), dim3(128), 0, st, p, Q, rho, D, buf + w.b, buf + w.M);
   if (cudaGetLastError() != cudaSuccess) return MDP_ERR_CUDA;
   mdp_status s = mdp_householder_qr_batched(p.N, p.mmax, p.nmax, 1, (mdp_c64 *)(buf + w.M), p.mmax, (long long)(p.nmax + 1) * p.mmax,
                                             (mdp_c64 *)(buf + w.tau), work, st);
   if (s != MDP_OK) return s;
   if (p.ns > 0) {
-    k_cp_gather<<<dim3((p.ms + 127) / 128, p.ns + 1), 128, 0, st>>>(p, buf + w.M, buf + w.S);
+    pdl(k_cp_gather, dim3((p.ms + 127) / 128, p.ns + 1), dim3(128), 0, st, p, buf + w.M, buf + w.S);
     if (cudaGetLastError() != cudaSuccess) return MDP_ERR_CUDA;
     s = mdp_householder_qr_batched(1, p.ms, p.ns, 1, (mdp_c64 *)(buf + w.S), p.ms, 0, (mdp_c64 *)(buf + w.tau + (long long)p.N * p.nmax),
                                    work + mdp_householder_qr_work_ints(p.N), st);
     if (s != MDP_OK) return s;
-    k_cp_shared<false><<<1, kTrThreads, sms, st>>>(p, buf + w.S, D, nullptr, nullptr, buf + w.ys, x);
+    pdl(k_cp_shared<false>, dim3(1), dim3(kTrThreads), sms, st, p, buf + w.S, D, nullptr, nullptr, buf + w.ys, x);
   }
-  k_cp_private<<<p.N, kTrThreads, smp, st>>>(p, buf + w.M, D, buf + w.ys, nullptr, x);
-  k_cp_vec<<<nv, 128, 0, st>>>(p, x, rho, eps, coef);
+  pdl(k_cp_private, dim3(p.N), dim3(kTrThreads), smp, st, p, buf + w.M, D, buf + w.ys, nullptr, x);
+  pdl(k_cp_vec, dim3(nv), dim3(128), 0, st, p, x, rho, eps, coef);
   return cudaGetLastError() == cudaSuccess ? MDP_OK : MDP_ERR_CUDA;
 }
 
@@ -443,18 +455,18 @@ extern "C" mdp_status mdp_couple_grad(const mdp_couple *c, const mdp_c64 *Q_, co
   const size_t sms = (size_t)p.ns * 16, smp = (size_t)p.nmax * 9 * 16;
   if (!smem_ok(k_cp_shared<true>, sms) || !smem_ok(k_cp_private, smp) || !smem_ok(k_cp_private_h, smp)) return MDP_ERR_CUDA;
   const long long nc = (long long)p.N * p.C;
-  k_cp_gx<<<(p.n + 127) / 128, 128, 0, st>>>(p, g, rho, D, tmp + t.gx);
-  k_cp_private_h<<<p.N, kTrThreads, smp, st>>>(p, buf + w.M, tmp + t.gx, tmp + t.yp, tmp + t.part);
-  if (p.ns > 0) k_cp_shared<true><<<1, kTrThreads, sms, st>>>(p, buf + w.S, D, tmp + t.gx, tmp + t.part, tmp + t.ys, tmp + t.w);
-  k_cp_private<<<p.N, kTrThreads, smp, st>>>(p, buf + w.M, D, tmp + t.ys, tmp + t.yp, tmp + t.w);
+  pdl(k_cp_gx, dim3((p.n + 127) / 128), dim3(128), 0, st, p, g, rho, D, tmp + t.gx);
+  pdl(k_cp_private_h, dim3(p.N), dim3(kTrThreads), smp, st, p, buf + w.M, tmp + t.gx, tmp + t.yp, tmp + t.part);
+  if (p.ns > 0) pdl(k_cp_shared<true>, dim3(1), dim3(kTrThreads), sms, st, p, buf + w.S, D, tmp + t.gx, tmp + t.part, tmp + t.ys, tmp + t.w);
+  pdl(k_cp_private, dim3(p.N), dim3(kTrThreads), smp, st, p, buf + w.M, D, tmp + t.ys, tmp + t.yp, tmp + t.w);
   if (cudaMemcpyAsync(tmp + t.sw, coef, sizeof(double2) * (size_t)nc, cudaMemcpyDeviceToDevice, st) != cudaSuccess) return MDP_ERR_CUDA;
-  k_cp_vec<<<(unsigned)((nc + 127) / 128), 128, 0, st>>>(p, tmp + t.w, rho, nullptr, tmp + t.sw + nc);
-  k_cp_gemv<2><<<dim3((p.mmax + 31) / 32, p.N), dim3(32, 16), 0, st>>>(Q, p.off, p.G, p.r0, p.C, tmp + t.sw, nc, tmp + t.u, p.rows, -1.0, 1.0, src);
+  pdl(k_cp_vec, dim3((unsigned)((nc + 127) / 128)), dim3(128), 0, st, p, tmp + t.w, rho, nullptr, tmp + t.sw + nc);
+  pdl(k_cp_gemv<2>, dim3((p.mmax + 31) / 32, p.N), dim3(32, 16), 0, st, Q, p.off, p.G, p.r0, p.C, tmp + t.sw, nc, tmp + t.u, p.rows, -1.0, 1.0, src);
   if (gQ)
-    k_cp_outer<2><<<dim3((p.mmax + 127) / 128, p.C, p.N), 128, 0, st>>>(p.off, p.G, p.r0, p.C, tmp + t.u, p.rows, tmp + t.sw + nc, coef, gQ);
+    pdl(k_cp_outer<2>, dim3((p.mmax + 127) / 128, p.C, p.N), dim3(128), 0, st, p.off, p.G, p.r0, p.C, tmp + t.u, p.rows, tmp + t.sw + nc, coef, gQ);
   if (p.no > 0) {
-    k_cp_dots<2><<<dim3(p.C, p.N), 128, 0, st>>>(Q, p.off, p.G, p.r0, p.C, tmp + t.u, p.rows, tmp + t.z, nc);
-    k_cp_sides<<<p.no, 128, 0, st>>>(p, g, tmp + t.z, x, tmp + t.w, (double2 *)grho_, (double2 *)geps_);
+    pdl(k_cp_dots<2>, dim3(p.C, p.N), dim3(128), 0, st, Q, p.off, p.G, p.r0, p.C, tmp + t.u, p.rows, tmp + t.z, nc);
+    pdl(k_cp_sides, dim3(p.no), dim3(128), 0, st, p, g, tmp + t.z, x, tmp + t.w, (double2 *)grho_, (double2 *)geps_);
   }
   return cudaGetLastError() == cudaSuccess ? MDP_OK : MDP_ERR_CUDA;
 }
@@ -462,7 +474,7 @@ extern "C" mdp_status mdp_couple_grad(const mdp_couple *c, const mdp_c64 *Q_, co
 extern "C" mdp_status mdp_block_values(int n_blocks, int cols, int max_len, const int *len, const int *yoff, const long long *off,
                                        const mdp_c64 *B, const mdp_c64 *v, mdp_c64 *y, void *cuda_stream) {
   if (n_blocks < 1 || n_blocks > 65535 || cols < 1 || max_len < 1 || !len || !yoff || !off || !B || !v || !y) return MDP_ERR_ARG;
-  k_cp_gemv<1><<<dim3((max_len + 31) / 32, n_blocks), dim3(32, 16), 0, (cudaStream_t)cuda_stream>>>(
+  pdl(k_cp_gemv<1>, dim3((max_len + 31) / 32, n_blocks), dim3(32, 16), 0, (cudaStream_t)cuda_stream, 
       (const double2 *)B, off, len, yoff, cols, (const double2 *)v, 0, (double2 *)y, 0, 1.0, 0.0, nullptr);
   return cudaGetLastError() == cudaSuccess ? MDP_OK : MDP_ERR_CUDA;
 }
@@ -475,8 +487,8 @@ extern "C" mdp_status mdp_block_values_grad(int n_blocks, int cols, int max_len,
   cudaStream_t st = (cudaStream_t)cuda_stream;
   const double2 *u = (const double2 *)gy;
   if (gB)
-    k_cp_outer<1><<<dim3((max_len + 127) / 128, cols, n_blocks), 128, 0, st>>>(off, len, yoff, cols, u, 0, (const double2 *)v, nullptr, (double2 *)gB);
+    pdl(k_cp_outer<1>, dim3((max_len + 127) / 128, cols, n_blocks), dim3(128), 0, st, off, len, yoff, cols, u, 0, (const double2 *)v, nullptr, (double2 *)gB);
   if (gv)
-    k_cp_dots<1><<<dim3(cols, n_blocks), 128, 0, st>>>((const double2 *)B, off, len, yoff, cols, u, 0, (double2 *)gv, 0);
+    pdl(k_cp_dots<1>, dim3(cols, n_blocks), dim3(128), 0, st, (const double2 *)B, off, len, yoff, cols, u, 0, (double2 *)gv, 0);
   return cudaGetLastError() == cudaSuccess ? MDP_OK : MDP_ERR_CUDA;
 }

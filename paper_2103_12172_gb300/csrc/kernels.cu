@@ -27,6 +27,7 @@ namespace mdp {
 // step is 14 FP64 instructions (22 with the terms formed one by one). Blocks of one warp: the few warps of a
 // call (a node each thread) share no SM's FP64 pipe.
 __global__ void __launch_bounds__(32) k_extend(Batch bt, const SubDesc *subs, const double *tab, double *ws, int grad) {
+  pdl_wait();
   Item it; int local;
   locate(bt, blockIdx.x, it, local);
   MDP_CHECK_ITEM(bt, subs, it, local, F_EXT);
@@ -115,6 +116,7 @@ __device__ __forceinline__ cplx ring_stencil(const SubDesc &d, const Item &it, c
 template <bool CIN, bool GRAD>
 __global__ void __launch_bounds__(256) k_residual(Batch bt, const SubDesc *subs, const double *tab, double *ws,
                                                   const double2 *xi_user) {
+  pdl_wait();
   Item it; int local;
   locate(bt, blockIdx.x, it, local);
   MDP_CHECK_ITEM(bt, subs, it, local, F_RES);
@@ -184,6 +186,7 @@ __device__ __forceinline__ double side_density(const SubDesc &d, const Item &it,
 }
 template <bool GRAD>
 __global__ void __launch_bounds__(256) k_ring(Batch bt, const SubDesc *subs, const double *tab, double *ws) {
+  pdl_wait();
   Item it; int local;
   locate(bt, blockIdx.x, it, local);
   MDP_CHECK_ITEM(bt, subs, it, local, F_RING);
@@ -1426,6 +1429,7 @@ __global__ void __launch_bounds__(256) k_basis_out(Item it, const SubDesc *subs,
 // elsewhere: the only nodes of M+ where L w is nonzero), written into the zeroed grid
 // u[c][n][m] that the full-grid solve then reads.
 __global__ void __launch_bounds__(256) k_pot_rhs(int sub, const SubDesc *subs, int ncols, const double2 *xi, double2 *u) {
+  pdl_wait();
   const SubDesc &d = subs[sub];
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= (long long)ncols * d.R) return;
@@ -1450,6 +1454,7 @@ __global__ void __launch_bounds__(256) k_pot_rhs(int sub, const SubDesc *subs, i
 
 // u <- w - u on every node (w = xi on gamma, 0 elsewhere): the difference potential.
 __global__ void __launch_bounds__(256) k_pot_fix(int sub, const SubDesc *subs, int ncols, const double2 *xi, double2 *u) {
+  pdl_wait();
   const SubDesc &d = subs[sub];
   const long long npt = (long long)d.nx * d.ny;
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1539,13 +1544,13 @@ cudaError_t launch_potential(const mdp_plan *p, int sub, int ncols, const double
   cudaError_t e = cudaMemsetAsync(u, 0, (size_t)ncols * npt * sizeof(double2), st);
   if (e != cudaSuccess) return e;
   const long long nr = (long long)ncols * d.R;
-  k_pot_rhs<<<(unsigned)((nr + 255) / 256), 256, 0, st>>>(sub, p->d_subs, ncols, xi, u);
+  pdl(k_pot_rhs, dim3((unsigned)((nr + 255) / 256)), dim3(256), 0, st, sub, p->d_subs, ncols, xi, u);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   e = launch_solve(p, sub, ncols, u, u, 0, st);
   if (e != cudaSuccess) return e;
   const long long nt = (long long)ncols * npt;
-  k_pot_fix<<<(unsigned)((nt + 255) / 256), 256, 0, st>>>(sub, p->d_subs, ncols, xi, u);
+  pdl(k_pot_fix, dim3((unsigned)((nt + 255) / 256)), dim3(256), 0, st, sub, p->d_subs, ncols, xi, u);
   return cudaGetLastError();
 }
 
@@ -1603,7 +1608,7 @@ cudaError_t launch_basis_densities(const mdp_plan *p, int sub, int col0, int nco
     std::memset(&b, 0, sizeof b);
     b.n_items = 1; b.one = it; b.total_blocks = blocks_for(F_EXT, d, it.ncols, it.col0);
     set_bounds(p, b, (long long)ncols * d.G, false);
-    k_extend<<<dim3((unsigned)b.total_blocks), 32, 0, st>>>(b, p->d_subs, p->d_tables, p->d_ws, 0);
+    pdl(k_extend, dim3((unsigned)b.total_blocks), dim3(32), 0, st, b, p->d_subs, p->d_tables, p->d_ws, 0);
     const long long n = (long long)it.ncols * d.G;
     k_basis_out<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(it, p->d_subs, p->d_tables, p->d_ws,
                                                               out + (long long)c * d.G);
@@ -1655,11 +1660,11 @@ cudaError_t launch_project(mdp_plan *p, const Batch *fb, int out_kind, const dou
     }                                             \
   } while (0)
 #define MDP_LAUNCH(fam, ...) MDP_LAUNCH_AS(fam, fam, __VA_ARGS__)
-  if (basis) MDP_LAUNCH(F_EXT, k_extend<<<grid1(fb[F_EXT].total_blocks), 32, 0, st>>>(fb[F_EXT], ds, tab, ws, 0));
+  if (basis) MDP_LAUNCH(F_EXT, pdl(k_extend, grid1(fb[F_EXT].total_blocks), dim3(32), 0, st, fb[F_EXT], ds, tab, ws, 0));
   if (basis) {
-    MDP_LAUNCH_AS(F_RING, F_RES, k_ring<false><<<grid1(fb[F_RING].total_blocks), b8, 0, st>>>(fb[F_RING], ds, tab, ws));
-    MDP_LAUNCH_AS(F_PRES, F_RES, k_residual<false, false><<<grid1(fb[F_PRES].total_blocks), b8, 0, st>>>(fb[F_PRES], ds, tab, ws, xi_user));
-  } else MDP_LAUNCH(F_RES, k_residual<true, false><<<grid1(fb[F_RES].total_blocks), b8, 0, st>>>(fb[F_RES], ds, tab, ws, xi_user));
+    MDP_LAUNCH_AS(F_RING, F_RES, pdl(k_ring<false>, grid1(fb[F_RING].total_blocks), b8, 0, st, fb[F_RING], ds, tab, ws));
+    MDP_LAUNCH_AS(F_PRES, F_RES, pdl(k_residual<false, false>, grid1(fb[F_PRES].total_blocks), b8, 0, st, fb[F_PRES], ds, tab, ws, xi_user));
+  } else MDP_LAUNCH(F_RES, pdl(k_residual<true, false>, grid1(fb[F_RES].total_blocks), b8, 0, st, fb[F_RES], ds, tab, ws, xi_user));
   if (basis) MDP_LAUNCH(F_FROWS, k_fwd_rows<false><<<grid1(fb[F_FROWS].total_blocks), b8, p->fft_smem, st>>>(fb[F_FROWS], ds, tab, ws));
   else MDP_LAUNCH(F_FROWS, k_fwd_rows<true><<<grid1(fb[F_FROWS].total_blocks), b8, p->fft_smem, st>>>(fb[F_FROWS], ds, tab, ws));
   cudaError_t e = launch_sep_project(p, fb, out_kind, xi_user, out, out_rec, st);
@@ -1693,11 +1698,11 @@ cudaError_t launch_adjoint(mdp_plan *p, const Batch *fb, int out_kind, const dou
   cudaError_t e = launch_adj_clear(p, fb, st);
   if (e != cudaSuccess) return e;
   if (grad_k) {  // the residual and the k-derivative sources; by sweeps: forward recompute with every mode-space row kept
-    if (basis) MDP_LAUNCH(F_EXT, k_extend<<<grid1(fb[F_EXT].total_blocks), 32, 0, st>>>(fb[F_EXT], ds, tab, ws, 1));
+    if (basis) MDP_LAUNCH(F_EXT, pdl(k_extend, grid1(fb[F_EXT].total_blocks), dim3(32), 0, st, fb[F_EXT], ds, tab, ws, 1));
     if (basis) {
-      MDP_LAUNCH_AS(F_RING, F_RES, k_ring<true><<<grid1(fb[F_RING].total_blocks), b8, 0, st>>>(fb[F_RING], ds, tab, ws));
-      MDP_LAUNCH_AS(F_PRES, F_RES, k_residual<false, true><<<grid1(fb[F_PRES].total_blocks), b8, 0, st>>>(fb[F_PRES], ds, tab, ws, xi_user));
-    } else MDP_LAUNCH(F_RES, k_residual<true, true><<<grid1(fb[F_RES].total_blocks), b8, 0, st>>>(fb[F_RES], ds, tab, ws, xi_user));
+      MDP_LAUNCH_AS(F_RING, F_RES, pdl(k_ring<true>, grid1(fb[F_RING].total_blocks), b8, 0, st, fb[F_RING], ds, tab, ws));
+      MDP_LAUNCH_AS(F_PRES, F_RES, pdl(k_residual<false, true>, grid1(fb[F_PRES].total_blocks), b8, 0, st, fb[F_PRES], ds, tab, ws, xi_user));
+    } else MDP_LAUNCH(F_RES, pdl(k_residual<true, true>, grid1(fb[F_RES].total_blocks), b8, 0, st, fb[F_RES], ds, tab, ws, xi_user));
     if (basis) MDP_LAUNCH(F_FROWS, k_fwd_rows<false><<<grid1(fb[F_FROWS].total_blocks), b8, p->fft_smem, st>>>(fb[F_FROWS], ds, tab, ws));
     else MDP_LAUNCH(F_FROWS, k_fwd_rows<true><<<grid1(fb[F_FROWS].total_blocks), b8, p->fft_smem, st>>>(fb[F_FROWS], ds, tab, ws));
     if (basis) MDP_LAUNCH(F_TRI, k_tri<false, true, 2><<<grid1(fb[F_TRI].total_blocks), btri, TRI_WARPS * 2 * full_stage_bytes<false>(), st>>>(fb[F_TRI], ds, tab, p->d_piv, ws, p->d_sep));

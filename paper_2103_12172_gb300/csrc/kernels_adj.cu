@@ -131,6 +131,7 @@ __global__ void __launch_bounds__(256) k_adj_rows(Batch bt, const SubDesc *subs,
 // (-1)^(q+1) sin(pi q m/Nx) for the mirrored column m') the slots hold the pairs
 // (c0 + c3, c0 - c3, c1 + c2, c1 - c2), and a mode needs two of them.
 __global__ void __launch_bounds__(256) k_adj_cols(Batch bt, const SubDesc *subs, double *ws, const double2 *cot) {
+  pdl_wait();
   Item it; int local;
   locate(bt, blockIdx.x, it, local);
   MDP_CHECK_ITEM(bt, subs, it, local, F_ACOLS);
@@ -581,6 +582,7 @@ __global__ void __launch_bounds__(256) k_adj_ring_cols(Batch bt, const SubDesc *
 template <bool CIN, bool DK>
 __global__ void __launch_bounds__(256) k_adj_gamma(Batch bt, const SubDesc *subs, const double *tab, double *ws,
                                                    const double2 *cot, double2 *grad_xi, int kind) {
+  pdl_wait();
   __shared__ double sh[256];
   Item it; int local;
   locate(bt, blockIdx.x, it, local);
@@ -627,6 +629,7 @@ __global__ void __launch_bounds__(256) k_adj_gamma(Batch bt, const SubDesc *subs
 
 // per item: the sum of its partials in slot order; then per subdomain in item order
 __global__ void __launch_bounds__(256) k_red_items(const Item *items, const SubDesc *subs, double *ws) {
+  pdl_wait();
   __shared__ double sh[256];
   const Item it = items[blockIdx.x];
   const SubDesc &d = subs[it.sub];
@@ -645,6 +648,7 @@ __global__ void __launch_bounds__(256) k_red_items(const Item *items, const SubD
 }
 
 __global__ void k_red_subs(const Item *items, int n_items, const SubDesc *subs, const double *ws, double *grad_k) {
+  pdl_wait();
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
   for (int i = 0; i < n_items; ++i) {
     const Item it = items[i];
@@ -677,7 +681,7 @@ cudaError_t launch_adjoint_tail(mdp_plan *p, const Batch *fb, int out_kind, cons
     }                                             \
   } while (0)
   ADJ_LAUNCH(F_AFWD, k_adj_rows<<<g1(fb[F_AFWD].total_blocks), b8, p->fft_smem, st>>>(fb[F_AFWD], ds, tab, ws, cot, cot_rec));
-  ADJ_LAUNCH(F_ACOLS, k_adj_cols<<<g1(fb[F_ACOLS].total_blocks), b8, 0, st>>>(fb[F_ACOLS], ds, ws, cot));
+  ADJ_LAUNCH(F_ACOLS, pdl(k_adj_cols, g1(fb[F_ACOLS].total_blocks), b8, 0, st, fb[F_ACOLS], ds, ws, cot));
   const cudaError_t e = launch_sep_adjoint(p, fb, !basis, dk, cot, cot_rec, st);
   if (e != cudaSuccess) return e;
   if (dk) ADJ_LAUNCH(F_ATRI, k_adj_tri<true><<<g1(fb[F_ATRI].total_blocks), b4, 4 * adj_warp_smem(), st>>>(fb[F_ATRI], ds, tab, p->d_piv, ws, cot_rec ? 1 : 0));
@@ -690,14 +694,14 @@ cudaError_t launch_adjoint_tail(mdp_plan *p, const Batch *fb, int out_kind, cons
     ADJ_LAUNCH(F_ARINGC, k_adj_ring_cols<false><<<g1(fb[F_ARINGC].total_blocks), b8, 0, st>>>(fb[F_ARINGC], ds, tab, ws));
   }
   if (dk && basis)
-    ADJ_LAUNCH(F_AGAM, k_adj_gamma<false, true><<<g1(fb[F_AGAM].total_blocks), b8, 0, st>>>(fb[F_AGAM], ds, tab, ws, cot, grad_xi, out_kind));
+    ADJ_LAUNCH(F_AGAM, pdl(k_adj_gamma<false, true>, g1(fb[F_AGAM].total_blocks), b8, 0, st, fb[F_AGAM], ds, tab, ws, cot, grad_xi, out_kind));
   else if (dk)
-    ADJ_LAUNCH(F_AGAM, k_adj_gamma<true, true><<<g1(fb[F_AGAM].total_blocks), b8, 0, st>>>(fb[F_AGAM], ds, tab, ws, cot, grad_xi, out_kind));
+    ADJ_LAUNCH(F_AGAM, pdl(k_adj_gamma<true, true>, g1(fb[F_AGAM].total_blocks), b8, 0, st, fb[F_AGAM], ds, tab, ws, cot, grad_xi, out_kind));
   else if (grad_xi)
-    ADJ_LAUNCH(F_AGAM, k_adj_gamma<true, false><<<g1(fb[F_AGAM].total_blocks), b8, 0, st>>>(fb[F_AGAM], ds, tab, ws, cot, grad_xi, out_kind));
+    ADJ_LAUNCH(F_AGAM, pdl(k_adj_gamma<true, false>, g1(fb[F_AGAM].total_blocks), b8, 0, st, fb[F_AGAM], ds, tab, ws, cot, grad_xi, out_kind));
   if (dk) {
-    k_red_items<<<fb[F_ATRI].n_items, 256, 0, st>>>(fb[F_ATRI].items, ds, ws);
-    k_red_subs<<<1, 32, 0, st>>>(fb[F_ATRI].items, fb[F_ATRI].n_items, ds, ws, grad_k);
+    pdl(k_red_items, dim3(fb[F_ATRI].n_items), dim3(256), 0, st, fb[F_ATRI].items, ds, ws);
+    pdl(k_red_subs, dim3(1), dim3(32), 0, st, fb[F_ATRI].items, fb[F_ATRI].n_items, ds, ws, grad_k);
   }
   return cudaGetLastError();
 }

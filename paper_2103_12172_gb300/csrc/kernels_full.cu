@@ -74,6 +74,7 @@ struct FullArg {
 // Row order (right-hand side, unknown row, part): a block's 8 rows are 4 grid rows, complex parts in turn.
 template <bool INV>
 __global__ void __launch_bounds__(256) k_full_cut(const __grid_constant__ FullArg p, const double2 *g) {
+  pdl_wait();
   const SubDesc &d = p.d;
   const SepGeo &geo = p.g;
   const FullWs &w = p.w;
@@ -158,6 +159,7 @@ struct FullSrc {
 
 template <bool INV>
 __global__ void __launch_bounds__(SG_THREADS, 1) k_full_gemm(const __grid_constant__ FullArg p, int *status) {
+  pdl_wait();
   const FullSrc<INV> src{p};
   digit_gemm(src, status);
 }
@@ -178,6 +180,7 @@ __device__ __forceinline__ double ipow(double x, int n) {
 }
 constexpr int FULL_Y_CTAS = 4, FULL_Y_WARPS = 8;   // CTAs of a cluster, most warps of one
 __global__ void __cluster_dims__(1, 1, FULL_Y_CTAS) __launch_bounds__(32 * FULL_Y_WARPS) k_full_y(const __grid_constant__ FullArg p) {
+  pdl_wait();
   extern __shared__ double ysh[];   // [2][warps][32] of this CTA, [2][all warps][32], then this CTA's rows [rows][32]
   const cg::cluster_group cl = cg::this_cluster();
   const SubDesc &d = p.d;
@@ -329,6 +332,7 @@ __global__ void __cluster_dims__(1, 1, FULL_Y_CTAS) __launch_bounds__(32 * FULL_
 
 // u(m) = U_0 + U_1, u(Nx - m) = U_0 - U_1 on the unknown rows, 0 on the Dirichlet ends.
 __global__ void __launch_bounds__(256) k_full_out(const __grid_constant__ FullArg p, double2 *u) {
+  pdl_wait();
   const SubDesc &d = p.d;
   const FullWs &w = p.w;
   const double *ws = p.ws;
@@ -389,13 +393,13 @@ cudaError_t launch_full_solve(const mdp_plan *p, int sub, int nrhs, const double
     cudaError_t e = cudaMemsetAsync(p->d_ws + w.mask, 0, 2LL * (w.R / 128) * SEP_MASK * 8, st);
     if (e != cudaSuccess) return e;
     const FullArg a{d, geo, w, nr, p->d_sep, p->d_ws};
-    k_full_cut<false><<<dim3(w.R / 8, 2), 256, 0, st>>>(a, gc);
-    k_full_gemm<false><<<gemm_grid(geo.nqh / 32), SG_THREADS, SG_SMEM, st>>>(a, p->d_status);
-    k_full_y<<<dim3(w.ldf / 16, nr, FULL_Y_CTAS), dim3(32, nw), ysm, st>>>(a);
-    k_full_cut<true><<<dim3(w.R / 8, 2), 256, 0, st>>>(a, gc);
-    k_full_gemm<true><<<gemm_grid(geo.ntx), SG_THREADS, SG_SMEM, st>>>(a, p->d_status);
+    pdl(k_full_cut<false>, dim3(w.R / 8, 2), dim3(256), 0, st, a, gc);
+    pdl(k_full_gemm<false>, dim3(gemm_grid(geo.nqh / 32)), dim3(SG_THREADS), SG_SMEM, st, a, p->d_status);
+    pdl(k_full_y, dim3(w.ldf / 16, nr, FULL_Y_CTAS), dim3(32, nw), ysm, st, a);
+    pdl(k_full_cut<true>, dim3(w.R / 8, 2), dim3(256), 0, st, a, gc);
+    pdl(k_full_gemm<true>, dim3(gemm_grid(geo.ntx)), dim3(SG_THREADS), SG_SMEM, st, a, p->d_status);
     const int nm = d.Nx / 2 + 1, tm = std::min(256, (nm + 31) / 32 * 32);
-    k_full_out<<<dim3((nm + tm - 1) / tm, d.ny, nr), tm, 0, st>>>(a, uc);
+    pdl(k_full_out, dim3((nm + tm - 1) / tm, d.ny, nr), dim3(tm), 0, st, a, uc);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }

@@ -492,6 +492,7 @@ __device__ __forceinline__ void sep_cut_body(const Item &it, const SubDesc &d, d
 
 template <bool CIN, int STAGE>
 __global__ void __launch_bounds__(256) k_sep_cut(Batch bt, const SubDesc *subs, double *ws, int fam) {
+  pdl_wait();
   Item it; int local;
   locate(bt, blockIdx.x, it, local);
   MDP_CHECK_ITEM(bt, subs, it, local, fam);
@@ -591,6 +592,7 @@ struct SepSrc {
 template <int STAGE>
 __global__ void __launch_bounds__(SG_THREADS, 1)
     k_sep_gemm(Batch bt, const SubDesc *subs, const unsigned char *sep, double *ws, int user, int fam, int *status) {
+  pdl_wait();
   const SepSrc<STAGE> src{bt, subs, sep, ws, user, fam};
   digit_gemm(src, status);
 }
@@ -684,6 +686,7 @@ __device__ __forceinline__ void sep_modes_body(const Item &it, const SubDesc &d,
 
 template <bool CIN>
 __global__ void __launch_bounds__(128) k_sep_modes(Batch bt, const SubDesc *subs, const unsigned char *sep, double *ws) {
+  pdl_wait();
   Item it; int local;
   locate(bt, blockIdx.x, it, local);
   MDP_CHECK_ITEM(bt, subs, it, local, F_SMODE);
@@ -785,6 +788,7 @@ __device__ __forceinline__ void sep_rows_out_body(const Item &it, const SubDesc 
 template <bool CIN>
 __global__ void __launch_bounds__(256) k_sep_out(Batch bt, const SubDesc *subs, const double *tab, const double *ws,
                                                  const double2 *xi_user, double2 *out, double2 *out_rec, int kind) {
+  pdl_wait();
   __shared__ double2 sh[2][32][33];
   Item it; int local;
   locate(bt, blockIdx.x, it, local);
@@ -872,8 +876,8 @@ cudaError_t launch_sep_sines(const mdp_plan *p, const SubDesc *ds, const double 
 }
 
 cudaError_t launch_sep_cut1(const Batch &b, const SubDesc *subs, double *ws, bool user, int fam, cudaStream_t st) {
-  if (user) k_sep_cut<true, 1><<<b.total_blocks, 256, 0, st>>>(b, subs, ws, fam);
-  else k_sep_cut<false, 1><<<b.total_blocks, 256, 0, st>>>(b, subs, ws, fam);
+  if (user) pdl(k_sep_cut<true, 1>, b.total_blocks, dim3(256), 0, st, b, subs, ws, fam);
+  else pdl(k_sep_cut<false, 1>, b.total_blocks, dim3(256), 0, st, b, subs, ws, fam);
   return cudaGetLastError();
 }
 
@@ -892,16 +896,16 @@ cudaError_t launch_sep_project(mdp_plan *p, const Batch *fb, int out_kind, const
     __VA_ARGS__;              \
     prof_end(p, as, st);      \
   } while (0)
-  if (user) SEP_LAUNCH(F_C1B, k_sep_cut<true, 1><<<grid(f1c), 256, 0, st>>>(fb[f1c], ds, ws, f1c));
-  else SEP_LAUNCH(F_C1B, k_sep_cut<false, 1><<<grid(f1c), 256, 0, st>>>(fb[f1c], ds, ws, f1c));
-  SEP_LAUNCH(F_G1B, k_sep_gemm<1><<<gemm_grid(f1), SG_THREADS, SG_SMEM, st>>>(fb[f1], ds, p->d_sep, ws, user, f1, p->d_status));
-  if (user) SEP_LAUNCH(F_SMODE, k_sep_modes<true><<<grid(F_SMODE), dim3(32, 4), 0, st>>>(fb[F_SMODE], ds, p->d_sep, ws));
-  else SEP_LAUNCH(F_SMODE, k_sep_modes<false><<<grid(F_SMODE), dim3(32, 4), 0, st>>>(fb[F_SMODE], ds, p->d_sep, ws));
-  if (user) SEP_LAUNCH(F_C3B, k_sep_cut<true, 3><<<grid(f3c), 256, 0, st>>>(fb[f3c], ds, ws, f3c));
-  else SEP_LAUNCH(F_C3B, k_sep_cut<false, 3><<<grid(f3c), 256, 0, st>>>(fb[f3c], ds, ws, f3c));
-  SEP_LAUNCH(F_TCOLS, k_sep_gemm<3><<<gemm_grid(f3), SG_THREADS, SG_SMEM, st>>>(fb[f3], ds, p->d_sep, ws, user, f3, p->d_status));
-  if (user) SEP_LAUNCH(F_SOUT, k_sep_out<true><<<grid(F_SOUT), dim3(32, 8), 0, st>>>(fb[F_SOUT], ds, p->d_tables, ws, xi_user, out, out_rec, out_kind));
-  else SEP_LAUNCH(F_SOUT, k_sep_out<false><<<grid(F_SOUT), dim3(32, 8), 0, st>>>(fb[F_SOUT], ds, p->d_tables, ws, xi_user, out, out_rec, out_kind));
+  if (user) SEP_LAUNCH(F_C1B, pdl(k_sep_cut<true, 1>, grid(f1c), dim3(256), 0, st, fb[f1c], ds, ws, f1c));
+  else SEP_LAUNCH(F_C1B, pdl(k_sep_cut<false, 1>, grid(f1c), dim3(256), 0, st, fb[f1c], ds, ws, f1c));
+  SEP_LAUNCH(F_G1B, pdl(k_sep_gemm<1>, dim3(gemm_grid(f1)), dim3(SG_THREADS), SG_SMEM, st, fb[f1], ds, p->d_sep, ws, user, f1, p->d_status));
+  if (user) SEP_LAUNCH(F_SMODE, pdl(k_sep_modes<true>, grid(F_SMODE), dim3(32, 4), 0, st, fb[F_SMODE], ds, p->d_sep, ws));
+  else SEP_LAUNCH(F_SMODE, pdl(k_sep_modes<false>, grid(F_SMODE), dim3(32, 4), 0, st, fb[F_SMODE], ds, p->d_sep, ws));
+  if (user) SEP_LAUNCH(F_C3B, pdl(k_sep_cut<true, 3>, grid(f3c), dim3(256), 0, st, fb[f3c], ds, ws, f3c));
+  else SEP_LAUNCH(F_C3B, pdl(k_sep_cut<false, 3>, grid(f3c), dim3(256), 0, st, fb[f3c], ds, ws, f3c));
+  SEP_LAUNCH(F_TCOLS, pdl(k_sep_gemm<3>, dim3(gemm_grid(f3)), dim3(SG_THREADS), SG_SMEM, st, fb[f3], ds, p->d_sep, ws, user, f3, p->d_status));
+  if (user) SEP_LAUNCH(F_SOUT, pdl(k_sep_out<true>, grid(F_SOUT), dim3(32, 8), 0, st, fb[F_SOUT], ds, p->d_tables, ws, xi_user, out, out_rec, out_kind));
+  else SEP_LAUNCH(F_SOUT, pdl(k_sep_out<false>, grid(F_SOUT), dim3(32, 8), 0, st, fb[F_SOUT], ds, p->d_tables, ws, xi_user, out, out_rec, out_kind));
 #undef SEP_LAUNCH
   return cudaGetLastError();
 }

@@ -470,6 +470,7 @@ __global__ void __launch_bounds__(256) k_adj_sines(const SubDesc *subs, int s0, 
 
 // ---------------------------------------------------------------- operands
 __global__ void __launch_bounds__(256) k_adj_clear(Batch bt, const SubDesc *subs, double *ws) {
+  pdl_wait();
   Item it; int local;
   locate(bt, blockIdx.x, it, local);
   MDP_CHECK_ITEM(bt, subs, it, local, F_ACLR);
@@ -568,6 +569,7 @@ __device__ __forceinline__ void adj_cut_body(const Item &it, const SubDesc &d, d
 template <int STAGE>
 __global__ void __launch_bounds__(256) k_adj_cut(Batch bt, const SubDesc *subs, double *ws, const double2 *cot,
                                                  const double2 *cot_rec) {
+  pdl_wait();
   Item it; int local;
   locate(bt, blockIdx.x, it, local);
   MDP_CHECK_ITEM(bt, subs, it, local, STAGE == 1 ? F_AC1 : F_AC3);
@@ -745,12 +747,14 @@ struct AdjSrc {
 __global__ void __launch_bounds__(SG_THREADS, 1)
     k_grad_gemm(Batch bt, const SubDesc *subs, const unsigned char *sep, const unsigned char *adj, double *ws, int user, int fam,
                 int *status) {
+  pdl_wait();
   const GradSrc src{bt, subs, sep, adj, ws, user, fam};
   digit_gemm(src, status);
 }
 template <int STAGE>
 __global__ void __launch_bounds__(SG_THREADS, 1)
     k_adj_gemm(Batch bt, const SubDesc *subs, const unsigned char *adj, double *ws, int *status) {
+  pdl_wait();
   const AdjSrc<STAGE> src{bt, subs, adj, ws};
   digit_gemm(src, status);
 }
@@ -902,6 +906,7 @@ __device__ __forceinline__ double adj_modes_body(const Item &it, const SubDesc &
 template <bool CIN, bool DK>
 __global__ void __launch_bounds__(128) k_adj_modes(Batch bt, const SubDesc *subs, const unsigned char *sep, const unsigned char *adj,
                                                    double *ws, int has_rec) {
+  pdl_wait();
   __shared__ double sh[128];
   Item it; int local;
   locate(bt, blockIdx.x, it, local);
@@ -931,6 +936,7 @@ __global__ void __launch_bounds__(128) k_adj_modes(Batch bt, const SubDesc *subs
 // k-gradient's parts -Re <mu, s> and, of the middle rows, -Re <c, (dK/dk r)>.
 template <bool CIN, bool DK>
 __global__ void __launch_bounds__(256) k_adj_out(Batch bt, const SubDesc *subs, double *ws, const double2 *cot) {
+  pdl_wait();
   __shared__ double sh[256];
   Item it; int local;
   locate(bt, blockIdx.x, it, local);
@@ -1081,8 +1087,8 @@ cudaError_t launch_sep_adj_residual(mdp_plan *p, const Batch *fb, bool user, cud
   prof_end(p, F_C1B, st);
   if (e != cudaSuccess) return e;
   prof_begin(p, F_GG1B, st);
-  k_grad_gemm<<<std::min(fb[fg].total_blocks, p->n_sm), SG_THREADS, SG_SMEM, st>>>(fb[fg], p->d_subs, p->d_sep, p->d_adj, p->d_ws,
-                                                                                  user, fg, p->d_status);
+  pdl(k_grad_gemm, dim3(std::min(fb[fg].total_blocks, p->n_sm)), dim3(SG_THREADS), SG_SMEM, st, fb[fg], p->d_subs, p->d_sep,
+      p->d_adj, p->d_ws, user, fg, p->d_status);
   prof_end(p, F_GG1B, st);
   return cudaGetLastError();
 }
@@ -1099,7 +1105,7 @@ cudaError_t launch_sep_adjoint(mdp_plan *p, const Batch *fb, bool user, bool dk,
 #define ADJ_LAUNCH(f, kern, grid, block, smem, ...)                                  \
   do {                                                                               \
     prof_begin(p, f, st);                                                            \
-    kern<<<grid, block, smem, st>>>(fb[f], ds, __VA_ARGS__);                         \
+    pdl(kern, dim3(grid), dim3(block), smem, st, fb[f], ds, __VA_ARGS__);            \
     prof_end(p, f, st);                                                              \
   } while (0)
   ADJ_LAUNCH(F_AC1, k_adj_cut<1>, fb[F_AC1].total_blocks, 256, 0, ws, cot, cot_rec);
@@ -1119,7 +1125,7 @@ cudaError_t launch_sep_adjoint(mdp_plan *p, const Batch *fb, bool user, bool dk,
 // the operand masks of a wave's items, before anything is cut into them
 cudaError_t launch_adj_clear(mdp_plan *p, const Batch *fb, cudaStream_t st) {
   if (fb[F_ACLR].total_blocks == 0) return cudaSuccess;
-  k_adj_clear<<<fb[F_ACLR].total_blocks, 256, 0, st>>>(fb[F_ACLR], p->d_subs, p->d_ws);
+  pdl(k_adj_clear, dim3(fb[F_ACLR].total_blocks), dim3(256), 0, st, fb[F_ACLR], p->d_subs, p->d_ws);
   return cudaGetLastError();
 }
 

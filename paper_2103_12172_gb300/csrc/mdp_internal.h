@@ -4,6 +4,7 @@
 #include <vector>
 #include <string>
 #include <algorithm>
+#include <utility>
 #include <cstdlib>
 #include <cmath>
 #include <cstring>
@@ -485,7 +486,7 @@ struct mdp_plan {
   unsigned char *d_sep = nullptr;        // separable tables (kernels_sep.cu), rebuilt with the factor tables
   unsigned char *d_adj = nullptr;        // gradient tables (kernels_sepadj.cu), one set: rebuilt by the gradient
   long long adj_bytes = 0, adj_masks = 0;   // pass when the wavenumbers have changed since (adj_stale)
-  bool adj_stale = true, adj_sines = false;
+  bool adj_stale = true, adj_sines = false, adj_captured = false;
   cudaStream_t side = nullptr;           // an update's factorisation beside its separable tables, with the events
   cudaEvent_t fork_ev = nullptr, join_ev = nullptr;   // that fork it from and join it to the caller's stream
   long long sep_bytes = 0, sep_masks = 0;   // size; its first bytes: the masks, cleared before a rebuild
@@ -676,6 +677,25 @@ cudaError_t launch_factor_to(const mdp_plan *p, const SubDesc *ds, double *tab, 
 void host_mode_solve(const HostSub &hs, int q, int adjoint, const double *b, double *x);
 // kernel launchers (kernels.cu)
 enum { PASS_FWD = 0, PASS_GRAD = 1 };
+#ifdef __CUDACC__
+// Launch whose set-up overlaps the kernel before it on the stream (programmatic dependent launch): its blocks come
+// as that kernel's last ones leave, and every kernel launched so first waits in pdl_wait(), which returns when
+// the kernels before it are complete and their writes visible. Eight kernels of a pass of 129^2: 84.6 -> 66.4 us;
+// 4 x 257^2: 231 -> 214 us. No earlier trigger: blocks that wait take the registers and shared memory of the
+// kernel before (279 us with one at each kernel's start).
+template <class... P, class... A>
+inline void pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A &&...args) {
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = grid; c.blockDim = block; c.dynamicSmemBytes = smem; c.stream = st; c.attrs = &at; c.numAttrs = 1;
+  cudaLaunchKernelEx(&c, kernel, std::forward<A>(args)...);
+}
+__device__ __forceinline__ void pdl_wait() {
+  cudaGridDependencySynchronize();
+}
+#endif
 cudaError_t set_kernel_attributes();      // kernels.cu: opt-in shared memory of the FFT kernels
 cudaError_t set_adj_kernel_attributes();  // kernels_adj.cu
 cudaError_t set_sep_kernel_attributes();  // kernels_sep.cu

@@ -160,3 +160,26 @@ def test_gradient_is_that_of_the_sweeps(mdp, name, sub, user, rec, kind):
         if user:
             assert rel_col_err(ga.view(nc, G).cpu().numpy(), gb.view(nc, G).cpu().numpy()) < 1e-10
         assert abs(ka.item() - kb.item()) < 1e-9 * abs(kb.item())
+
+
+def test_captured_gradient_follows_the_wavenumbers(mdp):
+    """A first gradient call inside a stream capture (its tables are allocated and made there), replayed after a
+    change of k, and plain calls afterwards: bit for bit those of a plan that never captured."""
+    sub = W.small_subdomain(65, 9.0, W.AP_DIRX_SOMMY, 2)
+    plan, ref = mdp.Plan([sub]), mdp.Plan([sub])
+    cot = torch.from_numpy(W.random_complex(plan.output_size, seed=15)).cuda()
+    s = torch.cuda.Stream()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.stream(s):
+        g.capture_begin()
+        gx, gk = plan.adjoint(cot)
+        g.capture_end()
+    for k in (9.0, 9.4):
+        for p in (plan, ref):
+            p.update_k([k])
+        g.replay()
+        torch.cuda.synchronize()
+        for p, out in ((ref, (gx, gk)), (plan, (gx, gk))):
+            rx, rk = p.adjoint(cot)
+            assert torch.equal(out[0], rx) and torch.equal(out[1], rk)
+    plan.status()
