@@ -69,14 +69,17 @@ enum { MDP_OUT_Q = 0, MDP_OUT_P = 1 };
  * subdomains (Section 4). User densities, receivers and the adjoint still run per subdomain
  * (on the shared tables). mdp_plan_update_k then requires equal k within each group. */
 #define MDP_PLAN_DEDUPE 0x4u
-/* Kernel variants (the same results to rounding; the autotuner times them): the gamma columns of
- * the middle rows by FP64 sums instead of the tensor-core contraction, and the sine transforms of
- * the dense ring and gamma rows by direct sums instead of the FFT. */
+/* Kernel variants (the same results to rounding; the autotuner times them): every pass by per-mode sweeps
+ * and FP64 sums instead of the separable Green's function with its contractions on the tensor cores
+ * (which subdomains take it: up to 2048 cells along x where M+ is centred, 1024 otherwise, and up to 2050, 1026
+ * rows of M+), and, in the sweeps, the sine transforms of the dense ring and gamma rows by direct sums
+ * instead of the FFT. */
 #define MDP_PLAN_FP64_COLS 0x8u
 #define MDP_PLAN_DIRECT_ROWS 0x10u
 
-/* Plan options (0 selects the default: environment MDP_TILE_COLS / MDP_WS_MB, else 256 columns
- * per work item and a 4 GiB workspace budget; 1024 points per FFT block; 2 staged rows). */
+/* Plan options (0 selects the default: environment MDP_TILE_COLS / MDP_WS_MB, else 512 columns per work
+ * item of the separable solve, 256 of the sweeps, and a 4 GiB workspace budget; 1024 points per FFT
+ * block; 2 staged rows; the last two concern the sweeps only). */
 typedef struct {
   int tile_cols;              /* columns per work item (the batching tile) */
   long long workspace_bytes;  /* budget that packs work items into waves */
@@ -121,8 +124,8 @@ mdp_status mdp_ap_plan_ex(const mdp_subdomain *subs, int n_subs, unsigned flags,
 /* Replace the wavenumbers (k[n_subs], host array, each > 0 and finite, else MDP_ERR_ARG) and
  * refactor every sine mode in place (Section 3.2.1: the per-mode tridiagonal systems of the
  * separable AP; same grids, no reallocation). On a device plan the factorisation runs on the
- * GPU, on cuda_stream (NULL: the legacy default stream): the pivoted LU of each mode, its
- * dT/dk rows and the projection's condensed sweep table are rebuilt in the device tables. The
+ * GPU, on cuda_stream (NULL: the legacy default stream): the pivoted LU of each mode and the tables
+ * of the separable solve, or of the sweeps, are rebuilt in the device tables. The
  * call returns when they are done; MDP_ERR_SINGULAR if a mode of the new k is singular (the
  * tables are then unusable until a successful update). Host-only plans factor on the host.
  * mdp_plan_update_k is mdp_plan_update_k_stream on the legacy default stream. */

@@ -51,11 +51,11 @@ class Plan:
     def __init__(self, subdomains, host_only: bool = False, graph: bool = False, tile_cols: int = 0,
                  workspace_bytes: int = 0, dedupe: bool = False, fp64_cols: bool = False,
                  direct_rows: bool = False, fft_block_points: int = 0, tri_stages: int = 0):
-        """Kernel variants (same results to rounding; see autotune.tune_plan): fp64_cols sums the
-        gamma columns of the middle rows on the FP64 pipe instead of the tensor cores, direct_rows
-        takes the dense-row sine transforms by direct sums instead of the FFT, fft_block_points
-        sets the complex values per FFT block (1024, 2048 or 4096), tri_stages the rows the per-mode
-        sweep stages ahead (2 or 4); 0 selects the defaults."""
+        """Kernel variants (same results to rounding; see autotune.tune_plan): fp64_cols takes per-mode
+        sweeps and FP64 sums instead of the separable solve on the tensor cores; in the sweeps,
+        direct_rows takes the dense-row sine transforms by direct sums instead of the FFT,
+        fft_block_points sets the complex values per FFT block (1024, 2048 or 4096), tri_stages the
+        rows staged ahead (2 or 4); 0 selects the defaults."""
         self.L = _lib.lib()
         self.subdomains = list(subdomains)
         self._c_subs = as_c_subdomains(self.subdomains)

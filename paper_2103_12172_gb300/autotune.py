@@ -5,16 +5,15 @@ _autotune_cache.json beside this module).
 
 Searched, by coordinate descent in this order (each step keeps the best of the previous ones):
   tile_cols         columns per work item (the batching tile);
-  fp64_cols         the gamma columns of the middle rows by FP64 sums instead of the tensor cores
-                    (only when some subdomain can take the tensor-core contraction);
-  direct_rows       the dense-row sine transforms by direct sums instead of the FFT (only when
-                    some subdomain has a power-of-two Nx);
+  fp64_cols         per-mode sweeps and FP64 sums instead of the separable solve on the tensor cores
+                    (only when some subdomain can take that);
+  direct_rows       in the sweeps, the dense-row sine transforms by direct sums instead of the FFT
+                    (only when some subdomain has a power-of-two Nx);
   fft_block_points  complex values per block of the dense-row FFT kernels (FFT rows only);
   tri_stages        table rows the per-mode sweep stages ahead in shared memory;
   workspace_bytes   not timed: the budget that packs work items into waves, as large as a quarter
                     of the free device memory allows up to 32 GiB (fewer, larger waves: fewer
-                    launch tails of the sweep; 224 -> 213 ms per step on the 8 x 8 workload from
-                    4 to 32 GiB), never below the 4 GiB default.
+                    launch tails), never below the 4 GiB default.
 Large workloads are timed on a sample: one subdomain of every (grid, AP, M*) class, all its
 columns; the per-item kernel choices carry over, the batching effects of the full workload less
 so (the bench reports the graph-replayed step beside the plain one for that)."""

@@ -126,7 +126,8 @@ __global__ void __launch_bounds__(256) k_adj_rows(Batch bt, const SubDesc *subs,
 
 // The cotangent at the 4 gamma columns (mlo-1, mlo, mhi, mhi+1) of the middle rows nlo+1 ..
 // nhi-1, gathered column-fastest into the r buffer ([4 (n - nlo - 1) + s][b], complex; r is free
-// between the forward recompute and k_adj_ring_rows) for the sine transform in k_adj_tri. On an
+// between the forward pass and the ring's adjoint field) for k_adj_tri's sine transform, or the separable
+// pass's operands (kernels_sepadj.cu). On an
 // x-symmetric subdomain (mhi + 1 = Nx - (mlo - 1), mhi = Nx - mlo, so sin(pi q m'/Nx) =
 // (-1)^(q+1) sin(pi q m/Nx) for the mirrored column m') the slots hold the pairs
 // (c0 + c3, c0 - c3, c1 + c2, c1 - c2), and a mode needs two of them.

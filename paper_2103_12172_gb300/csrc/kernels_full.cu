@@ -6,7 +6,8 @@
 //
 // Four kernels a pass: k_full_cut, k_full_gemm (forward), k_full_y, then cut and gemm again (inverse) and
 // k_full_out. They replaced direct O(N^2) sums on the FP64 pipe and one thread per mode sweeping an
-// uncoalesced column: 257^2, 32 right-hand sides 3.85 ms, 513^2, 4 right-hand sides 4.2 ms.
+// uncoalesced column: 257^2, 32 right-hand sides 3.85 ms -> 312 us; 513^2, 4 right-hand sides with the
+// potential's ring and correction 4.25 ms -> 250 us. k_full_y is half of it, FP64-bound.
 #include "sep_modes.cuh"
 
 #include <algorithm>

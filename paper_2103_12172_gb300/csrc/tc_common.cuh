@@ -1,4 +1,4 @@
-// tcgen05 / mbarrier helpers shared by the tensor-core kernels (kernels_tc.cu, kernels_sep.cu).
+// tcgen05 / mbarrier helpers of the contractions (digit_gemm.cuh).
 #pragma once
 #include "kernels_common.cuh"
 
