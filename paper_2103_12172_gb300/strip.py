@@ -399,9 +399,9 @@ class LayeredStrip:
             key = (str(device),) + tuple(complex(v) for v in vals)
             t = self._consts.get(key)
             if t is None:
-                if len(self._consts) >= 8:
-                    self._consts.clear()
-                t = self._consts[key] = torch.tensor(key[1:], dtype=torch.complex128).to(device)
+                t = torch.tensor(key[1:], dtype=torch.complex128).to(device)
+                if len(self._consts) < 16:
+                    self._consts[key] = t
             return t
         ts = [(v if isinstance(v, torch.Tensor) else torch.tensor(v)).to(torch.complex128) for v in vals]
         if len({t.device for t in ts}) > 1:
@@ -425,11 +425,11 @@ class LayeredStrip:
         st = self._structure(out.device)
         # boundary data of every outer side, analysed into Chebyshev coefficients in one product
         alphas = bcs = phi = None
-        if hasattr(self.bc, "sides") and st["outer"]:
+        if hasattr(self.bc, "sides_at_once") and st["outer"]:
             layer = st["layer"].get(str(k.device))
             if layer is None:
                 layer = st["layer"][str(k.device)] = torch.tensor([j for j, _ in st["outer"]]).to(k.device)
-            alphas, betas, phi = self.bc.sides(k.index_select(0, layer), [s for _, s in st["outer"]], *st["xy"])
+            alphas, betas, phi = self.bc.sides_at_once(k.index_select(0, layer), [s for _, s in st["outer"]], *st["xy"])
             if any(beta == 0 for beta in betas):
                 alphas, bcs = None, list(zip(alphas.unbind(0), betas))
         else:
@@ -545,25 +545,27 @@ class LayeredStrip:
 
 class incident_impedance_bc:
     """Outer data of config `strip4x1`: impedance sides du/dn + i k_j u = phi with phi from the
-    plane wave exp(i k_j (x cos theta + y sin theta)) of the layer's own wavenumber. sides() gives the data of
+    plane wave exp(i k_j (x cos theta + y sin theta)) of the layer's own wavenumber. sides_at_once() gives the data of
     many sides at once: their layers' wavenumbers [S], side numbers, points x, y [S, M] -> alpha [S],
     the numbers beta, phi [S, M]; LayeredStrip takes it where a boundary condition has it."""
 
     def __init__(self, theta):
         self.ct, self.sn = math.cos(theta), math.sin(theta)
         self.dirs = {1: -self.sn, 2: self.sn, 3: -self.ct, 4: self.ct}   # outward normal times direction
-        self._key = self._n = None
+        self._factors = {}
 
     def __call__(self, j, side, kj, x, y):
         ik = 1j * kj
         return ik, 1.0, torch.exp(ik * torch.add(x * self.ct, y, alpha=self.sn)) * (ik * (1.0 + self.dirs[side]))
 
-    def sides(self, ks, side, x, y):
+    def sides_at_once(self, ks, side, x, y):
         ik = 1j * ks.to(x.device)
         key = (tuple(side), x.dtype, x.device)
-        if key != self._key:   # the factors of these sides, on the device once
-            self._n, self._key = torch.tensor([1.0 + self.dirs[s] for s in side], dtype=x.dtype).to(x.device), key
-        n = self._n
+        n = self._factors.get(key)   # of these sides, on the device once
+        if n is None:
+            n = torch.tensor([1.0 + self.dirs[s] for s in side], dtype=x.dtype).to(x.device)
+            if len(self._factors) < 16:
+                self._factors[key] = n
         return ik, [1.0] * len(side), torch.exp(ik[:, None] * torch.add(x * self.ct, y, alpha=self.sn)) * (ik * n)[:, None]
 
 
