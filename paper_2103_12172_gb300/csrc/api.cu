@@ -226,7 +226,7 @@ cudaError_t end_use(mdp_plan *p, cudaStream_t st) {
   return cudaEventRecord(p->used_ev[p->set], st);
 }
 
-// The tables for new wavenumbers. The pivot chains (4 x 257^2: 213 us on some 80 warps) and the separable
+// The tables for new wavenumbers. The pivot chains (4 x 257^2: 200 us on some 80 warps) and the separable
 // tables (200 us of short kernels) do not depend on each other: the factorisation runs on the plan's side
 // stream, and the caller's waits for it.
 cudaError_t launch_update(mdp_plan *p, const SubDesc *ds, double *tab, uint8_t *piv, unsigned char *sep, int *status,

@@ -18,8 +18,8 @@
 //                   dependent FP64 operations (64 cycles each for a warp, whatever its lanes), so it
 //                   does nothing else, and its interior steps take real coefficients: 13
 //                   operations after a kept pivot, 18 after a swap, 6 for a swap. Propagating modes
-//                   swap every few rows, each at its own, so they have a warp each; 4 x 257^2: 471 us
-//                   with 32 neighbouring modes to a warp and general complex steps around swaps.
+//                   swap every few rows, each at its own, so they have a warp each; 4 x 257^2: 200 us,
+//                   471 with 32 neighbouring modes to a warp and general complex steps around swaps.
 //   k_factor_rows   everything row-local, one block per mode: u1 = du/d, u2 = du2/d, the
 //                   sweep rows (which also need row i+1's pivot, read through shared memory in
 //                   chunks so the rows can be rewritten in place), the dT/dk rows, and the runs
@@ -42,7 +42,8 @@ __device__ __forceinline__ bool czero(cplx a) { return a.re == 0.0 && a.im == 0.
 // operations instead of a full division on the factorisation's serial chains; x outside the
 // float range takes the division.
 __device__ __forceinline__ double rcp_pos(double x) {
-  if (!(x > 0x1p-120 && x < 0x1p120)) return 1.0 / x;
+  const int ex = __double2hiint(x) >> 20;   // sign and exponent: 2^-120 <= x < 2^120 (a compare takes the FP64 pipe)
+  if (ex < 1023 - 120 || ex >= 1023 + 120) return 1.0 / x;
   const double y0 = (double)__fdividef(1.0f, (float)x);
   const double e = fma(-x, y0, 1.0);
   return fma(y0, fma(e, e, e), y0);
@@ -147,7 +148,7 @@ __device__ __forceinline__ int mode_owner(const SubDesc *subs, int n_subs, int &
 // out(i, l, d, dinv, du, du2, sw) for every row in order. Interior steps (real a, dd entries) take
 // real coefficients. Returns false (status set) on a singular pivot.
 template <class Out>
-__device__ bool lu_chain(const ModeRows &M, int n, int mod, cplx sigma, double tol2, int *status, Out out) {
+__device__ bool lu_chain(const ModeRows &M, int n, int mod, cplx sigma, double tol2, int *status, bool settles, Out out) {
   const int N = M.N;
   auto ent = [&](int i, cplx &dl, cplx &dg, cplx &du) {
     M.entries(i, dl, dg, du);
@@ -163,22 +164,26 @@ __device__ bool lu_chain(const ModeRows &M, int n, int mod, cplx sigma, double t
   int i = 0;
   double r = 0.0;             // 1/|g|^2 of the previous kept pivot
   const double ia = crecip(cmk(a, 0.0)).re;
+  const long long a2_bits = __double_as_longlong(a2);
   while (i < n - 1) {
     // Interior steps: the pivot is kept while |g| >= a. Then |g|^2 >= a^2 > tol2 (a >= 1/(3h^2) is
     // within a factor 7 of max|T|), so no singularity test is needed. The pivots of a mode
     // settle to a fixed point, so 1/|g|^2 is refined from the previous row's: with
     // e = 1 - n2 r0, 1/n2 = r0 / (1 - e) = r0 (1 + e + e^2) + O(e^3 r0), full precision for
-    // |e| < 2^-20; otherwise a division.
+    // |e| < 2^-20; otherwise (and where they do not settle: propagating modes) a reciprocal.
     // The loop-carried chain is g -> |g|^2 -> 1/|g|^2 -> g' = dd - a u conj(g)/|g|^2 (u = a after a kept
     // pivot); the row's outputs branch off it. A swap takes row i+1 = (a, dd, a) as the pivot row.
     if (i > 0 || !M.cplx_ap)
       for (; i < fast_end; ++i) {
         const double n2 = fma(g.re, g.re, g.im * g.im);
-        if (n2 >= a2) {
-          const double e = fma(-n2, r, 1.0);
-          double rn = fma(r, fma(e, e, e), r);
-          if (!(fabs(e) < 0x1p-20)) rn = rcp_pos(n2);
-          r = rn;
+        if (__double_as_longlong(n2) >= a2_bits) {   // both positive: as integers (a NaN counts as kept)
+          if (settles) {
+            const double e = fma(-n2, r, 1.0);
+            const bool near = (__double2hiint(e) & 0x7fffffff) < 0x3eb00000;   // |e| < 2^-20
+            r = near ? fma(r, fma(e, e, e), r) : rcp_pos(n2);
+          } else {
+            r = rcp_pos(n2);
+          }
           const double gr = g.re * r, gi = g.im * r;   // 1/g = (gr, -gi)
           cplx gnext;
           if (u_is_a) gnext = cmk(fma(-a2, gr, dd), a2 * gi);
@@ -222,13 +227,13 @@ __device__ bool lu_chain(const ModeRows &M, int n, int mod, cplx sigma, double t
 }
 
 // Chain of the full LU: raw factor rows (l, 1/d, du, du2) and swap flags.
-__device__ void chain_full(const SubDesc &d, int q, double *tab, uint8_t *piv, int *status) {
+__device__ void chain_full(const SubDesc &d, int q, double *tab, uint8_t *piv, int *status, bool settles) {
   const ModeRows M = mode_rows(d, q);
   const int N = M.N, FW = d.cplx ? 8 : 4;
   const double tol2 = kSingularTolD * kSingularTolD * M.scale2();
   double *F = tab + d.fact_off + (long long)(q - 1) * N * FW;
   uint8_t *pv = piv + d.piv_off + (long long)(q - 1) * N;
-  lu_chain(M, N, -1, cmk(0.0, 0.0), tol2, status,
+  lu_chain(M, N, -1, cmk(0.0, 0.0), tol2, status, settles,
            [&](int i, cplx l, cplx, cplx dinv, cplx du, cplx du2, uint8_t sw) {
              if (FW == 8) {
                double *r = F + (long long)i * 8;
@@ -244,7 +249,7 @@ __device__ void chain_full(const SubDesc &d, int q, double *tab, uint8_t *piv, i
 // Chain of the condensed system (rows 0..itop, the rows above folded into the last pivot):
 // raw rows i >= i0 in the sweep table: l, d, 1/d, du, du2 (complex pairs) and the swap flag;
 // seg[4] = itop.
-__device__ void chain_sweep(const SubDesc &d, int q, double *tab, int *status) {
+__device__ void chain_sweep(const SubDesc &d, int q, double *tab, int *status, bool settles) {
   const ModeRows M = mode_rows(d, q);
   const int N = M.N;
   const double scale2 = M.scale2();
@@ -272,7 +277,7 @@ __device__ void chain_sweep(const SubDesc &d, int q, double *tab, int *status) {
   }
   tab[d.seg_off + 5 * (q - 1) + 4] = itop;
   double *T = tab + d.fs_off + (long long)(q - 1) * d.NYf * FSW;
-  lu_chain(M, itop + 1, itop, sigma, tol2, status,
+  lu_chain(M, itop + 1, itop, sigma, tol2, status, settles,
            [&](int i, cplx l, cplx dg, cplx dinv, cplx du, cplx du2, uint8_t sw) {
              if (i < d.i0) return;
              double *r = T + (long long)(i - d.i0) * FSW;
@@ -300,8 +305,8 @@ __global__ void __launch_bounds__(32) k_factor_chain(const SubDesc *subs, int n_
   if (si >= n_subs) return;
   const int q = prop ? t + 1 : subs[si].n_prop + t + 1;
   if (sweep) {
-    if (all || !subs[si].tc_cols) chain_sweep(subs[si], q, tab, status);
-  } else chain_full(subs[si], q, tab, piv, status);
+    if (all || !subs[si].tc_cols) chain_sweep(subs[si], q, tab, status, !prop);
+  } else chain_full(subs[si], q, tab, piv, status, !prop);
 }
 
 constexpr int kRowsThreads = 256;
