@@ -694,13 +694,14 @@ __global__ void __launch_bounds__(128) k_sep_modes(Batch bt, const SubDesc *subs
   MDP_CHECK_ITEM(bt, subs, it, local, F_SMODE);
   const SubDesc &d = subs[it.sub];
   const int cb = (it.ncols + 31) >> 5;
-  const int b = (local % cb) * 32 + threadIdx.x, q0 = (local / cb) * SEP_MODES_PER_BLOCK + threadIdx.y + 1;
+  const int per = sep_modes_per_block(d, it.ncols);
+  const int b = (local % cb) * 32 + threadIdx.x, q0 = (local / cb) * per + threadIdx.y + 1;
   if (b >= it.ncols) return;
   const SepGeo g = sep_geo(d);
   const SepWs w = sep_ws(d, it.ncols);
   const int row = CIN ? b : sep_row_of(d, it.col0, it.ncols, b);
   const int row1 = CIN ? b : row - sep_first34(d, it.col0, it.ncols);
-  for (int q = q0; q < q0 + SEP_MODES_PER_BLOCK - (int)threadIdx.y && q <= d.Nq; q += 4) {
+  for (int q = q0; q < q0 + per - (int)threadIdx.y && q <= d.Nq; q += 4) {
     if (d.cplx || CIN) sep_modes_body<true, CIN>(it, d, g, w, sep, ws, b, row, row1, q);
     else sep_modes_body<false, CIN>(it, d, g, w, sep, ws, b, row, row1, q);
   }

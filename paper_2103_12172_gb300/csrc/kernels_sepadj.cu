@@ -913,14 +913,15 @@ __global__ void __launch_bounds__(128) k_adj_modes(Batch bt, const SubDesc *subs
   MDP_CHECK_ITEM(bt, subs, it, local, F_AMODE);
   const SubDesc &d = subs[it.sub];
   const int cb = (it.ncols + 31) >> 5;
-  const int b = (local % cb) * 32 + threadIdx.x, q0 = (local / cb) * SEP_MODES_PER_BLOCK + threadIdx.y + 1;
+  const int per = sep_modes_per_block(d, it.ncols);
+  const int b = (local % cb) * 32 + threadIdx.x, q0 = (local / cb) * per + threadIdx.y + 1;
   double s = 0.0;
   if (b < it.ncols) {
     const SepGeo g = sep_geo(d);
     const SepWs sw = sep_ws(d, it.ncols);
     const AdjWs w = adj_ws(d, it.ncols);
     const int row1 = CIN ? b : sep_row_of(d, it.col0, it.ncols, b) - sep_first34(d, it.col0, it.ncols);
-    for (int q = q0; q < q0 + SEP_MODES_PER_BLOCK - (int)threadIdx.y && q <= d.Nq; q += 4)
+    for (int q = q0; q < q0 + per - (int)threadIdx.y && q <= d.Nq; q += 4)
       s += reinterpret_cast<const double *>(sep + d.sep_mt)[(long long)(q - 1) * SEP_MTW + MT_FAR] != 0.0
                ? adj_modes_body<CIN, DK, true>(it, d, g, sw, w, sep, adj, ws, has_rec && d.nrec >= 0, b, row1, q)
                : adj_modes_body<CIN, DK, false>(it, d, g, sw, w, sep, adj, ws, has_rec && d.nrec >= 0, b, row1, q);

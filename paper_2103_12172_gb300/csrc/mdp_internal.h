@@ -125,7 +125,6 @@ constexpr int SEP_MTW = 72;               // doubles per mode of the mode table
 constexpr int SEP_MXW = 20;               // doubles per mode of the full-grid solve's table
 constexpr int SEP_ABLK = 7 * 128 * 16 * 2;  // bytes of A: 7 digits x 128 rows x 16 values of K, fp16
 constexpr int SEP_BBLK = 7 * 32 * 16 * 2;   // bytes of B: 7 digits x 32 outputs x 16 values of K
-constexpr int SEP_MODES_PER_BLOCK = 16;   // k_sep_modes
 constexpr int SEP_MASK = 8;               // words of a K mask: at most 256 groups of 16
 
 // The contractions (jobs) of the projection: stage 1 runs MID (ring residuals of the middle rows
@@ -155,6 +154,11 @@ struct SepGeo {
 inline int propagating_modes(const SubDesc &d) {
   const double s = 0.5 * std::sqrt(d.k * d.k / (1.0 / (d.h * d.h) + d.k * d.k / 12.0));
   return s >= 1.0 ? d.Nq : std::min(d.Nq, (int)(2.0 * d.Nx / M_PI * std::asin(s)) + 1);
+}
+// modes per block (4 warps) of k_sep_modes and k_adj_modes: 16, or 4 where the item has fewer blocks of 16 than the
+// GPU has SMs (a block's modes follow one another: 129^2, 128 columns: k_sep_modes 14.8 -> 6.7 us)
+inline __host__ __device__ int sep_modes_per_block(const SubDesc &d, int ncols) {
+  return ((ncols + 31) / 32) * ((d.Nq + 15) / 16) < 152 ? 4 : 16;
 }
 inline __host__ __device__ SepGeo sep_geo(const SubDesc &d) {
   SepGeo g;
@@ -600,13 +604,16 @@ inline __host__ __device__ int blocks_for(int f, const SubDesc &d, int ncols, in
       if (f == F_AC1 || f == F_AC3) return adj_cut_blocks(d, a, j, ncols) + adj_cut_blocks(d, a, j + 1, ncols);
       return adj_tiles(d, a, j, ncols) + adj_tiles(d, a, j + 1, ncols);
     }
-    case F_AMODE: return d.tc_cols ? cb * ((d.Nq + SEP_MODES_PER_BLOCK - 1) / SEP_MODES_PER_BLOCK) : 0;
+    case F_SMODE: case F_AMODE: {
+      if (!d.tc_cols) return 0;
+      const int per = sep_modes_per_block(d, ncols);
+      return cb * ((d.Nq + per - 1) / per);
+    }
     case F_AOUT: {   // ring columns of the middle rows; dense ring rows; dK/dk against the cotangent
       if (!d.tc_cols) return 0;
       const SepGeo g = sep_geo(d);
       return cb * ((g.Pj + 7) / 8 + (4 * g.Kf + 7) / 8 + (g.Pi + 7) / 8);
     }
-    case F_SMODE: return d.tc_cols ? cb * ((d.Nq + SEP_MODES_PER_BLOCK - 1) / SEP_MODES_PER_BLOCK) : 0;
     case F_SOUT: {   // middle rows, 8 per block, then 32 folded columns of each row transformed back
       if (!d.tc_cols) return 0;
       const SepGeo g = sep_geo(d);
