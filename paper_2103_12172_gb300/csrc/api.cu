@@ -114,8 +114,7 @@ mdp_status alloc_device(mdp_plan *p) {
     CK(cudaMemcpy(p->d_sep + d.sep_ab, ab.data(), ab.size() * sizeof(double), cudaMemcpyHostToDevice));
   }
   CK(launch_sep_sines(p, p->d_subs, p->d_tables, p->d_sep, nullptr));
-  CK(launch_sep_tables(p, p->d_subs, p->d_tables, p->d_sep, false, nullptr));
-  CK(cudaStreamSynchronize(nullptr));
+  CK(launch_sep_tables(p, p->d_subs, p->d_tables, p->d_sep, false, nullptr));   // beside the host's work below
 #if MDP_CHECKED
   if (fault && !std::strcmp(fault, "factor") && !p->subs.empty() && p->subs[0].d.tc_cols) {
     double row[SEP_MTW];   // the same fault in the separable tables: the entries of mode 1
@@ -176,6 +175,7 @@ mdp_status alloc_device(mdp_plan *p) {
       hpre.push_back(pre);
     }
   }
+  CK(cudaStreamSynchronize(nullptr));
   return MDP_OK;
 }
 
