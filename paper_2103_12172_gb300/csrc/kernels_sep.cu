@@ -26,7 +26,7 @@
 // columns), which halves both dimensions: two classes with 2 columns each, else one with 4.
 //
 // Both contractions are to FP64 accuracy on the fp16 tensor cores (digit_gemm.cuh). 4 x 257^2, 1024 columns:
-// 215 us where the sweeps took 1393; 257^2 to 1025^2 x 8: 2.10 ms (41.3), of it k_sep_gemm 1.22, k_sep_cut 0.41,
+// 209 us where the sweeps took 1392; 257^2 to 1025^2 x 8: 2.09 ms (41.2), of it k_sep_gemm 1.22, k_sep_cut 0.41,
 // k_sep_out 0.19, k_sep_modes 0.14.
 // Against 64-bit sums over the closed form in extended precision (k = 10 on 129^2, k = 30 on
 // 257^2) the result is off by 1e-15 to 8e-15 (2-norm), plain FP64 sums by 4e-15 to 5e-14 and the

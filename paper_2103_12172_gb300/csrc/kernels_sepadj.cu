@@ -12,7 +12,7 @@
 // against d phi/dk (extra outputs of the stage 1 contractions) times the other side's coefficients; and
 // sum conj(c) (dK/dk r) on the middle rows, one more Toeplitz product of the residual. The recomputed field
 // of every mode and row and its adjoint, most of the pass by the recurrences, are gone: 4 x 257^2 with 1024
-// basis columns takes 630 us (4415 by the recurrences), 257^2 and 513^2 with user densities 680 us (4532).
+// basis columns takes 586 us (4418 by the recurrences), 257^2 and 513^2 with user densities 663 us (4536).
 // A first pass after a change of the wavenumbers makes the tables too, 400 us more.
 #include "sep_modes.cuh"
 

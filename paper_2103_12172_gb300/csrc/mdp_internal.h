@@ -687,7 +687,7 @@ enum { PASS_FWD = 0, PASS_GRAD = 1 };
 #ifdef __CUDACC__
 // Launch whose set-up overlaps the kernel before it on the stream (programmatic dependent launch): its blocks come
 // as that kernel's last ones leave, and every kernel launched so first waits in pdl_wait(), which returns when
-// the kernels before it are complete and their writes visible. Eight kernels of a pass of 129^2: 84.6 -> 66.4 us;
+// the kernels before it are complete and their writes visible. Eight kernels of a pass of 129^2: 84.6 -> 66.2 us;
 // 4 x 257^2: 231 -> 214 us. No earlier trigger: blocks that wait take the registers and shared memory of the
 // kernel before (279 us with one at each kernel's start).
 template <class... P, class... A>
