@@ -403,7 +403,8 @@ class LayeredStrip:
                 if len(self._consts) < 16:
                     self._consts[key] = t
             return t
-        ts = [(v if isinstance(v, torch.Tensor) else torch.tensor(v)).to(torch.complex128) for v in vals]
+        ts = [v.to(torch.complex128) if isinstance(v, torch.Tensor) else torch.tensor(complex(v), dtype=torch.complex128)
+              for v in vals]
         if len({t.device for t in ts}) > 1:
             ts = [t.to(device) for t in ts]
         return torch.stack(ts).to(device)

@@ -44,3 +44,15 @@ def test_least_squares_refuses_host_tensors():
     A = torch.randn(8, 3, dtype=torch.complex128)
     with pytest.raises(TypeError):
         LeastSquares.apply(A, torch.randn(8, dtype=torch.complex128))
+
+
+def test_boundary_coefficients_keep_their_64_bits():
+    """alpha and beta of the outer sides as numbers beside tensors, and as numbers alone: exactly the doubles
+    that the boundary condition returned (0.3 and 0.7 have no exact 32-bit form)."""
+    from paper_2103_12172_gb300.strip import LayeredStrip
+    lay = LayeredStrip.__new__(LayeredStrip)
+    lay._consts = {}
+    vals = [0.3, 0.7 + 0.1j, 2, torch.tensor(0.1, dtype=torch.float64), torch.tensor(0.2 - 0.6j, dtype=torch.complex128)]
+    want = [0.3, 0.7 + 0.1j, 2.0, 0.1, 0.2 - 0.6j]
+    assert lay._scalars(vals, torch.device("cpu")).tolist() == [complex(v) for v in want]
+    assert lay._scalars(vals[:3], torch.device("cpu")).tolist() == [complex(v) for v in want[:3]]
