@@ -394,7 +394,8 @@ class LayeredStrip:
         return self._st
 
     def _scalars(self, vals, device):
-        """The values as one complex tensor: numbers that are no tensors are put on the device once."""
+        """The values (numbers, tensors of one element) as one complex tensor: numbers that are no tensors are put
+        on the device once."""
         if not any(isinstance(v, torch.Tensor) for v in vals):
             key = (str(device),) + tuple(complex(v) for v in vals)
             t = self._consts.get(key)
@@ -403,8 +404,8 @@ class LayeredStrip:
                 if len(self._consts) < 16:
                     self._consts[key] = t
             return t
-        ts = [v.to(torch.complex128) if isinstance(v, torch.Tensor) else torch.tensor(complex(v), dtype=torch.complex128)
-              for v in vals]
+        ts = [v.reshape(()).to(torch.complex128) if isinstance(v, torch.Tensor)
+              else torch.tensor(complex(v), dtype=torch.complex128) for v in vals]
         if len({t.device for t in ts}) > 1:
             ts = [t.to(device) for t in ts]
         return torch.stack(ts).to(device)
@@ -453,7 +454,9 @@ class LayeredStrip:
         if cs is None:
             cs = st["systems"][kinds] = CoupledSystem(st, kinds, M, [lay[0] for lay in self.layout],
                                                       [lay[2] for lay in self.layout], out.device)
-        if not cs.ok:
+        # CoupledSolve takes one alpha and one beta per side; a side may also have one per coefficient
+        single = bcs is None or all(not isinstance(v, torch.Tensor) or v.dim() == 0 or v.shape == (1,) for ab in bcs for v in ab)
+        if not (cs.ok and single):
             bcs = list(zip(alphas.unbind(0), betas)) if bcs is None else bcs
             return torch.stack(self._dense_coefficients(out, bcs, d_all, st)), rec
         if not betas:
@@ -476,7 +479,8 @@ class LayeredStrip:
 
     def _dense_coefficients(self, out, bcs, d_all, st):
         """The coefficients by single tensor operations and LeastSquares, for systems CoupledSolve does not
-        take (a layer with fewer gamma nodes than unknowns, or triangles beyond a CTA's shared memory)."""
+        take (a layer with fewer gamma nodes than unknowns, triangles beyond a CTA's shared memory, or sides with an
+        alpha per coefficient)."""
         M, N, n = self.M, self.N, st["n"]
         A_rows, b_rows, coef = [], [], []
         q = 0

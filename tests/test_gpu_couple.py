@@ -47,3 +47,30 @@ def test_coupled_solve_and_gradient_are_those_of_the_dense_path(mdp, name, M):
         got.append((torch.cat(u).detach(), g, torch.cat([c for c in lay.coefficients(k.detach())[0]])))
     for a, b in zip(*got):
         assert (a - b).abs().max() < 1e-8 * b.abs().max()
+
+
+@pytest.mark.parametrize("form", ["one", "per_coefficient", "mixed"])
+def test_boundary_coefficients_of_one_element_and_per_coefficient(mdp, form):
+    """alpha (and the divisor of a Robin side) as a tensor of one element, alpha as one value per Chebyshev
+    coefficient: with equal values the solution and the gradient are those of the numbers."""
+    from paper_2103_12172_gb300.strip import LayeredStrip
+    pos, grids = LAYOUTS["strip3"]
+    M, ks = 5, [4.0, 4.7, 5.4]
+    subs = [W.unit_subdomain(i, jj, n, k, W.AP_DIRX_SOMMY, M) for (i, jj), n, k in zip(pos, grids, ks)]
+
+    def shaped(j, side, kj, x, y):
+        alpha, beta, phi = bc(j, side, kj, x, y)
+        alpha = torch.as_tensor(alpha, dtype=torch.complex128, device="cuda")
+        if form == "one" or (form == "mixed" and side == 2):
+            return alpha.reshape(1), beta if side in (1, 2) else beta.reshape(1), phi
+        return alpha.expand(M) if side != 2 or form == "per_coefficient" else alpha, beta, phi
+
+    got = []
+    for cond in (bc, shaped):
+        lay = LayeredStrip(subs, cond, [s.ny // 2 for s in subs], positions=pos)
+        k = torch.tensor(ks, dtype=torch.float64, device="cuda", requires_grad=True)
+        u = torch.cat(lay.receivers(k))
+        (g,) = torch.autograd.grad((u - 0.3j).abs().square().sum(), k)
+        got.append((u.detach(), g))
+    for a, b in zip(*got):
+        assert (a - b).abs().max() < 1e-8 * b.abs().max()
