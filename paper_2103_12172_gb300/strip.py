@@ -121,8 +121,9 @@ class BlockValues(torch.autograd.Function):
     def forward(ctx, B, v, blocks):
         v = v.contiguous()
         y = torch.empty(max(blocks.total, 1), dtype=torch.complex128, device=B.device)[:blocks.total]
-        _lib.check(_lib.lib().mdp_block_values(*blocks.args, _ptr(B), _ptr(v), _ptr(y), linalg._stream()),
-                   "mdp_block_values")
+        if blocks.total:
+            _lib.check(_lib.lib().mdp_block_values(*blocks.args, _ptr(B), _ptr(v), _ptr(y), linalg._stream()),
+                       "mdp_block_values")
         ctx.save_for_backward(B, v)
         ctx.blocks = blocks
         return y
@@ -130,6 +131,8 @@ class BlockValues(torch.autograd.Function):
     @staticmethod
     def backward(ctx, gy):
         B, v = ctx.saved_tensors
+        if not ctx.blocks.total:   # no receiver anywhere
+            return torch.zeros_like(B), torch.zeros_like(v), None
         gy = gy.resolve_conj().contiguous()
         gB = torch.empty_like(B) if ctx.needs_input_grad[0] else None
         gv = torch.empty_like(v) if ctx.needs_input_grad[1] else None

@@ -74,3 +74,15 @@ def test_boundary_coefficients_of_one_element_and_per_coefficient(mdp, form):
         got.append((u.detach(), g))
     for a, b in zip(*got):
         assert (a - b).abs().max() < 1e-8 * b.abs().max()
+
+
+def test_layout_without_receivers_gives_empty_values(mdp):
+    """No receiver row anywhere: every layer's values are empty, and so is their gradient (zero)."""
+    from paper_2103_12172_gb300.strip import LayeredStrip, incident_impedance_bc
+    subs = [W.unit_subdomain(j, 0, 33, 4.0 + j, W.AP_DIRX_SOMMY, 4) for j in range(2)]
+    lay = LayeredStrip(subs, incident_impedance_bc(0.3), [-1, -1])
+    k = torch.tensor([4.0, 5.0], dtype=torch.float64, device="cuda", requires_grad=True)
+    u = lay.receivers(k)
+    assert [v.numel() for v in u] == [0, 0]
+    (g,) = torch.autograd.grad(sum(v.abs().sum() for v in u), k)
+    assert torch.equal(g, torch.zeros_like(g))
