@@ -258,6 +258,17 @@ def cheb_points(n, device):
     return torch.cos(math.pi * (i + 0.5) / n)
 
 
+def _sides_at_once(bc):
+    """bc.sides_at_once where it stands for bc itself: defined with or below the class's __call__ (a subclass
+    that overrides __call__ alone is asked side by side)."""
+    for c in type(bc).__mro__:
+        if "sides_at_once" in vars(c):
+            break
+        if "__call__" in vars(c):
+            return None
+    return getattr(bc, "sides_at_once", None)
+
+
 class LayeredStrip:
     """A rectangular layout of square subdomains that share whole sides (default: a strip
     along x; `positions[j]` = cell (i, j) of subdomain j otherwise, Section 3.4) with outer
@@ -430,11 +441,12 @@ class LayeredStrip:
         st = self._structure(out.device)
         # boundary data of every outer side, analysed into Chebyshev coefficients in one product
         alphas = bcs = phi = None
-        if hasattr(self.bc, "sides_at_once") and st["outer"]:
+        at_once = _sides_at_once(self.bc)
+        if at_once is not None and st["outer"]:
             layer = st["layer"].get(str(k.device))
             if layer is None:
                 layer = st["layer"][str(k.device)] = torch.tensor([j for j, _ in st["outer"]]).to(k.device)
-            alphas, betas, phi = self.bc.sides_at_once(k.index_select(0, layer), [s for _, s in st["outer"]], *st["xy"])
+            alphas, betas, phi = at_once(k.index_select(0, layer), [s for _, s in st["outer"]], *st["xy"])
             if any(beta == 0 for beta in betas):
                 alphas, bcs = None, list(zip(alphas.unbind(0), betas))
         else:

@@ -56,3 +56,23 @@ def test_boundary_coefficients_keep_their_64_bits():
     want = [0.3, 0.7 + 0.1j, 2.0, 0.1, 0.2 - 0.6j]
     assert lay._scalars(vals, torch.device("cpu")).tolist() == [complex(v) for v in want]
     assert lay._scalars(vals[:3], torch.device("cpu")).tolist() == [complex(v) for v in want[:3]]
+
+
+def test_a_subclass_that_overrides_the_call_alone_is_asked_side_by_side():
+    from paper_2103_12172_gb300.strip import _sides_at_once, incident_impedance_bc
+
+    class Call(incident_impedance_bc):
+        def __call__(self, j, side, kj, x, y):
+            return 2.0, 1.0, x
+
+    class Both(Call):
+        def sides_at_once(self, ks, side, x, y):
+            return ks, [1.0] * len(side), x
+
+    class Deeper(Both):
+        pass
+
+    assert _sides_at_once(Call(0.3)) is None and _sides_at_once(lambda j, side, kj, x, y: (1.0, 1.0, x)) is None
+    for cls in (incident_impedance_bc, Both, Deeper):
+        bc = cls(0.3)
+        assert _sides_at_once(bc) == bc.sides_at_once
