@@ -580,10 +580,11 @@ class incident_impedance_bc:
 
     def sides_at_once(self, ks, side, x, y):
         ik = 1j * ks.to(x.device)
-        key = (tuple(side), x.dtype, x.device)
-        n = self._factors.get(key)   # of these sides, on the device once
+        dirs = tuple(self.dirs[s] for s in side)
+        key = (dirs, x.dtype, x.device)
+        n = self._factors.get(key)   # of these directions, on the device once
         if n is None:
-            n = torch.tensor([1.0 + self.dirs[s] for s in side], dtype=x.dtype).to(x.device)
+            n = torch.tensor([1.0 + v for v in dirs], dtype=x.dtype).to(x.device)
             if len(self._factors) < 16:
                 self._factors[key] = n
         return ik, [1.0] * len(side), torch.exp(ik[:, None] * torch.add(x * self.ct, y, alpha=self.sn)) * (ik * n)[:, None]

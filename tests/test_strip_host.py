@@ -76,3 +76,14 @@ def test_a_subclass_that_overrides_the_call_alone_is_asked_side_by_side():
     for cls in (incident_impedance_bc, Both, Deeper):
         bc = cls(0.3)
         assert _sides_at_once(bc) == bc.sides_at_once
+
+
+def test_sides_at_once_follow_a_change_of_direction():
+    from paper_2103_12172_gb300.strip import incident_impedance_bc
+    bc, other = incident_impedance_bc(0.3), incident_impedance_bc(1.1)
+    ks, x, y = torch.tensor([4.0, 5.0], dtype=torch.float64), torch.rand(2, 3).double(), torch.rand(2, 3).double()
+    for _ in range(2):
+        _, _, phi = bc.sides_at_once(ks, [1, 4], x, y)
+        for i, side in enumerate((1, 4)):
+            assert torch.allclose(phi[i], bc(0, side, ks[i], x[i], y[i])[2], rtol=1e-14, atol=0)
+        bc.ct, bc.sn, bc.dirs = other.ct, other.sn, other.dirs
