@@ -576,7 +576,7 @@ class incident_impedance_bc:
 
     def __call__(self, j, side, kj, x, y):
         ik = 1j * kj
-        return ik, 1.0, torch.exp(ik * torch.add(x * self.ct, y, alpha=self.sn)) * (ik * (1.0 + self.dirs[side]))
+        return ik, 1.0, torch.exp(ik * (x * self.ct + y * self.sn)) * (ik * (1.0 + self.dirs[side]))
 
     def sides_at_once(self, ks, side, x, y):
         ik = 1j * ks.to(x.device)

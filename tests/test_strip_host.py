@@ -87,3 +87,11 @@ def test_sides_at_once_follow_a_change_of_direction():
         for i, side in enumerate((1, 4)):
             assert torch.allclose(phi[i], bc(0, side, ks[i], x[i], y[i])[2], rtol=1e-14, atol=0)
         bc.ct, bc.sn, bc.dirs = other.ct, other.sn, other.dirs
+
+
+def test_incident_data_at_a_point_given_by_numbers():
+    """x, y as numbers with a tensor wavenumber: as at a point given by tensors."""
+    from paper_2103_12172_gb300.strip import incident_impedance_bc
+    bc, k = incident_impedance_bc(0.3), torch.tensor(5.0, dtype=torch.float64)
+    t = torch.tensor([0.25, 0.75], dtype=torch.float64)
+    assert torch.allclose(bc(0, 2, k, 0.25, 0.75)[2], bc(0, 2, k, t[0], t[1])[2], rtol=1e-14, atol=0)
