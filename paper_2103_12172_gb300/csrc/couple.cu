@@ -237,6 +237,7 @@ template <bool GRAM>
 __global__ void __launch_bounds__(kTrThreads) k_cp_shared(Cp p, const double2 *S, const double *D, const double2 *gx,
                                                           const double2 *part, double2 *ys, double2 *x) {
   pdl_wait();
+  __shared__ TrBlock T;
   extern __shared__ __align__(16) double2 xs[];
   for (int c = threadIdx.x; c < p.ns; c += kTrThreads) {
     if (!GRAM) { xs[c] = S[(long long)p.ns * p.ms + c]; continue; }
@@ -250,8 +251,8 @@ __global__ void __launch_bounds__(kTrThreads) k_cp_shared(Cp p, const double2 *S
     }
     xs[c] = v;
   }
-  if (GRAM) trsv_body<true>(p.ns, S, p.ms, xs);
-  trsv_body<false>(p.ns, S, p.ms, xs);
+  if (GRAM) trsv_body<true>(p.ns, S, p.ms, xs, T);
+  trsv_body<false>(p.ns, S, p.ms, xs, T);
   for (int c = threadIdx.x; c < p.ns; c += kTrThreads) {
     const double s = D[p.shu[c]];
     ys[c] = xs[c];
@@ -263,6 +264,7 @@ __global__ void __launch_bounds__(kTrThreads) k_cp_shared(Cp p, const double2 *S
 __global__ void __launch_bounds__(kTrThreads) k_cp_private(Cp p, const double2 *Mx, const double *D, const double2 *ys,
                                                            const double2 *yp, double2 *x) {
   pdl_wait();
+  __shared__ TrBlock T;
   extern __shared__ __align__(16) double2 xs[];   // [pj], then [8][pj] partial sums
   const int j = blockIdx.x, pj = p.pj[j], sj = p.nj[j] - pj, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const double2 *Mj = Mx + (long long)j * (p.nmax + 1) * p.mmax;
@@ -280,7 +282,7 @@ __global__ void __launch_bounds__(kTrThreads) k_cp_private(Cp p, const double2 *
     for (int w = 0; w < 8; ++w) { v.x -= ps[w * pj + i].x; v.y -= ps[w * pj + i].y; }
     xs[i] = v;
   }
-  trsv_body<false>(pj, Mj, p.mmax, xs);
+  trsv_body<false>(pj, Mj, p.mmax, xs, T);
   for (int i = threadIdx.x; i < pj; i += kTrThreads) {
     const int u = p.unk[(long long)j * p.nmax + i];
     x[u] = make_double2(D[u] * xs[i].x, D[u] * xs[i].y);
@@ -290,12 +292,13 @@ __global__ void __launch_bounds__(kTrThreads) k_cp_private(Cp p, const double2 *
 // yp = R_pp^{-H} gx_p and the subdomain's part R_ps^H yp of the shared right-hand side
 __global__ void __launch_bounds__(kTrThreads) k_cp_private_h(Cp p, const double2 *Mx, const double2 *gx, double2 *yp, double2 *part) {
   pdl_wait();
+  __shared__ TrBlock T;
   extern __shared__ __align__(16) double2 xs[];
   const int j = blockIdx.x, pj = p.pj[j], lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const double2 *Mj = Mx + (long long)j * (p.nmax + 1) * p.mmax;
   const long long jp = (long long)j * p.nmax;
   for (int i = threadIdx.x; i < pj; i += kTrThreads) xs[i] = gx[p.unk[jp + i]];
-  trsv_body<true>(pj, Mj, p.mmax, xs);
+  trsv_body<true>(pj, Mj, p.mmax, xs, T);
   for (int i = threadIdx.x; i < pj; i += kTrThreads) yp[jp + i] = xs[i];
   for (int c = pj + warp; c < p.nj[j]; c += 8) {
     double2 s = zero2();
@@ -389,6 +392,7 @@ bool valid(const mdp_couple *c) {
          c->max_cols < 65535 && c->n_outer >= 0 && c->rows >= 1 && c->tables && c->offsets && 8 * c->n_modes <= 65535 &&
          c->n_shared < 65535 && (size_t)c->n_shared * 16 <= 200 * 1024 && (size_t)c->max_cols * 9 * 16 <= 200 * 1024;
 }
+// dynamic shared memory beside the static 16.5 KiB of trsv_body; valid() keeps the sum below 217 KiB
 template <class K>
 bool smem_ok(K *k, size_t bytes) {
   return bytes <= 24 * 1024 || cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess;

@@ -481,10 +481,11 @@ __global__ void __launch_bounds__(kQrThreads) k_qr_cta(QrArgs q) {
 template <bool CT>
 __global__ void __launch_bounds__(kTrThreads) k_trsv(int n, const double2 *__restrict__ R, long long ldr,
                                                      double2 *B, long long ldb) {
+  __shared__ TrBlock T;
   extern __shared__ __align__(16) double2 xs[];
   double2 *bcol = B + (long long)blockIdx.x * ldb;
   for (int i = threadIdx.x; i < n; i += kTrThreads) xs[i] = bcol[i];
-  trsv_body<CT>(n, R, ldr, xs);
+  trsv_body<CT>(n, R, ldr, xs, T);
   for (int i = threadIdx.x; i < n; i += kTrThreads) bcol[i] = xs[i];
 }
 

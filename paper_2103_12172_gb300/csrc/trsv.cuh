@@ -24,9 +24,11 @@ __device__ __forceinline__ double2 crcp(double2 d) {   // 1 / d
 
 // xs: the n values in shared memory, written by the CTA's threads before a barrier-free call; replaced by
 // the solution (visible to every thread on return). Only rows <= columns of R are read.
+// T: shared memory for the diagonal block, T[col][row] = R(i0 + row, i0 + col); the caller's, as a kernel that
+// solves with R and R^H would hold two where the block is static here, past what a launch gets without opting in.
+typedef double2 TrBlock[32][33];
 template <bool CT>
-__device__ __forceinline__ void trsv_body(int n, const double2 *__restrict__ R, long long ldr, double2 *xs) {
-  __shared__ double2 T[32][33];   // the diagonal block: T[col][row] = R(i0 + row, i0 + col)
+__device__ __forceinline__ void trsv_body(int n, const double2 *__restrict__ R, long long ldr, double2 *xs, TrBlock &T) {
   const int nblk = (n + 31) / 32, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int t = 0; t < nblk; ++t) {
     const int bi = CT ? t : nblk - 1 - t;

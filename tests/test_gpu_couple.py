@@ -86,3 +86,26 @@ def test_layout_without_receivers_gives_empty_values(mdp):
     assert [v.numel() for v in u] == [0, 0]
     (g,) = torch.autograd.grad(sum(v.abs().sum() for v in u), k)
     assert torch.equal(g, torch.zeros_like(g))
+
+
+def test_gradient_of_a_layout_with_1120_shared_unknowns(mdp):
+    """8 x 8 subdomains, 10 unknowns per interface: the triangle of the shared unknowns and the vector take more
+    shared memory than a kernel has without opting in. The dense path's values, 1e-8 (as above)."""
+    from paper_2103_12172_gb300.strip import LayeredStrip, incident_impedance_bc
+    pos = [(i, j) for j in range(8) for i in range(8)]
+    ks = [4.0 + 0.02 * j for j in range(64)]
+    subs = [W.unit_subdomain(i, jj, 33, k, W.AP_DIRX_SOMMY, 5) for (i, jj), k in zip(pos, ks)]
+    got = []
+    for dense in (False, True):
+        lay = LayeredStrip(subs, incident_impedance_bc(0.3), [16] * 64, positions=pos)
+        k = torch.tensor(ks, dtype=torch.float64, device="cuda", requires_grad=True)
+        if dense:
+            lay.receivers(k.detach())
+            for cs in lay._st["systems"].values():
+                assert cs.ok and cs.c.n_shared == 1120
+                cs.ok = False
+        u = torch.cat(lay.receivers(k))
+        (g,) = torch.autograd.grad((u - 0.3j).abs().square().sum(), k)
+        got.append((u.detach(), g))
+    for a, b in zip(*got):
+        assert (a - b).abs().max() < 1e-8 * b.abs().max()
