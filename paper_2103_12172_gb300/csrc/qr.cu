@@ -616,12 +616,12 @@ extern "C" mdp_status mdp_triangular_solve(int n, int nrhs, const mdp_c64 *R, lo
   const double2 *r = reinterpret_cast<const double2 *>(R);
   double2 *b = reinterpret_cast<double2 *>(B);
   if (conj_trans) {
-    if (smem > 48 * 1024 &&
+    if (smem > 24 * 1024 &&   // beside the static block, more than a launch gets without opting in
         cudaFuncSetAttribute(mdp::k_trsv<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
       return MDP_ERR_CUDA;
     mdp::k_trsv<true><<<nrhs, mdp::kTrThreads, smem, st>>>(n, r, ldr, b, ldb);
   } else {
-    if (smem > 48 * 1024 &&
+    if (smem > 24 * 1024 &&
         cudaFuncSetAttribute(mdp::k_trsv<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
       return MDP_ERR_CUDA;
     mdp::k_trsv<false><<<nrhs, mdp::kTrThreads, smem, st>>>(n, r, ldr, b, ldb);

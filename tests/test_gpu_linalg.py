@@ -133,6 +133,20 @@ def test_triangular_solve_matches_numpy(mdp, n, nrhs, conj_trans):
     assert np.array_equal(xv.cpu().numpy(), X[:, 0])
 
 
+@pytest.mark.parametrize("n", [1536, 1537, 2100, 3072])
+@pytest.mark.parametrize("conj_trans", [False, True])
+def test_triangular_solve_beside_its_static_shared_memory(mdp, n, conj_trans):
+    """Sizes whose vector and diagonal block together pass 48 KiB, at the steps of the launch's limits. Bar: the
+    backward error of substitution, n units of rounding."""
+    from paper_2103_12172_gb300.linalg import triangular_solve
+    rng = np.random.default_rng(n)
+    R = np.triu(_rand(rng, n, n)) / np.sqrt(n) + 4.0 * np.eye(n)
+    b = _rand(rng, n)
+    x = triangular_solve(torch.from_numpy(R.T.copy()).cuda(), n, n, torch.from_numpy(b).cuda(), conj_trans).cpu().numpy()
+    Rop = R.conj().T if conj_trans else R
+    assert np.abs(Rop @ x - b).max() <= 1.2e-16 * n * (np.abs(Rop) @ np.abs(x)).max()
+
+
 def test_complex_matmul_strides_conjugation_and_empty_shapes(mdp):
     """mdp_complex_matmul against numpy: plain, transposed and conjugated views (the lazily
     conjugated torch view too), a matrix-vector product, ragged tiles, k = 0 and m = 0."""
