@@ -57,17 +57,25 @@ __device__ __forceinline__ long long fixed_of(double x, int E) {
 // values of K, except that with nkj the B block of group kb is a Toeplitz one (nkj groups per source
 // column, ND blocks per column, output group ti); the mask of groups with nonzero digits; the exponents of the rows and of the table.
 struct DigitTile {
-  const unsigned char *A, *B;
+  const unsigned char *A, *B, *B2 = nullptr;
+  int k2 = 1 << 30;          // groups of K from k2 on have their B blocks at B2
   int nkj, ND, ti;
   unsigned m[SEP_MASK];      // groups of K with nonzero digits in the tile's rows and in its outputs
   const int *ex;
   int eb;
-  __device__ __forceinline__ void masks(const unsigned *ma, const unsigned *mb) {   // mb may be null
+  // mb, mb2 may be null
+  __device__ __forceinline__ void masks(const unsigned *ma, const unsigned *mb, const unsigned *mb2 = nullptr) {
     const uint4 *p = reinterpret_cast<const uint4 *>(ma);
     uint4 a = p[0], b = p[1];
     if (mb) {
       const uint4 *r = reinterpret_cast<const uint4 *>(mb);
-      const uint4 c = r[0], e = r[1];
+      uint4 c = r[0], e = r[1];
+      if (mb2) {             // of the groups from k2 on
+        const uint4 *s = reinterpret_cast<const uint4 *>(mb2);
+        const uint4 c2 = s[0], e2 = s[1];
+        c.x |= c2.x; c.y |= c2.y; c.z |= c2.z; c.w |= c2.w;
+        e.x |= e2.x; e.y |= e2.y; e.z |= e2.z; e.w |= e2.w;
+      }
       a.x &= c.x; a.y &= c.y; a.z &= c.z; a.w &= c.w;
       b.x &= e.x; b.y &= e.y; b.z &= e.z; b.w &= e.w;
     }
@@ -189,7 +197,8 @@ __device__ __forceinline__ void digit_gemm(const Src &src, int *status) {
             asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(SG_STAGE_BYTES) : "memory");
             bulk_load(sbase + st * SEP_ABLK, t.A + (long long)kb * SEP_ABLK, SEP_ABLK, bar);
             const long long bo = t.nkj ? (long long)(kb / t.nkj) * t.ND + 2 * t.ti - kb % t.nkj + t.nkj - 1 : kb;
-            bulk_load(sbase + SG_B0 + (2 * st + 1) * SEP_BBLK, t.B + bo * SEP_BBLK, SEP_BBLK, bar);
+            bulk_load(sbase + SG_B0 + (2 * st + 1) * SEP_BBLK, kb < t.k2 ? t.B + bo * SEP_BBLK : t.B2 + (kb - t.k2) * SEP_BBLK,
+                      SEP_BBLK, bar);
           }
         if (!ok) break;
       }

@@ -101,10 +101,10 @@ enum {
   MT_P2G = 48,
   MT_R = 52,     // R11, R12, R22 (complex)
   MT_IMAG = 58,  // 1: R's imaginary part counts (above 2^-62 of kappa's scale)
-  MT_REC = 59,   // receiver row: phi_1, phi_2, 1 / (scale of its moment table)
+  MT_RFI = 61,   // 1 / MT_RF
   MT_T1 = 62,    // kappa(d) = T1 phi_1(J0 + d) + T2 phi_2(J0 + d)
   MT_T2 = 63,
-  MT_RF = 64,    // scale of the receiver's moment table (a power of two)
+  MT_RF = 64,    // scale of a receiver row's moment table (a power of two)
   MT_TH = 65,    // theta, kind, sign, normalisations of phi_1, phi_2 (for k_sep_phi)
   MT_KIND = 66,
   MT_SG = 67,

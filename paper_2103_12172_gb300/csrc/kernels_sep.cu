@@ -154,11 +154,7 @@ __global__ void __launch_bounds__(32) k_sep_mode_tab(const SubDesc *subs, int s0
   T[MT_R + 4] = R22.re; T[MT_R + 5] = R22.im;
   T[MT_IMAG] = imag ? 1.0 : 0.0;
   T[MT_FAR] = kind == 2 && lo2[0] < 0x1p-90 ? 1.0 : 0.0;   // 2^-90 of the other end is zero to working precision
-  if (d.nrec >= 0) {
-    T[MT_REC + 0] = sgn(d.nrec - J0) * (kind == 2 ? exp(-th * (d.nrec - J0)) : n1 * sep_c(kind, th, d.nrec - mid));
-    T[MT_REC + 1] = sgn(d.nrec - J0) * (kind == 2 ? exp(-th * (J1 - d.nrec)) : n2 * sep_s(kind, th, d.nrec - mid));
-  }
-  T[MT_REC + 2] = 1.0 / rf;
+  T[MT_RFI] = 1.0 / rf;
   T[MT_T1] = T1;
   T[MT_T2] = T2;
   T[MT_RF] = rf;
@@ -303,18 +299,21 @@ __global__ void __launch_bounds__(256) k_sep_tb(const SubDesc *subs, int s0, uns
 }
 
 // The moment tables, B of stage 1 beyond K: output (b, q), K index (c, j): sin(pi q m_c/Nx) phi_b(j),
-// and (b = 2, with a receiver row) sin(pi q m_c/Nx) kappa_q(|rec - j|) scaled to below 1.
+// and (b = 2, with a receiver row) sin(pi q m_c/Nx) kappa_q(|rec - j|) scaled to below 1: subdomains that
+// share their leader's tables may each have a row of their own, so b = 2 is made and kept per subdomain.
 __global__ void __launch_bounds__(256) k_sep_mb(const SubDesc *subs, int s0, const double *tab, unsigned char *sep) {
   const int si = s0 + blockIdx.z;
   const SubDesc &d = subs[si];
-  if (!d.tc_cols || d.leader != si) return;
+  if (!d.tc_cols) return;
   const SepGeo g = sep_geo(d);
   const int nto = g.nb * g.nqp / 32;
   const int e = blockIdx.y / nto, to = blockIdx.y % nto;
   const int kb = blockIdx.x * 4 + (threadIdx.x >> 6);
   if (e >= g.ncls || kb >= g.nk1) return;
   const int o = threadIdx.x & 31, half = (threadIdx.x >> 5) & 1;
-  const int b = to * 32 / g.nqp, qi = to * 32 % g.nqp + o, q = sep_mode(d, e, qi);
+  const int b = to * 32 / g.nqp;
+  if (b < 2 && d.leader != si) return;
+  const int qi = to * 32 % g.nqp + o, q = sep_mode(d, e, qi);
   const int c = kb / g.nkj, j0 = (kb % g.nkj) * 16 + 8 * half;
   long long V[8];
 #pragma unroll
@@ -337,8 +336,9 @@ __global__ void __launch_bounds__(256) k_sep_mb(const SubDesc *subs, int s0, con
       V[j] = fix54(v * sc);
     }
   }
-  mark_group(reinterpret_cast<unsigned *>(sep + d.sep_zm) + (e * (3 * g.nqp / 32) + to) * SEP_MASK, kb, V);
-  unsigned char *B = sep + d.sep_mb + (((long long)e * (3 * g.nqp / 32) + to) * g.nk1 + kb) * SEP_BBLK;
+  const SepMoment m = sep_moment(d, g, e, to);
+  mark_group(reinterpret_cast<unsigned *>(sep + m.mask), kb, V);
+  unsigned char *B = sep + m.blocks + (long long)kb * SEP_BBLK;
   store_digits(B + (o >> 3) * 256 + half * 128 + (o & 7) * 16, 1024, V);
 }
 
@@ -555,9 +555,9 @@ struct SepSrc {
       t.nkj = g.nkj; t.ND = g.ND; t.ti = t.nt % g.nti;
       t.eb = reinterpret_cast<const int *>(sep + d.sep_kde)[es];
     } else {                     // moments
-      const int mt = t.e * (3 * g.nqp / 32) + t.nt - g.nt3;
-      t.B = sep + d.sep_mb + (long long)mt * nk * SEP_BBLK;
-      mb = reinterpret_cast<const unsigned *>(sep + d.sep_zm) + mt * SEP_MASK;
+      const SepMoment m = sep_moment(d, g, t.e, t.nt - g.nt3);
+      t.B = sep + m.blocks;
+      mb = reinterpret_cast<const unsigned *>(sep + m.mask);
     }
     t.masks(ma, mb);
     return true;
@@ -678,7 +678,8 @@ __device__ __forceinline__ void sep_modes_body(const Item &it, const SubDesc &d,
 #pragma unroll
   for (int r = 0; r < 4; ++r) ystore(r, out[0][2 + r], CD ? out[1][2 + r] : 0.0);
   if (rec) {
-    const double p1 = T[MT_REC], p2 = T[MT_REC + 1], f = T[MT_REC + 2];
+    const double *phi = reinterpret_cast<const double *>(sep + d.sep_phi) + (long long)(d.nrec - d.nlo + 1) * d.Nq + q - 1;
+    const double p1 = phi[0], p2 = phi[(long long)(d.Py + 2) * d.Nq], f = T[MT_RFI];
     const double re = fma(p1, out[0][0], fma(p2, out[0][1], f * m3[0]));
     double im = 0.0;
     if (CD) im = fma(p1, out[1][0], fma(p2, out[1][1], CIN ? f * m3[P - 1] : 0.0));
@@ -826,6 +827,11 @@ cudaError_t launch_sep_tables(const mdp_plan *p, const SubDesc *ds, const double
   int mq = 0, mrow = 0, mdist = 0, mtb = 0, mes = 0, mmb = 0, mmk = 0, m3 = 0, m3k = 0;
   for (size_t i = 0; i < p->subs.size(); ++i) {
     const SubDesc &d = p->subs[i].d;
+    if (d.tc_cols && (d.leader == (int)i || d.nrec >= 0)) {   // a duplicate has its receiver row's moments
+      const SepGeo g = sep_geo(d);
+      mmb = std::max(mmb, g.ncls * g.nb * g.nqp / 32);
+      mmk = std::max(mmk, (g.nk1 + 3) / 4);
+    }
     if (d.leader != (int)i) continue;
     mq = std::max(mq, (d.Nq + 127) / 128);
     mrow = std::max(mrow, (d.Py + 2 + PHI_ROWS - 1) / PHI_ROWS);
@@ -834,8 +840,6 @@ cudaError_t launch_sep_tables(const mdp_plan *p, const SubDesc *ds, const double
     mdist = std::max(mdist, d.Py);
     mtb = std::max(mtb, (g.ND + 3) / 4);
     mes = std::max(mes, g.ncls * g.nS * g.nS);
-    mmb = std::max(mmb, g.ncls * g.nb * g.nqp / 32);
-    mmk = std::max(mmk, (g.nk1 + 3) / 4);
     m3 = std::max(m3, g.ncls * g.nt3);
     m3k = std::max(m3k, (g.nk3 + 3) / 4);
   }

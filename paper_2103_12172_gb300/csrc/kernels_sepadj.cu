@@ -55,8 +55,7 @@ enum {
   MD_T2 = 56,
   MD_RHO1 = 57,   // scales (powers of two) of d phi/dk in the moment tables
   MD_RHO2 = 58,
-  MD_RFD = 59,    // scale of d kappa/dk at the receiver's
-  MD_REC = 60,    // d phi_1, d phi_2 at the receiver row
+  MD_RFD = 59,    // scale of d kappa/dk in a receiver row's moment table
   MD_TC = 62,     // d theta/dk (kind 2), d cosh theta or cos theta / dk (kinds 0, 1)
   MD_COS = 63,    // cos or cosh theta, -4 t (1 - t) = cos^2 - 1, t
   MD_SS = 64,
@@ -110,10 +109,9 @@ __global__ void __launch_bounds__(32) k_adj_mode_tab(const SubDesc *subs, int s0
     al0 = {alpha, 0.5 * beta};
     al1 = {(-sg) * alpha, (0.5 * sg) * beta};
   }
-  Du lo1[3], lo2[3], hi1[3], hi2[3], kv[6], T1, T2 = du(0.0), el[3] = {du(0.0), du(0.0), du(0.0)}, r1 = du(0.0), r2 = du(0.0);
+  Du lo1[3], lo2[3], hi1[3], hi2[3], kv[6], T1, T2 = du(0.0), el[3] = {du(0.0), du(0.0), du(0.0)};
   Dc R11, R12, R22;
   double rho1, rho2, kb;
-  const int rec = d.nrec >= 0 ? d.nrec : J0;
   if (kind < 2) {
     const Du i2a = du(1.0) / (2.0 * a);
     // C and S at x, derivatives through c: dC/dc = x S
@@ -156,9 +154,6 @@ __global__ void __launch_bounds__(32) k_adj_mode_tab(const SubDesc *subs, int s0
     for (int j = 3; j < 6; ++j) { cs(L - 4 + j, C, S); kv[j] = S * i2a; }
     T1 = (1.0 / n1) * (Se * i2a);
     T2 = (1.0 / n2) * (Ce * i2a);
-    cs(rec - mid, C, S);
-    r1 = n1 * C;
-    r2 = n2 * S;
     // bounds of d phi/dk and d kappa/dk over the rows: |S| <= min(x, 1/sin theta) (its own value, growing, next to
     // the cutoff), |dC/dc| = x |S|, |dS/dc| <= max(1, x^2) times the bound of S
     const double x2 = fmax(1.0, Lh * Lh), sm = kind == 0 ? fmin(fmax(Lh, 1.0), fabs(isth)) : fmax(fabs(Se.v), 1.0);
@@ -184,8 +179,6 @@ __global__ void __launch_bounds__(32) k_adj_mode_tab(const SubDesc *subs, int s0
     kv[0] = c0; kv[1] = c0 * em; kv[2] = c0 * e2; kv[3] = c0 * fl; kv[4] = c0 * fl * em; kv[5] = c0 * fl * e2;
     el[0] = c0; el[1] = c0 * ep; el[2] = c0 * ep * ep;
     T1 = c0;
-    r1 = ex(rec - J0);
-    r2 = ex(J1 - rec);
     // max over x of x e^{-theta x}: 1 / (e theta), or its value at x = 1 when theta > 1
     rho1 = rho2 = fabs(th.d) * (thv > 1.0 ? exp(-thv) : 0.36788 / thv);
     kb = fabs(c0.d) + fabs(c0.v) * rho1;
@@ -233,8 +226,6 @@ __global__ void __launch_bounds__(32) k_adj_mode_tab(const SubDesc *subs, int s0
   D[MD_T1] = T1.d; D[MD_T2] = T2.d;
   auto scale = [](double bound) { return bound > 0.0 ? pow2i(-(ilogb(bound) + 1)) : 1.0; };
   D[MD_RHO1] = scale(rho1); D[MD_RHO2] = scale(rho2); D[MD_RFD] = scale(kb);
-  const double sr = sgn(rec - J0);
-  D[MD_REC] = sr * r1.d; D[MD_REC + 1] = sr * r2.d;
 }
 
 // d phi/dk on the rows J0 .. J1, [2][Py + 2][Nq], from phi
@@ -368,24 +359,25 @@ __device__ __forceinline__ void mark_tile(unsigned *mask, int kb, const long lon
 }
 
 // Moment tables: of the cotangent (res false: phi_1, phi_2 and their k-derivatives at the gamma columns), or
-// of the residual (res true: the k-derivatives of phi_1, phi_2 and of kappa at the receiver row).
+// of the residual (res true: the k-derivatives of phi_1, phi_2 and, per subdomain, of kappa at its receiver row).
 __global__ void __launch_bounds__(256) k_adj_mb(const SubDesc *subs, int s0, const double *tab, const unsigned char *sep,
                                                 unsigned char *adj, int res) {
   const int si = s0 + blockIdx.z;
   const SubDesc &d = subs[si];
-  if (!d.tc_cols || d.leader != si) return;
+  if (!d.tc_cols) return;
   const SepGeo g = sep_geo(d);
   const AdjGeo a = adj_geo(d, g);
-  const int nb = res ? ADJ_DMOM : ADJ_MOM, nto = nb * g.nqp / 32, nk = res ? g.nk1 : a.nk1, nkj = res ? g.nkj : a.nkj;
+  const int nb = res ? g.nb : ADJ_MOM, nto = nb * g.nqp / 32, nk = res ? g.nk1 : a.nk1, nkj = res ? g.nkj : a.nkj;
   const int e = blockIdx.y / nto, to = blockIdx.y % nto, kb = blockIdx.x * 4 + (threadIdx.x >> 6);
   if (e >= g.ncls || kb >= nk) return;
   const int o = threadIdx.x & 31, half = (threadIdx.x >> 5) & 1;
   const int b = to * 32 / g.nqp, q = sep_mode(d, e, to * 32 % g.nqp + o);
+  if (!(res && b == 2) && d.leader != si) return;
   const int c = kb / nkj, j0 = (kb % nkj) * 16 + 8 * half;
   long long V[8];
 #pragma unroll
   for (int j = 0; j < 8; ++j) V[j] = 0;
-  if (q <= d.Nq && !(res && b == 2 && d.nrec < 0)) {
+  if (q <= d.Nq) {
     const double sn = tab[d.sin_off + (int)(((long long)q * (res ? sep_src_col(d, c) : sep_out_col(d, c))) % (2 * d.Nx))];
     const double *P = reinterpret_cast<const double *>(sep + d.sep_phi), *Q = reinterpret_cast<const double *>(adj + d.adj_phid);
     const double *T = reinterpret_cast<const double *>(sep + d.sep_mt) + (long long)(q - 1) * SEP_MTW;
@@ -404,25 +396,29 @@ __global__ void __launch_bounds__(256) k_adj_mb(const SubDesc *subs, int s0, con
       V[j] = fix54(v * sn);
     }
   }
-  mark_tile(reinterpret_cast<unsigned *>(adj + (res ? d.adj_zd : d.adj_zm)) + (e * nto + to) * SEP_MASK, kb, V);
-  unsigned char *B = adj + (res ? d.adj_dmb : d.adj_mb) + (((long long)e * nto + to) * nk + kb) * SEP_BBLK;
+  const SepMoment m = res ? adj_dmoment(d, g, e, to)
+                          : SepMoment{d.adj_mb + ((long long)e * nto + to) * nk * SEP_BBLK, d.adj_zm + 4LL * SEP_MASK * (e * nto + to)};
+  mark_tile(reinterpret_cast<unsigned *>(adj + m.mask), kb, V);
+  unsigned char *B = adj + m.blocks + (long long)kb * SEP_BBLK;
   store_digits(B + (o >> 3) * 256 + half * 128 + (o & 7) * 16, 1024, V);
 }
 
 // The synthesis on the ring columns: output (c, j), K index (b, q): (2/Nx) sin(pi q m_c/Nx) times phi_b(j), or
-// (b = 2) kappa_q(|rec - j|) scaled to below 1.
+// (b = 2, per subdomain) kappa_q(|rec - j|) scaled to below 1.
 __global__ void __launch_bounds__(256) k_adj_b3(const SubDesc *subs, int s0, const double *tab, const unsigned char *sep,
                                                 unsigned char *adj) {
   const int si = s0 + blockIdx.z;
   const SubDesc &d = subs[si];
-  if (!d.tc_cols || d.leader != si) return;
+  if (!d.tc_cols) return;
   const SepGeo g = sep_geo(d);
   const AdjGeo a = adj_geo(d, g);
   const int e = blockIdx.y / a.nt3, to = blockIdx.y % a.nt3, kb = blockIdx.x * 4 + (threadIdx.x >> 6);
   if (e >= g.ncls || kb >= a.nk3) return;
   const int o = threadIdx.x & 31, half = (threadIdx.x >> 5) & 1;
   const int c = to / a.nti, i = (to % a.nti) * 32 + o, m = sep_src_col(d, c);
-  const int b = kb * 16 / g.nqp, q0 = kb * 16 % g.nqp + 8 * half, row = 3 + i;
+  const int k2 = 2 * g.nqp / 16, b = kb * 16 / g.nqp;
+  if (b < 2 && d.leader != si) return;
+  const int q0 = kb * 16 % g.nqp + 8 * half, row = 3 + i;
   const double *S = tab + d.sin_off, *P = reinterpret_cast<const double *>(sep + d.sep_phi), sc = inv_scale(d);
   const long long p2 = (long long)(d.Py + 2) * d.Nq;
   long long V[8];
@@ -440,8 +436,9 @@ __global__ void __launch_bounds__(256) k_adj_b3(const SubDesc *subs, int s0, con
     }
     V[j] = fix54(v * (sc * S[(int)(((long long)q * m) % (2 * d.Nx))]));
   }
-  mark_tile(reinterpret_cast<unsigned *>(adj + d.adj_z3) + (e * a.nt3 + to) * SEP_MASK, kb, V);
-  unsigned char *B = adj + d.adj_b3 + (((long long)e * a.nt3 + to) * a.nk3 + kb) * SEP_BBLK;
+  const long long t = (long long)e * a.nt3 + to;
+  mark_tile(reinterpret_cast<unsigned *>(adj + (b < 2 ? d.adj_z3 : d.adj_r3z)) + t * SEP_MASK, kb, V);
+  unsigned char *B = adj + (b < 2 ? d.adj_b3 + (t * k2 + kb) * SEP_BBLK : d.adj_r3 + (t * (k2 / 2) + kb - k2) * SEP_BBLK);
   store_digits(B + (o >> 3) * 256 + half * 128 + (o & 7) * 16, 1024, V);
 }
 
@@ -624,13 +621,13 @@ struct GradSrc {
       t.nkj = g.nkj; t.ND = g.ND; t.ti = t.nt % g.nti;
       t.eb = reinterpret_cast<const int *>(adj + d.adj_kde)[g.ncls * g.nS + es];
     } else if (t.nt < g.nt3 + nm) {
-      const int m = t.e * (3 * g.nqp / 32) + t.nt - g.nt3;
-      t.B = sep + d.sep_mb + (long long)m * nk * SEP_BBLK;
-      mb = reinterpret_cast<const unsigned *>(sep + d.sep_zm) + m * SEP_MASK;
+      const SepMoment m = sep_moment(d, g, t.e, t.nt - g.nt3);
+      t.B = sep + m.blocks;
+      mb = reinterpret_cast<const unsigned *>(sep + m.mask);
     } else {
-      const int m = t.e * (ADJ_DMOM * g.nqp / 32) + t.nt - g.nt3 - nm;
-      t.B = adj + d.adj_dmb + (long long)m * nk * SEP_BBLK;
-      mb = reinterpret_cast<const unsigned *>(adj + d.adj_zd) + m * SEP_MASK;
+      const SepMoment m = adj_dmoment(d, g, t.e, t.nt - g.nt3 - nm);
+      t.B = adj + m.blocks;
+      mb = reinterpret_cast<const unsigned *>(adj + m.mask);
     }
     t.masks(ma, mb);
     return true;
@@ -694,11 +691,18 @@ struct AdjSrc {
     t.A = reinterpret_cast<const unsigned char *>(ws + it.a_off + w.a[t.job]) + (long long)tr * nk * SEP_ABLK;
     t.ex = reinterpret_cast<const int *>(ws + it.a_off + w.ex[t.job]) + tr * 128;
     const unsigned *ma = reinterpret_cast<const unsigned *>(ws + it.a_off + w.mask) + adj_mask_of(t.job, it.ncols) + tr * SEP_MASK;
-    const unsigned *mb = nullptr;
+    const unsigned *mb = nullptr, *mb2 = nullptr;
     t.eb = t.nkj = t.ND = t.ti = 0;
     if (t.job == A_SYN) {
-      t.B = adj + d.adj_b3 + ((long long)t.e * a.nt3 + t.nt) * nk * SEP_BBLK;
-      mb = reinterpret_cast<const unsigned *>(adj + d.adj_z3) + (t.e * a.nt3 + t.nt) * SEP_MASK;
+      const long long v3 = (long long)t.e * a.nt3 + t.nt;
+      const int k2 = 2 * g.nqp / 16;
+      t.B = adj + d.adj_b3 + v3 * k2 * SEP_BBLK;
+      mb = reinterpret_cast<const unsigned *>(adj + d.adj_z3) + v3 * SEP_MASK;
+      if (a.nb == 3) {
+        t.k2 = k2;
+        t.B2 = adj + d.adj_r3 + v3 * (k2 / 2) * SEP_BBLK;
+        mb2 = reinterpret_cast<const unsigned *>(adj + d.adj_r3z) + v3 * SEP_MASK;
+      }
       t.eb = inv_exp(d);
     } else if (t.job == A_INV) {
       t.B = adj + d.adj_bi + ((long long)t.e * a.ntr + t.nt) * nk * SEP_BBLK;
@@ -715,7 +719,7 @@ struct AdjSrc {
       t.B = adj + d.adj_mb + (long long)m * nk * SEP_BBLK;
       mb = reinterpret_cast<const unsigned *>(adj + d.adj_zm) + m * SEP_MASK;
     }
-    t.masks(ma, mb);
+    t.masks(ma, mb, mb2);
     return true;
   }
   __device__ __forceinline__ void dest(const Tile &t, int r, int o, double *&dst, long long &step, int &cnt) const {
@@ -777,6 +781,9 @@ __device__ __forceinline__ double adj_modes_body(const Item &it, const SubDesc &
   const int cp = sep_pad128(it.ncols), R = 2 * cp;
   const long long nc = it.ncols;
   const double *ga = ws + it.a_off + w.ga;
+  // phi_1 at the receiver row; phi_2 lies p2 further on, and so in the table of their k-derivatives
+  const long long orec = (long long)(d.nrec - d.nlo + 1) * d.Nq + q - 1, p2 = (long long)(d.Py + 2) * d.Nq;
+  const double *prec = reinterpret_cast<const double *>(sep + d.sep_phi) + orec;
   const double *mom = ws + it.a_off + w.mom + ((long long)e * ADJ_MOM * g.nqp + qi) * R + b;
   cplx F[6], dM[2], f4 = cmk(0.0, 0.0);   // moments, gamma rows; derivative moments; receiver row
 #pragma unroll
@@ -789,8 +796,8 @@ __device__ __forceinline__ double adj_modes_body(const Item &it, const SubDesc &
   }
   if (rec) {
     f4 = ld2(ga + 2 * ((4LL * d.Nq + (q - 1)) * nc + b));
-    F[0] = caxpy(T[MT_REC], f4, F[0]);
-    F[1] = caxpy(T[MT_REC + 1], f4, F[1]);
+    F[0] = caxpy(prec[0], f4, F[0]);
+    F[1] = caxpy(prec[p2], f4, F[1]);
   }
   const bool imag = T[MT_IMAG] != 0.0;
   cplx m1 = F[0], m2 = F[1], iA = cmk(0.0, 0.0), iB = iA;   // moments of all rows; i Im R times them
@@ -821,7 +828,7 @@ __device__ __forceinline__ double adj_modes_body(const Item &it, const SubDesc &
 #pragma unroll
   for (int k = 0; k < 2; ++k) { ae[(long long)k * g.nqp * R] = A[k].re; ae[(long long)k * g.nqp * R + cp] = A[k].im; }
   if (d.nrec >= 0) {
-    const double s = T[MT_REC + 2];
+    const double s = T[MT_RFI];
     ae[2LL * g.nqp * R] = s * f4.re;
     ae[2LL * g.nqp * R + cp] = s * f4.im;
   }
@@ -899,7 +906,8 @@ __device__ __forceinline__ double adj_modes_body(const Item &it, const SubDesc &
   s += redotc(dM[0], a0) + redotc(dM[1], a1);
   if (rec) {
     const cplx m3 = at(rd, 2, inv2(D[MD_RFD]));
-    s += redotc(f4, cadd(caxpy(D[MD_REC], a0, caxpy(D[MD_REC + 1], a1, zero)), m3));
+    const double *dp = reinterpret_cast<const double *>(adj + d.adj_phid) + orec;
+    s += redotc(f4, cadd(caxpy(dp[0], a0, caxpy(dp[p2], a1, zero)), m3));
   }
   return s;
 }
@@ -1043,7 +1051,7 @@ cudaError_t launch_adj_tables(const mdp_plan *p, cudaStream_t st) {
   int mq = 0, mrow = 0, mdist = 0, mes = 0, mtb[2] = {0, 0}, mk[2] = {0, 0}, mt[2] = {0, 0}, m3 = 0, m3k = 0;
   for (size_t i = 0; i < p->subs.size(); ++i) {
     const SubDesc &d = p->subs[i].d;
-    if (!d.tc_cols || d.leader != (int)i) continue;
+    if (!d.tc_cols || (d.leader != (int)i && d.nrec < 0)) continue;   // a duplicate has its receiver row's tables
     const SepGeo g = sep_geo(d);
     const AdjGeo a = adj_geo(d, g);
     mq = std::max(mq, (d.Nq + 127) / 128);
@@ -1055,7 +1063,7 @@ cudaError_t launch_adj_tables(const mdp_plan *p, cudaStream_t st) {
     mk[0] = std::max(mk[0], (a.nk1 + 3) / 4);
     mk[1] = std::max(mk[1], (g.nk1 + 3) / 4);
     mt[0] = std::max(mt[0], g.ncls * ADJ_MOM * g.nqp / 32);
-    mt[1] = std::max(mt[1], g.ncls * ADJ_DMOM * g.nqp / 32);
+    mt[1] = std::max(mt[1], g.ncls * g.nb * g.nqp / 32);
     m3 = std::max(m3, g.ncls * a.nt3);
     m3k = std::max(m3k, (a.nk3 + 3) / 4);
   }

@@ -77,6 +77,10 @@ struct SubDesc {
   long long adj_zm, adj_z3, adj_zd, adj_md, adj_phid, adj_kdd, adj_kde, adj_tb, adj_mb, adj_b3, adj_bf, adj_bi, adj_dtb,
       adj_dmb;
   long long sep_mx;     // per mode SEP_MXW doubles: the full-grid solve along y (kernels_full.cu)
+  // what depends on the receiver row, each subdomain's own (the rest is its leader's): the third block of the
+  // moments and its masks; in the gradient tables that of the residual's derivative moments, and the third K block
+  // of the synthesis
+  long long sep_rz, sep_rb, adj_rz, adj_rb, adj_r3z, adj_r3;
   long long out_off;    // complex elements: start of the subdomain's output block
   long long rec_off;    // complex elements: start of the receiver block [n_cols][Px - 2]
   int *dstatus;         // the plan's device status word (bounds-checked build: first error; else unused)
@@ -190,6 +194,20 @@ inline __host__ __device__ SepGeo sep_geo(const SubDesc &d) {
 // mode number of entry qi of class e (past Nq: padding), of entry qi of parity e (0: odd modes)
 inline __host__ __device__ int sep_mode(const SubDesc &d, int e, int qi) { return d.xsym ? 2 * qi + 1 + e : qi + 1; }
 inline __host__ __device__ int sep_parity_mode(int e, int qi) { return 2 * qi + 1 + e; }
+// bytes into the separable tables of the moments of 32 modes (output group `to` of class e): blocks of all groups
+// of K, mask; the first two blocks of nqp modes phi_1, phi_2, the third a receiver row's
+struct SepMoment { long long blocks, mask; };
+inline __host__ __device__ SepMoment sep_moment(const SubDesc &d, const SepGeo &g, int e, int to) {
+  const int n = g.nqp / 32, i = to < 2 * n ? e * 2 * n + to : e * n + to - 2 * n;
+  return {(to < 2 * n ? d.sep_mb : d.sep_rb) + (long long)i * g.nk1 * SEP_BBLK,
+          (to < 2 * n ? d.sep_zm : d.sep_rz) + 4LL * SEP_MASK * i};
+}
+// the same into the gradient tables: the k-derivatives of the residual's moments
+inline __host__ __device__ SepMoment adj_dmoment(const SubDesc &d, const SepGeo &g, int e, int to) {
+  const int n = g.nqp / 32, i = to < 2 * n ? e * 2 * n + to : e * n + to - 2 * n;
+  return {(to < 2 * n ? d.adj_dmb : d.adj_rb) + (long long)i * g.nk1 * SEP_BBLK,
+          (to < 2 * n ? d.adj_zd : d.adj_rz) + 4LL * SEP_MASK * i};
+}
 // grid column of output s (gamma) and of source c (ring); x-centred: the left ones, the right ones mirrored
 inline __host__ __device__ int sep_out_col(const SubDesc &d, int s) {
   return s == 0 ? d.mlo - 1 : s == 1 ? d.mlo : s == 2 ? d.mhi : d.mhi + 1;
@@ -314,7 +332,7 @@ inline __host__ __device__ FullWs full_ws(const SubDesc &d, int nr) {
 // ---- separable gradient pass (kernels_sepadj.cu): the same contractions with gamma and the ring exchanged
 constexpr int ADJ_MDW = 68;               // doubles per mode of the k-derivative table
 constexpr int ADJ_MOM = 4;                // moments of the cotangent per mode: phi_1, phi_2, their k-derivatives
-constexpr int ADJ_DMOM = 3;               // k-derivative moments of the residual: phi_1, phi_2, receiver
+constexpr int ADJ_DMOM = 3;               // k-derivative moments of the residual: phi_1, phi_2, receiver (tables of its own)
 enum AdjJob { A_MID = 0, A_FWD, A_SYN, A_INV };
 struct AdjGeo {
   int ncls, nS, nqp, nqh;

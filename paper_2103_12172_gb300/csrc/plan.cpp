@@ -422,9 +422,11 @@ static bool layout_tables(mdp_plan *p) {
   auto take = [&](long long bytes) { const long long o = sep; sep += (bytes + 255) & ~255LL; return o; };
   for (auto &hs : p->subs) {
     SubDesc &d = hs.d;
-    if (d.leader != (int)(&hs - p->subs.data()) || !d.tc_cols) continue;
+    if (!d.tc_cols) continue;
     const SepGeo g = sep_geo(d);
-    d.sep_zm = take(4LL * SEP_MASK * g.ncls * (3 * g.nqp / 32));
+    d.sep_rz = take(4LL * SEP_MASK * g.ncls * (g.nqp / 32));
+    if (d.leader != (int)(&hs - p->subs.data())) continue;
+    d.sep_zm = take(4LL * SEP_MASK * g.ncls * (2 * g.nqp / 32));
     d.sep_z3 = take(4LL * SEP_MASK * g.ncls * g.nt3);
   }
   p->sep_masks = sep;
@@ -432,17 +434,26 @@ static bool layout_tables(mdp_plan *p) {
   auto take_adj = [&](long long bytes) { const long long o = adj; adj += (bytes + 255) & ~255LL; return o; };
   for (auto &hs : p->subs) {
     SubDesc &d = hs.d;
-    if (d.leader != (int)(&hs - p->subs.data()) || !d.tc_cols) continue;
+    if (!d.tc_cols) continue;
     const SepGeo g = sep_geo(d);
     const AdjGeo a = adj_geo(d, g);
+    d.adj_rz = take_adj(4LL * SEP_MASK * g.ncls * (g.nqp / 32));
+    d.adj_r3z = take_adj(4LL * SEP_MASK * g.ncls * a.nt3);
+    if (d.leader != (int)(&hs - p->subs.data())) continue;
     d.adj_zm = take_adj(4LL * SEP_MASK * g.ncls * (ADJ_MOM * g.nqp / 32));
     d.adj_z3 = take_adj(4LL * SEP_MASK * g.ncls * a.nt3);
-    d.adj_zd = take_adj(4LL * SEP_MASK * g.ncls * (ADJ_DMOM * g.nqp / 32));
+    d.adj_zd = take_adj(4LL * SEP_MASK * g.ncls * (2 * g.nqp / 32));
   }
   p->adj_masks = adj;
   for (auto &hs : p->subs) {
     SubDesc &d = hs.d;
-    if (d.leader != (int)(&hs - p->subs.data())) {   // a duplicate: the leader's tables
+    if (d.tc_cols) {   // the receiver row's tables, made where there is one
+      const SepGeo g = sep_geo(d);
+      d.sep_rb = take((long long)g.ncls * (g.nqp / 32) * g.nk1 * SEP_BBLK);
+      d.adj_rb = take_adj((long long)g.ncls * (g.nqp / 32) * g.nk1 * SEP_BBLK);
+      d.adj_r3 = take_adj((long long)g.ncls * adj_geo(d, g).nt3 * (g.nqp / 16) * SEP_BBLK);
+    }
+    if (d.leader != (int)(&hs - p->subs.data())) {   // a duplicate: the leader's other tables
       const SubDesc &ld = p->subs[d.leader].d;
       d.fact_off = ld.fact_off; d.dT_off = ld.dT_off; d.sin_off = ld.sin_off; d.geo_off = ld.geo_off;
       d.seg_off = ld.seg_off; d.fs_off = ld.fs_off; d.piv_off = ld.piv_off;
@@ -463,7 +474,7 @@ static bool layout_tables(mdp_plan *p) {
       d.sep_kd = take(8 * pairs * d.Py);
       d.sep_kde = take(4LL * g.ncls * g.nS);
       d.sep_tb = take(pairs * g.ND * SEP_BBLK);
-      d.sep_mb = take((long long)g.ncls * (3 * g.nqp / 32) * g.nk1 * SEP_BBLK);   // room for receivers
+      d.sep_mb = take((long long)g.ncls * (2 * g.nqp / 32) * g.nk1 * SEP_BBLK);
       d.sep_b3 = take((long long)g.ncls * g.nt3 * g.nk3 * SEP_BBLK);
       d.sep_bf = take(2LL * (g.nqh / 32) * g.nkf * SEP_BBLK);
       d.sep_bi = take(2LL * g.ntg * (g.nqh / 16) * SEP_BBLK);
@@ -476,11 +487,11 @@ static bool layout_tables(mdp_plan *p) {
       d.adj_kde = take_adj(8LL * g.ncls * g.nS);
       d.adj_tb = take_adj(pairs * a.ND * SEP_BBLK);
       d.adj_mb = take_adj((long long)g.ncls * (ADJ_MOM * g.nqp / 32) * a.nk1 * SEP_BBLK);
-      d.adj_b3 = take_adj((long long)g.ncls * a.nt3 * (3 * g.nqp / 16) * SEP_BBLK);   // room for receivers
+      d.adj_b3 = take_adj((long long)g.ncls * a.nt3 * (2 * g.nqp / 16) * SEP_BBLK);
       d.adj_bf = take_adj(2LL * (g.nqh / 32) * a.nkf * SEP_BBLK);
       d.adj_bi = take_adj(2LL * a.ntr * (g.nqh / 16) * SEP_BBLK);
       d.adj_dtb = take_adj(pairs * g.ND * SEP_BBLK);
-      d.adj_dmb = take_adj((long long)g.ncls * (ADJ_DMOM * g.nqp / 32) * g.nk1 * SEP_BBLK);
+      d.adj_dmb = take_adj((long long)g.ncls * (2 * g.nqp / 32) * g.nk1 * SEP_BBLK);
     }
     const int FW = d.cplx ? 8 : 4;
     d.fact_off = off; off += al((long long)d.Nq * d.Nt * FW);

@@ -183,3 +183,35 @@ def test_captured_gradient_follows_the_wavenumbers(mdp):
             rx, rk = p.adjoint(cot)
             assert torch.equal(out[0], rx) and torch.equal(out[1], rk)
     plan.status()
+
+
+@pytest.mark.parametrize("rows", [(-1, 16, 16), (9, 20, 9), (20, -1, 14)])
+@pytest.mark.parametrize("off", [0.0, 0.1])
+def test_deduplicated_subdomains_have_receiver_rows_of_their_own(mdp, rows, off):
+    """Three copies of a subdomain on one set of tables, with receiver rows that differ from the first one's, in
+    both orders of setting them: columns, receiver values and gradients (with and without the receivers' cotangent)
+    of the plain plan. Bar: 1e-12, the same sums on placements that differ in their last bits."""
+    from dataclasses import replace
+    b = box(37, 33, 9.0, W.AP_DIRX_SOMMY, 2, dx=off)
+    subs = [replace(b, x0=b.x0 + i, x1=b.x1 + i, ax0=b.ax0 + i) for i in range(3)]
+    dd, plain = mdp.Plan(subs, dedupe=True), mdp.Plan(subs)
+    assert dd.leaders() == [0, 0, 0]
+    dd.set_receivers(rows[::-1])
+    cot = torch.from_numpy(W.random_complex(plain.output_size, seed=16)).cuda()
+    xi = torch.from_numpy(W.random_complex(plain.output_size, seed=17)).cuda()
+    for p in (dd, plain):
+        p.set_receivers(rows)
+    cr = torch.from_numpy(W.random_complex(plain.receiver_size, seed=18)).cuda()
+    for k in (None, 9.3):
+        got = []
+        for p in (dd, plain):
+            if k is not None:
+                p.update_k([k] * 3)
+            res = list(p.project(out_rec=True)) + list(p.project(xi=xi, out_rec=True))
+            for c in (cr, None):
+                for x in (xi, None):
+                    res += p.adjoint(cot, xi=x, cot_rec=c)
+            p.status()
+            got.append(res)
+        for a, r in zip(*got):
+            assert (a - r).abs().max() <= 1e-12 * r.abs().max()
