@@ -337,8 +337,10 @@ long long mdp_ap_solve_noalloc_limit_bytes(void);
  * potential_solution_homo: u = P_N+ xi_gamma). rows[i] is the AP grid row n of subdomain i,
  * nlo+1 <= n <= nhi-1 (strictly inside the gamma ring), or -1 for none (host array of n_subs).
  * The receivers of subdomain i are the nodes (n, m), m = mlo+1 .. mhi-1 (not on gamma, where
- * w = 0, so P_N+ xi = -G^(h) L^(h) w there). Uploads a small descriptor array; allocates nothing
- * and synchronises the device. */
+ * w = 0, so P_N+ xi = -G^(h) L^(h) w there). Uploads small descriptor arrays and rebuilds the tables of
+ * the separable solve; allocates nothing and synchronises the device. Calls that a caller has captured into a CUDA
+ * graph without receiver arguments replay as before; one captured with them is to be captured again when a
+ * subdomain's receivers come or go. */
 mdp_status mdp_plan_set_receivers(mdp_plan *p, const int *rows);
 
 /* Receiver layout of subdomain `sub` (host): grid row (or -1), first node m, number of nodes

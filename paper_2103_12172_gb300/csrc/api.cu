@@ -71,12 +71,24 @@ void free_device(mdp_plan *p) {
 }
 
 mdp_status upload_subs_tables(mdp_plan *p) {
-  std::vector<SubDesc> ds;
-  for (auto &hs : p->subs) ds.push_back(hs.d);
+  std::vector<SubDesc> ds(2 * (size_t)p->n_subs);
+  fill_subs(p, ds.data());
   CK(cudaMemcpy(p->d_subs, ds.data(), ds.size() * sizeof(SubDesc), cudaMemcpyHostToDevice));
   CK(cudaMemcpy(p->d_tables, p->host_tables.data(), p->host_tables.size() * sizeof(double), cudaMemcpyHostToDevice));
   CK(cudaMemcpy(p->d_piv, p->host_piv.data(), p->host_piv.size(), cudaMemcpyHostToDevice));
   return MDP_OK;
+}
+
+// block prefix sums of a wave's items, without or with the receiver rows
+void fill_prefix(const mdp_plan *p, const std::vector<Item> &items, std::vector<int> &pre, bool rec) {
+  const size_t n = items.size();
+  for (int f = 0; f < NFAM; ++f) {
+    int *q = pre.data() + ((rec ? NFAM : 0) + f) * (n + 1);
+    for (size_t i = 0; i < n; ++i) {
+      const SubDesc &d = p->subs[items[i].sub].d;
+      q[i + 1] = q[i] + blocks_for((Fam)f, rec ? d : without_rec(d), items[i].ncols, items[i].col0);
+    }
+  }
 }
 
 mdp_status alloc_device(mdp_plan *p) {
@@ -84,11 +96,11 @@ mdp_status alloc_device(mdp_plan *p) {
   CK(cudaDeviceGetAttribute(&p->n_sm, cudaDevAttrMultiProcessorCount, p->device));
   CK(set_kernel_attributes());
   auto al = [&](void **ptr, size_t bytes) -> bool { return cudaMalloc(ptr, std::max<size_t>(bytes, 256)) == cudaSuccess; };
-  if (!al((void **)&p->d_subs, p->subs.size() * sizeof(SubDesc)) ||
+  if (!al((void **)&p->d_subs, 2 * p->subs.size() * sizeof(SubDesc)) ||
       !al((void **)&p->d_tables, p->n_tables * sizeof(double)) ||
       !al((void **)&p->d_piv, p->host_piv.size()) || !al((void **)&p->d_sep, (size_t)p->sep_bytes) || !al((void **)&p->d_ws, (size_t)p->ws_doubles * 8) ||
       !al((void **)&p->d_status, sizeof(int)) || !al((void **)&p->d_fstatus, sizeof(int)) ||
-      !p->sub_stage.alloc(p->subs.size(), true) || !p->h_fstatus.alloc(1, true))
+      !p->sub_stage.alloc(2 * p->subs.size(), true) || !p->h_fstatus.alloc(1, true))
     return MDP_ERR_NOMEM;
   CK(cudaMemset(p->d_status, 0, sizeof(int)));
   CK(cudaMemset(p->d_fstatus, 0, sizeof(int)));
@@ -135,13 +147,11 @@ mdp_status alloc_device(mdp_plan *p) {
       int *dp = nullptr;
       if (!al((void **)&di, n * sizeof(Item))) return MDP_ERR_NOMEM;
       ditems.push_back(di);
-      if (!al((void **)&dp, (size_t)NFAM * (n + 1) * sizeof(int))) return MDP_ERR_NOMEM;
+      if (!al((void **)&dp, 2 * (size_t)NFAM * (n + 1) * sizeof(int))) return MDP_ERR_NOMEM;
       dpre.push_back(dp);
-      std::vector<int> pre((size_t)NFAM * (n + 1), 0);
-      for (int f = 0; f < NFAM; ++f)
-        for (int i = 0; i < n; ++i)
-          pre[(size_t)f * (n + 1) + i + 1] =
-              pre[(size_t)f * (n + 1) + i] + blocks_for((Fam)f, p->subs[w.items[i].sub].d, w.items[i].ncols, w.items[i].col0);
+      std::vector<int> pre(2 * (size_t)NFAM * (n + 1), 0);
+      fill_prefix(p, w.items, pre, false);
+      fill_prefix(p, w.items, pre, true);
 #if MDP_CHECKED
       if (fault && !std::strcmp(fault, "desc") && sc == S_PROJ && &w == &waves.front() && n > 0) {
         std::vector<Item> bad(w.items);
@@ -179,21 +189,23 @@ mdp_status alloc_device(mdp_plan *p) {
   return MDP_OK;
 }
 
-void wave_batches(const mdp_plan *p, size_t w, Batch *fb, int sc) {
+void wave_batches(const mdp_plan *p, size_t w, Batch *fb, int sc, bool rec) {
   const int n = (int)p->sched[sc][w].items.size();
+  const size_t v = rec ? (size_t)NFAM * (n + 1) : 0;
   for (int f = 0; f < NFAM; ++f) {
     Batch &b = fb[f];
     std::memset(&b, 0, sizeof b);
     b.items = p->d_items[sc][w];
-    b.prefix = p->d_prefix[sc][w] + (size_t)f * (n + 1);
+    b.prefix = p->d_prefix[sc][w] + v + (size_t)f * (n + 1);
     b.order = f == F_TRI ? p->d_order[sc][w]
               : f == F_ATRI ? p->d_order[sc][w] + p->h_prefix[sc][w][(size_t)F_TRI * (n + 1) + n] : nullptr;
     b.n_items = n;
-    b.total_blocks = p->h_prefix[sc][w][(size_t)f * (n + 1) + n];
+    b.total_blocks = p->h_prefix[sc][w][v + (size_t)f * (n + 1) + n];
     set_bounds(p, b, p->out_size, sc == S_GRAD);
   }
 }
 
+// of a call without receivers
 void single_batches(const mdp_plan *p, const Item &it, Batch *fb, long long out_n) {
   for (int f = 0; f < NFAM; ++f) {
     Batch &b = fb[f];
@@ -202,7 +214,7 @@ void single_batches(const mdp_plan *p, const Item &it, Batch *fb, long long out_
     b.prefix = nullptr;
     b.n_items = 1;
     b.one = it;
-    b.total_blocks = blocks_for((Fam)f, p->subs[it.sub].d, it.ncols, it.col0);
+    b.total_blocks = blocks_for((Fam)f, without_rec(p->subs[it.sub].d), it.ncols, it.col0);
     set_bounds(p, b, out_n, false);
   }
 }
@@ -385,8 +397,8 @@ mdp_status mdp_plan_update_k_stream(mdp_plan *p, const double *k, void *cuda_str
   if (p->ready_ev[p->set]) CK(cudaEventSynchronize(p->ready_ev[p->set]));
   if (p->used_rec[p->set]) CK(cudaStreamWaitEvent(s, p->used_ev[p->set], 0));   // readers on other streams
   HostBuf<SubDesc> &stage = stage_of(p, p->set);
-  for (size_t i = 0; i < p->subs.size(); ++i) stage[i] = p->subs[i].d;
-  CK(cudaMemcpyAsync(p->d_subs, stage.data(), p->subs.size() * sizeof(SubDesc), cudaMemcpyHostToDevice, s));
+  fill_subs(p, stage.data());
+  CK(cudaMemcpyAsync(p->d_subs, stage.data(), stage.size() * sizeof(SubDesc), cudaMemcpyHostToDevice, s));
   CK(cudaMemsetAsync(p->d_fstatus, 0, sizeof(int), s));
   CK(launch_update(p, p->d_subs, p->d_tables, p->d_piv, p->d_sep, p->d_fstatus, s));
   CK(cudaMemcpyAsync(p->h_fstatus.data(), p->d_fstatus, sizeof(int), cudaMemcpyDeviceToHost, s));
@@ -407,10 +419,10 @@ mdp_status mdp_plan_update_k_async(mdp_plan *p, const double *k, void *cuda_stre
   if (!p->alt_tables) {   // first call: the second set starts as a copy of the first (k-independent tables)
     const size_t nt = std::max<size_t>(p->n_tables * sizeof(double), 256);
     const size_t np = std::max<size_t>(p->host_piv.size(), 256);
-    const size_t ns = std::max<size_t>(p->subs.size() * sizeof(SubDesc), 256);
+    const size_t ns = std::max<size_t>(2 * p->subs.size() * sizeof(SubDesc), 256);
     if (cudaMalloc((void **)&p->alt_tables, nt) != cudaSuccess || cudaMalloc((void **)&p->alt_piv, np) != cudaSuccess ||
         cudaMalloc((void **)&p->alt_sep, std::max<size_t>((size_t)p->sep_bytes, 256)) != cudaSuccess ||
-        cudaMalloc((void **)&p->alt_subs, ns) != cudaSuccess || !p->alt_stage.alloc(p->subs.size(), true))
+        cudaMalloc((void **)&p->alt_subs, ns) != cudaSuccess || !p->alt_stage.alloc(2 * p->subs.size(), true))
       return MDP_ERR_NOMEM;
     for (int s_ = 0; s_ < 2; ++s_) {
       CK(cudaEventCreateWithFlags(&p->ready_ev[s_], cudaEventDisableTiming));
@@ -426,8 +438,8 @@ mdp_status mdp_plan_update_k_async(mdp_plan *p, const double *k, void *cuda_stre
   HostBuf<SubDesc> &stage = stage_of(p, b);
   CK(cudaEventSynchronize(p->ready_ev[b]));   // the stage fed the upload of the last refactorisation into set b
   if (p->used_rec[b]) CK(cudaStreamWaitEvent(s, p->used_ev[b], 0));   // queued calls still reading set b
-  for (size_t i = 0; i < p->subs.size(); ++i) stage[i] = p->subs[i].d;
-  CK(cudaMemcpyAsync(p->alt_subs, stage.data(), p->subs.size() * sizeof(SubDesc), cudaMemcpyHostToDevice, s));
+  fill_subs(p, stage.data());
+  CK(cudaMemcpyAsync(p->alt_subs, stage.data(), stage.size() * sizeof(SubDesc), cudaMemcpyHostToDevice, s));
   CK(launch_update(p, p->alt_subs, p->alt_tables, p->alt_piv, p->alt_sep, p->d_status, s));
   CK(cudaEventRecord(p->ready_ev[b], s));
   std::swap(p->d_subs, p->alt_subs);
@@ -452,7 +464,7 @@ static mdp_status ensure_host_tables(const mdp_plan *cp) {
   return st;
 }
 
-long long mdp_plan_update_bytes(const mdp_plan *p) { return p ? (long long)(p->subs.size() * sizeof(SubDesc)) : 0; }
+long long mdp_plan_update_bytes(const mdp_plan *p) { return p ? (long long)(2 * p->subs.size() * sizeof(SubDesc)) : 0; }
 
 mdp_status mdp_plan_table_sizes(const mdp_plan *p, long long *n_doubles, long long *n_piv) {
   if (!p) return MDP_ERR_ARG;
@@ -530,7 +542,7 @@ mdp_status mdp_project_batch_rec(mdp_plan *p, const mdp_c64 *xi, mdp_c64 *out, m
   auto launch_all = [&]() -> cudaError_t {
     for (size_t w = 0; w < p->sched[sc].size(); ++w) {
       Batch fb[NFAM];
-      wave_batches(p, w, fb, sc);
+      wave_batches(p, w, fb, sc, out_rec != nullptr);
       cudaError_t e = launch_project(p, fb, out_kind, (const double2 *)xi, (double2 *)out, (double2 *)out_rec, st);
       if (e != cudaSuccess) return e;
     }
@@ -670,7 +682,7 @@ mdp_status mdp_ap_adjoint_rec(mdp_plan *p, const mdp_c64 *xi, const mdp_c64 *cot
   CK(te);
   for (size_t w = 0; w < p->sched[S_GRAD].size(); ++w) {
     Batch fb[NFAM];
-    wave_batches(p, w, fb, S_GRAD);
+    wave_batches(p, w, fb, S_GRAD, cot_rec != nullptr);
     CK(launch_adjoint(p, fb, out_kind, (const double2 *)xi, (const double2 *)cot, (const double2 *)cot_rec,
                       (double2 *)grad_xi, grad_k, st));
   }
@@ -777,26 +789,21 @@ mdp_status mdp_plan_set_receivers(mdp_plan *p, const int *rows) {
   if (!device_ok(p)) return MDP_OK;
   CK(cudaSetDevice(p->device));
   CK(cudaDeviceSynchronize());
-  std::vector<SubDesc> ds;
-  for (auto &hs : p->subs) ds.push_back(hs.d);
+  std::vector<SubDesc> ds(2 * (size_t)p->n_subs);
+  fill_subs(p, ds.data());
   CK(cudaMemcpy(p->d_subs, ds.data(), ds.size() * sizeof(SubDesc), cudaMemcpyHostToDevice));
   // the receiver row's moments, into the tables in use (the other set is rebuilt by its next update)
   CK(launch_sep_tables(p, p->d_subs, p->d_tables, p->d_sep, false, nullptr));
   CK(cudaStreamSynchronize(nullptr));
   p->adj_stale = true;
-  // the block counts of the receiver kernel and of the contractions changed: refresh the prefix sums
+  // the block counts with receivers changed
   for (int sc = 0; sc < 3; ++sc) {
     auto &waves = p->sched[sc];
     auto &dpre = p->d_prefix[sc];
     auto &hpre = p->h_prefix[sc];
     for (size_t w = 0; w < waves.size(); ++w) {
-      const int n = (int)waves[w].items.size();
       auto &pre = hpre[w];
-      for (const Fam f : {F_IREC, F_G1B, F_G1U, F_C3B, F_C3U, F_TCOLS, F_G3U, F_SOUT, F_GG1B, F_GG1U, F_AC1, F_AG1, F_ATCOLS})
-        for (int i = 0; i < n; ++i)
-          pre[(size_t)f * (n + 1) + i + 1] =
-              pre[(size_t)f * (n + 1) + i] +
-              blocks_for(f, p->subs[waves[w].items[i].sub].d, waves[w].items[i].ncols, waves[w].items[i].col0);
+      fill_prefix(p, waves[w].items, pre, true);
       CK(cudaMemcpy(dpre[w], pre.data(), pre.size() * sizeof(int), cudaMemcpyHostToDevice));
     }
   }

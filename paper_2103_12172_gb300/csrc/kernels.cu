@@ -1585,7 +1585,7 @@ cudaError_t launch_source_terms(mdp_plan *p, int sub, const double2 *f, const do
   Batch fb[NFAM];
   for (int f_ = 0; f_ < NFAM; ++f_) {
     std::memset(&fb[f_], 0, sizeof fb[f_]);
-    fb[f_].n_items = 1; fb[f_].one = it; fb[f_].total_blocks = blocks_for((Fam)f_, d, 1, 0);
+    fb[f_].n_items = 1; fb[f_].one = it; fb[f_].total_blocks = blocks_for((Fam)f_, without_rec(d), 1, 0);
     set_bounds(p, fb[f_], d.G, false);
   }
   e = launch_project(p, fb, MDP_OUT_Q, xi_i, F, nullptr, st);
@@ -1647,7 +1647,7 @@ cudaError_t set_kernel_attributes() {
 cudaError_t launch_project(mdp_plan *p, const Batch *fb, int out_kind, const double2 *xi_user, double2 *out,
                            double2 *out_rec, cudaStream_t st) {
   const bool basis = xi_user == nullptr;
-  const SubDesc *ds = p->d_subs;
+  const SubDesc *ds = subs_of(p, out_rec != nullptr);
   const double *tab = p->d_tables;
   double *ws = p->d_ws;
   const dim3 b8(32, 8), btri(32, TRI_WARPS);
@@ -1691,11 +1691,12 @@ cudaError_t launch_project(mdp_plan *p, const Batch *fb, int out_kind, const dou
 cudaError_t launch_adjoint(mdp_plan *p, const Batch *fb, int out_kind, const double2 *xi_user, const double2 *cot,
                            const double2 *cot_rec, double2 *grad_xi, double *grad_k, cudaStream_t st) {
   const bool basis = xi_user == nullptr;
-  const SubDesc *ds = p->d_subs;
+  const bool rec = cot_rec != nullptr;
+  const SubDesc *ds = subs_of(p, rec);
   const double *tab = p->d_tables;
   double *ws = p->d_ws;
   const dim3 b8(32, 8), btri(32, TRI_WARPS);
-  cudaError_t e = launch_adj_clear(p, fb, st);
+  cudaError_t e = launch_adj_clear(p, fb, rec, st);
   if (e != cudaSuccess) return e;
   if (grad_k) {  // the residual and the k-derivative sources; by sweeps: forward recompute with every mode-space row kept
     if (basis) MDP_LAUNCH(F_EXT, pdl(k_extend, grid1(fb[F_EXT].total_blocks), dim3(32), 0, st, fb[F_EXT], ds, tab, ws, 1));
@@ -1707,7 +1708,7 @@ cudaError_t launch_adjoint(mdp_plan *p, const Batch *fb, int out_kind, const dou
     else MDP_LAUNCH(F_FROWS, k_fwd_rows<true><<<grid1(fb[F_FROWS].total_blocks), b8, p->fft_smem, st>>>(fb[F_FROWS], ds, tab, ws));
     if (basis) MDP_LAUNCH(F_TRI, k_tri<false, true, 2><<<grid1(fb[F_TRI].total_blocks), btri, TRI_WARPS * 2 * full_stage_bytes<false>(), st>>>(fb[F_TRI], ds, tab, p->d_piv, ws, p->d_sep));
     else MDP_LAUNCH(F_TRI, k_tri<true, true, 2><<<grid1(fb[F_TRI].total_blocks), btri, TRI_WARPS * 2 * full_stage_bytes<true>(), st>>>(fb[F_TRI], ds, tab, p->d_piv, ws, p->d_sep));
-    e = launch_sep_adj_residual(p, fb, !basis, st);
+    e = launch_sep_adj_residual(p, fb, !basis, rec, st);
     if (e != cudaSuccess) return e;
   }
   e = cudaGetLastError();

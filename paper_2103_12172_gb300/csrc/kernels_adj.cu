@@ -668,7 +668,7 @@ cudaError_t set_adj_kernel_attributes() {
 
 cudaError_t launch_adjoint_tail(mdp_plan *p, const Batch *fb, int out_kind, const double2 *xi_user, const double2 *cot,
                                 const double2 *cot_rec, double2 *grad_xi, double *grad_k, cudaStream_t st) {
-  const SubDesc *ds = p->d_subs;
+  const SubDesc *ds = subs_of(p, cot_rec != nullptr);
   const double *tab = p->d_tables;
   double *ws = p->d_ws;
   const dim3 b8(32, 8), b4(32, 4);

@@ -892,7 +892,7 @@ cudaError_t launch_sep_project(mdp_plan *p, const Batch *fb, int out_kind, const
                                double2 *out_rec, cudaStream_t st) {
   const bool user = xi_user != nullptr;
   if (fb[F_SMODE].total_blocks == 0) return cudaSuccess;
-  const SubDesc *ds = p->d_subs;
+  const SubDesc *ds = subs_of(p, out_rec != nullptr);
   double *ws = p->d_ws;
   const int f1c = user ? F_C1U : F_C1B, f1 = user ? F_G1U : F_G1B, f3c = user ? F_C3U : F_C3B, f3 = user ? F_G3U : F_TCOLS;
   auto grid = [&](int f) { return dim3((unsigned)fb[f].total_blocks); };

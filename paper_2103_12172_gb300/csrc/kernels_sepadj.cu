@@ -367,8 +367,15 @@ __global__ void __launch_bounds__(256) k_adj_mb(const SubDesc *subs, int s0, con
   if (!d.tc_cols) return;
   const SepGeo g = sep_geo(d);
   const AdjGeo a = adj_geo(d, g);
-  const int nb = res ? g.nb : ADJ_MOM, nto = nb * g.nqp / 32, nk = res ? g.nk1 : a.nk1, nkj = res ? g.nkj : a.nkj;
-  const int e = blockIdx.y / nto, to = blockIdx.y % nto, kb = blockIdx.x * 4 + (threadIdx.x >> 6);
+  // the receiver row's groups come last: a launch captured without any makes the others all the same
+  const int n = g.nqp / 32, nto = (res ? 2 : ADJ_MOM) * n, nk = res ? g.nk1 : a.nk1, nkj = res ? g.nkj : a.nkj;
+  int e = blockIdx.y / nto, to = blockIdx.y % nto;
+  const int kb = blockIdx.x * 4 + (threadIdx.x >> 6);
+  if (res && e >= g.ncls && d.nrec >= 0) {
+    const int y = blockIdx.y - g.ncls * nto;
+    e = y / n;
+    to = nto + y % n;
+  }
   if (e >= g.ncls || kb >= nk) return;
   const int o = threadIdx.x & 31, half = (threadIdx.x >> 5) & 1;
   const int b = to * 32 / g.nqp, q = sep_mode(d, e, to * 32 % g.nqp + o);
@@ -1088,15 +1095,15 @@ cudaError_t launch_adj_tables(const mdp_plan *p, cudaStream_t st) {
 }
 
 // the residual's side (with the k-gradient), before the cotangent takes the ring buffer
-cudaError_t launch_sep_adj_residual(mdp_plan *p, const Batch *fb, bool user, cudaStream_t st) {
+cudaError_t launch_sep_adj_residual(mdp_plan *p, const Batch *fb, bool user, bool rec, cudaStream_t st) {
   const int fc = user ? F_C1U : F_C1B, fg = user ? F_GG1U : F_GG1B;
   if (fb[fc].total_blocks == 0) return cudaSuccess;
   prof_begin(p, F_C1B, st);
-  cudaError_t e = launch_sep_cut1(fb[fc], p->d_subs, p->d_ws, user, fc, st);
+  cudaError_t e = launch_sep_cut1(fb[fc], subs_of(p, rec), p->d_ws, user, fc, st);
   prof_end(p, F_C1B, st);
   if (e != cudaSuccess) return e;
   prof_begin(p, F_GG1B, st);
-  pdl(k_grad_gemm, dim3(std::min(fb[fg].total_blocks, p->n_sm)), dim3(SG_THREADS), SG_SMEM, st, fb[fg], p->d_subs, p->d_sep,
+  pdl(k_grad_gemm, dim3(std::min(fb[fg].total_blocks, p->n_sm)), dim3(SG_THREADS), SG_SMEM, st, fb[fg], subs_of(p, rec), p->d_sep,
       p->d_adj, p->d_ws, user, fg, p->d_status);
   prof_end(p, F_GG1B, st);
   return cudaGetLastError();
@@ -1106,7 +1113,7 @@ cudaError_t launch_sep_adj_residual(mdp_plan *p, const Batch *fb, bool user, cud
 cudaError_t launch_sep_adjoint(mdp_plan *p, const Batch *fb, bool user, bool dk, const double2 *cot, const double2 *cot_rec,
                                cudaStream_t st) {
   if (fb[F_AMODE].total_blocks == 0) return cudaSuccess;
-  const SubDesc *ds = p->d_subs;
+  const SubDesc *ds = subs_of(p, cot_rec != nullptr);
   double *ws = p->d_ws;
   const int hr = cot_rec ? 1 : 0;
   const dim3 b4(32, 4), b8(32, 8);
@@ -1132,9 +1139,9 @@ cudaError_t launch_sep_adjoint(mdp_plan *p, const Batch *fb, bool user, bool dk,
 }
 
 // the operand masks of a wave's items, before anything is cut into them
-cudaError_t launch_adj_clear(mdp_plan *p, const Batch *fb, cudaStream_t st) {
+cudaError_t launch_adj_clear(mdp_plan *p, const Batch *fb, bool rec, cudaStream_t st) {
   if (fb[F_ACLR].total_blocks == 0) return cudaSuccess;
-  pdl(k_adj_clear, dim3(fb[F_ACLR].total_blocks), dim3(256), 0, st, fb[F_ACLR], p->d_subs, p->d_ws);
+  pdl(k_adj_clear, dim3(fb[F_ACLR].total_blocks), dim3(256), 0, st, fb[F_ACLR], subs_of(p, rec), p->d_ws);
   return cudaGetLastError();
 }
 

@@ -502,7 +502,7 @@ struct mdp_plan {
   std::vector<mdp::Wave> sched[3];
   std::vector<int> leader;               // per subdomain: the subdomain whose tables and basis columns it shares
   // device side
-  mdp::SubDesc *d_subs = nullptr;
+  mdp::SubDesc *d_subs = nullptr;        // the subdomains, then the same without receiver rows (subs_of)
   double *d_tables = nullptr;
   uint8_t *d_piv = nullptr;
   unsigned char *d_sep = nullptr;        // separable tables (kernels_sep.cu), rebuilt with the factor tables
@@ -538,7 +538,7 @@ struct mdp_plan {
   // per schedule and wave: device items and prefix arrays (one prefix array per kernel family)
   std::vector<mdp::Item *> d_items[3];
   std::vector<int *> d_order[3];         // [wave] -> device int [k_tri + k_adj_tri blocks]: launch orders
-  std::vector<int *> d_prefix[3];        // [wave] -> device int [NFAM][n_items + 1]
+  std::vector<int *> d_prefix[3];        // [wave] -> device int [2][NFAM][n_items + 1]: without, with receiver rows
   std::vector<std::vector<int>> h_prefix[3];
   // CUDA graphs of mdp_project_batch, keyed by (xi, out, kind, stream, table set)
   struct GraphEntry {
@@ -565,6 +565,19 @@ inline void set_bounds(const mdp_plan *p, Batch &b, long long out_n, bool grad) 
   b.piv_n = (long long)p->host_piv.size();
   b.out_n = out_n;
   b.status = p->d_status;
+}
+
+// Device descriptors of a call: with the receiver rows where it reads or writes their values, else without, so that
+// such a call does no work for them and one captured before a change of the rows stays what it was.
+inline const SubDesc *subs_of(const mdp_plan *p, bool rec) { return p->d_subs + (rec ? 0 : p->n_subs); }
+inline SubDesc without_rec(SubDesc d) {
+  d.nrec = -1;
+  d.rec_off = 0;
+  return d;
+}
+// the descriptors of d_subs, 2 n_subs of them
+inline void fill_subs(const mdp_plan *p, SubDesc *s) {
+  for (int i = 0; i < p->n_subs; ++i) { s[i] = p->subs[i].d; s[p->n_subs + i] = without_rec(s[i]); }
 }
 
 // kernel families (each has its own block decomposition of an item). F_A* are the adjoint's. F_RING (basis
@@ -737,8 +750,9 @@ cudaError_t launch_sep_project(mdp_plan *p, const Batch *fb, int out_kind, const
 // ones; the separable gradient pass of a wave (forward: with the k-gradient)
 cudaError_t launch_adj_tables(const mdp_plan *p, cudaStream_t st);
 cudaError_t launch_adj_sines(const mdp_plan *p, cudaStream_t st);
-cudaError_t launch_adj_clear(mdp_plan *p, const Batch *fb, cudaStream_t st);
-cudaError_t launch_sep_adj_residual(mdp_plan *p, const Batch *fb, bool user, cudaStream_t st);
+// (rec: with the receivers' cotangent, see subs_of)
+cudaError_t launch_adj_clear(mdp_plan *p, const Batch *fb, bool rec, cudaStream_t st);
+cudaError_t launch_sep_adj_residual(mdp_plan *p, const Batch *fb, bool user, bool rec, cudaStream_t st);
 cudaError_t launch_sep_adjoint(mdp_plan *p, const Batch *fb, bool user, bool dk, const double2 *cot, const double2 *cot_rec,
                                cudaStream_t st);
 cudaError_t launch_sep_cut1(const Batch &b, const SubDesc *subs, double *ws, bool user, int fam, cudaStream_t st);

@@ -215,3 +215,28 @@ def test_deduplicated_subdomains_have_receiver_rows_of_their_own(mdp, rows, off)
             got.append(res)
         for a, r in zip(*got):
             assert (a - r).abs().max() <= 1e-12 * r.abs().max()
+
+
+@pytest.mark.parametrize("fp64", [False, True])
+def test_captured_calls_without_receivers_outlive_a_change_of_the_rows(mdp, fp64):
+    """Projection and gradient captured without receivers, replayed after set_receivers: bit for bit the values
+    before, as are plain calls without receiver arguments."""
+    subs = [W.unit_subdomain(i, 0, n, 7.0 + i, W.AP_DIRX_SOMMY, 3) for i, n in enumerate((33, 45, 33))]
+    plan = mdp.Plan(subs, fp64_cols=fp64)
+    cot = torch.from_numpy(W.random_complex(plan.output_size, seed=19)).cuda()
+    ref = [plan.project().clone(), *plan.adjoint(cot)]
+    g, s = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        g.capture_begin()
+        out = [plan.project(), *plan.adjoint(cot)]
+        g.capture_end()
+    for rows in ([-1, 20, -1], [16, 20, 16], [-1, -1, -1]):
+        plan.set_receivers(rows)
+        for t in out:
+            t.zero_()
+        torch.cuda.synchronize()
+        g.replay()
+        torch.cuda.synchronize()
+        for a, b, r in zip(out, [plan.project(), *plan.adjoint(cot)], ref):
+            assert torch.equal(a, r) and torch.equal(b, r)
+    plan.status()
