@@ -7,9 +7,11 @@
 //   - factor rows (l, 1/d, du/d, du2/d), the swap flags and dT_q/dk rows (gradient pass,
 //     full-grid solves), with the run of exactly-real rows around the middle row;
 //   - the condensed, pivot-scaled forward-sweep rows of the projection (rows above the ring
-//     folded into the last pivot by their Schur complement), with its run of real rows; only for
+//     folded into the last pivot by their Schur complement), with its run of real rows; stored only for
 //     subdomains that project by sweeps (without the separable solve), or when `all` is set (table
-//     introspection).
+//     introspection). Its pivots are looked at for every subdomain: close to an eigenvalue they fall below the
+//     tolerance where the full factors' may not (the last pivot is the distance over the square of
+//     the eigenvector's last entry, small next to a Dirichlet end), and plan creation refuses by both.
 // The host plan builds the same tables at plan creation (plan.cpp: mode_matrix, band_lu,
 // factor_mode, build_fs_mode). Two kernels:
 //   k_factor_chain  the pivot recurrences, the only sequential part: one thread per (mode,
@@ -248,8 +250,8 @@ __device__ void chain_full(const SubDesc &d, int q, double *tab, uint8_t *piv, i
 
 // Chain of the condensed system (rows 0..itop, the rows above folded into the last pivot):
 // raw rows i >= i0 in the sweep table: l, d, 1/d, du, du2 (complex pairs) and the swap flag;
-// seg[4] = itop.
-__device__ void chain_sweep(const SubDesc &d, int q, double *tab, int *status, bool settles) {
+// seg[4] = itop. Without `store` only the pivots are checked.
+__device__ void chain_sweep(const SubDesc &d, int q, double *tab, int *status, bool settles, bool store) {
   const ModeRows M = mode_rows(d, q);
   const int N = M.N;
   const double scale2 = M.scale2();
@@ -279,7 +281,7 @@ __device__ void chain_sweep(const SubDesc &d, int q, double *tab, int *status, b
   double *T = tab + d.fs_off + (long long)(q - 1) * d.NYf * FSW;
   lu_chain(M, itop + 1, itop, sigma, tol2, status, settles,
            [&](int i, cplx l, cplx dg, cplx dinv, cplx du, cplx du2, uint8_t sw) {
-             if (i < d.i0) return;
+             if (i < d.i0 || !store) return;
              double *r = T + (long long)(i - d.i0) * FSW;
              st2(r, l); st2(r + 2, dg); st2(r + 4, dinv); st2(r + 6, du); st2(r + 8, du2);
              r[22] = sw;
@@ -304,9 +306,8 @@ __global__ void __launch_bounds__(32) k_factor_chain(const SubDesc *subs, int n_
   }
   if (si >= n_subs) return;
   const int q = prop ? t + 1 : subs[si].n_prop + t + 1;
-  if (sweep) {
-    if (all || !subs[si].tc_cols) chain_sweep(subs[si], q, tab, status, !prop);
-  } else chain_full(subs[si], q, tab, piv, status, !prop);
+  if (sweep) chain_sweep(subs[si], q, tab, status, !prop, all || !subs[si].tc_cols);
+  else chain_full(subs[si], q, tab, piv, status, !prop);
 }
 
 constexpr int kRowsThreads = 256;
@@ -451,13 +452,11 @@ __global__ void k_probe_rcp(const double *x, double *y, int n) {
 cudaError_t launch_factor_to(const mdp_plan *p, const SubDesc *ds, double *tab, uint8_t *piv, int *status, bool all,
                              cudaStream_t st) {
   int n_modes = 0, n_prop = 0;
-  bool sweeps = all;
   for (size_t i = 0; i < p->subs.size(); ++i) {
-    sweeps = sweeps || !p->subs[i].d.tc_cols;
     if (p->subs[i].d.leader == (int)i) { n_modes += p->subs[i].d.Nq; n_prop += p->subs[i].d.n_prop; }
   }
   const int blocks = n_prop + (n_modes - n_prop + 31) / 32;
-  k_factor_chain<<<sweeps ? 2 * blocks : blocks, 32, 0, st>>>(ds, (int)p->subs.size(), n_prop, n_modes - n_prop, tab, piv, status, all);
+  k_factor_chain<<<2 * blocks, 32, 0, st>>>(ds, (int)p->subs.size(), n_prop, n_modes - n_prop, tab, piv, status, all);
   k_factor_rows<<<n_modes, kRowsThreads, 0, st>>>(ds, (int)p->subs.size(), tab, all);
   return cudaGetLastError();
 }

@@ -240,3 +240,22 @@ def test_captured_calls_without_receivers_outlive_a_change_of_the_rows(mdp, fp64
         for a, b, r in zip(out, [plan.project(), *plan.adjoint(cot)], ref):
             assert torch.equal(a, r) and torch.equal(b, r)
     plan.status()
+
+
+@pytest.mark.parametrize("n,q,p", [(65, 1, 61), (65, 61, 1), (129, 1, 1), (129, 51, 121), (129, 81, 121), (129, 101, 111),
+                                   (257, 1, 1), (257, 43, 253), (257, 190, 22), (257, 253, 1)])
+def test_update_refuses_the_wavenumbers_that_plan_creation_refuses(mdp, n, q, p):
+    """Discrete Dirichlet eigenvalues whose eigenvector is small at the ends: the pivots of the full factors
+    stay above the tolerance, those of the system without the rows above the ring do not."""
+    from paper_2103_12172_gb300 import MdpError
+    lq, lp = (-4 * np.sin(np.pi * m / (2 * (n - 1))) ** 2 for m in (q, p))
+    k = float(np.sqrt(-((lq + lp * (1 + lq / 6)) / (1.2 / (n - 1)) ** 2) / (1 + lq / 12 + lp / 12)))
+    sub = W.small_subdomain(n, 9.0, W.AP_DIRICHLET4, 1)
+    for plan in (mdp.Plan([sub]), mdp.Plan([sub], fp64_cols=True)):
+        with pytest.raises(MdpError) as e:
+            plan.update_k([k])
+        assert e.value.code == 4   # MDP_ERR_SINGULAR
+        plan.update_k([9.0])
+    with pytest.raises(MdpError) as e:
+        mdp.Plan([sub.with_k(k)], host_only=True)
+    assert e.value.code == 4
