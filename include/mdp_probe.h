@@ -39,8 +39,8 @@ const char *mdp_kernel_family_name(int family);
  * number of factor rows with complex entries swept by the projection, over all modes. */
 mdp_status mdp_plan_sub_info(const mdp_plan *p, int sub, int *info14);
 
-/* Bytes of the plan's tables (factors, sweep tables, sines, geometry, pivot flags), uploaded at
- * plan creation and rebuilt on the device by mdp_plan_update_k. */
+/* Bytes of the plan's tables: factors, sweep tables, sines, geometry, pivot flags, and on a device plan those of the
+ * separable solve and of its gradient pass (a second set of mdp_plan_update_k_async not counted). */
 long long mdp_plan_table_bytes(const mdp_plan *p);
 
 /* Bytes that mdp_plan_update_k copies host -> device on a device plan (the subdomain

@@ -98,12 +98,16 @@ mdp_status alloc_device(mdp_plan *p) {
   auto al = [&](void **ptr, size_t bytes) -> bool { return cudaMalloc(ptr, std::max<size_t>(bytes, 256)) == cudaSuccess; };
   if (!al((void **)&p->d_subs, 2 * p->subs.size() * sizeof(SubDesc)) ||
       !al((void **)&p->d_tables, p->n_tables * sizeof(double)) ||
-      !al((void **)&p->d_piv, p->host_piv.size()) || !al((void **)&p->d_sep, (size_t)p->sep_bytes) || !al((void **)&p->d_ws, (size_t)p->ws_doubles * 8) ||
+      !al((void **)&p->d_piv, p->host_piv.size()) || !al((void **)&p->d_sep, (size_t)p->sep_bytes) ||
+      !al((void **)&p->d_adj, (size_t)p->adj_bytes) || !al((void **)&p->d_ws, (size_t)p->ws_doubles * 8) ||
       !al((void **)&p->d_status, sizeof(int)) || !al((void **)&p->d_fstatus, sizeof(int)) ||
       !p->sub_stage.alloc(2 * p->subs.size(), true) || !p->h_fstatus.alloc(1, true))
     return MDP_ERR_NOMEM;
   CK(cudaMemset(p->d_status, 0, sizeof(int)));
   CK(cudaMemset(p->d_fstatus, 0, sizeof(int)));
+  CK(cudaStreamCreateWithFlags(&p->side, cudaStreamNonBlocking));
+  CK(cudaEventCreateWithFlags(&p->fork_ev, cudaEventDisableTiming));
+  CK(cudaEventCreateWithFlags(&p->join_ev, cudaEventDisableTiming));
   for (auto &hs : p->subs) hs.d.dstatus = p->d_status;
 #if MDP_CHECKED
   // fault injection (bounds-checked build only): MDP_FAULT_INJECT=factor scales one row of the
@@ -244,9 +248,6 @@ cudaError_t end_use(mdp_plan *p, cudaStream_t st) {
 cudaError_t launch_update(mdp_plan *p, const SubDesc *ds, double *tab, uint8_t *piv, unsigned char *sep, int *status,
                           cudaStream_t s) {
   cudaError_t e;
-  if (!p->side && ((e = cudaStreamCreateWithFlags(&p->side, cudaStreamNonBlocking)) != cudaSuccess)) return e;
-  if (!p->fork_ev && (e = cudaEventCreateWithFlags(&p->fork_ev, cudaEventDisableTiming)) != cudaSuccess) return e;
-  if (!p->join_ev && (e = cudaEventCreateWithFlags(&p->join_ev, cudaEventDisableTiming)) != cudaSuccess) return e;
   if ((e = cudaEventRecord(p->fork_ev, s)) != cudaSuccess) return e;
   if ((e = cudaStreamWaitEvent(p->side, p->fork_ev, 0)) != cudaSuccess) return e;
   const cudaError_t ef = launch_factor_to(p, ds, tab, piv, status, false, p->side);
@@ -256,25 +257,15 @@ cudaError_t launch_update(mdp_plan *p, const SubDesc *ds, double *tab, uint8_t *
   return ef != cudaSuccess ? ef : es;
 }
 
-// The gradient tables follow the wavenumbers only where a gradient is asked for: allocated by the first such
+// The gradient tables follow the wavenumbers only where a gradient is asked for: made by the first such
 // call, rebuilt by the first after a change. In a capture they are always rebuilt, so that a replay
-// follows the tables that it finds (and the allocation is no stream operation); from then on every call rebuilds
-// them, as a replay may have left those of another table set.
+// follows the tables that it finds; from then on every call rebuilds them, as a replay may have left those of
+// another table set.
 cudaError_t ensure_adj_tables(mdp_plan *p, cudaStream_t st) {
   if (p->adj_bytes == 0) return cudaSuccess;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   cudaError_t e = cudaStreamIsCapturing(st, &cap);
   if (e != cudaSuccess) return e;
-  if (!p->d_adj) {
-    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-    e = cudaThreadExchangeStreamCaptureMode(&mode);
-    if (e != cudaSuccess) return e;
-    const cudaError_t m = cudaMalloc((void **)&p->d_adj, (size_t)p->adj_bytes);
-    e = cudaThreadExchangeStreamCaptureMode(&mode);
-    if (m != cudaSuccess || e != cudaSuccess) return m != cudaSuccess ? m : e;
-    p->adj_sines = false;
-    p->adj_stale = true;
-  }
   const bool live = cap == cudaStreamCaptureStatusNone;
   if (!live) p->adj_captured = true;
   if (!p->adj_sines || !live) {
@@ -677,9 +668,7 @@ mdp_status mdp_ap_adjoint_rec(mdp_plan *p, const mdp_c64 *xi, const mdp_c64 *cot
   CK(cudaSetDevice(p->device));
   cudaStream_t st = (cudaStream_t)cuda_stream;
   CK(begin_use(p, st));
-  const cudaError_t te = ensure_adj_tables(p, st);
-  if (te == cudaErrorMemoryAllocation) { cudaGetLastError(); return MDP_ERR_NOMEM; }
-  CK(te);
+  CK(ensure_adj_tables(p, st));
   for (size_t w = 0; w < p->sched[S_GRAD].size(); ++w) {
     Batch fb[NFAM];
     wave_batches(p, w, fb, S_GRAD, cot_rec != nullptr);
@@ -825,7 +814,7 @@ mdp_status mdp_plan_receiver_layout(const mdp_plan *p, int sub, int *row, int *m
 long long mdp_plan_receiver_size(const mdp_plan *p) { return p ? p->rec_size : 0; }
 
 long long mdp_plan_table_bytes(const mdp_plan *p) {
-  return p ? (long long)(p->n_tables * sizeof(double) + p->host_piv.size()) : 0;
+  return p ? (long long)(p->n_tables * sizeof(double) + p->host_piv.size()) + (device_ok(p) ? p->sep_bytes + p->adj_bytes : 0) : 0;
 }
 
 int mdp_kernel_family_count(void) { return NFAM; }

@@ -144,3 +144,29 @@ def test_plan_variants_agree_and_the_tuner_picks_one(mdp, tmp_path):
     assert plan_kwargs(tune_plan(subs, tiles=(16, 64), cache_path=path)) == plan_kwargs(t)
     got = mdp.Plan(subs, **plan_kwargs(t)).project().cpu().numpy()
     assert np.abs(got - ref).max() <= 1e-12 * np.abs(ref).max()
+
+
+def test_compute_calls_allocate_nothing(mdp):
+    """Device memory is taken by plan creation alone: the free memory stays what it was through the first calls
+    of every kind on a new plan (the kernels and torch's pool warmed by another one), and a device plan's table
+    bytes count more than the host's."""
+    subs = [W.unit_subdomain(i, 0, 129, 9.0 + i, W.AP_DIRX_SOMMY, 8) for i in range(2)]
+
+    def calls(plan):
+        cot = torch.ones(plan.output_size, dtype=torch.complex128, device="cuda")
+        plan.update_k([9.5, 10.5])
+        out = plan.project()
+        gx, gk = plan.adjoint(cot, xi=out)
+        u = plan.solve(0, torch.ones((2, 129, 129), dtype=torch.complex128, device="cuda"))
+        torch.cuda.synchronize()
+        return out, gx, gk, u
+
+    warm = mdp.Plan(subs)
+    calls(warm)
+    plan = mdp.Plan(subs)
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    calls(plan)
+    assert torch.cuda.mem_get_info()[0] == free
+    host = mdp.Plan(subs, host_only=True)
+    assert plan.L.mdp_plan_table_bytes(plan.handle) > host.L.mdp_plan_table_bytes(host.handle)
