@@ -24,6 +24,21 @@ long long env_ll(const char *name, long long dflt) {
   return std::atoll(v);
 }
 
+void free_alt(mdp_plan *p) {
+  cudaFree(p->alt_subs);
+  cudaFree(p->alt_tables);
+  cudaFree(p->alt_piv);
+  cudaFree(p->alt_sep);
+  p->alt_subs = nullptr; p->alt_tables = nullptr; p->alt_piv = nullptr; p->alt_sep = nullptr;
+  p->alt_stage.release();
+  for (int s = 0; s < 2; ++s) {
+    if (p->ready_ev[s]) cudaEventDestroy(p->ready_ev[s]);
+    if (p->used_ev[s]) cudaEventDestroy(p->used_ev[s]);
+    p->ready_ev[s] = p->used_ev[s] = nullptr;
+    p->used_rec[s] = false;
+  }
+}
+
 void free_device(mdp_plan *p) {
   if (p->device < 0) return;
   int prev = -1;
@@ -33,31 +48,20 @@ void free_device(mdp_plan *p) {
   cudaFree(p->d_tables);
   cudaFree(p->d_piv);
   cudaFree(p->d_sep);
-  cudaFree(p->alt_sep);
   cudaFree(p->d_adj);
   p->d_adj = nullptr;
   if (p->side) cudaStreamDestroy(p->side);
   if (p->fork_ev) cudaEventDestroy(p->fork_ev);
   if (p->join_ev) cudaEventDestroy(p->join_ev);
   p->side = nullptr; p->fork_ev = p->join_ev = nullptr;
-  p->d_sep = p->alt_sep = nullptr;
+  p->d_sep = nullptr;
   cudaFree(p->d_ws);
   cudaFree(p->d_status);
   cudaFree(p->d_fstatus);
   p->d_fstatus = nullptr;
   p->sub_stage.release();
   p->h_fstatus.release();
-  cudaFree(p->alt_subs);
-  cudaFree(p->alt_tables);
-  cudaFree(p->alt_piv);
-  p->alt_subs = nullptr; p->alt_tables = nullptr; p->alt_piv = nullptr;
-  p->alt_stage.release();
-  for (int s_ = 0; s_ < 2; ++s_) {
-    if (p->ready_ev[s_]) cudaEventDestroy(p->ready_ev[s_]);
-    if (p->used_ev[s_]) cudaEventDestroy(p->used_ev[s_]);
-    p->ready_ev[s_] = p->used_ev[s_] = nullptr;
-    p->used_rec[s_] = false;
-  }
+  free_alt(p);
   for (int k = 0; k < 3; ++k) {
     for (auto x : p->d_items[k]) cudaFree(x);
     for (auto x : p->d_prefix[k]) cudaFree(x);
@@ -399,31 +403,51 @@ mdp_status mdp_plan_update_k_stream(mdp_plan *p, const double *k, void *cuda_str
   return (mdp_status)p->h_fstatus[0];
 }
 
+// The second table set, all of it or (MDP_ERR_NOMEM, MDP_ERR_CUDA) nothing: a later call may try again.
+static mdp_status alloc_alt(mdp_plan *p) {
+  const size_t nt = std::max<size_t>(p->n_tables * sizeof(double), 256);
+  const size_t np = std::max<size_t>(p->host_piv.size(), 256);
+  const size_t ns = std::max<size_t>(2 * p->subs.size() * sizeof(SubDesc), 256);
+  bool ok = cudaMalloc((void **)&p->alt_tables, nt) == cudaSuccess && cudaMalloc((void **)&p->alt_piv, np) == cudaSuccess &&
+            cudaMalloc((void **)&p->alt_subs, ns) == cudaSuccess && p->alt_stage.alloc(2 * p->subs.size(), true);
+#if MDP_CHECKED
+  const char *fault = std::getenv("MDP_FAULT_INJECT");   // "alt": the last allocation fails
+  ok = ok && !(fault && !std::strcmp(fault, "alt"));
+#endif
+  ok = ok && cudaMalloc((void **)&p->alt_sep, std::max<size_t>((size_t)p->sep_bytes, 256)) == cudaSuccess;
+  mdp_status st = ok ? MDP_OK : MDP_ERR_NOMEM;
+  auto run = [&](cudaError_t e) { if (st == MDP_OK && e != cudaSuccess) st = MDP_ERR_CUDA; };
+  for (int s = 0; s < 2 && st == MDP_OK; ++s) {
+    run(cudaEventCreateWithFlags(&p->ready_ev[s], cudaEventDisableTiming));
+    run(cudaEventCreateWithFlags(&p->used_ev[s], cudaEventDisableTiming));
+  }
+  if (st == MDP_OK) {   // it starts as a copy of the first (k-independent tables)
+    run(cudaDeviceSynchronize());
+    run(cudaMemcpy(p->alt_tables, p->d_tables, nt, cudaMemcpyDeviceToDevice));
+    run(cudaMemcpy(p->alt_piv, p->d_piv, np, cudaMemcpyDeviceToDevice));
+    run(launch_sep_sines(p, p->d_subs, p->d_tables, p->alt_sep, nullptr));
+    run(cudaStreamSynchronize(nullptr));
+  }
+  if (st != MDP_OK) {
+    free_alt(p);
+    cudaGetLastError();
+  }
+  return st;
+}
+
 // The refactorisation into the other table set, then the sets swap roles (see include/mdp.h).
 mdp_status mdp_plan_update_k_async(mdp_plan *p, const double *k, void *cuda_stream) {
   if (!p || !k) return MDP_ERR_ARG;
   if (!device_ok(p)) return refactor_host(p, k);
+  std::vector<double> before;
+  for (auto &hs : p->subs) before.push_back(hs.d.k);
   mdp_status st = set_k_fields(p, k);
   if (st != MDP_OK) return st;
   CK(cudaSetDevice(p->device));
   cudaStream_t s = (cudaStream_t)cuda_stream;
-  if (!p->alt_tables) {   // first call: the second set starts as a copy of the first (k-independent tables)
-    const size_t nt = std::max<size_t>(p->n_tables * sizeof(double), 256);
-    const size_t np = std::max<size_t>(p->host_piv.size(), 256);
-    const size_t ns = std::max<size_t>(2 * p->subs.size() * sizeof(SubDesc), 256);
-    if (cudaMalloc((void **)&p->alt_tables, nt) != cudaSuccess || cudaMalloc((void **)&p->alt_piv, np) != cudaSuccess ||
-        cudaMalloc((void **)&p->alt_sep, std::max<size_t>((size_t)p->sep_bytes, 256)) != cudaSuccess ||
-        cudaMalloc((void **)&p->alt_subs, ns) != cudaSuccess || !p->alt_stage.alloc(2 * p->subs.size(), true))
-      return MDP_ERR_NOMEM;
-    for (int s_ = 0; s_ < 2; ++s_) {
-      CK(cudaEventCreateWithFlags(&p->ready_ev[s_], cudaEventDisableTiming));
-      CK(cudaEventCreateWithFlags(&p->used_ev[s_], cudaEventDisableTiming));
-    }
-    CK(cudaDeviceSynchronize());
-    CK(cudaMemcpy(p->alt_tables, p->d_tables, nt, cudaMemcpyDeviceToDevice));
-    CK(cudaMemcpy(p->alt_piv, p->d_piv, np, cudaMemcpyDeviceToDevice));
-    CK(launch_sep_sines(p, p->d_subs, p->d_tables, p->alt_sep, nullptr));
-    CK(cudaStreamSynchronize(nullptr));
+  if (!p->alt_tables && (st = alloc_alt(p)) != MDP_OK) {
+    set_k_fields(p, before.data());   // the descriptors keep naming the tables in use
+    return st;
   }
   const int b = 1 - p->set;
   HostBuf<SubDesc> &stage = stage_of(p, b);

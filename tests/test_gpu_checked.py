@@ -102,3 +102,42 @@ def test_checked_build_parity_races_and_fault_injection():
     r = subprocess.run([sys.executable, "-c", CHILD, ROOT], env=env, capture_output=True, text=True, timeout=900)
     assert r.returncode == 0, r.stdout[-3000:] + r.stderr[-3000:]
     assert "checked build ok" in r.stdout
+
+
+ALT = r'''
+import os, sys
+import torch
+sys.path.insert(0, sys.argv[1])
+import workloads as W
+import paper_2103_12172_gb300 as mdp
+from paper_2103_12172_gb300 import _lib, MdpError
+sub = W.small_subdomain(65, 9.0, W.AP_DIRX_SOMMY, 2)
+plan, ref = mdp.Plan([sub]), mdp.Plan([sub])
+os.environ["MDP_FAULT_INJECT"] = "alt"
+for _ in range(2):
+    try:
+        plan.update_k_async([9.5])
+        raise SystemExit("the failed allocation was not reported")
+    except MdpError as e:
+        assert e.code == _lib.MDP_ERR_NOMEM, e.code
+del os.environ["MDP_FAULT_INJECT"]
+for k in (9.5, 10.0, 9.0):
+    plan.update_k_async([k])
+    ref.update_k([k])
+    assert torch.equal(plan.project(), ref.project())
+plan.status()
+print("second table set ok")
+'''
+
+
+@pytest.mark.gpu
+def test_a_second_table_set_that_does_not_fit_is_tried_again():
+    """A failed allocation in the first mdp_plan_update_k_async (made to fail on the host) leaves nothing behind that
+    a later call takes for a table set."""
+    from paper_2103_12172_gb300 import _build
+    _build.build(checked=True)
+    env = dict(os.environ, MDP_LIB_CHECKED="1")
+    env.pop("MDP_FAULT_INJECT", None)
+    r = subprocess.run([sys.executable, "-c", ALT, ROOT], env=env, capture_output=True, text=True, timeout=600)
+    assert r.returncode == 0, r.stdout[-3000:] + r.stderr[-3000:]
+    assert "second table set ok" in r.stdout
