@@ -117,7 +117,8 @@ mdp_status alloc_device(mdp_plan *p) {
   // fault injection (bounds-checked build only): MDP_FAULT_INJECT=factor scales one row of the
   // first subdomain's factored sweep table (row 5 of mode 1, which every projection column goes
   // through: wrong numbers, which the parity check must catch), =desc points the first
-  // projection item's mode-space slice past the end of the workspace (the checks must catch it and
+  // projection item's mode-space slice past the end of the workspace, =table the synthesis table of the
+  // first subdomain past the end of the separable tables (the checks must catch it and
   // skip every access through it)
   const char *fault = std::getenv("MDP_FAULT_INJECT");
   if (fault && !std::strcmp(fault, "factor") && !p->subs.empty() && p->subs[0].d.NYf > 6 && p->subs[0].fs)
@@ -142,6 +143,9 @@ mdp_status alloc_device(mdp_plan *p) {
     for (double &v : row) v *= 1.5;
     CK(cudaMemcpy(p->d_sep + p->subs[0].d.sep_mt, row, sizeof row, cudaMemcpyHostToDevice));
   }
+  if (fault && !std::strcmp(fault, "table") && !p->subs.empty() && p->subs[0].d.tc_cols)   // after the tables are made
+    for (int v = 0; v < 2; ++v)
+      CK(cudaMemcpy(&p->d_subs[v * p->n_subs].sep_b3, &p->sep_bytes, sizeof p->sep_bytes, cudaMemcpyHostToDevice));
 #endif
   for (int sc = 0; sc < 3; ++sc) {
     auto &waves = p->sched[sc];

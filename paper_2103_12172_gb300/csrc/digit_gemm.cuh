@@ -81,6 +81,25 @@ struct DigitTile {
     }
     m[0] = a.x; m[1] = a.y; m[2] = a.z; m[3] = a.w; m[4] = b.x; m[5] = b.y; m[6] = b.z; m[7] = b.w;
   }
+  // bounds-checked build: nk groups of K, their blocks and the exponents inside the workspace and the tables
+  __device__ __noinline__ bool in_bounds(const double *ws, long long ws_n, const unsigned char *t0, long long n0,
+                                         const unsigned char *t1, long long n1, int nk, int *status) const {
+    auto in = [](const void *p, long long n, const void *lo, long long size) {
+      const long long o = (const char *)p - (const char *)lo;
+      return o >= 0 && n >= 0 && o + n <= size;
+    };
+    auto tab = [&](const unsigned char *p, long long n) { return in(p, n, t0, n0) || in(p, n, t1, n1); };
+    const long long blocks = nkj ? (long long)((nk + nkj - 1) / nkj) * ND : min(nk, k2);
+    bool ok = nk <= 32 * SEP_MASK && in(A, (long long)nk * SEP_ABLK, ws, 8 * ws_n) && in(ex, 128 * sizeof(int), ws, 8 * ws_n) &&
+              tab(B, blocks * SEP_BBLK) && (nk <= k2 || tab(B2, (long long)(nk - k2) * SEP_BBLK));
+#pragma unroll
+    for (int wd = 0; wd < SEP_MASK; ++wd) {
+      const int left = nk - 32 * wd;   // groups of this word
+      ok = ok && !(left <= 0 ? m[wd] : left < 32 ? m[wd] >> left : 0u);
+    }
+    if (!ok) flag_bounds(status);
+    return ok;
+  }
   __device__ __forceinline__ int groups() const {
     int n = 0;
 #pragma unroll
@@ -146,7 +165,7 @@ __device__ __forceinline__ double sum_to_double(long long hi, long long lo, int 
 }
 
 // Src: total() tiles, tile(v, t) fills tile v (false: skipped by every warp), dest(t, row, o, ...) says where
-// the 8 outputs from o on of a row go. One CTA of SG_THREADS threads per SM with SG_SMEM bytes.
+// the 8 outputs from o on of a row go, inside out_n() doubles from out(). One CTA of SG_THREADS threads per SM with SG_SMEM bytes.
 template <class Src>
 __device__ __forceinline__ void digit_gemm(const Src &src, int *status) {
   extern __shared__ unsigned char sg_raw[];
@@ -286,6 +305,10 @@ __device__ __forceinline__ void digit_gemm(const Src &src, int *status) {
       int cnt;                   // outputs of this thread (of 8), `step` doubles apart
       long long step;
       src.dest(t, row, 8 * part, dst, step, cnt);
+      if (MDP_CHECKED && cnt > 0) {
+        const long long o = dst - src.out();
+        if (o < 0 || o + (min(cnt, 8) - 1) * step >= src.out_n()) { flag_bounds(status); cnt = 0; }
+      }
       if (step == 1 && cnt >= 8) {
 #pragma unroll
         for (int o = 0; o < 8; o += 2)

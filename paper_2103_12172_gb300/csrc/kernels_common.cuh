@@ -80,6 +80,18 @@ static __device__ __noinline__ bool item_in_bounds(const Batch &bt, const SubDes
     ok = ok && in_tab(d.fact_off, qt * (d.cplx ? 8 : 4)) && in_tab(d.dT_off, qt * 6) && in_tab(d.sin_off, 4LL * d.Nx) &&
          in_tab(d.geo_off, 4LL * d.G) && in_tab(d.seg_off, 5LL * d.Nq) && in_tab(d.fs_off, (long long)d.Nq * d.NYf * FSW);
     ok = ok && d.piv_off >= 0 && d.piv_off + qt <= bt.piv_n;
+    // the separable solve: every table, and the operands' rows and groups of K against the slices made for them
+    sep_tables(d, [&](const long long &o, long long n, int) { ok = ok && o >= 0 && o + n <= bt.sep_n; });
+    adj_tables(d, [&](const long long &o, long long n, int) { ok = ok && o >= 0 && o + n <= bt.adj_n; });
+    if (ok && d.tc_cols) {
+      const SepGeo g = sep_geo(d);
+      const int R = 2 * sep_pad128(it.ncols), most[4] = {R, 4 * R, R, 5 * R}, amost[4] = {R, 5 * R, R, 4 * R};
+      for (int j = 0; j < 4; ++j) {
+        ok = ok && sep_rows(d, j, it.ncols, it.col0, true) <= most[j] && sep_rows(d, j, it.ncols, it.col0, false) <= most[j];
+        ok = ok && sep_nk(g, j) <= 32 * SEP_MASK;
+        if (grad) ok = ok && adj_rows(d, j, it.ncols) <= amost[j] && adj_nk(adj_geo(d, g), j) <= 32 * SEP_MASK;
+      }
+    }
     ok = ok && it.io_off >= 0 && it.io_off + (long long)it.ncols * d.G <= bt.out_n;
   }
   if (!ok) flag_bounds(bt.status);

@@ -69,13 +69,29 @@ struct FullArg {
   int nr;
   const unsigned char *sep;
   double *ws;
+  long long ws_n, sep_n;   // doubles of the workspace, bytes of the tables; for the bounds-checked build
 };
+// bounds-checked build: the slices of this pass are those of its right-hand sides and lie in the workspace, and
+// so do the tables
+static __device__ __noinline__ bool full_in_bounds(const FullArg &p) {
+  const FullWs r = full_ws(p.d, p.nr);
+  bool ok = p.nr >= 1 && r.total <= p.ws_n && p.w.rows == r.rows && p.w.R == r.R && p.w.ldf == r.ldf && p.w.ldu == r.ldu &&
+            p.w.a == r.a && p.w.ex == r.ex && p.w.mask == r.mask && p.w.f == r.f && p.w.u == r.u;
+  sep_tables(p.d, [&](const long long &o, long long n, int) { ok = ok && o >= 0 && o + n <= p.sep_n; });
+  if (!ok) flag_bounds(p.d.dstatus);
+  return ok;
+}
+#define MDP_CHECK_FULL(p)                                   \
+  do {                                                      \
+    if (MDP_CHECKED && !full_in_bounds(p)) return;          \
+  } while (0)
 
 // A: the grid's rows on folded columns (INV false: g(m) +- g(Nx - m)) or the modes (INV), cut into digits.
 // Row order (right-hand side, unknown row, part): a block's 8 rows are 4 grid rows, complex parts in turn.
 template <bool INV>
 __global__ void __launch_bounds__(256) k_full_cut(const __grid_constant__ FullArg p, const double2 *g) {
   pdl_wait();
+  MDP_CHECK_FULL(p);
   const SubDesc &d = p.d;
   const SepGeo &geo = p.g;
   const FullWs &w = p.w;
@@ -147,8 +163,10 @@ struct FullSrc {
     t.eb = INV ? inv_exp(p.d) : 0;
     t.masks(reinterpret_cast<const unsigned *>(p.ws + p.w.mask) + ((INV ? 2 * nm : 0) + tr) * SEP_MASK, nullptr);
     t.ex = reinterpret_cast<const int *>(p.ws + p.w.ex) + tr * 128;
-    return true;
+    return !MDP_CHECKED || t.in_bounds(p.ws, p.ws_n, p.sep, p.sep_n, p.sep, p.sep_n, nk, p.d.dstatus);
   }
+  __device__ __forceinline__ const double *out() const { return p.ws; }
+  __device__ __forceinline__ long long out_n() const { return p.ws_n; }
   __device__ __forceinline__ void dest(const Tile &t, int r, int o, double *&dst, long long &step, int &cnt) const {
     const int row = t.mt * 128 + r, o0 = t.nt * 32 + o;
     step = 1;
@@ -161,6 +179,7 @@ struct FullSrc {
 template <bool INV>
 __global__ void __launch_bounds__(SG_THREADS, 1) k_full_gemm(const __grid_constant__ FullArg p, int *status) {
   pdl_wait();
+  MDP_CHECK_FULL(p);
   const FullSrc<INV> src{p};
   digit_gemm(src, status);
 }
@@ -182,6 +201,7 @@ __device__ __forceinline__ double ipow(double x, int n) {
 constexpr int FULL_Y_CTAS = 4, FULL_Y_WARPS = 8;   // CTAs of a cluster, most warps of one
 __global__ void __cluster_dims__(1, 1, FULL_Y_CTAS) __launch_bounds__(32 * FULL_Y_WARPS) k_full_y(const __grid_constant__ FullArg p) {
   pdl_wait();
+  MDP_CHECK_FULL(p);
   extern __shared__ double ysh[];   // [2][warps][32] of this CTA, [2][all warps][32], then this CTA's rows [rows][32]
   const cg::cluster_group cl = cg::this_cluster();
   const SubDesc &d = p.d;
@@ -334,6 +354,7 @@ __global__ void __cluster_dims__(1, 1, FULL_Y_CTAS) __launch_bounds__(32 * FULL_
 // u(m) = U_0 + U_1, u(Nx - m) = U_0 - U_1 on the unknown rows, 0 on the Dirichlet ends.
 __global__ void __launch_bounds__(256) k_full_out(const __grid_constant__ FullArg p, double2 *u) {
   pdl_wait();
+  MDP_CHECK_FULL(p);
   const SubDesc &d = p.d;
   const FullWs &w = p.w;
   const double *ws = p.ws;
@@ -393,7 +414,11 @@ cudaError_t launch_full_solve(const mdp_plan *p, int sub, int nrhs, const double
     auto gemm_grid = [&](int nt) { return dim3((unsigned)std::min(p->n_sm, 2 * (w.R / 128) * nt)); };
     cudaError_t e = cudaMemsetAsync(p->d_ws + w.mask, 0, 2LL * (w.R / 128) * SEP_MASK * 8, st);
     if (e != cudaSuccess) return e;
-    const FullArg a{d, geo, w, nr, p->d_sep, p->d_ws};
+    FullArg a{d, geo, w, nr, p->d_sep, p->d_ws, p->ws_doubles, p->sep_bytes};
+#if MDP_CHECKED
+    const char *fault = std::getenv("MDP_FAULT_INJECT");   // "full": the mode space past the workspace's end
+    if (fault && !std::strcmp(fault, "full")) a.w.f = p->ws_doubles;
+#endif
     pdl(k_full_cut<false>, dim3(w.R / 8, 2), dim3(256), 0, st, a, gc);
     pdl(k_full_gemm<false>, dim3(gemm_grid(geo.nqh / 32)), dim3(SG_THREADS), SG_SMEM, st, a, p->d_status);
     pdl(k_full_y, dim3(w.ldf / 16, nr, FULL_Y_CTAS), dim3(32, nw), ysm, st, a);

@@ -560,8 +560,10 @@ struct SepSrc {
       mb = reinterpret_cast<const unsigned *>(sep + m.mask);
     }
     t.masks(ma, mb);
-    return true;
+    return !MDP_CHECKED || t.in_bounds(ws, bt.ws_n, sep, bt.sep_n, sep, bt.sep_n, nk, bt.status);
   }
+  __device__ __forceinline__ const double *out() const { return ws; }
+  __device__ __forceinline__ long long out_n() const { return bt.ws_n; }
   __device__ __forceinline__ void dest(const Tile &t, int r, int o, double *&dst, long long &step, int &cnt) const {
     const Item &it = t.it;
     const SubDesc &d = subs[it.sub];
@@ -748,7 +750,7 @@ __device__ __forceinline__ void sep_out_body(const Item &it, const SubDesc &d, c
 template <bool CD, bool CIN>
 __device__ __forceinline__ void sep_rows_out_body(const Item &it, const SubDesc &d, const double *tab, const double *ws,
                                                   const double2 *xi_user, double2 *out, double2 *out_rec, int kind, int b0,
-                                                  int slot, int mt, double2 (*sh)[32][33]) {
+                                                  int slot, int mt, double2 (*sh)[32][33], long long rec_n) {
   const SepGeo g = sep_geo(d);
   const int cp = sep_pad128(it.ncols), parts = CD ? 2 : 1, R = sep_rows(d, J_INV, it.ncols, it.col0, CIN);
   const double *ui = ws + it.a_off + sep_ws(d, it.ncols).ui;
@@ -777,12 +779,16 @@ __device__ __forceinline__ void sep_rows_out_body(const Item &it, const SubDesc 
       if (side == 1 && m == m1) continue;
       const double2 v = sh[side][threadIdx.x][k];
       if (slot == 4) {
-        if (out_rec && m >= d.mlo + 1 && m <= d.mhi - 1)
-          out_rec[d.rec_off + (long long)(it.col0 + b0 + k) * (d.Px - 2) + (m - d.mlo - 1)] = make_double2(-v.x, -v.y);
+        if (out_rec && m >= d.mlo + 1 && m <= d.mhi - 1) {
+          const long long o = d.rec_off + (long long)(it.col0 + b0 + k) * (d.Px - 2) + (m - d.mlo - 1);
+          if (MDP_CHECKED && (o < 0 || o >= rec_n)) { flag_bounds(d.dstatus); continue; }
+          out_rec[o] = make_double2(-v.x, -v.y);
+        }
         continue;
       }
       if (m < d.mlo - 1 || m > d.mhi + 1) continue;
       const int gi = gbase + m - (d.mlo - 1);
+      if (MDP_CHECKED && (gi < 0 || gi >= d.G)) { flag_bounds(d.dstatus); continue; }
       cplx r = cmk(-v.x, CD ? -v.y : 0.0);
       if (kind == MDP_OUT_P) r = cadd(r, density<CIN>(d, it, ws, tab, xi_user, b0 + k, gi));
       out[it.io_off + (long long)(b0 + k) * d.G + gi] = make_double2(r.re, r.im);
@@ -803,8 +809,8 @@ __global__ void __launch_bounds__(256) k_sep_out(Batch bt, const SubDesc *subs, 
     local -= nmid;
     const int t = local / cb, ntg = sep_geo(d).ntg;
     const int b0 = (local % cb) * 32;
-    if (d.cplx || CIN) sep_rows_out_body<true, CIN>(it, d, tab, ws, xi_user, out, out_rec, kind, b0, t / ntg, t % ntg, sh);
-    else sep_rows_out_body<false, CIN>(it, d, tab, ws, xi_user, out, out_rec, kind, b0, t / ntg, t % ntg, sh);
+    if (d.cplx || CIN) sep_rows_out_body<true, CIN>(it, d, tab, ws, xi_user, out, out_rec, kind, b0, t / ntg, t % ntg, sh, bt.rec_n);
+    else sep_rows_out_body<false, CIN>(it, d, tab, ws, xi_user, out, out_rec, kind, b0, t / ntg, t % ntg, sh, bt.rec_n);
     return;
   }
   const int b = (local % cb) * 32 + threadIdx.x, i = (local / cb) * 8 + threadIdx.y;

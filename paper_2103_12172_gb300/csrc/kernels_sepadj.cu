@@ -637,8 +637,10 @@ struct GradSrc {
       mb = reinterpret_cast<const unsigned *>(adj + m.mask);
     }
     t.masks(ma, mb);
-    return true;
+    return !MDP_CHECKED || t.in_bounds(ws, bt.ws_n, sep, bt.sep_n, adj, bt.adj_n, nk, bt.status);
   }
+  __device__ __forceinline__ const double *out() const { return ws; }
+  __device__ __forceinline__ long long out_n() const { return bt.ws_n; }
   __device__ __forceinline__ void dest(const Tile &t, int r, int o, double *&dst, long long &step, int &cnt) const {
     const Item &it = t.it;
     const SubDesc &d = subs[it.sub];
@@ -727,8 +729,10 @@ struct AdjSrc {
       mb = reinterpret_cast<const unsigned *>(adj + d.adj_zm) + m * SEP_MASK;
     }
     t.masks(ma, mb, mb2);
-    return true;
+    return !MDP_CHECKED || t.in_bounds(ws, bt.ws_n, adj, bt.adj_n, adj, bt.adj_n, nk, bt.status);
   }
+  __device__ __forceinline__ const double *out() const { return ws; }
+  __device__ __forceinline__ long long out_n() const { return bt.ws_n; }
   __device__ __forceinline__ void dest(const Tile &t, int r, int o, double *&dst, long long &step, int &cnt) const {
     const Item &it = t.it;
     const SubDesc &d = subs[it.sub];

@@ -115,10 +115,11 @@ struct Batch {
   Item one;
   // ranges the bounds-checked build validates every block's item against: subdomains, workspace
   // doubles, table doubles, pivot-flag bytes, and complex elements of the output / density /
-  // cotangent arrays of the call; the status word that records the first violation
+  // cotangent and receiver arrays of the call; the status word that records the first violation
   int n_subs;
   int grad;             // the items are laid out for the gradient pass
-  long long ws_n, tab_n, piv_n, out_n;
+  long long ws_n, tab_n, piv_n, out_n, rec_n;
+  long long sep_n, adj_n;   // bytes of the separable and the gradient tables
   int *status;
 };
 
@@ -194,6 +195,33 @@ inline __host__ __device__ SepGeo sep_geo(const SubDesc &d) {
 // mode number of entry qi of class e (past Nq: padding), of entry qi of parity e (0: odd modes)
 inline __host__ __device__ int sep_mode(const SubDesc &d, int e, int qi) { return d.xsym ? 2 * qi + 1 + e : qi + 1; }
 inline __host__ __device__ int sep_parity_mode(int e, int qi) { return 2 * qi + 1 + e; }
+// The separable tables of a subdomain: f(offset, bytes, class) for each, in a fixed order; class TAB_MASK: masks, at the
+// plan's first bytes, TAB_OWN: a duplicate has its own (else its leader's).
+enum { TAB_MASK = 1, TAB_OWN = 2 };
+template <class D, class F>
+inline __host__ __device__ void sep_tables(D &d, F f) {
+  if (d.tc_cols) {
+    const SepGeo g = sep_geo(d);
+    const long long n = g.nqp / 32, zw = 4LL * SEP_MASK * g.ncls, pairs = (long long)g.ncls * g.nS * g.nS;
+    f(d.sep_rz, zw * n, TAB_MASK | TAB_OWN);
+    f(d.sep_zm, zw * 2 * n, TAB_MASK);
+    f(d.sep_z3, zw * g.nt3, TAB_MASK);
+    f(d.sep_rb, g.ncls * n * g.nk1 * SEP_BBLK, TAB_OWN);
+    f(d.sep_kd, 8 * pairs * d.Py, 0);
+    f(d.sep_kde, 4LL * g.ncls * g.nS, 0);
+    f(d.sep_tb, pairs * g.ND * SEP_BBLK, 0);
+    f(d.sep_mb, g.ncls * 2 * n * g.nk1 * SEP_BBLK, 0);
+    f(d.sep_b3, (long long)g.ncls * g.nt3 * g.nk3 * SEP_BBLK, 0);
+    f(d.sep_bf, 2LL * (g.nqh / 32) * g.nkf * SEP_BBLK, 0);
+    f(d.sep_bi, 2LL * g.ntg * (g.nqh / 16) * SEP_BBLK, 0);
+    f(d.sep_xf, 2LL * (g.nqh / 32) * g.nkx * SEP_BBLK, 0);
+    f(d.sep_xi, 2LL * g.ntx * (g.nqh / 16) * SEP_BBLK, 0);
+  }
+  f(d.sep_ab, 16LL * d.Nq, 0);
+  f(d.sep_mt, 8LL * SEP_MTW * d.Nq, 0);
+  f(d.sep_mx, 8LL * SEP_MXW * d.Nq, 0);
+  f(d.sep_phi, 16LL * (d.Py + 2) * d.Nq, 0);
+}
 // bytes into the separable tables of the moments of 32 modes (output group `to` of class e): blocks of all groups
 // of K, mask; the first two blocks of nqp modes phi_1, phi_2, the third a receiver row's
 struct SepMoment { long long blocks, mask; };
@@ -356,6 +384,32 @@ inline __host__ __device__ AdjGeo adj_geo(const SubDesc &d, const SepGeo &g) {
   a.nkf = (g.Ng + 15) / 16;
   a.ntr = (g.Kf + 31) / 32;
   return a;
+}
+// the gradient tables, as sep_tables
+template <class D, class F>
+inline __host__ __device__ void adj_tables(D &d, F f) {
+  if (!d.tc_cols) return;
+  const SepGeo g = sep_geo(d);
+  const AdjGeo a = adj_geo(d, g);
+  const long long n = g.nqp / 32, zw = 4LL * SEP_MASK * g.ncls, pairs = (long long)g.ncls * g.nS * g.nS;
+  f(d.adj_rz, zw * n, TAB_MASK | TAB_OWN);
+  f(d.adj_r3z, zw * a.nt3, TAB_MASK | TAB_OWN);
+  f(d.adj_zm, zw * ADJ_MOM * n, TAB_MASK);
+  f(d.adj_z3, zw * a.nt3, TAB_MASK);
+  f(d.adj_zd, zw * 2 * n, TAB_MASK);
+  f(d.adj_rb, g.ncls * n * g.nk1 * SEP_BBLK, TAB_OWN);
+  f(d.adj_r3, g.ncls * a.nt3 * 2 * n * SEP_BBLK, TAB_OWN);
+  f(d.adj_md, 8LL * ADJ_MDW * d.Nq, 0);
+  f(d.adj_phid, 16LL * (d.Py + 2) * d.Nq, 0);
+  f(d.adj_kdd, 8 * pairs * d.Py, 0);
+  f(d.adj_kde, 8LL * g.ncls * g.nS, 0);
+  f(d.adj_tb, pairs * a.ND * SEP_BBLK, 0);
+  f(d.adj_mb, g.ncls * ADJ_MOM * n * a.nk1 * SEP_BBLK, 0);
+  f(d.adj_b3, g.ncls * a.nt3 * 4 * n * SEP_BBLK, 0);
+  f(d.adj_bf, 2LL * (g.nqh / 32) * a.nkf * SEP_BBLK, 0);
+  f(d.adj_bi, 2LL * a.ntr * (g.nqh / 16) * SEP_BBLK, 0);
+  f(d.adj_dtb, pairs * g.ND * SEP_BBLK, 0);
+  f(d.adj_dmb, g.ncls * 2 * n * g.nk1 * SEP_BBLK, 0);
 }
 // rows of A: the columns padded to 128, real and imaginary parts, times the rows transformed
 inline __host__ __device__ int adj_rows(const SubDesc &d, int job, int ncols) {
@@ -564,6 +618,9 @@ inline void set_bounds(const mdp_plan *p, Batch &b, long long out_n, bool grad) 
   b.tab_n = p->n_tables;
   b.piv_n = (long long)p->host_piv.size();
   b.out_n = out_n;
+  b.rec_n = p->rec_size;
+  b.sep_n = p->sep_bytes;
+  b.adj_n = p->adj_bytes;
   b.status = p->d_status;
 }
 

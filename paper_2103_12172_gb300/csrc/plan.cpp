@@ -419,79 +419,42 @@ bool bind_tables(mdp_plan *p, long long n, bool pinned) {
 static bool layout_tables(mdp_plan *p) {
   long long off = 0, poff = 0, out = 0, sep = 0;
   auto al = [](long long v) { return (v + 31) & ~31LL; };
-  auto take = [&](long long bytes) { const long long o = sep; sep += (bytes + 255) & ~255LL; return o; };
-  for (auto &hs : p->subs) {
-    SubDesc &d = hs.d;
-    if (!d.tc_cols) continue;
-    const SepGeo g = sep_geo(d);
-    d.sep_rz = take(4LL * SEP_MASK * g.ncls * (g.nqp / 32));
-    if (d.leader != (int)(&hs - p->subs.data())) continue;
-    d.sep_zm = take(4LL * SEP_MASK * g.ncls * (2 * g.nqp / 32));
-    d.sep_z3 = take(4LL * SEP_MASK * g.ncls * g.nt3);
-  }
-  p->sep_masks = sep;
   long long adj = 0;
-  auto take_adj = [&](long long bytes) { const long long o = adj; adj += (bytes + 255) & ~255LL; return o; };
-  for (auto &hs : p->subs) {
-    SubDesc &d = hs.d;
-    if (!d.tc_cols) continue;
-    const SepGeo g = sep_geo(d);
-    const AdjGeo a = adj_geo(d, g);
-    d.adj_rz = take_adj(4LL * SEP_MASK * g.ncls * (g.nqp / 32));
-    d.adj_r3z = take_adj(4LL * SEP_MASK * g.ncls * a.nt3);
-    if (d.leader != (int)(&hs - p->subs.data())) continue;
-    d.adj_zm = take_adj(4LL * SEP_MASK * g.ncls * (ADJ_MOM * g.nqp / 32));
-    d.adj_z3 = take_adj(4LL * SEP_MASK * g.ncls * a.nt3);
-    d.adj_zd = take_adj(4LL * SEP_MASK * g.ncls * (2 * g.nqp / 32));
-  }
-  p->adj_masks = adj;
-  for (auto &hs : p->subs) {
-    SubDesc &d = hs.d;
-    if (d.tc_cols) {   // the receiver row's tables, made where there is one
-      const SepGeo g = sep_geo(d);
-      d.sep_rb = take((long long)g.ncls * (g.nqp / 32) * g.nk1 * SEP_BBLK);
-      d.adj_rb = take_adj((long long)g.ncls * (g.nqp / 32) * g.nk1 * SEP_BBLK);
-      d.adj_r3 = take_adj((long long)g.ncls * adj_geo(d, g).nt3 * (g.nqp / 16) * SEP_BBLK);
+  auto is_leader = [&](const HostSub &hs) { return hs.d.leader == (int)(&hs - p->subs.data()); };
+  // the masks of all subdomains, then the other tables; a duplicate's own ones only
+  for (const int mask : {(int)TAB_MASK, 0}) {
+    for (auto &hs : p->subs) {
+      auto take = [&](long long &end) {
+        return [&](long long &o, long long bytes, int cls) {
+          if ((cls & TAB_MASK) != mask || !(is_leader(hs) || (cls & TAB_OWN))) return;
+          o = end;
+          end += (bytes + 255) & ~255LL;
+        };
+      };
+      sep_tables(hs.d, take(sep));
+      adj_tables(hs.d, take(adj));
     }
-    if (d.leader != (int)(&hs - p->subs.data())) {   // a duplicate: the leader's other tables
-      const SubDesc &ld = p->subs[d.leader].d;
+    if (mask) { p->sep_masks = sep; p->adj_masks = adj; }
+  }
+  for (auto &hs : p->subs) {
+    SubDesc &d = hs.d;
+    if (!is_leader(hs)) {   // a duplicate: the leader's other tables
+      SubDesc ld = p->subs[d.leader].d;
       d.fact_off = ld.fact_off; d.dT_off = ld.dT_off; d.sin_off = ld.sin_off; d.geo_off = ld.geo_off;
       d.seg_off = ld.seg_off; d.fs_off = ld.fs_off; d.piv_off = ld.piv_off;
-      d.sep_zm = ld.sep_zm; d.sep_z3 = ld.sep_z3; d.sep_ab = ld.sep_ab; d.sep_mt = ld.sep_mt; d.sep_phi = ld.sep_phi; d.sep_kd = ld.sep_kd; d.sep_kde = ld.sep_kde;
-      d.sep_tb = ld.sep_tb; d.sep_mb = ld.sep_mb; d.sep_b3 = ld.sep_b3; d.sep_bf = ld.sep_bf; d.sep_bi = ld.sep_bi; d.sep_xf = ld.sep_xf; d.sep_xi = ld.sep_xi; d.sep_mx = ld.sep_mx;
-      d.adj_zm = ld.adj_zm; d.adj_z3 = ld.adj_z3; d.adj_zd = ld.adj_zd; d.adj_md = ld.adj_md; d.adj_phid = ld.adj_phid; d.adj_kdd = ld.adj_kdd; d.adj_kde = ld.adj_kde;
-      d.adj_tb = ld.adj_tb; d.adj_mb = ld.adj_mb; d.adj_b3 = ld.adj_b3; d.adj_bf = ld.adj_bf; d.adj_bi = ld.adj_bi; d.adj_dtb = ld.adj_dtb; d.adj_dmb = ld.adj_dmb;
+      std::vector<long long> from;
+      auto get = [&](long long &o, long long, int) { from.push_back(o); };
+      sep_tables(ld, get);
+      adj_tables(ld, get);
+      size_t i = 0;
+      auto put = [&](long long &o, long long, int cls) {
+        if (!(cls & TAB_OWN)) o = from[i];
+        ++i;
+      };
+      sep_tables(d, put);
+      adj_tables(d, put);
       d.out_off = out;  out += (long long)d.G * d.n_cols;
       continue;
-    }
-    d.sep_ab = take(16LL * d.Nq);
-    d.sep_mt = take(8LL * SEP_MTW * d.Nq);
-    d.sep_mx = take(8LL * SEP_MXW * d.Nq);
-    d.sep_phi = take(16LL * (d.Py + 2) * d.Nq);
-    if (d.tc_cols) {
-      const SepGeo g = sep_geo(d);
-      const long long pairs = (long long)g.ncls * g.nS * g.nS;
-      d.sep_kd = take(8 * pairs * d.Py);
-      d.sep_kde = take(4LL * g.ncls * g.nS);
-      d.sep_tb = take(pairs * g.ND * SEP_BBLK);
-      d.sep_mb = take((long long)g.ncls * (2 * g.nqp / 32) * g.nk1 * SEP_BBLK);
-      d.sep_b3 = take((long long)g.ncls * g.nt3 * g.nk3 * SEP_BBLK);
-      d.sep_bf = take(2LL * (g.nqh / 32) * g.nkf * SEP_BBLK);
-      d.sep_bi = take(2LL * g.ntg * (g.nqh / 16) * SEP_BBLK);
-      d.sep_xf = take(2LL * (g.nqh / 32) * g.nkx * SEP_BBLK);
-      d.sep_xi = take(2LL * g.ntx * (g.nqh / 16) * SEP_BBLK);
-      const AdjGeo a = adj_geo(d, g);
-      d.adj_md = take_adj(8LL * ADJ_MDW * d.Nq);
-      d.adj_phid = take_adj(16LL * (d.Py + 2) * d.Nq);
-      d.adj_kdd = take_adj(8 * pairs * d.Py);
-      d.adj_kde = take_adj(8LL * g.ncls * g.nS);
-      d.adj_tb = take_adj(pairs * a.ND * SEP_BBLK);
-      d.adj_mb = take_adj((long long)g.ncls * (ADJ_MOM * g.nqp / 32) * a.nk1 * SEP_BBLK);
-      d.adj_b3 = take_adj((long long)g.ncls * a.nt3 * (2 * g.nqp / 16) * SEP_BBLK);
-      d.adj_bf = take_adj(2LL * (g.nqh / 32) * a.nkf * SEP_BBLK);
-      d.adj_bi = take_adj(2LL * a.ntr * (g.nqh / 16) * SEP_BBLK);
-      d.adj_dtb = take_adj(pairs * g.ND * SEP_BBLK);
-      d.adj_dmb = take_adj((long long)g.ncls * (2 * g.nqp / 32) * g.nk1 * SEP_BBLK);
     }
     const int FW = d.cplx ? 8 : 4;
     d.fact_off = off; off += al((long long)d.Nq * d.Nt * FW);

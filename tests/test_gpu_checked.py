@@ -141,3 +141,68 @@ def test_a_second_table_set_that_does_not_fit_is_tried_again():
     r = subprocess.run([sys.executable, "-c", ALT, ROOT], env=env, capture_output=True, text=True, timeout=600)
     assert r.returncode == 0, r.stdout[-3000:] + r.stderr[-3000:]
     assert "second table set ok" in r.stdout
+
+
+SEPARABLE = r'''
+import os, sys
+import numpy as np
+import torch
+sys.path.insert(0, sys.argv[1])
+import workloads as W
+import paper_2103_12172_gb300 as mdp
+from paper_2103_12172_gb300 import _lib, MdpError
+
+def refused(plan, what):
+    torch.cuda.synchronize()
+    try:
+        plan.status()
+    except MdpError as e:
+        assert e.code == _lib.MDP_ERR_BOUNDS, (what, e.code)
+        return
+    raise SystemExit(what + " not reported")
+
+# clean passes report nothing: ragged columns, receivers, duplicates, user densities, solves in passes
+subs = [W.unit_subdomain(i, 0, n, 7.0, W.AP_DIRX_SOMMY, 3) for i, n in enumerate((33, 65, 33))]
+for dedupe in (False, True):
+    plan = mdp.Plan(subs, tile_cols=7, dedupe=dedupe, workspace_bytes=1 << 20)
+    for rows in ([-1, 20, 9], [16, -1, 12]):
+        plan.set_receivers(rows)
+        out, rec = plan.project(out_rec=True)
+        plan.project(xi=out, kind="P")
+        for xi in (None, out):
+            plan.adjoint(out, xi=xi, cot_rec=rec)
+            plan.adjoint(out, xi=xi)
+    g = torch.from_numpy(W.random_complex((9, 65, 65), seed=3)).cuda()
+    u = plan.solve(1, g)
+    plan.potential(0, plan.basis_densities(0))
+    plan.status()
+# a table's offset past the end of the tables: every pass through it is skipped and reported
+os.environ["MDP_FAULT_INJECT"] = "table"
+bad = mdp.Plan([W.small_subdomain(65, 9.0, W.AP_DIRX_SOMMY, 2)])
+del os.environ["MDP_FAULT_INJECT"]
+bad.project()
+refused(bad, "projection")
+bad.adjoint(torch.ones(bad.output_size, dtype=torch.complex128, device="cuda"))
+refused(bad, "gradient")
+# a slice of a full-grid solve past the end of the workspace
+os.environ["MDP_FAULT_INJECT"] = "full"
+plan.solve(1, g)
+refused(plan, "solve")
+del os.environ["MDP_FAULT_INJECT"]
+assert torch.equal(plan.solve(1, g), u)
+plan.status()
+print("separable checks ok")
+'''
+
+
+@pytest.mark.gpu
+def test_checked_build_covers_the_separable_passes():
+    """The tables, operands and sums of the separable projection, gradient and full-grid solves: clean passes
+    report nothing, a table or a slice out of its range (corrupted on the host) is found and skipped."""
+    from paper_2103_12172_gb300 import _build
+    _build.build(checked=True)
+    env = dict(os.environ, MDP_LIB_CHECKED="1")
+    env.pop("MDP_FAULT_INJECT", None)
+    r = subprocess.run([sys.executable, "-c", SEPARABLE, ROOT], env=env, capture_output=True, text=True, timeout=600)
+    assert r.returncode == 0, r.stdout[-3000:] + r.stderr[-3000:]
+    assert "separable checks ok" in r.stdout
