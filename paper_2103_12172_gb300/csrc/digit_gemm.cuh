@@ -41,9 +41,9 @@ __device__ __forceinline__ double inv_scale(const SubDesc &d) { return (double)(
 // table value |x| <= 1 on the fixed scale 2^54
 __device__ __forceinline__ long long fix54(double x) { return __double2ll_rn(x * 0x1p54); }
 
-// round(x 2^(1076 - E)) for |x| < 2^(E - 1022), 53 <= E (nothing for E = 2047: Inf or NaN in the row), by
-// integer operations: the significand (53 bits) lies e - 1075 up, so it moves up one bit for e = E and
-// down E - e - 1 bits otherwise, rounded half up
+// round(x 2^(1076 - E)) for |x| < 2^(E - 1022), 1 <= E (nothing for E = 2047: Inf or NaN in the row), by
+// integer operations: the significand (53 bits) lies e - 1075 up (e = 1 for subnormal numbers), so it moves up one
+// bit for e = E and down E - e - 1 bits otherwise, rounded half up
 __device__ __forceinline__ long long fixed_of(double x, int E) {
   const long long b = __double_as_longlong(x);
   const int e = (int)((b >> 52) & 0x7ff);
@@ -156,9 +156,11 @@ __device__ __forceinline__ double sum_to_double(long long hi, long long lo, int 
   // the leading 64 bits of the 96, then 53 of them rounded
   unsigned long long top = lz <= 32 ? ((unsigned long long)l << lz) >> 32 : (unsigned long long)l << ((lz - 32) & 63);
   if (lz < 64) top |= (unsigned long long)h << lz;
-  const int e = 1023 + 95 - lz + ex;      // biased exponent
-  unsigned long long v = ((unsigned long long)(e - 1) << 52) + (top >> 11) + ((top >> 10) & 1);
-  if (lz == 96 || e < 1) v = 0;
+  const int e = 1023 + 95 - lz + ex;      // biased exponent; below 1 the result is subnormal and loses 1 - e bits more
+  const int sh = min(max(11 - e, 10), 63);
+  const unsigned long long t = top >> sh;
+  unsigned long long v = ((unsigned long long)max(e - 1, 0) << 52) + (t >> 1) + (t & 1);
+  if (lz == 96 || e < -52) v = 0;
   if (e > 2046) v = 0x7ff0000000000000ULL;
   if (ex == INT_MAX) v = 0x7ff8000000000000ULL;
   return __longlong_as_double((long long)(v | ((unsigned long long)neg << 63)));

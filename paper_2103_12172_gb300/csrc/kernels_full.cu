@@ -126,7 +126,7 @@ __global__ void __launch_bounds__(256) k_full_cut(const __grid_constant__ FullAr
   for (int off = 16; off >= 8; off >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, off));
   if ((threadIdx.x & 31) < 8) atomicMax(&emax[threadIdx.x & 7], m);
   __syncthreads();
-  const int E = max(emax[threadIdx.x & 7], 53), t = e * (w.R / 128) + row / 128;
+  const int E = max(emax[threadIdx.x & 7], 1), t = e * (w.R / 128) + row / 128;
   if (kl == 0) reinterpret_cast<int *>(ws + w.ex)[e * w.R + row] = E;
   unsigned char *A = reinterpret_cast<unsigned char *>(ws + w.a) + (long long)t * nk * SEP_ABLK;
   const int r = row & 127, off0 = (r >> 3) * 256 + (r & 7) * 16;

@@ -550,7 +550,7 @@ __device__ __forceinline__ void adj_cut_body(const Item &it, const SubDesc &d, d
   for (int off = 16; off >= 8; off >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, off));
   if ((threadIdx.x & 31) < 8) atomicMax(&emax[threadIdx.x & 7], m);
   __syncthreads();
-  const int E = max(emax[threadIdx.x & 7], 53), tr = e * (R / 128) + row / 128;
+  const int E = max(emax[threadIdx.x & 7], 1), tr = e * (R / 128) + row / 128;
   if (kl == 0) reinterpret_cast<int *>(ws + it.a_off + w.ex[JOB])[e * R + row] = E;
   unsigned char *A = reinterpret_cast<unsigned char *>(ws + it.a_off + w.a[JOB]) + (long long)tr * nk * SEP_ABLK;
   const int r = row & 127, off0 = (r >> 3) * 256 + (r & 7) * 16;

@@ -259,3 +259,30 @@ def test_update_refuses_the_wavenumbers_that_plan_creation_refuses(mdp, n, q, p)
     with pytest.raises(MdpError) as e:
         mdp.Plan([sub.with_k(k)], host_only=True)
     assert e.value.code == 4
+
+
+@pytest.mark.parametrize("power", [-1000, -1020, 960])
+@pytest.mark.parametrize("off", [0.0, 0.1])
+def test_densities_near_the_ends_of_the_exponents_range(mdp, power, off):
+    """Densities, cotangents and right-hand sides times a power of two that leaves the largest values in range: the
+    same results times that power. Bar: the rounding of what falls below 2^-1074, some hundred terms of it, and 1e-14
+    of a column's largest value."""
+    sub = box(49, 45, 9.0, W.AP_DIRX_SOMMY, 2, dx=off)
+    plan = mdp.Plan([sub])
+    G, nc, _, _ = plan.layout(0)
+    s = 2.0 ** power
+    xi = torch.from_numpy(W.random_complex(nc * G, seed=20)).cuda()
+    g = torch.from_numpy(W.random_complex((2, sub.ny, sub.nx), seed=21)).cuda()
+
+    half = 2.0 ** (-power // 2)        # back in two steps
+
+    def scaled(t):
+        return torch.view_as_complex(torch.view_as_real(t) * s)
+
+    for f, x, n in ((lambda x: plan.project(xi=x, kind="P"), xi, nc), (lambda x: plan.adjoint(x, grad_k=False)[0], xi, nc),
+                    (lambda x: plan.solve(0, x.view(2, sub.ny, sub.nx)), g, 2)):
+        ref, got = f(x).reshape(n, -1), f(scaled(x)).reshape(n, -1)
+        plan.status()
+        err = (torch.view_as_real(got) * half * half - torch.view_as_real(ref)).abs()
+        tiny = 200 * 2.0 ** (-1074 - power) / sub.h**2
+        assert (err.amax(dim=(1, 2)) <= 1e-14 * ref.abs().amax(dim=1) + tiny).all()
