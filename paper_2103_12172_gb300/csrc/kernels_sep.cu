@@ -162,6 +162,19 @@ __global__ void __launch_bounds__(32) k_sep_mode_tab(const SubDesc *subs, int s0
   T[MT_TH] = th; T[MT_KIND] = kind; T[MT_SG] = sg; T[MT_N1] = n1; T[MT_N2] = n2;
 }
 
+// phi_1, phi_2 at a subdomain's receiver row
+__global__ void __launch_bounds__(32) k_sep_rec(const SubDesc *subs, int s0, unsigned char *sep) {
+  const SubDesc &d = subs[s0 + blockIdx.y];
+  const int q = blockIdx.x * 32 + threadIdx.x + 1;
+  if (!d.tc_cols || d.nrec < 0 || q > d.Nq) return;
+  const double *T = reinterpret_cast<const double *>(sep + d.sep_mt) + (long long)(q - 1) * SEP_MTW;
+  double *P = reinterpret_cast<double *>(sep + d.sep_rp) + q - 1;
+  const int kind = (int)T[MT_KIND], J0 = d.nlo - 1, J1 = d.nhi + 1;
+  const double th = T[MT_TH], sr = T[MT_SG] < 0.0 && ((d.nrec - J0) & 1) ? -1.0 : 1.0, x = d.nrec - 0.5 * (J0 + J1);
+  P[0] = sr * (kind == 2 ? exp(-th * (d.nrec - J0)) : T[MT_N1] * sep_c(kind, th, x));
+  P[d.Nq] = sr * (kind == 2 ? exp(-th * (J1 - d.nrec)) : T[MT_N2] * sep_s(kind, th, x));
+}
+
 // phi_1, phi_2 on the rows J0 .. J1, [2][Py + 2][Nq]: a thread takes one mode and 8 rows, the
 // first by exp / sincos, the others by multiplying on (a rotation or a decay: 8 roundings).
 constexpr int PHI_ROWS = 8;
@@ -680,8 +693,8 @@ __device__ __forceinline__ void sep_modes_body(const Item &it, const SubDesc &d,
 #pragma unroll
   for (int r = 0; r < 4; ++r) ystore(r, out[0][2 + r], CD ? out[1][2 + r] : 0.0);
   if (rec) {
-    const double *phi = reinterpret_cast<const double *>(sep + d.sep_phi) + (long long)(d.nrec - d.nlo + 1) * d.Nq + q - 1;
-    const double p1 = phi[0], p2 = phi[(long long)(d.Py + 2) * d.Nq], f = T[MT_RFI];
+    const double *phi = reinterpret_cast<const double *>(sep + d.sep_rp) + q - 1;
+    const double p1 = phi[0], p2 = phi[d.Nq], f = T[MT_RFI];
     const double re = fma(p1, out[0][0], fma(p2, out[0][1], f * m3[0]));
     double im = 0.0;
     if (CD) im = fma(p1, out[1][0], fma(p2, out[1][1], CIN ? f * m3[P - 1] : 0.0));
@@ -830,9 +843,10 @@ cudaError_t set_sep_kernel_attributes() {
 
 cudaError_t launch_sep_tables(const mdp_plan *p, const SubDesc *ds, const double *tab, unsigned char *sep, bool entries,
                               cudaStream_t st) {
-  int mq = 0, mrow = 0, mdist = 0, mtb = 0, mes = 0, mmb = 0, mmk = 0, m3 = 0, m3k = 0;
+  int mq = 0, mrow = 0, mdist = 0, mtb = 0, mes = 0, mmb = 0, mmk = 0, m3 = 0, m3k = 0, mrec = 0;
   for (size_t i = 0; i < p->subs.size(); ++i) {
     const SubDesc &d = p->subs[i].d;
+    if (d.tc_cols && d.nrec >= 0) mrec = std::max(mrec, (d.Nq + 31) / 32);
     if (d.tc_cols && (d.leader == (int)i || d.nrec >= 0)) {   // a duplicate has its receiver row's moments
       const SepGeo g = sep_geo(d);
       mmb = std::max(mmb, g.ncls * g.nb * g.nqp / 32);
@@ -858,6 +872,7 @@ cudaError_t launch_sep_tables(const mdp_plan *p, const SubDesc *ds, const double
     const unsigned n = (unsigned)std::min(65535, ns - s0);
     k_sep_mode_tab<<<dim3(4 * mq, n), 32, 0, st>>>(ds, s0, sep, entries);
     k_full_modes<<<dim3(4 * mq, n), 32, 0, st>>>(ds, s0, sep);
+    if (mrec > 0) k_sep_rec<<<dim3(mrec, n), 32, 0, st>>>(ds, s0, sep);
     k_sep_phi<<<dim3(mq, mrow, n), 128, 0, st>>>(ds, s0, sep);
     if (mdist == 0) continue;   // no subdomain on the tensor cores
     k_sep_kd<<<dim3(mdist, n), 128, 0, st>>>(ds, s0, tab, sep);

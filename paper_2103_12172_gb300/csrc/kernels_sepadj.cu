@@ -228,6 +228,32 @@ __global__ void __launch_bounds__(32) k_adj_mode_tab(const SubDesc *subs, int s0
   D[MD_RHO1] = scale(rho1); D[MD_RHO2] = scale(rho2); D[MD_RFD] = scale(kb);
 }
 
+// d phi/dk at a subdomain's receiver row
+__global__ void __launch_bounds__(32) k_adj_rec(const SubDesc *subs, int s0, const unsigned char *sep, unsigned char *adj) {
+  const SubDesc &d = subs[s0 + blockIdx.y];
+  const int q = blockIdx.x * 32 + threadIdx.x + 1;
+  if (!d.tc_cols || d.nrec < 0 || q > d.Nq) return;
+  const double *T = reinterpret_cast<const double *>(sep + d.sep_mt) + (long long)(q - 1) * SEP_MTW;
+  const double *D = reinterpret_cast<const double *>(adj + d.adj_md) + (long long)(q - 1) * ADJ_MDW;
+  double *Q = reinterpret_cast<double *>(adj + d.adj_rp) + q - 1;
+  const int kind = (int)T[MT_KIND], J0 = d.nlo - 1, J1 = d.nhi + 1;
+  const double th = T[MT_TH], tc = D[MD_TC], sr = T[MT_SG] < 0.0 && ((d.nrec - J0) & 1) ? -1.0 : 1.0;
+  if (kind == 2) {
+    Q[0] = sr * (-(d.nrec - J0) * tc * exp(-th * (d.nrec - J0)));
+    Q[d.Nq] = sr * (-(J1 - d.nrec) * tc * exp(-th * (J1 - d.nrec)));
+    return;
+  }
+  const double x = d.nrec - 0.5 * (J0 + J1), iss = th > 0.0 ? 1.0 / D[MD_SS] : 0.0;
+  double C = 1.0, S = x;
+  if (th > 0.0) {
+    if (kind == 0) sincos(x * th, &S, &C);
+    else { C = cosh(x * th); S = sinh(x * th); }
+    S *= 1.0 / (kind == 0 ? sin(th) : sinh(th));
+  }
+  Q[0] = sr * (T[MT_N1] * (x * S * tc));
+  Q[d.Nq] = sr * (T[MT_N2] * (tc * ds_dc(x, th, D[MD_COS], D[MD_T], iss, C, S)));
+}
+
 // d phi/dk on the rows J0 .. J1, [2][Py + 2][Nq], from phi
 __global__ void __launch_bounds__(128) k_adj_phid(const SubDesc *subs, int s0, const unsigned char *sep, unsigned char *adj) {
   const int si = s0 + blockIdx.z;
@@ -792,9 +818,7 @@ __device__ __forceinline__ double adj_modes_body(const Item &it, const SubDesc &
   const int cp = sep_pad128(it.ncols), R = 2 * cp;
   const long long nc = it.ncols;
   const double *ga = ws + it.a_off + w.ga;
-  // phi_1 at the receiver row; phi_2 lies p2 further on, and so in the table of their k-derivatives
-  const long long orec = (long long)(d.nrec - d.nlo + 1) * d.Nq + q - 1, p2 = (long long)(d.Py + 2) * d.Nq;
-  const double *prec = reinterpret_cast<const double *>(sep + d.sep_phi) + orec;
+  const double *prec = reinterpret_cast<const double *>(sep + d.sep_rp) + q - 1;   // phi at the receiver row
   const double *mom = ws + it.a_off + w.mom + ((long long)e * ADJ_MOM * g.nqp + qi) * R + b;
   cplx F[6], dM[2], f4 = cmk(0.0, 0.0);   // moments, gamma rows; derivative moments; receiver row
 #pragma unroll
@@ -808,7 +832,7 @@ __device__ __forceinline__ double adj_modes_body(const Item &it, const SubDesc &
   if (rec) {
     f4 = ld2(ga + 2 * ((4LL * d.Nq + (q - 1)) * nc + b));
     F[0] = caxpy(prec[0], f4, F[0]);
-    F[1] = caxpy(prec[p2], f4, F[1]);
+    F[1] = caxpy(prec[d.Nq], f4, F[1]);
   }
   const bool imag = T[MT_IMAG] != 0.0;
   cplx m1 = F[0], m2 = F[1], iA = cmk(0.0, 0.0), iB = iA;   // moments of all rows; i Im R times them
@@ -917,8 +941,8 @@ __device__ __forceinline__ double adj_modes_body(const Item &it, const SubDesc &
   s += redotc(dM[0], a0) + redotc(dM[1], a1);
   if (rec) {
     const cplx m3 = at(rd, 2, inv2(D[MD_RFD]));
-    const double *dp = reinterpret_cast<const double *>(adj + d.adj_phid) + orec;
-    s += redotc(f4, cadd(caxpy(dp[0], a0, caxpy(dp[p2], a1, zero)), m3));
+    const double *dp = reinterpret_cast<const double *>(adj + d.adj_rp) + q - 1;
+    s += redotc(f4, cadd(caxpy(dp[0], a0, caxpy(dp[d.Nq], a1, zero)), m3));
   }
   return s;
 }
@@ -1059,12 +1083,13 @@ cudaError_t launch_adj_sines(const mdp_plan *p, cudaStream_t st) {
 }
 
 cudaError_t launch_adj_tables(const mdp_plan *p, cudaStream_t st) {
-  int mq = 0, mrow = 0, mdist = 0, mes = 0, mtb[2] = {0, 0}, mk[2] = {0, 0}, mt[2] = {0, 0}, m3 = 0, m3k = 0;
+  int mq = 0, mrow = 0, mdist = 0, mes = 0, mtb[2] = {0, 0}, mk[2] = {0, 0}, mt[2] = {0, 0}, m3 = 0, m3k = 0, mrec = 0;
   for (size_t i = 0; i < p->subs.size(); ++i) {
     const SubDesc &d = p->subs[i].d;
     if (!d.tc_cols || (d.leader != (int)i && d.nrec < 0)) continue;   // a duplicate has its receiver row's tables
     const SepGeo g = sep_geo(d);
     const AdjGeo a = adj_geo(d, g);
+    if (d.nrec >= 0) mrec = std::max(mrec, (d.Nq + 31) / 32);
     mq = std::max(mq, (d.Nq + 127) / 128);
     mrow = std::max(mrow, (d.Py + 2 + 7) / 8);
     mdist = std::max(mdist, d.Py);
@@ -1087,6 +1112,7 @@ cudaError_t launch_adj_tables(const mdp_plan *p, cudaStream_t st) {
   for (int s0 = 0; s0 < ns; s0 += 65535) {
     const unsigned n = (unsigned)std::min(65535, ns - s0);
     k_adj_mode_tab<<<dim3(4 * mq, n), 32, 0, st>>>(ds, s0, p->d_sep, p->d_adj);
+    if (mrec > 0) k_adj_rec<<<dim3(mrec, n), 32, 0, st>>>(ds, s0, p->d_sep, p->d_adj);
     k_adj_phid<<<dim3(mq, mrow, n), 128, 0, st>>>(ds, s0, p->d_sep, p->d_adj);
     k_adj_kd<<<dim3(mdist, n), 128, 0, st>>>(ds, s0, tab, p->d_sep, p->d_adj);
     for (int w = 0; w < 2; ++w) {

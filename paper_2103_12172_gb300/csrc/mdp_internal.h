@@ -77,10 +77,10 @@ struct SubDesc {
   long long adj_zm, adj_z3, adj_zd, adj_md, adj_phid, adj_kdd, adj_kde, adj_tb, adj_mb, adj_b3, adj_bf, adj_bi, adj_dtb,
       adj_dmb;
   long long sep_mx;     // per mode SEP_MXW doubles: the full-grid solve along y (kernels_full.cu)
-  // what depends on the receiver row, each subdomain's own (the rest is its leader's): the third block of the
-  // moments and its masks; in the gradient tables that of the residual's derivative moments, and the third K block
-  // of the synthesis
-  long long sep_rz, sep_rb, adj_rz, adj_rb, adj_r3z, adj_r3;
+  // what depends on the receiver row, each subdomain's own (the rest is its leader's): phi_1, phi_2 there
+  // (doubles [2][Nq]), the third block of the moments and its masks; in the gradient tables d phi/dk, the
+  // third block of the residual's derivative moments, and the third K block of the synthesis
+  long long sep_rp, sep_rz, sep_rb, adj_rp, adj_rz, adj_rb, adj_r3z, adj_r3;
   long long out_off;    // complex elements: start of the subdomain's output block
   long long rec_off;    // complex elements: start of the receiver block [n_cols][Px - 2]
   int *dstatus;         // the plan's device status word (bounds-checked build: first error; else unused)
@@ -206,6 +206,7 @@ inline __host__ __device__ void sep_tables(D &d, F f) {
     f(d.sep_rz, zw * n, TAB_MASK | TAB_OWN);
     f(d.sep_zm, zw * 2 * n, TAB_MASK);
     f(d.sep_z3, zw * g.nt3, TAB_MASK);
+    f(d.sep_rp, 16LL * d.Nq, TAB_OWN);
     f(d.sep_rb, g.ncls * n * g.nk1 * SEP_BBLK, TAB_OWN);
     f(d.sep_kd, 8 * pairs * d.Py, 0);
     f(d.sep_kde, 4LL * g.ncls * g.nS, 0);
@@ -397,6 +398,7 @@ inline __host__ __device__ void adj_tables(D &d, F f) {
   f(d.adj_zm, zw * ADJ_MOM * n, TAB_MASK);
   f(d.adj_z3, zw * a.nt3, TAB_MASK);
   f(d.adj_zd, zw * 2 * n, TAB_MASK);
+  f(d.adj_rp, 16LL * d.Nq, TAB_OWN);
   f(d.adj_rb, g.ncls * n * g.nk1 * SEP_BBLK, TAB_OWN);
   f(d.adj_r3, g.ncls * a.nt3 * 2 * n * SEP_BBLK, TAB_OWN);
   f(d.adj_md, 8LL * ADJ_MDW * d.Nq, 0);
