@@ -73,7 +73,8 @@ enum { MDP_OUT_Q = 0, MDP_OUT_P = 1 };
  * and FP64 sums instead of the separable Green's function with its contractions on the tensor cores
  * (which subdomains take it: up to 2048 cells along x where M+ is centred, 1024 otherwise, and up to 2050, 1026
  * rows of M+), and, in the sweeps, the sine transforms of the dense ring and gamma rows by direct sums
- * instead of the FFT. */
+ * instead of the FFT. The projection's sweep of a mode at or below its cutoff is the closed form with running
+ * moments, where pivots never settle; full-grid solves and the gradient pass factor every mode. */
 #define MDP_PLAN_FP64_COLS 0x8u
 #define MDP_PLAN_DIRECT_ROWS 0x10u
 

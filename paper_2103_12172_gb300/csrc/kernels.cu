@@ -170,7 +170,7 @@ __global__ void __launch_bounds__(256) k_residual(Batch bt, const SubDesc *subs,
 
 // ---------------------------------------------------------------- k_ring
 // The ring residuals of basis columns for the separable solve, in k_residual's layout, only where they are
-// not zero by construction (sep_support in the operand cutting): a column's density lives on its own side,
+// not zero by construction (sep_cut_body knows what it leaves unwritten): a column's density lives on its own side,
 // so a column of side 1 or 2 has them on the two dense rows next to it, one of side 3 or 4 on the two ring
 // columns next to it and the ends of the dense rows. One thread per (unit, column); a unit is, for sides 1
 // and 2, a node pair (m, Nx - m) of both dense rows (x-centred; else a node of them), and for sides 3 and 4 a

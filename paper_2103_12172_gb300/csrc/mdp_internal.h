@@ -160,10 +160,12 @@ inline int propagating_modes(const SubDesc &d) {
   const double s = 0.5 * std::sqrt(d.k * d.k / (1.0 / (d.h * d.h) + d.k * d.k / 12.0));
   return s >= 1.0 ? d.Nq : std::min(d.Nq, (int)(2.0 * d.Nx / M_PI * std::asin(s)) + 1);
 }
-// modes per block (4 warps) of k_sep_modes and k_adj_modes: 16, or 4 where the item has fewer blocks of 16 than the
-// GPU has SMs (a block's modes follow one another: 129^2, 128 columns: k_sep_modes 14.8 -> 6.7 us)
+// modes per block (4 warps) of k_sep_modes and k_adj_modes: 16, or 4 where the item has fewer blocks of 16 than a
+// GB300 has SMs (a block's modes follow one another: 129^2, 128 columns: k_sep_modes 14.8 -> 6.7 us). The workspace is
+// laid out by it before the device is asked, so the number is the part's; another part's runs as well, less well split.
+constexpr int GB300_SMS = 152;
 inline __host__ __device__ int sep_modes_per_block(const SubDesc &d, int ncols) {
-  return ((ncols + 31) / 32) * ((d.Nq + 15) / 16) < 152 ? 4 : 16;
+  return ((ncols + 31) / 32) * ((d.Nq + 15) / 16) < GB300_SMS ? 4 : 16;
 }
 inline __host__ __device__ SepGeo sep_geo(const SubDesc &d) {
   SepGeo g;
@@ -547,8 +549,8 @@ struct mdp_plan {
   mdp::HostBuf<uint8_t> host_piv;
   long long out_size = 0;
   long long rec_size = 0;
-  int tile_cols = 256;                   // columns per work item of sweeps and of the gradient pass
-  int sep_cols = 512;                    // columns per work item of the separable solve
+  int tile_cols = 256;                   // columns per work item of subdomains that take the sweeps
+  int sep_cols = 512;                    // of those that take the separable solve, in its gradient pass too
   int fft_block_points = mdp::FFT_BLOCK_POINTS;  // complex values per block of the dense-row FFT kernels
   int tri_stages = 2;                    // table rows the projection sweep stages ahead (2 or 4)
   long long ws_budget = 0;               // bytes of workspace

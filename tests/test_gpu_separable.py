@@ -286,3 +286,43 @@ def test_densities_near_the_ends_of_the_exponents_range(mdp, power, off):
         err = (torch.view_as_real(got) * half * half - torch.view_as_real(ref)).abs()
         tiny = 200 * 2.0 ** (-1074 - power) / sub.h**2
         assert (err.amax(dim=(1, 2)) <= 1e-14 * ref.abs().amax(dim=1) + tiny).all()
+
+
+def column(py, dx=0):
+    """py rows and 25 (dx cells off centre) columns of M+ in a grid of margins of 19 and 4 cells."""
+    h = 1.0 / 25
+    return W.Subdomain(0.0, 1.0, 0.0, py * h, -(4.5 + dx) * h, -19.5 * h, h, 35 + dx, py + 40, 7.0, W.AP_DIRX_SOMMY, 1)
+
+
+@pytest.mark.parametrize("py,dx", [(2049, 0), (2050, 0), (2051, 0), (3300, 0), (1026, 3), (1027, 3)])
+def test_columns_of_tall_grids_are_those_of_the_pivoted_factors(mdp, py, dx):
+    """On either side of the limits the projection's columns are the traces of the basis densities' potentials
+    solved by the pivoted factors of every mode (the sweeps' plan), which share no closed form with
+    them. Bar: the factors' own error at these heights, 1e-9."""
+    sub = column(py, dx)
+    plan, ref = mdp.Plan([sub]), mdp.Plan([sub], fp64_cols=True)
+    info = plan.sub_info(0)
+    assert (info["Py"], info["xsym"]) == (py, int(dx == 0))
+    G, nc, _, nm = plan.layout(0)
+    u = ref.potential(0, ref.basis_densities(0)).cpu().numpy()
+    plan.status()
+    for p in (plan, ref):
+        assert rel_col_err(p.project(kind="P").view(nc, G).cpu().numpy(), u[:, nm[:, 0], nm[:, 1]]) < 1e-9
+
+
+def test_subdomains_beyond_the_limits_beside_others(mdp):
+    """One plan with subdomains of the sweeps and of the separable solve, centred and not: projection and
+    gradients bit for bit those of plans of their own."""
+    subs = [column(2051), W.small_subdomain(33, 8.0, W.AP_DIRICHLET4, 1), column(1027, 3), box(37, 33, 9.0, W.AP_DIRX_SOMMY, 1, dx=0.1)]
+    plan = mdp.Plan(subs)
+    cot = torch.from_numpy(W.random_complex(plan.output_size, seed=22)).cuda()
+    xi = torch.from_numpy(W.random_complex(plan.output_size, seed=23)).cuda()
+    got = [plan.blocks(plan.project()), plan.blocks(plan.project(xi=xi))] + [plan.adjoint(cot, xi=x) for x in (None, xi)]
+    plan.status()
+    for i, sub in enumerate(subs):
+        one = mdp.Plan([sub])
+        x, c = plan.blocks(xi)[i].reshape(-1), plan.blocks(cot)[i].reshape(-1)
+        assert torch.equal(got[0][i].reshape(-1), one.project()) and torch.equal(got[1][i].reshape(-1), one.project(xi=x))
+        for (gx, gk), d in zip(got[2:], (None, x)):
+            rx, rk = one.adjoint(c, xi=d)
+            assert torch.equal(plan.blocks(gx)[i].reshape(-1), rx) and gk[i] == rk[0]
