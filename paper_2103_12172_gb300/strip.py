@@ -428,7 +428,7 @@ class LayeredStrip:
         """The Chebyshev coefficients [c^(0) sides 1..4, c^(1) sides 1..4] of every layer's boundary
         data from the coupled least-squares solve, and the receiver output of the projection."""
         coef, rec = self._coefficients(k)
-        return list(coef.unbind(0)), rec
+        return [c.clone() for c in coef.unbind(0)], rec   # tensors of their own, as the caller may change them in place
 
     def _coefficients(self, k):
         """coefficients() as one tensor [N, 8 M].

@@ -109,3 +109,19 @@ def test_gradient_of_a_layout_with_1120_shared_unknowns(mdp):
         got.append((u.detach(), g))
     for a, b in zip(*got):
         assert (a - b).abs().max() < 1e-8 * b.abs().max()
+
+
+def test_coefficients_may_be_changed_in_place(mdp):
+    """The layers' coefficients are tensors of their own: an in-place change of one is differentiated and leaves the
+    others as they are."""
+    from paper_2103_12172_gb300.strip import LayeredStrip, incident_impedance_bc
+    subs = [W.unit_subdomain(j, 0, 33, 4.0 + j, W.AP_DIRX_SOMMY, 4) for j in range(2)]
+    lay = LayeredStrip(subs, incident_impedance_bc(0.3), [16, 16])
+    k = torch.tensor([4.0, 5.0], dtype=torch.float64, device="cuda", requires_grad=True)
+    c, _ = lay.coefficients(k)
+    ref = [v.detach().clone() for v in c]
+    c[0].mul_(2.0)
+    assert torch.equal(c[0].detach(), 2.0 * ref[0]) and torch.equal(c[1].detach(), ref[1])
+    (g,) = torch.autograd.grad(c[0].abs().square().sum(), k)
+    (h,) = torch.autograd.grad(lay.coefficients(k)[0][0].abs().square().sum(), k)
+    assert (g - 4.0 * h).abs().max() <= 1e-12 * h.abs().max()
