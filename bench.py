@@ -47,6 +47,16 @@ def hbm_peak():
         return 6800.0, "fallback"
 
 
+def tensor_peak():
+    """(TFLOP/s, source) of the fp16 tensor cores: the measured dense bf16 GEMM rate (the same rate as fp16's) when
+    the measured-peaks file is present, else the recipe's fallback figure."""
+    try:
+        v = float(json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json")))["bf16_tflops"])
+        return v, "measured"
+    except (OSError, ValueError, KeyError, TypeError):
+        return 1900.0, "fallback"
+
+
 # ------------------------------------------------------------------ oracle timing (CPU)
 def _oracle_worker_init(sub_dict):
     os.environ.setdefault("OMP_NUM_THREADS", "1")
@@ -236,8 +246,8 @@ def kernel_flops(plan, items, fp64_cols=False):
     solve: the real multiply-adds of its two contractions as dense products (k_sep_gemm1: the ring's middle
     rows against K and the moment tables, the dense rows' sine transforms; k_inv_cols_tc: the modes against
     the synthesis table, the gamma rows' inverse transforms) and of the modes' 6 x 6 matrices. The tensor
-    cores form them from fp16 digits and leave out groups whose digits are all zero, so a rate by this
-    count may exceed the FP64 pipe's. Others: the arithmetic of the ring-sparse sweeps as the kernels
+    cores form each product by 56 fp16 multiply-adds of digits and leave out groups whose digits are all zero
+    (k_inv_cols_tc is the name of stage 3 in the plan's profile). Others: the arithmetic of the ring-sparse sweeps as the kernels
     perform it -- complex factor rows cost complex multiply-adds, rows whose LU factors are real cost
     real-by-complex ones, and a centred subdomain pairs m with Nx - m in the sine transforms."""
     tot = {}
@@ -303,10 +313,10 @@ def kernel_source_sha():
     return h.hexdigest()
 
 
-def recorded_traffic(kernel, workload):
-    """DRAM bytes per step of `kernel` on `workload` from profiles/traffic.json (an ncu capture
-    of every launch of one step, or a smaller capture scaled by the units processed, as recorded
-    there), or None when absent or taken on a different kernel source. Per step, not per launch:
+def recorded(kernel, workload):
+    """The record of `kernel` on `workload` in profiles/traffic.json (DRAM bytes per step and the tensor pipe's
+    active share from an ncu capture of every launch of one step), or {} when absent or taken on a different kernel
+    source. Per step, not per launch:
     the plan's workspace budget decides how many waves (launches) a step takes; the record is
     taken with the plan the autotuner picks, whose packing also sets how many table rows come
     from L2."""
@@ -314,8 +324,8 @@ def recorded_traffic(kernel, workload):
     try:
         rec = json.load(open(path))[workload][kernel]
     except (OSError, ValueError, KeyError):
-        return None
-    return rec["dram_bytes_per_step"] if rec.get("source_sha256") == kernel_source_sha() else None
+        return {}
+    return rec if rec.get("source_sha256") == kernel_source_sha() else {}
 
 
 # ------------------------------------------------------------------ reference arm
@@ -505,17 +515,31 @@ def measure(mdp, wl, steps, warmup, world=1, barrier=None, clocks=None, full=Tru
     launch_s = dom_ms / dom_launches / 1e3
     achieved = flops_per_launch / launch_s / 1e12
     peak = NOMINAL_FP64_GFLOPS / 1e3
-    step_traffic = recorded_traffic(dom, wl.name)
+    step_tflops = sum(flops.values()) / (total_ms / steps / 1e3) / 1e12
+    rec = recorded(dom, wl.name)
+    step_traffic = rec.get("dram_bytes_per_step")
     traffic = step_traffic / launches_per_step if step_traffic else None
     hbm, hbm_src = hbm_peak()
-    roof = {"bound": "tensor" if dom in ("k_sep_gemm1", "k_inv_cols_tc") else "alu", "kernel": dom, "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
-            "frac": achieved / peak, "traffic": traffic,
-            "rate_note": "FP64-equivalent: the contractions as dense FP64 products, which the tensor cores form exactly "
-                         "from fp16 digits with zero groups left out",
-            "peak_note": "FP64 FMA: 152 SMs x 2 DFMA/clk x 2 flop x 2.07 GHz (derived from unit counts and "
-                         "clock; the DFMA rate per SM is measured by the probe)",
-            "step_flop_frac": sum(flops.values()) / (total_ms / steps / 1e3) / 1e12 / peak,
-            "launches_per_step": launches_per_step}
+    if dom in ("k_sep_gemm1", "k_inv_cols_tc"):
+        # an FP64 product is 7 MMAs of N = 256 for 32 outputs: 56 fp16 multiply-adds
+        tpeak, tsrc = tensor_peak()
+        active = rec.get("tensor_pipe_active")
+        roof = {"bound": "tensor", "kernel": dom, "achieved": 56 * achieved, "peak": tpeak, "unit": "TFLOP/s",
+                "frac": active, "traffic": traffic, "fp64_equivalent_tflops": achieved,
+                "rate_note": "achieved: fp16 flops of the dense digit products (56 multiply-adds per FP64 product); groups "
+                             "whose digits are all zero are left out, so it can exceed the peak. frac: the tensor pipe's "
+                             "active cycles, recorded by ncu for this kernel source (null without such a record)",
+                "peak_note": f"{tsrc} dense bf16 GEMM", "step_flop_frac": None}
+    else:
+        roof = {"bound": "alu", "kernel": dom, "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
+                "frac": achieved / peak, "traffic": traffic,
+                "peak_note": "FP64 FMA: 152 SMs x 2 DFMA/clk x 2 flop x 2.07 GHz (derived from unit counts and "
+                             "clock; the DFMA rate per SM is measured by the probe)",
+                "step_flop_frac": step_tflops / peak}
+    roof["step_fp64_equivalent_tflops"] = step_tflops
+    roof["launches_per_step"] = launches_per_step
+    roof["times_note"] = ("kernel times from as many further steps with an event around every launch, which keeps the "
+                          "launches from overlapping; the timed steps have no events inside")
     if traffic:
         roof["dram_gbs"] = traffic / launch_s / 1e9
         roof["dram_frac"] = roof["dram_gbs"] / hbm

@@ -1,11 +1,13 @@
-// Contractions to FP64 accuracy on the fp16 tensor cores by error-free splitting (Ozaki, Ogita, Oishi and
-// Rump, Numer. Algorithms 59, 2012): the operands' cut into digits, and the kernel body that streams
-// digit blocks, issues the MMAs and adds their exact sums (kernels_sep.cu, kernels_full.cu).
+// Contractions on the fp16 tensor cores, to FP64 accuracy relative to the largest values of a row and of a table,
+// by error-free splitting (Ozaki, Ogita, Oishi and Rump, Numer. Algorithms 59, 2012): the operands' cut
+// into digits, and the kernel body that streams digit blocks, issues the MMAs and adds their exact sums
+// (kernels_sep.cu, kernels_full.cu).
 //
 // Every operand value becomes an integer |V| <= 2^54 on one scale (a row of A: its largest value; B: a
-// bound of its table) and V 7 balanced base-256 digits, exact in fp16. Of the 49 digit products those of
-// weight t + u <= 7 are kept (34; the largest dropped one is 2^-64 of the leading one, below the
-// operands' own 2^-54). Products of equal weight share one FP32 accumulator: at most 7 x 128 x 2^14
+// bound of its table) and V 7 balanced base-256 digits, exact in fp16: a value is kept to 2^-55 of the scale, so one
+// 2^-30 of the row's largest has 24 bits of its own. Of the 49 digit products those of weight t + u <= 7 are kept
+// (34): the five of weight 8, the largest left out, are together below 2^-59 of the product of the two
+// scales for a value of K, under the operands' own rounding. Products of equal weight share one FP32 accumulator: at most 7 x 128 x 2^14
 // < 2^24 between two read-backs of 128 values of K, so every sum is an exact integer.
 #pragma once
 #include "tc_common.cuh"

@@ -20,6 +20,8 @@ using cd = std::complex<double>;
 static const double kTieTol = 1e-9;       // side-ownership ties within 1e-9*h
 static const double kSingularTol = 1e-13; // pivot below this x max|T| -> singular
 
+// (k_inv_cols_tc and k_adj_ring_cols_tc: the contractions that give the gamma and the ring columns of the middle rows,
+// stage 3 of k_sep_gemm and k_adj_gemm; programs look them up by these names)
 const char *fam_name(int f) {
   static const char *names[NFAM] = {"k_extend", "k_residual", "k_fwd_rows", "k_tri", "k_inv_rows", "k_inv_cols",
                                     "k_adj_rows", "k_adj_tri", "k_adj_ring_rows", "k_adj_ring_cols", "k_adj_gamma",
