@@ -9,9 +9,11 @@
 //   - the condensed, pivot-scaled forward-sweep rows of the projection (rows above the ring
 //     folded into the last pivot by their Schur complement), with its run of real rows; stored only for
 //     subdomains that project by sweeps (without the separable solve), or when `all` is set (table
-//     introspection). Its pivots are looked at for every subdomain: close to an eigenvalue they fall below the
-//     tolerance where the full factors' may not (the last pivot is the distance over the square of
-//     the eigenvector's last entry, small next to a Dirichlet end), and plan creation refuses by both.
+//     introspection). Its pivots are looked at for every subdomain's propagating modes: close to an
+//     eigenvalue they fall below the tolerance where the full factors' may not (the last pivot is the distance
+//     over the square of the eigenvector's last entry, small next to a Dirichlet end), and plan creation refuses by
+//     both. The other modes' rows are diagonally dominant: no pivot of theirs comes near the tolerance (1e-3 of
+//     the largest entry over random grids, APs and wavenumbers, tolerance 1e-13).
 // The host plan builds the same tables at plan creation (plan.cpp: mode_matrix, band_lu,
 // factor_mode, build_fs_mode). Two kernels:
 //   k_factor_chain  the pivot recurrences, the only sequential part: one thread per (mode,
@@ -289,7 +291,7 @@ __device__ void chain_sweep(const SubDesc &d, int q, double *tab, int *status, b
 }
 
 // Blocks of one warp: n_prop of them with a propagating mode each, then the other modes 32 to a block; and
-// the same again for the sweep tables.
+// the same again for the sweep tables (n_prop blocks again where none is stored).
 __global__ void __launch_bounds__(32) k_factor_chain(const SubDesc *subs, int n_subs, int n_prop, int n_rest, double *tab,
                                                      uint8_t *piv, int *status, int all) {
   const int per = n_prop + (n_rest + 31) / 32, sweep = blockIdx.x >= per, blk = blockIdx.x - (sweep ? per : 0);
@@ -306,8 +308,10 @@ __global__ void __launch_bounds__(32) k_factor_chain(const SubDesc *subs, int n_
   }
   if (si >= n_subs) return;
   const int q = prop ? t + 1 : subs[si].n_prop + t + 1;
-  if (sweep) chain_sweep(subs[si], q, tab, status, !prop, all || !subs[si].tc_cols);
-  else chain_full(subs[si], q, tab, piv, status, !prop);
+  if (sweep) {
+    const bool store = all || !subs[si].tc_cols;
+    if (store || prop) chain_sweep(subs[si], q, tab, status, !prop, store);
+  } else chain_full(subs[si], q, tab, piv, status, !prop);
 }
 
 constexpr int kRowsThreads = 256;
@@ -452,11 +456,13 @@ __global__ void k_probe_rcp(const double *x, double *y, int n) {
 cudaError_t launch_factor_to(const mdp_plan *p, const SubDesc *ds, double *tab, uint8_t *piv, int *status, bool all,
                              cudaStream_t st) {
   int n_modes = 0, n_prop = 0;
+  bool store = all;
   for (size_t i = 0; i < p->subs.size(); ++i) {
+    store = store || !p->subs[i].d.tc_cols;
     if (p->subs[i].d.leader == (int)i) { n_modes += p->subs[i].d.Nq; n_prop += p->subs[i].d.n_prop; }
   }
   const int blocks = n_prop + (n_modes - n_prop + 31) / 32;
-  k_factor_chain<<<2 * blocks, 32, 0, st>>>(ds, (int)p->subs.size(), n_prop, n_modes - n_prop, tab, piv, status, all);
+  k_factor_chain<<<blocks + (store ? blocks : n_prop), 32, 0, st>>>(ds, (int)p->subs.size(), n_prop, n_modes - n_prop, tab, piv, status, all);
   k_factor_rows<<<n_modes, kRowsThreads, 0, st>>>(ds, (int)p->subs.size(), tab, all);
   return cudaGetLastError();
 }
