@@ -158,11 +158,10 @@ __device__ __forceinline__ double sum_to_double(long long hi, long long lo, int 
   // the leading 64 bits of the 96, then 53 of them rounded
   unsigned long long top = lz <= 32 ? ((unsigned long long)l << lz) >> 32 : (unsigned long long)l << ((lz - 32) & 63);
   if (lz < 64) top |= (unsigned long long)h << lz;
-  const int e = 1023 + 95 - lz + ex;      // biased exponent; below 1 the result is subnormal and loses 1 - e bits more
-  const int sh = min(max(11 - e, 10), 63);
-  const unsigned long long t = top >> sh;
-  unsigned long long v = ((unsigned long long)max(e - 1, 0) << 52) + (t >> 1) + (t & 1);
-  if (lz == 96 || e < -52) v = 0;
+  const int e = 1023 + 95 - lz + ex;      // biased exponent
+  unsigned long long v = ((unsigned long long)(e - 1) << 52) + (top >> 11) + ((top >> 10) & 1);
+  if (e < 1) v = e < -52 ? 0 : ((top >> (11 - e)) + 1) >> 1;   // subnormal: 1 - e bits less
+  if (lz == 96) v = 0;
   if (e > 2046) v = 0x7ff0000000000000ULL;
   if (ex == INT_MAX) v = 0x7ff8000000000000ULL;
   return __longlong_as_double((long long)(v | ((unsigned long long)neg << 63)));
