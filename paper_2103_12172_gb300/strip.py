@@ -329,7 +329,11 @@ class LayeredStrip:
         (without a source; the source terms are not differentiated)."""
         if self.source is not None and k.requires_grad:
             raise NotImplementedError("the k-gradient of the source terms is not implemented")
-        coef, rec = self._coefficients(k)
+        if getattr(self.coefficients, "__func__", None) is LayeredStrip.coefficients:
+            coef, rec = self._coefficients(k)
+        else:                              # a subclass's own coefficients
+            cvecs, rec = self.coefficients(k)
+            coef = torch.stack(list(cvecs)).to(torch.complex128)
         if self._rec_blocks is None:
             self._rec_blocks = _Blocks(self.layout[0][1], [r[2] for r in self.rlayout], [r[3] for r in self.rlayout],
                                        rec.device)

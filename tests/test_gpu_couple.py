@@ -125,3 +125,21 @@ def test_coefficients_may_be_changed_in_place(mdp):
     (g,) = torch.autograd.grad(c[0].abs().square().sum(), k)
     (h,) = torch.autograd.grad(lay.coefficients(k)[0][0].abs().square().sum(), k)
     assert (g - 4.0 * h).abs().max() <= 1e-12 * h.abs().max()
+
+
+def test_receivers_take_a_subclass_s_coefficients(mdp):
+    from paper_2103_12172_gb300.strip import LayeredStrip, incident_impedance_bc
+
+    class Twice(LayeredStrip):
+        def coefficients(self, k):
+            c, rec = super().coefficients(k)
+            return [2.0 * v for v in c], rec
+
+    subs = [W.unit_subdomain(j, 0, 33, 4.0 + j, W.AP_DIRX_SOMMY, 4) for j in range(2)]
+    k = torch.tensor([4.0, 5.0], dtype=torch.float64, device="cuda", requires_grad=True)
+    got = []
+    for cls in (LayeredStrip, Twice):
+        u = torch.cat(cls(subs, incident_impedance_bc(0.3), [16, 16]).receivers(k))
+        got.append((u.detach(), torch.autograd.grad(u.abs().square().sum(), k)[0]))
+    assert torch.equal(got[1][0], 2.0 * got[0][0])
+    assert (got[1][1] - 4.0 * got[0][1]).abs().max() <= 1e-12 * got[1][1].abs().max()
