@@ -629,9 +629,8 @@ __device__ __forceinline__ void sep_modes_body(const Item &it, const SubDesc &d,
   const long long nc = it.ncols;
   const double *gr = ws + it.gr_off;
   const double *mom = ws + it.a_off + w.mom + ((long long)e * 3 * g.nqp + qi) * R1 + row1;
-  const bool rec = d.nrec >= 0;
   constexpr int P = CIN ? 2 : 1;
-  double in[P][6], m3[P], out[2][6];   // [part][input], [part][output]
+  double in[P][6], out[2][6];   // [part][input], [part][output]
 #pragma unroll
   for (int r = 0; r < 4; ++r) {
     const long long o = ((long long)r * d.Nq + (q - 1)) * nc + b;
@@ -642,7 +641,6 @@ __device__ __forceinline__ void sep_modes_body(const Item &it, const SubDesc &d,
   for (int p = 0; p < P; ++p) {        // row1 < 0: no source on the middle rows
     in[p][4] = row1 >= 0 ? mom[p * cp] : 0.0;
     in[p][5] = row1 >= 0 ? mom[(long long)g.nqp * R1 + p * cp] : 0.0;
-    m3[p] = rec && row1 >= 0 ? mom[2LL * g.nqp * R1 + p * cp] : 0.0;
   }
   if (T[MT_FAR] != 0.0) {   // the two ends do not see each other: two 3 x 3 blocks
 #pragma unroll
@@ -692,18 +690,29 @@ __device__ __forceinline__ void sep_modes_body(const Item &it, const SubDesc &d,
   };
 #pragma unroll
   for (int r = 0; r < 4; ++r) ystore(r, out[0][2 + r], CD ? out[1][2 + r] : 0.0);
-  if (rec) {
-    const double *phi = reinterpret_cast<const double *>(sep + d.sep_rp) + q - 1;
-    const double p1 = phi[0], p2 = phi[d.Nq], f = T[MT_RFI];
-    const double re = fma(p1, out[0][0], fma(p2, out[0][1], f * m3[0]));
-    double im = 0.0;
-    if (CD) im = fma(p1, out[1][0], fma(p2, out[1][1], CIN ? f * m3[P - 1] : 0.0));
-    ystore(4, re, im);
-  }
+}
+// The field at the subdomain's receiver row, from the coefficients that the thread has stored and the third moment: in a
+// pass of its own, so that calls without receivers keep the modes' matrix to 62 and 70 registers, 8 and 7 blocks to
+// an SM (72 and 94 with the row's pointers beside it: 4 x 257^2 209.5 -> 208.9 us, complex data 257.8 -> 255.7).
+template <bool CD, bool CIN>
+__device__ __forceinline__ void sep_rec_body(const Item &it, const SubDesc &d, const SepGeo &g, const SepWs &w,
+                                             const unsigned char *sep, double *ws, int b, int row, int row1, int q) {
+  const double f = reinterpret_cast<const double *>(sep + d.sep_mt)[(long long)(q - 1) * SEP_MTW + MT_RFI];
+  const double *phi = reinterpret_cast<const double *>(sep + d.sep_rp) + q - 1;
+  const double p1 = phi[0], p2 = phi[d.Nq];
+  const int e = d.xsym ? ((q & 1) ? 0 : 1) : 0, qi = d.xsym ? (q - 1) >> 1 : q - 1;
+  const int cp = sep_pad128(it.ncols), R1 = sep_rows(d, J_MID, it.ncols, it.col0, CIN), R3 = (CD ? 2 : 1) * cp;
+  const double *m3 = ws + it.a_off + w.mom + ((long long)(3 * e + 2) * g.nqp + qi) * R1 + row1;
+  const double *ae = ws + it.a_off + w.aeff + ((long long)e * 2 * g.nqp + qi) * R3 + row, *be = ae + (long long)g.nqp * R3;
+  const double re = fma(p1, ae[0], fma(p2, be[0], row1 >= 0 ? f * m3[0] : 0.0));
+  const long long o = ((long long)(q - 1) * 5 + 4) * it.ncols + b;
+  double *y = ws + it.y_off;
+  if (CD) st2(y + 2 * o, cmk(re, fma(p1, ae[cp], fma(p2, be[cp], CIN && row1 >= 0 ? f * m3[cp] : 0.0))));
+  else y[o] = re;
 }
 
 template <bool CIN>
-__global__ void __launch_bounds__(128) k_sep_modes(Batch bt, const SubDesc *subs, const unsigned char *sep, double *ws) {
+__global__ void __launch_bounds__(128, CIN ? 7 : 8) k_sep_modes(Batch bt, const SubDesc *subs, const unsigned char *sep, double *ws) {
   pdl_wait();
   Item it; int local;
   locate(bt, blockIdx.x, it, local);
@@ -720,6 +729,11 @@ __global__ void __launch_bounds__(128) k_sep_modes(Batch bt, const SubDesc *subs
   for (int q = q0; q < q0 + per - (int)threadIdx.y && q <= d.Nq; q += 4) {
     if (d.cplx || CIN) sep_modes_body<true, CIN>(it, d, g, w, sep, ws, b, row, row1, q);
     else sep_modes_body<false, CIN>(it, d, g, w, sep, ws, b, row, row1, q);
+  }
+  if (d.nrec < 0) return;
+  for (int q = q0; q < q0 + per - (int)threadIdx.y && q <= d.Nq; q += 4) {
+    if (d.cplx || CIN) sep_rec_body<true, CIN>(it, d, g, w, sep, ws, b, row, row1, q);
+    else sep_rec_body<false, CIN>(it, d, g, w, sep, ws, b, row, row1, q);
   }
 }
 
